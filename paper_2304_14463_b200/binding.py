@@ -1,8 +1,10 @@
 """Thin ctypes binding of libmoc_b200.so (argument marshalling only; see include/moc.h).
 
 Function names mirror the C ABI.  PyTorch supplies device memory and streams: tensors are passed as
-``data_ptr()`` and the stream as ``torch.cuda.current_stream().cuda_stream``.  If the CUDA library
-has not been built, importing this module raises -- there is no CPU path.
+``data_ptr()`` and the stream as ``torch.cuda.current_stream().cuda_stream``.  The calls that only
+enqueue work on device tensors take their arguments apart in native code (_moc_torch.so, built from
+csrc/moc_torch.cpp): on small batches the interpreter would otherwise take longer than the GPU.  If the
+libraries have not been built, importing this module raises -- there is no CPU path.
 """
 from __future__ import annotations
 
@@ -27,6 +29,13 @@ EXPORTS = ["moc_graph_create", "moc_graph_set_max_copies", "moc_graph_destroy", 
 if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2304_14463_b200.build` "
                       "(nvcc, sm_100a). There is no CPU fallback.")
+
+import torch  # noqa: E402  (its libraries have to be loaded in front of _moc_torch.so)
+try:
+    from . import _moc_torch as _fast
+except ImportError as _e:
+    raise ImportError(f"_moc_torch.so is missing or does not load ({_e}): build it with "
+                      "`python -m paper_2304_14463_b200.build`") from _e
 
 lib = ctypes.CDLL(LIB_PATH)
 _P, _i32, _i64 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
@@ -86,6 +95,8 @@ lib.moc_last_launch_count.restype = ctypes.c_int
 lib.moc_last_launch_count.argtypes = []
 lib.moc_last_error.restype = ctypes.c_char_p
 lib.moc_last_error.argtypes = []
+# the native side of the binding calls the library through the same addresses
+_fast.bind({name: ctypes.cast(getattr(lib, name), _P).value for name in EXPORTS})
 
 
 class MocError(RuntimeError):
@@ -101,12 +112,10 @@ def _check(rc, where):
 
 
 def _stream():
-    import torch
     return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
 
 
 def _dev(t, dtype, name):
-    import torch
     if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous()):
         raise TypeError(f"{name}: expected a contiguous CUDA tensor of {dtype}")
     return ctypes.c_void_p(t.data_ptr())
@@ -115,16 +124,12 @@ def _dev(t, dtype, name):
 def _host(a, dtype, name):
     """numpy array or CPU torch tensor -> pointer (the object must stay alive during the call)."""
     import numpy as np
-    try:
-        import torch
-        if isinstance(a, torch.Tensor):
-            if a.is_cuda or not a.is_contiguous():
-                raise TypeError(f"{name}: expected a contiguous CPU tensor")
-            if a.numpy().dtype != np.dtype(dtype):
-                raise TypeError(f"{name}: expected dtype {dtype}")
-            return ctypes.c_void_p(a.data_ptr())
-    except ImportError:
-        pass
+    if isinstance(a, torch.Tensor):
+        if a.is_cuda or not a.is_contiguous():
+            raise TypeError(f"{name}: expected a contiguous CPU tensor")
+        if a.numpy().dtype != np.dtype(dtype):
+            raise TypeError(f"{name}: expected dtype {dtype}")
+        return ctypes.c_void_p(a.data_ptr())
     if not (isinstance(a, np.ndarray) and a.dtype == np.dtype(dtype) and a.flags.c_contiguous):
         raise TypeError(f"{name}: expected a C-contiguous numpy array of {dtype}")
     return ctypes.c_void_p(a.ctypes.data)
@@ -206,7 +211,9 @@ def _check_outputs(lens, outs):
 
 def moc_eval_batch(g, seqs, lens, M, out_peak=None, out_dur=None, out_feasible=None):
     """Device tensors in, device tensors out (allocated with torch if not given). Asynchronous."""
-    import torch
+    r = _fast.eval_batch(g, seqs, lens, M, out_peak, out_dur, out_feasible)
+    if r is not None:
+        return r if r.__class__ is tuple else _check(r, "moc_eval_batch")
     B = lens.numel()
     if out_peak is None:
         out_peak = torch.empty(B, dtype=torch.int64, device=lens.device)
@@ -229,7 +236,6 @@ def moc_eval_batch_noalloc(g, seqs, lens, M, out_peak, out_dur, out_feasible):
     """moc_eval_batch for callers that must not allocate: every tensor, outputs included, is passed
     in, and the library keeps its packing offsets in a fixed array of its own device image (at most
     MOC_NOALLOC_MAX_B sequences per call; calls on one device must not overlap on the GPU)."""
-    import torch
     _check_outputs(lens, (("out_peak", out_peak), ("out_dur", out_dur), ("out_feasible", out_feasible)))
     rc = lib.moc_eval_batch_noalloc(g, _dev(seqs, torch.int32, "seqs"), _dev(lens, torch.int32, "lens"),
                                     lens.numel(), int(M), _dev(out_peak, torch.int64, "out_peak"),
@@ -263,7 +269,9 @@ def moc_eval_batch_host16(g, seqs, lens, M, out_peak, out_dur, out_feasible):
 
 def moc_mem_profile(g, seq, want_free=True):
     """One device sequence -> (profile[int64], free[int32] or None, status[int32 tensor of 1])."""
-    import torch
+    r = _fast.mem_profile(g, seq, want_free)
+    if r is not None:
+        return r if r.__class__ is tuple else _check(r, "moc_mem_profile")
     T = seq.numel()
     profile = torch.empty(T, dtype=torch.int64, device=seq.device)
     free = torch.empty(T, dtype=torch.int32, device=seq.device) if want_free else None
@@ -282,7 +290,10 @@ def moc_last_launch_count():
 def moc_check_intervals(g, s, e, a, M, D, topo_index=None, want_seqs=True):
     """Device tensors s, e, a of shape [B, n, C] (int32) -> dict of device tensors mask, peak, dur and,
     with want_seqs, seqs [B, n*C] and lens."""
-    import torch
+    r = _fast.check_intervals(g, s, e, a, M, D, topo_index, want_seqs)
+    if r is not None:
+        _check(r if r.__class__ is int else MOC_OK, "moc_check_intervals")
+        return dict(zip(("mask", "peak", "dur", "seqs", "lens"), r))
     B, K = s.shape[0], s.shape[1] * s.shape[2]
     peak = torch.empty(B, dtype=torch.int64, device=s.device)
     dur = torch.empty(B, dtype=torch.int64, device=s.device)
@@ -301,7 +312,6 @@ def moc_check_intervals(g, s, e, a, M, D, topo_index=None, want_seqs=True):
 
 def moc_search_create(g, seqs, lens, M, seed, first_chain=0):
     """Device tensors (packed sequences, lengths) -> search handle; synchronous."""
-    import torch
     h = _P()
     rc = lib.moc_search_create(g, _dev(seqs, torch.int32, "seqs"), _dev(lens, torch.int32, "lens"), lens.numel(),
                                int(M), ctypes.c_uint64(int(seed)), ctypes.c_uint32(int(first_chain)), _stream(),
@@ -311,7 +321,8 @@ def moc_search_create(g, seqs, lens, M, seed, first_chain=0):
 
 
 def moc_search_run(s, n_generations):
-    _check(lib.moc_search_run(s, int(n_generations), _stream()), "moc_search_run")
+    r = _fast.search_run(s, n_generations)
+    _check(lib.moc_search_run(s, int(n_generations), _stream()) if r is None else r, "moc_search_run")
 
 
 MOC_EDIT_INSERT, MOC_EDIT_DELETE, MOC_EDIT_MOVE = 1, 2, 4
@@ -329,7 +340,10 @@ def moc_search_info(s):
 
 def moc_search_state(s, want_rows=True):
     """-> dict of device tensors: rows [P, stride] (or None), lens, peak, dur, status, accepted."""
-    import torch
+    r = _fast.search_state(s, want_rows)
+    if r is not None:
+        _check(r if r.__class__ is int else MOC_OK, "moc_search_state")
+        return dict(zip(("rows", "lens", "peak", "dur", "status", "accepted"), r))
     info = moc_search_info(s)
     P = info["P"]
     rows = torch.zeros((P, info["stride"]), dtype=torch.int32, device="cuda") if want_rows else None
@@ -348,7 +362,6 @@ def moc_search_state(s, want_rows=True):
 
 def moc_search_best(s, max_len):
     """-> (seq tensor of max_len ints on the device, out_best tensor of 6 int64 on the device)."""
-    import torch
     seq = torch.zeros(max_len, dtype=torch.int32, device="cuda")
     best = torch.empty(6, dtype=torch.int64, device="cuda")
     _check(lib.moc_search_best(s, ctypes.c_void_p(seq.data_ptr()), ctypes.c_void_p(best.data_ptr()), _stream()),
@@ -422,7 +435,6 @@ class Graph:
     def no_remat_peak(self):
         """Peak of the identity order 0..n-1 (the input topological order when ids are topological),
         the reference point for budgets given in percent (Section 4.3)."""
-        import torch
         seq = torch.arange(self.n, dtype=torch.int32, device="cuda")
         lens = torch.tensor([self.n], dtype=torch.int32, device="cuda")
         peak, _, st = self.eval_batch(seq, lens, (1 << 62))
@@ -467,7 +479,6 @@ class Search:
 
     def best(self):
         """-> dict(index, seq (numpy), peak, dur, status, accepted); synchronises."""
-        import torch
         seq, b = moc_search_best(self.h, self.graph.C * self.graph.n)
         torch.cuda.synchronize()
         b = b.cpu().numpy()
@@ -497,7 +508,9 @@ class EditCache:
 
     def build(self, seqs, lens, M):
         """Device tensors (packed parents) -> (peak, dur, status) device tensors of the parents."""
-        import torch
+        r = _fast.cache_build(self.h, seqs, lens, M)
+        if r is not None:
+            return r if r.__class__ is tuple else _check(r, "moc_cache_build")
         P = lens.numel()
         peak = torch.empty(P, dtype=torch.int64, device=lens.device)
         dur = torch.empty(P, dtype=torch.int64, device=lens.device)
@@ -511,7 +524,10 @@ class EditCache:
     def eval_edits(self, parent, op, q, j, M, out=None, window=None):
         """int32 device tensors of B edits -> (peak, dur, status) device tensors; window: optional int32
         device tensor that receives the number of recomputed steps per edit."""
-        import torch
+        if out is None and window is None:
+            r = _fast.eval_edits(self.h, parent, op, q, j, M)
+            if r is not None:
+                return r if r.__class__ is tuple else _check(r, "moc_eval_edits")
         B = parent.numel()
         if out is None:
             out = (torch.empty(B, dtype=torch.int64, device=parent.device), torch.empty(B, dtype=torch.int64, device=parent.device),

@@ -1,4 +1,5 @@
-"""Builds libmoc_b200.so (nvcc, sm_100a only) next to this file.  ``python -m paper_2304_14463_b200.build``"""
+"""Builds libmoc_b200.so (nvcc, sm_100a only) and _moc_torch.so (g++: the torch side of the binding)
+next to this file.  ``python -m paper_2304_14463_b200.build``"""
 from __future__ import annotations
 
 import os
@@ -14,16 +15,39 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-Xcompiler", "-fPIC", "-shared", "--use_fast_math"]
 
 
-def _stale():
-    if not os.path.exists(LIB):
+TORCH_LIB = os.path.join(HERE, "_moc_torch.so")
+TORCH_SOURCES = ["moc_torch.cpp", os.path.join("..", "..", "include", "moc.h")]
+
+
+def _stale(lib, files):
+    if not os.path.exists(lib):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in SOURCES + HEADERS] + [os.path.abspath(__file__)]
+    t = os.path.getmtime(lib)
+    deps = [os.path.join(CSRC, f) for f in files] + [os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_torch(force: bool = False) -> str:
+    if not force and not _stale(TORCH_LIB, TORCH_SOURCES):
+        return TORCH_LIB
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    lib_dirs = [os.path.join(os.path.dirname(torch.__file__), "lib")]
+    tmp = TORCH_LIB + f".{os.getpid()}.tmp"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    cmd += [f"-I{d}" for d in cpp_extension.include_paths("cuda") + [sysconfig.get_paths()["include"]]]
+    cmd += ["-o", tmp, os.path.join(CSRC, "moc_torch.cpp")]
+    cmd += [f for d in lib_dirs for f in (f"-L{d}", f"-Wl,-rpath,{d}")]
+    cmd += ["-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"]
+    subprocess.run(cmd, check=True)
+    os.replace(tmp, TORCH_LIB)
+    return TORCH_LIB
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not force and not _stale():
+    build_torch(force)
+    if not force and not _stale(LIB, SOURCES + HEADERS):
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     tmp = LIB + f".{os.getpid()}.tmp"
