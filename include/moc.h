@@ -333,8 +333,9 @@ int moc_search_create(const moc_graph* g, const int32_t* seqs, const int32_t* le
                       int64_t M, uint64_t seed, uint32_t first_chain, void* stream,
                       moc_search** out);
 
-/* Enqueues n_generations further generations on `stream` (asynchronous; two kernels per generation
- * plus one at the end, no allocation, no synchronisation).  Generations are numbered from 0 over
+/* Enqueues n_generations further generations on `stream` (asynchronous, no allocation, no
+ * synchronisation; one proposal per chain and C <= 2: one kernel for all generations of the call, a warp
+ * per chain; otherwise two kernels per generation plus one at the end, or as moc_search_set_samples says).  Generations are numbered from 0 over
  * the life of the handle; the result does not depend on how they are split over calls. */
 int moc_search_run(moc_search* s, int32_t n_generations, void* stream);
 
@@ -358,8 +359,7 @@ int moc_search_set_kinds(moc_search* s, uint32_t kinds);
  *                proposal with the smallest key among those with status >= 0, the lowest e among
  *                equals, and it replaces the chain's sequence when its key is not larger.  E = 1 is
  *                the single proposal described above.
- *   incremental  0 (MOC_SEARCH_WRITTEN_OUT): every proposal is written out and evaluated from scratch
- *                (E must be 1);
+ *   incremental  0 (MOC_SEARCH_WRITTEN_OUT): no cache; proposals are evaluated in full (E must be 1);
  *                1 (MOC_SEARCH_SCORE_AUTO): proposals are scored from the cached evaluation of the chain's
  *                sequence and only accepted ones are written out; the library picks the scoring kernel
  *                (a warp per chain from E = 24 on when the graph fits it, else the kernel of moc_eval_edits);

@@ -9,6 +9,7 @@
 #include "moc_cache_host.cuh"
 #include "moc_search_kernels.cuh"
 #include "moc_search_score_kernel.cuh"
+#include "moc_search_walk_kernel.cuh"
 
 using namespace moc_host;
 
@@ -34,6 +35,13 @@ struct moc_search {
     int score_wpb = 0, score_grid_cap = 0;
     const void* score_fn = nullptr;
     size_t score_smem = 0;
+    // all generations in one kernel, one proposal per chain (moc_search_walk_kernel.cuh)
+    uint64_t graph_generation = 0;     // the graph's C and caps when the chains were evaluated
+    moc::WalkParams wp{};
+    const void* walk_fn = nullptr;     // null: not planned yet, or the graph does not fit (walk_planned)
+    bool walk_planned = false;
+    int walk_wpb = 0, walk_grid = 0;
+    size_t walk_smem = 0;
 };
 
 namespace {
@@ -88,6 +96,57 @@ bool plan_fused(moc_search* s) {
     return true;
 }
 
+// Launch shape of the kernel that takes a warp per chain through all generations; leaves walk_fn null when the
+// graph has no warp-per-sequence layout (C > 2, very uneven degrees) or fewer than four warps fit an SM.
+void plan_walk(moc_search* s) {
+    s->walk_planned = true;
+    s->walk_fn = nullptr;
+    const moc_graph* g = s->g;
+    if (g->C > 2 || g->d_rec32 == nullptr) return;
+    const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    const size_t per_vec = wide ? 2 : 4, nvec = ((size_t)g->C * g->n + 2 + per_vec - 1) / per_vec, v_max = ((nvec + 31) / 32) | 1;
+    moc::WalkParams& w = s->wp;
+    w.n = g->n;
+    w.C = g->C;
+    w.n_tiles = g->n_tiles;
+    w.rec = wide ? g->d_rec64 : g->d_rec32;
+    w.sell = g->d_sell;
+    w.succ_start = g->d_succ_start;
+    w.succ = g->d_succ;
+    w.pred_start = g->d_pred_start;
+    w.pred = g->d_pred;
+    w.w = g->d_w;
+    w.rec_bytes = (wide ? 16u : 8u) * 64u * (uint32_t)g->n_tiles;
+    w.sell_bytes = (4u * (uint32_t)g->sell_len + 15u) & ~15u;
+    w.word_bytes = (4u * ((uint32_t)g->n + 2u) + 15u) & ~15u;
+    w.delta_bytes = (uint32_t)(moc::kPairDeltaFront + 32 * v_max * 16);
+    const size_t warp_b = moc::walk_warp_bytes(w.word_bytes, w.delta_bytes), graph_b = (size_t)w.rec_bytes + w.sell_bytes;
+    const void* fn = wide ? (const void*)moc::search_walk_kernel<int64_t> : (const void*)moc::search_walk_kernel<int32_t>;
+    const size_t cap = g->smem_optin;
+    if (graph_b + 4 * warp_b > cap) return;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    // Chains that fit the device at once get one round with as few warps per SM as that takes; larger
+    // populations the shape with the smallest rounds * warps (an SM's rate hardly depends on its warps beyond 16).
+    const int sm = g->sm_count, most = (int)std::min<size_t>(moc::kWalkThreads / 32, (cap - graph_b) / warp_b);
+    int best = 0;
+    int64_t best_cost = 0;
+    for (int k = most; k >= 1; --k) {
+        const int64_t rounds = ((int64_t)s->P + (int64_t)sm * k - 1) / ((int64_t)sm * k);
+        const int64_t cost = rounds * std::max(k, std::min(most, 16));
+        if (best == 0 || cost < best_cost || (cost == best_cost && rounds == 1)) { best = k; best_cost = cost; }
+    }
+    s->walk_wpb = best;
+    s->walk_grid = (int)std::min<int64_t>(sm, ((int64_t)s->P + best - 1) / best);
+    s->walk_smem = graph_b + (size_t)best * warp_b;
+    s->walk_fn = fn;
+}
+
+// Generations of one launch: long enough that the launch does not show, short enough for a caller who waits.
+constexpr int32_t kWalkGenerations = 4096;
+
 }  // namespace
 
 extern "C" {
@@ -115,6 +174,7 @@ int moc_search_create(const moc_graph* g, const int32_t* seqs, const int32_t* le
     s->stride = (int32_t)stride;
     s->M = M;
     s->seed = seed;
+    s->graph_generation = g->generation;
     const size_t bP = (size_t)P;
     const size_t o_rows = 0, o_offs = o_rows + up256(2 * bP * (size_t)stride * 4), o_peak = o_offs + up256((bP + 1) * 8),
                  o_dur = o_peak + up256(bP * 8), o_cpeak = o_dur + up256(bP * 8), o_cdur = o_cpeak + up256(bP * 8),
@@ -230,6 +290,25 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
             launches += 4;
         }
         MOC_CUDA(cudaGetLastError());
+        s->generation += (uint32_t)n_generations;
+        launch_counter() = launches;
+        return MOC_OK;
+    }
+    // The walk kernel relies on the chains' evaluations: not after a change of the graph's C or caps, and not
+    // when the caller chose another evaluation kernel for the graph.
+    const moc_graph* g = s->g;
+    if (!s->walk_planned) plan_walk(s);
+    if (s->walk_fn && g->generation == s->graph_generation && g->want_G == 0 &&
+        (g->want_kind == MOC_KERNEL_AUTO || g->want_kind == MOC_KERNEL_WARP)) {
+        for (int32_t k = 0; k < n_generations; k += kWalkGenerations) {
+            s->wp.s = p;
+            s->wp.s.generation = s->generation + (uint32_t)k;
+            s->wp.n_gen = std::min(kWalkGenerations, n_generations - k);
+            s->wp.cap = g->d_cap;
+            void* args[] = {&s->wp};
+            MOC_CUDA(cudaLaunchKernel(s->walk_fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, s->walk_smem, st));
+            ++launches;
+        }
         s->generation += (uint32_t)n_generations;
         launch_counter() = launches;
         return MOC_OK;

@@ -1,0 +1,358 @@
+// The search with one proposal per chain and generation (paper: Section 3, the two-phase local search),
+// all generations of a call in one kernel.  The chains are independent, so a warp takes its chain through
+// every generation of the launch with the chain's copy positions in shared memory; nothing is exchanged
+// between warps.  C <= 2 and graphs of the warp-per-sequence layout (moc_pair_kernel.cuh).
+//
+// What a generation costs.  About four proposals of five are refused by a test on the edited node alone
+// (copy count, Eq. 5 on the edges that touch the node).  Lane k therefore draws and tests the proposal
+// of generation base + k, 32 generations at a time against the chain's present sequence, and the warp
+// evaluates only the admissible ones, in order.  An accepted one changes the sequence: the generations
+// behind it are tested again (a draw does not depend on the sequence, only its reading does).
+// An admissible proposal is evaluated in full, but not from its sequence: the copy positions of the edited
+// sequence are the parent's, shifted by at most one step, which is two packed instructions per word, so that
+// the occurrence pass of the evaluation kernel (data-dependent exchanges) falls away.  A proposal that
+// cannot be accepted whatever its peak (longer duration while the chain is within the budget) is not
+// evaluated: the key of the chain decides already.
+//
+// The sequence itself stays in global memory (L2): the tests read one element per proposal, and an
+// accepted edit shifts the elements between its two places by one.  It is kept there because 3.5 KB per warp
+// less (n = 442) let 28 warps share an SM instead of 22.
+//
+// Chains without a valid sequence (status < 0) have no test to rely on: their proposals are evaluated from
+// the written-out order, one generation at a time, until one is valid.
+//
+// Bound: instruction issue and the shared-memory data pipe, like the evaluation kernel, on a fifth of the
+// proposals.  n = 442, 4096 chains, 20 generations with the copy-out of the chains' state: 436 -> 67.7 us
+// against two kernels per generation that write every proposal out and evaluate it.
+#pragma once
+#include "moc_edit_kernels.cuh"
+#include "moc_search_kernels.cuh"
+
+namespace moc {
+
+constexpr int kWalkThreads = 896;     // 28 warps, 72 registers per thread
+
+struct WalkParams {
+    SearchParams s;            // s.generation: number of the first generation
+    int32_t n_gen;             // generations of this launch
+    int32_t n, C, n_tiles;
+    const void* rec;           // node records and successor tiles of the warp-per-sequence layout
+    const uint32_t* sell;
+    const int32_t* succ_start;
+    const int32_t* succ;
+    const int32_t* pred_start;
+    const int32_t* pred;
+    const int64_t* w;
+    const int32_t* cap;        // per-node caps or nullptr
+    uint32_t rec_bytes, sell_bytes;      // graph, once per block
+    uint32_t word_bytes;       // occurrence words (n + 2, padded) without the constant word behind them
+    uint32_t delta_bytes;      // front pad + deltas for C * n steps
+};
+
+// Bytes of one warp: two sets of words, each followed by the constant word, and the deltas.
+__host__ __device__ inline size_t walk_warp_bytes(uint32_t word_bytes, uint32_t delta_bytes) {
+    return 2 * ((size_t)word_bytes + kPairWordTail) + delta_bytes;
+}
+
+// [p > k] per 16-bit half (p, k < 2^15): max(min(p - k, 1), 0).
+__device__ __forceinline__ uint32_t walk_above(uint32_t p, uint32_t k) {
+    return __viaddmin_s16x2_relu(p, ((0x00010000u - k) & 0xFFFFu) * 0x10001u, 0x00010001u);
+}
+
+// Stages 2 to 4 of the evaluation (moc_pair_kernel.cuh) on the occurrence words at `wa`: the peak, and
+// whether a consumer lacks a producer copy.  The deltas are zero on entry and on return.
+template <typename MemT>
+__device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec0, uint32_t sell0, int n_tiles, int32_t T, int lane,
+                                          bool& dep) {
+    constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
+    constexpr int kPerVec = 16 / (int)sizeof(MemT), kShift = sizeof(MemT) == 4 ? 2 : 3;
+    const uint32_t da1 = da - (uint32_t)sizeof(MemT);
+    uint32_t depw = 0, prec = rec0, ps = sell0;
+    for (int d = 0; d < n_tiles; ++d, prec += 64u * kRecB) {
+        uint32_t ab[2], naa[2], nbb[2], Ga[2], Gb[2];
+        MemT m[2];
+        int rows = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t x;
+            if constexpr (sizeof(MemT) == 4) {
+                const uint2 r = lds_v2(prec + 32u * kRecB * h);
+                x = r.x;
+                m[h] = (MemT)r.y;
+            } else {
+                const uint4 r = lds_v4(prec + 32u * kRecB * h);
+                x = r.x;
+                m[h] = (MemT)((uint64_t)r.z | ((uint64_t)r.w << 32));
+            }
+            if (h == 0) rows = (int)(x >> 16);
+            const uint32_t own = lds_u32(wa + (x & 0xFFFFu)), sw = swap_halves(own);
+            const uint32_t mn = min_u16x2(own, sw), mx = max_u16x2(own, sw);
+            ab[h] = __byte_perm(mn, mx, 0x7610);
+            naa[h] = 0x00010000u - mn;
+            nbb[h] = 0x00010000u - mx;
+            Ga[h] = mx - mn;
+            Gb[h] = 0x00010000u - Ga[h];
+        }
+        rows = __shfl_sync(kFull, rows, 0);
+#pragma unroll 2
+        for (int k = 0; k < rows; ++k) {
+            const uint32_t e = lds_u32(ps);
+            ps += 128u;
+            const uint32_t r0 = lds_u32(wa + (e & 0xFFFFu)), r1 = lds_u32(wa + (e >> 16));
+            Ga[0] = __viaddmax_u16x2(r0, naa[0], Ga[0]);
+            Ga[1] = __viaddmax_u16x2(r1, naa[1], Ga[1]);
+            Gb[0] = __viaddmax_u16x2(r0, nbb[0], Gb[0]);
+            Gb[1] = __viaddmax_u16x2(r1, nbb[1], Gb[1]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            depw |= Ga[h];
+            const uint32_t gg = max_u16x2(__byte_perm(Ga[h], Gb[h], 0x5410), __byte_perm(Ga[h], Gb[h], 0x7632));
+            const uint32_t v = gg + ab[h], a16 = ab[h] & 0xFFFFu, b16 = ab[h] >> 16;
+            red_add_shared(da1 + (b16 << kShift), m[h]);
+            red_add_shared(da + ((v & 0xFFFFu) << kShift), (MemT)-m[h]);
+            if (a16 != b16) {
+                red_add_shared(da1 + (a16 << kShift), m[h]);
+                red_add_shared(da + ((v >> 16) << kShift), (MemT)-m[h]);
+            }
+        }
+    }
+    dep = __any_sync(kFull, (depw & 0x80008000u) != 0);
+    __syncwarp();
+    // prefix sum and running maximum; lane owns V consecutive vectors, which it clears behind itself
+    const int nvec = (T + 2 + kPerVec - 1) / kPerVec, V = ((nvec + 31) >> 5) | 1;
+    uint32_t ad = da + 16u * (uint32_t)(lane * V);
+    MemT run = 0, top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
+    for (int j = 0; j < V; ++j, ad += 16u) {
+        const uint4 q = lds_v4(ad);
+        asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(ad), "r"(0) : "memory");
+        if constexpr (sizeof(MemT) == 4) {
+            run += (MemT)q.x; top = max(top, run);
+            run += (MemT)q.y; top = max(top, run);
+            run += (MemT)q.z; top = max(top, run);
+            run += (MemT)q.w; top = max(top, run);
+        } else {
+            run += (MemT)((uint64_t)q.x | (uint64_t)q.y << 32); top = run > top ? run : top;
+            run += (MemT)((uint64_t)q.z | (uint64_t)q.w << 32); top = run > top ? run : top;
+        }
+    }
+    const MemT peak = warp_max_t((MemT)(warp_inclusive_sum(run, lane) - run + top));
+    __syncwarp();
+    return peak;
+}
+
+// Shifts row[a..b) by one place to the left (dir = -1) or to the right (dir = 1) with the lanes of a warp.
+__device__ __forceinline__ void walk_shift(int32_t* row, int32_t a, int32_t b, int dir, int lane) {
+    for (int32_t done = 0; done < b - a; done += 256) {
+        int32_t v[8];
+        // ascending pieces to the left, descending pieces to the right: no element is overwritten unread
+        const int32_t base = dir < 0 ? a + done : b - done - 256;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int32_t i = base + lane + 32 * k;
+            if (i >= a && i < b) v[k] = row[i];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int32_t i = base + lane + 32 * k;
+            if (i >= a && i < b) row[i + dir] = v[k];
+        }
+        __syncwarp();
+    }
+}
+
+// Element qd taken out of row[0..T) (none: kEditNone), then x put in front of index ji of what is left (none:
+// kEditNone), in place.
+__device__ __forceinline__ void walk_apply(int32_t* row, int32_t T, int32_t qd, int32_t ji, int32_t x, int lane) {
+    if (qd == kEditNone) walk_shift(row, ji, T, 1, lane);
+    else if (ji == kEditNone) walk_shift(row, qd + 1, T, -1, lane);
+    else if (ji >= qd) walk_shift(row, qd + 1, ji + 1, -1, lane);
+    else walk_shift(row, ji, qd, 1, lane);
+    if (ji != kEditNone && lane == 0) row[ji] = x;
+    __syncwarp();
+}
+
+template <typename MemT>
+__global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const WalkParams p) {
+    extern __shared__ __align__(16) char smem[];
+    const SearchParams& s = p.s;
+    constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    {
+        int4* s4 = reinterpret_cast<int4*>(smem);
+        const uint32_t n_rec = p.rec_bytes >> 4, n_all = (p.rec_bytes + p.sell_bytes) >> 4;
+        for (uint32_t i = threadIdx.x; i < n_all; i += blockDim.x)
+            s4[i] = i < n_rec ? __ldg(reinterpret_cast<const int4*>(p.rec) + i) : __ldg(reinterpret_cast<const int4*>(p.sell) + (i - n_rec));
+    }
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
+    const uint32_t word_set = p.word_bytes + kPairWordTail;
+    const uint32_t mine = sbase + p.rec_bytes + p.sell_bytes + (uint32_t)warp * (2u * word_set + p.delta_bytes);
+    const uint32_t da = mine + 2u * word_set + kPairDeltaFront;      // &delta[0]
+    const uint32_t rec0 = sbase + kRecB * (uint32_t)lane, sell0 = sbase + p.rec_bytes + 4u * (uint32_t)lane;
+    const int n = p.n, n_tiles = p.n_tiles;
+    if (lane < 2) sts_u32(mine + word_set * (uint32_t)lane + p.word_bytes, 0x00010001u);   // owned by empty node slots
+    for (uint32_t o = 16u * (uint32_t)lane; o < p.delta_bytes; o += 512u)
+        asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(da - kPairDeltaFront + o), "r"(0) : "memory");
+    __syncthreads();
+
+    for (int32_t c = blockIdx.x * wpb + warp; c < s.P; c += gridDim.x * wpb) {
+        int32_t* row = s.rows + ((int64_t)s.cur[c] * s.P + c) * s.stride;
+        int32_t T = s.lens[c], st = s.status[c], n_acc = 0;
+        int64_t pk = s.peak[c], du = s.dur[c];
+        uint32_t wa = mine, wb = mine + word_set;       // the chain's words, and those of a proposal
+        // occurrence words of the edited row (qd = ji = kEditNone: the row itself) by exchanges, as in the
+        // evaluation kernel; returns the summed durations of the lane's elements.  Invalid ids go to the spare word n.
+        auto words_of = [&](uint32_t w0, int32_t Tc, int32_t qd, int32_t ji, int32_t x) -> int64_t {
+            for (uint32_t o = 16u * (uint32_t)lane; o < p.word_bytes; o += 512u)
+                asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(w0 + o), "r"(0) : "memory");
+            __syncwarp();
+            int64_t sum = 0;
+            for (int32_t t = lane; t < Tc; t += 32) {
+                int32_t v = x;
+                if (t != ji) {
+                    const int32_t k = t - (t > ji ? 1 : 0);
+                    v = row[k + (k >= qd ? 1 : 0)];
+                }
+                if ((uint32_t)v < (uint32_t)n) sum += __ldg(p.w + v);
+                const uint32_t addr = w0 + 4u * min((uint32_t)v, (uint32_t)n);
+                const uint32_t old = exch_shared(addr, ((uint32_t)t + 1u) * 0x10001u);
+                sts_u16_if_nonzero(old, addr + 2, old);
+            }
+            __syncwarp();
+            if (lane == 0) sts_u32(w0 + 4u * (uint32_t)(n + 1), (uint32_t)Tc * 0x10001u);
+            __syncwarp();
+            return sum;
+        };
+        if (st >= 0) words_of(wa, T, kEditNone, kEditNone, 0);
+
+        for (int32_t g0 = 0; g0 < p.n_gen; g0 += 32) {
+            const uint4 r = philox4x32_10(make_uint4(s.generation + (uint32_t)(g0 + lane), s.chain0 + (uint32_t)c, 0u, 0u),
+                                          make_uint2(s.seed_lo, s.seed_hi));
+            const int32_t op = (int32_t)search_pick_kind(s.kinds, r.x);
+            uint32_t pending = p.n_gen - g0 >= 32 ? kFull : (1u << (p.n_gen - g0)) - 1u;
+            while (pending && T > 0) {
+                // ---- the pending generations against the present sequence, a lane each
+                const bool live = (pending >> lane & 1u) != 0;
+                const int32_t q = (int32_t)(r.y % (uint32_t)T);
+                const int32_t j = op == 0 ? (int32_t)(r.z % ((uint32_t)T + 1u)) : (int32_t)(r.z % (uint32_t)T);
+                const int32_t qd = op >= 1 ? q : kEditNone, ji = op != 1 ? j : kEditNone;
+                const int32_t Tc = T + (op == 0 ? 1 : 0) - (op == 1 ? 1 : 0);
+                const int32_t x = row[q];
+                bool adm = live && Tc >= n && Tc <= s.max_T;
+                uint32_t wx_new = 0;        // the edited node's word after the edit
+                int64_t du_c = 0;
+                if (adm && st >= 0) {
+                    const uint32_t wx = lds_u32(wa + 4u * (uint32_t)x);
+                    const int32_t xa = (int32_t)min(wx & 0xFFFFu, wx >> 16) - 1, xb = (int32_t)max(wx & 0xFFFFu, wx >> 16) - 1;
+                    const int32_t cnt = xa == xb ? 1 : 2, cnt2 = cnt - (op >= 1 ? 1 : 0) + (op != 1 ? 1 : 0);
+                    adm = cnt2 == 1 || (cnt2 == 2 && p.C >= 2 && (p.cap == nullptr || __ldg(p.cap + x) >= 2));
+                    if (adm) {
+                        auto map = [&](int32_t t) -> int32_t { const int32_t t1 = t - (t > qd ? 1 : 0); return t1 + (t1 >= ji ? 1 : 0); };
+                        // first child copy c0 (and c1), with the parent steps of other nodes' copies that lie in front
+                        // of c0 (r < tb0) and behind it (r > ta0), 1-based, as in moc_edit_pass.cuh
+                        int32_t c0 = kEditNone, c1 = kEditNone, ta0 = 0, tb0 = 0;
+                        auto push = [&](int32_t cs, int32_t ta, int32_t tb) {
+                            if (c0 == kEditNone) { c0 = cs; ta0 = ta; tb0 = tb; }
+                            else if (cs < c0) { c1 = c0; c0 = cs; ta0 = ta; tb0 = tb; }
+                            else { c1 = cs; }
+                        };
+                        if (xa != qd) push(map(xa), xa + 1, xa + 1);
+                        if (cnt == 2 && xb != qd) push(map(xb), xb + 1, xb + 1);
+                        if (ji != kEditNone) { const int32_t thr = ji + (ji >= qd ? 1 : 0); push(ji, thr, thr + 1); }
+                        wx_new = (uint32_t)(c0 + 1) | (uint32_t)((c1 == kEditNone ? c0 : c1) + 1) << 16;
+                        du_c = du + __ldg(p.w + x) * (cnt2 - cnt);
+                        // within the budget only the duration decides
+                        adm = pk > s.M || du_c <= du;
+                        if (adm) {
+                            bool viol = false;
+                            const int32_t p0 = __ldg(p.pred_start + x), p1 = __ldg(p.pred_start + x + 1);
+                            const int32_t s0 = __ldg(p.succ_start + x), s1 = __ldg(p.succ_start + x + 1);
+#pragma unroll 1
+                            for (int32_t k = p0; k < p1; ++k) {
+                                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.pred + k));
+                                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) > ta0;
+                            }
+#pragma unroll 1
+                            for (int32_t k = s0; k < s1; ++k) {
+                                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.succ + k));
+                                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) < tb0;
+                            }
+                            adm = !viol;
+                        }
+                    }
+                }
+                // ---- the admissible ones in order, until one is accepted
+                uint32_t todo = __ballot_sync(kFull, adm);
+                pending = 0;
+                while (todo) {
+                    const int sl = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    const int32_t qd_s = __shfl_sync(kFull, qd, sl), ji_s = __shfl_sync(kFull, ji, sl), x_s = __shfl_sync(kFull, x, sl);
+                    const int32_t Tc_s = __shfl_sync(kFull, Tc, sl);
+                    int64_t du_s = __shfl_sync(kFull, du_c, sl), pk_s = -1;
+                    bool valid = true, dep;
+                    if (st >= 0) {
+                        // words of the edited sequence: out with step qd, in at index ji
+                        const uint32_t kq = qd_s == kEditNone ? 0x7FFFu : (uint32_t)qd_s + 1u, kj = ji_s == kEditNone ? 0x7FFFu : (uint32_t)ji_s;
+                        const uint32_t wx_s = __shfl_sync(kFull, wx_new, sl);
+                        for (uint32_t o = 16u * (uint32_t)lane; o < p.word_bytes; o += 512u) {
+                            uint4 v = lds_v4(wa + o);
+                            v.x -= walk_above(v.x, kq); v.x += walk_above(v.x, kj);
+                            v.y -= walk_above(v.y, kq); v.y += walk_above(v.y, kj);
+                            v.z -= walk_above(v.z, kq); v.z += walk_above(v.z, kj);
+                            v.w -= walk_above(v.w, kq); v.w += walk_above(v.w, kj);
+                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(wb + o), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+                        }
+                        __syncwarp();
+                        if (lane == 0) {
+                            sts_u32(wb + 4u * (uint32_t)x_s, wx_s);
+                            sts_u32(wb + 4u * (uint32_t)(n + 1), (uint32_t)Tc_s * 0x10001u);
+                        }
+                        __syncwarp();
+                    } else {
+                        // from scratch: every node present, as many second copies as steps beyond n, caps
+                        du_s = warp_sum64(words_of(wb, Tc_s, qd_s, ji_s, x_s));
+                        uint32_t two = 0;
+                        bool bad = false;
+                        for (int32_t v = lane; v < n; v += 32) {
+                            const uint32_t wv = lds_u32(wb + 4u * (uint32_t)v);
+                            const bool t2 = (wv & 0xFFFFu) != wv >> 16;
+                            two += t2 ? 1u : 0u;
+                            bad |= wv == 0 || (t2 && (p.C < 2 || (p.cap != nullptr && __ldg(p.cap + v) < 2)));
+                        }
+                        two = __reduce_add_sync(kFull, two);
+                        valid = !__any_sync(kFull, bad) && (int32_t)two == Tc_s - n;
+                    }
+                    if (!valid) continue;
+                    pk_s = (int64_t)walk_eval<MemT>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, dep);
+                    if (dep || !search_not_worse(pk_s, du_s, 1, pk, du, st, s.M)) continue;
+                    walk_apply(row, T, qd_s, ji_s, x_s, lane);
+                    const uint32_t sw = wa;
+                    wa = wb;
+                    wb = sw;
+                    T = Tc_s;
+                    pk = pk_s;
+                    du = du_s;
+                    st = pk <= s.M ? 1 : 0;
+                    ++n_acc;
+                    // the generations behind this one see the new sequence
+                    pending = sl == 31 ? 0u : (kFull << (sl + 1)) & (p.n_gen - g0 >= 32 ? kFull : (1u << (p.n_gen - g0)) - 1u);
+                    break;
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0 && n_acc) {
+            s.lens[c] = T;
+            s.peak[c] = pk;
+            s.dur[c] = du;
+            s.status[c] = st;
+            s.n_acc[c] += n_acc;
+        }
+        __syncwarp();
+    }
+}
+
+}  // namespace moc

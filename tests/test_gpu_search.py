@@ -156,6 +156,34 @@ def test_search_restricted_kinds(B, kinds):
         S.set_kinds(8)
 
 
+@pytest.mark.parametrize("n,scale,caps,P,gens", [(1, 1, False, 3, (1, 40)), (5, 1, False, 33, (31, 1, 33)), (63, 1, True, 200, (32, 70)),
+                                                 (65, 1 << 26, False, 7, (64, 3)), (442, 1 << 26, True, 149, (33,)), (2000, 1, False, 5, (32, 9))])
+def test_search_walk_edges(B, n, scale, caps, P, gens):
+    """All generations in one kernel: counts around the 32 draws a warp tests at once, graphs around the 64 node
+    slots of a tile, per-node caps, 64-bit sums, chains that start invalid, fewer and more chains than SMs."""
+    rs = np.random.RandomState(n)
+    edges = [] if n == 1 else W.layered_dag(n, min(2 * n, n * (n - 1) // 4), max(2, min(10, n // 4)), n)
+    w, m = W.weights_uniform(n, 0, 9, n, 1), W.weights_lognormal(n, 5.0, 1.5, n, 2) * scale
+    seqs, lens = W.schedules(n, edges, 2, 0.3, P, n)
+    if n > 1:
+        seqs, lens = W.mutate(seqs, lens, n, 1, seed=5, frac=1 / 6)
+    keep = [r for r in W.unpack(seqs, lens) if len(r) <= 2 * n]
+    seqs, lens = W.pack(keep)
+    cap = rs.randint(1, 3, n).astype(np.int32) if caps else None
+    G, O = B.Graph(n, edges, w, m, 2), OracleGraph(n, edges, w, m, 2)
+    if caps:
+        G.set_caps(cap)
+        O.set_caps(cap)
+    M = OracleGraph(n, edges, w, m, 2).eval(np.arange(n), 1 << 62)["peak"] * 85 // 100
+    S = B.Search(G, dev(seqs), dev(lens), M, 99)
+    OS = OracleSearch(O, seqs, lens, M, 99, stride=S.info()["stride"])
+    for g in gens:
+        S.run(g)
+        assert B.moc_last_launch_count() == 1
+        OS.run(g)
+        assert_state_equal(S, OS, f"n {n} after {OS.generation} generations")
+
+
 def test_search_full_size(B):
     """The benchmark's shape: the headline graph with 16384 chains, every chain compared."""
     wl = W.make(2, seed=1)
