@@ -422,24 +422,27 @@ int moc_search_set_samples(moc_search* s, int32_t samples, int32_t incremental) 
     return MOC_OK;
 }
 
-int moc_search_state(const moc_search* s, int32_t* out_rows, int32_t* out_lens, int64_t* out_peak,
-                     int64_t* out_dur, int32_t* out_status, int32_t* out_accepted, void* stream) {
+static int export_state(const moc_search* s, int32_t* out_rows, bool fill, int32_t* out_lens, int64_t* out_peak, int64_t* out_dur,
+                        int32_t* out_status, int32_t* out_accepted, void* stream) {
     clear_error();
     if (!s) return fail(MOC_ERR_ARG, "moc_search_state: null handle");
     DeviceGuard dg(s->device);
     if (!dg.ok) return fail(MOC_ERR_CUDA, "cannot select device %d", s->device);
-    cudaStream_t st = (cudaStream_t)stream;
-    const size_t bP = (size_t)s->P;
-    if (out_rows) {
-        moc::search_export_kernel<<<chain_blocks(s->P), moc::kSearchThreads, 0, st>>>(s->p, out_rows);
-        MOC_CUDA(cudaGetLastError());
-    }
-    if (out_lens) MOC_CUDA(cudaMemcpyAsync(out_lens, s->p.lens, bP * 4, cudaMemcpyDeviceToDevice, st));
-    if (out_peak) MOC_CUDA(cudaMemcpyAsync(out_peak, s->p.peak, bP * 8, cudaMemcpyDeviceToDevice, st));
-    if (out_dur) MOC_CUDA(cudaMemcpyAsync(out_dur, s->p.dur, bP * 8, cudaMemcpyDeviceToDevice, st));
-    if (out_status) MOC_CUDA(cudaMemcpyAsync(out_status, s->p.status, bP * 4, cudaMemcpyDeviceToDevice, st));
-    if (out_accepted) MOC_CUDA(cudaMemcpyAsync(out_accepted, s->p.n_acc, bP * 4, cudaMemcpyDeviceToDevice, st));
+    moc::search_export_kernel<<<chain_blocks(s->P), moc::kSearchThreads, 0, (cudaStream_t)stream>>>(
+        s->p, out_rows, fill, out_lens, out_peak, out_dur, out_status, out_accepted);
+    MOC_CUDA(cudaGetLastError());
     return MOC_OK;
+}
+
+int moc_search_state(const moc_search* s, int32_t* out_rows, int32_t* out_lens, int64_t* out_peak,
+                     int64_t* out_dur, int32_t* out_status, int32_t* out_accepted, void* stream) {
+    return export_state(s, out_rows, false, out_lens, out_peak, out_dur, out_status, out_accepted, stream);
+}
+
+// For the torch side of the binding: the whole of out_rows is written, zeros behind the sequences.
+int moc_search_state_filled(const moc_search* s, int32_t* out_rows, int32_t* out_lens, int64_t* out_peak,
+                            int64_t* out_dur, int32_t* out_status, int32_t* out_accepted, void* stream) {
+    return export_state(s, out_rows, true, out_lens, out_peak, out_dur, out_status, out_accepted, stream);
 }
 
 int moc_search_best(const moc_search* s, int32_t* out_seq, int64_t* out_best, void* stream) {

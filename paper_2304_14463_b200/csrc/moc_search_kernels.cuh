@@ -285,16 +285,47 @@ __global__ void search_offsets_kernel(const SearchParams p) {
     if (c == 0) p.c_offs[p.P] = (int64_t)2 * p.P * p.stride;
 }
 
-// Copies every chain's current sequence to out_rows (P rows of `stride` ints; only the first
-// lens[c] entries of a row are written).  One warp per chain.
-__global__ void __launch_bounds__(kSearchThreads) search_export_kernel(const SearchParams p, int32_t* __restrict__ out_rows) {
+// Copies the chains' state out: the current sequences to out_rows (P rows of `stride` ints; entries behind a
+// row's length are left alone, or zeroed with `fill`, in the same pass: the caller need not clear 4 * P * stride
+// bytes first) and the evaluations.  Any output may be null.  One warp per chain; 16-byte accesses (rows start
+// on 16-byte boundaries when out_rows does).
+__global__ void __launch_bounds__(kSearchThreads) search_export_kernel(const SearchParams p, int32_t* __restrict__ out_rows, bool fill,
+                                                                       int32_t* __restrict__ out_lens, int64_t* __restrict__ out_peak,
+                                                                       int64_t* __restrict__ out_dur, int32_t* __restrict__ out_status,
+                                                                       int32_t* __restrict__ out_acc) {
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * (kSearchThreads / 32) + (threadIdx.x >> 5);
     if (c >= p.P) return;
     const int32_t T = p.lens[c];
+    if (lane == 0) {
+        if (out_lens) out_lens[c] = T;
+        if (out_peak) out_peak[c] = p.peak[c];
+        if (out_dur) out_dur[c] = p.dur[c];
+        if (out_status) out_status[c] = p.status[c];
+        if (out_acc) out_acc[c] = p.n_acc[c];
+    }
+    if (!out_rows) return;
     const int32_t* src = p.rows + ((int64_t)p.cur[c] * p.P + c) * p.stride;
     int32_t* dst = out_rows + (int64_t)c * p.stride;
-    for (int32_t i = lane; i < T; i += 32) dst[i] = src[i];
+    if ((reinterpret_cast<uintptr_t>(out_rows) & 15) == 0) {
+        const int4* s4 = reinterpret_cast<const int4*>(src);
+        int4* d4 = reinterpret_cast<int4*>(dst);
+        const int32_t nv = (fill ? p.stride : T) >> 2;            // the stride is a multiple of 4
+        for (int32_t i = lane; i < nv; i += 32) {
+            int4 v = make_int4(0, 0, 0, 0);
+            if (4 * i < T) {
+                v = s4[i];
+                if (4 * i + 1 >= T) v.y = 0;
+                if (4 * i + 2 >= T) v.z = 0;
+                if (4 * i + 3 >= T) v.w = 0;
+            }
+            d4[i] = v;
+        }
+        if (!fill)
+            for (int32_t i = (T & ~3) + lane; i < T; i += 32) dst[i] = src[i];
+        return;
+    }
+    for (int32_t i = lane; i < (fill ? p.stride : T); i += 32) dst[i] = i < T ? src[i] : 0;
 }
 
 // Best chain: smallest key (max(peak, M), duration) among the chains with status >= 0, lowest

@@ -30,7 +30,7 @@ decltype(&moc_check_intervals) f_check_intervals;
 decltype(&moc_cache_build) f_cache_build;
 decltype(&moc_eval_edits) f_eval_edits;
 decltype(&moc_search_run) f_search_run;
-decltype(&moc_search_state) f_search_state;
+decltype(&moc_search_state) f_search_state_filled;   // writes the whole rows, zeros behind the sequences
 decltype(&moc_search_info) f_search_info;
 
 PyObject* s_value;   // interned "value" (the pointer in a ctypes.c_void_p)
@@ -286,10 +286,9 @@ PyObject* py_search_state(PyObject*, PyObject* const* a, Py_ssize_t na) {
                          st = empty({P}, at::kInt, d), acc = empty({P}, at::kInt, d);
         if (want) {
             rows = empty({P, stride}, at::kInt, d);
-            rows.zero_();
         }
         const int rc = unlocked([&] {
-            return f_search_state((const moc_search*)s, want ? ptr<int32_t>(rows) : nullptr, ptr<int32_t>(lens), ptr<int64_t>(pk),
+            return f_search_state_filled((const moc_search*)s, want ? ptr<int32_t>(rows) : nullptr, ptr<int32_t>(lens), ptr<int64_t>(pk),
                                   ptr<int64_t>(du), ptr<int32_t>(st), ptr<int32_t>(acc), cs);
         });
         if (rc != MOC_OK) return PyLong_FromLong(rc);
@@ -316,7 +315,7 @@ PyObject* py_bind(PyObject*, PyObject* d) {
     MOC_BIND(cache_build);
     MOC_BIND(eval_edits);
     MOC_BIND(search_run);
-    MOC_BIND(search_state);
+    MOC_BIND(search_state_filled);
     MOC_BIND(search_info);
 #undef MOC_BIND
     Py_RETURN_NONE;
