@@ -35,11 +35,12 @@ struct moc_search {
     int score_wpb = 0, score_grid_cap = 0;
     const void* score_fn = nullptr;
     size_t score_smem = 0;
-    // all generations in one kernel, one proposal per chain (moc_search_walk_kernel.cuh)
+    // all generations of a call in one kernel (moc_search_walk_kernel.cuh)
     uint64_t graph_generation = 0;     // the graph's C and caps when the chains were evaluated
     moc::WalkParams wp{};
     const void* walk_fn = nullptr;     // null: not planned yet, or the graph does not fit (walk_planned)
     bool walk_planned = false;
+    bool walk_scores = false;          // incremental, and the walk kernel does it (no cache)
     int walk_wpb = 0, walk_grid = 0;
     size_t walk_smem = 0;
 };
@@ -144,8 +145,8 @@ void plan_walk(moc_search* s) {
     s->walk_fn = fn;
 }
 
-// Generations of one launch: long enough that the launch does not show, short enough for a caller who waits.
-constexpr int32_t kWalkGenerations = 4096;
+// Proposals per chain of one launch: enough that the launch does not show, few enough for a caller who waits.
+constexpr int32_t kWalkProposals = 4096;
 
 }  // namespace
 
@@ -180,7 +181,7 @@ int moc_search_create(const moc_graph* g, const int32_t* seqs, const int32_t* le
                  o_dur = o_peak + up256(bP * 8), o_cpeak = o_dur + up256(bP * 8), o_cdur = o_cpeak + up256(bP * 8),
                  o_cur = o_cdur + up256(bP * 8), o_lens = o_cur + up256(bP * 4), o_st = o_lens + up256(bP * 4),
                  o_acc = o_st + up256(bP * 4), o_clens = o_acc + up256(bP * 4), o_cst = o_clens + up256(bP * 4),
-                 o_bad = o_cst + up256(bP * 4), total = o_bad + 256;
+                 o_bad = o_cst + up256(bP * 4), o_at = o_bad + 256, total = o_at + up256(bP * 4);
     cudaError_t e = cudaMalloc((void**)&s->d_block, total);
     if (e != cudaSuccess) {
         delete s;
@@ -211,10 +212,11 @@ int moc_search_create(const moc_graph* g, const int32_t* seqs, const int32_t* le
     p.c_lens = (int32_t*)(b + o_clens);
     p.c_status = (int32_t*)(b + o_cst);
     s->d_bad = (int32_t*)(b + o_bad);
+    s->wp.peak_at = (int32_t*)(b + o_at);
     int rc = MOC_OK;
     int32_t bad = 0;
     auto run = [&]() -> int {
-        MOC_CUDA(cudaMemsetAsync(s->d_bad, 0, 4, st));
+        MOC_CUDA(cudaMemsetAsync(s->d_bad, 0, 256 + bP * 4, st));      // with the peaks' places behind it: not known
         // packed offsets of the caller's sequences, then the rows, then their evaluation
         moc::offsets_kernel<<<(P + moc::kOffsTile - 1) / moc::kOffsTile, moc::kOffsThreads, 0, st>>>(lens, P, p.c_offs);
         moc::search_init_kernel<<<chain_blocks(P), moc::kSearchThreads, 0, st>>>(p, seqs, lens, p.c_offs, s->d_bad);
@@ -251,6 +253,34 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
     moc::SearchParams& p = s->p;
     const int blocks = chain_blocks(s->P);
     int launches = 0;
+    // The walk kernel relies on the chains' evaluations: not after a change of the graph's C or caps, and without
+    // samples not when the caller chose another evaluation kernel for the graph.
+    const moc_graph* g = s->g;
+    if (s->walk_scores && g->generation != s->graph_generation)
+        return fail(MOC_ERR_ARG, "moc_search_run: the graph's C or node caps changed after the search's chains were evaluated");
+    if (!s->walk_planned) plan_walk(s);
+    if (s->incremental ? s->walk_scores
+                       : s->walk_fn && g->generation == s->graph_generation && g->want_G == 0 &&
+                             (g->want_kind == MOC_KERNEL_AUTO || g->want_kind == MOC_KERNEL_WARP)) {
+        moc::WalkParams& w = s->wp;
+        w.samples = s->samples;
+        w.lanes_per_gen = 1;
+        while (w.lanes_per_gen < std::min(s->samples, 32)) w.lanes_per_gen *= 2;
+        w.cap = g->d_cap;
+        const int32_t most = std::max(1, kWalkProposals / s->samples);
+        for (int32_t k = 0; k < n_generations; k += most) {
+            w.s = p;
+            w.s.generation = s->generation + (uint32_t)k;
+            w.n_gen = std::min(most, n_generations - k);
+            void* args[] = {&w};
+            MOC_CUDA(cudaLaunchKernel(s->walk_fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, s->walk_smem, st));
+            ++launches;
+        }
+        s->generation += (uint32_t)n_generations;
+        launch_counter() = launches;
+        return MOC_OK;
+    }
+    MOC_CUDA(cudaMemsetAsync(s->wp.peak_at, 0, (size_t)s->P * 4, st));       // the kernels below do not keep it
     if (s->incremental && s->fused) {
         moc_cache* h = s->cache;
         if (h->graph_generation != h->g->generation)
@@ -294,25 +324,6 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
         launch_counter() = launches;
         return MOC_OK;
     }
-    // The walk kernel relies on the chains' evaluations: not after a change of the graph's C or caps, and not
-    // when the caller chose another evaluation kernel for the graph.
-    const moc_graph* g = s->g;
-    if (!s->walk_planned) plan_walk(s);
-    if (s->walk_fn && g->generation == s->graph_generation && g->want_G == 0 &&
-        (g->want_kind == MOC_KERNEL_AUTO || g->want_kind == MOC_KERNEL_WARP)) {
-        for (int32_t k = 0; k < n_generations; k += kWalkGenerations) {
-            s->wp.s = p;
-            s->wp.s.generation = s->generation + (uint32_t)k;
-            s->wp.n_gen = std::min(kWalkGenerations, n_generations - k);
-            s->wp.cap = g->d_cap;
-            void* args[] = {&s->wp};
-            MOC_CUDA(cudaLaunchKernel(s->walk_fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, s->walk_smem, st));
-            ++launches;
-        }
-        s->generation += (uint32_t)n_generations;
-        launch_counter() = launches;
-        return MOC_OK;
-    }
     for (int32_t k = 0; k < n_generations; ++k) {
         p.generation = s->generation + (uint32_t)k;
         // settle the previous generation's proposals (none before the first one), propose the next
@@ -352,6 +363,7 @@ int moc_search_set_samples(moc_search* s, int32_t samples, int32_t incremental) 
     if (!incremental) {
         s->incremental = false;
         s->fused = false;
+        s->walk_scores = false;
         s->samples = 1;
         return MOC_OK;
     }
@@ -362,6 +374,14 @@ int moc_search_set_samples(moc_search* s, int32_t samples, int32_t incremental) 
         if (st[c] < 0)
             return fail(MOC_ERR_ARG, "moc_search_set_samples: chain %d has no valid sequence (status %d); the incremental "
                         "evaluation starts from valid sequences only", c, st[c]);
+    // by default the kernel that takes a warp per chain through all generations (no cache), where the graph fits it
+    if (!s->walk_planned) plan_walk(s);
+    s->walk_scores = incremental == MOC_SEARCH_SCORE_AUTO && s->walk_fn && s->g->generation == s->graph_generation;
+    if (s->walk_scores) {
+        s->samples = samples;
+        s->incremental = true;
+        return MOC_OK;
+    }
     if (!s->cache) {
         moc_cache* h = nullptr;
         int rc = moc_cache_create(s->g, s->P, &h);

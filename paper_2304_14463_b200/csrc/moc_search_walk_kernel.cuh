@@ -35,6 +35,9 @@ constexpr int kWalkThreads = 896;     // 28 warps, 72 registers per thread
 struct WalkParams {
     SearchParams s;            // s.generation: number of the first generation
     int32_t n_gen;             // generations of this launch
+    int32_t samples;           // E: proposals per chain and generation
+    int32_t lanes_per_gen;     // E rounded up to a power of two, at most 32
+    int32_t* peak_at;          // P: where the peak of each chain's sequence lies (walk_eval's `at`), 0: not known
     int32_t n, C, n_tiles;
     const void* rec;           // node records and successor tiles of the warp-per-sequence layout
     const uint32_t* sell;
@@ -59,11 +62,12 @@ __device__ __forceinline__ uint32_t walk_above(uint32_t p, uint32_t k) {
     return __viaddmin_s16x2_relu(p, ((0x00010000u - k) & 0xFFFFu) * 0x10001u, 0x00010001u);
 }
 
-// Stages 2 to 4 of the evaluation (moc_pair_kernel.cuh) on the occurrence words at `wa`: the peak, and
-// whether a consumer lacks a producer copy.  The deltas are zero on entry and on return.
+// Stages 2 to 4 of the evaluation (moc_pair_kernel.cuh) on the occurrence words at `wa`: the peak, whether a
+// consumer lacks a producer copy, and `at`: the peak is reached at one of the steps at .. at + 16 / sizeof(MemT) - 1
+// (1-based; one vector of deltas).  The deltas are zero on entry and on return.
 template <typename MemT>
 __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec0, uint32_t sell0, int n_tiles, int32_t T, int lane,
-                                          bool& dep) {
+                                       bool& dep, int32_t& at) {
     constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
     constexpr int kPerVec = 16 / (int)sizeof(MemT), kShift = sizeof(MemT) == 4 ? 2 : 3;
     const uint32_t da1 = da - (uint32_t)sizeof(MemT);
@@ -123,20 +127,26 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
     const int nvec = (T + 2 + kPerVec - 1) / kPerVec, V = ((nvec + 31) >> 5) | 1;
     uint32_t ad = da + 16u * (uint32_t)(lane * V);
     MemT run = 0, top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
+    int vec = 0;                       // the lane's vector that holds its maximum
     for (int j = 0; j < V; ++j, ad += 16u) {
         const uint4 q = lds_v4(ad);
         asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(ad), "r"(0) : "memory");
+        MemT hi;
         if constexpr (sizeof(MemT) == 4) {
-            run += (MemT)q.x; top = max(top, run);
-            run += (MemT)q.y; top = max(top, run);
-            run += (MemT)q.z; top = max(top, run);
-            run += (MemT)q.w; top = max(top, run);
+            run += (MemT)q.x; hi = run;
+            run += (MemT)q.y; hi = max(hi, run);
+            run += (MemT)q.z; hi = max(hi, run);
+            run += (MemT)q.w; hi = max(hi, run);
         } else {
-            run += (MemT)((uint64_t)q.x | (uint64_t)q.y << 32); top = run > top ? run : top;
-            run += (MemT)((uint64_t)q.z | (uint64_t)q.w << 32); top = run > top ? run : top;
+            run += (MemT)((uint64_t)q.x | (uint64_t)q.y << 32); hi = run;
+            run += (MemT)((uint64_t)q.z | (uint64_t)q.w << 32); hi = run > hi ? run : hi;
         }
+        if (hi > top) { top = hi; vec = j; }
     }
-    const MemT peak = warp_max_t((MemT)(warp_inclusive_sum(run, lane) - run + top));
+    top += warp_inclusive_sum(run, lane) - run;
+    const MemT peak = warp_max_t(top);
+    const int src = __ffs(__ballot_sync(kFull, top == peak)) - 1;
+    at = kPerVec * (src * V + __shfl_sync(kFull, vec, src)) + 1;
     __syncwarp();
     return peak;
 }
@@ -189,7 +199,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t word_set = p.word_bytes + kPairWordTail;
     const uint32_t mine = sbase + p.rec_bytes + p.sell_bytes + (uint32_t)warp * (2u * word_set + p.delta_bytes);
-    const uint32_t da = mine + 2u * word_set + kPairDeltaFront;      // &delta[0]
+    const uint32_t note = mine + 2u * word_set;                      // 16 bytes in front of the deltas: the chosen proposal
+    const uint32_t da = note + kPairDeltaFront;                      // &delta[0]
     const uint32_t rec0 = sbase + kRecB * (uint32_t)lane, sell0 = sbase + p.rec_bytes + 4u * (uint32_t)lane;
     const int n = p.n, n_tiles = p.n_tiles;
     if (lane < 2) sts_u32(mine + word_set * (uint32_t)lane + p.word_bytes, 0x00010001u);   // owned by empty node slots
@@ -199,7 +210,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
 
     for (int32_t c = blockIdx.x * wpb + warp; c < s.P; c += gridDim.x * wpb) {
         int32_t* row = s.rows + ((int64_t)s.cur[c] * s.P + c) * s.stride;
-        int32_t T = s.lens[c], st = s.status[c], n_acc = 0;
+        int32_t T = s.lens[c], st = s.status[c], n_acc = 0, tp = p.peak_at[c];
         int64_t pk = s.peak[c], du = s.dur[c];
         uint32_t wa = mine, wb = mine + word_set;       // the chain's words, and those of a proposal
         // occurrence words of the edited row (qd = ji = kEditNone: the row itself) by exchanges, as in the
@@ -226,122 +237,193 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             return sum;
         };
         if (st >= 0) words_of(wa, T, kEditNone, kEditNone, 0);
+        // out with step qd_s, in at index ji_s: the words of the edited sequence at w1, from the parent's at w0
+        auto shift_words = [&](uint32_t w0, uint32_t w1, int32_t Tc_s, int32_t qd_s, int32_t ji_s, int32_t x_s, uint32_t wx_s) {
+            const uint32_t kq = qd_s == kEditNone ? 0x7FFFu : (uint32_t)qd_s + 1u, kj = ji_s == kEditNone ? 0x7FFFu : (uint32_t)ji_s;
+            for (uint32_t o = 16u * (uint32_t)lane; o < p.word_bytes; o += 512u) {
+                uint4 v = lds_v4(w0 + o);
+                v.x -= walk_above(v.x, kq); v.x += walk_above(v.x, kj);
+                v.y -= walk_above(v.y, kq); v.y += walk_above(v.y, kj);
+                v.z -= walk_above(v.z, kq); v.z += walk_above(v.z, kj);
+                v.w -= walk_above(v.w, kq); v.w += walk_above(v.w, kj);
+                asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(w1 + o), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+            }
+            __syncwarp();
+            if (lane == 0) {
+                sts_u32(w1 + 4u * (uint32_t)x_s, wx_s);
+                sts_u32(w1 + 4u * (uint32_t)(n + 1), (uint32_t)Tc_s * 0x10001u);
+            }
+            __syncwarp();
+        };
 
-        for (int32_t g0 = 0; g0 < p.n_gen; g0 += 32) {
-            const uint4 r = philox4x32_10(make_uint4(s.generation + (uint32_t)(g0 + lane), s.chain0 + (uint32_t)c, 0u, 0u),
-                                          make_uint2(s.seed_lo, s.seed_hi));
-            const int32_t op = (int32_t)search_pick_kind(s.kinds, r.x);
-            uint32_t pending = p.n_gen - g0 >= 32 ? kFull : (1u << (p.n_gen - g0)) - 1u;
-            while (pending && T > 0) {
-                // ---- the pending generations against the present sequence, a lane each
-                const bool live = (pending >> lane & 1u) != 0;
-                const int32_t q = (int32_t)(r.y % (uint32_t)T);
-                const int32_t j = op == 0 ? (int32_t)(r.z % ((uint32_t)T + 1u)) : (int32_t)(r.z % (uint32_t)T);
-                const int32_t qd = op >= 1 ? q : kEditNone, ji = op != 1 ? j : kEditNone;
-                const int32_t Tc = T + (op == 0 ? 1 : 0) - (op == 1 ? 1 : 0);
-                const int32_t x = row[q];
-                bool adm = live && Tc >= n && Tc <= s.max_T;
-                uint32_t wx_new = 0;        // the edited node's word after the edit
-                int64_t du_c = 0;
-                if (adm && st >= 0) {
-                    const uint32_t wx = lds_u32(wa + 4u * (uint32_t)x);
-                    const int32_t xa = (int32_t)min(wx & 0xFFFFu, wx >> 16) - 1, xb = (int32_t)max(wx & 0xFFFFu, wx >> 16) - 1;
-                    const int32_t cnt = xa == xb ? 1 : 2, cnt2 = cnt - (op >= 1 ? 1 : 0) + (op != 1 ? 1 : 0);
-                    adm = cnt2 == 1 || (cnt2 == 2 && p.C >= 2 && (p.cap == nullptr || __ldg(p.cap + x) >= 2));
-                    if (adm) {
-                        auto map = [&](int32_t t) -> int32_t { const int32_t t1 = t - (t > qd ? 1 : 0); return t1 + (t1 >= ji ? 1 : 0); };
-                        // first child copy c0 (and c1), with the parent steps of other nodes' copies that lie in front
-                        // of c0 (r < tb0) and behind it (r > ta0), 1-based, as in moc_edit_pass.cuh
-                        int32_t c0 = kEditNone, c1 = kEditNone, ta0 = 0, tb0 = 0;
-                        auto push = [&](int32_t cs, int32_t ta, int32_t tb) {
-                            if (c0 == kEditNone) { c0 = cs; ta0 = ta; tb0 = tb; }
-                            else if (cs < c0) { c1 = c0; c0 = cs; ta0 = ta; tb0 = tb; }
-                            else { c1 = cs; }
-                        };
-                        if (xa != qd) push(map(xa), xa + 1, xa + 1);
-                        if (cnt == 2 && xb != qd) push(map(xb), xb + 1, xb + 1);
-                        if (ji != kEditNone) { const int32_t thr = ji + (ji >= qd ? 1 : 0); push(ji, thr, thr + 1); }
-                        wx_new = (uint32_t)(c0 + 1) | (uint32_t)((c1 == kEditNone ? c0 : c1) + 1) << 16;
-                        du_c = du + __ldg(p.w + x) * (cnt2 - cnt);
-                        // within the budget only the duration decides
-                        adm = pk > s.M || du_c <= du;
-                        if (adm) {
-                            bool viol = false;
-                            const int32_t p0 = __ldg(p.pred_start + x), p1 = __ldg(p.pred_start + x + 1);
-                            const int32_t s0 = __ldg(p.succ_start + x), s1 = __ldg(p.succ_start + x + 1);
+        // The edit (qd, ji) of node x against the chain's valid sequence: can it be accepted, as far as the copies of x
+        // and of its neighbours tell; the node's word after the edit and the new duration.
+        auto test = [&](int32_t op, int32_t qd, int32_t ji, int32_t x, uint32_t& wx_new, int64_t& du_c) -> bool {
+            const uint32_t wx = lds_u32(wa + 4u * (uint32_t)x);
+            const int32_t xa = (int32_t)min(wx & 0xFFFFu, wx >> 16) - 1, xb = (int32_t)max(wx & 0xFFFFu, wx >> 16) - 1;
+            const int32_t cnt = xa == xb ? 1 : 2, cnt2 = cnt - (op >= 1 ? 1 : 0) + (op != 1 ? 1 : 0);
+            if (!(cnt2 == 1 || (cnt2 == 2 && p.C >= 2 && (p.cap == nullptr || __ldg(p.cap + x) >= 2)))) return false;
+            du_c = du + __ldg(p.w + x) * (cnt2 - cnt);
+            const bool longer = du_c > du;
+            if (longer && pk <= s.M) return false;      // within the budget only the duration decides
+            auto map = [&](int32_t t) -> int32_t { const int32_t t1 = t - (t > qd ? 1 : 0); return t1 + (t1 >= ji ? 1 : 0); };
+            // first child copy c0 (and c1), with the parent steps of other nodes' copies that lie in front of c0
+            // (r < tb0) and behind it (r > ta0), 1-based, as in moc_edit_pass.cuh
+            int32_t c0 = kEditNone, c1 = kEditNone, ta0 = 0, tb0 = 0;
+            auto push = [&](int32_t cs, int32_t ta, int32_t tb) {
+                if (c0 == kEditNone) { c0 = cs; ta0 = ta; tb0 = tb; }
+                else if (cs < c0) { c1 = c0; c0 = cs; ta0 = ta; tb0 = tb; }
+                else { c1 = cs; }
+            };
+            if (xa != qd) push(map(xa), xa + 1, xa + 1);
+            if (cnt == 2 && xb != qd) push(map(xb), xb + 1, xb + 1);
+            if (ji != kEditNone) { const int32_t thr = ji + (ji >= qd ? 1 : 0); push(ji, thr, thr + 1); }
+            wx_new = (uint32_t)(c0 + 1) | (uint32_t)((c1 == kEditNone ? c0 : c1) + 1) << 16;
+            // Over the budget a longer sequence has to lower the peak.  A second copy of x lowers the usage at the
+            // peak's step only when the first copy, which is resident there for a later consumer, can end in front of it:
+            // the peak lies behind the first copy and in front of the second, and so does no consumer from the
+            // peak on.  (Everything else an inserted copy does to the profile adds to it.)
+            const bool must_drop = longer && tp > 0;
+            const int32_t tmax = tp + 16 / (int32_t)sizeof(MemT) - 1;
+            if (must_drop && !(xa + 1 < tmax && ji >= tp)) return false;
+            bool viol = false, later = false;
+            const int32_t p0 = __ldg(p.pred_start + x), p1 = __ldg(p.pred_start + x + 1);
+            const int32_t s0 = __ldg(p.succ_start + x), s1 = __ldg(p.succ_start + x + 1);
 #pragma unroll 1
-                            for (int32_t k = p0; k < p1; ++k) {
-                                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.pred + k));
-                                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) > ta0;
-                            }
+            for (int32_t k = p0; k < p1; ++k) {
+                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.pred + k));
+                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) > ta0;
+            }
 #pragma unroll 1
-                            for (int32_t k = s0; k < s1; ++k) {
-                                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.succ + k));
-                                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) < tb0;
+            for (int32_t k = s0; k < s1; ++k) {
+                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.succ + k));
+                const int32_t r0 = (int32_t)min(wv & 0xFFFFu, wv >> 16), r1 = (int32_t)max(wv & 0xFFFFu, wv >> 16);
+                viol |= r0 < tb0 || (must_drop && ((r0 >= tmax && r0 <= ji) || (r1 >= tmax && r1 <= ji)));
+                later |= r1 > ji;
+            }
+            return !viol && (!must_drop || later || s0 == s1);
+        };
+        // smallest of the lanes' values >= 0
+        auto min64 = [&](int64_t v, bool in) -> int64_t {
+            const uint32_t hi = in ? (uint32_t)((uint64_t)v >> 32) : kFull, hmin = __reduce_min_sync(kFull, hi);
+            const uint32_t lo = (in && hi == hmin) ? (uint32_t)v : kFull, lmin = __reduce_min_sync(kFull, lo);
+            return (int64_t)((uint64_t)hmin << 32 | lmin);
+        };
+
+        // A batch is `span` generations of E proposals with a lane each, or, for E > 32, 32 proposals of one
+        // generation; the best proposal of the generation is then carried from batch to batch.
+        const int32_t E = p.samples, per = p.lanes_per_gen, span = 32 / per, my_gen = lane / per, my_e = lane % per;
+        bool b_has = false, b_here = false;         // a proposal is chosen; its words are at wb
+        int64_t b_a = 0, b_d = 0, b_pk = 0;         // key and peak of the chosen one; without one the chain's key
+        int32_t b_tp = 0;
+        auto fresh = [&]() {                        // a chain without a valid sequence takes any valid proposal
+            b_has = false;
+            b_a = st < 0 ? INT64_MAX : (pk > s.M ? pk : s.M);
+            b_d = du;
+        };
+        // the chosen proposal replaces the chain's sequence
+        auto settle = [&]() {
+            const int32_t qd_s = (int32_t)lds_u32(note), ji_s = (int32_t)lds_u32(note + 4u), x_s = (int32_t)lds_u32(note + 8u);
+            const int32_t Tc_s = T + (qd_s == kEditNone ? 1 : 0) - (ji_s == kEditNone ? 1 : 0);
+            if (!b_here) shift_words(wa, wb, Tc_s, qd_s, ji_s, x_s, lds_u32(note + 12u));
+            walk_apply(row, T, qd_s, ji_s, x_s, lane);
+            const uint32_t sw = wa;
+            wa = wb;
+            wb = sw;
+            T = Tc_s;
+            pk = b_pk;
+            du = b_d;
+            tp = b_tp;
+            st = pk <= s.M ? 1 : 0;
+            ++n_acc;
+        };
+        for (int32_t g0 = 0; g0 < p.n_gen && T > 0; g0 += span) {
+            fresh();
+            for (int32_t e0 = 0; e0 < E; e0 += 32) {
+                const uint4 r = philox4x32_10(make_uint4(s.generation + (uint32_t)(g0 + my_gen), s.chain0 + (uint32_t)c, (uint32_t)(e0 + my_e), 0u),
+                                              make_uint2(s.seed_lo, s.seed_hi));
+                const int32_t op = (int32_t)search_pick_kind(s.kinds, r.x);
+                const uint32_t drawn = __ballot_sync(kFull, g0 + my_gen < p.n_gen && e0 + my_e < E);
+                uint32_t pending = drawn;
+                while (pending && T > 0) {
+                    // ---- the pending proposals against the present sequence, a lane each
+                    const int32_t q = (int32_t)(r.y % (uint32_t)T);
+                    const int32_t j = op == 0 ? (int32_t)(r.z % ((uint32_t)T + 1u)) : (int32_t)(r.z % (uint32_t)T);
+                    const int32_t qd = op >= 1 ? q : kEditNone, ji = op != 1 ? j : kEditNone;
+                    const int32_t Tc = T + (op == 0 ? 1 : 0) - (op == 1 ? 1 : 0);
+                    const int32_t x = row[q];
+                    bool adm = (pending >> lane & 1u) != 0 && Tc >= n && Tc <= s.max_T;
+                    uint32_t wx_new = 0;
+                    int64_t du_c = 0;
+                    if (adm && st >= 0) adm = test(op, qd, ji, x, wx_new, du_c);
+                    uint32_t todo = __ballot_sync(kFull, adm);
+                    pending = 0;
+                    while (todo) {
+                        // ---- the earliest generation that has proposals left: in order of duration, then number
+                        const int gen = (__ffs(todo) - 1) / per;
+                        const uint32_t group = (per == 32 ? kFull : (1u << per) - 1u) << (gen * per);
+                        uint32_t cand = todo & group;
+                        todo &= ~group;
+                        while (cand) {
+                            int sl = __ffs(cand) - 1;
+                            if (cand & (cand - 1u)) {
+                                const bool in = (cand >> lane & 1u) != 0;
+                                const int64_t d_min = min64(du_c, in);
+                                sl = __ffs(__ballot_sync(kFull, in && du_c == d_min)) - 1;
                             }
-                            adm = !viol;
+                            cand &= ~(1u << sl);
+                            const int32_t qd_s = __shfl_sync(kFull, qd, sl), ji_s = __shfl_sync(kFull, ji, sl), x_s = __shfl_sync(kFull, x, sl);
+                            const int32_t Tc_s = __shfl_sync(kFull, Tc, sl);
+                            const uint32_t wx_s = __shfl_sync(kFull, wx_new, sl);
+                            int64_t du_s = __shfl_sync(kFull, du_c, sl);
+                            // a proposal within the budget is known: those that are no shorter cannot be better
+                            if (b_has && b_a == s.M && du_s >= b_d) break;
+                            b_here = false;
+                            if (st >= 0) {
+                                shift_words(wa, wb, Tc_s, qd_s, ji_s, x_s, wx_s);
+                            } else {
+                                // from scratch: every node present, as many second copies as steps beyond n, caps
+                                du_s = warp_sum64(words_of(wb, Tc_s, qd_s, ji_s, x_s));
+                                uint32_t two = 0;
+                                bool bad = false;
+                                for (int32_t v = lane; v < n; v += 32) {
+                                    const uint32_t wv = lds_u32(wb + 4u * (uint32_t)v);
+                                    const bool t2 = (wv & 0xFFFFu) != wv >> 16;
+                                    two += t2 ? 1u : 0u;
+                                    bad |= wv == 0 || (t2 && (p.C < 2 || (p.cap != nullptr && __ldg(p.cap + v) < 2)));
+                                }
+                                two = __reduce_add_sync(kFull, two);
+                                if (__any_sync(kFull, bad) || (int32_t)two != Tc_s - n) continue;
+                            }
+                            bool dep;
+                            int32_t at;
+                            const int64_t pk_s = (int64_t)walk_eval<MemT>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, dep, at);
+                            const int64_t a_s = pk_s > s.M ? pk_s : s.M;
+                            if (dep || a_s > b_a || (a_s == b_a && (b_has ? du_s >= b_d : (st >= 0 && du_s > b_d)))) continue;
+                            b_has = b_here = true;
+                            b_a = a_s;
+                            b_d = du_s;
+                            b_pk = pk_s;
+                            b_tp = at;
+                            if (lane == 0) {
+                                sts_u32(note, (uint32_t)qd_s);
+                                sts_u32(note + 4u, (uint32_t)ji_s);
+                                sts_u32(note + 8u, (uint32_t)x_s);
+                                sts_u32(note + 12u, wx_s);
+                            }
+                            __syncwarp();
+                        }
+                        if (b_has && E <= 32) {
+                            settle();
+                            fresh();
+                            // the generations behind this one see the new sequence
+                            pending = gen == span - 1 ? 0u : (kFull << ((gen + 1) * per)) & drawn;
+                            break;
                         }
                     }
-                }
-                // ---- the admissible ones in order, until one is accepted
-                uint32_t todo = __ballot_sync(kFull, adm);
-                pending = 0;
-                while (todo) {
-                    const int sl = __ffs(todo) - 1;
-                    todo &= todo - 1;
-                    const int32_t qd_s = __shfl_sync(kFull, qd, sl), ji_s = __shfl_sync(kFull, ji, sl), x_s = __shfl_sync(kFull, x, sl);
-                    const int32_t Tc_s = __shfl_sync(kFull, Tc, sl);
-                    int64_t du_s = __shfl_sync(kFull, du_c, sl), pk_s = -1;
-                    bool valid = true, dep;
-                    if (st >= 0) {
-                        // words of the edited sequence: out with step qd, in at index ji
-                        const uint32_t kq = qd_s == kEditNone ? 0x7FFFu : (uint32_t)qd_s + 1u, kj = ji_s == kEditNone ? 0x7FFFu : (uint32_t)ji_s;
-                        const uint32_t wx_s = __shfl_sync(kFull, wx_new, sl);
-                        for (uint32_t o = 16u * (uint32_t)lane; o < p.word_bytes; o += 512u) {
-                            uint4 v = lds_v4(wa + o);
-                            v.x -= walk_above(v.x, kq); v.x += walk_above(v.x, kj);
-                            v.y -= walk_above(v.y, kq); v.y += walk_above(v.y, kj);
-                            v.z -= walk_above(v.z, kq); v.z += walk_above(v.z, kj);
-                            v.w -= walk_above(v.w, kq); v.w += walk_above(v.w, kj);
-                            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(wb + o), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-                        }
-                        __syncwarp();
-                        if (lane == 0) {
-                            sts_u32(wb + 4u * (uint32_t)x_s, wx_s);
-                            sts_u32(wb + 4u * (uint32_t)(n + 1), (uint32_t)Tc_s * 0x10001u);
-                        }
-                        __syncwarp();
-                    } else {
-                        // from scratch: every node present, as many second copies as steps beyond n, caps
-                        du_s = warp_sum64(words_of(wb, Tc_s, qd_s, ji_s, x_s));
-                        uint32_t two = 0;
-                        bool bad = false;
-                        for (int32_t v = lane; v < n; v += 32) {
-                            const uint32_t wv = lds_u32(wb + 4u * (uint32_t)v);
-                            const bool t2 = (wv & 0xFFFFu) != wv >> 16;
-                            two += t2 ? 1u : 0u;
-                            bad |= wv == 0 || (t2 && (p.C < 2 || (p.cap != nullptr && __ldg(p.cap + v) < 2)));
-                        }
-                        two = __reduce_add_sync(kFull, two);
-                        valid = !__any_sync(kFull, bad) && (int32_t)two == Tc_s - n;
-                    }
-                    if (!valid) continue;
-                    pk_s = (int64_t)walk_eval<MemT>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, dep);
-                    if (dep || !search_not_worse(pk_s, du_s, 1, pk, du, st, s.M)) continue;
-                    walk_apply(row, T, qd_s, ji_s, x_s, lane);
-                    const uint32_t sw = wa;
-                    wa = wb;
-                    wb = sw;
-                    T = Tc_s;
-                    pk = pk_s;
-                    du = du_s;
-                    st = pk <= s.M ? 1 : 0;
-                    ++n_acc;
-                    // the generations behind this one see the new sequence
-                    pending = sl == 31 ? 0u : (kFull << (sl + 1)) & (p.n_gen - g0 >= 32 ? kFull : (1u << (p.n_gen - g0)) - 1u);
-                    break;
                 }
             }
+            if (b_has) settle();
         }
         __syncwarp();
         if (lane == 0 && n_acc) {
@@ -350,6 +432,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             s.dur[c] = du;
             s.status[c] = st;
             s.n_acc[c] += n_acc;
+            p.peak_at[c] = tp;
         }
         __syncwarp();
     }
