@@ -1,11 +1,10 @@
-// The search with one proposal per chain and generation (paper: Section 3, the two-phase local search),
-// all generations of a call in one kernel.  The chains are independent, so a warp takes its chain through
+// The search (paper: Section 3, the two-phase local search), all generations of a call in one kernel.  The chains are independent, so a warp takes its chain through
 // every generation of the launch with the chain's copy positions in shared memory; nothing is exchanged
 // between warps.  C <= 2 and graphs of the warp-per-sequence layout (moc_pair_kernel.cuh).
 //
 // What a generation costs.  About four proposals of five are refused by a test on the edited node alone
-// (copy count, Eq. 5 on the edges that touch the node).  Lane k therefore draws and tests the proposal
-// of generation base + k, 32 generations at a time against the chain's present sequence, and the warp
+// (copy count, Eq. 5 on the edges that touch the node).  A lane therefore draws and tests one proposal, 32 of
+// one generation or of several generations at a time against the chain's present sequence, and the warp
 // evaluates only the admissible ones, in order.  An accepted one changes the sequence: the generations
 // behind it are tested again (a draw does not depend on the sequence, only its reading does).
 // An admissible proposal is evaluated in full, but not from its sequence: the copy positions of the edited
@@ -21,9 +20,11 @@
 // Chains without a valid sequence (status < 0) have no test to rely on: their proposals are evaluated from
 // the written-out order, one generation at a time, until one is valid.
 //
-// Bound: instruction issue and the shared-memory data pipe, like the evaluation kernel, on a fifth of the
-// proposals.  n = 442, 4096 chains, 20 generations with the copy-out of the chains' state: 436 -> 67.7 us
-// against two kernels per generation that write every proposal out and evaluate it.
+// Bound: instruction issue (53 % of the slots, 2100 instructions per generation of 32 proposals) and the latency of
+// its dependent shared-memory reads; 28 warps beat 24 and 20 with more registers each, and 30 with fewer.
+// n = 442, state copied out: 4096 chains x 20 generations 436 -> 41.9 us against two kernels per generation that
+// write every proposal out; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us against a cached
+// evaluation per chain that is rebuilt after every acceptance.
 #pragma once
 #include "moc_edit_kernels.cuh"
 #include "moc_search_kernels.cuh"
@@ -52,9 +53,17 @@ struct WalkParams {
     uint32_t delta_bytes;      // front pad + deltas for C * n steps
 };
 
-// Bytes of one warp: two sets of words, each followed by the constant word, and the deltas.
+// Scalars of the warp's chain that are needed between evaluations only.  They are kept in shared memory: as
+// registers they were spilled, and the local memory of 28 warps is far larger than the L1 that is left beside
+// the chains' state.
+constexpr uint32_t kWalkQd = 0, kWalkJi = 4, kWalkX = 8, kWalkWx = 12;           // the chosen proposal
+constexpr uint32_t kWalkBestA = 16, kWalkBestD = 24, kWalkBestPk = 32;           // its key and peak (without one: the chain's key)
+constexpr uint32_t kWalkBestAt = 40, kWalkAcc = 44, kWalkPk = 48, kWalkDu = 56;  // its `at`; the chain: accepted, peak, duration
+constexpr uint32_t kWalkNoteBytes = 64;
+
+// Bytes of one warp: two sets of words, each followed by the constant word, the scalars, and the deltas.
 __host__ __device__ inline size_t walk_warp_bytes(uint32_t word_bytes, uint32_t delta_bytes) {
-    return 2 * ((size_t)word_bytes + kPairWordTail) + delta_bytes;
+    return 2 * ((size_t)word_bytes + kPairWordTail) + kWalkNoteBytes + delta_bytes;
 }
 
 // [p > k] per 16-bit half (p, k < 2^15): max(min(p - k, 1), 0).
@@ -151,34 +160,25 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
     return peak;
 }
 
-// Shifts row[a..b) by one place to the left (dir = -1) or to the right (dir = 1) with the lanes of a warp.
-__device__ __forceinline__ void walk_shift(int32_t* row, int32_t a, int32_t b, int dir, int lane) {
+// Element qd taken out of row[0..T) (none: kEditNone), then x put in front of index ji of what is left (none:
+// kEditNone), in place: the elements between the two places move by one.  Not inlined: its eight loads in
+// flight would cost the whole kernel registers.
+static __device__ __noinline__ void walk_apply(int32_t* row, int32_t T, int32_t qd, int32_t ji, int32_t x, int lane) {
+    const bool left = qd != kEditNone && (ji == kEditNone || ji >= qd);
+    const int32_t a = left ? qd + 1 : ji, b = left ? (ji == kEditNone ? T : ji + 1) : (qd == kEditNone ? T : qd), dir = left ? -1 : 1;
     for (int32_t done = 0; done < b - a; done += 256) {
         int32_t v[8];
         // ascending pieces to the left, descending pieces to the right: no element is overwritten unread
-        const int32_t base = dir < 0 ? a + done : b - done - 256;
+        const int32_t base = (left ? a + done : b - done - 256) + lane;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int32_t i = base + lane + 32 * k;
-            if (i >= a && i < b) v[k] = row[i];
-        }
+        for (int k = 0; k < 8; ++k)
+            if (base + 32 * k >= a && base + 32 * k < b) v[k] = row[base + 32 * k];
         __syncwarp();
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int32_t i = base + lane + 32 * k;
-            if (i >= a && i < b) row[i + dir] = v[k];
-        }
+        for (int k = 0; k < 8; ++k)
+            if (base + 32 * k >= a && base + 32 * k < b) row[base + 32 * k + dir] = v[k];
         __syncwarp();
     }
-}
-
-// Element qd taken out of row[0..T) (none: kEditNone), then x put in front of index ji of what is left (none:
-// kEditNone), in place.
-__device__ __forceinline__ void walk_apply(int32_t* row, int32_t T, int32_t qd, int32_t ji, int32_t x, int lane) {
-    if (qd == kEditNone) walk_shift(row, ji, T, 1, lane);
-    else if (ji == kEditNone) walk_shift(row, qd + 1, T, -1, lane);
-    else if (ji >= qd) walk_shift(row, qd + 1, ji + 1, -1, lane);
-    else walk_shift(row, ji, qd, 1, lane);
     if (ji != kEditNone && lane == 0) row[ji] = x;
     __syncwarp();
 }
@@ -198,9 +198,9 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
     }
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t word_set = p.word_bytes + kPairWordTail;
-    const uint32_t mine = sbase + p.rec_bytes + p.sell_bytes + (uint32_t)warp * (2u * word_set + p.delta_bytes);
-    const uint32_t note = mine + 2u * word_set;                      // 16 bytes in front of the deltas: the chosen proposal
-    const uint32_t da = note + kPairDeltaFront;                      // &delta[0]
+    const uint32_t mine = sbase + p.rec_bytes + p.sell_bytes + (uint32_t)warp * (2u * word_set + kWalkNoteBytes + p.delta_bytes);
+    const uint32_t note = mine + 2u * word_set;
+    const uint32_t da = note + kWalkNoteBytes + kPairDeltaFront;     // &delta[0]
     const uint32_t rec0 = sbase + kRecB * (uint32_t)lane, sell0 = sbase + p.rec_bytes + 4u * (uint32_t)lane;
     const int n = p.n, n_tiles = p.n_tiles;
     if (lane < 2) sts_u32(mine + word_set * (uint32_t)lane + p.word_bytes, 0x00010001u);   // owned by empty node slots
@@ -210,8 +210,15 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
 
     for (int32_t c = blockIdx.x * wpb + warp; c < s.P; c += gridDim.x * wpb) {
         int32_t* row = s.rows + ((int64_t)s.cur[c] * s.P + c) * s.stride;
-        int32_t T = s.lens[c], st = s.status[c], n_acc = 0, tp = p.peak_at[c];
-        int64_t pk = s.peak[c], du = s.dur[c];
+        int32_t T = s.lens[c], tp = p.peak_at[c];
+        bool valid = s.status[c] >= 0;
+        bool over = valid && s.peak[c] > s.M;       // over the budget
+        if (lane == 0) {
+            sts_u64(note + kWalkPk, (uint64_t)s.peak[c]);
+            sts_u64(note + kWalkDu, (uint64_t)s.dur[c]);
+            sts_u32(note + kWalkAcc, 0u);
+        }
+        __syncwarp();
         uint32_t wa = mine, wb = mine + word_set;       // the chain's words, and those of a proposal
         // occurrence words of the edited row (qd = ji = kEditNone: the row itself) by exchanges, as in the
         // evaluation kernel; returns the summed durations of the lane's elements.  Invalid ids go to the spare word n.
@@ -236,7 +243,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             __syncwarp();
             return sum;
         };
-        if (st >= 0) words_of(wa, T, kEditNone, kEditNone, 0);
+        if (valid) words_of(wa, T, kEditNone, kEditNone, 0);
         // out with step qd_s, in at index ji_s: the words of the edited sequence at w1, from the parent's at w0
         auto shift_words = [&](uint32_t w0, uint32_t w1, int32_t Tc_s, int32_t qd_s, int32_t ji_s, int32_t x_s, uint32_t wx_s) {
             const uint32_t kq = qd_s == kEditNone ? 0x7FFFu : (uint32_t)qd_s + 1u, kj = ji_s == kEditNone ? 0x7FFFu : (uint32_t)ji_s;
@@ -263,9 +270,10 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             const int32_t xa = (int32_t)min(wx & 0xFFFFu, wx >> 16) - 1, xb = (int32_t)max(wx & 0xFFFFu, wx >> 16) - 1;
             const int32_t cnt = xa == xb ? 1 : 2, cnt2 = cnt - (op >= 1 ? 1 : 0) + (op != 1 ? 1 : 0);
             if (!(cnt2 == 1 || (cnt2 == 2 && p.C >= 2 && (p.cap == nullptr || __ldg(p.cap + x) >= 2)))) return false;
-            du_c = du + __ldg(p.w + x) * (cnt2 - cnt);
-            const bool longer = du_c > du;
-            if (longer && pk <= s.M) return false;      // within the budget only the duration decides
+            const int64_t more = __ldg(p.w + x) * (cnt2 - cnt);
+            du_c = (int64_t)lds_u64(note + kWalkDu) + more;
+            const bool longer = more > 0;
+            if (longer && !over) return false;      // within the budget only the duration decides
             auto map = [&](int32_t t) -> int32_t { const int32_t t1 = t - (t > qd ? 1 : 0); return t1 + (t1 >= ji ? 1 : 0); };
             // first child copy c0 (and c1), with the parent steps of other nodes' copies that lie in front of c0
             // (r < tb0) and behind it (r > ta0), 1-based, as in moc_edit_pass.cuh
@@ -314,39 +322,47 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
         // generation; the best proposal of the generation is then carried from batch to batch.
         const int32_t E = p.samples, per = p.lanes_per_gen, span = 32 / per, my_gen = lane / per, my_e = lane % per;
         bool b_has = false, b_here = false;         // a proposal is chosen; its words are at wb
-        int64_t b_a = 0, b_d = 0, b_pk = 0;         // key and peak of the chosen one; without one the chain's key
-        int32_t b_tp = 0;
         auto fresh = [&]() {                        // a chain without a valid sequence takes any valid proposal
             b_has = false;
-            b_a = st < 0 ? INT64_MAX : (pk > s.M ? pk : s.M);
-            b_d = du;
+            if (lane == 0) {
+                sts_u64(note + kWalkBestA, !valid ? (uint64_t)INT64_MAX : over ? lds_u64(note + kWalkPk) : (uint64_t)s.M);
+                sts_u64(note + kWalkBestD, lds_u64(note + kWalkDu));
+            }
+            __syncwarp();
         };
         // the chosen proposal replaces the chain's sequence
         auto settle = [&]() {
-            const int32_t qd_s = (int32_t)lds_u32(note), ji_s = (int32_t)lds_u32(note + 4u), x_s = (int32_t)lds_u32(note + 8u);
+            const int32_t qd_s = (int32_t)lds_u32(note + kWalkQd), ji_s = (int32_t)lds_u32(note + kWalkJi), x_s = (int32_t)lds_u32(note + kWalkX);
             const int32_t Tc_s = T + (qd_s == kEditNone ? 1 : 0) - (ji_s == kEditNone ? 1 : 0);
-            if (!b_here) shift_words(wa, wb, Tc_s, qd_s, ji_s, x_s, lds_u32(note + 12u));
+            if (!b_here) shift_words(wa, wb, Tc_s, qd_s, ji_s, x_s, lds_u32(note + kWalkWx));
             walk_apply(row, T, qd_s, ji_s, x_s, lane);
             const uint32_t sw = wa;
             wa = wb;
             wb = sw;
             T = Tc_s;
-            pk = b_pk;
-            du = b_d;
-            tp = b_tp;
-            st = pk <= s.M ? 1 : 0;
-            ++n_acc;
+            tp = (int32_t)lds_u32(note + kWalkBestAt);
+            valid = true;
+            over = (int64_t)lds_u64(note + kWalkBestPk) > s.M;
+            if (lane == 0) {
+                sts_u64(note + kWalkPk, lds_u64(note + kWalkBestPk));
+                sts_u64(note + kWalkDu, lds_u64(note + kWalkBestD));
+                sts_u32(note + kWalkAcc, lds_u32(note + kWalkAcc) + 1u);
+            }
+            __syncwarp();
         };
         for (int32_t g0 = 0; g0 < p.n_gen && T > 0; g0 += span) {
             fresh();
             for (int32_t e0 = 0; e0 < E; e0 += 32) {
-                const uint4 r = philox4x32_10(make_uint4(s.generation + (uint32_t)(g0 + my_gen), s.chain0 + (uint32_t)c, (uint32_t)(e0 + my_e), 0u),
-                                              make_uint2(s.seed_lo, s.seed_hi));
-                const int32_t op = (int32_t)search_pick_kind(s.kinds, r.x);
                 const uint32_t drawn = __ballot_sync(kFull, g0 + my_gen < p.n_gen && e0 + my_e < E);
                 uint32_t pending = drawn;
                 while (pending && T > 0) {
-                    // ---- the pending proposals against the present sequence, a lane each
+                    // ---- the pending proposals against the present sequence, a lane each (drawn again after an
+                    // acceptance: cheaper than the registers that would hold the draws over the evaluations)
+                    uint2 key = make_uint2(s.seed_lo, s.seed_hi);
+                    MOC_KEEP(key.x);        // the twenty round keys are not worth holding (and spilling) over the loop
+                    MOC_KEEP(key.y);
+                    const uint4 r = philox4x32_10(make_uint4(s.generation + (uint32_t)(g0 + my_gen), s.chain0 + (uint32_t)c, (uint32_t)(e0 + my_e), 0u), key);
+                    const int32_t op = (int32_t)search_pick_kind(s.kinds, r.x);
                     const int32_t q = (int32_t)(r.y % (uint32_t)T);
                     const int32_t j = op == 0 ? (int32_t)(r.z % ((uint32_t)T + 1u)) : (int32_t)(r.z % (uint32_t)T);
                     const int32_t qd = op >= 1 ? q : kEditNone, ji = op != 1 ? j : kEditNone;
@@ -355,7 +371,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                     bool adm = (pending >> lane & 1u) != 0 && Tc >= n && Tc <= s.max_T;
                     uint32_t wx_new = 0;
                     int64_t du_c = 0;
-                    if (adm && st >= 0) adm = test(op, qd, ji, x, wx_new, du_c);
+                    if (adm && valid) adm = test(op, qd, ji, x, wx_new, du_c);
+                    const uint32_t places = (uint32_t)q | (uint32_t)j << 15 | (uint32_t)op << 30;     // T < 2^15
                     uint32_t todo = __ballot_sync(kFull, adm);
                     pending = 0;
                     while (todo) {
@@ -372,14 +389,15 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                                 sl = __ffs(__ballot_sync(kFull, in && du_c == d_min)) - 1;
                             }
                             cand &= ~(1u << sl);
-                            const int32_t qd_s = __shfl_sync(kFull, qd, sl), ji_s = __shfl_sync(kFull, ji, sl), x_s = __shfl_sync(kFull, x, sl);
-                            const int32_t Tc_s = __shfl_sync(kFull, Tc, sl);
-                            const uint32_t wx_s = __shfl_sync(kFull, wx_new, sl);
+                            const uint32_t at_s = __shfl_sync(kFull, places, sl), wx_s = __shfl_sync(kFull, wx_new, sl);
+                            const int32_t op_s = (int32_t)(at_s >> 30), x_s = __shfl_sync(kFull, x, sl);
+                            const int32_t qd_s = op_s >= 1 ? (int32_t)(at_s & 0x7FFFu) : kEditNone, ji_s = op_s != 1 ? (int32_t)(at_s >> 15 & 0x7FFFu) : kEditNone;
+                            const int32_t Tc_s = T + (op_s == 0 ? 1 : 0) - (op_s == 1 ? 1 : 0);
                             int64_t du_s = __shfl_sync(kFull, du_c, sl);
                             // a proposal within the budget is known: those that are no shorter cannot be better
-                            if (b_has && b_a == s.M && du_s >= b_d) break;
+                            if (b_has && (int64_t)lds_u64(note + kWalkBestA) == s.M && du_s >= (int64_t)lds_u64(note + kWalkBestD)) break;
                             b_here = false;
-                            if (st >= 0) {
+                            if (valid) {
                                 shift_words(wa, wb, Tc_s, qd_s, ji_s, x_s, wx_s);
                             } else {
                                 // from scratch: every node present, as many second copies as steps beyond n, caps
@@ -398,18 +416,19 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                             bool dep;
                             int32_t at;
                             const int64_t pk_s = (int64_t)walk_eval<MemT>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, dep, at);
-                            const int64_t a_s = pk_s > s.M ? pk_s : s.M;
-                            if (dep || a_s > b_a || (a_s == b_a && (b_has ? du_s >= b_d : (st >= 0 && du_s > b_d)))) continue;
+                            const int64_t a_s = pk_s > s.M ? pk_s : s.M, b_a = (int64_t)lds_u64(note + kWalkBestA), b_d = (int64_t)lds_u64(note + kWalkBestD);
+                            if (dep || a_s > b_a || (a_s == b_a && (b_has ? du_s >= b_d : du_s > b_d))) continue;
                             b_has = b_here = true;
-                            b_a = a_s;
-                            b_d = du_s;
-                            b_pk = pk_s;
-                            b_tp = at;
+                            __syncwarp();
                             if (lane == 0) {
-                                sts_u32(note, (uint32_t)qd_s);
-                                sts_u32(note + 4u, (uint32_t)ji_s);
-                                sts_u32(note + 8u, (uint32_t)x_s);
-                                sts_u32(note + 12u, wx_s);
+                                sts_u64(note + kWalkBestA, (uint64_t)a_s);
+                                sts_u64(note + kWalkBestD, (uint64_t)du_s);
+                                sts_u64(note + kWalkBestPk, (uint64_t)pk_s);
+                                sts_u32(note + kWalkBestAt, (uint32_t)at);
+                                sts_u32(note + kWalkQd, (uint32_t)qd_s);
+                                sts_u32(note + kWalkJi, (uint32_t)ji_s);
+                                sts_u32(note + kWalkX, (uint32_t)x_s);
+                                sts_u32(note + kWalkWx, wx_s);
                             }
                             __syncwarp();
                         }
@@ -426,12 +445,14 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             if (b_has) settle();
         }
         __syncwarp();
+        const uint32_t n_acc = lds_u32(note + kWalkAcc);
         if (lane == 0 && n_acc) {
+            const int64_t pk = (int64_t)lds_u64(note + kWalkPk);
             s.lens[c] = T;
             s.peak[c] = pk;
-            s.dur[c] = du;
-            s.status[c] = st;
-            s.n_acc[c] += n_acc;
+            s.dur[c] = (int64_t)lds_u64(note + kWalkDu);
+            s.status[c] = pk <= s.M ? 1 : 0;
+            s.n_acc[c] += (int32_t)n_acc;
             p.peak_at[c] = tp;
         }
         __syncwarp();
