@@ -102,6 +102,20 @@ QuadFn quad_fn(bool wide, int C) {
     return wide ? (QuadFn)moc::eval_quad_kernel<int64_t, 4> : (QuadFn)moc::eval_quad_kernel<int32_t, 4>;
 }
 
+template <typename SumT, int W>
+LiveFn live_fn_k(int C) {
+    return C <= 2 ? (LiveFn)moc::eval_live_kernel<SumT, W, 2> : (LiveFn)moc::eval_live_kernel<SumT, W, 4>;
+}
+template <typename SumT>
+LiveFn live_fn_w(int words, int C) {
+    switch (words) {
+        case 1: return live_fn_k<SumT, 1>(C);
+        case 2: return live_fn_k<SumT, 2>(C);
+        default: return live_fn_k<SumT, 4>(C);
+    }
+}
+int live_words(int n) { return n <= 32 ? 1 : (n <= 64 ? 2 : 4); }
+
 // Raises a kernel's dynamic shared-memory limit to all the device offers beside its static part.
 cudaError_t raise_smem_limit(const void* fn, size_t smem_optin) {
     cudaFuncAttributes a{};
@@ -205,6 +219,16 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, Plan* out) {
     return nullptr;
 }
 
+// Backward walk with a lane per sequence: n <= 128, C <= 4.  Used for the batches live_serves() names.
+void plan_live(const moc_graph* g, Plan* pl) {
+    if (!g->d_live64 || g->C > moc::kLivePlanes) return;
+    const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C || g->sum_w > (int64_t)INT32_MAX / g->C;
+    pl->live_image = wide ? g->d_live64 : g->d_live32;
+    LiveFn fn = wide ? live_fn_w<int64_t>(live_words(g->n), g->C) : live_fn_w<int32_t>(live_words(g->n), g->C);
+    if (raise_smem_limit((const void*)fn, g->smem_optin) != cudaSuccess) { cudaGetLastError(); return; }
+    pl->live_fn = fn;
+}
+
 // Chooses kernel variant, group size and grid for the handle's current n and C.  The dynamic
 // shared-memory limit of a kernel is a property of the kernel, not of the handle: it is always
 // raised to the device maximum, so that handles with different needs can share one kernel.
@@ -221,6 +245,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     const size_t smem_cap = g->smem_optin > 1024 ? g->smem_optin - 1024 : 0;  // 1 KB per block is reserved
     const int kind = profile ? MOC_KERNEL_GROUP : g->want_kind;
     const bool shape_given = g->want_G != 0 || g->want_gpc != 0;       // moc_graph_set_launch
+    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile) plan_live(g, &pl);
     // Order of preference when nothing is forced: warp per sequence, then sequence per lane (it also
     // serves graphs whose degrees are too uneven for the warp kernel's padded successor tiles), then
     // the thread-group kernel, which serves everything.
@@ -508,6 +533,46 @@ moc::EvalParams base_params(const moc_graph* g, const Plan& pl) {
     return p;
 }
 
+// Batches the backward walk serves.  Its time hardly depends on the batch until every SM has 16 warps: about
+// 6 us + 0.17 us per node (a lane's steps follow one another), while the warp-per-sequence kernel takes 1.2 us per
+// 1000 sequences of these sizes (2 us with 64-bit sums; the block-per-sequence kernel with C >= 3 likewise).
+// Measured crossings: n = 20 at 7000, 50 at 11000, 100 at 17000 sequences; 100 with 64-bit sums or C = 3 at 9000.
+bool live_serves(const moc_graph* g, const Plan& pl, int32_t B) {
+    if (pl.live_fn == nullptr) return false;
+    return (int64_t)B * (g->C <= 2 && !pl.wide ? 6 : 10) >= 30000 + 850 * (int64_t)g->n;
+}
+
+int enqueue_live(const moc_graph* g, const Plan& pl, const int64_t* offs, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
+                 int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {
+    moc::LiveParams q{};
+    q.n = g->n;
+    q.C = g->C;
+    q.B = B;
+    q.M = M;
+    q.image = (const uint4*)pl.live_image;
+    q.sink_m = g->sink_m;
+    for (int k = 0; k < moc::kLiveMaxN / 32; ++k) q.sinks[k] = g->live_sinks[k];
+    for (int c = 2; c <= moc::kLivePlanes; ++c)
+        for (int32_t v = 0; v < g->n; ++v)
+            if (c <= (g->h_cap.empty() ? g->C : g->h_cap[v])) q.allow[c - 2][g->h_live_place[v] >> 5] |= 1u << (g->h_live_place[v] & 31);
+    q.seqs = seqs;
+    q.lens = lens;
+    q.offs = offs;
+    q.out_peak = out_peak;
+    q.out_dur = out_dur;
+    q.out_status = out_feasible;
+    // groups of 32 sequences; one block per SM, as many warps as it takes to have every group at once (at most 16)
+    const int64_t groups = ((int64_t)B + 31) / 32, per_sm = (groups + g->sm_count - 1) / g->sm_count, rounds = (per_sm + 15) / 16;
+    const int wpb = (int)std::max<int64_t>((per_sm + rounds - 1) / rounds, 1);
+    const int grid = (int)std::min<int64_t>(g->sm_count, (groups + wpb - 1) / wpb);
+    if (g->ev_before) MOC_CUDA(cudaEventRecord(g->ev_before, st));
+    pl.live_fn<<<grid, 32 * wpb, moc::live_smem_bytes(g->n, live_words(g->n)), st>>>(q);
+    ++g_launches;
+    MOC_CUDA(cudaGetLastError());
+    if (g->ev_after) MOC_CUDA(cudaEventRecord(g->ev_after, st));
+    return MOC_OK;
+}
+
 // Enqueues the evaluation of plan `pl`.  With `offs` the evaluation kernel reads the row offsets
 // from that array, which the offsets kernel fills first from the lengths when `fill_offs` is set
 // (packed rows) and which the caller has filled otherwise; with offs == nullptr (only the
@@ -646,6 +711,7 @@ int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, in
         if (rc != MOC_OK) return rc;
     }
     const Plan& pl = g->plan_eval;
+    if (live_serves(g, pl, B)) return enqueue_live(g, pl, nullptr, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     if (rows_without_scratch(pl, B))
         return enqueue_eval(g, pl, nullptr, false, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     int rc = ensure((void**)&g->d_offs, &g->offs_cap, ((size_t)B + 1) * sizeof(int64_t));
@@ -667,6 +733,7 @@ int eval_rows(const moc_graph* g, const int64_t* offs, const int32_t* seqs, cons
         if (rc != MOC_OK) return rc;
     }
     const Plan& pl = g->plan_eval;
+    if (live_serves(g, pl, B)) return enqueue_live(g, pl, offs, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     if (pl.global_state) {
         int rc = ensure((void**)&g->d_state, &g->state_cap, (size_t)pl.grid * pl.group_bytes);
         if (rc != MOC_OK) return rc;
@@ -787,6 +854,49 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
             if (succ_start[v + 1] == succ_start[v]) g->sink_m += m[v];
         up((void**)&g->d_pred_start, pred_start.data(), ((size_t)n + 1) * 4);
         up((void**)&g->d_pred, pred.data(), (size_t)ne * 4);
+    }
+    if (n <= moc::kLiveMaxN) {
+        // The nodes are dealt to the mask words so that the predecessors of a node lie in different words where
+        // possible (moc_live_kernel.cuh): each node, most consumers first, goes to the word with the fewest other
+        // predecessors of its consumers.
+        const int words = live_words(n);
+        std::vector<uint32_t> preds;
+        try {
+            preds.assign((size_t)n * words, 0u);
+                        std::vector<int32_t> order((size_t)n), clash((size_t)n * words, 0), fill((size_t)words, 0);
+            for (int32_t v = 0; v < n; ++v) order[v] = v;
+            std::stable_sort(order.begin(), order.end(),
+                             [&](int32_t x, int32_t y) { return succ_start[x + 1] - succ_start[x] > succ_start[y + 1] - succ_start[y]; });
+            g->h_live_place.assign((size_t)n, 0);
+            for (int32_t u : order) {
+                int best = -1, best_clash = 0;
+                for (int k = 0; k < words; ++k) {
+                    int c = 0;
+                    for (int32_t e = succ_start[u]; e < succ_start[u + 1]; ++e) c += clash[(size_t)succ[e] * words + k];
+                    c += clash[(size_t)u * words + k];          // the node counts among its predecessors
+                    if (fill[k] < 32 && (best < 0 || c < best_clash || (c == best_clash && fill[k] < fill[best]))) { best = k; best_clash = c; }
+                }
+                for (int32_t e = succ_start[u]; e < succ_start[u + 1]; ++e) {
+                    ++clash[(size_t)succ[e] * words + best];
+                    preds[(size_t)succ[e] * words + best] |= 1u << fill[best];
+                }
+                ++clash[(size_t)u * words + best];
+                if (succ_start[u + 1] == succ_start[u]) g->live_sinks[best] |= 1u << fill[best];
+                g->h_live_place[u] = best << 5 | fill[best]++;
+            }
+        } catch (const std::bad_alloc&) {
+            moc_graph_destroy(g);
+            return fail(MOC_ERR_NOMEM, "host allocation failed");
+        }
+        for (int wide = 0; wide < 2; ++wide) {
+            try {
+                const std::vector<uint32_t> image = moc::live_image(n, words, wide != 0, g->h_live_place, preds, m, w);
+                up((void**)(wide ? &g->d_live64 : &g->d_live32), image.data(), image.size() * 4);
+            } catch (const std::bad_alloc&) {
+                moc_graph_destroy(g);
+                return fail(MOC_ERR_NOMEM, "host allocation failed");
+            }
+        }
     }
     up((void**)&g->d_w, w, (size_t)n * 8);
     up((void**)&g->d_m64, m, (size_t)n * 8);
@@ -1047,6 +1157,8 @@ void moc_graph_destroy(moc_graph* g) {
     cudaFree(g->d_order32);
     cudaFree(g->d_order64);
     cudaFree(g->d_succ16);
+    cudaFree(g->d_live32);
+    cudaFree(g->d_live64);
     if (g->h_stage) cudaFreeHost(g->h_stage);
     if (g->copy_stream) {
         cudaStreamDestroy(g->copy_stream);

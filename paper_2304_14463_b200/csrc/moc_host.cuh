@@ -12,6 +12,7 @@
 #include "moc_pair_kernel.cuh"
 #include "moc_lane_kernel.cuh"
 #include "moc_quad_kernel.cuh"
+#include "moc_live_kernel.cuh"
 
 namespace moc_host {
 
@@ -19,6 +20,7 @@ using KernelFn = void (*)(const moc::EvalParams);
 using PairFn = void (*)(const moc::PairParams);
 using LaneFn = void (*)(const moc::LaneParams);
 using QuadFn = void (*)(const moc::QuadParams);
+using LiveFn = void (*)(const moc::LiveParams);
 
 struct Plan {
     bool valid = false;
@@ -39,6 +41,9 @@ struct Plan {
     bool quad = false;
     QuadFn quad_fn = nullptr;
     uint32_t quad_word_b = 0, quad_cnt_b = 0;
+    // small graphs, large batches: a lane per sequence, walked backwards (null: the graph or a forced kind rules it out)
+    LiveFn live_fn = nullptr;
+    const uint32_t* live_image = nullptr;
     // sequence-per-lane path for C <= 2: a block keeps a group of 8, 16 or 32 sequences on chip
     bool lane = false;
     LaneFn lane_fn = nullptr;
@@ -113,6 +118,10 @@ struct moc_graph {
     uint4* d_order32 = nullptr;           // block-per-sequence kernel: 32-byte node records by falling out-degree (32- / 64-bit m)
     uint4* d_order64 = nullptr;
     uint16_t* d_succ16 = nullptr;         // ... and the successors beyond a node's eighth
+    uint32_t* d_live32 = nullptr;         // backward walk (n <= 128): its tables for 32-bit and for 64-bit sums
+    uint32_t* d_live64 = nullptr;
+    std::vector<int32_t> h_live_place;
+    uint32_t live_sinks[moc::kLiveMaxN / 32] = {};
     cudaEvent_t ev_before = nullptr, ev_after = nullptr;  // measurement hook around the evaluation kernel
     // sliced-ELL successor lists in out-degree order (null when the fast path cannot serve the graph)
     int32_t sell_len = 0, n_tiles = 0;

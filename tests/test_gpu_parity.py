@@ -61,6 +61,33 @@ def test_pins_through_the_gpu(B):
         pin(lambda n, e, w, m, C: GpuGraph(n, e, w, m, C))
 
 
+@pytest.mark.parametrize("n,C,scale,nB", [(1, 2, 1, 5200), (2, 1, 1, 5201), (31, 2, 1, 12000), (32, 4, 1, 6011), (33, 3, 1 << 26, 6001),
+                                          (64, 2, 1 << 26, 9003), (65, 3, 1, 9009), (96, 2, 1, 19200), (127, 4, 1, 14001),
+                                          (128, 2, 1, 70001), (128, 1, 1 << 26, 14400)])
+def test_backward_walk_edges(B, n, C, scale, nB):
+    """Batches that the lane-per-sequence walk serves: mask words full and just begun, both sum widths, one to
+    four copies, per-node caps, damaged sequences, groups of 32 that do not come out even, more groups than one
+    round holds, rows and lengths off a 16-byte boundary."""
+    edges = [] if n < 3 else W.layered_dag(n, min(3 * n, n * (n - 1) // 4), max(2, min(11, n // 3)), n)
+    w, m = W.weights_uniform(n, 0, 30, n, 1), W.weights_lognormal(n, 6.0, 1.5, n, 2) * scale
+    seqs, lens = W.schedules(n, edges, C, 0.3, nB, n)
+    if n > 1:
+        seqs, lens = W.mutate(seqs, lens, n, C, seed=5, frac=1 / 16)
+    O, G = OracleGraph(n, edges, w, m, C), B.Graph(n, edges, w, m, C)
+    M = O.eval(np.arange(n), 1 << 62)["peak"] * 95 // 100
+    assert_batch_equal(G, O, seqs, lens, M, "uniform cap")
+    assert B.moc_last_launch_count() == 1
+    caps = np.random.RandomState(n).randint(1, C + 1, n).astype(np.int32)
+    G.set_caps(caps)
+    O.set_caps(caps)
+    s, l = torch.zeros(len(seqs) + 3, dtype=torch.int32, device="cuda"), torch.zeros(nB + 1, dtype=torch.int32, device="cuda")
+    s[3:], l[1:] = dev(seqs), dev(lens)
+    got = G.eval_batch(s[3:], l[1:], M)
+    torch.cuda.synchronize()
+    for a, b in zip(got, O.eval_batch(seqs, lens, M)):
+        assert (a.cpu().numpy() == b).all()
+
+
 # ------------------------------------------------------------------ the five configurations
 SMALL_B = [1024, 4096, 2048, 512, 64]
 
