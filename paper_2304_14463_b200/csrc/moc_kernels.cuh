@@ -344,15 +344,15 @@ __global__ void __launch_bounds__(1024) eval_global_kernel(const EvalParams p) {
 // offs = exclusive prefix sum of max(lens, 0); offs[B] = total.
 // Block j owns elements [j*kOffsTile, (j+1)*kOffsTile): it first adds up everything in front of its
 // tile (redundantly with the other blocks -- B is small, and this needs no cross-block handshake),
-// then scans its own tile.
-constexpr int kOffsThreads = 256;
-constexpr int kOffsPer = 4;
-constexpr int kOffsTile = kOffsThreads * kOffsPer;
+// then scans its own tile.  The last block's sum decides: 1024 threads with eight 16-byte loads in flight each take
+// two rounds of memory latency for 61440 lengths, where 256 threads with four took fifteen (18 us at B = 65536).
+constexpr int kOffsThreads = 1024;
+constexpr int kOffsTile = kOffsThreads;
 
 static __global__ void __launch_bounds__(kOffsThreads) offsets_kernel(const int32_t* __restrict__ lens, int32_t B,
                                                                 int64_t* __restrict__ offs) {
-    __shared__ int64_t wsum[kOffsThreads / 32];
-    __shared__ int64_t wtot[kOffsThreads / 32];
+    static_assert(kOffsThreads == 1024, "one warp combines the sums of 32 warps");
+    __shared__ int64_t wsum[32], wtot[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t tile0 = (int64_t)blockIdx.x * kOffsTile;
     // ---- sum of everything before the tile (16-byte loads, several in flight per thread)
@@ -360,21 +360,13 @@ static __global__ void __launch_bounds__(kOffsThreads) offsets_kernel(const int3
     if ((reinterpret_cast<uintptr_t>(lens) & 15) == 0) {
         const int4* l4 = reinterpret_cast<const int4*>(lens);
         const int64_t n4 = tile0 >> 2;  // the tile size is a multiple of 4
-        int64_t s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-        int64_t i = tid;
-        for (; i + 3 * kOffsThreads < n4; i += 4 * kOffsThreads) {
-            const int4 a = __ldg(l4 + i), b = __ldg(l4 + i + kOffsThreads), c = __ldg(l4 + i + 2 * kOffsThreads),
-                       d = __ldg(l4 + i + 3 * kOffsThreads);
-            s0 += (int64_t)max(a.x, 0) + max(a.y, 0) + max(a.z, 0) + max(a.w, 0);
-            s1 += (int64_t)max(b.x, 0) + max(b.y, 0) + max(b.z, 0) + max(b.w, 0);
-            s2 += (int64_t)max(c.x, 0) + max(c.y, 0) + max(c.z, 0) + max(c.w, 0);
-            s3 += (int64_t)max(d.x, 0) + max(d.y, 0) + max(d.z, 0) + max(d.w, 0);
+        for (int64_t i = tid; i < n4; i += 8 * kOffsThreads) {
+            int4 a[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) a[k] = i + k * kOffsThreads < n4 ? __ldg(l4 + i + k * kOffsThreads) : make_int4(0, 0, 0, 0);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s += (int64_t)max(a[k].x, 0) + max(a[k].y, 0) + max(a[k].z, 0) + max(a[k].w, 0);
         }
-        for (; i < n4; i += kOffsThreads) {
-            const int4 a = __ldg(l4 + i);
-            s0 += (int64_t)max(a.x, 0) + max(a.y, 0) + max(a.z, 0) + max(a.w, 0);
-        }
-        s = s0 + s1 + s2 + s3;
     } else {
         for (int64_t i = tid; i < tile0; i += kOffsThreads) {
             const int32_t v = __ldg(lens + i);
@@ -383,31 +375,20 @@ static __global__ void __launch_bounds__(kOffsThreads) offsets_kernel(const int3
     }
     s = warp_sum(s);
     if (lane == 0) wtot[warp] = s;
-    // ---- own tile: kOffsPer consecutive elements per thread
-    int32_t loc[kOffsPer];
-    int64_t t = 0;
-#pragma unroll
-    for (int k = 0; k < kOffsPer; ++k) {
-        const int64_t i = tile0 + tid * kOffsPer + k;
-        const int32_t v = i < B ? __ldg(lens + i) : 0;
-        loc[k] = v > 0 ? v : 0;
-        t += loc[k];
-    }
-    const int64_t incl = warp_inclusive_sum(t, lane);
+    // ---- own tile: one element per thread, then the warps' sums
+    const int64_t i = tile0 + tid;
+    const int32_t v = i < B ? max(__ldg(lens + i), 0) : 0;
+    const int64_t incl = warp_inclusive_sum((int64_t)v, lane);
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
-    int64_t run = incl - t;
-    for (int k = 0; k < kOffsThreads / 32; ++k) {
-        run += wtot[k];
-        if (k < warp) run += wsum[k];
+    if (warp == 0) {
+        const int64_t mine = wsum[lane];
+        wsum[lane] = warp_sum(wtot[lane]) + warp_inclusive_sum(mine, lane) - mine;
     }
-#pragma unroll
-    for (int k = 0; k < kOffsPer; ++k) {
-        const int64_t i = tile0 + tid * kOffsPer + k;
-        if (i < B) offs[i] = run;
-        run += loc[k];
-        if (i == B - 1) offs[B] = run;
-    }
+    __syncthreads();
+    const int64_t run = wsum[warp] + incl - v;
+    if (i < B) offs[i] = run;
+    if (i == B - 1) offs[B] = run + v;
 }
 
 // 16-bit node ids -> 32-bit node ids (the evaluation kernels read int32 rows); 8 ids per thread and
