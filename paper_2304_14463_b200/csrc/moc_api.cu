@@ -249,7 +249,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     // Order of preference when nothing is forced: warp per sequence, then sequence per lane (it also
     // serves graphs whose degrees are too uneven for the warp kernel's padded successor tiles), then
     // the thread-group kernel, which serves everything.
-    const bool warp_ok = C <= 2 && g->d_rec32 != nullptr && (__int128)C * g->sum_w < ((__int128)1 << 48);
+    const bool warp_ok = C <= 2 && g->d_rec32 != nullptr && (!pl.wide || g->split_ok) && (__int128)C * g->sum_w < ((__int128)1 << 48);
     if (kind == MOC_KERNEL_LANE || (kind == MOC_KERNEL_AUTO && !shape_given && !warp_ok)) {
         const char* why = plan_lane(g, smem_cap, &pl);
         if (!why) {
@@ -267,7 +267,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         if (kind == MOC_KERNEL_BLOCK) return fail(MOC_ERR_ARG, "the block-per-sequence kernel cannot serve this graph: %s", why);
     }
     if (kind == MOC_KERNEL_WARP && !warp_ok)
-        return fail(MOC_ERR_ARG, "the warp-per-sequence kernel cannot serve this graph (C > 2, degrees too uneven or C * sum(w) >= 2^48)");
+        return fail(MOC_ERR_ARG, "the warp-per-sequence kernel cannot serve this graph (C > 2, degrees too uneven, C * sum(w) >= 2^48 or sum(m) too large)");
     if (!profile && g->want_G == 0 && kind != MOC_KERNEL_GROUP && warp_ok) {
         // warp-per-sequence fast path
         const size_t msz = pl.wide ? 8 : 4, per_vec = 16 / msz;
@@ -604,9 +604,17 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
                 best_nb = nb;
             }
         }
+        grid = (int)std::min<int64_t>((int64_t)pl.sm_count * best_nb, ((int64_t)B + best_w - 1) / best_w);
+        // A batch that one round of 16 warps per SM holds is bound by the latency of a sequence: spread it over all
+        // SMs, with at least eight warps per block to stage the graph (n = 353, 64-bit sums, B = 1501: 11 warps on
+        // 148 SMs instead of 16 on 94).
+        const int spread = (int)std::max<int64_t>(8, ((int64_t)B + pl.sm_count - 1) / pl.sm_count);
+        if (spread <= 16 && pl.pair_nb[spread] >= 1 && (g->want_kind != MOC_KERNEL_WARP || g->want_b == 0)) {
+            best_w = spread;
+            grid = std::min(B, pl.sm_count);
+        }
         block = 32 * best_w;
         smem = pl.pair_graph_b + (size_t)best_w * pl.pair_warp_b;
-        grid = (int)std::min<int64_t>((int64_t)pl.sm_count * best_nb, ((int64_t)B + best_w - 1) / best_w);
     }
     if (offs && fill_offs) {
         moc::offsets_kernel<<<(B + moc::kOffsTile - 1) / moc::kOffsTile, moc::kOffsThreads, 0, st>>>(lens, B, offs);
@@ -678,6 +686,7 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         q.out_status = out_feasible;
         q.rec_bytes = pl.rec_bytes; q.w_bytes = pl.w_bytes; q.sell_bytes = pl.sell_bytes;
         q.word_bytes = pl.word_bytes; q.delta_bytes = pl.delta_bytes;
+        q.split = g->split;
         MOC_CUDA(cudaLaunchKernelEx(&cfg, pl.pair_fn, q));
     } else {
         moc::EvalParams p = base_params(g, pl);
@@ -933,6 +942,11 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
             if (sell_len <= 2 * ne + 4096 && sell_len < (1 << 20) && max_rows < (1 << 12) && 4 * ((int64_t)n + 3) < 65536) {
                 const uint32_t word_b = (uint32_t)align16(4 * ((size_t)n + 2));   // the constant word (1, 1) sits right after the words
                 std::vector<uint32_t> rec32((size_t)n_halves * 32 * 2), rec64((size_t)n_halves * 32 * 4, 0u);
+                // 64-bit sums: parts of m that 32-bit atomics can add (moc_pair_kernel.cuh), where sum(m) permits
+                int k = 31;
+                while (((int64_t)1 << (31 - k)) < n) --k;
+                g->split_ok = (sum_m >> k) < ((int64_t)1 << 31);
+                g->split = g->split_ok ? k : 32;
                 // entry (row k, lane l) of a tile: word of the k-th successor of the node in half 0 | same for half 1 << 16;
                 // a list that is used up continues with the node's own word
                 std::vector<uint32_t> sell((size_t)std::max<int64_t>(sell_len, 1), word_b | (word_b << 16));
@@ -945,7 +959,7 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
                     rec32[2 * r + 1] = v >= 0 ? (uint32_t)m32[v] : 0u;
                     rec64[4 * r + 0] = x;
                     rec64[4 * r + 2] = (uint32_t)(mv & 0xFFFFFFFFu);
-                    rec64[4 * r + 3] = (uint32_t)(mv >> 32);
+                    rec64[4 * r + 3] = (uint32_t)(mv >> g->split);
                 }
                 uint32_t pos = 0;
                 std::vector<std::vector<int32_t>> rem(32);

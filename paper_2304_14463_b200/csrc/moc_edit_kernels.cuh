@@ -66,6 +66,7 @@ struct PrepParams {
     // successor tiles of the warp-per-sequence evaluation kernel (moc_pair_kernel.cuh), read through L1;
     // n_tiles = 0: not available, the node pass walks the plain successor lists
     int32_t n_tiles;
+    int32_t split;              // records with 64-bit sums: bits of the low part of m
     const void* rec;
     const uint64_t* wslot;
     const uint32_t* sell;
@@ -233,7 +234,8 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                             const uint4 r = kChip ? lds_v4((uint32_t)__cvta_generic_to_shared(prec + 32 * kRecB * h))
                                                   : __ldg(reinterpret_cast<const uint4*>(prec + 32 * kRecB * h));
                             x = r.x;
-                            mm[h] = (MemT)((uint64_t)r.z | ((uint64_t)r.w << 32));
+                            // m from its two parts (moc_pair_kernel.cuh)
+                            mm[h] = (MemT)((uint64_t)r.w << p.split | (r.z & (uint32_t)(((uint64_t)1 << p.split) - 1)));
                         }
                         if (h == 0) rows = (int)(x >> 16);
                         xoff[h] = x & 0xFFFFu;

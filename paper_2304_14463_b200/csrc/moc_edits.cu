@@ -38,6 +38,7 @@ int cache_prepare(moc_cache* h, const int32_t* seqs, const int32_t* lens, const 
     const bool tiles = g->d_rec32 != nullptr && g->C <= 2 && (__int128)g->C * g->sum_w < ((__int128)1 << 48);
     p.n_tiles = tiles ? g->n_tiles : 0;
     p.rec = h->wide ? g->d_rec64 : g->d_rec32;
+    p.split = g->split;
     p.wslot = g->d_wslot;
     p.sell = g->d_sell;
     p.base_dur = g->sum_w;

@@ -125,6 +125,8 @@ struct moc_graph {
     cudaEvent_t ev_before = nullptr, ev_after = nullptr;  // measurement hook around the evaluation kernel
     // sliced-ELL successor lists in out-degree order (null when the fast path cannot serve the graph)
     int32_t sell_len = 0, n_tiles = 0;
+    int32_t split = 32;                   // d_rec64: m as (m mod 2^32, m >> split); split_ok: the kernels may add the parts separately
+    bool split_ok = false;
     void* d_rec32 = nullptr;  // node records with 32-bit / 64-bit output sizes
     void* d_rec64 = nullptr;
     uint64_t* d_wslot = nullptr;

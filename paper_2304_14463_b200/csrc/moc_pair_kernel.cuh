@@ -63,10 +63,24 @@ struct PairParams {
     // shared-memory layout, bytes (multiples of 16)
     uint32_t rec_bytes, w_bytes, sell_bytes;     // graph, once per block
     uint32_t word_bytes, delta_bytes;            // per warp; 16 bytes after the words hold the constant (1, 1)
+    int32_t split;                               // 64-bit sums: position k of the high part of an amount (below)
 };
 
-// Node record: {byte offset of the node's word | rows of the tile << 16, m}; m takes 32 bits, or 64
-// bits after a pad word.
+// Node record: {byte offset of the node's word | rows of the tile << 16, m}; m takes 32 bits, or, for 64-bit
+// sums, two words after a pad word: m mod 2^32 and m >> k.
+//
+// 64-bit sums without 64-bit atomics (which shared memory emulates with compare-and-swap loops: twice the time
+// of the whole kernel).  A delta entry is two 32-bit words that are added to separately: the amounts mod 2^32, and the
+// amounts >> k.  A sum S of deltas up to some step is a difference of two sets of resident outputs, at most
+// n of them each, so that with L and H the sums of the two words
+//     S = 2^k H + (something below n 2^k in absolute value),   S = L (mod 2^32),
+// which determines S when n 2^k <= 2^31: S = 2^k H + sign-extended (L - 2^k H mod 2^32).  H itself fits 32 bits when
+// sum(m) < 2^(31 + k); graphs beyond that (sum(m) >= 2^53 at n = 442) use the general kernels.
+template <typename MemT> struct Amount { MemT v; };
+template <> struct Amount<int64_t> { uint32_t lo, hi; };
+__device__ __forceinline__ int64_t split_value(uint32_t lo, uint32_t hi, int32_t k) {
+    return ((int64_t)(int32_t)hi << k) + (int32_t)(lo - (hi << k));
+}
 constexpr uint64_t kPairDurMask = (uint64_t(1) << 48) - 1;   // bits 0..47 of the summed wslot entries: w of the second copies
 constexpr int kPairCntShift = 48;                             // bits 48..62: number of nodes with two copies
 
@@ -113,6 +127,16 @@ __device__ __forceinline__ void red_add_shared(uint32_t addr, int32_t v) {
 }
 __device__ __forceinline__ void red_add_shared(uint32_t addr, int64_t v) {
     asm volatile("red.shared.add.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void red_add_amount(uint32_t addr, Amount<int32_t> a) { red_add_shared(addr, a.v); }
+__device__ __forceinline__ void red_sub_amount(uint32_t addr, Amount<int32_t> a) { red_add_shared(addr, -a.v); }
+__device__ __forceinline__ void red_add_amount(uint32_t addr, Amount<int64_t> a) {
+    red_add_shared(addr, (int32_t)a.lo);
+    red_add_shared(addr + 4u, (int32_t)a.hi);
+}
+__device__ __forceinline__ void red_sub_amount(uint32_t addr, Amount<int64_t> a) {
+    red_add_shared(addr, (int32_t)(0u - a.lo));
+    red_add_shared(addr + 4u, (int32_t)(0u - a.hi));
 }
 __device__ __forceinline__ uint32_t lds_u32_nv(uint32_t addr) {
     uint32_t v;
@@ -221,7 +245,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
         return (int64_t)lo + ((int64_t)hi << 16);
     };
     if (!self) {
-        b = blockIdx.x * wpb + warp;
+        b = blockIdx.x + gridDim.x * warp;      // a batch smaller than the grid's warps spreads over all blocks
         b_end = p.B;
         b_step = n_warps;
         if (b < b_end) { off = __ldg(&p.offs[b]); T = __ldg(&p.lens[b]); }
@@ -373,7 +397,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                 uint32_t prec = rec0, pw = w0, ps = sell0;
                 for (int d = 0; d < n_tiles; ++d, prec += 64u * kRecB, pw += 512u) {
                     uint32_t ab[2], naa[2], nbb[2], Ga[2], Gb[2];
-                    MemT m[2];
+                    Amount<MemT> m[2];
                     int rows = 0;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -381,11 +405,12 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                         if constexpr (sizeof(MemT) == 4) {
                             const uint2 r = lds_v2(prec + 32u * kRecB * h);
                             x = r.x;
-                            m[h] = (MemT)r.y;
+                            m[h].v = (MemT)r.y;
                         } else {
                             const uint4 r = lds_v4(prec + 32u * kRecB * h);
                             x = r.x;
-                            m[h] = (MemT)((uint64_t)r.z | ((uint64_t)r.w << 32));
+                            m[h].lo = r.z;
+                            m[h].hi = r.w;
                         }
                         if (h == 0) rows = (int)(x >> 16);
                         const uint32_t own = lds_u32(wa + (x & 0xFFFFu));
@@ -417,12 +442,11 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                         const uint32_t gg = max_u16x2(__byte_perm(Ga[h], Gb[h], 0x5410), __byte_perm(Ga[h], Gb[h], 0x7632));
                         const uint32_t v = gg + ab[h];                           // (end of b, end of a) mod 2^16
                         const uint32_t a16 = ab[h] & 0xFFFFu, b16 = ab[h] >> 16;
-                        const MemT neg_m = -m[h];
-                        red_add_shared(da1 + (b16 << kShift), m[h]);
-                        red_add_shared(da + ((v & 0xFFFFu) << kShift), neg_m);
+                        red_add_amount(da1 + (b16 << kShift), m[h]);
+                        red_sub_amount(da + ((v & 0xFFFFu) << kShift), m[h]);
                         if (a16 != b16) {
-                            red_add_shared(da1 + (a16 << kShift), m[h]);
-                            red_add_shared(da + ((v >> 16) << kShift), neg_m);
+                            red_add_amount(da1 + (a16 << kShift), m[h]);
+                            red_sub_amount(da + ((v >> 16) << kShift), m[h]);
                             // bit 63 of the duration marks a node that may have one copy only (C_v = 1)
                             const uint64_t wx = lds_u64(pw + 256u * h);
                             capw |= (uint32_t)(wx >> 32);
@@ -449,34 +473,38 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                 // One pass: the lane's running prefix and the largest prefix it sees; the largest
                 // usage inside the lane's chunk is then (sum of the chunks before it) + that maximum.
                 const int4* d4 = reinterpret_cast<const int4*>(delta_base + kPairDeltaFront) + lane * V;
-                MemT run = 0, top;
-                {
-                    const int4 q = d4[0];
-                    if constexpr (sizeof(MemT) == 4) {
+                MemT peak;
+                if constexpr (sizeof(MemT) == 4) {
+                    MemT run = 0, top;
+                    {
+                        const int4 q = d4[0];
                         run = q.x; top = run;
                         run += q.y; top = max(top, run);
                         run += q.z; top = max(top, run);
                         run += q.w; top = max(top, run);
-                    } else {
-                        const longlong2 l = *reinterpret_cast<const longlong2*>(&q);
-                        run = (MemT)l.x; top = run;
-                        run += (MemT)l.y; top = run > top ? run : top;
                     }
-                }
-                for (int j = 1; j < V; ++j) {
-                    const int4 q = d4[j];
-                    if constexpr (sizeof(MemT) == 4) {
+                    for (int j = 1; j < V; ++j) {
+                        const int4 q = d4[j];
                         run += q.x; top = max(top, run);
                         run += q.y; top = max(top, run);
                         run += q.z; top = max(top, run);
                         run += q.w; top = max(top, run);
-                    } else {
-                        const longlong2 l = *reinterpret_cast<const longlong2*>(&q);
-                        run += (MemT)l.x; top = run > top ? run : top;
-                        run += (MemT)l.y; top = run > top ? run : top;
                     }
+                    peak = warp_inclusive_sum(run, lane) - run + top;
+                } else {
+                    uint32_t lo = 0, hi = 0;
+                    int64_t top = INT64_MIN;
+                    for (int j = 0; j < V; ++j) {
+                        const int4 q = d4[j];
+                        lo += (uint32_t)q.x; hi += (uint32_t)q.y;
+                        const int64_t u = split_value(lo, hi, p.split);
+                        lo += (uint32_t)q.z; hi += (uint32_t)q.w;
+                        const int64_t w = split_value(lo, hi, p.split);
+                        top = u > top ? u : top;
+                        top = w > top ? w : top;
+                    }
+                    peak = split_value(warp_inclusive_sum(lo, lane) - lo, warp_inclusive_sum(hi, lane) - hi, p.split) + top;
                 }
-                const MemT peak = warp_inclusive_sum(run, lane) - run + top;
                 out_pk = (int64_t)warp_max_t(peak);
                 out_du = p.base_dur + dur_extra;
                 out_st = out_pk <= p.M ? 1 : 0;

@@ -105,11 +105,13 @@ void plan_walk(moc_search* s) {
     const moc_graph* g = s->g;
     if (g->C > 2 || g->d_rec32 == nullptr) return;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    if (wide && !g->split_ok) return;
     const size_t per_vec = wide ? 2 : 4, nvec = ((size_t)g->C * g->n + 2 + per_vec - 1) / per_vec, v_max = ((nvec + 31) / 32) | 1;
     moc::WalkParams& w = s->wp;
     w.n = g->n;
     w.C = g->C;
     w.n_tiles = g->n_tiles;
+    w.split = g->split;
     w.rec = wide ? g->d_rec64 : g->d_rec32;
     w.sell = g->d_sell;
     w.succ_start = g->d_succ_start;

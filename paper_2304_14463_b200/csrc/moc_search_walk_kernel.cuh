@@ -40,6 +40,7 @@ struct WalkParams {
     int32_t lanes_per_gen;     // E rounded up to a power of two, at most 32
     int32_t* peak_at;          // P: where the peak of each chain's sequence lies (walk_eval's `at`), 0: not known
     int32_t n, C, n_tiles;
+    int32_t split;             // 64-bit sums: as in PairParams
     const void* rec;           // node records and successor tiles of the warp-per-sequence layout
     const uint32_t* sell;
     const int32_t* succ_start;
@@ -76,14 +77,14 @@ __device__ __forceinline__ uint32_t walk_above(uint32_t p, uint32_t k) {
 // (1-based; one vector of deltas).  The deltas are zero on entry and on return.
 template <typename MemT>
 __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec0, uint32_t sell0, int n_tiles, int32_t T, int lane,
-                                       bool& dep, int32_t& at) {
+                                       int32_t split, bool& dep, int32_t& at) {
     constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
     constexpr int kPerVec = 16 / (int)sizeof(MemT), kShift = sizeof(MemT) == 4 ? 2 : 3;
     const uint32_t da1 = da - (uint32_t)sizeof(MemT);
     uint32_t depw = 0, prec = rec0, ps = sell0;
     for (int d = 0; d < n_tiles; ++d, prec += 64u * kRecB) {
         uint32_t ab[2], naa[2], nbb[2], Ga[2], Gb[2];
-        MemT m[2];
+        Amount<MemT> m[2];
         int rows = 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -91,11 +92,12 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
             if constexpr (sizeof(MemT) == 4) {
                 const uint2 r = lds_v2(prec + 32u * kRecB * h);
                 x = r.x;
-                m[h] = (MemT)r.y;
+                m[h].v = (MemT)r.y;
             } else {
                 const uint4 r = lds_v4(prec + 32u * kRecB * h);
                 x = r.x;
-                m[h] = (MemT)((uint64_t)r.z | ((uint64_t)r.w << 32));
+                m[h].lo = r.z;
+                m[h].hi = r.w;
             }
             if (h == 0) rows = (int)(x >> 16);
             const uint32_t own = lds_u32(wa + (x & 0xFFFFu)), sw = swap_halves(own);
@@ -122,11 +124,11 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
             depw |= Ga[h];
             const uint32_t gg = max_u16x2(__byte_perm(Ga[h], Gb[h], 0x5410), __byte_perm(Ga[h], Gb[h], 0x7632));
             const uint32_t v = gg + ab[h], a16 = ab[h] & 0xFFFFu, b16 = ab[h] >> 16;
-            red_add_shared(da1 + (b16 << kShift), m[h]);
-            red_add_shared(da + ((v & 0xFFFFu) << kShift), (MemT)-m[h]);
+            red_add_amount(da1 + (b16 << kShift), m[h]);
+            red_sub_amount(da + ((v & 0xFFFFu) << kShift), m[h]);
             if (a16 != b16) {
-                red_add_shared(da1 + (a16 << kShift), m[h]);
-                red_add_shared(da + ((v >> 16) << kShift), (MemT)-m[h]);
+                red_add_amount(da1 + (a16 << kShift), m[h]);
+                red_sub_amount(da + ((v >> 16) << kShift), m[h]);
             }
         }
     }
@@ -135,24 +137,30 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
     // prefix sum and running maximum; lane owns V consecutive vectors, which it clears behind itself
     const int nvec = (T + 2 + kPerVec - 1) / kPerVec, V = ((nvec + 31) >> 5) | 1;
     uint32_t ad = da + 16u * (uint32_t)(lane * V);
-    MemT run = 0, top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
+    MemT top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
     int vec = 0;                       // the lane's vector that holds its maximum
+    MemT run = 0;
+    uint32_t lo = 0, hi = 0;           // 64-bit sums: the two parts of the running sum (moc_pair_kernel.cuh)
     for (int j = 0; j < V; ++j, ad += 16u) {
         const uint4 q = lds_v4(ad);
         asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(ad), "r"(0) : "memory");
-        MemT hi;
+        MemT most;
         if constexpr (sizeof(MemT) == 4) {
-            run += (MemT)q.x; hi = run;
-            run += (MemT)q.y; hi = max(hi, run);
-            run += (MemT)q.z; hi = max(hi, run);
-            run += (MemT)q.w; hi = max(hi, run);
+            run += (MemT)q.x; most = run;
+            run += (MemT)q.y; most = max(most, run);
+            run += (MemT)q.z; most = max(most, run);
+            run += (MemT)q.w; most = max(most, run);
         } else {
-            run += (MemT)((uint64_t)q.x | (uint64_t)q.y << 32); hi = run;
-            run += (MemT)((uint64_t)q.z | (uint64_t)q.w << 32); hi = run > hi ? run : hi;
+            lo += q.x; hi += q.y;
+            most = split_value(lo, hi, split);
+            lo += q.z; hi += q.w;
+            const MemT u = split_value(lo, hi, split);
+            most = u > most ? u : most;
         }
-        if (hi > top) { top = hi; vec = j; }
+        if (most > top) { top = most; vec = j; }
     }
-    top += warp_inclusive_sum(run, lane) - run;
+    if constexpr (sizeof(MemT) == 4) top += warp_inclusive_sum(run, lane) - run;
+    else top += split_value(warp_inclusive_sum(lo, lane) - lo, warp_inclusive_sum(hi, lane) - hi, split);
     const MemT peak = warp_max_t(top);
     const int src = __ffs(__ballot_sync(kFull, top == peak)) - 1;
     at = kPerVec * (src * V + __shfl_sync(kFull, vec, src)) + 1;
@@ -415,7 +423,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                             }
                             bool dep;
                             int32_t at;
-                            const int64_t pk_s = (int64_t)walk_eval<MemT>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, dep, at);
+                            const int64_t pk_s = (int64_t)walk_eval<MemT>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, p.split, dep, at);
                             const int64_t a_s = pk_s > s.M ? pk_s : s.M, b_a = (int64_t)lds_u64(note + kWalkBestA), b_d = (int64_t)lds_u64(note + kWalkBestD);
                             if (dep || a_s > b_a || (a_s == b_a && (b_has ? du_s >= b_d : du_s > b_d))) continue;
                             b_has = b_here = true;
