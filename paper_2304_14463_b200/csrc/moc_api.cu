@@ -97,9 +97,13 @@ LaneFn lane_fn_lg(int lg, int kp) {
 }
 LaneFn lane_fn(bool wide, int lg, int kp) { return wide ? lane_fn_lg<int64_t>(lg, kp) : lane_fn_lg<int32_t>(lg, kp); }
 
-QuadFn quad_fn(bool wide, int C) {
-    if (C <= 3) return wide ? (QuadFn)moc::eval_quad_kernel<int64_t, 3> : (QuadFn)moc::eval_quad_kernel<int32_t, 3>;
-    return wide ? (QuadFn)moc::eval_quad_kernel<int64_t, 4> : (QuadFn)moc::eval_quad_kernel<int32_t, 4>;
+template <typename MemT, bool kTiles>
+QuadFn quad_fn_c(int C) {
+    return C <= 3 ? (QuadFn)moc::eval_quad_kernel<MemT, 3, kTiles> : (QuadFn)moc::eval_quad_kernel<MemT, 4, kTiles>;
+}
+QuadFn quad_fn(bool wide, int C, bool tiles) {
+    if (tiles) return wide ? quad_fn_c<int64_t, true>(C) : quad_fn_c<int32_t, true>(C);
+    return wide ? quad_fn_c<int64_t, false>(C) : quad_fn_c<int32_t, false>(C);
 }
 
 template <typename SumT, int W>
@@ -191,32 +195,51 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, Plan* out) {
     Plan pl = *out;
     const int64_t n = g->n, C = g->C, t_max = C * n;
     if (C > 4) return "C > 4";
-    if (!g->d_order32) return "n above 32000 or a degree above 65535";
+    if (!g->d_rec32 && !g->d_order) return "n above 32000 or a degree above 65535";
     if (t_max > 32766) return "sequences of more than 32766 steps";
+    if (pl.wide && !g->split_ok) return "sum(m) too large for two-part sums";
     const size_t msz = pl.wide ? 8 : 4;
-    const size_t word_b = align16(8 * (size_t)(n + 2)), cnt_b = align16(2 * (size_t)(n + 2)), delta_b = align16(msz * (size_t)(t_max + 4));
+    const size_t word_b = 2 * align16(4 * (size_t)(n + 2)) + 16, cnt_b = align16(2 * (size_t)(n + 2)), delta_b = align16(msz * (size_t)(t_max + 4));
     const size_t sm = word_b + cnt_b + delta_b;
     if (sm > smem_cap) return "the state of a sequence exceeds shared memory";
-    QuadFn fn = quad_fn(pl.wide, (int)C);
+    QuadFn fn = quad_fn(pl.wide, (int)C, g->d_rec32 != nullptr);
     if (raise_smem_limit((const void*)fn, g->smem_optin) != cudaSuccess) { cudaGetLastError(); return "cudaFuncSetAttribute failed"; }
-    // threads per sequence, from measurements at n = 100, 1000 and 5000 (more threads lose to the block-wide
-    // barriers, fewer to the length of the per-thread loops); or as requested
-    int thr = n < 200 ? 64 : (n < 1600 ? 128 : (n < 12000 ? 512 : 1024));
-    if (g->want_kind == MOC_KERNEL_BLOCK && g->want_a) thr = g->want_a;
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, thr, sm) != cudaSuccess || nb < 1) { cudaGetLastError(); return "kernel does not fit on an SM"; }
+    const int forced = g->want_kind == MOC_KERNEL_BLOCK ? g->want_a : 0;
+    bool any = false;
+    for (int k = 0; k < 5; ++k) {
+        const int thr = forced ? forced : 64 << k;
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, thr, sm) != cudaSuccess) { cudaGetLastError(); nb = 0; }
+        pl.quad_nb[k] = nb;
+        any = any || nb > 0;
+    }
+    if (!any) return "kernel does not fit on an SM";
     pl.quad = true;
     pl.quad_fn = fn;
-    pl.G = thr;
+    pl.quad_forced = forced;
     pl.gpc = 1;
-    pl.block = thr;
     pl.smem = sm;
-    pl.grid = g->sm_count * nb;
+    pl.sm_count = g->sm_count;
+    pl.grid = g->sm_count * std::max(1, pl.quad_nb[1]);
     pl.quad_word_b = (uint32_t)word_b;
     pl.quad_cnt_b = (uint32_t)cnt_b;
     pl.valid = true;
     *out = pl;
     return nullptr;
+}
+
+// Threads per sequence of the block-per-sequence kernel, as an index into Plan::quad_nb (64 << k).  With many sequences,
+// from measurements at n = 100 to 5000: more threads lose to the block-wide barriers, fewer to the length of the
+// per-thread loops.  With few, enough to give every SM about 16 warps.
+int quad_shape(const Plan& pl, int64_t n, int32_t B) {
+    if (pl.quad_forced) return 0;
+    int k = n < 200 ? 0 : (n < 1600 ? 1 : (n < 4000 ? 2 : 3));
+    const int64_t per_sm = ((int64_t)B + pl.sm_count - 1) / pl.sm_count;
+    while (k < 3 && per_sm * (2 << (k + 1)) <= 16) ++k;
+    if (n >= 3000 && per_sm == 1) k = 4;
+    while (k < 4 && pl.quad_nb[k] == 0) ++k;
+    while (k > 0 && pl.quad_nb[k] == 0) --k;
+    return k;
 }
 
 // Backward walk with a lane per sequence: n <= 128, C <= 4.  Used for the batches live_serves() names.
@@ -473,47 +496,36 @@ int build_lane_layouts(moc_graph* g, const std::vector<int32_t>& succ_start, con
     return upload_lane_rec(g);
 }
 
-// Layout for the block-per-sequence kernel: the nodes in order of falling out-degree (a sink counts one:
-// its made-up successor n + 1) with the place of their successor lists, and the lists as 16-bit ids.
-int build_quad_layout(moc_graph* g, const std::vector<int32_t>& succ_start, const std::vector<int32_t>& succ,
-                      const int64_t* m, const std::vector<int32_t>& m32) {
+// Layout for the block-per-sequence kernel on graphs without successor tiles: the nodes in order of falling
+// out-degree (a sink counts one: its made-up successor n + 1) with the place of their successor lists, and the
+// lists as 16-bit ids.
+int build_quad_layout(moc_graph* g, const std::vector<int32_t>& succ_start, const std::vector<int32_t>& succ) {
     const int32_t n = g->n;
-    if (n > 32000) return MOC_OK;
+    if (g->d_rec32 || n > 32000) return MOC_OK;
     auto deg = [&](int32_t v) { return std::max(1, succ_start[v + 1] - succ_start[v]); };
     std::vector<int32_t> order((size_t)n);
     for (int32_t v = 0; v < n; ++v) order[v] = v;
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return deg(x) > deg(y); });
     if (deg(order[0]) > 65535) return MOC_OK;
-    for (int wide = 0; wide < 2; ++wide) {
-        std::vector<uint32_t> rec((size_t)n * 8, 0u);
-        std::vector<uint16_t> rest;
-        for (int32_t i = 0; i < n; ++i) {
-            const int32_t v = order[i];
-            std::vector<uint16_t> ids;
-            if (succ_start[v + 1] == succ_start[v]) ids.push_back((uint16_t)(n + 1));
-            for (int32_t e = succ_start[v]; e < succ_start[v + 1]; ++e) ids.push_back((uint16_t)succ[e]);
-            uint32_t* r = &rec[(size_t)i * 8];
-            r[0] = (uint32_t)v | ((uint32_t)ids.size() << 16);
-            r[1] = (uint32_t)rest.size();
-            if (wide) {
-                r[2] = (uint32_t)((uint64_t)m[v] & 0xFFFFFFFFu);
-                r[3] = (uint32_t)((uint64_t)m[v] >> 32);
-            } else {
-                r[2] = (uint32_t)m32[v];
-            }
-            for (size_t k = 0; k < ids.size(); ++k) {
-                if (k < 8) r[4 + k / 2] |= (uint32_t)ids[k] << (16 * (k & 1));
-                else rest.push_back(ids[k]);
-            }
-        }
-        uint4** dst = wide ? &g->d_order64 : &g->d_order32;
-        MOC_CUDA(cudaMalloc((void**)dst, rec.size() * 4));
-        MOC_CUDA(cudaMemcpy(*dst, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice));
-        if (!wide) {
-            MOC_CUDA(cudaMalloc((void**)&g->d_succ16, std::max<size_t>(rest.size() * 2, 16)));
-            if (!rest.empty()) MOC_CUDA(cudaMemcpy(g->d_succ16, rest.data(), rest.size() * 2, cudaMemcpyHostToDevice));
+    std::vector<uint32_t> rec((size_t)n * 8, 0u);
+    std::vector<uint16_t> rest;
+    for (int32_t i = 0; i < n; ++i) {
+        const int32_t v = order[i];
+        std::vector<uint16_t> ids;
+        if (succ_start[v + 1] == succ_start[v]) ids.push_back((uint16_t)(n + 1));
+        for (int32_t e = succ_start[v]; e < succ_start[v + 1]; ++e) ids.push_back((uint16_t)succ[e]);
+        uint32_t* r = &rec[(size_t)i * 8];
+        r[0] = (uint32_t)v | ((uint32_t)ids.size() << 16);
+        r[1] = (uint32_t)rest.size();
+        for (size_t k = 0; k < ids.size(); ++k) {
+            if (k < 8) r[4 + k / 2] |= (uint32_t)ids[k] << (16 * (k & 1));
+            else rest.push_back(ids[k]);
         }
     }
+    MOC_CUDA(cudaMalloc((void**)&g->d_order, rec.size() * 4));
+    MOC_CUDA(cudaMemcpy(g->d_order, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice));
+    MOC_CUDA(cudaMalloc((void**)&g->d_succ16, std::max<size_t>(rest.size() * 2, 16)));
+    if (!rest.empty()) MOC_CUDA(cudaMemcpy(g->d_succ16, rest.data(), rest.size() * 2, cudaMemcpyHostToDevice));
     return MOC_OK;
 }
 
@@ -616,6 +628,11 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         block = 32 * best_w;
         smem = pl.pair_graph_b + (size_t)best_w * pl.pair_warp_b;
     }
+    if (pl.quad) {
+        const int k = quad_shape(pl, g->n, B);
+        block = pl.quad_forced ? pl.quad_forced : 64 << k;
+        grid = (int)std::min<int64_t>((int64_t)pl.sm_count * std::max(1, pl.quad_nb[k]), B);
+    }
     if (offs && fill_offs) {
         moc::offsets_kernel<<<(B + moc::kOffsTile - 1) / moc::kOffsTile, moc::kOffsThreads, 0, st>>>(lens, B, offs);
         ++g_launches;
@@ -633,8 +650,14 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         q.max_T = g->C * g->n;
         q.B = B;
         q.M = M;
-        q.order = pl.wide ? g->d_order64 : g->d_order32;
+        q.n_tiles = g->n_tiles;
+        q.split = g->split;
+        q.rec = pl.wide ? g->d_rec64 : g->d_rec32;
+        q.sell = g->d_sell;
+        q.tile_row = g->d_tile_row;
+        q.order = g->d_order;
         q.succ = g->d_succ16;
+        q.base_dur = g->sum_w;
         q.m = pl.wide ? (const void*)g->d_m64 : (const void*)g->d_m32;
         q.w = g->d_w;
         q.cap = g->d_cap;
@@ -710,7 +733,7 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
 // Each block of the self-addressing kernel re-reads the lengths in front of its range: worth it
 // while that redundant traffic (grid * B/2 * 4 bytes from L2) stays small next to a second launch.
 bool rows_without_scratch(const Plan& pl, int32_t B) {
-    return (pl.pair || pl.lane) && (int64_t)pl.grid * B * 2 <= (int64_t)16 << 20;
+    return (pl.pair || pl.lane || pl.quad) && (int64_t)pl.grid * B * 2 <= (int64_t)16 << 20;
 }
 
 int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
@@ -910,6 +933,13 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
     up((void**)&g->d_w, w, (size_t)n * 8);
     up((void**)&g->d_m64, m, (size_t)n * 8);
     up((void**)&g->d_m32, m32.data(), (size_t)n * 4);
+    {
+        // 64-bit sums: parts of m that 32-bit atomics can add (moc_pair_kernel.cuh), where sum(m) permits
+        int k = 31;
+        while (k > 0 && ((int64_t)1 << (31 - k)) < n) --k;
+        g->split_ok = (sum_m >> k) < ((int64_t)1 << 31);
+        g->split = g->split_ok ? k : 32;
+    }
     if (n <= 16000) {
         // Layout for the warp-per-sequence kernel.  Lane l serves the nodes with id = l (mod 32);
         // each residue class is sorted by out-degree (descending, ties by id); half j holds the
@@ -942,11 +972,6 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
             if (sell_len <= 2 * ne + 4096 && sell_len < (1 << 20) && max_rows < (1 << 12) && 4 * ((int64_t)n + 3) < 65536) {
                 const uint32_t word_b = (uint32_t)align16(4 * ((size_t)n + 2));   // the constant word (1, 1) sits right after the words
                 std::vector<uint32_t> rec32((size_t)n_halves * 32 * 2), rec64((size_t)n_halves * 32 * 4, 0u);
-                // 64-bit sums: parts of m that 32-bit atomics can add (moc_pair_kernel.cuh), where sum(m) permits
-                int k = 31;
-                while (((int64_t)1 << (31 - k)) < n) --k;
-                g->split_ok = (sum_m >> k) < ((int64_t)1 << 31);
-                g->split = g->split_ok ? k : 32;
                 // entry (row k, lane l) of a tile: word of the k-th successor of the node in half 0 | same for half 1 << 16;
                 // a list that is used up continues with the node's own word
                 std::vector<uint32_t> sell((size_t)std::max<int64_t>(sell_len, 1), word_b | (word_b << 16));
@@ -1001,6 +1026,9 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
                     }
                     pos += 32 * (uint32_t)rows[d];
                 }
+                std::vector<int32_t> tile_row((size_t)n_tiles, 0);
+                for (int32_t d = 1; d < n_tiles; ++d) tile_row[d] = tile_row[d - 1] + rows[d - 1];
+                up((void**)&g->d_tile_row, tile_row.data(), tile_row.size() * 4);
                 g->sell_len = (int32_t)sell_len;
                 g->h_slot = slot;
                 g->n_tiles = n_tiles;
@@ -1024,7 +1052,7 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
     try {
         rc = build_lane_layouts(g, succ_start, succ, m, m32);
         if (rc == MOC_OK) rc = upload_wslot(g);
-        if (rc == MOC_OK) rc = build_quad_layout(g, succ_start, succ, m, m32);
+        if (rc == MOC_OK) rc = build_quad_layout(g, succ_start, succ);
     } catch (const std::bad_alloc&) {
         rc = fail(MOC_ERR_NOMEM, "host allocation failed");
     }
@@ -1168,8 +1196,8 @@ void moc_graph_destroy(moc_graph* g) {
     cudaFree(g->d_stage_seqs);
     cudaFree(g->d_stage_u16);
     cudaFree(g->d_stage_io);
-    cudaFree(g->d_order32);
-    cudaFree(g->d_order64);
+    cudaFree(g->d_order);
+    cudaFree(g->d_tile_row);
     cudaFree(g->d_succ16);
     cudaFree(g->d_live32);
     cudaFree(g->d_live64);

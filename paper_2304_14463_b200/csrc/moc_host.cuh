@@ -41,6 +41,8 @@ struct Plan {
     bool quad = false;
     QuadFn quad_fn = nullptr;
     uint32_t quad_word_b = 0, quad_cnt_b = 0;
+    int quad_nb[5] = {0};          // blocks per SM with 64 << k threads
+    int quad_forced = 0;           // threads per sequence the caller asked for
     // small graphs, large batches: a lane per sequence, walked backwards (null: the graph or a forced kind rules it out)
     LiveFn live_fn = nullptr;
     const uint32_t* live_image = nullptr;
@@ -115,8 +117,7 @@ struct moc_graph {
     int32_t want_G = 0, want_gpc = 0;
     int32_t want_kind = 0, want_a = 0, want_b = 0;   // moc_graph_set_kernel
     moc_host::LaneLayout lane[3];         // groups of 32, 16, 8 sequences
-    uint4* d_order32 = nullptr;           // block-per-sequence kernel: 32-byte node records by falling out-degree (32- / 64-bit m)
-    uint4* d_order64 = nullptr;
+    uint4* d_order = nullptr;             // block-per-sequence kernel without tiles: 32-byte node records by falling out-degree
     uint16_t* d_succ16 = nullptr;         // ... and the successors beyond a node's eighth
     uint32_t* d_live32 = nullptr;         // backward walk (n <= 128): its tables for 32-bit and for 64-bit sums
     uint32_t* d_live64 = nullptr;
@@ -135,6 +136,7 @@ struct moc_graph {
     std::vector<int64_t> h_w;             // durations (host copy, to rebuild d_wslot)
     std::vector<int32_t> h_cap;           // per-node caps (empty: uniform)
     uint32_t* d_sell = nullptr;
+    int32_t* d_tile_row = nullptr;        // first row of every successor tile
     // grow-only scratch; mutable because evaluation takes a const handle
     mutable moc_host::Plan plan_eval, plan_profile;
     mutable int64_t* d_offs = nullptr;

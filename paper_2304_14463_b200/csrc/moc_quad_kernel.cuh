@@ -6,17 +6,15 @@
 //
 // Representation.  Positions are 1-based and 16 bits wide (sequences of at most 32766 steps: the packed
 // comparisons tell earlier from later by the sign of a 16-bit difference).  After
-// stage 1b a node's word holds its copies in ascending order; a node with fewer than four copies
-// repeats its last copy in the remaining quarters, so that no quarter is empty.
+// stage 1b a node's word holds its copies in order of arrival, and copies again in the quarters that are
+// left, so that no quarter is empty; only the owner sorts them.
 //
 // Stages for one sequence seq[0..T) (paper: Section 2, Eqs. 1-8):
 //   1a. occurrence words  step t takes the next free quarter of its node's word (a 16-bit counter per
 //                         node, two counters per 32-bit atomic) and stores t + 1 there.
-//   1b. per node          count in [1, min(C, C_v)] (Eq. 7 and the cap), duration += count * w
-//                         (Eq. 1); the quarters are sorted with a five-comparator network on packed
-//                         halves (empty quarters last) and the empty ones filled with the last copy;
-//                         delta[p - 1] = m for every copy p ("+m at the copy's own step" of stage 3:
-//                         a plain store, every step belongs to exactly one copy).
+//   1b. per node          count in [1, min(C, C_v)] (Eq. 7 and the cap), duration of the further copies
+//                         (Eq. 1); empty quarters filled; delta[p - 1] = m for every copy p ("+m at the copy's
+//                         own step" of stage 3: a plain store, every step belongs to exactly one copy).
 //   2.  free steps        one thread per node u with copies a_1 <= ... <= a_4, nodes taken in order of
 //                         falling out-degree so that the lanes of a warp run about the same number of
 //                         rounds; per successor word r (both halves, two packed operations each):
@@ -32,6 +30,12 @@
 //                         A sink's only successor is a made-up word that holds T in every quarter.
 //   3.  memory profile    delta[free + 1] -= m_u per copy, prefix sum over the steps (Eq. 4).
 //   4.  reductions        peak (Section 2), status against the budget.
+//
+// Stage 2 walks the successor tiles of the warp-per-sequence kernel (two node slots per lane, uniform trip counts, packed
+// word offsets; read through L1, a block has no room for a copy) where the graph has them, else a record per node
+// with bounds tests.  Rows are found from the lengths (each block sums those in front of its range), or through `offs`.
+// The kernel is bound by instruction issue and by the barriers between its stages; the threads per sequence
+// follow the batch (plan_quad).  FIGURES
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -46,24 +50,28 @@ struct QuadParams {
     int32_t max_T;             // C * n
     int32_t B;
     int64_t M;
-    const uint4* order;        // n records of 32 bytes in order of falling out-degree (below)
-    const uint16_t* succ;      // the successors beyond the eighth of the nodes that have more
+    int32_t n_tiles, split;    // as in PairParams
+    const void* rec;
+    const uint32_t* sell;
+    const int32_t* tile_row;   // first row of every tile in `sell`
+    const uint4* order;        // without tiles: n records of 32 bytes in order of falling out-degree (below)
+    const uint16_t* succ;      // ... and the successors beyond the eighth of the nodes that have more
     const void* m;             // n output sizes, int32 or int64
     const int64_t* w;          // n durations
+    int64_t base_dur;          // sum of all w
     const int32_t* cap;        // n per-node caps, or nullptr
     const int32_t* seqs;
     const int32_t* lens;
-    const int64_t* offs;       // B + 1 row offsets
+    const int64_t* offs;       // B + 1 row offsets, or nullptr: the kernel finds the packed rows itself
     int64_t* out_peak;
     int64_t* out_dur;
     int32_t* out_status;
-    uint32_t word_bytes;       // 8 (n + 2), rounded to 16
+    uint32_t word_bytes;       // 8 (n + 2) rounded to 32, and 16 for the word of empty node slots
     uint32_t cnt_bytes;        // 2 (n + 2), rounded to 16
 };
 
-// Node record: word 0 = node | out-degree << 16 (a sink: 1, its successor the id n + 1), word 1 = index
-// of its ninth successor in `succ`, words 2-3 = m (int32: word 2), words 4-7 = its first eight successor
-// ids, 16 bits each.
+// Node record of `order`: word 0 = node | out-degree << 16 (a sink: 1, its successor the id n + 1), word 1 = index
+// of its ninth successor in `succ`, words 4-7 = its first eight successor ids, 16 bits each.
 
 __device__ __forceinline__ void sts_u64(uint32_t addr, uint64_t v) {
     asm volatile("st.shared.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
@@ -87,15 +95,69 @@ __device__ __forceinline__ void sort4_u16(uint32_t& lo, uint32_t& hi) {
 }
 __device__ __forceinline__ uint32_t max_halves(uint32_t v) { return max_u16x2(v, swap_halves(v)) & 0xFFFFu; }
 
+__device__ __forceinline__ void quad_store(uint32_t addr, Amount<int32_t> a) { sts_u32(addr, (uint32_t)a.v); }
+__device__ __forceinline__ void quad_store(uint32_t addr, Amount<int64_t> a) {
+    asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(addr), "r"(a.lo), "r"(a.hi) : "memory");
+}
+
+// The copies a_1 <= ... of one node and its running reductions over successor words.
+template <int kAcc>
+struct QuadNode {
+    uint32_t base[kAcc], na[kAcc], G[kAcc];
+    // own word after stage 1b
+    __device__ __forceinline__ void open(uint2 own) {
+        uint32_t last;
+        if constexpr (kAcc == 3) {          // the fourth quarter is a repetition
+            const uint32_t x0 = own.x & 0xFFFFu, x1 = own.x >> 16, x2 = own.y & 0xFFFFu;
+            const uint32_t lo = min(x0, x1), hi = max(x0, x1), mid = min(hi, x2);
+            last = max(hi, x2);
+            base[0] = min(lo, mid);
+            base[1] = max(lo, mid);
+            base[2] = last;
+        } else {
+            sort4_u16(own.x, own.y);
+            base[0] = own.x & 0xFFFFu;
+            base[1] = own.x >> 16;
+            base[2] = own.y & 0xFFFFu;
+            base[3] = last = own.y >> 16;
+        }
+#pragma unroll
+        for (int j = 0; j < kAcc; ++j) na[j] = 0x00010000u - base[j] * 0x10001u;     // (-a, -a) mod 2^16
+        G[0] = (last - base[0]) * 0x10001u;                                          // the last copy ends at itself at least
+#pragma unroll
+        for (int j = 1; j < kAcc; ++j) G[j] = ((base[j - 1] - base[j]) & 0xFFFFu) * 0x10001u;   // copy j ends at itself at least
+    }
+    __device__ __forceinline__ void visit(uint2 r) {
+#pragma unroll
+        for (int j = 0; j < kAcc; ++j) {
+            G[j] = __viaddmax_u16x2(r.x, na[j], G[j]);
+            G[j] = __viaddmax_u16x2(r.y, na[j], G[j]);
+        }
+    }
+    // -m behind the end of every copy; returns a word whose bit 15 tells of a successor copy before a_1
+    template <typename MemT, int kShift>
+    __device__ __forceinline__ uint32_t close(uint32_t da, Amount<MemT> m) {
+        const uint32_t g0 = max_halves(G[0]);
+        red_sub_amount(da + (((base[0] + g0) & 0xFFFFu) << kShift), m);
+#pragma unroll
+        for (int j = 1; j < kAcc; ++j)
+            if (base[j] != base[j - 1]) red_sub_amount(da + (((base[j] + max_halves(G[j])) & 0xFFFFu) << kShift), m);   // copy j exists apart from copy j + 1
+        return g0;
+    }
+};
+
 // kAcc: number of copies the node pass keeps apart (3 or 4).
-template <typename MemT, int kAcc>
+template <typename MemT, int kAcc, bool kTiles>
 __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
     extern __shared__ __align__(16) char smem[];
     __shared__ int64_t s_dur[32];
-    __shared__ MemT s_sum[32], s_top[32];
+    __shared__ uint32_t s_lo[32], s_hi[32];
+    __shared__ int64_t s_top[32];
     __shared__ uint32_t s_flags;
     constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
-    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, n_warps = nthr >> 5;
+    constexpr uint32_t kFull = 0xFFFFFFFFu;
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, n_warps = nthr >> 5;
+    const int warp = __shfl_sync(kFull, tid >> 5, 0);
     int n = p.n;
     MOC_KEEP(n);
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
@@ -103,15 +165,50 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
     MOC_KEEP(wa);
     MOC_KEEP(ca);
     MOC_KEEP(da);
-    const MemT* gm = reinterpret_cast<const MemT*>(p.m);
+    const uint32_t dm1 = da - (uint32_t)sizeof(MemT);
+    auto amount = [&](int v) -> Amount<MemT> {       // m of node v in the form of the deltas
+        Amount<MemT> a;
+        if constexpr (sizeof(MemT) == 4) {
+            a.v = __ldg(reinterpret_cast<const int32_t*>(p.m) + v);
+        } else {
+            const int64_t mv = __ldg(reinterpret_cast<const int64_t*>(p.m) + v);
+            a.lo = (uint32_t)mv;
+            a.hi = (uint32_t)(mv >> p.split);
+        }
+        return a;
+    };
 
-    for (int b = blockIdx.x; b < p.B; b += gridDim.x) {
-        const int64_t off = __ldg(p.offs + b);
+    // ---- rows: block c takes [c * B / grid, (c + 1) * B / grid), or every grid-th one with the offsets given
+    const bool self = p.offs == nullptr;
+    int b = blockIdx.x, b_end = p.B, b_step = gridDim.x;
+    int64_t off = 0;
+    if (self) {
+        b = (int)((int64_t)blockIdx.x * p.B / gridDim.x);
+        b_end = (int)(((int64_t)blockIdx.x + 1) * p.B / gridDim.x);
+        b_step = 1;
+        int64_t sum = 0;
+        int i = tid;
+        if ((reinterpret_cast<uintptr_t>(p.lens) & 15) == 0) {
+            const int4* l4 = reinterpret_cast<const int4*>(p.lens);
+            for (int k = tid; k < b >> 2; k += nthr) {
+                const int4 x = __ldg(l4 + k);
+                sum += (int64_t)max(x.x, 0) + max(x.y, 0) + max(x.z, 0) + max(x.w, 0);
+            }
+            i += b & ~3;
+        }
+        for (; i < b; i += nthr) sum += max(__ldg(p.lens + i), 0);
+        sum = warp_sum64(sum);
+        if (lane == 0) s_dur[warp] = sum;
+        __syncthreads();
+        for (int k = 0; k < n_warps; ++k) off += s_dur[k];
+    }
+    for (; b < b_end; b += b_step) {
         const int32_t T = __ldg(p.lens + b);
+        if (!self) off = __ldg(p.offs + b);
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
         if (T >= n && T <= p.max_T) {      // uniform over the block
-            // ---- clear words and counters (stage 1a writes every delta the prefix sum reads)
+            // ---- clear words and counters (stage 1b writes every delta the prefix sum reads)
             {
                 const int4 z = make_int4(0, 0, 0, 0);
                 int4* s4 = reinterpret_cast<int4*>(smem);
@@ -143,39 +240,34 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                     put(i3, t + 3 * nthr);
                 }
                 for (; t < T; t += nthr) put((uint32_t)__ldg(row + t), t);
-                if (tid == 0) sts_u64(wa + ((uint32_t)(n + 1) << 3), (uint64_t)(uint32_t)T * 0x0001000100010001ull);
+                if (tid == 0) {
+                    sts_u64(wa + ((uint32_t)(n + 1) << 3), (uint64_t)(uint32_t)T * 0x0001000100010001ull);
+                    sts_u64(wa + p.word_bytes - 16u, 0x0001000100010001ull);      // owned by empty node slots
+                }
             }
             __syncthreads();
             // ---- stage 1b
             int64_t dur = 0;
             for (int v = tid; v < n; v += nthr) {
-                const uint32_t c = (lds_u32(ca + ((uint32_t)(v >> 1) << 2)) >> ((v & 1) << 4)) & 0xFFFFu;
-                uint32_t limit = (uint32_t)p.C;
+                uint32_t c, limit = (uint32_t)p.C;
+                asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(c) : "r"(ca + 2u * (uint32_t)v) : "memory");
                 if (p.cap != nullptr) limit = min(limit, (uint32_t)__ldg(p.cap + v));
-                if (c < 1 || c > limit) flags |= 1;
-                dur += (int64_t)c * __ldg(p.w + v);
                 const uint2 q = lds_v2(wa + ((uint32_t)v << 3));
-                // keys x - 1: an empty quarter becomes the largest key and sorts last
-                uint32_t lo = __viaddmin_u16x2(q.x, 0xFFFFFFFFu, 0xFFFFFFFFu), hi = __viaddmin_u16x2(q.y, 0xFFFFFFFFu, 0xFFFFFFFFu);
-                const uint32_t top = max_halves(max_u16x2(q.x, q.y));                  // the last copy
-                const uint32_t cap_key = (top - 1u) * 0x10001u;
-                sort4_u16(lo, hi);
-                lo = __viaddmax_u16x2(min_u16x2(lo, cap_key), 0x00010001u, 0u);        // back to positions, empties = last copy
-                hi = __viaddmax_u16x2(min_u16x2(hi, cap_key), 0x00010001u, 0u);
-                sts_u64(wa + ((uint32_t)v << 3), (uint64_t)lo | ((uint64_t)hi << 32));
-                // +m at every copy's own step; repeated quarters write the same value to the same place.  Only
-                // for a node with a valid count: then every quarter is a step of the row (1..T); the word of an
-                // absent or overfull node holds no usable positions and the sequence is malformed anyway.
-                if (c >= 1 && c <= limit) {
-                    const MemT mv = __ldg(gm + v);
-                    const uint32_t dm1 = da - (uint32_t)sizeof(MemT);
-                    sts_mem(dm1 + ((lo & 0xFFFFu) << kShift), mv);
-                    sts_mem(dm1 + ((lo >> 16) << kShift), mv);
-                    sts_mem(dm1 + ((hi & 0xFFFFu) << kShift), mv);
-                    sts_mem(dm1 + ((hi >> 16) << kShift), mv);
+                const Amount<MemT> mv = amount(v);
+                if (c - 1u >= limit) {       // absent or overfull: its word holds no usable positions
+                    flags |= 1;
+                    continue;
                 }
+                if (c > 1) dur += (int64_t)(c - 1) * __ldg(p.w + v);
+                const uint32_t lo = c == 1 ? q.x * 0x10001u : q.x;
+                const uint32_t hi = c < 3 ? lo : (c == 3 ? __byte_perm(q.y, q.x, 0x5410) : q.y);
+                if (c < 4) sts_u64(wa + ((uint32_t)v << 3), (uint64_t)lo | ((uint64_t)hi << 32));
+                quad_store(dm1 + ((lo & 0xFFFFu) << kShift), mv);
+                if (c > 1) quad_store(dm1 + ((lo >> 16) << kShift), mv);
+                if (c > 2) quad_store(dm1 + ((hi & 0xFFFFu) << kShift), mv);
+                if (kAcc > 3 && c > 3) quad_store(dm1 + ((hi >> 16) << kShift), mv);
             }
-            flags = __reduce_or_sync(0xFFFFFFFFu, flags);
+            flags = __reduce_or_sync(kFull, flags);
             dur = warp_sum64(dur);
             if (lane == 0) {
                 if (flags) atomicOr(&s_flags, flags);
@@ -186,70 +278,74 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
             if (!malformed) {
                 // ---- stage 2 and the scatter of stage 3
                 uint32_t depw = 0;
-                const int n_round = (n + 31) & ~31;
-                for (int i = tid; i < n_round; i += nthr) {
-                    uint32_t node = 0, deg = 0, e8 = 0;
-                    uint4 inl = make_uint4(0, 0, 0, 0);
-                    MemT neg_m = 0;
-                    if (i < n) {
-                        const uint4 r = __ldg(p.order + 2 * i);
-                        inl = __ldg(p.order + 2 * i + 1);
-                        node = r.x & 0xFFFFu;
-                        deg = r.x >> 16;
-                        e8 = r.y;
-                        if constexpr (sizeof(MemT) == 4) neg_m = -(MemT)r.z;
-                        else neg_m = -(MemT)((uint64_t)r.z | ((uint64_t)r.w << 32));
-                    }
-                    const int rounds = __reduce_max_sync(0xFFFFFFFFu, (int)deg);
-                    const uint2 own = lds_v2(wa + (node << 3));
-                    // copies a_1..a_4 ascending: own.x = (a_1, a_2), own.y = (a_3, a_4)
-                    uint32_t base[kAcc], na[kAcc], G[kAcc];
-                    base[0] = own.x & 0xFFFFu;
-                    base[1] = own.x >> 16;
-                    base[2] = own.y & 0xFFFFu;
-                    if constexpr (kAcc == 4) base[3] = own.y >> 16;
-                    const uint32_t last = own.y >> 16;
+                if constexpr (kTiles) {
+                    for (int d = warp; d < p.n_tiles; d += n_warps) {
+                        QuadNode<kAcc> u[2];
+                        Amount<MemT> m[2];
+                        uint32_t x0 = 0;
 #pragma unroll
-                    for (int j = 0; j < kAcc; ++j) na[j] = 0x00010000u - base[j] * 0x10001u;     // (-a, -a) mod 2^16
-                    G[0] = (last - base[0]) * 0x10001u;                                          // the last copy ends at itself at least
-#pragma unroll
-                    for (int j = 1; j < kAcc; ++j) G[j] = ((base[j - 1] - base[j]) & 0xFFFFu) * 0x10001u;   // copy j ends at itself at least
-                    auto visit = [&](uint32_t sid) {
-                        const uint2 r = lds_v2(wa + (sid << 3));
-#pragma unroll
-                        for (int j = 0; j < kAcc; ++j) {
-                            G[j] = __viaddmax_u16x2(r.x, na[j], G[j]);
-                            G[j] = __viaddmax_u16x2(r.y, na[j], G[j]);
+                        for (int h = 0; h < 2; ++h) {
+                            uint32_t x;
+                            if constexpr (sizeof(MemT) == 4) {
+                                const uint2 r = __ldg(reinterpret_cast<const uint2*>(p.rec) + (2 * d + h) * 32 + lane);
+                                x = r.x;
+                                m[h].v = (MemT)r.y;
+                            } else {
+                                const uint4 r = __ldg(reinterpret_cast<const uint4*>(p.rec) + (2 * d + h) * 32 + lane);
+                                x = r.x;
+                                m[h].lo = r.z;
+                                m[h].hi = r.w;
+                            }
+                            if (h == 0) x0 = x;
+                            u[h].open(lds_v2(wa + ((x & 0xFFFFu) << 1)));
                         }
-                    };
-                    const uint32_t in8[4] = {inl.x, inl.y, inl.z, inl.w};
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        if (k < rounds) {
-                            if ((uint32_t)k < deg) visit((k & 1) ? in8[k >> 1] >> 16 : in8[k >> 1] & 0xFFFFu);
+                        const int rows = __shfl_sync(kFull, (int)(x0 >> 16), 0);
+                        const uint32_t* ps = p.sell + 32 * __ldg(p.tile_row + d) + lane;
+                        uint32_t e_next = __ldg(ps);
+                        for (int k = 0; k < rows; ++k) {
+                            const uint32_t e = e_next;
+                            ps += 32;
+                            if (k + 1 < rows) e_next = __ldg(ps);
+                            const uint2 r0 = lds_v2(wa + ((e & 0xFFFFu) << 1)), r1 = lds_v2(wa + ((e >> 16) << 1));
+                            u[0].visit(r0);
+                            u[1].visit(r1);
                         }
+                        depw |= u[0].template close<MemT, kShift>(da, m[0]);
+                        depw |= u[1].template close<MemT, kShift>(da, m[1]);
                     }
-                    for (int k = 8; k < rounds; ++k)
-                        if ((uint32_t)k < deg) visit((uint32_t)__ldg(p.succ + e8 + (k - 8)));
-                    if (i < n) {
-                        const uint32_t g0 = max_halves(G[0]);
-                        depw |= g0;                                           // bit 15: a successor copy before a_1
-                        red_add_shared(da + (((base[0] + g0) & 0xFFFFu) << kShift), neg_m);
+                } else {
+                    const int n_round = (n + 31) & ~31;
+                    for (int i = tid; i < n_round; i += nthr) {
+                        uint32_t node = 0, deg = 0, e8 = 0;
+                        uint4 inl = make_uint4(0, 0, 0, 0);
+                        if (i < n) {
+                            const uint4 r = __ldg(p.order + 2 * i);
+                            inl = __ldg(p.order + 2 * i + 1);
+                            node = r.x & 0xFFFFu;
+                            deg = r.x >> 16;
+                            e8 = r.y;
+                        }
+                        const int rounds = __reduce_max_sync(kFull, (int)deg);
+                        QuadNode<kAcc> u;
+                        u.open(lds_v2(wa + (node << 3)));
+                        const uint32_t in8[4] = {inl.x, inl.y, inl.z, inl.w};
 #pragma unroll
-                        for (int j = 1; j < kAcc; ++j) {
-                            if (base[j] != base[j - 1]) {                    // copy j exists apart from copy j + 1
-                                const uint32_t x = (base[j] + max_halves(G[j])) & 0xFFFFu;
-                                red_add_shared(da + (x << kShift), neg_m);
+                        for (int k = 0; k < 8; ++k) {
+                            if (k < rounds) {
+                                if ((uint32_t)k < deg) u.visit(lds_v2(wa + (((k & 1) ? in8[k >> 1] >> 16 : in8[k >> 1] & 0xFFFFu) << 3)));
                             }
                         }
+                        for (int k = 8; k < rounds; ++k)
+                            if ((uint32_t)k < deg) u.visit(lds_v2(wa + ((uint32_t)__ldg(p.succ + e8 + (k - 8)) << 3)));
+                        if (i < n) depw |= u.template close<MemT, kShift>(da, amount((int)node));
                     }
                 }
-                if (__any_sync(0xFFFFFFFFu, (depw & 0x8000u) != 0) && lane == 0) atomicOr(&s_flags, 2u);
+                if (__any_sync(kFull, (depw & 0x8000u) != 0) && lane == 0) atomicOr(&s_flags, 2u);
             }
             __syncthreads();
             const uint32_t fl = s_flags;
             if (!(fl & 1u)) {
-                out_du = 0;
+                out_du = p.base_dur;
                 for (int k = 0; k < n_warps; ++k) out_du += s_dur[k];
                 out_st = -1;
             }
@@ -257,25 +353,45 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 // ---- stages 3 and 4: prefix sum, each thread a chunk of consecutive steps (odd length: no bank conflicts)
                 const int chunk = ((T + nthr - 1) / nthr) | 1;
                 const int tb = min(tid * chunk, T), te = min(tb + chunk, T);
-                MemT run = 0, top = 0;
-                uint32_t ad = da + ((uint32_t)tb << kShift);
+                uint32_t ad = da + ((uint32_t)tb << kShift), lo = 0, hi = 0;
+                MemT top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
                 for (int t = tb; t < te; ++t, ad += (uint32_t)sizeof(MemT)) {
-                    run += lds_mem(ad, MemT());
-                    top = (t == tb || run > top) ? run : top;
+                    MemT at;
+                    if constexpr (sizeof(MemT) == 4) {
+                        lo += lds_u32(ad);
+                        at = (MemT)lo;
+                    } else {
+                        const uint2 q = lds_v2(ad);
+                        lo += q.x;
+                        hi += q.y;
+                        at = split_value(lo, hi, p.split);
+                    }
+                    top = at > top ? at : top;
                 }
                 // chunk sums -> usage in front of every chunk; a thread without steps passes its prefix on
-                MemT incl = warp_inclusive_sum(run, lane);
-                if (lane == 31) s_sum[warp] = incl;
+                uint32_t lo_in = warp_inclusive_sum(lo, lane), hi_in = 0;
+                if constexpr (sizeof(MemT) == 8) hi_in = warp_inclusive_sum(hi, lane);
+                if (lane == 31) {
+                    s_lo[warp] = lo_in;
+                    s_hi[warp] = hi_in;
+                }
                 __syncthreads();
-                MemT before = incl - run;
-                for (int k = 0; k < warp; ++k) before += s_sum[k];
+                lo_in -= lo;
+                hi_in -= hi;
+                for (int k = 0; k < warp; ++k) {
+                    lo_in += s_lo[k];
+                    if constexpr (sizeof(MemT) == 8) hi_in += s_hi[k];
+                }
+                MemT before;
+                if constexpr (sizeof(MemT) == 4) before = (MemT)lo_in;
+                else before = split_value(lo_in, hi_in, p.split);
                 MemT peak = tb < te ? before + top : MemT(0);
                 peak = warp_max_t(peak);
-                if (lane == 0) s_top[warp] = peak;
+                if (lane == 0) s_top[warp] = (int64_t)peak;
                 __syncthreads();
                 if (tid == 0) {
-                    for (int k = 1; k < n_warps; ++k) peak = s_top[k] > peak ? s_top[k] : peak;
-                    out_pk = (int64_t)peak;
+                    out_pk = s_top[0];
+                    for (int k = 1; k < n_warps; ++k) out_pk = s_top[k] > out_pk ? s_top[k] : out_pk;
                     out_st = out_pk <= p.M ? 1 : 0;
                 }
             }
@@ -285,6 +401,7 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
             p.out_dur[b] = out_du;
             p.out_status[b] = out_st;
         }
+        off += max(T, 0);
         __syncthreads();    // the state is reused by the next sequence
     }
 }
