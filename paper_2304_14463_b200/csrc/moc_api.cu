@@ -631,7 +631,14 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
     if (pl.quad) {
         const int k = quad_shape(pl, g->n, B);
         block = pl.quad_forced ? pl.quad_forced : 64 << k;
-        grid = (int)std::min<int64_t>((int64_t)pl.sm_count * std::max(1, pl.quad_nb[k]), B);
+        // blocks per SM: the least rounds * warps (a last round of few blocks costs a sequence's whole latency)
+        int nb = 1;
+        int64_t best = INT64_MAX;
+        for (int c = 1; c <= std::max(1, pl.quad_nb[k]); ++c) {
+            const int64_t rounds = (B + (int64_t)pl.sm_count * c - 1) / ((int64_t)pl.sm_count * c), cost = rounds * std::max(c * block / 32, 24);
+            if (cost <= best) { best = cost; nb = c; }
+        }
+        grid = (int)std::min<int64_t>((int64_t)pl.sm_count * nb, B);
     }
     if (offs && fill_offs) {
         moc::offsets_kernel<<<(B + moc::kOffsTile - 1) / moc::kOffsTile, moc::kOffsThreads, 0, st>>>(lens, B, offs);

@@ -248,12 +248,14 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
             __syncthreads();
             // ---- stage 1b
             int64_t dur = 0;
+            Amount<MemT> m_next = amount(min(tid, n - 1));          // one round ahead
             for (int v = tid; v < n; v += nthr) {
                 uint32_t c, limit = (uint32_t)p.C;
                 asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(c) : "r"(ca + 2u * (uint32_t)v) : "memory");
                 if (p.cap != nullptr) limit = min(limit, (uint32_t)__ldg(p.cap + v));
                 const uint2 q = lds_v2(wa + ((uint32_t)v << 3));
-                const Amount<MemT> mv = amount(v);
+                const Amount<MemT> mv = m_next;
+                m_next = amount(min(v + nthr, n - 1));
                 if (c - 1u >= limit) {       // absent or overfull: its word holds no usable positions
                     flags |= 1;
                     continue;
@@ -279,29 +281,43 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 // ---- stage 2 and the scatter of stage 3
                 uint32_t depw = 0;
                 if constexpr (kTiles) {
+                    // records and first successor row of a tile are requested while the tile before it is worked on
+                    uint4 r_next[2];
+                    const uint32_t* ps_next = nullptr;
+                    uint32_t e_first = 0;
+                    auto request = [&](int d) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if constexpr (sizeof(MemT) == 4) {
+                                const uint2 r = __ldg(reinterpret_cast<const uint2*>(p.rec) + (2 * d + h) * 32 + lane);
+                                r_next[h].x = r.x;
+                                r_next[h].z = r.y;
+                            } else {
+                                r_next[h] = __ldg(reinterpret_cast<const uint4*>(p.rec) + (2 * d + h) * 32 + lane);
+                            }
+                        }
+                        ps_next = p.sell + 32 * __ldg(p.tile_row + d) + lane;
+                        e_first = __ldg(ps_next);
+                    };
+                    if (warp < p.n_tiles) request(warp);
                     for (int d = warp; d < p.n_tiles; d += n_warps) {
                         QuadNode<kAcc> u[2];
                         Amount<MemT> m[2];
-                        uint32_t x0 = 0;
+                        const uint32_t x0 = r_next[0].x;
+                        const uint32_t* ps = ps_next;
+                        uint32_t e_next = e_first;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            uint32_t x;
                             if constexpr (sizeof(MemT) == 4) {
-                                const uint2 r = __ldg(reinterpret_cast<const uint2*>(p.rec) + (2 * d + h) * 32 + lane);
-                                x = r.x;
-                                m[h].v = (MemT)r.y;
+                                m[h].v = (MemT)r_next[h].z;
                             } else {
-                                const uint4 r = __ldg(reinterpret_cast<const uint4*>(p.rec) + (2 * d + h) * 32 + lane);
-                                x = r.x;
-                                m[h].lo = r.z;
-                                m[h].hi = r.w;
+                                m[h].lo = r_next[h].z;
+                                m[h].hi = r_next[h].w;
                             }
-                            if (h == 0) x0 = x;
-                            u[h].open(lds_v2(wa + ((x & 0xFFFFu) << 1)));
+                            u[h].open(lds_v2(wa + ((r_next[h].x & 0xFFFFu) << 1)));
                         }
+                        if (d + n_warps < p.n_tiles) request(d + n_warps);
                         const int rows = __shfl_sync(kFull, (int)(x0 >> 16), 0);
-                        const uint32_t* ps = p.sell + 32 * __ldg(p.tile_row + d) + lane;
-                        uint32_t e_next = __ldg(ps);
                         for (int k = 0; k < rows; ++k) {
                             const uint32_t e = e_next;
                             ps += 32;
