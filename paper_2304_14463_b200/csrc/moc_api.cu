@@ -233,7 +233,7 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, Plan* out) {
 // per-thread loops.  With few, enough to give every SM about 16 warps.
 int quad_shape(const Plan& pl, int64_t n, int32_t B) {
     if (pl.quad_forced) return 0;
-    int k = n < 200 ? 0 : (n < 1600 ? 1 : (n < 4000 ? 2 : 3));
+    int k = n < 700 ? 0 : (n < 1600 ? 1 : (n < 4000 ? 2 : 3));
     const int64_t per_sm = ((int64_t)B + pl.sm_count - 1) / pl.sm_count;
     while (k < 3 && per_sm * (2 << (k + 1)) <= 16) ++k;
     if (n >= 3000 && per_sm == 1) k = 4;
@@ -333,6 +333,12 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
             *out = pl;
             return MOC_OK;
         }
+    }
+    // sequences too long for eight warps of the warp-per-sequence kernel on an SM (n = 2000, B = 2000: 69.6 us with a
+    // thread group per sequence, 53.5 with the block-per-sequence kernel)
+    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, &pl)) {
+        *out = pl;
+        return MOC_OK;
     }
     if (t_max <= 65534 && sh_group <= smem_cap) {
         pl.global_state = false;
@@ -743,14 +749,38 @@ bool rows_without_scratch(const Plan& pl, int32_t B) {
     return (pl.pair || pl.lane || pl.quad) && (int64_t)pl.grid * B * 2 <= (int64_t)16 << 20;
 }
 
+// The plan for a batch of B: where the warp-per-sequence kernel serves the graph, the block-per-sequence kernel still
+// takes the batches in which a warp's latency decides (a sequence has several warps there) and the long sequences,
+// whose state leaves too few warps on an SM (make_plan).  Measured at C = 2, warp / block: n = 442 10.4 / 8.8 us at B = 148,
+// 10.3 / 10.3 at 296, 10.4 / 12.4 at 600; n = 1000 16.5 / 10.3 at 296, 16.5 / 14.5 at 600, 16.5 / 16.5 at 1000, 18.6 / 26.8
+// at 2000; n = 1500 36 / 37 at 2000.
+const Plan& plan_for(const moc_graph* g, int32_t B) {
+    const Plan& pl = g->plan_eval;
+    if (!pl.pair || !g->plan_block.valid) return pl;
+    const int64_t n = g->n, sm = pl.sm_count;
+    const bool block = (n >= 700 && B <= 6 * sm) || (n >= 400 && B <= 2 * sm);
+    return block ? g->plan_block : pl;
+}
+
+// Makes the plans of the handle on first use.
+int ensure_plans(const moc_graph* g) {
+    if (g->plan_eval.valid) return MOC_OK;
+    g->plan_block = Plan();
+    int rc = make_plan(g, false, &g->plan_eval);
+    if (rc == MOC_OK && g->plan_eval.pair && g->want_kind == MOC_KERNEL_AUTO) {
+        Plan pl;
+        pl.wide = g->plan_eval.wide;
+        if (!plan_quad(g, g->smem_optin > 1024 ? g->smem_optin - 1024 : 0, &pl)) g->plan_block = pl;
+    }
+    return rc;
+}
+
 int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
                 int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {
-    if (!g->plan_eval.valid) {
-        int rc = make_plan(g, false, &g->plan_eval);
-        if (rc != MOC_OK) return rc;
-    }
-    const Plan& pl = g->plan_eval;
-    if (live_serves(g, pl, B)) return enqueue_live(g, pl, nullptr, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
+    int rc0 = ensure_plans(g);
+    if (rc0 != MOC_OK) return rc0;
+    const Plan& pl = plan_for(g, B);
+    if (live_serves(g, g->plan_eval, B)) return enqueue_live(g, g->plan_eval, nullptr, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     if (rows_without_scratch(pl, B))
         return enqueue_eval(g, pl, nullptr, false, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     int rc = ensure((void**)&g->d_offs, &g->offs_cap, ((size_t)B + 1) * sizeof(int64_t));
@@ -767,12 +797,10 @@ int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, in
 namespace moc_host {
 int eval_rows(const moc_graph* g, const int64_t* offs, const int32_t* seqs, const int32_t* lens, int32_t B,
               int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {
-    if (!g->plan_eval.valid) {
-        int rc = make_plan(g, false, &g->plan_eval);
-        if (rc != MOC_OK) return rc;
-    }
-    const Plan& pl = g->plan_eval;
-    if (live_serves(g, pl, B)) return enqueue_live(g, pl, offs, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
+    int rc0 = ensure_plans(g);
+    if (rc0 != MOC_OK) return rc0;
+    const Plan& pl = plan_for(g, B);
+    if (live_serves(g, g->plan_eval, B)) return enqueue_live(g, g->plan_eval, offs, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     if (pl.global_state) {
         int rc = ensure((void**)&g->d_state, &g->state_cap, (size_t)pl.grid * pl.group_bytes);
         if (rc != MOC_OK) return rc;
@@ -1420,11 +1448,9 @@ int moc_eval_batch_noalloc(const moc_graph* g, const int32_t* seqs, const int32_
     int64_t* offs = nullptr;
     int rc = noalloc_offsets(g->device, &offs);
     if (rc != MOC_OK) return rc;
-    if (!g->plan_eval.valid) {
-        rc = make_plan(g, false, &g->plan_eval);  // attribute and occupancy queries only
-        if (rc != MOC_OK) return rc;
-    }
-    const Plan& pl = g->plan_eval;
+    rc = ensure_plans(g);  // attribute and occupancy queries only
+    if (rc != MOC_OK) return rc;
+    const Plan& pl = plan_for(g, B);
     if (pl.global_state)
         return fail(MOC_ERR_ARG, "moc_eval_batch_noalloc: this graph needs a global workspace "
                     "(per-sequence state exceeds shared memory); use moc_eval_batch");

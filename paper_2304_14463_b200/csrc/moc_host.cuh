@@ -139,6 +139,7 @@ struct moc_graph {
     int32_t* d_tile_row = nullptr;        // first row of every successor tile
     // grow-only scratch; mutable because evaluation takes a const handle
     mutable moc_host::Plan plan_eval, plan_profile;
+    mutable moc_host::Plan plan_block;    // block-per-sequence kernel beside the warp-per-sequence one in plan_eval
     mutable int64_t* d_offs = nullptr;
     mutable size_t offs_cap = 0;
     mutable char* d_state = nullptr;

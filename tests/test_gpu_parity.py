@@ -88,6 +88,23 @@ def test_backward_walk_edges(B, n, C, scale, nB):
         assert (a.cpu().numpy() == b).all()
 
 
+@pytest.mark.parametrize("n,C,bits,nB", [(399, 2, 0, 5), (400, 2, 0, 296), (400, 2, 0, 297), (442, 2, 39, 297), (442, 2, 44, 37), (442, 3, 39, 300),
+                                         (442, 3, 44, 37), (442, 4, 38, 60), (700, 2, 0, 888), (1999, 2, 20, 150), (2300, 2, 0, 20), (3001, 3, 0, 149)])
+def test_small_batches_and_two_part_sums(B, n, C, bits, nB):
+    """Batches around the line between a warp and a block per sequence, sequences too long for the warp kernel, and
+    64-bit sums up to and beyond what the two-part additions cover (bits: m is shifted left by that many)."""
+    edges = W.layered_dag(n, 3 * n, 20, n)
+    w, m = W.weights_uniform(n, 0, 30, n, 1), np.minimum(W.weights_lognormal(n, 3.0, 1.0, n, 2), 255) << bits
+    seqs, lens = W.schedules(n, edges, C, 0.3, nB, n)
+    seqs, lens = W.mutate(seqs, lens, n, C, seed=5, frac=1 / 8)
+    O, G = OracleGraph(n, edges, w, m, C), B.Graph(n, edges, w, m, C)
+    M = O.eval(np.arange(n), 1 << 62)["peak"] * 90 // 100
+    assert_batch_equal(G, O, seqs, lens, M, f"n {n}")
+    if C > 2 or n >= 700:
+        G.set_kernel(B.MOC_KERNEL_GROUP)
+        assert_batch_equal(G, O, seqs, lens, M, f"n {n}, thread groups")
+
+
 # ------------------------------------------------------------------ the five configurations
 SMALL_B = [1024, 4096, 2048, 512, 64]
 
