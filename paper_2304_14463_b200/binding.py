@@ -96,7 +96,7 @@ lib.moc_last_launch_count.argtypes = []
 lib.moc_last_error.restype = ctypes.c_char_p
 lib.moc_last_error.argtypes = []
 # the native side of the binding calls the library through the same addresses
-_fast.bind({name: ctypes.cast(getattr(lib, name), _P).value for name in EXPORTS + ["moc_search_state_filled"]})
+_fast.bind({name: ctypes.cast(getattr(lib, name), _P).value for name in EXPORTS + ["moc_search_state_filled", "moc_check_intervals_filled"]})
 
 
 class MocError(RuntimeError):

@@ -969,10 +969,11 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
     up((void**)&g->d_m64, m, (size_t)n * 8);
     up((void**)&g->d_m32, m32.data(), (size_t)n * 4);
     {
-        // 64-bit sums: parts of m that 32-bit atomics can add (moc_pair_kernel.cuh), where sum(m) permits
-        int k = 31;
-        while (k > 0 && ((int64_t)1 << (31 - k)) < n) --k;
-        g->split_ok = (sum_m >> k) < ((int64_t)1 << 31);
+        // 64-bit sums: parts of m that 32-bit atomics can add (moc_pair_kernel.cuh), where sum(m) permits; with room for
+        // two amounts per node at a time (the interval checker adds up intervals that may overlap)
+        int k = 30;
+        while (k > 0 && ((int64_t)1 << (30 - k)) < n) --k;
+        g->split_ok = (sum_m >> k) < ((int64_t)1 << 30);
         g->split = g->split_ok ? k : 32;
     }
     if (n <= 16000) {
@@ -1064,6 +1065,19 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
                 std::vector<int32_t> tile_row((size_t)n_tiles, 0);
                 for (int32_t d = 1; d < n_tiles; ++d) tile_row[d] = tile_row[d - 1] + rows[d - 1];
                 up((void**)&g->d_tile_row, tile_row.data(), tile_row.size() * 4);
+                // the same tiles for the interval checker: its padding repeats a successor, a sink reads its own word
+                std::vector<uint32_t> sell_iv(sell);
+                for (size_t r = 0; r < slot.size(); ++r) {
+                    const int32_t v = slot[r];
+                    const uint32_t own = own_word(v), pad = v >= 0 && deg(v) > 0 ? 4u * (uint32_t)succ[succ_start[v]] : own;
+                    const int sh = (r & 32) ? 16 : 0;
+                    for (int32_t k = 0; k < rows[r / 64]; ++k) {
+                        uint32_t& e = sell_iv[32 * (size_t)(tile_row[r / 64] + k) + (r & 31)];
+                        const uint32_t off = e >> sh & 0xFFFFu;
+                        if (off == own || off == 4u * ((uint32_t)n + 1)) e = (e & ~(0xFFFFu << sh)) | pad << sh;
+                    }
+                }
+                up((void**)&g->d_sell_iv, sell_iv.data(), sell_iv.size() * 4);
                 g->sell_len = (int32_t)sell_len;
                 g->h_slot = slot;
                 g->n_tiles = n_tiles;
@@ -1226,6 +1240,7 @@ void moc_graph_destroy(moc_graph* g) {
     cudaFree(g->d_wslot);
     cudaFree(g->d_cap);
     cudaFree(g->d_sell);
+    cudaFree(g->d_sell_iv);
     cudaFree(g->d_offs);
     cudaFree(g->d_state);
     cudaFree(g->d_stage_seqs);

@@ -136,6 +136,7 @@ struct moc_graph {
     std::vector<int64_t> h_w;             // durations (host copy, to rebuild d_wslot)
     std::vector<int32_t> h_cap;           // per-node caps (empty: uniform)
     uint32_t* d_sell = nullptr;
+    uint32_t* d_sell_iv = nullptr;        // the same for the interval checker: other padding
     int32_t* d_tile_row = nullptr;        // first row of every successor tile
     // grow-only scratch; mutable because evaluation takes a const handle
     mutable moc_host::Plan plan_eval, plan_profile;

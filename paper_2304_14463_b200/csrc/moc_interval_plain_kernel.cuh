@@ -1,0 +1,275 @@
+// Interval-form checker for the plain event domain with two slots per node (C = 2, D <= 32766: the setting of
+// Section 4.3 with D = C n of Section 2).  Same quantities as check_intervals_kernel (moc_interval_kernels.cuh),
+// which serves every other case; a warp per solution, the graph staged once per block.
+//
+// What differs.  The domain is about as large as the number of slots, so nothing is compressed to ranks: the usage
+// of Eq. 4 is a difference array over the events themselves, and the execution sequence is read off an array
+// that holds, per event, the node whose active interval starts there (plain 16-bit stores), 32 events at a time
+// with ballots, so that the row is written in order with full sectors (scattered 4-byte stores before) and
+// the entries behind it in the same pass.  Eq. 5 walks the successor tiles of the evaluation kernel (two nodes per lane,
+// uniform trip counts) with both starts of a successor tested at once: with lo = s + 1 and len = e - lo per slot,
+//     max(t - lo, len) = len  iff  t in (s, e]            (one packed 16-bit operation per slot, modulo 2^16)
+// and a start is served iff one of the two differences vanishes.
+//
+// An inactive slot's start is replaced by that of the other slot (it then asks for nothing new); a solution in which
+// some node has no active slot at all takes a plain loop over the edges instead.
+//
+// Bound: MEASURED
+#pragma once
+#include "moc_interval_kernels.cuh"
+#include "moc_pair_kernel.cuh"
+
+namespace moc {
+
+constexpr int kIvPlainThreads = 896;
+
+struct IntervalPlainParams {
+    IntervalParams q;
+    int32_t n_tiles, split;      // as in PairParams
+    const void* rec;             // node records of the warp-per-sequence layout
+    const uint32_t* sell;        // its successor tiles; a used-up list repeats a successor, a sink reads its own word
+    uint32_t rec_bytes, sell_bytes;     // graph, once per block
+    uint32_t word_bytes;         // start words (4 (n + 2), rounded to 16) without the word of empty slots behind them
+    uint32_t event_bytes;        // marks, later the difference array
+    bool fill;                   // write -1 behind the sequences (and to the rows without one)
+};
+
+// Bytes of the event area of one warp: marks (2 + 1 bytes per event), or deltas in a whole odd number of 16-byte
+// vectors per lane.
+__host__ __device__ inline size_t interval_plain_event_bytes(int32_t D, size_t mem_sz) {
+    const size_t vec = ((size_t)D + 2 + 16 / mem_sz - 1) / (16 / mem_sz), marks = (3 * ((size_t)D + 64) + 15) / 16;
+    return 32 * 16 * ((((vec > marks ? vec : marks) + 31) / 32) | 1);
+}
+
+template <typename MemT>
+__global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const IntervalPlainParams pp) {
+    extern __shared__ __align__(16) char smem[];
+    const IntervalParams& p = pp.q;
+    constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
+    constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    {
+        int4* s4 = reinterpret_cast<int4*>(smem);
+        const uint32_t n_rec = pp.rec_bytes >> 4, n_all = (pp.rec_bytes + pp.sell_bytes) >> 4;
+        for (uint32_t i = threadIdx.x; i < n_all; i += blockDim.x)
+            s4[i] = i < n_rec ? __ldg(reinterpret_cast<const int4*>(pp.rec) + i) : __ldg(reinterpret_cast<const int4*>(pp.sell) + (i - n_rec));
+    }
+    const int32_t n = p.n, K = 2 * n, D = p.D;
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
+    const uint32_t word_set = pp.word_bytes + kPairWordTail;
+    const uint32_t sa = sbase + pp.rec_bytes + pp.sell_bytes + (uint32_t)warp * (2u * word_set + pp.event_bytes);   // start words
+    const uint32_t ea = sa + word_set;                               // end words: e | active << 15 per slot
+    const uint32_t da = ea + word_set;                               // events
+    const uint32_t all = da + 2u * (uint32_t)((D + 64) & ~31);       // byte marks of all starts, behind the owners (16 bits)
+    const uint32_t rec0 = sbase + kRecB * (uint32_t)lane, sell0 = sbase + pp.rec_bytes + 4u * (uint32_t)lane;
+    if (lane == 0) {
+        sts_u32(sa + pp.word_bytes, 0u);          // empty node slots: inactive
+        sts_u32(ea + pp.word_bytes, 0u);
+    }
+    __syncthreads();
+    auto clear_events = [&]() {
+        for (uint32_t o = 16u * (uint32_t)lane; o < pp.event_bytes; o += 512u)
+            asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(da + o), "r"(0) : "memory");
+        __syncwarp();
+    };
+
+    const int32_t step = gridDim.x * wpb;
+    for (int32_t b = blockIdx.x * wpb + warp; b < p.B; b += step) {
+        const int2* gs = reinterpret_cast<const int2*>(p.s + (int64_t)b * K);
+        const int2* ge = reinterpret_cast<const int2*>(p.e + (int64_t)b * K);
+        const int2* ga = reinterpret_cast<const int2*>(p.a + (int64_t)b * K);
+        if (b + step < p.B) {                     // the next solution comes into L2 meanwhile
+            const int64_t ahead = (int64_t)step * K * 4;
+            for (int32_t o = 128 * lane; o < 4 * K; o += 4096) {
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(gs) + ahead + o));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(ge) + ahead + o));
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(ga) + ahead + o));
+            }
+        }
+        clear_events();
+        // ---- pass 1, per node: Eqs. 1, 2, 3, 7, 8; marks of the starts; the solution on chip
+        int32_t mask = 0, n_act = 0, n_distinct = 0;
+        int64_t dur = 0;
+        bool idle = false;                        // some node has no active slot
+        auto node = [&](int32_t v, const int2 s2, const int2 e2, const int2 a2, const int64_t wv) {
+            const bool in0 = (uint32_t)(s2.x - 1) < (uint32_t)D, in1 = (uint32_t)(s2.y - 1) < (uint32_t)D;
+            if (!in0 || !in1 || (uint32_t)(e2.x - 1) >= (uint32_t)D || (uint32_t)(e2.y - 1) >= (uint32_t)D || (uint32_t)a2.x > 1u || (uint32_t)a2.y > 1u)
+                mask |= kIvEq8;
+            if (s2.x > e2.x || s2.y > e2.y) mask |= kIvEq2;
+            if (e2.x > s2.y) mask |= kIvEq3;
+            const bool act0 = a2.x == 1, act1 = a2.y == 1;
+            if (!act0) mask |= kIvEq7;
+            const int32_t k = (act0 ? 1 : 0) + (act1 ? 1 : 0);
+            n_act += k;
+            dur += wv * k;
+            idle |= k == 0;
+            const int32_t t0 = act0 ? s2.x : (act1 ? s2.y : 0), t1 = act1 ? s2.y : t0;
+            sts_u32(sa + 4u * (uint32_t)v, (uint32_t)(t0 & 0xFFFF) | (uint32_t)t1 << 16);
+            sts_u32(ea + 4u * (uint32_t)v, ((uint32_t)e2.x & 0x7FFFu) | (act0 ? 0x8000u : 0u) | ((uint32_t)e2.y & 0x7FFFu) << 16 | (act1 ? 0x80000000u : 0u));
+            if (in0) {
+                if (act0) sts_u16(da + 2u * (uint32_t)s2.x, (uint32_t)v + 1u);
+                asm volatile("st.shared.u8 [%0], %1;" ::"r"(all + (uint32_t)s2.x), "r"(1) : "memory");
+            }
+            if (in1) {
+                if (act1) sts_u16(da + 2u * (uint32_t)s2.y, (uint32_t)v + 1u);
+                asm volatile("st.shared.u8 [%0], %1;" ::"r"(all + (uint32_t)s2.y), "r"(1) : "memory");
+            }
+            n_distinct += s2.x != s2.y ? 2 : 1;
+        };
+        for (int32_t v = lane; v < n; v += 64) {              // two nodes' loads in flight
+            const int32_t u = min(v + 32, n - 1);
+            const int2 s0 = __ldg(gs + v), e0 = __ldg(ge + v), a0 = __ldg(ga + v), s1 = __ldg(gs + u), e1 = __ldg(ge + u), a1 = __ldg(ga + u);
+            const int64_t w0 = __ldg(p.w + v), w1 = __ldg(p.w + u);
+            node(v, s0, e0, a0, w0);
+            if (v + 32 < n) node(v + 32, s1, e1, a1, w1);
+        }
+        mask = __reduce_or_sync(kFull, mask);
+        if (mask & kIvEq8) {                                  // nothing else is evaluated
+            if (lane == 0) {
+                p.out_mask[b] = kIvEq8;
+                p.out_peak[b] = -1;
+                p.out_dur[b] = -1;
+                if (p.out_lens) p.out_lens[b] = -1;
+            }
+            if (pp.fill && p.out_seqs)
+                for (int32_t i = lane; i < K; i += 32) p.out_seqs[(int64_t)b * K + i] = -1;
+            __syncwarp();
+            continue;
+        }
+        __syncwarp();
+        // ---- events: distinct active starts, distinct starts (Eq. 6: as many as the nodes marked), and the sequence
+        const int32_t total = __reduce_add_sync(kFull, n_act);
+        int32_t R = 0, marked = 0;
+        for (int32_t t = lane; t < ((D + 32) & ~31); t += 32) {
+            uint32_t owner, any;
+            asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(owner) : "r"(da + 2u * (uint32_t)t) : "memory");
+            asm volatile("ld.shared.u8 %0, [%1];" : "=r"(any) : "r"(all + (uint32_t)t) : "memory");
+            R += owner != 0 ? 1 : 0;
+            marked += (int32_t)any;
+        }
+        R = __reduce_add_sync(kFull, R);
+        marked = __reduce_add_sync(kFull, marked);
+        if (marked != __reduce_add_sync(kFull, n_distinct)) mask |= kIvEq6;
+        const bool has_seq = R == total;
+        if (p.out_seqs) {
+            int32_t* row = p.out_seqs + (int64_t)b * K;
+            int32_t at = 0;
+            if (has_seq) {
+                for (int32_t t = lane; t < ((D + 32) & ~31); t += 32) {
+                    uint32_t owner;
+                    asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(owner) : "r"(da + 2u * (uint32_t)t) : "memory");
+                    const uint32_t here = __ballot_sync(kFull, owner != 0);
+                    if (owner != 0) row[at + __popc(here & ((1u << lane) - 1u))] = (int32_t)owner - 1;
+                    at += __popc(here);
+                }
+            }
+            if (pp.fill)
+                for (int32_t i = at + lane; i < K; i += 32) row[i] = -1;
+        }
+        __syncwarp();
+        clear_events();
+        // ---- pass 2, per node slot: Eq. 4 and Eq. 5
+        uint32_t viol = 0, prec = rec0, ps = sell0;
+        for (int d = 0; d < pp.n_tiles; ++d, prec += 64u * kRecB) {
+            uint32_t nlo[2][2], len[2][2];        // [slot][half]: -(s + 1) and e - s - 1 of the half's node, in both 16-bit halves
+            uint32_t rows_x = 0;
+            const uint32_t e_first = lds_u32(ps);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t x;
+                Amount<MemT> m;
+                if constexpr (sizeof(MemT) == 4) {
+                    const uint2 r = lds_v2(prec + 32u * kRecB * h);
+                    x = r.x;
+                    m.v = (MemT)r.y;
+                } else {
+                    const uint4 r = lds_v4(prec + 32u * kRecB * h);
+                    x = r.x;
+                    m.lo = r.z;
+                    m.hi = r.w;
+                }
+                if (h == 0) rows_x = x;
+                const uint32_t off = x & 0xFFFFu, sp = lds_u32(sa + off), ep = lds_u32(ea + off);
+                const bool sink = (h == 0 ? e_first & 0xFFFFu : e_first >> 16) == off;       // no successor: everything is served
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const uint32_t s = i == 0 ? sp & 0xFFFFu : sp >> 16, e = (i == 0 ? ep : ep >> 16) & 0x7FFFu;
+                    const bool act = (ep & (i == 0 ? 0x8000u : 0x80000000u)) != 0;
+                    if (act && s <= e) {
+                        red_add_amount(da + (s << kShift), m);
+                        red_sub_amount(da + ((e + 1u) << kShift), m);
+                    }
+                    const bool serves = act && e > s;
+                    const uint32_t lo = serves ? s + 1u : 0xFFFFu, ln = serves ? e - s - 1u : 0u;
+                    nlo[i][h] = sink ? 0u : ((0u - lo) & 0xFFFFu) * 0x10001u;
+                    len[i][h] = sink ? 0xFFFFFFFFu : ln * 0x10001u;
+                }
+            }
+            const int rows = __shfl_sync(kFull, (int)(rows_x >> 16), 0);
+            uint32_t e = e_first;
+            for (int k = 0; k < rows; ++k) {
+                ps += 128u;
+                const uint32_t r0 = lds_u32(sa + (e & 0xFFFFu)), r1 = lds_u32(sa + (e >> 16));
+                if (k + 1 < rows) e = lds_u32(ps);
+                viol |= min_u16x2(__viaddmax_u16x2(r0, nlo[0][0], len[0][0]) - len[0][0], __viaddmax_u16x2(r0, nlo[1][0], len[1][0]) - len[1][0]);
+                viol |= min_u16x2(__viaddmax_u16x2(r1, nlo[0][1], len[0][1]) - len[0][1], __viaddmax_u16x2(r1, nlo[1][1], len[1][1]) - len[1][1]);
+            }
+        }
+        if (__any_sync(kFull, idle)) {
+            // a successor without an active slot asks for nothing: Eq. 5 edge by edge
+            viol = 0;
+            for (int32_t u = lane; u < n; u += 32) {
+                const uint32_t sp = lds_u32(sa + 4u * (uint32_t)u), ep = lds_u32(ea + 4u * (uint32_t)u);
+                const uint32_t s0 = sp & 0xFFFFu, s1 = sp >> 16, e0 = (ep & 0x8000u) ? ep & 0x7FFFu : 0u, e1 = ep >> 31 ? ep >> 16 & 0x7FFFu : 0u;
+                for (int32_t k = __ldg(p.succ_start + u); k < __ldg(p.succ_start + u + 1); ++k) {
+                    const uint32_t r = lds_u32(sa + 4u * (uint32_t)__ldg(p.succ + k));
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const uint32_t t = i == 0 ? r & 0xFFFFu : r >> 16;
+                        if (t != 0 && !((t > s0 && t <= e0) || (t > s1 && t <= e1))) viol = 1;
+                    }
+                }
+            }
+        }
+        if (__any_sync(kFull, viol != 0)) mask |= kIvEq5;
+        __syncwarp();
+        // ---- usage per event and its maximum: lane owns V consecutive vectors
+        int64_t peak;
+        {
+            const int V = (int)(pp.event_bytes / 512u);
+            uint32_t ad = da + 16u * (uint32_t)(lane * V), lo = 0, hi = 0;
+            MemT top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
+            for (int j = 0; j < V; ++j, ad += 16u) {
+                const uint4 q = lds_v4(ad);
+                if constexpr (sizeof(MemT) == 4) {
+                    lo += q.x; top = max(top, (MemT)lo);
+                    lo += q.y; top = max(top, (MemT)lo);
+                    lo += q.z; top = max(top, (MemT)lo);
+                    lo += q.w; top = max(top, (MemT)lo);
+                } else {
+                    lo += q.x; hi += q.y;
+                    MemT at = split_value(lo, hi, pp.split);
+                    top = at > top ? at : top;
+                    lo += q.z; hi += q.w;
+                    at = split_value(lo, hi, pp.split);
+                    top = at > top ? at : top;
+                }
+            }
+            if constexpr (sizeof(MemT) == 4) top += (MemT)(warp_inclusive_sum(lo, lane) - lo);
+            else top += split_value(warp_inclusive_sum(lo, lane) - lo, warp_inclusive_sum(hi, lane) - hi, pp.split);
+            peak = (int64_t)warp_max_t(top);
+        }
+        if (peak > p.M) mask |= kIvEq4;
+        dur = warp_sum64(dur);
+        if (lane == 0) {
+            p.out_mask[b] = mask;
+            p.out_peak[b] = peak;
+            p.out_dur[b] = dur;
+            if (p.out_lens) p.out_lens[b] = has_seq ? R : -1;
+        }
+        __syncwarp();
+    }
+}
+
+}  // namespace moc

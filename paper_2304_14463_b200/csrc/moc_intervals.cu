@@ -3,13 +3,46 @@
 
 #include "moc_host.cuh"
 #include "moc_interval_kernels.cuh"
+#include "moc_interval_plain_kernel.cuh"
 
 using namespace moc_host;
 
-extern "C" int moc_check_intervals(const moc_graph* g, const int32_t* s, const int32_t* e, const int32_t* a,
-                                   int32_t B, int64_t D, const int32_t* topo_index, int64_t M, int64_t* out_peak,
-                                   int64_t* out_dur, int32_t* out_mask, int32_t* out_seqs, int32_t* out_lens,
-                                   void* stream) {
+namespace {
+
+// Launch of the kernel for the plain domain with two slots per node; false when the case is not its own.
+bool launch_plain(const moc_graph* g, const moc::IntervalParams& q, bool fill, cudaStream_t st, cudaError_t* err) {
+    const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    if (q.topo_index || g->C != 2 || q.D > 32766 || !g->d_rec32 || (wide && !g->split_ok)) return false;
+    if ((reinterpret_cast<uintptr_t>(q.s) | reinterpret_cast<uintptr_t>(q.e) | reinterpret_cast<uintptr_t>(q.a)) & 7) return false;
+    moc::IntervalPlainParams p{};
+    p.q = q;
+    p.n_tiles = g->n_tiles;
+    p.split = g->split;
+    p.rec = wide ? g->d_rec64 : g->d_rec32;
+    p.sell = g->d_sell_iv;
+    p.rec_bytes = (wide ? 16u : 8u) * 64u * (uint32_t)g->n_tiles;
+    p.sell_bytes = (4u * (uint32_t)g->sell_len + 15u) & ~15u;
+    p.word_bytes = (4u * ((uint32_t)g->n + 2u) + 15u) & ~15u;
+    p.event_bytes = (uint32_t)moc::interval_plain_event_bytes(q.D, wide ? 8 : 4);
+    p.fill = fill;
+    const size_t warp_b = 2 * ((size_t)p.word_bytes + moc::kPairWordTail) + p.event_bytes, graph_b = (size_t)p.rec_bytes + p.sell_bytes;
+    if (graph_b + 4 * warp_b > g->smem_optin) return false;
+    const void* fn = wide ? (const void*)moc::check_plain_kernel<int64_t> : (const void*)moc::check_plain_kernel<int32_t>;
+    *err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_optin);
+    if (*err != cudaSuccess) return true;
+    // one block per SM; warps: the rounds a full block needs, evenly filled, at least eight to stage the graph
+    const int most = (int)std::min<size_t>(moc::kIvPlainThreads / 32, (g->smem_optin - graph_b) / warp_b);
+    const int64_t per_sm = ((int64_t)q.B + g->sm_count - 1) / g->sm_count, rounds = (per_sm + most - 1) / most;
+    const int wpb = (int)std::min<int64_t>(most, std::max<int64_t>(8, (per_sm + rounds - 1) / rounds));
+    const int grid = (int)std::min<int64_t>(g->sm_count, q.B);
+    void* args[] = {&p};
+    *err = cudaLaunchKernel(fn, dim3(grid), dim3(32 * wpb), args, graph_b + (size_t)wpb * warp_b, st);
+    return true;
+}
+
+int check_intervals(const moc_graph* g, const int32_t* s, const int32_t* e, const int32_t* a, int32_t B, int64_t D,
+                    const int32_t* topo_index, int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_mask, int32_t* out_seqs,
+                    int32_t* out_lens, bool fill, void* stream) {
     clear_error();
     launch_counter() = 0;
     if (!g || B < 0) return fail(MOC_ERR_ARG, "moc_check_intervals: null handle or B < 0");
@@ -42,6 +75,12 @@ extern "C" int moc_check_intervals(const moc_graph* g, const int32_t* s, const i
     p.out_mask = out_mask;
     p.out_seqs = out_seqs;
     p.out_lens = out_lens;
+    cudaError_t err = cudaSuccess;
+    if (launch_plain(g, p, fill, (cudaStream_t)stream, &err)) {
+        MOC_CUDA(err);
+        launch_counter() = 1;
+        return MOC_OK;
+    }
     p.words = (uint32_t)((D + 32) / 32);
     const bool plain = topo_index == nullptr;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;     // C * sum(m) bounds every partial usage sum
@@ -62,6 +101,7 @@ extern "C" int moc_check_intervals(const moc_graph* g, const int32_t* s, const i
         const int fit = blk <= cap + 1024 ? (int)((g->smem_optin) / blk) * k : 0;
         if (fit > best) { best = fit; wpb = k; }
     }
+    if (fill && out_seqs) MOC_CUDA(cudaMemsetAsync(out_seqs, 0xFF, (size_t)B * (size_t)K * 4, (cudaStream_t)stream));
     const size_t smem = warp_b * wpb;
     using Fn = void (*)(const moc::IntervalParams);
     const int cp = g->C <= 2 ? 2 : (g->C <= 4 ? 4 : 8);
@@ -85,4 +125,19 @@ extern "C" int moc_check_intervals(const moc_graph* g, const int32_t* s, const i
     MOC_CUDA(cudaGetLastError());
     launch_counter() = 1;
     return MOC_OK;
+}
+
+}  // namespace
+
+extern "C" int moc_check_intervals(const moc_graph* g, const int32_t* s, const int32_t* e, const int32_t* a, int32_t B, int64_t D,
+                                   const int32_t* topo_index, int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_mask,
+                                   int32_t* out_seqs, int32_t* out_lens, void* stream) {
+    return check_intervals(g, s, e, a, B, D, topo_index, M, out_peak, out_dur, out_mask, out_seqs, out_lens, false, stream);
+}
+
+// For the torch side of the binding: the whole of out_seqs is written, -1 behind the sequences.
+extern "C" int moc_check_intervals_filled(const moc_graph* g, const int32_t* s, const int32_t* e, const int32_t* a, int32_t B, int64_t D,
+                                          const int32_t* topo_index, int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_mask,
+                                          int32_t* out_seqs, int32_t* out_lens, void* stream) {
+    return check_intervals(g, s, e, a, B, D, topo_index, M, out_peak, out_dur, out_mask, out_seqs, out_lens, true, stream);
 }

@@ -72,10 +72,10 @@ struct PairParams {
 // 64-bit sums without 64-bit atomics (which shared memory emulates with compare-and-swap loops: twice the time
 // of the whole kernel).  A delta entry is two 32-bit words that are added to separately: the amounts mod 2^32, and the
 // amounts >> k.  A sum S of deltas up to some step is a difference of two sets of resident outputs, at most
-// n of them each, so that with L and H the sums of the two words
-//     S = 2^k H + (something below n 2^k in absolute value),   S = L (mod 2^32),
-// which determines S when n 2^k <= 2^31: S = 2^k H + sign-extended (L - 2^k H mod 2^32).  H itself fits 32 bits when
-// sum(m) < 2^(31 + k); graphs beyond that (sum(m) >= 2^53 at n = 442) use the general kernels.
+// 2 n of them each, so that with L and H the sums of the two words
+//     S = 2^k H + (something below 2 n 2^k in absolute value),   S = L (mod 2^32),
+// which determines S when 2 n 2^k <= 2^31: S = 2^k H + sign-extended (L - 2^k H mod 2^32).  H itself fits 32 bits when
+// 2 sum(m) < 2^(31 + k); graphs beyond that (sum(m) >= 2^51 at n = 442) use the general kernels.
 template <typename MemT> struct Amount { MemT v; };
 template <> struct Amount<int64_t> { uint32_t lo, hi; };
 __device__ __forceinline__ int64_t split_value(uint32_t lo, uint32_t hi, int32_t k) {

@@ -26,7 +26,7 @@ namespace {
 
 decltype(&moc_eval_batch) f_eval_batch;
 decltype(&moc_mem_profile) f_mem_profile;
-decltype(&moc_check_intervals) f_check_intervals;
+decltype(&moc_check_intervals) f_check_intervals_filled;   // writes the whole rows, -1 behind the sequences
 decltype(&moc_cache_build) f_cache_build;
 decltype(&moc_eval_edits) f_eval_edits;
 decltype(&moc_search_run) f_search_run;
@@ -244,12 +244,11 @@ PyObject* py_check_intervals(PyObject*, PyObject* const* a, Py_ssize_t na) {
         at::Tensor pk = empty({B}, at::kLong, d), du = empty({B}, at::kLong, d), mask = empty({B}, at::kInt, d), seqs, lens;
         if (want) {
             seqs = empty({B, K}, at::kInt, d);
-            seqs.fill_(-1);
             lens = empty({B}, at::kInt, d);
         }
         void* cs = stream();
         const int rc = unlocked([&] {
-            return f_check_intervals((const moc_graph*)g, ptr<int32_t>(*s), ptr<int32_t>(*e), ptr<int32_t>(*f), (int32_t)B, D,
+            return f_check_intervals_filled((const moc_graph*)g, ptr<int32_t>(*s), ptr<int32_t>(*e), ptr<int32_t>(*f), (int32_t)B, D,
                                      topo ? ptr<int32_t>(*topo) : nullptr, M, ptr<int64_t>(pk), ptr<int64_t>(du), ptr<int32_t>(mask),
                                      want ? ptr<int32_t>(seqs) : nullptr, want ? ptr<int32_t>(lens) : nullptr, cs);
         });
@@ -311,7 +310,7 @@ PyObject* py_bind(PyObject*, PyObject* d) {
     if (PyErr_Occurred()) return nullptr
     MOC_BIND(eval_batch);
     MOC_BIND(mem_profile);
-    MOC_BIND(check_intervals);
+    MOC_BIND(check_intervals_filled);
     MOC_BIND(cache_build);
     MOC_BIND(eval_edits);
     MOC_BIND(search_run);
