@@ -79,94 +79,94 @@ __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const I
         const int2* gs = reinterpret_cast<const int2*>(p.s + (int64_t)b * K);
         const int2* ge = reinterpret_cast<const int2*>(p.e + (int64_t)b * K);
         const int2* ga = reinterpret_cast<const int2*>(p.a + (int64_t)b * K);
-        if (b + step < p.B) {                     // the next solution comes into L2 meanwhile
-            const int64_t ahead = (int64_t)step * K * 4;
-            for (int32_t o = 128 * lane; o < 4 * K; o += 4096) {
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(gs) + ahead + o));
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(ge) + ahead + o));
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(ga) + ahead + o));
-            }
-        }
         clear_events();
-        // ---- pass 1, per node: Eqs. 1, 2, 3, 7, 8; marks of the starts; the solution on chip
-        int32_t mask = 0, n_act = 0, n_distinct = 0;
-        int64_t dur = 0;
-        bool idle = false;                        // some node has no active slot
-        auto node = [&](int32_t v, const int2 s2, const int2 e2, const int2 a2, const int64_t wv) {
-            const bool in0 = (uint32_t)(s2.x - 1) < (uint32_t)D, in1 = (uint32_t)(s2.y - 1) < (uint32_t)D;
-            if (!in0 || !in1 || (uint32_t)(e2.x - 1) >= (uint32_t)D || (uint32_t)(e2.y - 1) >= (uint32_t)D || (uint32_t)a2.x > 1u || (uint32_t)a2.y > 1u)
-                mask |= kIvEq8;
-            if (s2.x > e2.x || s2.y > e2.y) mask |= kIvEq2;
-            if (e2.x > s2.y) mask |= kIvEq3;
-            const bool act0 = a2.x == 1, act1 = a2.y == 1;
-            if (!act0) mask |= kIvEq7;
-            const int32_t k = (act0 ? 1 : 0) + (act1 ? 1 : 0);
-            n_act += k;
-            dur += wv * k;
-            idle |= k == 0;
-            const int32_t t0 = act0 ? s2.x : (act1 ? s2.y : 0), t1 = act1 ? s2.y : t0;
-            sts_u32(sa + 4u * (uint32_t)v, (uint32_t)(t0 & 0xFFFF) | (uint32_t)t1 << 16);
-            sts_u32(ea + 4u * (uint32_t)v, ((uint32_t)e2.x & 0x7FFFu) | (act0 ? 0x8000u : 0u) | ((uint32_t)e2.y & 0x7FFFu) << 16 | (act1 ? 0x80000000u : 0u));
-            if (in0) {
-                if (act0) sts_u16(da + 2u * (uint32_t)s2.x, (uint32_t)v + 1u);
-                asm volatile("st.shared.u8 [%0], %1;" ::"r"(all + (uint32_t)s2.x), "r"(1) : "memory");
-            }
-            if (in1) {
-                if (act1) sts_u16(da + 2u * (uint32_t)s2.y, (uint32_t)v + 1u);
-                asm volatile("st.shared.u8 [%0], %1;" ::"r"(all + (uint32_t)s2.y), "r"(1) : "memory");
-            }
-            n_distinct += s2.x != s2.y ? 2 : 1;
+        // ---- pass 1, per node: Eqs. 1, 2, 3, 7, 8; marks of the starts; the solution on chip.  The tests gather as running
+        // extremes that are looked at once: a value outside its domain makes the rest meaningless, but harmless.
+        uint32_t far = 0, flag = 0, first = 1, none = 1, n_act = 0, n_same = 0, dur_hi = 0;
+        int32_t late = INT32_MIN, lap = INT32_MIN;
+        uint64_t dur_lo = 0;
+        auto node = [&](uint32_t v4, const int2 s2, const int2 e2, const int2 a2, const uint2 w2) {
+            far = __viaddmax_u32((uint32_t)s2.x, 0xFFFFFFFFu, far);           // Eq. 8: largest s - 1, e - 1 and a
+            far = __viaddmax_u32((uint32_t)s2.y, 0xFFFFFFFFu, far);
+            far = __viaddmax_u32((uint32_t)e2.x, 0xFFFFFFFFu, far);
+            far = __viaddmax_u32((uint32_t)e2.y, 0xFFFFFFFFu, far);
+            const uint32_t a0 = (uint32_t)a2.x, a1 = (uint32_t)a2.y;
+            flag = max(flag, a0 | a1);
+            late = max(late, max(s2.x - e2.x, s2.y - e2.y));                  // Eq. 2: s > e
+            lap = max(lap, e2.x - s2.y);                                      // Eq. 3: e > next s
+            first = min(first, a0);                                           // Eq. 7
+            none = min(none, a0 | a1);
+            n_act += a0 + a1;
+            dur_lo += (uint64_t)w2.x * (a0 + a1);
+            dur_hi += w2.y * (a0 + a1);
+            n_same += s2.x == s2.y ? 1u : 0u;
+            const int32_t t0 = a0 ? s2.x : (a1 ? s2.y : 0), t1 = a1 ? s2.y : t0;
+            sts_u32(sa + v4, __byte_perm((uint32_t)t0, (uint32_t)t1, 0x5410));
+            sts_u32(ea + v4, __byte_perm((uint32_t)e2.x, (uint32_t)e2.y, 0x5410) | a0 << 15 | a1 << 31);
+            const uint32_t m0 = min((uint32_t)s2.x, (uint32_t)D), m1 = min((uint32_t)s2.y, (uint32_t)D);
+            asm volatile("st.shared.u8 [%0], %1;" ::"r"(all + m0), "r"(1) : "memory");
+            asm volatile("st.shared.u8 [%0], %1;" ::"r"(all + m1), "r"(1) : "memory");
+            if (a0) sts_u16(da + 2u * m0, (v4 >> 2) + 1u);
+            if (a1) sts_u16(da + 2u * m1, (v4 >> 2) + 1u);
         };
-        for (int32_t v = lane; v < n; v += 64) {              // two nodes' loads in flight
-            const int32_t u = min(v + 32, n - 1);
-            const int2 s0 = __ldg(gs + v), e0 = __ldg(ge + v), a0 = __ldg(ga + v), s1 = __ldg(gs + u), e1 = __ldg(ge + u), a1 = __ldg(ga + u);
-            const int64_t w0 = __ldg(p.w + v), w1 = __ldg(p.w + u);
-            node(v, s0, e0, a0, w0);
-            if (v + 32 < n) node(v + 32, s1, e1, a1, w1);
+        const uint2* gw = reinterpret_cast<const uint2*>(p.w);
+        for (int32_t v = lane; v < n; v += 128) {             // four nodes' loads in flight
+            int2 s4[4], e4[4], a4[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int32_t u = min(v + 32 * k, n - 1);
+                s4[k] = __ldg(gs + u);
+                e4[k] = __ldg(ge + u);
+                a4[k] = __ldg(ga + u);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (v + 32 * k < n) node(4u * (uint32_t)(v + 32 * k), s4[k], e4[k], a4[k], __ldg(gw + v + 32 * k));
         }
-        mask = __reduce_or_sync(kFull, mask);
-        if (mask & kIvEq8) {                                  // nothing else is evaluated
+        int32_t* row = p.out_seqs ? p.out_seqs + (int64_t)b * K : nullptr;
+        if (__any_sync(kFull, far >= (uint32_t)D || flag > 1u)) {     // Eq. 8: nothing else is evaluated
             if (lane == 0) {
                 p.out_mask[b] = kIvEq8;
                 p.out_peak[b] = -1;
                 p.out_dur[b] = -1;
                 if (p.out_lens) p.out_lens[b] = -1;
             }
-            if (pp.fill && p.out_seqs)
-                for (int32_t i = lane; i < K; i += 32) p.out_seqs[(int64_t)b * K + i] = -1;
+            if (pp.fill && row)
+                for (int32_t i = lane; i < K; i += 32) row[i] = -1;
             __syncwarp();
             continue;
         }
+        int32_t mask = (late > 0 ? kIvEq2 : 0) | (lap > 0 ? kIvEq3 : 0) | (first != 1u ? kIvEq7 : 0);
+        const bool idle = none == 0;              // some node has no active slot
         __syncwarp();
-        // ---- events: distinct active starts, distinct starts (Eq. 6: as many as the nodes marked), and the sequence
-        const int32_t total = __reduce_add_sync(kFull, n_act);
-        int32_t R = 0, marked = 0;
-        for (int32_t t = lane; t < ((D + 32) & ~31); t += 32) {
-            uint32_t owner, any;
+        // ---- events: distinct starts (Eq. 6: as many as the nodes marked), distinct active starts, and the sequence
+        const int32_t total = (int32_t)__reduce_add_sync(kFull, n_act), n_ev = (D + 32) & ~31;
+        {
+            uint32_t marked = 0;
+            for (uint32_t o = 4u * (uint32_t)lane; o < (uint32_t)n_ev; o += 128u) marked = __dp4a(lds_u32(all + o), 0x01010101u, marked);
+            if ((int32_t)__reduce_add_sync(kFull, marked) != 2 * n - (int32_t)__reduce_add_sync(kFull, n_same)) mask |= kIvEq6;
+        }
+        auto owner_of = [&](int32_t t) -> uint32_t {
+            uint32_t owner;
             asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(owner) : "r"(da + 2u * (uint32_t)t) : "memory");
-            asm volatile("ld.shared.u8 %0, [%1];" : "=r"(any) : "r"(all + (uint32_t)t) : "memory");
-            R += owner != 0 ? 1 : 0;
-            marked += (int32_t)any;
-        }
-        R = __reduce_add_sync(kFull, R);
-        marked = __reduce_add_sync(kFull, marked);
-        if (marked != __reduce_add_sync(kFull, n_distinct)) mask |= kIvEq6;
-        const bool has_seq = R == total;
-        if (p.out_seqs) {
-            int32_t* row = p.out_seqs + (int64_t)b * K;
+            return owner;
+        };
+        // The row is written while its length is counted when it may be repaired afterwards (two active intervals with
+        // one start leave no sequence), else after the count.
+        int32_t R = 0;
+        for (int pass = (pp.fill && row) ? 1 : 0; pass < 2; ++pass) {
+            if (pass == 1 && (!row || (!pp.fill && R != total))) break;
             int32_t at = 0;
-            if (has_seq) {
-                for (int32_t t = lane; t < ((D + 32) & ~31); t += 32) {
-                    uint32_t owner;
-                    asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(owner) : "r"(da + 2u * (uint32_t)t) : "memory");
-                    const uint32_t here = __ballot_sync(kFull, owner != 0);
-                    if (owner != 0) row[at + __popc(here & ((1u << lane) - 1u))] = (int32_t)owner - 1;
-                    at += __popc(here);
-                }
+            for (int32_t t = lane; t < n_ev; t += 32) {
+                const uint32_t owner = owner_of(t), here = __ballot_sync(kFull, owner != 0);
+                if (pass == 1 && owner != 0) row[at + __popc(here & ((1u << lane) - 1u))] = (int32_t)owner - 1;
+                at += __popc(here);
             }
-            if (pp.fill)
-                for (int32_t i = at + lane; i < K; i += 32) row[i] = -1;
+            R = at;
         }
+        const bool has_seq = R == total;
+        if (pp.fill && row)
+            for (int32_t i = (has_seq ? R : 0) + lane; i < K; i += 32) row[i] = -1;
         __syncwarp();
         clear_events();
         // ---- pass 2, per node slot: Eq. 4 and Eq. 5
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const I
                 }
             }
         }
-        if (__any_sync(kFull, viol != 0)) mask |= kIvEq5;
+        if (viol != 0) mask |= kIvEq5;
         __syncwarp();
         // ---- usage per event and its maximum: lane owns V consecutive vectors
         int64_t peak;
@@ -261,7 +261,8 @@ __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const I
             peak = (int64_t)warp_max_t(top);
         }
         if (peak > p.M) mask |= kIvEq4;
-        dur = warp_sum64(dur);
+        const int64_t dur = warp_sum64((int64_t)(dur_lo + ((uint64_t)dur_hi << 32)));
+        mask = __reduce_or_sync(kFull, mask);
         if (lane == 0) {
             p.out_mask[b] = mask;
             p.out_peak[b] = peak;
