@@ -133,16 +133,18 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
             ss0 = Gr.succ_start(x); ss1 = Gr.succ_start(x + 1);
             // ---- precedence (Eq. 5) can only break on edges that touch x: no first copy of a
             // predecessor behind the first copy of x, no first copy of a successor in front of it
+            // (four reads of each kind in flight: with the parent in global memory their latency is what the test costs)
             bool viol = false;
-#pragma unroll 1
-            for (int32_t k = ps0; k < ps1; ++k) {
-                const uint32_t wv = P.occ(Gr.pred(k));
-                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) > ta0;
-            }
-#pragma unroll 1
-            for (int32_t k = ss0; k < ss1; ++k) {
-                const uint32_t wv = P.occ(Gr.succ(k));
-                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) < tb0;
+            for (int32_t k = 0; k < max(ps1 - ps0, ss1 - ss0); k += 4) {
+                uint32_t pw[4], sw[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    pw[i] = ps0 + k + i < ps1 ? P.occ(Gr.pred(ps0 + k + i)) : 0u;
+                    sw[i] = ss0 + k + i < ss1 ? P.occ(Gr.succ(ss0 + k + i)) : 0xFFFFFFFFu;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    viol |= (int32_t)min(pw[i] & 0xFFFFu, pw[i] >> 16) > ta0 || (int32_t)min(sw[i] & 0xFFFFu, sw[i] >> 16) < tb0;
             }
             if (viol) out_st = -1;
             else adm = true;
@@ -186,11 +188,18 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
                 const uint32_t seed = (uint32_t)(ta - tb) & 0xFFFFu;
                 uint32_t G = seed | seed << 16, m2 = 0;
 #pragma unroll 1
-                for (int32_t z = s0; z < s1; ++z) {
-                    const int32_t v = Gr.succ(z);
-                    const uint32_t wv = v == x ? 0u : P.occ(v);          // the copies of x are added in child steps
-                    G = __viaddmax_u16x2(wv, nbb, G);
-                    m2 = max_u16x2(m2, wv);
+                for (int32_t z = s0; z < s1; z += 4) {
+                    uint32_t wv[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int32_t v = z + i < s1 ? Gr.succ(z + i) : x;
+                        wv[i] = v == x ? 0u : P.occ(v);                  // the copies of x are added in child steps
+                    }
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        G = __viaddmax_u16x2(wv[i], nbb, G);
+                        m2 = max_u16x2(m2, wv[i]);
+                    }
                 }
                 mx = max(m2 & 0xFFFFu, m2 >> 16);
                 R = ((uint32_t)tb + max(G & 0xFFFFu, G >> 16)) & 0xFFFFu;
