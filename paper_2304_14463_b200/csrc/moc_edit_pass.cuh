@@ -223,14 +223,17 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
                 emit(n0, f0, mxv);
                 if (two) emit(n1, f1, mxv);
             }
+            uint32_t wy_next = ps0 < ps1 ? P.occ(Gr.pred(ps0)) : 0u;
 #pragma unroll 1
             for (int32_t k = ps0; k < ps1; ++k) {                   // ---- the predecessors of x
                 const int32_t y = Gr.pred(k);
                 const MemT my = Gr.m(y);
-                const uint32_t wy = P.occ(y);
+                const uint32_t wy = wy_next;                        // one predecessor ahead
+                if (k + 1 < ps1) wy_next = P.occ(Gr.pred(k + 1));
                 const int32_t ya1 = (int32_t)min(wy & 0xFFFFu, wy >> 16), yb1 = (int32_t)max(wy & 0xFFFFu, wy >> 16);
                 const int32_t ya = ya1 - 1, yb = yb1 - 1;
                 const bool two = ya != yb;
+                const int32_t fa = P.fre(ya), fb = P.fre(yb);         // in flight with the successors' words
                 const int32_t n0 = map(ya), n1 = map(yb);
                 uint32_t mx, R;
                 scan_succ(Gr.succ_start(y), Gr.succ_start(y + 1), ya1, yb1, mx, R);
@@ -241,10 +244,10 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
                 if (c1 != kEditNone && c1 > n0 && c1 < n1) f0 = max(f0, c1);
                 if (!two) f0 = f1;
                 int32_t l, h;
-                old_range(ya, P.fre(ya), false, l, h);
+                old_range(ya, fa, false, l, h);
                 if (h != f0) emit(min(h, f0) + 1, max(h, f0), f0 > h ? my : (MemT)(-my));
                 if (two) {
-                    old_range(yb, P.fre(yb), false, l, h);
+                    old_range(yb, fb, false, l, h);
                     if (h != f1) emit(min(h, f1) + 1, max(h, f1), f1 > h ? my : (MemT)(-my));
                 }
             }
