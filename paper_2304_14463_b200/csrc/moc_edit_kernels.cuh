@@ -205,6 +205,7 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                 // word (end of the last copy with the precedence test, end of the first copy).
                 constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u;
                 const uint32_t wa = (uint32_t)__cvta_generic_to_shared(word);
+                uint16_t* fre16 = reinterpret_cast<uint16_t*>(arrB);
                 const char* prec = (kChip ? smem : reinterpret_cast<const char*>(p.rec)) + kRecB * lane;
                 const uint64_t* pw = (kChip ? reinterpret_cast<const uint64_t*>(smem + p.chip_w_b) : p.wslot) + lane;
                 const uint32_t* ps = (kChip ? reinterpret_cast<const uint32_t*>(smem + p.chip_sell_b) : p.sell) + lane;
@@ -268,11 +269,11 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                         const uint32_t a16 = ab[h] & 0xFFFFu, b16 = ab[h] >> 16, fb = v & 0xFFFFu, fa = v >> 16;
                         const bool real = xoff[h] != empty_off;          // empty slots own the constant word: no step is theirs
                         if (real && b16 != 0) {
-                            arrB[b16 - 1] = (MemT)fb - 1;                // free steps gather on chip, written out in order below
+                            fre16[b16 - 1] = (uint16_t)(fb - 1);         // free steps gather on chip, written out in order below
                             edit_add(&arrA[b16 - 1], mm[h]);
                             edit_add(&arrA[fb], (MemT)(-mm[h]));
                             if (a16 != b16) {
-                                arrB[a16 - 1] = (MemT)fa - 1;
+                                fre16[a16 - 1] = (uint16_t)(fa - 1);
                                 edit_add(&arrA[a16 - 1], mm[h]);
                                 edit_add(&arrA[fa], (MemT)(-mm[h]));
                                 const uint64_t wx = ld64(pw + 32 * h);
@@ -290,12 +291,8 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                 over = __any_sync(kFull, (int32_t)capw < 0) || (int)((acc_all >> kPairCntShift) & 0x7FFFu) != T - n;
                 dep = (depw & 0x80008000u) != 0;
                 __syncwarp();
-                for (int32_t t = 8 * lane; t < T; t += 256) {             // eight free steps per 16-byte store
-                    uint32_t q[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) q[i] = ((uint32_t)arrB[t + 2 * i] & 0xFFFFu) | (uint32_t)arrB[t + 2 * i + 1] << 16;
-                    *reinterpret_cast<uint4*>(fre + t) = make_uint4(q[0], q[1], q[2], q[3]);
-                }
+                for (int32_t t = 8 * lane; t < T; t += 256)               // eight free steps per 16-byte store
+                    *reinterpret_cast<uint4*>(fre + t) = *reinterpret_cast<const uint4*>(fre16 + t);
                 // position sum and duration in the form the rest of the kernel expects
                 vsum = lane == 0 ? (uint32_t)T * ((uint32_t)T + 1u) / 2u : 0u;
                 dur = lane == 0 ? p.base_dur + (int64_t)(acc_all & kPairDurMask) : 0;
