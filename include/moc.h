@@ -124,10 +124,10 @@ int moc_eval_batch(const moc_graph* g, const int32_t* seqs, const int32_t* lens,
  * with respect to the host, pageable memory works too): copies seqs (n_steps ints, which must be
  * at least sum(max(lens[b],0))) and lens to device staging owned by the handle, evaluates, copies
  * the three outputs back and synchronises `stream` before returning.  Large batches travel in
- * four chunks of whole sequences (a half, a quarter and two eighths of the steps): a copy stream
- * owned by the handle brings one chunk while `stream` evaluates the one before, so that only the
- * evaluation of the small last chunk is not hidden, and the results return in a single copy
- * through a pinned block of the handle.  One call at a time per handle.
+ * three parts (11, 4 and 1 sixteenths of the ids): a copy stream owned by the handle brings one part while
+ * `stream` evaluates the sequences that are complete with the one before, so that only the evaluation of
+ * the small last part is not hidden; results return to pinned arrays straight from the device and to
+ * pageable ones through a pinned block of the handle.  One call at a time per handle.
  */
 int moc_eval_batch_host(const moc_graph* g, const int32_t* seqs, int64_t n_steps,
                         const int32_t* lens, int32_t B, int64_t M, int64_t* out_peak,

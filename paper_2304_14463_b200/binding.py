@@ -247,6 +247,9 @@ def moc_eval_batch_noalloc(g, seqs, lens, M, out_peak, out_dur, out_feasible):
 
 def moc_eval_batch_host(g, seqs, lens, M, out_peak, out_dur, out_feasible):
     """Host arrays (numpy or CPU tensors, ideally pinned) in and out; returns after the results landed."""
+    r = _fast.eval_batch_host(g, seqs, lens, M, out_peak, out_dur, out_feasible, 32)
+    if r is not None:
+        return r if r.__class__ is tuple else _check(r, "moc_eval_batch_host")
     import numpy as np
     B = int(lens.shape[0])
     rc = lib.moc_eval_batch_host(g, _host(seqs, np.int32, "seqs"), int(seqs.shape[0]), _host(lens, np.int32, "lens"),
@@ -258,6 +261,9 @@ def moc_eval_batch_host(g, seqs, lens, M, out_peak, out_dur, out_feasible):
 
 def moc_eval_batch_host16(g, seqs, lens, M, out_peak, out_dur, out_feasible):
     """moc_eval_batch_host with uint16 node ids (n <= 65535): half the bytes over the host link."""
+    r = _fast.eval_batch_host(g, seqs, lens, M, out_peak, out_dur, out_feasible, 16)
+    if r is not None:
+        return r if r.__class__ is tuple else _check(r, "moc_eval_batch_host16")
     import numpy as np
     B = int(lens.shape[0])
     rc = lib.moc_eval_batch_host16(g, _host(seqs, np.uint16, "seqs"), int(seqs.shape[0]), _host(lens, np.int32, "lens"),

@@ -1289,12 +1289,26 @@ int moc_eval_batch(const moc_graph* g, const int32_t* seqs, const int32_t* lens,
     return launch_eval(g, seqs, lens, B, M, out_peak, out_dur, out_feasible, (cudaStream_t)stream);
 }
 
-// Host entry points.  The batch is cut into chunks of whole sequences; a copy stream owned by the
-// handle brings chunk k + 1 to the device while the caller's stream evaluates chunk k (one
-// cudaMemcpyAsync per chunk and an event between the two streams), and the three result arrays come
-// back with one copy into a pinned staging block, from which they are handed to the caller's arrays.
+// Host entry points.
+//
+// A large batch travels in three parts of 11/16, 4/16 and 1/16 of the ids on a copy stream owned by the handle, and the
+// caller's stream evaluates the sequences that have arrived in full while the next part is under way: the link is
+// busy throughout, every further part would cost it 4 us, and only the evaluation of the last sixteenth is exposed.  The
+// first part starts before the host has added up the lengths.  A batch whose copy is shorter than the calls
+// that would cut it goes in one piece on the caller's stream.
+//
+// Results go to pinned arrays of the caller straight from the device, behind the copies of later parts; to
+// pageable ones with one copy into a pinned block of the handle and a memcpy.  Short batches in pinned memory
+// are also fetched by a kernel: one launch instead of two copies and the widening.
+//
+// n = 442, B = 16384, ids as 16-bit words (17.4 MB, 318 us at the link's 54.8 GB/s; one copy alone
+// takes 327): 445 -> 406 us a call.  B = 8: 49 -> 24 us, B = 200: 59 -> 32.
 namespace {
-constexpr int kHostChunks = 4;
+constexpr int kHostChunks = 3;
+constexpr int kHostPart[kHostChunks] = {11, 4, 1};       // sixteenths
+constexpr int64_t kHostCutSteps = (int64_t)1 << 21;      // from here on in chunks (4 MB of 16-bit ids: 80 us of copy)
+constexpr int64_t kHostFetchBytes = 256 << 10;           // up to here fetched by a kernel (about 45 GB/s, no call per array)
+constexpr int32_t kHostDirect = 2048;                    // up to here sequences' results are written by the evaluation itself
 
 int host_streams(const moc_graph* g) {
     if (g->copy_stream) return MOC_OK;
@@ -1303,89 +1317,130 @@ int host_streams(const moc_graph* g) {
     return MOC_OK;
 }
 
+// Address under which kernels reach a host array, or nullptr for pageable memory.
+void* mapped_address(const void* host) {
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+}
+
 // ids: host array of `need` node ids, 4 bytes each (wide_ids) or 2 bytes each.
 int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_steps, const int32_t* lens, int32_t B,
               int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st, const char* who) {
-    // chunk boundaries: about equal numbers of steps, whole sequences
-    int64_t need = 0;
-    for (int32_t b = 0; b < B; ++b) need += lens[b] > 0 ? lens[b] : 0;
-    if (need > n_steps) return fail(MOC_ERR_ARG, "%s: lens sum to %lld > n_steps %lld", who, (long long)need, (long long)n_steps);
-    int32_t cb[kHostChunks + 1];
-    int64_t co[kHostChunks + 1];
-    int n_chunks = 0;
-    {
-        // Chunks of 1/2, 1/4, 1/8, 1/8 of the steps (whole sequences): the evaluation of all but the last
-        // chunk hides behind the copy of the next, and the last one is small.  Short batches go in one piece.
-        const int want = need >= (int64_t(1) << 21) ? kHostChunks : 1;
-        int64_t run = 0, bound = need - need / 2;
-        cb[0] = 0;
-        co[0] = 0;
-        for (int32_t b = 0; b < B; ++b) {
-            run += lens[b] > 0 ? lens[b] : 0;
-            if (n_chunks + 1 < want && run >= bound) {
-                ++n_chunks;
-                cb[n_chunks] = b + 1;
-                co[n_chunks] = run;
-                bound = run + (need - run + 1) / 2;
-            }
-        }
-        ++n_chunks;
-        cb[n_chunks] = B;
-        co[n_chunks] = need;
-    }
+    const size_t id_b = wide_ids ? 4 : 2, bB = (size_t)B;
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(MOC_ERR_CUDA, "cannot select device %d", g->device);
-    int rc = host_streams(g);
+    int rc = ensure((void**)&g->d_stage_seqs, &g->stage_seqs_cap, std::max<size_t>((size_t)n_steps * 4 + 16, 16));
     if (rc != MOC_OK) return rc;
-    rc = ensure((void**)&g->d_stage_seqs, &g->stage_seqs_cap, std::max<size_t>((size_t)need * 4 + 16, 16));
-    if (rc != MOC_OK) return rc;
-    if (!wide_ids) {
-        rc = ensure((void**)&g->d_stage_u16, &g->stage_u16_cap, std::max<size_t>((size_t)need * 2 + 16, 16));
-        if (rc != MOC_OK) return rc;
-    }
-    const size_t bB = (size_t)B, o_peak = 0, o_dur = bB * 8, o_st = 2 * bB * 8, o_lens = align16(o_st + bB * 4),
-                 res_bytes = o_st + bB * 4, io_bytes = o_lens + bB * 4;
+    const size_t o_peak = 0, o_dur = bB * 8, o_st = 2 * bB * 8, o_lens = align16(o_st + bB * 4), res_bytes = o_st + bB * 4, io_bytes = o_lens + bB * 4;
     rc = ensure((void**)&g->d_stage_io, &g->stage_io_cap, io_bytes);
     if (rc != MOC_OK) return rc;
-    if (res_bytes > g->h_stage_cap) {
+    int64_t* d_peak = (int64_t*)(g->d_stage_io + o_peak);
+    int64_t* d_dur = (int64_t*)(g->d_stage_io + o_dur);
+    int32_t* d_st = (int32_t*)(g->d_stage_io + o_st);
+    int32_t* d_lens = (int32_t*)(g->d_stage_io + o_lens);
+    // how the ids come: fetched by a kernel, copied in one piece, or in parts
+    const void* m_ids = nullptr;
+    const int32_t* m_lens = nullptr;
+    if (n_steps > 0 && n_steps * (int64_t)id_b <= kHostFetchBytes && (m_ids = mapped_address(ids)) != nullptr) m_lens = (const int32_t*)mapped_address(lens);
+    const bool parts = n_steps >= kHostCutSteps;
+    if (!m_lens && !wide_ids) {
+        rc = ensure((void**)&g->d_stage_u16, &g->stage_u16_cap, std::max<size_t>((size_t)n_steps * 2 + 16, 16));
+        if (rc != MOC_OK) return rc;
+    }
+    void* stage = wide_ids ? (void*)g->d_stage_seqs : (void*)g->d_stage_u16;
+    cudaStream_t cs = st;
+    int64_t at[kHostChunks + 1] = {0};         // ids on the device once part k has arrived
+    auto copy_part = [&](int k) -> int {       // part k of the ids, and the lengths behind the first
+        const int64_t cnt = at[k + 1] - at[k];
+        if (cnt) MOC_CUDA(cudaMemcpyAsync((char*)stage + at[k] * id_b, (const char*)ids + at[k] * id_b, (size_t)cnt * id_b, cudaMemcpyHostToDevice, cs));
+        if (k == 0) MOC_CUDA(cudaMemcpyAsync(d_lens, lens, bB * 4, cudaMemcpyHostToDevice, cs));
+        if (parts) MOC_CUDA(cudaEventRecord(g->chunk_ev[k], cs));
+        return MOC_OK;
+    };
+    const int n_parts = parts ? kHostChunks : 1;
+    for (int k = 0, sum = 0; k < n_parts; ++k) {
+        sum += parts ? kHostPart[k] : 16;
+        at[k + 1] = sum == 16 ? n_steps : n_steps / 16 * sum;
+    }
+    if (parts) {
+        rc = host_streams(g);
+        if (rc != MOC_OK) return rc;
+        cs = g->copy_stream;
+        // the copy stream starts once the caller's stream has reached this call
+        MOC_CUDA(cudaEventRecord(g->chunk_ev[kHostChunks], st));
+        MOC_CUDA(cudaStreamWaitEvent(cs, g->chunk_ev[kHostChunks], 0));
+    }
+    if (!m_lens)
+        for (int k = 0; k < n_parts; ++k) {
+            rc = copy_part(k);
+            if (rc != MOC_OK) return rc;
+        }
+    // sequences that are complete with each part, while the first is under way
+    int32_t cb[kHostChunks + 1] = {0};
+    int64_t co[kHostChunks + 1] = {0}, need = 0;
+    for (int32_t b = 0, k = 0; b < B; b += 64) {
+        const int32_t b1 = std::min<int32_t>(B, b + 64);
+        int64_t sum = 0;
+        for (int32_t i = b; i < b1; ++i) sum += std::max(lens[i], 0);
+        while (k + 1 < n_parts && need + sum > at[k + 1]) {       // this piece of 64 sequences reaches beyond part k
+            cb[++k] = b;
+            co[k] = need;
+        }
+        need += sum;
+        if (b1 == B)
+            for (++k; k <= n_parts; ++k) { cb[k] = B; co[k] = need; }
+    }
+    if (need > n_steps) {
+        if (!m_lens) cudaStreamSynchronize(cs);                   // the caller's arrays are still being read
+        return fail(MOC_ERR_ARG, "%s: lens sum to %lld > n_steps %lld", who, (long long)need, (long long)n_steps);
+    }
+    int64_t *m_peak = (int64_t*)mapped_address(out_peak), *m_dur = m_peak ? (int64_t*)mapped_address(out_dur) : nullptr;
+    int32_t* m_st = m_dur ? (int32_t*)mapped_address(out_feasible) : nullptr;
+    if (!m_st && res_bytes > g->h_stage_cap) {
         if (g->h_stage) MOC_CUDA(cudaFreeHost(g->h_stage));
         g->h_stage = nullptr;
         g->h_stage_cap = 0;
         MOC_CUDA(cudaMallocHost((void**)&g->h_stage, res_bytes * 2));
         g->h_stage_cap = res_bytes * 2;
     }
-    int64_t* d_peak = (int64_t*)(g->d_stage_io + o_peak);
-    int64_t* d_dur = (int64_t*)(g->d_stage_io + o_dur);
-    int32_t* d_st = (int32_t*)(g->d_stage_io + o_st);
-    int32_t* d_lens = (int32_t*)(g->d_stage_io + o_lens);
-    cudaStream_t cs = g->copy_stream;
-    // the copy stream starts once the caller's stream has reached this call
-    MOC_CUDA(cudaEventRecord(g->chunk_ev[kHostChunks], st));
-    MOC_CUDA(cudaStreamWaitEvent(cs, g->chunk_ev[kHostChunks], 0));
-    MOC_CUDA(cudaMemcpyAsync(d_lens, lens, bB * 4, cudaMemcpyHostToDevice, cs));
     int launches = 0;
-    for (int k = 0; k < n_chunks; ++k) {
-        const int64_t s0 = co[k], cnt = co[k + 1] - co[k];
-        if (cnt) {
-            if (wide_ids)
-                MOC_CUDA(cudaMemcpyAsync(g->d_stage_seqs + s0, (const int32_t*)ids + s0, (size_t)cnt * 4, cudaMemcpyHostToDevice, cs));
-            else
-                MOC_CUDA(cudaMemcpyAsync(g->d_stage_u16 + s0, (const uint16_t*)ids + s0, (size_t)cnt * 2, cudaMemcpyHostToDevice, cs));
-        }
-        MOC_CUDA(cudaEventRecord(g->chunk_ev[k], cs));
-        MOC_CUDA(cudaStreamWaitEvent(st, g->chunk_ev[k], 0));
-        if (cnt && !wide_ids) {
+    if (m_lens) {
+        const int blocks = (int)std::min<int64_t>((std::max<int64_t>(need / 4, B) + 255) / 256, (int64_t)g->sm_count * 2);
+        if (wide_ids) moc::fetch_kernel<int32_t><<<blocks, 256, 0, st>>>((const int32_t*)m_ids, need, g->d_stage_seqs, m_lens, B, d_lens);
+        else moc::fetch_kernel<uint16_t><<<blocks, 256, 0, st>>>((const uint16_t*)m_ids, need, g->d_stage_seqs, m_lens, B, d_lens);
+        MOC_CUDA(cudaGetLastError());
+        ++launches;
+    }
+    for (int k = 0; k < n_parts; ++k) {
+        if (parts) MOC_CUDA(cudaStreamWaitEvent(st, g->chunk_ev[k], 0));
+        const int64_t cnt = at[k + 1] - at[k];
+        if (!m_lens && !wide_ids && cnt) {
             const int blocks = (int)std::min<int64_t>((cnt / 8 + 255) / 256 + 1, (int64_t)g->sm_count * 8);
-            moc::widen_ids_kernel<<<blocks, 256, 0, st>>>(g->d_stage_u16 + s0, g->d_stage_seqs + s0, cnt);
+            moc::widen_ids_kernel<<<blocks, 256, 0, st>>>(g->d_stage_u16 + at[k], g->d_stage_seqs + at[k], cnt);
             ++launches;
         }
         const int32_t b0 = cb[k], nb = cb[k + 1] - cb[k];
-        if (nb > 0) {
-            rc = launch_eval(g, g->d_stage_seqs + s0, d_lens + b0, nb, M, d_peak + b0, d_dur + b0, d_st + b0, st);
-            if (rc != MOC_OK) return rc;
+        if (nb <= 0) continue;
+        const bool direct = m_st && nb <= kHostDirect;
+        rc = launch_eval(g, g->d_stage_seqs + co[k], d_lens + b0, nb, M, (direct ? m_peak : d_peak) + b0, (direct ? m_dur : d_dur) + b0,
+                         (direct ? m_st : d_st) + b0, st);
+        if (rc != MOC_OK) return rc;
+        if (m_st && !direct) {
+            moc::deliver_kernel<<<std::min((nb + 255) / 256, g->sm_count), 256, 0, st>>>(d_peak + b0, d_dur + b0, d_st + b0, nb, m_peak + b0,
+                                                                                       m_dur + b0, m_st + b0);
+            MOC_CUDA(cudaGetLastError());
+            ++launches;
         }
     }
     g_launches += launches;      // the evaluation launches were counted as they were enqueued
+    if (m_st) {
+        MOC_CUDA(cudaStreamSynchronize(st));
+        return MOC_OK;
+    }
     MOC_CUDA(cudaMemcpyAsync(g->h_stage, g->d_stage_io, res_bytes, cudaMemcpyDeviceToHost, st));
     MOC_CUDA(cudaStreamSynchronize(st));
     memcpy(out_peak, g->h_stage + o_peak, bB * 8);

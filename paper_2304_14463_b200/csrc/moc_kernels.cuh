@@ -410,4 +410,37 @@ static __global__ void __launch_bounds__(256) widen_ids_kernel(const uint16_t* _
     }
 }
 
+// Ids (widened) and lengths from pinned host memory to the device in one kernel: a batch of a few thousand steps is
+// here sooner than two copies can be started.
+template <typename Id>
+static __global__ void __launch_bounds__(256) fetch_kernel(const Id* __restrict__ ids, int64_t count, int32_t* __restrict__ dst,
+                                                    const int32_t* __restrict__ lens, int32_t B, int32_t* __restrict__ dst_lens) {
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = tid; i < B; i += stride) dst_lens[i] = __ldg(lens + i);
+    constexpr int kPer = 16 / (int)sizeof(Id);
+    const bool aligned = (reinterpret_cast<uintptr_t>(ids) & 15) == 0;
+    const int64_t nv = aligned ? count / kPer : 0;
+    for (int64_t i = tid; i < nv; i += stride) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(ids) + i);
+        if constexpr (sizeof(Id) == 4) {
+            reinterpret_cast<uint4*>(dst)[i] = v;
+        } else {
+            reinterpret_cast<uint4*>(dst)[2 * i] = make_uint4(v.x & 0xFFFFu, v.x >> 16, v.y & 0xFFFFu, v.y >> 16);
+            reinterpret_cast<uint4*>(dst)[2 * i + 1] = make_uint4(v.z & 0xFFFFu, v.z >> 16, v.w & 0xFFFFu, v.w >> 16);
+        }
+    }
+    for (int64_t i = nv * kPer + tid; i < count; i += stride) dst[i] = (int32_t)__ldg(ids + i);
+}
+
+// Results of a chunk to pinned arrays of the caller.
+static __global__ void __launch_bounds__(256) deliver_kernel(const int64_t* __restrict__ peak, const int64_t* __restrict__ dur,
+                                                      const int32_t* __restrict__ status, int32_t B, int64_t* __restrict__ out_peak,
+                                                      int64_t* __restrict__ out_dur, int32_t* __restrict__ out_status) {
+    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < B; i += gridDim.x * blockDim.x) {
+        out_peak[i] = peak[i];
+        out_dur[i] = dur[i];
+        out_status[i] = status[i];
+    }
+}
+
 }  // namespace moc

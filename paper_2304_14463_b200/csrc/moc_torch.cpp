@@ -25,6 +25,8 @@
 namespace {
 
 decltype(&moc_eval_batch) f_eval_batch;
+decltype(&moc_eval_batch_host) f_eval_batch_host;
+decltype(&moc_eval_batch_host16) f_eval_batch_host16;
 decltype(&moc_mem_profile) f_mem_profile;
 decltype(&moc_check_intervals) f_check_intervals_filled;   // writes the whole rows, -1 behind the sequences
 decltype(&moc_cache_build) f_cache_build;
@@ -152,6 +154,34 @@ PyObject* py_eval_batch(PyObject*, PyObject* const* a, Py_ssize_t na) {
         });
         if (rc != MOC_OK) return PyLong_FromLong(rc);
         return tuple_of(pk, du, st);
+    });
+}
+
+// eval_batch_host(g, seqs, lens, M, out_peak, out_dur, out_feasible, bits): CPU tensors; returns its outputs
+PyObject* py_eval_batch_host(PyObject*, PyObject* const* a, Py_ssize_t na) {
+    return guarded([&]() -> PyObject* {
+        void* g;
+        int64_t M, bits;
+        MOC_NONE_IF(na != 8 || !handle_of(a[0], &g) || !int_of(a[3], &M) || !int_of(a[7], &bits));
+        const at::ScalarType want[5] = {bits == 16 ? at::kUInt16 : at::kInt, at::kInt, at::kLong, at::kLong, at::kInt};
+        const int where[5] = {1, 2, 4, 5, 6};
+        const at::Tensor* t[5];
+        for (int k = 0; k < 5; ++k) {
+            MOC_NONE_IF(!THPVariable_Check(a[where[k]]));
+            t[k] = &THPVariable_Unpack(a[where[k]]);
+            MOC_NONE_IF(!t[k]->is_cpu() || t[k]->scalar_type() != want[k] || !t[k]->is_contiguous() || t[k]->dim() < 1);
+        }
+        const int64_t B = t[1]->size(0), n_steps = t[0]->size(0);
+        MOC_NONE_IF(B > INT32_MAX);
+        void* cs = stream();
+        const int rc = unlocked([&] {
+            return bits == 16 ? f_eval_batch_host16((const moc_graph*)g, ptr<uint16_t>(*t[0]), n_steps, ptr<int32_t>(*t[1]), (int32_t)B, M,
+                                                    ptr<int64_t>(*t[2]), ptr<int64_t>(*t[3]), ptr<int32_t>(*t[4]), cs)
+                              : f_eval_batch_host((const moc_graph*)g, ptr<int32_t>(*t[0]), n_steps, ptr<int32_t>(*t[1]), (int32_t)B, M,
+                                                  ptr<int64_t>(*t[2]), ptr<int64_t>(*t[3]), ptr<int32_t>(*t[4]), cs);
+        });
+        if (rc != MOC_OK) return PyLong_FromLong(rc);
+        return tuple_of(*t[2], *t[3], *t[4]);
     });
 }
 
@@ -309,6 +339,8 @@ PyObject* py_bind(PyObject*, PyObject* d) {
     f_##fn = (decltype(f_##fn))get("moc_" #fn);    \
     if (PyErr_Occurred()) return nullptr
     MOC_BIND(eval_batch);
+    MOC_BIND(eval_batch_host);
+    MOC_BIND(eval_batch_host16);
     MOC_BIND(mem_profile);
     MOC_BIND(check_intervals_filled);
     MOC_BIND(cache_build);
@@ -321,7 +353,7 @@ PyObject* py_bind(PyObject*, PyObject* d) {
 }
 
 #define MOC_FAST(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {MOC_FAST(eval_batch),      MOC_FAST(mem_profile), MOC_FAST(cache_build),  MOC_FAST(eval_edits),
+PyMethodDef methods[] = {MOC_FAST(eval_batch),      MOC_FAST(eval_batch_host), MOC_FAST(mem_profile), MOC_FAST(cache_build),  MOC_FAST(eval_edits),
                          MOC_FAST(check_intervals), MOC_FAST(search_run),  MOC_FAST(search_state), {"bind", py_bind, METH_O, nullptr},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_moc_torch", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
