@@ -98,12 +98,13 @@ LaneFn lane_fn_lg(int lg, int kp) {
 LaneFn lane_fn(bool wide, int lg, int kp) { return wide ? lane_fn_lg<int64_t>(lg, kp) : lane_fn_lg<int32_t>(lg, kp); }
 
 template <typename MemT, bool kTiles>
-QuadFn quad_fn_c(int C) {
-    return C <= 3 ? (QuadFn)moc::eval_quad_kernel<MemT, 3, kTiles> : (QuadFn)moc::eval_quad_kernel<MemT, 4, kTiles>;
+QuadFn quad_fn_c(int C, bool profile) {
+    if (profile) return C <= 3 ? (QuadFn)moc::eval_quad_kernel<MemT, 3, kTiles, true> : (QuadFn)moc::eval_quad_kernel<MemT, 4, kTiles, true>;
+    return C <= 3 ? (QuadFn)moc::eval_quad_kernel<MemT, 3, kTiles, false> : (QuadFn)moc::eval_quad_kernel<MemT, 4, kTiles, false>;
 }
-QuadFn quad_fn(bool wide, int C, bool tiles) {
-    if (tiles) return wide ? quad_fn_c<int64_t, true>(C) : quad_fn_c<int32_t, true>(C);
-    return wide ? quad_fn_c<int64_t, false>(C) : quad_fn_c<int32_t, false>(C);
+QuadFn quad_fn(bool wide, int C, bool tiles, bool profile) {
+    if (tiles) return wide ? quad_fn_c<int64_t, true>(C, profile) : quad_fn_c<int32_t, true>(C, profile);
+    return wide ? quad_fn_c<int64_t, false>(C, profile) : quad_fn_c<int32_t, false>(C, profile);
 }
 
 template <typename SumT, int W>
@@ -191,7 +192,7 @@ const char* plan_lane(const moc_graph* g, size_t smem_cap, Plan* out) {
 }
 
 // Plan of the block-per-sequence path with packed words (C <= 4).  Returns nullptr on success.
-const char* plan_quad(const moc_graph* g, size_t smem_cap, Plan* out) {
+const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, Plan* out) {
     Plan pl = *out;
     const int64_t n = g->n, C = g->C, t_max = C * n;
     if (C > 4) return "C > 4";
@@ -202,9 +203,9 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, Plan* out) {
     const size_t word_b = 2 * align16(4 * (size_t)(n + 2)) + 16, cnt_b = align16(2 * (size_t)(n + 2)), delta_b = align16(msz * (size_t)(t_max + 4));
     const size_t sm = word_b + cnt_b + delta_b;
     if (sm > smem_cap) return "the state of a sequence exceeds shared memory";
-    QuadFn fn = quad_fn(pl.wide, (int)C, g->d_rec32 != nullptr);
+    QuadFn fn = quad_fn(pl.wide, (int)C, g->d_rec32 != nullptr, profile);
     if (raise_smem_limit((const void*)fn, g->smem_optin) != cudaSuccess) { cudaGetLastError(); return "cudaFuncSetAttribute failed"; }
-    const int forced = g->want_kind == MOC_KERNEL_BLOCK ? g->want_a : 0;
+    const int forced = !profile && g->want_kind == MOC_KERNEL_BLOCK ? g->want_a : 0;
     bool any = false;
     for (int k = 0; k < 5; ++k) {
         const int thr = forced ? forced : 64 << k;
@@ -269,6 +270,10 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     const int kind = profile ? MOC_KERNEL_GROUP : g->want_kind;
     const bool shape_given = g->want_G != 0 || g->want_gpc != 0;       // moc_graph_set_launch
     if (kind == MOC_KERNEL_AUTO && !shape_given && !profile) plan_live(g, &pl);
+    if (profile && !plan_quad(g, smem_cap, true, &pl)) {
+        *out = pl;
+        return MOC_OK;
+    }
     // Order of preference when nothing is forced: warp per sequence, then sequence per lane (it also
     // serves graphs whose degrees are too uneven for the warp kernel's padded successor tiles), then
     // the thread-group kernel, which serves everything.
@@ -282,7 +287,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         if (kind == MOC_KERNEL_LANE) return fail(MOC_ERR_ARG, "the sequence-per-lane kernel cannot serve this graph: %s", why);
     }
     if (kind == MOC_KERNEL_BLOCK || (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C >= 3)) {
-        const char* why = plan_quad(g, smem_cap, &pl);
+        const char* why = plan_quad(g, smem_cap, profile, &pl);
         if (!why) {
             *out = pl;
             return MOC_OK;
@@ -336,7 +341,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     }
     // sequences too long for eight warps of the warp-per-sequence kernel on an SM (n = 2000, B = 2000: 69.6 us with a
     // thread group per sequence, 53.5 with the block-per-sequence kernel)
-    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, &pl)) {
+    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, profile, &pl)) {
         *out = pl;
         return MOC_OK;
     }
@@ -551,6 +556,27 @@ moc::EvalParams base_params(const moc_graph* g, const Plan& pl) {
     return p;
 }
 
+moc::QuadParams quad_params(const moc_graph* g, const Plan& pl) {
+    moc::QuadParams q{};
+    q.n = g->n;
+    q.C = g->C;
+    q.max_T = g->C * g->n;
+    q.n_tiles = g->n_tiles;
+    q.split = g->split;
+    q.rec = pl.wide ? g->d_rec64 : g->d_rec32;
+    q.sell = g->d_sell;
+    q.tile_row = g->d_tile_row;
+    q.order = g->d_order;
+    q.succ = g->d_succ16;
+    q.base_dur = g->sum_w;
+    q.m = pl.wide ? (const void*)g->d_m64 : (const void*)g->d_m32;
+    q.w = g->d_w;
+    q.cap = g->d_cap;
+    q.word_bytes = pl.quad_word_b;
+    q.cnt_bytes = pl.quad_cnt_b;
+    return q;
+}
+
 // Batches the backward walk serves.  Its time hardly depends on the batch until every SM has 16 warps: about
 // 6 us + 0.17 us per node (a lane's steps follow one another), while the warp-per-sequence kernel takes 1.2 us per
 // 1000 sequences of these sizes (2 us with 64-bit sums; the block-per-sequence kernel with C >= 3 likewise).
@@ -657,31 +683,15 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     if (pl.quad) {
-        moc::QuadParams q{};
-        q.n = g->n;
-        q.C = g->C;
-        q.max_T = g->C * g->n;
+        moc::QuadParams q = quad_params(g, pl);
         q.B = B;
         q.M = M;
-        q.n_tiles = g->n_tiles;
-        q.split = g->split;
-        q.rec = pl.wide ? g->d_rec64 : g->d_rec32;
-        q.sell = g->d_sell;
-        q.tile_row = g->d_tile_row;
-        q.order = g->d_order;
-        q.succ = g->d_succ16;
-        q.base_dur = g->sum_w;
-        q.m = pl.wide ? (const void*)g->d_m64 : (const void*)g->d_m32;
-        q.w = g->d_w;
-        q.cap = g->d_cap;
         q.seqs = seqs;
         q.lens = lens;
         q.offs = offs;
         q.out_peak = out_peak;
         q.out_dur = out_dur;
         q.out_status = out_feasible;
-        q.word_bytes = pl.quad_word_b;
-        q.cnt_bytes = pl.quad_cnt_b;
         MOC_CUDA(cudaLaunchKernelEx(&cfg, pl.quad_fn, q));
     } else if (pl.lane) {
         const LaneLayout& L = g->lane[5 - pl.lane_lg];
@@ -770,7 +780,7 @@ int ensure_plans(const moc_graph* g) {
     if (rc == MOC_OK && g->plan_eval.pair && g->want_kind == MOC_KERNEL_AUTO) {
         Plan pl;
         pl.wide = g->plan_eval.wide;
-        if (!plan_quad(g, g->smem_optin > 1024 ? g->smem_optin - 1024 : 0, &pl)) g->plan_block = pl;
+        if (!plan_quad(g, g->smem_optin > 1024 ? g->smem_optin - 1024 : 0, false, &pl)) g->plan_block = pl;
     }
     return rc;
 }
@@ -1543,6 +1553,23 @@ int moc_mem_profile(const moc_graph* g, const int32_t* seq, int32_t len, int64_t
         if (rc != MOC_OK) return rc;
     }
     const Plan& pl = g->plan_profile;
+    if (pl.quad) {
+        moc::QuadParams q = quad_params(g, pl);
+        q.B = 1;
+        q.M = INT64_MAX;
+        q.seqs = seq;
+        q.single_len = len;
+        q.out_status = out_status;
+        q.out_profile = out_profile;
+        q.out_free = out_free;
+        // threads from measurements at n = 20, 100, 442, 1000, 2000 and 5000 (us per call with 128 / 512 / 1024 threads:
+        // 6.1 / 6.2 / 10.6, 6.1 / 6.9 / 8.6, 8.2 / 7.4 / 8.2, 12.3 / 8.3 / 8.2, 17.0 / 10.3 / 10.3, 32.8 / 18.0 / 16.4)
+        const int thr = g->n < 200 ? 128 : (g->n < 1500 ? 512 : 1024);
+        pl.quad_fn<<<1, thr, pl.smem, st>>>(q);
+        ++g_launches;
+        MOC_CUDA(cudaGetLastError());
+        return MOC_OK;
+    }
     if (pl.global_state) {
         int rc = ensure((void**)&g->d_state, &g->state_cap, (size_t)pl.group_bytes);
         if (rc != MOC_OK) return rc;

@@ -66,6 +66,9 @@ struct QuadParams {
     int64_t* out_peak;
     int64_t* out_dur;
     int32_t* out_status;
+    int32_t single_len;        // profile: length of the one sequence at seqs[0..)
+    int64_t* out_profile;      // ... usage per step, free step per step (may be null)
+    int32_t* out_free;
     uint32_t word_bytes;       // 8 (n + 2) rounded to 32, and 16 for the word of empty node slots
     uint32_t cnt_bytes;        // 2 (n + 2), rounded to 16
 };
@@ -134,20 +137,27 @@ struct QuadNode {
             G[j] = __viaddmax_u16x2(r.y, na[j], G[j]);
         }
     }
-    // -m behind the end of every copy; returns a word whose bit 15 tells of a successor copy before a_1
-    template <typename MemT, int kShift>
-    __device__ __forceinline__ uint32_t close(uint32_t da, Amount<MemT> m) {
-        const uint32_t g0 = max_halves(G[0]);
-        red_sub_amount(da + (((base[0] + g0) & 0xFFFFu) << kShift), m);
+    // -m behind the end of every copy (and the ends themselves to `ends`, for a profile); returns a word whose bit 15
+    // tells of a successor copy before a_1
+    template <typename MemT, int kShift, bool kEnds>
+    __device__ __forceinline__ uint32_t close(uint32_t da, Amount<MemT> m, int32_t* ends, bool real) {
+        const uint32_t g0 = max_halves(G[0]), last = (base[0] + g0) & 0xFFFFu;
+        red_sub_amount(da + (last << kShift), m);
+        if (kEnds && real && !(g0 & 0x8000u)) ends[base[kAcc - 1] - 1] = (int32_t)last - 1;
 #pragma unroll
         for (int j = 1; j < kAcc; ++j)
-            if (base[j] != base[j - 1]) red_sub_amount(da + (((base[j] + max_halves(G[j])) & 0xFFFFu) << kShift), m);   // copy j exists apart from copy j + 1
+            if (base[j] != base[j - 1]) {                                       // copy j exists apart from copy j + 1
+                const uint32_t end = (base[j] + max_halves(G[j])) & 0xFFFFu;
+                red_sub_amount(da + (end << kShift), m);
+                if (kEnds && real) ends[base[j - 1] - 1] = (int32_t)end - 1;
+            }
         return g0;
     }
 };
 
 // kAcc: number of copies the node pass keeps apart (3 or 4).
-template <typename MemT, int kAcc, bool kTiles>
+// kProfile: one sequence, whose usage per step and free steps are written out (moc_mem_profile).
+template <typename MemT, int kAcc, bool kTiles, bool kProfile>
 __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
     extern __shared__ __align__(16) char smem[];
     __shared__ int64_t s_dur[32];
@@ -179,7 +189,7 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
     };
 
     // ---- rows: block c takes [c * B / grid, (c + 1) * B / grid), or every grid-th one with the offsets given
-    const bool self = p.offs == nullptr;
+    const bool self = !kProfile && p.offs == nullptr;
     int b = blockIdx.x, b_end = p.B, b_step = gridDim.x;
     int64_t off = 0;
     if (self) {
@@ -203,8 +213,8 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
         for (int k = 0; k < n_warps; ++k) off += s_dur[k];
     }
     for (; b < b_end; b += b_step) {
-        const int32_t T = __ldg(p.lens + b);
-        if (!self) off = __ldg(p.offs + b);
+        const int32_t T = kProfile ? p.single_len : __ldg(p.lens + b);
+        if (!self && !kProfile) off = __ldg(p.offs + b);
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
         if (T >= n && T <= p.max_T) {      // uniform over the block
@@ -303,7 +313,7 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                     for (int d = warp; d < p.n_tiles; d += n_warps) {
                         QuadNode<kAcc> u[2];
                         Amount<MemT> m[2];
-                        const uint32_t x0 = r_next[0].x;
+                        const uint32_t x0 = r_next[0].x, x1 = r_next[1].x;
                         const uint32_t* ps = ps_next;
                         uint32_t e_next = e_first;
 #pragma unroll
@@ -326,8 +336,10 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                             u[0].visit(r0);
                             u[1].visit(r1);
                         }
-                        depw |= u[0].template close<MemT, kShift>(da, m[0]);
-                        depw |= u[1].template close<MemT, kShift>(da, m[1]);
+                        // an empty node slot owns the last word of the area: no step is its own
+                        const bool real0 = !kProfile || (x0 & 0xFFFFu) << 1 != p.word_bytes - 16u, real1 = !kProfile || (x1 & 0xFFFFu) << 1 != p.word_bytes - 16u;
+                        depw |= u[0].template close<MemT, kShift, kProfile>(da, m[0], p.out_free, real0 && p.out_free != nullptr);
+                        depw |= u[1].template close<MemT, kShift, kProfile>(da, m[1], p.out_free, real1 && p.out_free != nullptr);
                     }
                 } else {
                     const int n_round = (n + 31) & ~31;
@@ -353,7 +365,7 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                         }
                         for (int k = 8; k < rounds; ++k)
                             if ((uint32_t)k < deg) u.visit(lds_v2(wa + ((uint32_t)__ldg(p.succ + e8 + (k - 8)) << 3)));
-                        if (i < n) depw |= u.template close<MemT, kShift>(da, amount((int)node));
+                        if (i < n) depw |= u.template close<MemT, kShift, kProfile>(da, amount((int)node), p.out_free, p.out_free != nullptr);
                     }
                 }
                 if (__any_sync(kFull, (depw & 0x8000u) != 0) && lane == 0) atomicOr(&s_flags, 2u);
@@ -402,6 +414,22 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 if constexpr (sizeof(MemT) == 4) before = (MemT)lo_in;
                 else before = split_value(lo_in, hi_in, p.split);
                 MemT peak = tb < te ? before + top : MemT(0);
+                if constexpr (kProfile) {
+                    ad = da + ((uint32_t)tb << kShift);
+                    lo = lo_in;
+                    hi = hi_in;
+                    for (int t = tb; t < te; ++t, ad += (uint32_t)sizeof(MemT)) {
+                        if constexpr (sizeof(MemT) == 4) {
+                            lo += lds_u32(ad);
+                            p.out_profile[t] = (int64_t)(MemT)lo;
+                        } else {
+                            const uint2 q = lds_v2(ad);
+                            lo += q.x;
+                            hi += q.y;
+                            p.out_profile[t] = split_value(lo, hi, p.split);
+                        }
+                    }
+                }
                 peak = warp_max_t(peak);
                 if (lane == 0) s_top[warp] = (int64_t)peak;
                 __syncthreads();
@@ -411,6 +439,19 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                     out_st = out_pk <= p.M ? 1 : 0;
                 }
             }
+        }
+        if constexpr (kProfile) {
+            if (tid == 0) s_flags = (uint32_t)out_st;      // only thread 0 knows 0 or 1; nothing reads the flags any more
+            __syncthreads();
+            const int32_t st = (int32_t)s_flags;
+            if (tid == 0) p.out_status[0] = st;
+            if (st < 0) {
+                for (int t = tid; t < T; t += nthr) {
+                    p.out_profile[t] = -1;
+                    if (p.out_free) p.out_free[t] = -1;
+                }
+            }
+            return;
         }
         if (tid == 0) {
             p.out_peak[b] = out_pk;
