@@ -187,17 +187,17 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
     extern __shared__ __align__(16) char smem[];
     __shared__ int64_t s_part[16];
     constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u;
-    // ---- graph -> shared memory, once per block: records | durations | successor tiles
+    // ---- graph -> shared memory, once per block: records | durations | successor tiles.  Asynchronous copies: they
+    // complete behind the search for the rows (a launch of few sequences is a chain of such latencies).
     const uint32_t graph_bytes = p.rec_bytes + p.w_bytes + p.sell_bytes;
     {
-        int4* s4 = reinterpret_cast<int4*>(smem);
-        const uint32_t n_rec = p.rec_bytes >> 4, n_w = p.w_bytes >> 4, n_all = (p.rec_bytes + p.w_bytes + p.sell_bytes) >> 4;
+        const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
+        const uint32_t n_rec = p.rec_bytes >> 4, n_w = p.w_bytes >> 4, n_all = graph_bytes >> 4;
         for (uint32_t i = threadIdx.x; i < n_all; i += blockDim.x) {
-            int4 v;
-            if (i < n_rec) v = __ldg(reinterpret_cast<const int4*>(p.rec) + i);
-            else if (i < n_rec + n_w) v = __ldg(reinterpret_cast<const int4*>(p.wslot) + (i - n_rec));
-            else v = __ldg(reinterpret_cast<const int4*>(p.sell) + (i - n_rec - n_w));
-            s4[i] = v;
+            const void* src = i < n_rec ? (const void*)(reinterpret_cast<const int4*>(p.rec) + i)
+                                        : i < n_rec + n_w ? (const void*)(reinterpret_cast<const int4*>(p.wslot) + (i - n_rec))
+                                                          : (const void*)(reinterpret_cast<const int4*>(p.sell) + (i - n_rec - n_w));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s0 + 16u * i), "l"(src) : "memory");
         }
     }
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
@@ -222,7 +222,6 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
     MOC_KEEP(sell0);
     MOC_KEEP(n_tiles);
     if (lane == 0) *reinterpret_cast<uint32_t*>(ws + p.word_bytes) = 0x00010001u;   // owned by empty node slots
-    __syncthreads();
 
     const int n = p.n;
     const int n_warps = gridDim.x * wpb;
@@ -254,6 +253,10 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
         b_end = (int)(((int64_t)blockIdx.x + 1) * p.B / gridDim.x);
         b_step = wpb;
         int64_t sum = 0;
+        b = c0 + warp;
+        // lengths of the first wpb sequences of the range (this warp starts at the warp-th of them), and of those from b on
+        const int32_t len_c0 = (c0 + lane < p.B) ? __ldg(p.lens + c0 + lane) : 0;
+        len_raw = (b + lane < p.B) ? __ldg(p.lens + b + lane) : 0;
         if ((reinterpret_cast<uintptr_t>(p.lens) & 15) == 0) {
             const int4* l4 = reinterpret_cast<const int4*>(p.lens);
             for (int i = threadIdx.x; i < (c0 >> 2); i += blockDim.x) {
@@ -268,14 +271,11 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
         if (lane == 0) s_part[warp] = sum;
         __syncthreads();
         for (int k = 0; k < wpb; ++k) off += s_part[k];
-        // lengths of the first wpb sequences of the range; this warp starts at the warp-th of them
-        len_raw = (c0 + lane < p.B) ? __ldg(p.lens + c0 + lane) : 0;
-        off += group_sum(len_raw, warp);
-        b = c0 + warp;
-        // shift so that lane k holds the length of sequence b + k
-        len_raw = (b + lane < p.B) ? __ldg(p.lens + b + lane) : 0;
+        off += group_sum(len_c0, warp);
         T = __shfl_sync(0xFFFFFFFFu, len_raw, 0);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();                        // the graph is there
     // The first kPre 16-byte vectors per lane of the NEXT row are loaded into registers while the
     // current sequence is still being worked on, so that stage 1 does not wait for HBM.
     int4 pre[kPre > 0 ? kPre : 1];

@@ -190,10 +190,10 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
 
     // ---- rows: block c takes [c * B / grid, (c + 1) * B / grid), or every grid-th one with the offsets given
     const bool self = !kProfile && p.offs == nullptr;
-    int b = blockIdx.x, b_end = p.B, b_step = gridDim.x;
+    int b = self ? (int)((int64_t)blockIdx.x * p.B / gridDim.x) : (int)blockIdx.x, b_end = p.B, b_step = gridDim.x;
     int64_t off = 0;
+    int32_t T_next = kProfile ? p.single_len : (b < p.B ? __ldg(p.lens + b) : 0);      // one sequence ahead
     if (self) {
-        b = (int)((int64_t)blockIdx.x * p.B / gridDim.x);
         b_end = (int)(((int64_t)blockIdx.x + 1) * p.B / gridDim.x);
         b_step = 1;
         int64_t sum = 0;
@@ -213,7 +213,8 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
         for (int k = 0; k < n_warps; ++k) off += s_dur[k];
     }
     for (; b < b_end; b += b_step) {
-        const int32_t T = kProfile ? p.single_len : __ldg(p.lens + b);
+        const int32_t T = T_next;
+        if (!kProfile && b + b_step < b_end) T_next = __ldg(p.lens + b + b_step);
         if (!self && !kProfile) off = __ldg(p.offs + b);
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
@@ -227,6 +228,7 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 if (tid == 0) s_flags = 0;
             }
             __syncthreads();
+            Amount<MemT> m_next = amount(min(tid, n - 1));          // for stage 1b, one round ahead
             // ---- stage 1a
             uint32_t flags = 0;    // bit 0: malformed, bit 1: precedence violated
             {
@@ -256,9 +258,27 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 }
             }
             __syncthreads();
+            // records and first successor row of a tile are requested while the tile before it (or stage 1b) is worked on
+            uint4 r_next[2];
+            const uint32_t* ps_next = nullptr;
+            uint32_t e_first = 0;
+            auto request = [&](int d) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if constexpr (sizeof(MemT) == 4) {
+                        const uint2 r = __ldg(reinterpret_cast<const uint2*>(p.rec) + (2 * d + h) * 32 + lane);
+                        r_next[h].x = r.x;
+                        r_next[h].z = r.y;
+                    } else {
+                        r_next[h] = __ldg(reinterpret_cast<const uint4*>(p.rec) + (2 * d + h) * 32 + lane);
+                    }
+                }
+                ps_next = p.sell + 32 * __ldg(p.tile_row + d) + lane;
+                e_first = __ldg(ps_next);
+            };
+            if (kTiles && warp < p.n_tiles) request(warp);
             // ---- stage 1b
             int64_t dur = 0;
-            Amount<MemT> m_next = amount(min(tid, n - 1));          // one round ahead
             for (int v = tid; v < n; v += nthr) {
                 uint32_t c, limit = (uint32_t)p.C;
                 asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(c) : "r"(ca + 2u * (uint32_t)v) : "memory");
@@ -291,25 +311,6 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 // ---- stage 2 and the scatter of stage 3
                 uint32_t depw = 0;
                 if constexpr (kTiles) {
-                    // records and first successor row of a tile are requested while the tile before it is worked on
-                    uint4 r_next[2];
-                    const uint32_t* ps_next = nullptr;
-                    uint32_t e_first = 0;
-                    auto request = [&](int d) {
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if constexpr (sizeof(MemT) == 4) {
-                                const uint2 r = __ldg(reinterpret_cast<const uint2*>(p.rec) + (2 * d + h) * 32 + lane);
-                                r_next[h].x = r.x;
-                                r_next[h].z = r.y;
-                            } else {
-                                r_next[h] = __ldg(reinterpret_cast<const uint4*>(p.rec) + (2 * d + h) * 32 + lane);
-                            }
-                        }
-                        ps_next = p.sell + 32 * __ldg(p.tile_row + d) + lane;
-                        e_first = __ldg(ps_next);
-                    };
-                    if (warp < p.n_tiles) request(warp);
                     for (int d = warp; d < p.n_tiles; d += n_warps) {
                         QuadNode<kAcc> u[2];
                         Amount<MemT> m[2];
