@@ -733,6 +733,7 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         q.rec_bytes = pl.rec_bytes; q.w_bytes = pl.w_bytes; q.sell_bytes = pl.sell_bytes;
         q.word_bytes = pl.word_bytes; q.delta_bytes = pl.delta_bytes;
         q.split = g->split;
+        q.small_w = g->sum_w < ((int64_t)1 << 32) ? 1 : 0;
         MOC_CUDA(cudaLaunchKernelEx(&cfg, pl.pair_fn, q));
     } else {
         moc::EvalParams p = base_params(g, pl);

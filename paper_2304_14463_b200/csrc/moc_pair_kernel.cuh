@@ -52,6 +52,7 @@ struct PairParams {
     const uint64_t* wslot;     // 64 * n_tiles, same slots: w | 1 << 48 | (C_v == 1) << 63
     const uint32_t* sell;      // successor tiles: byte offsets of the successor words of a lane's two nodes, 16 bits each
     int64_t base_dur;          // sum of all w
+    int32_t small_w;           // sum of all w below 2^32
     const int32_t* seqs;
     const int32_t* lens;
     const int64_t* offs;       // exclusive prefix sum of the lengths, or nullptr: the kernel finds the rows itself
@@ -289,6 +290,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
             if (b_next < b_end) { off_next = __ldg(&p.offs[b_next]); T_next = __ldg(&p.lens[b_next]); }
         } else {
             if (b_next < b_end) len_next = (b_next + lane < p.B) ? __ldg(p.lens + b_next + lane) : 0;
+            off_next = off + group_sum(len_raw, wpb);   // skip the wpb sequences b .. b+wpb-1
         }
 
         const bool use_pre = have_pre;   // pre[] holds this row only if the previous iteration fetched it
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
 
             // request the next row now: the loads complete behind stages 2-4
             if (kPre > 0 && b_next < b_end) {
-                const int64_t off_n = self ? off + group_sum(len_raw, wpb) : off_next;
+                const int64_t off_n = off_next;
                 const int32_t T_n = self ? __shfl_sync(0xFFFFFFFFu, len_next, 0) : T_next;
                 if (T_n >= n && T_n <= p.max_T) {
                     const int32_t* nrow = p.seqs + off_n;
@@ -380,7 +382,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
 
             if (kPre == 0 && b_next < b_end) {
                 // short rows are read in place; ask for the next one to be brought into L2 meanwhile
-                const int64_t off_n = self ? off + group_sum(len_raw, wpb) : off_next;
+                const int64_t off_n = off_next;
                 const int32_t T_n = self ? __shfl_sync(0xFFFFFFFFu, len_next, 0) : T_next;
                 if (T_n >= n && T_n <= p.max_T) {
                     const char* nrow = reinterpret_cast<const char*>(p.seqs + off_n);
@@ -456,7 +458,9 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                 }
             }
             vmin = __reduce_min_sync(0xFFFFFFFFu, vmin);
-            const uint64_t acc_all = (uint64_t)warp_sum64((int64_t)acc);
+            // the low words add up without a carry when all durations together fit 32 bits
+            const uint64_t acc_all = p.small_w ? (uint64_t)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)(acc >> 32)) << 32 | __reduce_add_sync(0xFFFFFFFFu, (uint32_t)acc)
+                                               : (uint64_t)warp_sum64((int64_t)acc);
             const bool cap_ok = !__any_sync(0xFFFFFFFFu, (int32_t)capw < 0);
             const bool well_formed = cap_ok && vmin != 0 && (int)((acc_all >> kPairCntShift) & 0x7FFFu) == T - n;
             const bool dep = __any_sync(0xFFFFFFFFu, (depw & 0x80008000u) != 0);
@@ -517,7 +521,6 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
             p.out_status[b] = out_st;
         }
         if (self) {
-            off_next = off + group_sum(len_raw, wpb);   // skip the wpb sequences b .. b+wpb-1
             len_raw = len_next;
             T_next = __shfl_sync(0xFFFFFFFFu, len_next, 0);
         }
