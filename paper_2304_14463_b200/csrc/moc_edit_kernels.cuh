@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                         Ga[h] = mx - mn;
                         Gb[h] = 0x00010000u - Ga[h];
                     }
-                    rows = __shfl_sync(kFull, rows, 0);
+
                     uint32_t e_next = rows > 0 ? ld32(ps) : 0u;            // one row ahead
                     for (int k = 0; k < rows; ++k, ps += 32) {
                         const uint32_t e = e_next;

@@ -226,6 +226,12 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
 
     const int n = p.n;
     const int n_warps = gridDim.x * wpb;
+    auto clear_deltas = [&]() {             // all of them, with the front pad: after a sequence that was not scanned
+        int4* d4 = reinterpret_cast<int4*>(delta_base);
+        for (int i = lane; i < (int)(p.delta_bytes >> 4); i += 32) d4[i] = make_int4(0, 0, 0, 0);
+        __syncwarp();
+    };
+    clear_deltas();
     constexpr int kPerVec = 16 / (int)sizeof(MemT);  // delta entries per 16-byte vector
     constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
 
@@ -260,9 +266,12 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
         len_raw = (b + lane < p.B) ? __ldg(p.lens + b + lane) : 0;
         if ((reinterpret_cast<uintptr_t>(p.lens) & 15) == 0) {
             const int4* l4 = reinterpret_cast<const int4*>(p.lens);
-            for (int i = threadIdx.x; i < (c0 >> 2); i += blockDim.x) {
-                const int4 q = __ldg(l4 + i);
-                sum += (int64_t)max(q.x, 0) + max(q.y, 0) + max(q.z, 0) + max(q.w, 0);
+            for (int i = threadIdx.x; i < (c0 >> 2); i += 8 * blockDim.x) {       // eight loads in flight
+                int4 q[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) q[k] = i + k * (int)blockDim.x < (c0 >> 2) ? __ldg(l4 + i + k * blockDim.x) : make_int4(0, 0, 0, 0);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) sum += (int64_t)max(q[k].x, 0) + max(q[k].y, 0) + max(q[k].z, 0) + max(q[k].w, 0);
             }
             for (int i = (c0 & ~3) + threadIdx.x; i < c0; i += blockDim.x) sum += max(__ldg(p.lens + i), 0);
         } else {
@@ -298,16 +307,13 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
         if (T >= n && T <= p.max_T) {
-            // ---- clear: words, and the deltas the scan will read (whole vectors per lane)
+            // ---- clear the words (the deltas are zero: the scan clears behind itself)
             const int nvec_d = (T + 2 + kPerVec - 1) / kPerVec;        // vectors covering delta[0..T+1]
             const int V = ((nvec_d + 31) >> 5) | 1;                      // vectors per lane, odd
             {
                 const int4 z = make_int4(0, 0, 0, 0);
                 int4* w4 = reinterpret_cast<int4*>(word);
                 for (int i = lane; i < (int)(p.word_bytes >> 4); i += 32) w4[i] = z;
-                int4* d4 = reinterpret_cast<int4*>(delta_base);
-                const int nd4 = 32 * V + 1;                              // front pad + 32*V vectors
-                for (int i = lane; i < nd4; i += 32) d4[i] = z;
             }
             __syncwarp();
             if (lane == 0) word[n + 1] = (uint32_t)T * 0x10001u;   // the made-up successor of sinks
@@ -425,8 +431,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                         Ga[h] = mx - mn;                       // (b - a, b - a)
                         Gb[h] = 0x00010000u - Ga[h];           // (a - b, a - b) mod 2^16 when a < b
                     }
-                    // successors of the tile: uniform trip count, used-up lists read the node's own word
-                    rows = __shfl_sync(0xFFFFFFFFu, rows, 0);
+                    // successors of the tile: the same trip count in every lane, used-up lists read the node's own word
 #pragma unroll 2
                     for (int k = 0; k < rows; ++k) {
                         const uint32_t e = lds_u32(ps);
@@ -466,6 +471,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
             const bool dep = __any_sync(0xFFFFFFFFu, (depw & 0x80008000u) != 0);
             const int64_t dur_extra = (int64_t)(acc_all & kPairDurMask);
             __syncwarp();
+            if (!well_formed || dep) clear_deltas();
 
             if (!well_formed) {
                 // status -2, sentinels already set
@@ -476,12 +482,14 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                 // ---- stage 3 + 4: prefix sum and running maximum; lane owns V consecutive vectors
                 // One pass: the lane's running prefix and the largest prefix it sees; the largest
                 // usage inside the lane's chunk is then (sum of the chunks before it) + that maximum.
-                const int4* d4 = reinterpret_cast<const int4*>(delta_base + kPairDeltaFront) + lane * V;
+                int4* d4 = reinterpret_cast<int4*>(delta_base + kPairDeltaFront) + lane * V;
+                const int4 z = make_int4(0, 0, 0, 0);
                 MemT peak;
                 if constexpr (sizeof(MemT) == 4) {
                     MemT run = 0, top;
                     {
                         const int4 q = d4[0];
+                        d4[0] = z;
                         run = q.x; top = run;
                         run += q.y; top = max(top, run);
                         run += q.z; top = max(top, run);
@@ -489,6 +497,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                     }
                     for (int j = 1; j < V; ++j) {
                         const int4 q = d4[j];
+                        d4[j] = z;
                         run += q.x; top = max(top, run);
                         run += q.y; top = max(top, run);
                         run += q.z; top = max(top, run);
@@ -500,6 +509,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                     int64_t top = INT64_MIN;
                     for (int j = 0; j < V; ++j) {
                         const int4 q = d4[j];
+                        d4[j] = z;
                         lo += (uint32_t)q.x; hi += (uint32_t)q.y;
                         const int64_t u = split_value(lo, hi, p.split);
                         lo += (uint32_t)q.z; hi += (uint32_t)q.w;

@@ -108,7 +108,7 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
             Ga[h] = mx - mn;
             Gb[h] = 0x00010000u - Ga[h];
         }
-        rows = __shfl_sync(kFull, rows, 0);
+
 #pragma unroll 2
         for (int k = 0; k < rows; ++k) {
             const uint32_t e = lds_u32(ps);
