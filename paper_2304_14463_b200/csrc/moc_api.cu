@@ -245,7 +245,7 @@ int quad_shape(const Plan& pl, int64_t n, int32_t B) {
 
 // Backward walk with a lane per sequence: n <= 128, C <= 4.  Used for the batches live_serves() names.
 void plan_live(const moc_graph* g, Plan* pl) {
-    if (!g->d_live64 || g->C > moc::kLivePlanes) return;
+    if (!g->d_live32 || g->C > moc::kLivePlanes) return;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C || g->sum_w > (int64_t)INT32_MAX / g->C;
     pl->live_image = wide ? g->d_live64 : g->d_live32;
     LiveFn fn = wide ? live_fn_w<int64_t>(live_words(g->n), g->C) : live_fn_w<int32_t>(live_words(g->n), g->C);
@@ -966,7 +966,9 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
             moc_graph_destroy(g);
             return fail(MOC_ERR_NOMEM, "host allocation failed");
         }
-        for (int wide = 0; wide < 2; ++wide) {
+        // tables for both widths, or the one that every C <= MOC_MAX_COPIES selects
+        const bool narrow = sum_m <= INT32_MAX / MOC_MAX_COPIES && sum_w <= INT32_MAX / MOC_MAX_COPIES;
+        for (int wide = 0; wide < (narrow ? 1 : 2); ++wide) {
             try {
                 const std::vector<uint32_t> image = moc::live_image(n, words, wide != 0, g->h_live_place, preds, m, w);
                 up((void**)(wide ? &g->d_live64 : &g->d_live32), image.data(), image.size() * 4);
