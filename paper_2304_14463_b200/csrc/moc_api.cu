@@ -1346,7 +1346,9 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     const size_t id_b = wide_ids ? 4 : 2, bB = (size_t)B;
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(MOC_ERR_CUDA, "cannot select device %d", g->device);
-    int rc = ensure((void**)&g->d_stage_seqs, &g->stage_seqs_cap, std::max<size_t>((size_t)n_steps * 4 + 16, 16));
+    int rc = ensure_plans(g);                  // before anything is in flight: a first call looks its kernels up
+    if (rc != MOC_OK) return rc;
+    rc = ensure((void**)&g->d_stage_seqs, &g->stage_seqs_cap, std::max<size_t>((size_t)n_steps * 4 + 16, 16));
     if (rc != MOC_OK) return rc;
     const size_t o_peak = 0, o_dur = bB * 8, o_st = 2 * bB * 8, o_lens = align16(o_st + bB * 4), res_bytes = o_st + bB * 4, io_bytes = o_lens + bB * 4;
     rc = ensure((void**)&g->d_stage_io, &g->stage_io_cap, io_bytes);
