@@ -284,12 +284,15 @@ __global__ void __launch_bounds__(kLiveThreads, 1) eval_live_kernel(const LivePa
         // eight steps at a time (a 32-byte sector of the row), the next eight on their way
         int i = ((T + a + 3) >> 2) - 1;
         const int trips = (int)__reduce_max_sync(kFull, (unsigned)(T > 0 ? (i + 2) >> 1 : 0));
-        int4 n1 = fetch(i), n0 = fetch(i - 1);
+        int4 n1 = fetch(i), n0 = fetch(i - 1), f1 = fetch(i - 2), f0 = fetch(i - 3);
+        i -= 2;
         for (int r = 0; r < trips; ++r) {
             const int4 q1 = n1, q0 = n0;
+            n1 = f1;
+            n0 = f0;
             i -= 2;
-            n1 = fetch(i);
-            n0 = fetch(i - 1);
+            f1 = fetch(i);
+            f0 = fetch(i - 1);
             four(q1);
             four(q0);
         }
