@@ -360,19 +360,20 @@ int moc_search_set_kinds(moc_search* s, uint32_t kinds);
  *                equals, and it replaces the chain's sequence when its key is not larger.  E = 1 is
  *                the single proposal described above.
  *   incremental  0 (MOC_SEARCH_WRITTEN_OUT): no cache; proposals are evaluated in full (E must be 1);
- *                1 (MOC_SEARCH_SCORE_AUTO): proposals are scored from the cached evaluation of the chain's
- *                sequence and only accepted ones are written out; the library picks the scoring kernel
- *                (a warp per chain from E = 24 on when the graph fits it, else the kernel of moc_eval_edits);
- *                2 (MOC_SEARCH_SCORE_EDIT): the same through moc_eval_edits: a generation is four
+ *                1 (MOC_SEARCH_SCORE_AUTO): the library picks the fastest way: one kernel for all generations
+ *                of a call, a warp per chain, without a cache where the graph fits it; else proposals are scored
+ *                from the cached evaluation of the chain's sequence and only accepted ones are written out (3 from
+ *                E = 24 on when the graph fits it, else 2);
+ *                2 (MOC_SEARCH_SCORE_EDIT): from the cache through moc_eval_edits: a generation is four
  *                kernels (draw, moc_eval_edits, pick, rebuild of the changed cache entries);
- *                3 (MOC_SEARCH_SCORE_CHAIN): the same with a warp per chain: the chain's cache entry is
+ *                3 (MOC_SEARCH_SCORE_CHAIN): from the cache with a warp per chain: the chain's cache entry is
  *                staged in shared memory once and its E proposals are drawn, scored and settled there;
  *                a generation is two kernels (that one and the rebuild).  MOC_ERR_ARG when the entry
  *                and the correction lists (4 + 2 * largest in-degree entries) of four chains do not
  *                fit the shared memory of an SM.
  *                1 to 3 need C <= 2 and a valid sequence (status >= 0) in every chain at the time of
  *                the call (MOC_ERR_ARG otherwise).  All four give identical chains.
- * Synchronises the device, allocates (the cache of the chains, 28 bytes per proposal); after it
+ * Synchronises the device, allocates (where a cache is used: it and 28 bytes per proposal); after it
  * moc_search_run allocates nothing.
  */
 #define MOC_SEARCH_WRITTEN_OUT 0

@@ -472,9 +472,9 @@ class Search:
         moc_search_set_kinds(self.h, kinds)
 
     def set_samples(self, samples, incremental=True):
-        """samples proposals per chain and generation; incremental: False / 0 written out and evaluated from
-        scratch, True / 1 scored from the cached evaluation (the library picks the kernel), 2 with a warp per
-        proposal, 3 with a warp per chain (MOC_SEARCH_*)."""
+        """samples proposals per chain and generation; incremental: False / 0 evaluated in full (samples = 1),
+        True / 1 the library picks the way, 2 scored from the cached evaluation with a warp per proposal, 3 with a
+        warp per chain (MOC_SEARCH_*)."""
         _check(lib.moc_search_set_samples(self.h, int(samples), int(incremental)), "moc_search_set_samples")
 
     def info(self):

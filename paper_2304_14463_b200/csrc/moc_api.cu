@@ -1330,14 +1330,20 @@ int host_streams(const moc_graph* g) {
     return MOC_OK;
 }
 
-// Address under which kernels reach a host array, or nullptr for pageable memory.
-void* mapped_address(const void* host) {
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+// Address under which kernels reach a host array of `bytes` bytes (at least one), or nullptr unless the whole of it,
+// judged by its two ends, is pinned and mapped.
+void* mapped_address(const void* host, size_t bytes) {
+    char* end[2] = {nullptr, nullptr};
+    for (int k = 0; k < 2; ++k) {
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, (const char*)host + (k ? bytes - 1 : 0)) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+        end[k] = (char*)at.devicePointer;
     }
-    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+    return end[1] - end[0] == (ptrdiff_t)(bytes - 1) ? end[0] : nullptr;
 }
 
 // ids: host array of `need` node ids, 4 bytes each (wide_ids) or 2 bytes each.
@@ -1360,7 +1366,8 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     // how the ids come: fetched by a kernel, copied in one piece, or in parts
     const void* m_ids = nullptr;
     const int32_t* m_lens = nullptr;
-    if (n_steps > 0 && n_steps * (int64_t)id_b <= kHostFetchBytes && (m_ids = mapped_address(ids)) != nullptr) m_lens = (const int32_t*)mapped_address(lens);
+    if (n_steps > 0 && n_steps * (int64_t)id_b <= kHostFetchBytes && (m_ids = mapped_address(ids, (size_t)n_steps * id_b)) != nullptr)
+        m_lens = (const int32_t*)mapped_address(lens, bB * 4);
     const bool parts = n_steps >= kHostCutSteps;
     if (!m_lens && !wide_ids) {
         rc = ensure((void**)&g->d_stage_u16, &g->stage_u16_cap, std::max<size_t>((size_t)n_steps * 2 + 16, 16));
@@ -1413,8 +1420,8 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         if (!m_lens) cudaStreamSynchronize(cs);                   // the caller's arrays are still being read
         return fail(MOC_ERR_ARG, "%s: lens sum to %lld > n_steps %lld", who, (long long)need, (long long)n_steps);
     }
-    int64_t *m_peak = (int64_t*)mapped_address(out_peak), *m_dur = m_peak ? (int64_t*)mapped_address(out_dur) : nullptr;
-    int32_t* m_st = m_dur ? (int32_t*)mapped_address(out_feasible) : nullptr;
+    int64_t *m_peak = (int64_t*)mapped_address(out_peak, bB * 8), *m_dur = m_peak ? (int64_t*)mapped_address(out_dur, bB * 8) : nullptr;
+    int32_t* m_st = m_dur ? (int32_t*)mapped_address(out_feasible, bB * 4) : nullptr;
     if (!m_st && res_bytes > g->h_stage_cap) {
         if (g->h_stage) MOC_CUDA(cudaFreeHost(g->h_stage));
         g->h_stage = nullptr;

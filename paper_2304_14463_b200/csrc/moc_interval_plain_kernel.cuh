@@ -14,7 +14,9 @@
 // An inactive slot's start is replaced by that of the other slot (it then asks for nothing new); a solution in which
 // some node has no active slot at all takes a plain loop over the edges instead.
 //
-// Bound: MEASURED
+// Bound: instruction issue (58 % of the slots, 3330 instructions per solution against 6310) and the shared-memory
+// data pipe (52 %).  n = 442, D = 884, 16384 solutions with their sequences: 179.8 -> 90.5 us, where the 207 MB of
+// DRAM traffic alone take 32.  Fetching the next solution into L2 ahead of time cost 5 us and 60 MB of traffic.
 #pragma once
 #include "moc_interval_kernels.cuh"
 #include "moc_pair_kernel.cuh"

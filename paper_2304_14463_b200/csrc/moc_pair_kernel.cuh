@@ -180,6 +180,12 @@ __device__ __forceinline__ void sts_u16_if_nonzero(uint32_t old, uint32_t addr, 
 #define MOC_KEEP(x) asm volatile("" : "+r"(x))
 
 
+// Bound: the shared-memory data pipe (76 % of one wavefront per clock, 528 wavefronts per sequence) and instruction issue
+// (66 %, 1750 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 43.0 -> 41.0 us (duration
+// and copy count by two warp reductions instead of ten 64-bit shuffles, row offsets added up once per sequence,
+// deltas cleared by the scan that reads them).  n = 353 with 64-bit sums, B = 1501: 18.4 -> 12.3 us (sums in two parts,
+// batch spread over all SMs).
+//
 // kPre: how many 16-byte vectors of the next row each lane fetches ahead (rows of about 128*kPre
 // steps; 0 for short rows, where the extra registers cost more than the wait).  Blocks have up to 16
 // warps and two of them share an SM (62 registers per thread, no spills).
