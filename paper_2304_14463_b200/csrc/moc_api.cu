@@ -229,18 +229,30 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, Plan* o
     return nullptr;
 }
 
-// Threads per sequence of the block-per-sequence kernel, as an index into Plan::quad_nb (64 << k).  With many sequences,
-// from measurements at n = 100 to 5000: more threads lose to the block-wide barriers, fewer to the length of the
-// per-thread loops.  With few, enough to give every SM about 16 warps.
-int quad_shape(const Plan& pl, int64_t n, int32_t B) {
-    if (pl.quad_forced) return 0;
-    int k = n < 700 ? 0 : (n < 1600 ? 1 : (n < 4000 ? 2 : 3));
+// Shape of the block-per-sequence kernel for a batch: threads per sequence (64 << k) and blocks per SM.  The time is
+// rounds x (latency or throughput of the sequences on an SM, whichever is longer, and a third of the other); both
+// follow measurements at n = 442, 1000 and 5000 (C = 3, 64 to 1024 threads, B = 1 to 16384; microseconds):
+//     latency of a sequence      0.93 per 64 nodes and 64 threads + 1.2 + 0.35 per 64 threads (barriers)
+//     SM time of a sequence      0.10 per 64 nodes + 0.16 per 64 threads
+// With the blocks per SM that the state and the registers allow, a batch takes ceil(sequences per SM / blocks) rounds;
+// as few blocks as that number of rounds needs keeps them even.
+void quad_shape(const Plan& pl, int64_t n, int32_t B, int* threads, int* blocks) {
     const int64_t per_sm = ((int64_t)B + pl.sm_count - 1) / pl.sm_count;
-    while (k < 3 && per_sm * (2 << (k + 1)) <= 16) ++k;
-    if (n >= 3000 && per_sm == 1) k = 4;
-    while (k < 4 && pl.quad_nb[k] == 0) ++k;
-    while (k > 0 && pl.quad_nb[k] == 0) --k;
-    return k;
+    const double units = (double)n / 64.0;
+    double best = 0;
+    *threads = 0;
+    for (int k = 0; k < 5; ++k) {
+        const int nb = pl.quad_nb[k], wide = 1 << k;
+        if (nb < 1) continue;
+        const int64_t rounds = (per_sm + nb - 1) / nb, even = (per_sm + rounds - 1) / rounds;
+        const double lat = 0.93 * units / wide + 1.2 + 0.35 * wide, thr = (double)even * (0.10 * units + 0.16 * wide);
+        const double cost = (double)rounds * (std::max(lat, thr) + 0.35 * std::min(lat, thr));
+        if (*threads == 0 || cost < best) {
+            best = cost;
+            *threads = pl.quad_forced ? pl.quad_forced : 64 << k;
+            *blocks = (int)even;
+        }
+    }
 }
 
 // Backward walk with a lane per sequence: n <= 128, C <= 4.  Used for the batches live_serves() names.
@@ -661,15 +673,8 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         smem = pl.pair_graph_b + (size_t)best_w * pl.pair_warp_b;
     }
     if (pl.quad) {
-        const int k = quad_shape(pl, g->n, B);
-        block = pl.quad_forced ? pl.quad_forced : 64 << k;
-        // blocks per SM: the least rounds * warps (a last round of few blocks costs a sequence's whole latency)
         int nb = 1;
-        int64_t best = INT64_MAX;
-        for (int c = 1; c <= std::max(1, pl.quad_nb[k]); ++c) {
-            const int64_t rounds = (B + (int64_t)pl.sm_count * c - 1) / ((int64_t)pl.sm_count * c), cost = rounds * std::max(c * block / 32, 24);
-            if (cost <= best) { best = cost; nb = c; }
-        }
+        quad_shape(pl, g->n, B, &block, &nb);
         grid = (int)std::min<int64_t>((int64_t)pl.sm_count * nb, B);
     }
     if (offs && fill_offs) {
