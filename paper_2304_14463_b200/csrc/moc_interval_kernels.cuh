@@ -11,6 +11,10 @@
 // rank(t) = number of marked events <= t, and every active interval [s, e] with s <= e adds m to the
 // marked events rank(s) .. rank(e): a difference array over at most n*C ranks and one prefix sum.
 // The same ranks order the active intervals into the execution sequence the solution stands for.
+//
+// Bound: latency at the few warps whose bitmaps fit an SM (staged domain, n = 442: 97903 events, 12 KB a warp).  The rank
+// bases therefore take 16 bits per four bitmap words, and the staged rule a 32-bit float root: staged, 16384 solutions,
+// n = 442: 1355 -> 529 us (6 -> 9 warps per SM), n = 900, 2000 solutions: 900 -> 559 us, n = 100: 66.7 -> 58.8 us.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -39,27 +43,28 @@ struct IntervalParams {
     int32_t* out_mask;
     int32_t* out_seqs;           // B rows of n*C ints, or nullptr
     int32_t* out_lens;           // B, or nullptr
-    uint32_t words;              // bitmap words: (D + 32) / 32  (bit t of the bitmap = event t, bit 0 unused)
+    uint32_t words;              // bitmap words: (D + 32) / 32, rounded up to a multiple of 4  (bit t of the bitmap = event t, bit 0 unused)
     uint32_t warp_bytes;         // shared memory of one warp
     int32_t byte_marks;          // plain model, and two bytes per event fit the space of the difference array
 };
 
 // Shared memory of one warp, in this order: bitmap of active starts [words], bitmap of all starts
-// [words] (plain model only, else absent), rank base per word [words], difference array [n*C + 2]
+// [words] (plain model only, else absent; words a multiple of 4), rank base per four words (16 bits each: there are
+// fewer than 65536 intervals on chip), difference array [n*C + 2]
 // (MemT), then -- when it fits -- the solution: start of every active slot (0 = inactive) and end of
 // every slot, [n*C] int32 each, written while the solution is read from HBM for the only time.
 __host__ __device__ inline size_t interval_bitmap_bytes(uint32_t words, bool plain) {
-    return (((size_t)words * 4 * (plain ? 3 : 2)) + 15) & ~size_t(15);
+    return ((size_t)words * 4 * (plain ? 2 : 1) + (size_t)words / 4 * 2 + 15) & ~size_t(15);
 }
 __host__ __device__ inline size_t interval_clear_bytes(uint32_t words, int64_t K, bool plain, size_t mem_sz) {
     return interval_bitmap_bytes(words, plain) + (((size_t)(K + 2) * mem_sz + 15) & ~size_t(15));
 }
 __host__ __device__ inline size_t interval_stage_bytes(int64_t K, size_t pos_sz) { return ((size_t)K * 2 * pos_sz + 15) & ~size_t(15); }
 
-// exact test "x = j(j-1)/2 for an integer j >= jmin"; x >= 0
-__device__ __forceinline__ bool is_triangular_from(int64_t x, int64_t jmin) {
-    // j = (1 + sqrt(1 + 8x)) / 2, corrected to the integer root
-    int64_t j = (int64_t)((1.0 + sqrt(1.0 + 8.0 * (double)x)) * 0.5);
+// exact test "x = j(j-1)/2 for an integer j >= jmin"; 0 <= x < 2^30
+__device__ __forceinline__ bool is_triangular_from(uint32_t x, uint32_t jmin) {
+    // j = (1 + sqrt(1 + 8x)) / 2 up to rounding (j < 46342, an error below 1), corrected to the integer root
+    uint32_t j = max((uint32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)x)) * 0.5f), 1u);
     while (j * (j - 1) / 2 > x) --j;
     while ((j + 1) * j / 2 <= x) ++j;
     return j * (j - 1) / 2 == x && j >= jmin;
@@ -84,7 +89,7 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
     char* ws = smem + (size_t)warp * p.warp_bytes;
     uint32_t* bm_act = reinterpret_cast<uint32_t*>(ws);
     uint32_t* bm_all = bm_act + p.words;                               // plain model only
-    uint32_t* rbase = bm_act + p.words * (kPlain ? 2u : 1u);
+    uint16_t* rbase = reinterpret_cast<uint16_t*>(bm_act + p.words * (kPlain ? 2u : 1u));
     MemT* delta = reinterpret_cast<MemT*>(ws + interval_bitmap_bytes(p.words, kPlain));
     PosT* sS = reinterpret_cast<PosT*>(ws + interval_clear_bytes(p.words, K, kPlain, sizeof(MemT)));
     PosT* sE = sS + K;
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
                         if (act) {
                             if (kPlain && p.byte_marks) by_act[2 * sv[i]] = 1;
                             else atomicOr(&bm_act[sv[i] >> 5], bit);
-                            if (!kPlain && !((int64_t)sv[i] >= k && is_triangular_from((int64_t)sv[i] - k, k))) mask |= kIvStage;
+                            if (!kPlain && !((int64_t)sv[i] >= k && is_triangular_from((uint32_t)((int64_t)sv[i] - k), (uint32_t)k))) mask |= kIvStage;
                         }
                         if (kPlain) {
                             bool seen = false;
@@ -217,22 +222,27 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
             __syncwarp();
         }
 
-        // ---- rank base of every bitmap word: exclusive prefix sum of the popcounts
+        // ---- rank base of every four bitmap words: exclusive prefix sum of the popcounts
         int32_t R;
         {
-            const uint32_t per = (p.words + 31) / 32;
-            const uint32_t w0 = min(p.words, (uint32_t)lane * per), w1 = min(p.words, w0 + per);
+            const uint32_t groups = p.words / 4, per = ((groups + 31) / 32) | 1u;      // odd: the lanes' vectors fall into different banks
+            const uint32_t g0 = min(groups, (uint32_t)lane * per), g1 = min(groups, g0 + per);
+            const uint4* v4 = reinterpret_cast<const uint4*>(bm_act);
             uint32_t cnt = 0;
-            for (uint32_t i = w0; i < w1; ++i) cnt += __popc(bm_act[i]);
+            for (uint32_t i = g0; i < g1; ++i) {
+                const uint4 v = v4[i];
+                cnt += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+            }
             uint32_t incl = cnt;
             for (int d = 1; d < 32; d <<= 1) {
                 const uint32_t o = __shfl_up_sync(kFull, incl, d);
                 if (lane >= d) incl += o;
             }
             uint32_t run = incl - cnt;
-            for (uint32_t i = w0; i < w1; ++i) {
-                rbase[i] = run;
-                run += __popc(bm_act[i]);
+            for (uint32_t i = g0; i < g1; ++i) {
+                rbase[i] = (uint16_t)run;
+                const uint4 v = v4[i];
+                run += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
             }
             R = (int32_t)__shfl_sync(kFull, incl, 31);       // number of distinct active starts
         }
@@ -248,8 +258,11 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
         int32_t* row = (p.out_seqs != nullptr && has_seq) ? p.out_seqs + (int64_t)b * K : nullptr;
         __syncwarp();
         auto rank = [&](int32_t t) -> int32_t {   // marked events <= t
-            const uint32_t wd = bm_act[t >> 5];
-            return (int32_t)(rbase[t >> 5] + __popc(wd & (0xFFFFFFFFu >> (31 - (t & 31)))));
+            const uint4 v = reinterpret_cast<const uint4*>(bm_act)[t >> 7];
+            const int32_t w = t >> 5 & 3;
+            const uint32_t upto = 0xFFFFFFFFu >> (31 - (t & 31));       // of word w; the words in front of it count whole
+            return (int32_t)rbase[t >> 7] + __popc(w == 0 ? v.x & upto : v.x) + (w < 1 ? 0 : __popc(w == 1 ? v.y & upto : v.y)) +
+                   (w < 2 ? 0 : __popc(w == 2 ? v.z & upto : v.z)) + (w < 3 ? 0 : __popc(v.w & upto));
         };
         // start (0 = inactive) and end of slot i of node v
         // both slots of node v at once (C = 2, positions staged in 16 bits)

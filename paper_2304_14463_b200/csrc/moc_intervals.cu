@@ -81,7 +81,7 @@ int check_intervals(const moc_graph* g, const int32_t* s, const int32_t* e, cons
         launch_counter() = 1;
         return MOC_OK;
     }
-    p.words = (uint32_t)((D + 32) / 32);
+    p.words = (uint32_t)(((D + 32) / 32 + 3) & ~int64_t(3));
     const bool plain = topo_index == nullptr;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;     // C * sum(m) bounds every partial usage sum
     const size_t cap = g->smem_optin > 2048 ? g->smem_optin - 2048 : 0;
