@@ -89,9 +89,10 @@ int check_intervals(const moc_graph* g, const int32_t* s, const int32_t* e, cons
     if (base_b > cap || K > (int64_t)INT32_MAX / 2)
         return fail(MOC_ERR_ARG, "moc_check_intervals: domain of %lld events with %lld intervals needs %zu bytes of "
                     "shared memory per solution, the device offers %zu", (long long)D, (long long)K, base_b, cap);
-    // keep the solution on chip after the first pass while at least eight solutions per SM still fit
+    // keep the solution on chip after the first pass while two solutions per SM still fit: reading it again costs more than the
+    // warps that its place would hold (staged, 4000 solutions: n = 600 344 -> 323 us, 700 582 -> 442, 1000 1658 -> 1271)
     p.byte_marks = plain && 2 * (((size_t)D + 1 + 15) & ~size_t(15)) <= ((((size_t)K + 2) * (wide ? 8 : 4) + 15) & ~size_t(15)) ? 1 : 0;
-    const bool stage = (base_b + stage_b) * 8 <= cap;
+    const bool stage = (base_b + stage_b) * 2 <= cap;
     const size_t warp_b = base_b + (stage ? stage_b : 0);
     p.warp_bytes = (uint32_t)warp_b;
     // warps per block: the count that puts most warps on an SM (each block loses 1 KB to the system)
