@@ -1,5 +1,7 @@
 // Host side of libmoc_b200.so: graph handle, validation, launch planning and the C ABI declared in
 // include/moc.h.  Every step of the evaluation itself runs in the kernels of moc_kernels.cuh.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cstdarg>
 #include <cstdio>
@@ -1335,20 +1337,31 @@ int host_streams(const moc_graph* g) {
     return MOC_OK;
 }
 
-// Address under which kernels reach a host array of `bytes` bytes (at least one), or nullptr unless the whole of it,
-// judged by its two ends, is pinned and mapped.
+// Address under which kernels reach a host array of `bytes` bytes (at least one), or nullptr unless every byte of it lies
+// in pinned memory that is mapped at its own address.  The array is followed from one registration to the next: an
+// array whose two ends are registered may still have a hole.
 void* mapped_address(const void* host, size_t bytes) {
-    char* end[2] = {nullptr, nullptr};
-    for (int k = 0; k < 2; ++k) {
-        cudaPointerAttributes at{};
-        if (cudaPointerGetAttributes(&at, (const char*)host + (k ? bytes - 1 : 0)) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
-        end[k] = (char*)at.devicePointer;
+    using Query = CUresult (*)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static const Query query = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found{};
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess) cudaGetLastError();
+        return found == cudaDriverEntryPointSuccess ? (Query)fn : nullptr;
+    }();
+    if (!query) return nullptr;
+    const CUdeviceptr first = (CUdeviceptr)(uintptr_t)host, end = first + bytes;
+    for (CUdeviceptr at = first; at < end;) {
+        unsigned int type = 0, managed = 0;
+        CUdeviceptr device = 0, start = 0;
+        size_t size = 0;
+        CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                      CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+        void* out[] = {&type, &managed, &device, &start, &size};
+        if (query(5, what, out, at) != CUDA_SUCCESS) return nullptr;
+        if (type != CU_MEMORYTYPE_HOST || managed || device != at || at < start || at - start >= size) return nullptr;
+        at = start + size;
     }
-    return end[1] - end[0] == (ptrdiff_t)(bytes - 1) ? end[0] : nullptr;
+    return const_cast<void*>(host);
 }
 
 // ids: host array of `need` node ids, 4 bytes each (wide_ids) or 2 bytes each.

@@ -454,6 +454,41 @@ def test_host_entry_point_u16(B):
     assert (p2 == op).all() and (d2 == od).all() and (s2 == os_).all()
 
 
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("nB", [1, 3, 250, 1500, 2100])
+@pytest.mark.parametrize("shift", [0, 1, 3])
+def test_short_pinned_host_batches(B, bits, nB, shift):
+    """Pinned ids up to 256 KB are fetched by a kernel, longer ones copied: element-wise tails, rows off a 16-byte
+    boundary (views into a pinned block), results written next to each other without touching their neighbours."""
+    n = 37
+    edges = W.layered_dag(n, 80, 6, 3)
+    w, m = W.weights_uniform(n, 0, 30, n, 1), W.weights_lognormal(n, 6.0, 1.5, n, 2)
+    seqs, lens = W.schedules(n, edges, 2, 0.3, nB, 7)
+    seqs, lens = W.mutate(seqs, lens, n, 2, seed=5, frac=1 / 8)
+    seqs = np.where(seqs < 0, 65535, seqs).astype(np.uint16 if bits == 16 else np.int32)
+    O, G = OracleGraph(n, edges, w, m, 2), B.Graph(n, edges, w, m, 2)
+    M = O.eval(np.arange(n), BIG)["peak"] * 90 // 100
+    want = O.eval_batch(seqs.astype(np.int32), lens, M)[:3]
+    ids = torch.from_numpy(np.concatenate([seqs[:shift], seqs, seqs[:5]])).pin_memory()[shift:shift + len(seqs)]
+    lens_p = torch.from_numpy(np.concatenate([lens, lens[:1]])).pin_memory()[:nB]
+    outs = [torch.full((nB + 2,), -77, dtype=d).pin_memory() for d in (torch.int64, torch.int64, torch.int32)]
+    call = G.eval_batch_host16 if bits == 16 else G.eval_batch_host
+    for _ in range(2):
+        call(ids, lens_p, M, *[o[1:nB + 1] for o in outs])
+        fetched = len(seqs) * bits // 8 <= 256 << 10
+        deliver = nB > 2048
+        assert B.moc_last_launch_count() == 1 + (fetched or bits == 16) + deliver
+        for o, r in zip(outs, want):
+            o = o.numpy()
+            assert (o[1:nB + 1] == r).all() and o[0] == -77 and o[nB + 1] == -77
+    # pageable ids with pinned results and the other way round
+    call(torch.from_numpy(seqs.copy()), lens_p, M, *[o[1:nB + 1] for o in outs])
+    pageable = [np.empty(nB, o.numpy().dtype) for o in outs]
+    call(ids, lens_p, M, *[torch.from_numpy(o) for o in pageable])
+    for o, p_, r in zip(outs, pageable, want):
+        assert (o.numpy()[1:nB + 1] == r).all() and (p_ == r).all()
+
+
 def test_host_entry_points_in_chunks(B):
     """A batch large enough to travel in several chunks (copy of one chunk under the evaluation of the
     one before), cut at sequence boundaries that do not divide the batch evenly; damaged sequences and

@@ -1,0 +1,111 @@
+"""The host side of the library (moc_api.cu) on a stand-in for the CUDA runtime (fake_cudart.cpp): which kernels are
+looked up and launched, what is copied, and what an error leaves behind.  Runs without a GPU; no kernel runs."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2304_14463_b200 import build, workloads
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+P, i32, i64 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    workloads.build()
+    lib = str(tmp_path_factory.mktemp("fake") / "libmoc_fake.so")
+    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    # no machine code and no optimisation of the kernels: they are never run
+    subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-Xcicc", "-O0", "-std=c++17", "-cudart", "none", "-shared",
+                    "-Xcompiler", "-fPIC", "-Xlinker", "-Bsymbolic,--no-undefined", "-t", "2", "-o", lib,
+                    os.path.join(build.CSRC, "moc_api.cu"), os.path.join(HERE, "fake_cudart.cpp")], check=True)
+    L = ctypes.CDLL(lib)
+    L.fake_log.restype = ctypes.c_char_p
+    L.fake_pin.argtypes = [P, ctypes.c_size_t]
+    L.moc_last_error.restype = ctypes.c_char_p
+    L.moc_graph_create.argtypes = [i32, i64, P, P, P, ctypes.POINTER(P)]
+    L.moc_graph_set_max_copies.argtypes = [P, i32]
+    L.moc_graph_destroy.argtypes = [P]
+    L.moc_graph_destroy.restype = None
+    L.moc_eval_batch.argtypes = [P, P, P, i32, i64, P, P, P, P]
+    for f in (L.moc_eval_batch_host, L.moc_eval_batch_host16):
+        f.argtypes = [P, P, i64, P, i32, i64, P, P, P, P]
+    yield L
+    L.fake_reset(0)
+
+
+class Graph:
+    def __init__(self, L, n, C=2, scale=1):
+        self.L, self.n, self.h = L, n, P()
+        edges = np.ascontiguousarray(workloads.layered_dag(n, 2 * n, max(2, n // 10), 1), np.int32)
+        w, m = np.ones(n, np.int64), np.full(n, scale, np.int64)
+        assert L.moc_graph_create(n, len(edges), edges.ctypes.data, w.ctypes.data, m.ctypes.data, ctypes.byref(self.h)) == 0
+        assert L.moc_graph_set_max_copies(self.h, C) == 0
+
+    def close(self):
+        self.L.moc_graph_destroy(self.h)
+
+
+class HostBatch:
+    """nB sequences of n ids in a buffer with `spare` more behind them."""
+
+    def __init__(self, n, nB, bits, spare=0):
+        self.nB, self.bits, self.need = nB, bits, n * nB
+        page = 4096
+        self.raw = np.zeros((self.need + spare) * bits // 8 + 2 * page, np.uint8)
+        self.start = (-self.raw.ctypes.data) % page
+        self.n_steps = self.need + spare
+        self.ids = self.raw.ctypes.data + self.start
+        self.lens = np.full(nB, n, np.int32)
+        self.out = [np.zeros(nB, d) for d in (np.int64, np.int64, np.int32)]
+
+    def pin(self, L, ids=True):
+        L.fake_unpin_all()
+        for a in [self.lens] + self.out:
+            L.fake_pin(a.ctypes.data, a.nbytes)
+        if ids:
+            L.fake_pin(self.ids, self.n_steps * self.bits // 8)
+
+    def run(self, G):
+        call = G.L.moc_eval_batch_host16 if self.bits == 16 else G.L.moc_eval_batch_host
+        return call(G.h, self.ids, self.n_steps, self.lens.ctypes.data, self.nB, 1000, *[o.ctypes.data for o in self.out], None)
+
+
+def log(L):
+    return L.fake_log().decode().splitlines()
+
+
+def launched(L, name):
+    return [x for x in log(L) if x.startswith("launch ") and name in x]
+
+
+@pytest.mark.parametrize("bits", [16, 32])
+def test_a_kernel_touches_host_memory_only_where_all_of_it_is_mapped(fake, bits):
+    """Ids that lie in one registration, in two that meet, and in two with an unregistered page between them."""
+    G, b = Graph(fake, 20), HostBatch(20, 400, bits)
+    size, page = b.n_steps * bits // 8, 4096
+    for cut, gap, kernel in ((size, 0, True), (page, 0, True), (page, page, False), (page + 1, 1, False)):
+        b.pin(fake, ids=False)
+        fake.fake_pin(b.ids, cut)
+        if cut + gap < size:
+            fake.fake_pin(b.ids + cut + gap, size - cut - gap)
+        fake.fake_reset(0)
+        assert b.run(G) == 0
+        assert bool(launched(fake, "fetch_kernel")) == kernel, (cut, gap)
+    b.pin(fake)
+    for k in range(3):                         # the same for the results: the k-th array has a hole
+        b.pin(fake)
+        fake.fake_unpin_all()
+        for i, a in enumerate(b.out):
+            if i == k:
+                fake.fake_pin(a.ctypes.data, 64)
+                fake.fake_pin(a.ctypes.data + 128, a.nbytes - 128)
+            else:
+                fake.fake_pin(a.ctypes.data, a.nbytes)
+        fake.fake_reset(0)
+        assert b.run(G) == 0
+        assert any(x.startswith("copy d2h") for x in log(fake)) and not launched(fake, "deliver_kernel")
+    G.close()
