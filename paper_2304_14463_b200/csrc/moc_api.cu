@@ -1364,6 +1364,19 @@ void* mapped_address(const void* host, size_t bytes) {
     return const_cast<void*>(host);
 }
 
+// Work of a host entry point that reads or writes the caller's arrays: whatever way the call returns, it is over by then.
+struct HostWork {
+    cudaStream_t copies = nullptr, work = nullptr;
+    bool begun = false;
+    HostWork() = default;
+    HostWork(const HostWork&) = delete;
+    ~HostWork() {
+        if (!begun) return;
+        cudaStreamSynchronize(copies);
+        if (work != copies) cudaStreamSynchronize(work);
+    }
+};
+
 // ids: host array of `need` node ids, 4 bytes each (wide_ids) or 2 bytes each.
 int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_steps, const int32_t* lens, int32_t B,
               int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st, const char* who) {
@@ -1393,6 +1406,7 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     }
     void* stage = wide_ids ? (void*)g->d_stage_seqs : (void*)g->d_stage_u16;
     cudaStream_t cs = st;
+    HostWork in_flight;
     int64_t at[kHostChunks + 1] = {0};         // ids on the device once part k has arrived
     auto copy_part = [&](int k) -> int {       // part k of the ids, and the lengths behind the first
         const int64_t cnt = at[k + 1] - at[k];
@@ -1414,6 +1428,9 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         MOC_CUDA(cudaEventRecord(g->chunk_ev[kHostChunks], st));
         MOC_CUDA(cudaStreamWaitEvent(cs, g->chunk_ev[kHostChunks], 0));
     }
+    in_flight.copies = cs;
+    in_flight.work = st;
+    in_flight.begun = true;
     if (!m_lens)
         for (int k = 0; k < n_parts; ++k) {
             rc = copy_part(k);
@@ -1434,10 +1451,7 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         if (b1 == B)
             for (++k; k <= n_parts; ++k) { cb[k] = B; co[k] = need; }
     }
-    if (need > n_steps) {
-        if (!m_lens) cudaStreamSynchronize(cs);                   // the caller's arrays are still being read
-        return fail(MOC_ERR_ARG, "%s: lens sum to %lld > n_steps %lld", who, (long long)need, (long long)n_steps);
-    }
+    if (need > n_steps) return fail(MOC_ERR_ARG, "%s: lens sum to %lld > n_steps %lld", who, (long long)need, (long long)n_steps);
     int64_t *m_peak = (int64_t*)mapped_address(out_peak, bB * 8), *m_dur = m_peak ? (int64_t*)mapped_address(out_dur, bB * 8) : nullptr;
     int32_t* m_st = m_dur ? (int32_t*)mapped_address(out_feasible, bB * 4) : nullptr;
     if (!m_st && res_bytes > g->h_stage_cap) {
@@ -1477,12 +1491,10 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         }
     }
     g_launches += launches;      // the evaluation launches were counted as they were enqueued
-    if (m_st) {
-        MOC_CUDA(cudaStreamSynchronize(st));
-        return MOC_OK;
-    }
-    MOC_CUDA(cudaMemcpyAsync(g->h_stage, g->d_stage_io, res_bytes, cudaMemcpyDeviceToHost, st));
-    MOC_CUDA(cudaStreamSynchronize(st));
+    if (!m_st) MOC_CUDA(cudaMemcpyAsync(g->h_stage, g->d_stage_io, res_bytes, cudaMemcpyDeviceToHost, st));
+    MOC_CUDA(cudaStreamSynchronize(st));       // which waits for the copy stream's events
+    in_flight.begun = false;
+    if (m_st) return MOC_OK;
     memcpy(out_peak, g->h_stage + o_peak, bB * 8);
     memcpy(out_dur, g->h_stage + o_dur, bB * 8);
     memcpy(out_feasible, g->h_stage + o_st, bB * 4);

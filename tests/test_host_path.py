@@ -109,3 +109,32 @@ def test_a_kernel_touches_host_memory_only_where_all_of_it_is_mapped(fake, bits)
         assert b.run(G) == 0
         assert any(x.startswith("copy d2h") for x in log(fake)) and not launched(fake, "deliver_kernel")
     G.close()
+
+
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("nB", [300, 4000, 110000])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_no_work_outlives_a_failed_call(fake, bits, nB, pinned):
+    """Every call into the runtime fails in turn: the error is returned, nothing that reads or writes the caller's arrays
+    is still in flight by then, and the handle goes on working.  So with lengths that exceed the buffer."""
+    fake.fake_unpin_all()
+    k = 0
+    while True:
+        G, b = Graph(fake, 20), HostBatch(20, nB, bits)
+        if pinned:
+            b.pin(fake)
+        k += 1
+        fake.fake_reset(k)
+        rc = b.run(G)
+        calls = fake.fake_calls()
+        if rc != 0:
+            assert fake.fake_in_flight() == 0, (k, log(fake))
+        fake.fake_reset(0)
+        assert b.run(G) == 0 and fake.fake_in_flight() == 0
+        b.n_steps -= 1
+        fake.fake_reset(0)
+        assert b.run(G) == -1 and fake.fake_in_flight() == 0
+        G.close()
+        if calls < k:
+            break
+    assert k > 10
