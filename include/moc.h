@@ -124,7 +124,8 @@ int moc_eval_batch(const moc_graph* g, const int32_t* seqs, const int32_t* lens,
  * with respect to the host, pageable memory works too): copies seqs (n_steps ints, which must be
  * at least sum(max(lens[b],0))) and lens to device staging owned by the handle, evaluates, copies
  * the three outputs back and synchronises `stream` before returning.  Large batches travel in
- * three parts (11, 4 and 1 sixteenths of the ids): a copy stream owned by the handle brings one part while
+ * three parts (11, 4 and 1 sixteenths of the ids; what lies behind the batch in seqs is not needed and not sent, but for a
+ * few ids where that is cheaper than to know): a copy stream owned by the handle brings one part while
  * `stream` evaluates the sequences that are complete with the one before, so that only the evaluation of
  * the small last part is not hidden; results return to pinned arrays straight from the device and to
  * pageable ones through a pinned block of the handle.  One call at a time per handle.

@@ -1313,27 +1313,32 @@ int moc_eval_batch(const moc_graph* g, const int32_t* seqs, const int32_t* lens,
 //
 // A large batch travels in three parts of 11/16, 4/16 and 1/16 of the ids on a copy stream owned by the handle, and the
 // caller's stream evaluates the sequences that have arrived in full while the next part is under way: the link is
-// busy throughout, every further part would cost it 4 us, and only the evaluation of the last sixteenth is exposed.  The
-// first part starts before the host has added up the lengths.  A batch whose copy is shorter than the calls
-// that would cut it goes in one piece on the caller's stream.
+// busy throughout, every further part would cost it 4 us, and only the evaluation of the last sixteenth is exposed.  A
+// batch whose copy is shorter than the calls that would cut it goes in one piece on the caller's stream.
+//
+// A caller's buffer may be much larger than the batch in it, and only the ids that the lengths add up to should travel.  Adding
+// up 16384 lengths takes 3.4 us, so the first part starts before that where a sample of the lengths says that
+// the batch fills the buffer (a wrong guess costs time, nothing else); otherwise, and for short batches, the lengths
+// come first.  Buffers of 2 and 4 times the batch: 673 and 1303 us with the whole buffer sent, 410 and 408 now.
 //
 // Results go to pinned arrays of the caller straight from the device, behind the copies of later parts; to
 // pageable ones with one copy into a pinned block of the handle and a memcpy.  Short batches in pinned memory
 // are also fetched by a kernel: one launch instead of two copies and the widening.
 //
 // n = 442, B = 16384, ids as 16-bit words (17.4 MB, 318 us at the link's 54.8 GB/s; one copy alone
-// takes 327): 445 -> 406 us a call.  B = 8: 49 -> 24 us, B = 200: 59 -> 32.
+// takes 327): 445 -> 385 us a call.  B = 8: 49 -> 24 us, B = 200: 59 -> 32.
 namespace {
 constexpr int kHostChunks = 3;
 constexpr int kHostPart[kHostChunks] = {11, 4, 1};       // sixteenths
-constexpr int64_t kHostCutSteps = (int64_t)1 << 21;      // from here on in chunks (4 MB of 16-bit ids: 80 us of copy)
+constexpr int64_t kHostCutSteps = (int64_t)1 << 21;      // from here on in parts (4 MB of 16-bit ids: 80 us of copy)
 constexpr int64_t kHostFetchBytes = 256 << 10;           // up to here fetched by a kernel (about 45 GB/s, no call per array)
 constexpr int32_t kHostDirect = 2048;                    // up to here sequences' results are written by the evaluation itself
+constexpr int32_t kHostSumFirst = 4096;                  // up to here the lengths are always added up first (1 us)
 
 int host_streams(const moc_graph* g) {
     if (g->copy_stream) return MOC_OK;
     MOC_CUDA(cudaStreamCreateWithFlags(&g->copy_stream, cudaStreamNonBlocking));
-    for (int k = 0; k < kHostChunks + 1; ++k) MOC_CUDA(cudaEventCreateWithFlags(&g->chunk_ev[k], cudaEventDisableTiming));   // chunk_ev has room for 9
+    for (int k = 0; k < kHostChunks + 1; ++k) MOC_CUDA(cudaEventCreateWithFlags(&g->chunk_ev[k], cudaEventDisableTiming));
     return MOC_OK;
 }
 
@@ -1377,15 +1382,36 @@ struct HostWork {
     }
 };
 
-// ids: host array of `need` node ids, 4 bytes each (wide_ids) or 2 bytes each.
+// Ids of the sequences b0 .. b1 - 1: the sum of max(lens, 0), in two 16-bit halves that the compiler adds up in vectors.
+int64_t steps_of(const int32_t* lens, int32_t b0, int32_t b1) {
+    int64_t sum = 0;
+    for (int32_t b = b0; b < b1;) {
+        const int32_t e = (int32_t)std::min<int64_t>(b1, (int64_t)b + 32768);
+        uint32_t lo = 0, hi = 0;
+        for (; b < e; ++b) {
+            const uint32_t x = (uint32_t)std::max(lens[b], 0);
+            lo += x & 0xFFFFu;
+            hi += x >> 16;
+        }
+        sum += (int64_t)lo + ((int64_t)hi << 16);
+    }
+    return sum;
+}
+
+// What 64 of the lengths, evenly spread, let the sum of all be.
+int64_t sampled_steps(const int32_t* lens, int32_t B) {
+    int64_t sum = 0;
+    for (int32_t k = 0; k < 64; ++k) sum += std::max(lens[(int64_t)B * k / 64], 0);
+    return (int64_t)((double)sum / 64 * B);
+}
+
+// ids: host array of n_steps node ids, 4 bytes each (wide_ids) or 2 bytes each, of which the sequences take the first.
 int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_steps, const int32_t* lens, int32_t B,
               int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st, const char* who) {
     const size_t id_b = wide_ids ? 4 : 2, bB = (size_t)B;
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(MOC_ERR_CUDA, "cannot select device %d", g->device);
     int rc = ensure_plans(g);                  // before anything is in flight: a first call looks its kernels up
-    if (rc != MOC_OK) return rc;
-    rc = ensure((void**)&g->d_stage_seqs, &g->stage_seqs_cap, std::max<size_t>((size_t)n_steps * 4 + 16, 16));
     if (rc != MOC_OK) return rc;
     const size_t o_peak = 0, o_dur = bB * 8, o_st = 2 * bB * 8, o_lens = align16(o_st + bB * 4), res_bytes = o_st + bB * 4, io_bytes = o_lens + bB * 4;
     rc = ensure((void**)&g->d_stage_io, &g->stage_io_cap, io_bytes);
@@ -1394,16 +1420,28 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     int64_t* d_dur = (int64_t*)(g->d_stage_io + o_dur);
     int32_t* d_st = (int32_t*)(g->d_stage_io + o_st);
     int32_t* d_lens = (int32_t*)(g->d_stage_io + o_lens);
+    auto too_long = [&](int64_t sum) {
+        return fail(MOC_ERR_ARG, "%s: lens sum to %lld > n_steps %lld", who, (long long)sum, (long long)n_steps);
+    };
+    const bool room = g->stage_seqs_cap >= (size_t)n_steps * 4 + 16 && (wide_ids || g->stage_u16_cap >= (size_t)n_steps * 2 + 16);
+    int64_t need = -1;                         // ids of the batch: not known yet
+    if (B <= kHostSumFirst || !room || sampled_steps(lens, B) / 32 * 33 < n_steps) {
+        need = steps_of(lens, 0, B);
+        if (need > n_steps) return too_long(need);
+        rc = ensure((void**)&g->d_stage_seqs, &g->stage_seqs_cap, (size_t)need * 4 + 16);
+        if (rc != MOC_OK) return rc;
+    }
+    const int64_t send = need >= 0 ? need : n_steps;
     // how the ids come: fetched by a kernel, copied in one piece, or in parts
     const void* m_ids = nullptr;
     const int32_t* m_lens = nullptr;
-    if (n_steps > 0 && n_steps * (int64_t)id_b <= kHostFetchBytes && (m_ids = mapped_address(ids, (size_t)n_steps * id_b)) != nullptr)
+    if (send > 0 && send * (int64_t)id_b <= kHostFetchBytes && (m_ids = mapped_address(ids, (size_t)send * id_b)) != nullptr)
         m_lens = (const int32_t*)mapped_address(lens, bB * 4);
-    const bool parts = n_steps >= kHostCutSteps;
     if (!m_lens && !wide_ids) {
-        rc = ensure((void**)&g->d_stage_u16, &g->stage_u16_cap, std::max<size_t>((size_t)n_steps * 2 + 16, 16));
+        rc = ensure((void**)&g->d_stage_u16, &g->stage_u16_cap, (size_t)send * 2 + 16);
         if (rc != MOC_OK) return rc;
     }
+    const bool parts = send >= kHostCutSteps;
     void* stage = wide_ids ? (void*)g->d_stage_seqs : (void*)g->d_stage_u16;
     cudaStream_t cs = st;
     HostWork in_flight;
@@ -1418,7 +1456,7 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     const int n_parts = parts ? kHostChunks : 1;
     for (int k = 0, sum = 0; k < n_parts; ++k) {
         sum += parts ? kHostPart[k] : 16;
-        at[k + 1] = sum == 16 ? n_steps : n_steps / 16 * sum;
+        at[k + 1] = sum == 16 ? send : (send / 16 * sum) & ~int64_t(7);      // every part starts on a 16-byte boundary
     }
     if (parts) {
         rc = host_streams(g);
@@ -1431,27 +1469,43 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     in_flight.copies = cs;
     in_flight.work = st;
     in_flight.begun = true;
-    if (!m_lens)
-        for (int k = 0; k < n_parts; ++k) {
-            rc = copy_part(k);
-            if (rc != MOC_OK) return rc;
-        }
-    // sequences that are complete with each part, while the first is under way
+    if (!m_lens) {
+        rc = copy_part(0);
+        if (rc != MOC_OK) return rc;
+    }
+    // the rest while the first part is under way
+    if (need < 0) {
+        need = steps_of(lens, 0, B);
+        if (need > n_steps) return too_long(need);
+        for (int k = 1; k < n_parts; ++k) at[k + 1] = std::min(at[k + 1], std::max(need, at[1]));
+    }
+    for (int k = 1; k < n_parts && !m_lens; ++k) {
+        rc = copy_part(k);
+        if (rc != MOC_OK) return rc;
+    }
+    // sequences that are complete with each part
     int32_t cb[kHostChunks + 1] = {0};
-    int64_t co[kHostChunks + 1] = {0}, need = 0;
-    for (int32_t b = 0, k = 0; b < B; b += 64) {
-        const int32_t b1 = std::min<int32_t>(B, b + 64);
-        int64_t sum = 0;
-        for (int32_t i = b; i < b1; ++i) sum += std::max(lens[i], 0);
-        while (k + 1 < n_parts && need + sum > at[k + 1]) {       // this piece of 64 sequences reaches beyond part k
-            cb[++k] = b;
+    int64_t co[kHostChunks + 1] = {0};
+    cb[n_parts] = B;
+    co[n_parts] = need;
+    if (parts) {
+        int64_t here = 0;
+        int k = 0;
+        for (int32_t b = 0; b < B && k + 1 < n_parts;) {
+            const int32_t b1 = (int32_t)std::min<int64_t>(B, (int64_t)b + 64);
+            const int64_t sum = steps_of(lens, b, b1);
+            while (k + 1 < n_parts && here + sum > at[k + 1]) {      // this piece of 64 sequences reaches beyond part k
+                cb[++k] = b;
+                co[k] = here;
+            }
+            here += sum;
+            b = b1;
+        }
+        for (++k; k < n_parts; ++k) {
+            cb[k] = B;
             co[k] = need;
         }
-        need += sum;
-        if (b1 == B)
-            for (++k; k <= n_parts; ++k) { cb[k] = B; co[k] = need; }
     }
-    if (need > n_steps) return fail(MOC_ERR_ARG, "%s: lens sum to %lld > n_steps %lld", who, (long long)need, (long long)n_steps);
     int64_t *m_peak = (int64_t*)mapped_address(out_peak, bB * 8), *m_dur = m_peak ? (int64_t*)mapped_address(out_dur, bB * 8) : nullptr;
     int32_t* m_st = m_dur ? (int32_t*)mapped_address(out_feasible, bB * 4) : nullptr;
     if (!m_st && res_bytes > g->h_stage_cap) {

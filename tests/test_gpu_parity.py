@@ -515,6 +515,30 @@ def test_host_entry_points_in_chunks(B):
     assert_batch_equal(G, O, seqs[:int(np.clip(lens[:100], 0, None).sum())], lens[:100], M, "after host calls")
 
 
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("nB", [4097, 9001])
+def test_host_buffers_larger_than_the_batch(B, bits, nB):
+    """One handle, buffers that fit, exceed by little and exceed by far: whatever is known before the first copy
+    starts, and with one length in between that no sample sees."""
+    wl = W.make(2, seed=11, B=nB)
+    O, G = OracleGraph(wl.n, wl.edges, wl.w, wl.m, wl.C), B.Graph(wl.n, wl.edges, wl.w, wl.m, wl.C)
+    lens = wl.lens.copy()
+    lens[nB // 64 + 1] += 3 * wl.n                                     # a sequence too long, over the ids of the next ones
+    rows = int(lens.sum())
+    seqs = np.resize(wl.seqs, 3 * rows)
+    M = O.eval(np.arange(wl.n), BIG)["peak"] * 80 // 100
+    want = O.eval_batch(seqs[:rows], lens, M)[:3]
+    ids = torch.from_numpy(seqs.astype(np.uint16) if bits == 16 else seqs).pin_memory()
+    l = torch.from_numpy(lens).pin_memory()
+    outs = [torch.empty(nB, dtype=dt).pin_memory() for dt in (torch.int64, torch.int64, torch.int32)]
+    call = G.eval_batch_host16 if bits == 16 else G.eval_batch_host
+    for n_steps in (3 * rows, rows, rows + 11, 3 * rows, rows):
+        call(ids[:n_steps], l, M, *outs)
+        assert all((o.numpy() == r).all() for o, r in zip(outs, want)), n_steps
+        for o in outs:
+            o.zero_()
+
+
 def test_state_in_global_memory(B):
     """A graph whose per-sequence state exceeds shared memory (and > 65534 steps per sequence)."""
     n, C = 40000, 2

@@ -40,7 +40,8 @@ def fake(tmp_path_factory):
 class Graph:
     def __init__(self, L, n, C=2, scale=1):
         self.L, self.n, self.h = L, n, P()
-        edges = np.ascontiguousarray(workloads.layered_dag(n, 2 * n, max(2, n // 10), 1), np.int32)
+        edges = workloads.layered_dag(n, 2 * n, max(2, n // 10), 1) if n >= 20 else np.zeros((0, 2), np.int32)
+        edges = np.ascontiguousarray(edges, np.int32)
         w, m = np.ones(n, np.int64), np.full(n, scale, np.int64)
         assert L.moc_graph_create(n, len(edges), edges.ctypes.data, w.ctypes.data, m.ctypes.data, ctypes.byref(self.h)) == 0
         assert L.moc_graph_set_max_copies(self.h, C) == 0
@@ -138,3 +139,59 @@ def test_no_work_outlives_a_failed_call(fake, bits, nB, pinned):
         if calls < k:
             break
     assert k > 10
+
+
+@pytest.mark.parametrize("bits", [16, 32])
+@pytest.mark.parametrize("n,nB", [(20, 1), (20, 300), (20, 4096), (3, 8192), (20, 8000), (20, 65536), (20, 110000), (700, 4001)])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_ids_behind_the_batch_do_not_travel(fake, bits, n, nB, pinned):
+    """A buffer of four times the batch: every id of the batch crosses the link once and none behind it, the first time (staging
+    grows to the batch, not to the buffer) and later; a few more ids than the batch may travel with a long batch in
+    one piece.  Batches in parts go through more than one evaluation."""
+    fake.fake_unpin_all()
+    G, b = Graph(fake, n), HostBatch(n, nB, bits, spare=3 * n * nB)
+    if pinned:
+        b.pin(fake)
+    for spare in (3 * n * nB, 0, 5, -1, 0, 5, 3 * n * nB):
+        if spare < 0:                         # from here on there is room for twice the batch
+            assert HostBatch(n, 2 * nB, bits).run(G) == 0
+            continue
+        b.n_steps = b.need + spare
+        fake.fake_reset(0)
+        assert b.run(G) == 0
+        lines = [x.split() for x in log(fake)]
+        moved = sum(int(x[3]) for x in lines if x[:2] == ["copy", "h2d"] and b.ids <= int(x[2]) < b.ids + b.need * bits // 8)
+        fetched = bool(launched(fake, "fetch_kernel"))
+        assert fetched and moved == 0 or b.need <= moved * 8 // bits <= b.need + (5 if spare == 5 else 0)
+        assert not any(b.ids + b.need * bits // 8 <= int(x[2]) < b.ids + b.n_steps * bits // 8 for x in lines if x[:2] == ["copy", "h2d"])
+        assert all(int(x[1]) <= max(4 * b.need + 16, 24 * nB + 16, 8 * (nB + 1)) for x in lines if x[0] == "malloc")
+        assert fetched == (pinned and b.need * bits // 8 <= 256 << 10)
+        assert len(launched(fake, "eval_")) == (3 if b.need >= 1 << 21 else 1)
+    G.close()
+
+
+def test_lengths_that_lie(fake):
+    """Negative lengths count as zero; lengths beyond 16 bits and beyond the buffer are found wherever they stand."""
+    for nB, n in ((300, 20), (8000, 20), (110000, 20)):
+        G, b = Graph(fake, n), HostBatch(n, nB, 16, spare=100000)
+        fake.fake_reset(0)
+        b.lens[nB // 2] = -7
+        b.lens[nB - 2] = 70000
+        assert b.run(G) == 0
+        for where in (0, nB // 8, nB // 2, nB - 1):
+            for _ in range(2):
+                lens = b.lens.copy()
+                b.lens[where] = 2 ** 31 - 1
+                fake.fake_reset(0)
+                assert b.run(G) == -1 and fake.fake_in_flight() == 0
+                assert str(int(np.maximum(b.lens.astype(np.int64), 0).sum())) in fake.moc_last_error().decode()
+                b.lens[:] = lens
+        # a sample of the lengths that promises much more than there is: the batch is evaluated all the same, once
+        b.lens[:] = 1
+        b.lens[[nB * k // 64 for k in range(64)]] = n
+        for steps in (n * nB, int(b.lens.sum())):
+            b.n_steps = steps
+            fake.fake_reset(0)
+            assert b.run(G) == 0 and fake.fake_in_flight() == 0
+            assert len(launched(fake, "eval_")) == 1
+        G.close()
