@@ -1272,11 +1272,9 @@ void moc_graph_destroy(moc_graph* g) {
     cudaFree(g->d_live32);
     cudaFree(g->d_live64);
     if (g->h_stage) cudaFreeHost(g->h_stage);
-    if (g->copy_stream) {
-        cudaStreamDestroy(g->copy_stream);
-        for (cudaEvent_t ev : g->chunk_ev)
-            if (ev) cudaEventDestroy(ev);
-    }
+    if (g->copy_stream) cudaStreamDestroy(g->copy_stream);
+    for (cudaEvent_t ev : g->chunk_ev)
+        if (ev) cudaEventDestroy(ev);
     for (int li = 0; li < 3; ++li) {
         cudaFree(g->lane[li].d_rec32);
         cudaFree(g->lane[li].d_rec64);
@@ -1328,17 +1326,16 @@ int moc_eval_batch(const moc_graph* g, const int32_t* seqs, const int32_t* lens,
 // n = 442, B = 16384, ids as 16-bit words (17.4 MB, 318 us at the link's 54.8 GB/s; one copy alone
 // takes 327): 445 -> 385 us a call.  B = 8: 49 -> 24 us, B = 200: 59 -> 32.
 namespace {
-constexpr int kHostChunks = 3;
-constexpr int kHostPart[kHostChunks] = {11, 4, 1};       // sixteenths
+constexpr int kHostPart[kHostParts] = {11, 4, 1};       // sixteenths
 constexpr int64_t kHostCutSteps = (int64_t)1 << 21;      // from here on in parts (4 MB of 16-bit ids: 80 us of copy)
 constexpr int64_t kHostFetchBytes = 256 << 10;           // up to here fetched by a kernel (about 45 GB/s, no call per array)
 constexpr int32_t kHostDirect = 2048;                    // up to here sequences' results are written by the evaluation itself
 constexpr int32_t kHostSumFirst = 4096;                  // up to here the lengths are always added up first (1 us)
 
 int host_streams(const moc_graph* g) {
-    if (g->copy_stream) return MOC_OK;
-    MOC_CUDA(cudaStreamCreateWithFlags(&g->copy_stream, cudaStreamNonBlocking));
-    for (int k = 0; k < kHostChunks + 1; ++k) MOC_CUDA(cudaEventCreateWithFlags(&g->chunk_ev[k], cudaEventDisableTiming));
+    if (!g->copy_stream) MOC_CUDA(cudaStreamCreateWithFlags(&g->copy_stream, cudaStreamNonBlocking));
+    for (cudaEvent_t& ev : g->chunk_ev)
+        if (!ev) MOC_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     return MOC_OK;
 }
 
@@ -1445,7 +1442,7 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     void* stage = wide_ids ? (void*)g->d_stage_seqs : (void*)g->d_stage_u16;
     cudaStream_t cs = st;
     HostWork in_flight;
-    int64_t at[kHostChunks + 1] = {0};         // ids on the device once part k has arrived
+    int64_t at[kHostParts + 1] = {0};         // ids on the device once part k has arrived
     auto copy_part = [&](int k) -> int {       // part k of the ids, and the lengths behind the first
         const int64_t cnt = at[k + 1] - at[k];
         if (cnt) MOC_CUDA(cudaMemcpyAsync((char*)stage + at[k] * id_b, (const char*)ids + at[k] * id_b, (size_t)cnt * id_b, cudaMemcpyHostToDevice, cs));
@@ -1453,7 +1450,7 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         if (parts) MOC_CUDA(cudaEventRecord(g->chunk_ev[k], cs));
         return MOC_OK;
     };
-    const int n_parts = parts ? kHostChunks : 1;
+    const int n_parts = parts ? kHostParts : 1;
     for (int k = 0, sum = 0; k < n_parts; ++k) {
         sum += parts ? kHostPart[k] : 16;
         at[k + 1] = sum == 16 ? send : (send / 16 * sum) & ~int64_t(7);      // every part starts on a 16-byte boundary
@@ -1463,8 +1460,8 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         if (rc != MOC_OK) return rc;
         cs = g->copy_stream;
         // the copy stream starts once the caller's stream has reached this call
-        MOC_CUDA(cudaEventRecord(g->chunk_ev[kHostChunks], st));
-        MOC_CUDA(cudaStreamWaitEvent(cs, g->chunk_ev[kHostChunks], 0));
+        MOC_CUDA(cudaEventRecord(g->chunk_ev[kHostParts], st));
+        MOC_CUDA(cudaStreamWaitEvent(cs, g->chunk_ev[kHostParts], 0));
     }
     in_flight.copies = cs;
     in_flight.work = st;
@@ -1484,8 +1481,8 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         if (rc != MOC_OK) return rc;
     }
     // sequences that are complete with each part
-    int32_t cb[kHostChunks + 1] = {0};
-    int64_t co[kHostChunks + 1] = {0};
+    int32_t cb[kHostParts + 1] = {0};
+    int64_t co[kHostParts + 1] = {0};
     cb[n_parts] = B;
     co[n_parts] = need;
     if (parts) {

@@ -22,6 +22,8 @@ using LaneFn = void (*)(const moc::LaneParams);
 using QuadFn = void (*)(const moc::QuadParams);
 using LiveFn = void (*)(const moc::LiveParams);
 
+constexpr int kHostParts = 3;          // parts in which the host entry points send a large batch
+
 struct Plan {
     bool valid = false;
     KernelFn fn = nullptr;
@@ -154,7 +156,7 @@ struct moc_graph {
     mutable char* h_stage = nullptr;     // pinned: peak | dur | status as they come back in one copy
     mutable size_t h_stage_cap = 0;
     mutable cudaStream_t copy_stream = nullptr;   // host entry points: brings the next chunk while one is evaluated
-    mutable cudaEvent_t chunk_ev[9] = {};
+    mutable cudaEvent_t chunk_ev[moc_host::kHostParts + 1] = {};   // one per part, and the caller's stream having come to the call
 };
 
 

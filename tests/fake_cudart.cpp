@@ -135,12 +135,12 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
 }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st) {
-    if (fails()) return cudaErrorUnknown;
+    if (fails() || !e) return cudaErrorUnknown;
     g_events[e].behind = g_streams[st].ops;
     return cudaSuccess;
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned) {
-    if (fails()) return cudaErrorUnknown;
+    if (fails() || !e) return cudaErrorUnknown;
     std::vector<size_t>& ops = g_streams[st].ops;
     for (size_t i : g_events[e].behind)
         if (std::find(ops.begin(), ops.end(), i) == ops.end()) ops.push_back(i);
