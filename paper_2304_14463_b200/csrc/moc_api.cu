@@ -35,92 +35,6 @@ namespace {
 
 size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
-template <int G, typename MemT>
-KernelFn shared_fn_cp(int CP, bool profile) {
-    if (profile && G != 1024) return nullptr;
-    switch (CP) {
-        case 2: return profile ? (KernelFn)moc::eval_shared_kernel<1024, MemT, 2, true>
-                               : (KernelFn)moc::eval_shared_kernel<G, MemT, 2, false>;
-        case 4: return profile ? (KernelFn)moc::eval_shared_kernel<1024, MemT, 4, true>
-                               : (KernelFn)moc::eval_shared_kernel<G, MemT, 4, false>;
-        default: return profile ? (KernelFn)moc::eval_shared_kernel<1024, MemT, 8, true>
-                                : (KernelFn)moc::eval_shared_kernel<G, MemT, 8, false>;
-    }
-}
-template <typename MemT>
-KernelFn shared_fn_g(int G, int CP, bool profile) {
-    switch (G) {
-        case 32: return shared_fn_cp<32, MemT>(CP, profile);
-        case 64: return shared_fn_cp<64, MemT>(CP, profile);
-        case 128: return shared_fn_cp<128, MemT>(CP, profile);
-        case 256: return shared_fn_cp<256, MemT>(CP, profile);
-        case 512: return shared_fn_cp<512, MemT>(CP, profile);
-        case 1024: return shared_fn_cp<1024, MemT>(CP, profile);
-        default: return nullptr;
-    }
-}
-KernelFn global_fn(int CP, bool profile) {
-    switch (CP) {
-        case 2: return profile ? (KernelFn)moc::eval_global_kernel<2, true> : (KernelFn)moc::eval_global_kernel<2, false>;
-        case 4: return profile ? (KernelFn)moc::eval_global_kernel<4, true> : (KernelFn)moc::eval_global_kernel<4, false>;
-        default: return profile ? (KernelFn)moc::eval_global_kernel<8, true> : (KernelFn)moc::eval_global_kernel<8, false>;
-    }
-}
-
-template <typename MemT>
-PairFn pair_fn_t(int pre) {
-    switch (pre) {
-        case 0: return (PairFn)moc::eval_pair_kernel<MemT, 0>;
-        case 1: return (PairFn)moc::eval_pair_kernel<MemT, 1>;
-        case 2: return (PairFn)moc::eval_pair_kernel<MemT, 2>;
-        case 3: return (PairFn)moc::eval_pair_kernel<MemT, 3>;
-        case 4: return (PairFn)moc::eval_pair_kernel<MemT, 4>;
-        default: return (PairFn)moc::eval_pair_kernel<MemT, 5>;
-    }
-}
-PairFn pair_fn(bool wide, int pre) { return wide ? pair_fn_t<int64_t>(pre) : pair_fn_t<int32_t>(pre); }
-
-template <typename MemT, int LG>
-LaneFn lane_fn_kp(int kp) {
-    switch (kp) {
-        case 2: return (LaneFn)moc::eval_lane_kernel<MemT, LG, 2>;
-        case 4: return (LaneFn)moc::eval_lane_kernel<MemT, LG, 4>;
-        case 6: return (LaneFn)moc::eval_lane_kernel<MemT, LG, 6>;
-        default: return (LaneFn)moc::eval_lane_kernel<MemT, LG, 8>;
-    }
-}
-template <typename MemT>
-LaneFn lane_fn_lg(int lg, int kp) {
-    switch (lg) {
-        case 5: return lane_fn_kp<MemT, 5>(kp);
-        case 4: return lane_fn_kp<MemT, 4>(kp);
-        default: return lane_fn_kp<MemT, 3>(kp);
-    }
-}
-LaneFn lane_fn(bool wide, int lg, int kp) { return wide ? lane_fn_lg<int64_t>(lg, kp) : lane_fn_lg<int32_t>(lg, kp); }
-
-template <typename MemT, bool kTiles>
-QuadFn quad_fn_c(int C, bool profile) {
-    if (profile) return C <= 3 ? (QuadFn)moc::eval_quad_kernel<MemT, 3, kTiles, true> : (QuadFn)moc::eval_quad_kernel<MemT, 4, kTiles, true>;
-    return C <= 3 ? (QuadFn)moc::eval_quad_kernel<MemT, 3, kTiles, false> : (QuadFn)moc::eval_quad_kernel<MemT, 4, kTiles, false>;
-}
-QuadFn quad_fn(bool wide, int C, bool tiles, bool profile) {
-    if (tiles) return wide ? quad_fn_c<int64_t, true>(C, profile) : quad_fn_c<int32_t, true>(C, profile);
-    return wide ? quad_fn_c<int64_t, false>(C, profile) : quad_fn_c<int32_t, false>(C, profile);
-}
-
-template <typename SumT, int W>
-LiveFn live_fn_k(int C) {
-    return C <= 2 ? (LiveFn)moc::eval_live_kernel<SumT, W, 2> : (LiveFn)moc::eval_live_kernel<SumT, W, 4>;
-}
-template <typename SumT>
-LiveFn live_fn_w(int words, int C) {
-    switch (words) {
-        case 1: return live_fn_k<SumT, 1>(C);
-        case 2: return live_fn_k<SumT, 2>(C);
-        default: return live_fn_k<SumT, 4>(C);
-    }
-}
 int live_words(int n) { return n <= 32 ? 1 : (n <= 64 ? 2 : 4); }
 
 // Raises a kernel's dynamic shared-memory limit to all the device offers beside its static part.
@@ -259,12 +173,18 @@ void quad_shape(const Plan& pl, int64_t n, int32_t B, int* threads, int* blocks)
 
 // Backward walk with a lane per sequence: n <= 128, C <= 4.  Used for the batches live_serves() names.
 void plan_live(const moc_graph* g, Plan* pl) {
-    if (!g->d_live32 || g->C > moc::kLivePlanes) return;
+    pl->valid = true;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C || g->sum_w > (int64_t)INT32_MAX / g->C;
     pl->live_image = wide ? g->d_live64 : g->d_live32;
-    LiveFn fn = wide ? live_fn_w<int64_t>(live_words(g->n), g->C) : live_fn_w<int32_t>(live_words(g->n), g->C);
+    LiveFn fn = live_fn(wide, live_words(g->n), g->C);
     if (raise_smem_limit((const void*)fn, g->smem_optin) != cudaSuccess) { cudaGetLastError(); return; }
     pl->live_fn = fn;
+}
+
+// Whether the warp-per-sequence kernel can serve the graph, as far as the host can tell.
+bool warp_serves(const moc_graph* g) {
+    const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    return g->C <= 2 && g->d_rec32 != nullptr && (!wide || g->split_ok) && (__int128)g->C * g->sum_w < ((__int128)1 << 48);
 }
 
 // Chooses kernel variant, group size and grid for the handle's current n and C.  The dynamic
@@ -283,7 +203,6 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     const size_t smem_cap = g->smem_optin > 1024 ? g->smem_optin - 1024 : 0;  // 1 KB per block is reserved
     const int kind = profile ? MOC_KERNEL_GROUP : g->want_kind;
     const bool shape_given = g->want_G != 0 || g->want_gpc != 0;       // moc_graph_set_launch
-    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile) plan_live(g, &pl);
     if (profile && !plan_quad(g, smem_cap, true, &pl)) {
         *out = pl;
         return MOC_OK;
@@ -291,7 +210,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     // Order of preference when nothing is forced: warp per sequence, then sequence per lane (it also
     // serves graphs whose degrees are too uneven for the warp kernel's padded successor tiles), then
     // the thread-group kernel, which serves everything.
-    const bool warp_ok = C <= 2 && g->d_rec32 != nullptr && (!pl.wide || g->split_ok) && (__int128)C * g->sum_w < ((__int128)1 << 48);
+    const bool warp_ok = warp_serves(g);
     if (kind == MOC_KERNEL_LANE || (kind == MOC_KERNEL_AUTO && !shape_given && !warp_ok)) {
         const char* why = plan_lane(g, smem_cap, &pl);
         if (!why) {
@@ -323,7 +242,8 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         const int pre = n < 256 ? 0 : (int)std::min<int64_t>(5, (n * 13 / 10 + 96) / 128);
         PairFn fn = pair_fn(pl.wide, pre);
         int best_wpb = 0, best_warps = 0, best_nb = 0;
-        if (raise_smem_limit((const void*)fn, g->smem_optin) != cudaSuccess) cudaGetLastError();
+        cudaError_t e = raise_smem_limit((const void*)fn, g->smem_optin);
+        if (e != cudaSuccess) return fail(MOC_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
         for (int wpb = 16; wpb >= 4; --wpb) {    // every kernel variant is compiled for up to 512 threads, two blocks per SM
             if (g->want_gpc && wpb != std::min(g->want_gpc, 16)) continue;
             const size_t sm = graph_b + wpb * warp_b;
@@ -346,8 +266,6 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
             pl.grid = g->sm_count * best_nb;
             pl.rec_bytes = (uint32_t)rec_b; pl.w_bytes = (uint32_t)w_b;
             pl.sell_bytes = (uint32_t)jds_b; pl.word_bytes = (uint32_t)word_b; pl.delta_bytes = (uint32_t)delta_b;
-            cudaError_t e = raise_smem_limit((const void*)fn, g->smem_optin);
-            if (e != cudaSuccess) return fail(MOC_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
             pl.valid = true;
             *out = pl;
             return MOC_OK;
@@ -378,7 +296,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         pl.gpc = gpc;
         pl.block = G * gpc;
         pl.smem = (size_t)gpc * sh_group;
-        pl.fn = pl.wide ? shared_fn_g<int64_t>(G, pl.CP, profile) : shared_fn_g<int32_t>(G, pl.CP, profile);
+        pl.fn = shared_fn(pl.wide, G, pl.CP, profile);
         if (!pl.fn) return fail(MOC_ERR_ARG, "unsupported launch shape");
         cudaError_t e = raise_smem_limit((const void*)pl.fn, g->smem_optin);
         if (e != cudaSuccess) return fail(MOC_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
@@ -595,9 +513,10 @@ moc::QuadParams quad_params(const moc_graph* g, const Plan& pl) {
 // 6 us + 0.17 us per node (a lane's steps follow one another), while the warp-per-sequence kernel takes 1.2 us per
 // 1000 sequences of these sizes (2 us with 64-bit sums; the block-per-sequence kernel with C >= 3 likewise).
 // Measured crossings: n = 20 at 7000, 50 at 11000, 100 at 17000 sequences; 100 with 64-bit sums or C = 3 at 9000.
-bool live_serves(const moc_graph* g, const Plan& pl, int32_t B) {
-    if (pl.live_fn == nullptr) return false;
-    return (int64_t)B * (g->C <= 2 && !pl.wide ? 6 : 10) >= 30000 + 850 * (int64_t)g->n;
+bool live_serves(const moc_graph* g, int32_t B) {
+    if (!g->d_live32 || g->C > moc::kLivePlanes || g->want_kind != MOC_KERNEL_AUTO || g->want_G || g->want_gpc) return false;
+    const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    return (int64_t)B * (g->C <= 2 && !wide ? 6 : 10) >= 30000 + 850 * (int64_t)g->n;
 }
 
 int enqueue_live(const moc_graph* g, const Plan& pl, const int64_t* offs, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
@@ -767,41 +686,53 @@ bool rows_without_scratch(const Plan& pl, int32_t B) {
     return (pl.pair || pl.lane || pl.quad) && (int64_t)pl.grid * B * 2 <= (int64_t)16 << 20;
 }
 
-// The plan for a batch of B: where the warp-per-sequence kernel serves the graph, the block-per-sequence kernel still
+// Where the warp-per-sequence kernel serves the graph, the block-per-sequence kernel still
 // takes the batches in which a warp's latency decides (a sequence has several warps there) and the long sequences,
 // whose state leaves too few warps on an SM (make_plan).  Measured at C = 2, warp / block: n = 442 10.4 / 8.8 us at B = 148,
 // 10.3 / 10.3 at 296, 10.4 / 12.4 at 600; n = 1000 16.5 / 10.3 at 296, 16.5 / 14.5 at 600, 16.5 / 16.5 at 1000, 18.6 / 26.8
 // at 2000; n = 1500 36 / 37 at 2000.
-const Plan& plan_for(const moc_graph* g, int32_t B) {
-    const Plan& pl = g->plan_eval;
-    if (!pl.pair || !g->plan_block.valid) return pl;
-    const int64_t n = g->n, sm = pl.sm_count;
-    const bool block = (n >= 700 && B <= 6 * sm) || (n >= 400 && B <= 2 * sm);
-    return block ? g->plan_block : pl;
+bool block_serves(const moc_graph* g, int32_t B) {
+    if (g->want_kind != MOC_KERNEL_AUTO || g->want_G || !warp_serves(g)) return false;
+    const int64_t n = g->n, sm = g->sm_count;
+    return (n >= 700 && B <= 6 * sm) || (n >= 400 && B <= 2 * sm);
 }
 
-// Makes the plans of the handle on first use.
-int ensure_plans(const moc_graph* g) {
-    if (g->plan_eval.valid) return MOC_OK;
-    g->plan_block = Plan();
-    int rc = make_plan(g, false, &g->plan_eval);
-    if (rc == MOC_OK && g->plan_eval.pair && g->want_kind == MOC_KERNEL_AUTO) {
-        Plan pl;
-        pl.wide = g->plan_eval.wide;
-        if (!plan_quad(g, g->smem_optin > 1024 ? g->smem_optin - 1024 : 0, false, &pl)) g->plan_block = pl;
+// The plan for a batch of B, made when a batch first needs it: looking a kernel up loads it, and a kernel that is never
+// launched should cost a program nothing (first evaluation of a handle, kernels loaded: 28 us with every kernel that may
+// serve it looked up, 25 with one; the next evaluation takes 18).  `walk`: the backward walk may serve it (which is
+// told by live_fn); nullptr: the error is in *rc.
+const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
+    *rc = MOC_OK;
+    if (walk && live_serves(g, B)) {
+        if (!g->plan_live.valid) plan_live(g, &g->plan_live);
+        if (g->plan_live.live_fn) return &g->plan_live;
     }
-    return rc;
+    if (block_serves(g, B)) {
+        if (!g->plan_block.valid) {
+            Plan pl;
+            pl.wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+            plan_quad(g, g->smem_optin > 1024 ? g->smem_optin - 1024 : 0, false, &pl);
+            pl.valid = true;
+            g->plan_block = pl;
+        }
+        if (g->plan_block.quad) return &g->plan_block;
+    }
+    if (!g->plan_eval.valid) *rc = make_plan(g, false, &g->plan_eval);
+    return *rc == MOC_OK ? &g->plan_eval : nullptr;
 }
+
+void forget_plans(moc_graph* g) { g->plan_eval = g->plan_block = g->plan_live = Plan(); }
 
 int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
                 int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {
-    int rc0 = ensure_plans(g);
-    if (rc0 != MOC_OK) return rc0;
-    const Plan& pl = plan_for(g, B);
-    if (live_serves(g, g->plan_eval, B)) return enqueue_live(g, g->plan_eval, nullptr, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
+    int rc;
+    const Plan* plan = plan_for(g, B, true, &rc);
+    if (!plan) return rc;
+    const Plan& pl = *plan;
+    if (pl.live_fn) return enqueue_live(g, pl, nullptr, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     if (rows_without_scratch(pl, B))
         return enqueue_eval(g, pl, nullptr, false, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
-    int rc = ensure((void**)&g->d_offs, &g->offs_cap, ((size_t)B + 1) * sizeof(int64_t));
+    rc = ensure((void**)&g->d_offs, &g->offs_cap, ((size_t)B + 1) * sizeof(int64_t));
     if (rc != MOC_OK) return rc;
     if (pl.global_state) {
         rc = ensure((void**)&g->d_state, &g->state_cap, (size_t)pl.grid * pl.group_bytes);
@@ -815,12 +746,13 @@ int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, in
 namespace moc_host {
 int eval_rows(const moc_graph* g, const int64_t* offs, const int32_t* seqs, const int32_t* lens, int32_t B,
               int64_t M, int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {
-    int rc0 = ensure_plans(g);
-    if (rc0 != MOC_OK) return rc0;
-    const Plan& pl = plan_for(g, B);
-    if (live_serves(g, g->plan_eval, B)) return enqueue_live(g, g->plan_eval, offs, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
+    int rc;
+    const Plan* plan = plan_for(g, B, true, &rc);
+    if (!plan) return rc;
+    const Plan& pl = *plan;
+    if (pl.live_fn) return enqueue_live(g, pl, offs, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
     if (pl.global_state) {
-        int rc = ensure((void**)&g->d_state, &g->state_cap, (size_t)pl.grid * pl.group_bytes);
+        rc = ensure((void**)&g->d_state, &g->state_cap, (size_t)pl.grid * pl.group_bytes);
         if (rc != MOC_OK) return rc;
     }
     return enqueue_eval(g, pl, const_cast<int64_t*>(offs), false, seqs, lens, B, M, out_peak, out_dur, out_feasible, st);
@@ -1143,7 +1075,7 @@ int moc_graph_set_max_copies(moc_graph* g, int32_t C) {
     }
     g->C = C;
     ++g->generation;
-    g->plan_eval.valid = false;
+    forget_plans(g);
     g->plan_profile.valid = false;
     return MOC_OK;
 }
@@ -1219,7 +1151,7 @@ int moc_graph_set_kernel(moc_graph* g, int32_t kind, int32_t a, int32_t b) {
     g->want_b = b;
     g->want_G = kind == MOC_KERNEL_GROUP ? a : 0;
     g->want_gpc = (kind == MOC_KERNEL_GROUP || kind == MOC_KERNEL_WARP) ? b : 0;
-    g->plan_eval.valid = false;
+    forget_plans(g);
     return MOC_OK;
 }
 
@@ -1232,7 +1164,7 @@ int moc_graph_set_launch(moc_graph* g, int32_t tps, int32_t spb) {
     g->want_a = g->want_b = 0;
     g->want_G = tps;
     g->want_gpc = spb;
-    g->plan_eval.valid = false;
+    forget_plans(g);
     return MOC_OK;
 }
 
@@ -1408,8 +1340,7 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
     const size_t id_b = wide_ids ? 4 : 2, bB = (size_t)B;
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(MOC_ERR_CUDA, "cannot select device %d", g->device);
-    int rc = ensure_plans(g);                  // before anything is in flight: a first call looks its kernels up
-    if (rc != MOC_OK) return rc;
+    int rc = MOC_OK;
     const size_t o_peak = 0, o_dur = bB * 8, o_st = 2 * bB * 8, o_lens = align16(o_st + bB * 4), res_bytes = o_st + bB * 4, io_bytes = o_lens + bB * 4;
     rc = ensure((void**)&g->d_stage_io, &g->stage_io_cap, io_bytes);
     if (rc != MOC_OK) return rc;
@@ -1439,6 +1370,8 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         if (rc != MOC_OK) return rc;
     }
     const bool parts = send >= kHostCutSteps;
+    for (int k = 0; k < (parts ? kHostParts : 1); ++k)         // before anything is in flight: a first call looks its kernels up
+        if (!plan_for(g, parts ? (int32_t)((int64_t)B * kHostPart[k] / 16) : B, true, &rc)) return rc;
     void* stage = wide_ids ? (void*)g->d_stage_seqs : (void*)g->d_stage_u16;
     cudaStream_t cs = st;
     HostWork in_flight;
@@ -1621,9 +1554,9 @@ int moc_eval_batch_noalloc(const moc_graph* g, const int32_t* seqs, const int32_
     int64_t* offs = nullptr;
     int rc = noalloc_offsets(g->device, &offs);
     if (rc != MOC_OK) return rc;
-    rc = ensure_plans(g);  // attribute and occupancy queries only
-    if (rc != MOC_OK) return rc;
-    const Plan& pl = plan_for(g, B);
+    const Plan* plan = plan_for(g, B, false, &rc);  // attribute and occupancy queries only
+    if (!plan) return rc;
+    const Plan& pl = *plan;
     if (pl.global_state)
         return fail(MOC_ERR_ARG, "moc_eval_batch_noalloc: this graph needs a global workspace "
                     "(per-sequence state exceeds shared memory); use moc_eval_batch");

@@ -13,6 +13,7 @@
 #include "moc_lane_kernel.cuh"
 #include "moc_quad_kernel.cuh"
 #include "moc_live_kernel.cuh"
+#include "moc_interval_kernels.cuh"
 
 namespace moc_host {
 
@@ -21,6 +22,22 @@ using PairFn = void (*)(const moc::PairParams);
 using LaneFn = void (*)(const moc::LaneParams);
 using QuadFn = void (*)(const moc::QuadParams);
 using LiveFn = void (*)(const moc::LiveParams);
+using IntervalFn = void (*)(const moc::IntervalParams);
+
+// Every family of kernels has a source file, and with it a module, of its own: the first use of a kernel loads its whole
+// module, and a program uses few of them (first evaluation of a process, n = 20, B = 64: 15.0 ms with all kernels of the
+// evaluator in one module, 1.0 ms so).  nullptr: no such variant.
+KernelFn shared_fn(bool wide, int G, int CP, bool profile);
+KernelFn global_fn(int CP, bool profile);
+PairFn pair_fn(bool wide, int pre);
+LaneFn lane_fn(bool wide, int lg, int kp);
+QuadFn quad_fn(bool wide, int C, bool tiles, bool profile);
+LiveFn live_fn(bool wide, int words, int C);
+const void* check_plain_fn(bool wide);
+IntervalFn check_general_fn(int cp, bool wide, int kept);      // kept: bytes per event of the solution kept on chip, 0: not kept
+IntervalFn check_staged_fn(int cp, bool wide, int kept);
+const void* score_fn(bool wide, bool graph_on_chip);
+const void* walk_fn(bool wide);
 
 constexpr int kHostParts = 3;          // parts in which the host entry points send a large batch
 
@@ -45,7 +62,7 @@ struct Plan {
     uint32_t quad_word_b = 0, quad_cnt_b = 0;
     int quad_nb[5] = {0};          // blocks per SM with 64 << k threads
     int quad_forced = 0;           // threads per sequence the caller asked for
-    // small graphs, large batches: a lane per sequence, walked backwards (null: the graph or a forced kind rules it out)
+    // small graphs, large batches: a lane per sequence, walked backwards (null: another kernel)
     LiveFn live_fn = nullptr;
     const uint32_t* live_image = nullptr;
     // sequence-per-lane path for C <= 2: a block keeps a group of 8, 16 or 32 sequences on chip
@@ -143,6 +160,7 @@ struct moc_graph {
     // grow-only scratch; mutable because evaluation takes a const handle
     mutable moc_host::Plan plan_eval, plan_profile;
     mutable moc_host::Plan plan_block;    // block-per-sequence kernel beside the warp-per-sequence one in plan_eval
+    mutable moc_host::Plan plan_live;     // backward walk beside either
     mutable int64_t* d_offs = nullptr;
     mutable size_t offs_cap = 0;
     mutable char* d_state = nullptr;

@@ -27,7 +27,7 @@ bool launch_plain(const moc_graph* g, const moc::IntervalParams& q, bool fill, c
     p.fill = fill;
     const size_t warp_b = 2 * ((size_t)p.word_bytes + moc::kPairWordTail) + p.event_bytes, graph_b = (size_t)p.rec_bytes + p.sell_bytes;
     if (graph_b + 4 * warp_b > g->smem_optin) return false;
-    const void* fn = wide ? (const void*)moc::check_plain_kernel<int64_t> : (const void*)moc::check_plain_kernel<int32_t>;
+    const void* fn = check_plain_fn(wide);
     *err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g->smem_optin);
     if (*err != cudaSuccess) return true;
     // one block per SM; warps: the rounds a full block needs, evenly filled, at least eight to stage the graph
@@ -104,19 +104,8 @@ int check_intervals(const moc_graph* g, const int32_t* s, const int32_t* e, cons
     }
     if (fill && out_seqs) MOC_CUDA(cudaMemsetAsync(out_seqs, 0xFF, (size_t)B * (size_t)K * 4, (cudaStream_t)stream));
     const size_t smem = warp_b * wpb;
-    using Fn = void (*)(const moc::IntervalParams);
-    const int cp = g->C <= 2 ? 2 : (g->C <= 4 ? 4 : 8);
-    const bool narrow = D < 65536;
-    Fn table[2][3][2][3] = {
-#define MOC_IV_ROW(PL, CPV) {{(Fn)moc::check_intervals_kernel<PL, CPV, int32_t, false, int32_t>, (Fn)moc::check_intervals_kernel<PL, CPV, int32_t, true, int32_t>, \
-                             (Fn)moc::check_intervals_kernel<PL, CPV, int32_t, true, uint16_t>},                                                            \
-                            {(Fn)moc::check_intervals_kernel<PL, CPV, int64_t, false, int32_t>, (Fn)moc::check_intervals_kernel<PL, CPV, int64_t, true, int32_t>, \
-                             (Fn)moc::check_intervals_kernel<PL, CPV, int64_t, true, uint16_t>}}
-        {MOC_IV_ROW(false, 2), MOC_IV_ROW(false, 4), MOC_IV_ROW(false, 8)},
-        {MOC_IV_ROW(true, 2), MOC_IV_ROW(true, 4), MOC_IV_ROW(true, 8)}
-#undef MOC_IV_ROW
-    };
-    Fn fn = table[plain ? 1 : 0][cp == 2 ? 0 : (cp == 4 ? 1 : 2)][wide ? 1 : 0][stage ? (narrow ? 2 : 1) : 0];
+    const int cp = g->C <= 2 ? 2 : (g->C <= 4 ? 4 : 8), kept = !stage ? 0 : (D < 65536 ? 2 : 4);      // bytes per kept event
+    const IntervalFn fn = plain ? check_general_fn(cp, wide, kept) : check_staged_fn(cp, wide, kept);
     MOC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
     int nb = 0;
     MOC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, 32 * wpb, smem));

@@ -71,8 +71,7 @@ bool plan_fused(moc_search* s) {
     int best = 0;
     for (int chip = 1; chip >= 0; --chip) {
         if (chip && (g->n > 65535 || graph_b > cap / 4)) continue;
-        s->score_fn = chip ? (h->wide ? (const void*)moc::search_score_kernel<int64_t, true> : (const void*)moc::search_score_kernel<int32_t, true>)
-                           : (h->wide ? (const void*)moc::search_score_kernel<int64_t, false> : (const void*)moc::search_score_kernel<int32_t, false>);
+        s->score_fn = score_fn(h->wide, chip != 0);
         if (cudaFuncSetAttribute(s->score_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g->smem_optin - 1024)) != cudaSuccess) {
             cudaGetLastError();
             return false;
@@ -124,7 +123,7 @@ void plan_walk(moc_search* s) {
     w.word_bytes = (4u * ((uint32_t)g->n + 2u) + 15u) & ~15u;
     w.delta_bytes = (uint32_t)(moc::kPairDeltaFront + 32 * v_max * 16);
     const size_t warp_b = moc::walk_warp_bytes(w.word_bytes, w.delta_bytes), graph_b = (size_t)w.rec_bytes + w.sell_bytes;
-    const void* fn = wide ? (const void*)moc::search_walk_kernel<int64_t> : (const void*)moc::search_walk_kernel<int32_t>;
+    const void* fn = walk_fn(wide);
     const size_t cap = g->smem_optin;
     if (graph_b + 4 * warp_b > cap) return;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {

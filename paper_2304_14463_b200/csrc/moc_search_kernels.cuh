@@ -185,7 +185,7 @@ struct SearchIncParams {
 };
 
 // One thread per proposal: proposal e of chain c draws Philox4x32-10 with counter (generation, chain0 + c, e, 0).
-__global__ void __launch_bounds__(256) search_draw_kernel(const SearchIncParams p) {
+static __global__ void __launch_bounds__(256) search_draw_kernel(const SearchIncParams p) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) *p.todo_count = 0;
     if (t >= (int64_t)p.s.P * p.samples) return;
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(256) search_draw_kernel(const SearchIncParams 
 // One warp per chain: the best proposal of the chain (smallest key among status >= 0, lowest sample
 // among equals) replaces the chain's sequence when it is not worse; its row is written to the chain's
 // other row, and the chain is listed for the rebuild of its cache entry.
-__global__ void __launch_bounds__(kSearchThreads) search_pick_kernel(const SearchIncParams p) {
+static __global__ void __launch_bounds__(kSearchThreads) search_pick_kernel(const SearchIncParams p) {
     const SearchParams& s = p.s;
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * (kSearchThreads / 32) + (threadIdx.x >> 5);
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_pick_kernel(const Searc
 }
 
 // Offsets of the chains' current rows, for the build of the whole cache.
-__global__ void search_row_offsets_kernel(const SearchIncParams p) {
+static __global__ void search_row_offsets_kernel(const SearchIncParams p) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < p.s.P) p.row_offs[c] = ((int64_t)p.s.cur[c] * p.s.P + c) * p.s.stride;
     if (c == 0) p.row_offs[p.s.P] = (int64_t)2 * p.s.P * p.s.stride;
@@ -259,7 +259,7 @@ __global__ void search_row_offsets_kernel(const SearchIncParams p) {
 // Start of a search: packed sequences (offs = exclusive prefix sum of the lengths) become rows
 // 0..P-1; every chain starts in row set 0 with no accepted proposal.  A length outside [0, C*n]
 // sets *bad_len (and is clamped, so that nothing is written outside a row).  One warp per chain.
-__global__ void __launch_bounds__(kSearchThreads) search_init_kernel(const SearchParams p, const int32_t* __restrict__ seqs,
+static __global__ void __launch_bounds__(kSearchThreads) search_init_kernel(const SearchParams p, const int32_t* __restrict__ seqs,
                                                                      const int32_t* __restrict__ in_lens,
                                                                      const int64_t* __restrict__ offs,
                                                                      int32_t* __restrict__ bad_len) {
@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_init_kernel(const Searc
 }
 
 // Row offsets of the chains' current sequences (used to score the initial population).
-__global__ void search_offsets_kernel(const SearchParams p) {
+static __global__ void search_offsets_kernel(const SearchParams p) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < p.P) p.c_offs[c] = ((int64_t)p.cur[c] * p.P + c) * p.stride;
     if (c == 0) p.c_offs[p.P] = (int64_t)2 * p.P * p.stride;
@@ -289,7 +289,7 @@ __global__ void search_offsets_kernel(const SearchParams p) {
 // row's length are left alone, or zeroed with `fill`, in the same pass: the caller need not clear 4 * P * stride
 // bytes first) and the evaluations.  Any output may be null.  One warp per chain; 16-byte accesses (rows start
 // on 16-byte boundaries when out_rows does).
-__global__ void __launch_bounds__(kSearchThreads) search_export_kernel(const SearchParams p, int32_t* __restrict__ out_rows, bool fill,
+static __global__ void __launch_bounds__(kSearchThreads) search_export_kernel(const SearchParams p, int32_t* __restrict__ out_rows, bool fill,
                                                                        int32_t* __restrict__ out_lens, int64_t* __restrict__ out_peak,
                                                                        int64_t* __restrict__ out_dur, int32_t* __restrict__ out_status,
                                                                        int32_t* __restrict__ out_acc) {
@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(kSearchThreads) search_export_kernel(const Sea
 // index among equals.  One block.  out_best: index (-1: no valid chain), length, peak, duration,
 // status, total number of accepted proposals; out_seq (may be null) receives the sequence.
 constexpr int kBestThreads = 1024;
-__global__ void __launch_bounds__(kBestThreads) search_best_kernel(const SearchParams p, int32_t* __restrict__ out_seq,
+static __global__ void __launch_bounds__(kBestThreads) search_best_kernel(const SearchParams p, int32_t* __restrict__ out_seq,
                                                                    int64_t* __restrict__ out_best) {
     __shared__ int64_t s_a[kBestThreads / 32], s_d[kBestThreads / 32], s_acc[kBestThreads / 32];
     __shared__ int32_t s_i[kBestThreads / 32];

@@ -169,6 +169,9 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* nb, const void* f
     *nb = (int)std::min<size_t>(std::min<size_t>(by_smem, by_regs), 32);
     return cudaSuccess;
 }
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* nb, const void* fn, int threads, size_t smem, unsigned) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, threads, smem);
+}
 cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void**, size_t, cudaStream_t st) {
     note("launch " + name_of(fn));
     if (fails()) return cudaErrorUnknown;
@@ -226,11 +229,23 @@ cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* sm, void* st) {
     *(void**)st = g_stream;
     return cudaSuccess;
 }
+// every source file registers a module, and then its kernels with it
+static std::map<void*, std::string>& modules() {
+    static std::map<void*, std::string> m;
+    return m;
+}
 void** __cudaRegisterFatBinary(void*) { return (void**)calloc(1, sizeof(void*)); }
+const char* fake_modules() {
+    static std::string all;
+    all.clear();
+    for (auto& m : modules()) all += m.second + "\n";
+    return all.c_str();
+}
 void __cudaRegisterFatBinaryEnd(void**) {}
 char __cudaInitModule(void**) { return 1; }
 void __cudaUnregisterFatBinary(void** h) { free(h); }
-void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, void*, void*, void*, void*, int*) {
+void __cudaRegisterFunction(void** module, const char* host, char*, const char* name, int, void*, void*, void*, void*, int*) {
+    modules()[module] += std::string(name) + " ";
     names()[host] = name;
 }
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}

@@ -1,4 +1,4 @@
-"""The host side of the library (moc_api.cu) on a stand-in for the CUDA runtime (fake_cudart.cpp): which kernels are
+"""The host side of the library on a stand-in for the CUDA runtime (fake_cudart.cpp): which kernels are
 looked up and launched, what is copied, and what an error leaves behind.  Runs without a GPU; no kernel runs."""
 import ctypes
 import os
@@ -20,10 +20,10 @@ def fake(tmp_path_factory):
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     # no machine code and no optimisation of the kernels: they are never run
     subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=compute_100a", "-Xcicc", "-O0", "-std=c++17", "-cudart", "none", "-shared",
-                    "-Xcompiler", "-fPIC", "-Xlinker", "-Bsymbolic,--no-undefined", "-t", "2", "-o", lib,
-                    os.path.join(build.CSRC, "moc_api.cu"), os.path.join(HERE, "fake_cudart.cpp")], check=True)
+                    "-Xcompiler", "-fPIC", "-Xlinker", "-Bsymbolic,--no-undefined", "-t", "8", "-o", lib,
+                    *[os.path.join(build.CSRC, f) for f in build.SOURCES], os.path.join(HERE, "fake_cudart.cpp")], check=True)
     L = ctypes.CDLL(lib)
-    L.fake_log.restype = ctypes.c_char_p
+    L.fake_log.restype = L.fake_modules.restype = ctypes.c_char_p
     L.fake_pin.argtypes = [P, ctypes.c_size_t]
     L.moc_last_error.restype = ctypes.c_char_p
     L.moc_graph_create.argtypes = [i32, i64, P, P, P, ctypes.POINTER(P)]
@@ -195,3 +195,37 @@ def test_lengths_that_lie(fake):
             assert b.run(G) == 0 and fake.fake_in_flight() == 0
             assert len(launched(fake, "eval_")) == 1
         G.close()
+
+
+@pytest.mark.parametrize("n,C,scale,nB,kernel", [(20, 2, 1, 64, "eval_pair"), (20, 2, 1, 60000, "eval_live"), (100, 2, 1 << 30, 64, "eval_pair"),
+                                                 (100, 3, 1, 64, "eval_quad"), (100, 4, 1, 60000, "eval_live"), (100, 5, 1, 64, "eval_shared"),
+                                                 (442, 2, 1, 64, "eval_quad"), (442, 2, 1, 5000, "eval_pair"), (442, 3, 1, 5000, "eval_quad")])
+def test_only_kernels_that_run_are_looked_up(fake, n, C, scale, nB, kernel):
+    """A first evaluation on a handle prepares the kernel it launches and no other; a later one of another size adds its own."""
+    G = Graph(fake, n, C, scale)
+    x = np.zeros(8, np.int64)
+
+    def looked_up(nB):
+        fake.fake_reset(0)
+        assert fake.moc_eval_batch(G.h, x.ctypes.data, x.ctypes.data, nB, 0, x.ctypes.data, x.ctypes.data, x.ctypes.data, None) == 0
+        names = {x.split()[1] for x in log(fake) if x.startswith("lookup ")}
+        run = {x.split()[1] for x in log(fake) if x.startswith("launch ") and "offsets" not in x}
+        return names, run
+
+    names, run = looked_up(nB)
+    assert len(run) == 1 and kernel in next(iter(run)) and names == run
+    assert looked_up(nB) == (set(), run)
+    for other in (1, 200, 3000, 65536):
+        names, run = looked_up(other)
+        assert names <= run
+    G.close()
+
+
+def test_kernel_families_do_not_share_a_module(fake):
+    """The first use of a kernel loads the whole module it lies in."""
+    families = ["eval_pair_kernel", "eval_quad_kernel", "eval_live_kernel", "eval_lane_kernel", "eval_shared_kernel", "check_plain_kernel",
+                "check_intervals_kernelILb0E", "check_intervals_kernelILb1E", "search_score_kernel", "search_walk_kernel", "edit_prepare_kernel"]
+    modules = fake.fake_modules().decode().splitlines()
+    for f in families:
+        assert sum(f in m for m in modules) == 1, f
+    assert all(sum(f in m for f in families) <= 1 for m in modules)
