@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -346,12 +347,55 @@ int ensure(void** ptr, size_t* cap, size_t need) {
 }
 
 
+// The arrays of a handle, gathered for one allocation and, unless they are large, one copy, so that a further table
+// costs a new handle its bytes and no calls.  Creating a handle of n = 20, 100, 442, 1000: 540, 600, 690 and 900 us
+// with an allocation and a copy per array (23 of them at n = 442), 390, 395, 540 and 745 so; freeing it 340 and 275.
+class Tables {
+  public:
+    // A device array for *dst, filled from `src` (alive until upload) or, without one, not at all.
+    template <typename T>
+    void add(T** dst, const void* src, size_t bytes) {
+        parts_.push_back({(void**)dst, src, size_, bytes});
+        size_ += (std::max<size_t>(bytes, 16) + 255) & ~size_t(255);
+    }
+    template <typename T, typename V>
+    void add(T** dst, std::vector<V>&& v) {
+        auto kept = std::make_shared<std::vector<V>>(std::move(v));
+        keep_.push_back(kept);
+        add(dst, kept->data(), kept->size() * sizeof(V));
+    }
+    cudaError_t upload(char** block) {
+        cudaError_t e = cudaMalloc((void**)block, size_);
+        if (e != cudaSuccess) return e;
+        for (const Part& p : parts_) *p.dst = *block + p.at;
+        if (size_ <= kTogether) {
+            std::vector<char> all(size_);
+            for (const Part& p : parts_)
+                if (p.src) memcpy(all.data() + p.at, p.src, p.bytes);
+            return cudaMemcpy(*block, all.data(), size_, cudaMemcpyHostToDevice);
+        }
+        for (const Part& p : parts_)
+            if (p.src && p.bytes && e == cudaSuccess) e = cudaMemcpy(*p.dst, p.src, p.bytes, cudaMemcpyHostToDevice);
+        return e;
+    }
+
+  private:
+    static constexpr size_t kTogether = 1 << 20;       // up to here a second copy on the host costs less than the calls
+    struct Part {
+        void** dst;
+        const void* src;
+        size_t at, bytes;
+    };
+    std::vector<Part> parts_;
+    std::vector<std::shared_ptr<void>> keep_;
+    size_t size_ = 0;
+};
+
 // Words 4-5 of the node records of the sequence-per-lane layouts: w | 1 << 40 (counts the node when
-// it has two copies) | 1 << 52 when the node's cap C_v is 1.  Uploads both record arrays.
-int upload_lane_rec(moc_graph* g) {
+// it has two copies) | 1 << 52 when the node's cap C_v is 1.
+void set_lane_caps(moc_graph* g) {
     for (int li = 0; li < 3; ++li) {
         LaneLayout& L = g->lane[li];
-        if (!L.ok) continue;
         for (size_t r = 0; r < L.h_node.size(); ++r) {
             const int32_t v = L.h_node[r];
             uint64_t x = 0;
@@ -362,25 +406,38 @@ int upload_lane_rec(moc_graph* g) {
             L.h_rec32[8 * r + 4] = L.h_rec64[8 * r + 4] = (uint32_t)(x & 0xFFFFFFFFu);
             L.h_rec32[8 * r + 5] = L.h_rec64[8 * r + 5] = (uint32_t)(x >> 32);
         }
-        MOC_CUDA(cudaMemcpy(L.d_rec32, L.h_rec32.data(), L.h_rec32.size() * 4, cudaMemcpyHostToDevice));
-        MOC_CUDA(cudaMemcpy(L.d_rec64, L.h_rec64.data(), L.h_rec64.size() * 4, cudaMemcpyHostToDevice));
     }
-    return MOC_OK;
+}
+
+// Durations by slot of the warp-per-sequence layout: w | 1 << 48 (counts the node when it has two copies) | 1 << 63
+// for nodes whose cap C_v is 1.
+std::vector<uint64_t> slot_durations(const moc_graph* g) {
+    std::vector<uint64_t> wslot(g->h_slot.size());
+    for (size_t r = 0; r < wslot.size(); ++r) {
+        const int32_t v = g->h_slot[r];
+        uint64_t x = 0;
+        if (v >= 0) {
+            x = (uint64_t)g->h_w[v] | (uint64_t(1) << moc::kPairCntShift);
+            if (!g->h_cap.empty() && g->h_cap[v] == 1) x |= uint64_t(1) << 63;
+        }
+        wslot[r] = x;
+    }
+    return wslot;
 }
 
 // Layouts for the sequence-per-lane kernel, one per group size g = 32, 16, 8 (S = 1, 2, 4 sub-lanes).
 // Nodes in order of falling out-degree (a sink counts one: its made-up successor), S consecutive
 // nodes form a bundle and share a row count; entry (k, h) of a bundle is the byte offset of the
 // word row of the k-th successor of its h-th node, the node's own row once its list is used up.
-int build_lane_layouts(moc_graph* g, const std::vector<int32_t>& succ_start, const std::vector<int32_t>& succ,
-                       const int64_t* m, const std::vector<int32_t>& m32) {
+void build_lane_layouts(moc_graph* g, const std::vector<int32_t>& succ_start, const std::vector<int32_t>& succ,
+                        const int64_t* m, const std::vector<int32_t>& m32, Tables* tables) {
     const int32_t n = g->n;
-    if (n >= 4096) return MOC_OK;                       // the count of two-copy nodes has 12 bits
+    if (n >= 4096) return;                              // the count of two-copy nodes has 12 bits
     auto deg = [&](int32_t v) { return std::max(1, succ_start[v + 1] - succ_start[v]); };
     std::vector<int32_t> order((size_t)n);
     for (int32_t v = 0; v < n; ++v) order[v] = v;
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return deg(x) > deg(y); });
-    if (deg(order[0]) > 255) return MOC_OK;
+    if (deg(order[0]) > 255) return;
     for (int li = 0; li < 3; ++li) {
         const int lg = 5 - li, gsz = 1 << lg, S = 32 >> lg;
         LaneLayout& L = g->lane[li];
@@ -423,33 +480,30 @@ int build_lane_layouts(moc_graph* g, const std::vector<int32_t>& succ_start, con
         while (se.size() % 4) se.push_back(one_row);
         if (se.empty()) se.assign(4, one_row);
         if (se.size() * 4 + 64 >= (size_t(1) << 24)) continue;
-        cudaError_t e = cudaMalloc(&L.d_rec32, rec32.size() * 4);
-        if (e == cudaSuccess) e = cudaMalloc(&L.d_rec64, rec64.size() * 4);
-        if (e == cudaSuccess) e = cudaMalloc((void**)&L.d_succ, se.size() * 4);
-        if (e == cudaSuccess) e = cudaMemcpy(L.d_succ, se.data(), se.size() * 4, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess)
-            return fail(e == cudaErrorMemoryAllocation ? MOC_ERR_NOMEM : MOC_ERR_CUDA, "moc_graph_create: %s", cudaGetErrorString(e));
         L.n_bundles = nb;
         L.succ_len = (int64_t)se.size();
-        L.h_node = node;
-        L.h_rec32 = rec32;
-        L.h_rec64 = rec64;
+        L.h_node = std::move(node);
+        L.h_rec32 = std::move(rec32);
+        L.h_rec64 = std::move(rec64);
         L.ok = true;
+        tables->add(&L.d_rec32, L.h_rec32.data(), L.h_rec32.size() * 4);       // the handle's copies: complete before they are sent
+        tables->add(&L.d_rec64, L.h_rec64.data(), L.h_rec64.size() * 4);
+        tables->add(&L.d_succ, std::move(se));
     }
-    return upload_lane_rec(g);
+    set_lane_caps(g);
 }
 
 // Layout for the block-per-sequence kernel on graphs without successor tiles: the nodes in order of falling
 // out-degree (a sink counts one: its made-up successor n + 1) with the place of their successor lists, and the
 // lists as 16-bit ids.
-int build_quad_layout(moc_graph* g, const std::vector<int32_t>& succ_start, const std::vector<int32_t>& succ) {
+void build_quad_layout(moc_graph* g, const std::vector<int32_t>& succ_start, const std::vector<int32_t>& succ, Tables* tables) {
     const int32_t n = g->n;
-    if (g->d_rec32 || n > 32000) return MOC_OK;
+    if (g->n_tiles || n > 32000) return;
     auto deg = [&](int32_t v) { return std::max(1, succ_start[v + 1] - succ_start[v]); };
     std::vector<int32_t> order((size_t)n);
     for (int32_t v = 0; v < n; ++v) order[v] = v;
     std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return deg(x) > deg(y); });
-    if (deg(order[0]) > 65535) return MOC_OK;
+    if (deg(order[0]) > 65535) return;
     std::vector<uint32_t> rec((size_t)n * 8, 0u);
     std::vector<uint16_t> rest;
     for (int32_t i = 0; i < n; ++i) {
@@ -465,11 +519,186 @@ int build_quad_layout(moc_graph* g, const std::vector<int32_t>& succ_start, cons
             else rest.push_back(ids[k]);
         }
     }
-    MOC_CUDA(cudaMalloc((void**)&g->d_order, rec.size() * 4));
-    MOC_CUDA(cudaMemcpy(g->d_order, rec.data(), rec.size() * 4, cudaMemcpyHostToDevice));
-    MOC_CUDA(cudaMalloc((void**)&g->d_succ16, std::max<size_t>(rest.size() * 2, 16)));
-    if (!rest.empty()) MOC_CUDA(cudaMemcpy(g->d_succ16, rest.data(), rest.size() * 2, cudaMemcpyHostToDevice));
-    return MOC_OK;
+    tables->add(&g->d_order, std::move(rec));
+    tables->add(&g->d_succ16, std::move(rest));
+}
+
+// The arrays that the kernels read of a graph: `keys` are its edges (u << 32 | v) in order, grouped by u in succ_start and succ;
+// m32 is m cut to 32 bits.  What is not moved into `tables` outlives the upload.
+void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::vector<int32_t>& succ_start, const std::vector<int32_t>& succ,
+                  const int64_t* w, const int64_t* m, const std::vector<int32_t>& m32, Tables* tables) {
+    const int32_t n = g->n;
+    const int64_t ne = g->n_edges;
+    tables->add(&g->d_succ_start, succ_start.data(), ((size_t)n + 1) * 4);
+    tables->add(&g->d_succ, succ.data(), (size_t)ne * 4);
+    {
+        // predecessor lists (grouped by consumer) and the total output size of the sinks
+        std::vector<int32_t> pred_start((size_t)n + 1, 0), pred((size_t)ne);
+        for (int64_t k = 0; k < ne; ++k) pred_start[(keys[k] & 0xFFFFFFFFu) + 1]++;
+        for (int32_t v = 0; v < n; ++v) g->max_indeg = std::max(g->max_indeg, pred_start[v + 1]);
+        for (int32_t v = 0; v < n; ++v) pred_start[v + 1] += pred_start[v];
+        std::vector<int32_t> fill(pred_start.begin(), pred_start.end() - 1);
+        for (int64_t k = 0; k < ne; ++k) pred[fill[keys[k] & 0xFFFFFFFFu]++] = (int32_t)(keys[k] >> 32);
+        for (int32_t v = 0; v < n; ++v)
+            if (succ_start[v + 1] == succ_start[v]) g->sink_m += m[v];
+        tables->add(&g->d_pred_start, std::move(pred_start));
+        tables->add(&g->d_pred, std::move(pred));
+    }
+    if (n <= moc::kLiveMaxN) {
+        // The nodes are dealt to the mask words so that the predecessors of a node lie in different words where
+        // possible (moc_live_kernel.cuh): each node, most consumers first, goes to the word with the fewest other
+        // predecessors of its consumers.
+        const int words = live_words(n);
+        std::vector<uint32_t> preds((size_t)n * words, 0u);
+        std::vector<int32_t> order((size_t)n), clash((size_t)n * words, 0), fill((size_t)words, 0);
+        for (int32_t v = 0; v < n; ++v) order[v] = v;
+        std::stable_sort(order.begin(), order.end(),
+                         [&](int32_t x, int32_t y) { return succ_start[x + 1] - succ_start[x] > succ_start[y + 1] - succ_start[y]; });
+        g->h_live_place.assign((size_t)n, 0);
+        for (int32_t u : order) {
+            int best = -1, best_clash = 0;
+            for (int k = 0; k < words; ++k) {
+                int c = 0;
+                for (int32_t e = succ_start[u]; e < succ_start[u + 1]; ++e) c += clash[(size_t)succ[e] * words + k];
+                c += clash[(size_t)u * words + k];          // the node counts among its predecessors
+                if (fill[k] < 32 && (best < 0 || c < best_clash || (c == best_clash && fill[k] < fill[best]))) { best = k; best_clash = c; }
+            }
+            for (int32_t e = succ_start[u]; e < succ_start[u + 1]; ++e) {
+                ++clash[(size_t)succ[e] * words + best];
+                preds[(size_t)succ[e] * words + best] |= 1u << fill[best];
+            }
+            ++clash[(size_t)u * words + best];
+            if (succ_start[u + 1] == succ_start[u]) g->live_sinks[best] |= 1u << fill[best];
+            g->h_live_place[u] = best << 5 | fill[best]++;
+        }
+        // tables for both widths, or the one that every C <= MOC_MAX_COPIES selects
+        const bool narrow = g->sum_m <= INT32_MAX / MOC_MAX_COPIES && g->sum_w <= INT32_MAX / MOC_MAX_COPIES;
+        for (int wide = 0; wide < (narrow ? 1 : 2); ++wide)
+            tables->add(wide ? &g->d_live64 : &g->d_live32, moc::live_image(n, words, wide != 0, g->h_live_place, preds, m, w));
+    }
+    tables->add(&g->d_w, w, (size_t)n * 8);
+    tables->add(&g->d_m64, m, (size_t)n * 8);
+    tables->add(&g->d_m32, m32.data(), (size_t)n * 4);
+    {
+        // 64-bit sums: parts of m that 32-bit atomics can add (moc_pair_kernel.cuh), where sum(m) permits; with room for
+        // two amounts per node at a time (the interval checker adds up intervals that may overlap)
+        int k = 30;
+        while (k > 0 && ((int64_t)1 << (30 - k)) < n) --k;
+        g->split_ok = (g->sum_m >> k) < ((int64_t)1 << 30);
+        g->split = g->split_ok ? k : 32;
+    }
+    if (n <= 16000) {
+        // Layout for the warp-per-sequence kernel.  Lane l serves the nodes with id = l (mod 32);
+        // each residue class is sorted by out-degree (descending, ties by id); half j holds the
+        // j-th node of every class, a tile is two halves.  A tile stores, row by row, the word
+        // offsets (4 * id) of its nodes' successors, two halves packed per 32-bit entry, padded with
+        // the offset of a dummy word (4 * n).  Within a half the order of each node's successors
+        // is chosen greedily so that the 32 words a row touches fall in different banks where
+        // possible.  Skipped when padding would more than double the storage (a few very high
+        // degrees): such graphs use the general kernel.
+        auto deg = [&](int32_t v) { return succ_start[v + 1] - succ_start[v]; };
+        const int32_t n_halves = 2 * ((n + 63) / 64), n_tiles = n_halves / 2;
+        std::vector<int32_t> slot((size_t)n_halves * 32, -1);  // node at (half, lane) or -1
+        for (int32_t l = 0; l < 32; ++l) {
+            std::vector<int32_t> cls;
+            for (int32_t v = l; v < n; v += 32) cls.push_back(v);
+            std::stable_sort(cls.begin(), cls.end(), [&](int32_t x, int32_t y) { return deg(x) > deg(y); });
+            for (size_t j = 0; j < cls.size(); ++j) slot[j * 32 + l] = cls[j];
+        }
+        std::vector<int32_t> rows((size_t)n_tiles, 0);
+        int64_t sell_len = 0;
+        for (int32_t d = 0; d < n_tiles; ++d) {
+            for (int32_t s = 0; s < 64; ++s)
+                if (slot[(size_t)d * 64 + s] >= 0)
+                    rows[d] = std::max(rows[d], std::max(1, deg(slot[(size_t)d * 64 + s])));  // a sink gets one entry
+            sell_len += 32 * (int64_t)rows[d];
+        }
+        int32_t max_rows = 0;
+        for (int32_t d = 0; d < n_tiles; ++d) max_rows = std::max(max_rows, rows[d]);
+        if (sell_len <= 2 * ne + 4096 && sell_len < (1 << 20) && max_rows < (1 << 12) && 4 * ((int64_t)n + 3) < 65536) {
+            const uint32_t word_b = (uint32_t)align16(4 * ((size_t)n + 2));   // the constant word (1, 1) sits right after the words
+            std::vector<uint32_t> rec32((size_t)n_halves * 32 * 2), rec64((size_t)n_halves * 32 * 4, 0u);
+            // entry (row k, lane l) of a tile: word of the k-th successor of the node in half 0 | same for half 1 << 16;
+            // a list that is used up continues with the node's own word
+            std::vector<uint32_t> sell((size_t)std::max<int64_t>(sell_len, 1), word_b | (word_b << 16));
+            auto own_word = [&](int32_t v) { return v >= 0 ? 4u * (uint32_t)v : word_b; };
+            for (size_t r = 0; r < slot.size(); ++r) {
+                const int32_t v = slot[r];
+                const uint32_t x = own_word(v) | ((uint32_t)rows[r / 64] << 16);
+                const uint64_t mv = v >= 0 ? (uint64_t)m[v] : 0;
+                rec32[2 * r + 0] = x;
+                rec32[2 * r + 1] = v >= 0 ? (uint32_t)m32[v] : 0u;
+                rec64[4 * r + 0] = x;
+                rec64[4 * r + 2] = (uint32_t)(mv & 0xFFFFFFFFu);
+                rec64[4 * r + 3] = (uint32_t)(mv >> g->split);
+            }
+            uint32_t pos = 0;
+            std::vector<std::vector<int32_t>> rem(32);
+            for (int32_t d = 0; d < n_tiles; ++d) {
+                for (int32_t h = 0; h < 2; ++h) {
+                    std::vector<int32_t> lanes;
+                    for (int32_t l = 0; l < 32; ++l) {
+                        const int32_t v = slot[((size_t)2 * d + h) * 32 + l];
+                        rem[l].clear();
+                        if (v >= 0) rem[l].assign(succ.begin() + succ_start[v], succ.begin() + succ_start[v + 1]);
+                        if (v >= 0 && rem[l].empty()) rem[l].push_back(n + 1);  // sink: the word that holds T
+                        lanes.push_back(l);
+                        for (int32_t k = 0; k < rows[d]; ++k) {
+                            uint32_t& e = sell[(size_t)pos + 32 * (size_t)k + l];
+                            e = h == 0 ? ((e & 0xFFFF0000u) | own_word(v)) : ((e & 0x0000FFFFu) | (own_word(v) << 16));
+                        }
+                    }
+                    for (int32_t k = 0; k < rows[d]; ++k) {
+                        int used[32] = {0};
+                        for (int32_t l = 0; l < 32; ++l)
+                            if (rem[l].empty()) used[l]++;   // reads its own word, which lies in bank l
+                        std::stable_sort(lanes.begin(), lanes.end(),
+                                         [&](int32_t x, int32_t y) { return rem[x].size() > rem[y].size(); });
+                        for (int32_t l : lanes) {
+                            if (rem[l].empty()) continue;  // stays the own word
+                            const bool forced = (int32_t)rem[l].size() >= rows[d] - k;
+                            int pick = -1;
+                            for (size_t c = 0; c < rem[l].size(); ++c)
+                                if (!used[rem[l][c] & 31]) { pick = (int)c; break; }
+                            if (pick < 0 && !forced) continue;  // wait for a row where its bank is free
+                            if (pick < 0) pick = 0;
+                            used[rem[l][pick] & 31]++;
+                            uint32_t& e = sell[(size_t)pos + 32 * (size_t)k + l];
+                            const uint32_t off = 4u * (uint32_t)rem[l][pick];
+                            e = h == 0 ? ((e & 0xFFFF0000u) | off) : ((e & 0x0000FFFFu) | (off << 16));
+                            rem[l].erase(rem[l].begin() + pick);
+                        }
+                    }
+                }
+                pos += 32 * (uint32_t)rows[d];
+            }
+            std::vector<int32_t> tile_row((size_t)n_tiles, 0);
+            for (int32_t d = 1; d < n_tiles; ++d) tile_row[d] = tile_row[d - 1] + rows[d - 1];
+            // the same tiles for the interval checker: its padding repeats a successor, a sink reads its own word
+            std::vector<uint32_t> sell_iv(sell);
+            for (size_t r = 0; r < slot.size(); ++r) {
+                const int32_t v = slot[r];
+                const uint32_t own = own_word(v), pad = v >= 0 && deg(v) > 0 ? 4u * (uint32_t)succ[succ_start[v]] : own;
+                const int sh = (r & 32) ? 16 : 0;
+                for (int32_t k = 0; k < rows[r / 64]; ++k) {
+                    uint32_t& e = sell_iv[32 * (size_t)(tile_row[r / 64] + k) + (r & 31)];
+                    const uint32_t off = e >> sh & 0xFFFFu;
+                    if (off == own || off == 4u * ((uint32_t)n + 1)) e = (e & ~(0xFFFFu << sh)) | pad << sh;
+                }
+            }
+            tables->add(&g->d_sell_iv, std::move(sell_iv));
+            tables->add(&g->d_tile_row, std::move(tile_row));
+            g->sell_len = (int32_t)sell_len;
+            g->h_slot = std::move(slot);
+            g->n_tiles = n_tiles;
+            tables->add(&g->d_rec32, std::move(rec32));
+            tables->add(&g->d_rec64, std::move(rec64));
+            tables->add(&g->d_wslot, slot_durations(g));
+            tables->add(&g->d_sell, std::move(sell));
+        }
+    }
+    build_lane_layouts(g, succ_start, succ, m, m32, tables);
+    build_quad_layout(g, succ_start, succ, tables);
 }
 
 moc::EvalParams base_params(const moc_graph* g, const Plan& pl) {
@@ -761,8 +990,6 @@ int eval_rows(const moc_graph* g, const int64_t* offs, const int32_t* seqs, cons
 
 extern "C" {
 
-static int upload_wslot(moc_graph* g);
-
 const char* moc_last_error(void) { return g_err; }
 int moc_last_launch_count(void) { return g_launches; }
 
@@ -829,235 +1056,30 @@ int moc_graph_create(int32_t n, int64_t n_edges, const int32_t* edges, const int
 
     moc_graph* g = new (std::nothrow) moc_graph();
     if (!g) return fail(MOC_ERR_NOMEM, "host allocation failed");
-    try {
-        g->h_w.assign(w, w + n);
-    } catch (const std::bad_alloc&) {
-        delete g;
-        return fail(MOC_ERR_NOMEM, "host allocation failed");
-    }
     g->n = n;
     g->n_edges = ne;
     g->sum_m = sum_m;
     g->sum_w = sum_w;
-    int rc = MOC_OK;
     cudaError_t e = cudaGetDevice(&g->device);
     int smem = 0;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g->sm_count, cudaDevAttrMultiProcessorCount, g->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, g->device);
     g->smem_optin = (size_t)smem;
-    auto up = [&](void** dst, const void* src, size_t bytes) {
-        if (e != cudaSuccess) return;
-        e = cudaMalloc(dst, std::max<size_t>(bytes, 16));
-        if (e == cudaSuccess && bytes && src) e = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
-    };
-    up((void**)&g->d_succ_start, succ_start.data(), ((size_t)n + 1) * 4);
-    up((void**)&g->d_succ, succ.data(), (size_t)ne * 4);
-    {
-        // predecessor lists (grouped by consumer) and the total output size of the sinks
-        std::vector<int32_t> pred_start, pred;
-        try {
-            pred_start.assign((size_t)n + 1, 0);
-            pred.resize((size_t)std::max<int64_t>(ne, 1));
-            for (int64_t k = 0; k < ne; ++k) pred_start[(keys[k] & 0xFFFFFFFFu) + 1]++;
-            for (int32_t v = 0; v < n; ++v) g->max_indeg = std::max(g->max_indeg, pred_start[v + 1]);
-            for (int32_t v = 0; v < n; ++v) pred_start[v + 1] += pred_start[v];
-            std::vector<int32_t> fill(pred_start.begin(), pred_start.end() - 1);
-            for (int64_t k = 0; k < ne; ++k) pred[fill[keys[k] & 0xFFFFFFFFu]++] = (int32_t)(keys[k] >> 32);
-        } catch (const std::bad_alloc&) {
-            moc_graph_destroy(g);
-            return fail(MOC_ERR_NOMEM, "host allocation failed");
-        }
-        for (int32_t v = 0; v < n; ++v)
-            if (succ_start[v + 1] == succ_start[v]) g->sink_m += m[v];
-        up((void**)&g->d_pred_start, pred_start.data(), ((size_t)n + 1) * 4);
-        up((void**)&g->d_pred, pred.data(), (size_t)ne * 4);
-    }
-    if (n <= moc::kLiveMaxN) {
-        // The nodes are dealt to the mask words so that the predecessors of a node lie in different words where
-        // possible (moc_live_kernel.cuh): each node, most consumers first, goes to the word with the fewest other
-        // predecessors of its consumers.
-        const int words = live_words(n);
-        std::vector<uint32_t> preds;
-        try {
-            preds.assign((size_t)n * words, 0u);
-                        std::vector<int32_t> order((size_t)n), clash((size_t)n * words, 0), fill((size_t)words, 0);
-            for (int32_t v = 0; v < n; ++v) order[v] = v;
-            std::stable_sort(order.begin(), order.end(),
-                             [&](int32_t x, int32_t y) { return succ_start[x + 1] - succ_start[x] > succ_start[y + 1] - succ_start[y]; });
-            g->h_live_place.assign((size_t)n, 0);
-            for (int32_t u : order) {
-                int best = -1, best_clash = 0;
-                for (int k = 0; k < words; ++k) {
-                    int c = 0;
-                    for (int32_t e = succ_start[u]; e < succ_start[u + 1]; ++e) c += clash[(size_t)succ[e] * words + k];
-                    c += clash[(size_t)u * words + k];          // the node counts among its predecessors
-                    if (fill[k] < 32 && (best < 0 || c < best_clash || (c == best_clash && fill[k] < fill[best]))) { best = k; best_clash = c; }
-                }
-                for (int32_t e = succ_start[u]; e < succ_start[u + 1]; ++e) {
-                    ++clash[(size_t)succ[e] * words + best];
-                    preds[(size_t)succ[e] * words + best] |= 1u << fill[best];
-                }
-                ++clash[(size_t)u * words + best];
-                if (succ_start[u + 1] == succ_start[u]) g->live_sinks[best] |= 1u << fill[best];
-                g->h_live_place[u] = best << 5 | fill[best]++;
-            }
-        } catch (const std::bad_alloc&) {
-            moc_graph_destroy(g);
-            return fail(MOC_ERR_NOMEM, "host allocation failed");
-        }
-        // tables for both widths, or the one that every C <= MOC_MAX_COPIES selects
-        const bool narrow = sum_m <= INT32_MAX / MOC_MAX_COPIES && sum_w <= INT32_MAX / MOC_MAX_COPIES;
-        for (int wide = 0; wide < (narrow ? 1 : 2); ++wide) {
-            try {
-                const std::vector<uint32_t> image = moc::live_image(n, words, wide != 0, g->h_live_place, preds, m, w);
-                up((void**)(wide ? &g->d_live64 : &g->d_live32), image.data(), image.size() * 4);
-            } catch (const std::bad_alloc&) {
-                moc_graph_destroy(g);
-                return fail(MOC_ERR_NOMEM, "host allocation failed");
-            }
-        }
-    }
-    up((void**)&g->d_w, w, (size_t)n * 8);
-    up((void**)&g->d_m64, m, (size_t)n * 8);
-    up((void**)&g->d_m32, m32.data(), (size_t)n * 4);
-    {
-        // 64-bit sums: parts of m that 32-bit atomics can add (moc_pair_kernel.cuh), where sum(m) permits; with room for
-        // two amounts per node at a time (the interval checker adds up intervals that may overlap)
-        int k = 30;
-        while (k > 0 && ((int64_t)1 << (30 - k)) < n) --k;
-        g->split_ok = (sum_m >> k) < ((int64_t)1 << 30);
-        g->split = g->split_ok ? k : 32;
-    }
-    if (n <= 16000) {
-        // Layout for the warp-per-sequence kernel.  Lane l serves the nodes with id = l (mod 32);
-        // each residue class is sorted by out-degree (descending, ties by id); half j holds the
-        // j-th node of every class, a tile is two halves.  A tile stores, row by row, the word
-        // offsets (4 * id) of its nodes' successors, two halves packed per 32-bit entry, padded with
-        // the offset of a dummy word (4 * n).  Within a half the order of each node's successors
-        // is chosen greedily so that the 32 words a row touches fall in different banks where
-        // possible.  Skipped when padding would more than double the storage (a few very high
-        // degrees): such graphs use the general kernel.
-        try {
-            auto deg = [&](int32_t v) { return succ_start[v + 1] - succ_start[v]; };
-            const int32_t n_halves = 2 * ((n + 63) / 64), n_tiles = n_halves / 2;
-            std::vector<int32_t> slot((size_t)n_halves * 32, -1);  // node at (half, lane) or -1
-            for (int32_t l = 0; l < 32; ++l) {
-                std::vector<int32_t> cls;
-                for (int32_t v = l; v < n; v += 32) cls.push_back(v);
-                std::stable_sort(cls.begin(), cls.end(), [&](int32_t x, int32_t y) { return deg(x) > deg(y); });
-                for (size_t j = 0; j < cls.size(); ++j) slot[j * 32 + l] = cls[j];
-            }
-            std::vector<int32_t> rows((size_t)n_tiles, 0);
-            int64_t sell_len = 0;
-            for (int32_t d = 0; d < n_tiles; ++d) {
-                for (int32_t s = 0; s < 64; ++s)
-                    if (slot[(size_t)d * 64 + s] >= 0)
-                        rows[d] = std::max(rows[d], std::max(1, deg(slot[(size_t)d * 64 + s])));  // a sink gets one entry
-                sell_len += 32 * (int64_t)rows[d];
-            }
-            int32_t max_rows = 0;
-            for (int32_t d = 0; d < n_tiles; ++d) max_rows = std::max(max_rows, rows[d]);
-            if (sell_len <= 2 * ne + 4096 && sell_len < (1 << 20) && max_rows < (1 << 12) && 4 * ((int64_t)n + 3) < 65536) {
-                const uint32_t word_b = (uint32_t)align16(4 * ((size_t)n + 2));   // the constant word (1, 1) sits right after the words
-                std::vector<uint32_t> rec32((size_t)n_halves * 32 * 2), rec64((size_t)n_halves * 32 * 4, 0u);
-                // entry (row k, lane l) of a tile: word of the k-th successor of the node in half 0 | same for half 1 << 16;
-                // a list that is used up continues with the node's own word
-                std::vector<uint32_t> sell((size_t)std::max<int64_t>(sell_len, 1), word_b | (word_b << 16));
-                auto own_word = [&](int32_t v) { return v >= 0 ? 4u * (uint32_t)v : word_b; };
-                for (size_t r = 0; r < slot.size(); ++r) {
-                    const int32_t v = slot[r];
-                    const uint32_t x = own_word(v) | ((uint32_t)rows[r / 64] << 16);
-                    const uint64_t mv = v >= 0 ? (uint64_t)m[v] : 0;
-                    rec32[2 * r + 0] = x;
-                    rec32[2 * r + 1] = v >= 0 ? (uint32_t)m32[v] : 0u;
-                    rec64[4 * r + 0] = x;
-                    rec64[4 * r + 2] = (uint32_t)(mv & 0xFFFFFFFFu);
-                    rec64[4 * r + 3] = (uint32_t)(mv >> g->split);
-                }
-                uint32_t pos = 0;
-                std::vector<std::vector<int32_t>> rem(32);
-                for (int32_t d = 0; d < n_tiles; ++d) {
-                    for (int32_t h = 0; h < 2; ++h) {
-                        std::vector<int32_t> lanes;
-                        for (int32_t l = 0; l < 32; ++l) {
-                            const int32_t v = slot[((size_t)2 * d + h) * 32 + l];
-                            rem[l].clear();
-                            if (v >= 0) rem[l].assign(succ.begin() + succ_start[v], succ.begin() + succ_start[v + 1]);
-                            if (v >= 0 && rem[l].empty()) rem[l].push_back(n + 1);  // sink: the word that holds T
-                            lanes.push_back(l);
-                            for (int32_t k = 0; k < rows[d]; ++k) {
-                                uint32_t& e = sell[(size_t)pos + 32 * (size_t)k + l];
-                                e = h == 0 ? ((e & 0xFFFF0000u) | own_word(v)) : ((e & 0x0000FFFFu) | (own_word(v) << 16));
-                            }
-                        }
-                        for (int32_t k = 0; k < rows[d]; ++k) {
-                            int used[32] = {0};
-                            for (int32_t l = 0; l < 32; ++l)
-                                if (rem[l].empty()) used[l]++;   // reads its own word, which lies in bank l
-                            std::stable_sort(lanes.begin(), lanes.end(),
-                                             [&](int32_t x, int32_t y) { return rem[x].size() > rem[y].size(); });
-                            for (int32_t l : lanes) {
-                                if (rem[l].empty()) continue;  // stays the own word
-                                const bool forced = (int32_t)rem[l].size() >= rows[d] - k;
-                                int pick = -1;
-                                for (size_t c = 0; c < rem[l].size(); ++c)
-                                    if (!used[rem[l][c] & 31]) { pick = (int)c; break; }
-                                if (pick < 0 && !forced) continue;  // wait for a row where its bank is free
-                                if (pick < 0) pick = 0;
-                                used[rem[l][pick] & 31]++;
-                                uint32_t& e = sell[(size_t)pos + 32 * (size_t)k + l];
-                                const uint32_t off = 4u * (uint32_t)rem[l][pick];
-                                e = h == 0 ? ((e & 0xFFFF0000u) | off) : ((e & 0x0000FFFFu) | (off << 16));
-                                rem[l].erase(rem[l].begin() + pick);
-                            }
-                        }
-                    }
-                    pos += 32 * (uint32_t)rows[d];
-                }
-                std::vector<int32_t> tile_row((size_t)n_tiles, 0);
-                for (int32_t d = 1; d < n_tiles; ++d) tile_row[d] = tile_row[d - 1] + rows[d - 1];
-                up((void**)&g->d_tile_row, tile_row.data(), tile_row.size() * 4);
-                // the same tiles for the interval checker: its padding repeats a successor, a sink reads its own word
-                std::vector<uint32_t> sell_iv(sell);
-                for (size_t r = 0; r < slot.size(); ++r) {
-                    const int32_t v = slot[r];
-                    const uint32_t own = own_word(v), pad = v >= 0 && deg(v) > 0 ? 4u * (uint32_t)succ[succ_start[v]] : own;
-                    const int sh = (r & 32) ? 16 : 0;
-                    for (int32_t k = 0; k < rows[r / 64]; ++k) {
-                        uint32_t& e = sell_iv[32 * (size_t)(tile_row[r / 64] + k) + (r & 31)];
-                        const uint32_t off = e >> sh & 0xFFFFu;
-                        if (off == own || off == 4u * ((uint32_t)n + 1)) e = (e & ~(0xFFFFu << sh)) | pad << sh;
-                    }
-                }
-                up((void**)&g->d_sell_iv, sell_iv.data(), sell_iv.size() * 4);
-                g->sell_len = (int32_t)sell_len;
-                g->h_slot = slot;
-                g->n_tiles = n_tiles;
-                up(&g->d_rec32, rec32.data(), rec32.size() * 4);
-                up(&g->d_rec64, rec64.data(), rec64.size() * 4);
-                up((void**)&g->d_wslot, nullptr, slot.size() * 8);
-                up((void**)&g->d_sell, sell.data(), sell.size() * 4);
-            }
-        } catch (const std::bad_alloc&) {
-            moc_graph_destroy(g);
-            return fail(MOC_ERR_NOMEM, "host allocation failed");
-        }
-    }
     if (e != cudaSuccess) {
-        rc = fail(e == cudaErrorMemoryAllocation ? MOC_ERR_NOMEM : MOC_ERR_CUDA,
-                  "moc_graph_create: %s", cudaGetErrorString(e));
-        cudaGetLastError();
-        moc_graph_destroy(g);
-        return rc;
+        delete g;
+        return fail(MOC_ERR_CUDA, "moc_graph_create: %s", cudaGetErrorString(e));
     }
     try {
-        rc = build_lane_layouts(g, succ_start, succ, m, m32);
-        if (rc == MOC_OK) rc = upload_wslot(g);
-        if (rc == MOC_OK) rc = build_quad_layout(g, succ_start, succ);
+        g->h_w.assign(w, w + n);
+        Tables tables;
+        build_tables(g, keys, succ_start, succ, w, m, m32, &tables);
+        e = tables.upload(&g->d_tables);
     } catch (const std::bad_alloc&) {
-        rc = fail(MOC_ERR_NOMEM, "host allocation failed");
+        moc_graph_destroy(g);
+        return fail(MOC_ERR_NOMEM, "host allocation failed");
     }
-    if (rc != MOC_OK) {
+    if (e != cudaSuccess) {
+        const int rc = fail(e == cudaErrorMemoryAllocation ? MOC_ERR_NOMEM : MOC_ERR_CUDA, "moc_graph_create: %s", cudaGetErrorString(e));
         cudaGetLastError();
         moc_graph_destroy(g);
         return rc;
@@ -1077,24 +1099,6 @@ int moc_graph_set_max_copies(moc_graph* g, int32_t C) {
     ++g->generation;
     forget_plans(g);
     g->plan_profile.valid = false;
-    return MOC_OK;
-}
-
-// Uploads the slot durations of the warp-per-sequence layout: w | 1 << 48 (counts the node when it has
-// two copies) | 1 << 63 for nodes whose cap C_v is 1.
-static int upload_wslot(moc_graph* g) {
-    if (!g->d_wslot) return MOC_OK;
-    std::vector<uint64_t> wslot(g->h_slot.size());
-    for (size_t r = 0; r < wslot.size(); ++r) {
-        const int32_t v = g->h_slot[r];
-        uint64_t x = 0;
-        if (v >= 0) {
-            x = (uint64_t)g->h_w[v] | (uint64_t(1) << moc::kPairCntShift);
-            if (!g->h_cap.empty() && g->h_cap[v] == 1) x |= uint64_t(1) << 63;
-        }
-        wslot[r] = x;
-    }
-    MOC_CUDA(cudaMemcpy(g->d_wslot, wslot.data(), wslot.size() * 8, cudaMemcpyHostToDevice));
     return MOC_OK;
 }
 
@@ -1125,9 +1129,22 @@ int moc_graph_set_node_caps(moc_graph* g, const int32_t* caps) {
         MOC_CUDA(cudaFree(g->d_cap));
         g->d_cap = nullptr;
     }
-    int rc = upload_wslot(g);
-    if (rc != MOC_OK) return rc;
-    return upload_lane_rec(g);
+    // the caps are part of the node data of two layouts
+    try {
+        if (g->d_wslot) {
+            const std::vector<uint64_t> wslot = slot_durations(g);
+            MOC_CUDA(cudaMemcpy(g->d_wslot, wslot.data(), wslot.size() * 8, cudaMemcpyHostToDevice));
+        }
+    } catch (const std::bad_alloc&) {
+        return fail(MOC_ERR_NOMEM, "host allocation failed");
+    }
+    set_lane_caps(g);
+    for (const LaneLayout& L : g->lane) {
+        if (!L.ok) continue;
+        MOC_CUDA(cudaMemcpy(L.d_rec32, L.h_rec32.data(), L.h_rec32.size() * 4, cudaMemcpyHostToDevice));
+        MOC_CUDA(cudaMemcpy(L.d_rec64, L.h_rec64.data(), L.h_rec64.size() * 4, cudaMemcpyHostToDevice));
+    }
+    return MOC_OK;
 }
 
 int moc_graph_set_kernel(moc_graph* g, int32_t kind, int32_t a, int32_t b) {
@@ -1180,38 +1197,17 @@ int moc_graph_set_timing_events(moc_graph* g, void* before, void* after) {
 void moc_graph_destroy(moc_graph* g) {
     if (!g) return;
     DeviceGuard dg(g->device);
-    cudaFree(g->d_succ_start);
-    cudaFree(g->d_succ);
-    cudaFree(g->d_pred_start);
-    cudaFree(g->d_pred);
-    cudaFree(g->d_w);
-    cudaFree(g->d_m64);
-    cudaFree(g->d_m32);
-    cudaFree(g->d_rec32);
-    cudaFree(g->d_rec64);
-    cudaFree(g->d_wslot);
+    cudaFree(g->d_tables);
     cudaFree(g->d_cap);
-    cudaFree(g->d_sell);
-    cudaFree(g->d_sell_iv);
     cudaFree(g->d_offs);
     cudaFree(g->d_state);
     cudaFree(g->d_stage_seqs);
     cudaFree(g->d_stage_u16);
     cudaFree(g->d_stage_io);
-    cudaFree(g->d_order);
-    cudaFree(g->d_tile_row);
-    cudaFree(g->d_succ16);
-    cudaFree(g->d_live32);
-    cudaFree(g->d_live64);
     if (g->h_stage) cudaFreeHost(g->h_stage);
     if (g->copy_stream) cudaStreamDestroy(g->copy_stream);
     for (cudaEvent_t ev : g->chunk_ev)
         if (ev) cudaEventDestroy(ev);
-    for (int li = 0; li < 3; ++li) {
-        cudaFree(g->lane[li].d_rec32);
-        cudaFree(g->lane[li].d_rec64);
-        cudaFree(g->lane[li].d_succ);
-    }
     delete g;
 }
 

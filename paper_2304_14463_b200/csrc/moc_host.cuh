@@ -124,6 +124,7 @@ struct moc_graph {
     int sm_count = 0;
     size_t smem_optin = 0;
     int64_t sum_m = 0, sum_w = 0;
+    char* d_tables = nullptr;            // one allocation for all arrays that a graph is made of; the pointers to them follow
     int32_t* d_succ_start = nullptr;
     int32_t* d_succ = nullptr;
     int32_t* d_pred_start = nullptr;     // predecessor lists (CSR), for the incremental evaluation

@@ -74,6 +74,7 @@ int fake_in_flight() {
     for (const Op& o : g_ops) k += !o.done;
     return k;
 }
+int fake_allocations() { return (int)g_device.size(); }
 void fake_pin(const void* p, size_t size) { g_pinned.push_back({(uintptr_t)p, size}); }
 void fake_unpin_all() { g_pinned.clear(); }
 

@@ -40,11 +40,14 @@ def fake(tmp_path_factory):
 class Graph:
     def __init__(self, L, n, C=2, scale=1):
         self.L, self.n, self.h = L, n, P()
+        assert self.create(n, scale) == 0
+        assert L.moc_graph_set_max_copies(self.h, C) == 0
+
+    def create(self, n, scale):
         edges = workloads.layered_dag(n, 2 * n, max(2, n // 10), 1) if n >= 20 else np.zeros((0, 2), np.int32)
         edges = np.ascontiguousarray(edges, np.int32)
         w, m = np.ones(n, np.int64), np.full(n, scale, np.int64)
-        assert L.moc_graph_create(n, len(edges), edges.ctypes.data, w.ctypes.data, m.ctypes.data, ctypes.byref(self.h)) == 0
-        assert L.moc_graph_set_max_copies(self.h, C) == 0
+        return self.L.moc_graph_create(n, len(edges), edges.ctypes.data, w.ctypes.data, m.ctypes.data, ctypes.byref(self.h))
 
     def close(self):
         self.L.moc_graph_destroy(self.h)
@@ -229,3 +232,19 @@ def test_kernel_families_do_not_share_a_module(fake):
     for f in families:
         assert sum(f in m for m in modules) == 1, f
     assert all(sum(f in m for f in families) <= 1 for m in modules)
+
+
+@pytest.mark.parametrize("n,scale,copies", [(1, 1, 1), (20, 1, 1), (128, 1 << 30, 1), (442, 1, 1), (5000, 1, 1), (17000, 1, None)])
+def test_a_handle_is_one_allocation(fake, n, scale, copies):
+    """Tables for every kernel family, one allocation and one copy (one per array for graphs with more than a megabyte of
+    them), all of it given back; a failing call leaves nothing."""
+    fake.fake_reset(0)
+    G = Graph(fake, n, 2, scale)
+    lines = [x.split()[0] for x in log(fake)]
+    assert lines.count("malloc") == 1 and (copies is None or lines.count("memcpy") == copies)
+    calls = fake.fake_calls()
+    G.close()
+    assert fake.fake_allocations() == 0 and "free of a foreign pointer" not in log(fake)
+    for k in range(1, calls + 1):
+        fake.fake_reset(k)
+        assert G.create(n, scale) in (-5, -6) and not G.h.value and fake.fake_allocations() == 0
