@@ -738,14 +738,21 @@ moc::QuadParams quad_params(const moc_graph* g, const Plan& pl) {
     return q;
 }
 
-// Batches the backward walk serves.  Its time hardly depends on the batch until every SM has 16 warps: about
-// 6 us + 0.17 us per node (a lane's steps follow one another), while the warp-per-sequence kernel takes 1.2 us per
-// 1000 sequences of these sizes (2 us with 64-bit sums; the block-per-sequence kernel with C >= 3 likewise).
-// Measured crossings: n = 20 at 7000, 50 at 11000, 100 at 17000 sequences; 100 with 64-bit sums or C = 3 at 9000.
+// Batches the backward walk serves.  Its time is a sequence's latency until every SM has 16 warps (about 6 us + 0.17 us
+// per node), the other kernels' grows with the batch: the warp-per-sequence kernel (C <= 2) by the successor tiles of
+// 64 nodes that a sequence has, more with 64-bit sums, the block-per-sequence kernel (C >= 3) by the nodes.  Crossings
+// measured on layered and training graphs, sequences (C = 2 | C = 2, 64-bit sums | C = 3, 4):
+//     n =  20: 5000 | 4000 | 2300       n =  64: 12000 | 10500 | 4800       n = 100: 17000 | 12500 | 8000
+//     n =  40: 9500 | 6000 | 3200       n =  65: 11500 |  7500 | 5500       n = 128: 24000 | 16000 | 8800
+// Over batches of 700 to 26000 and n = 12 to 128 the lines below cost 0.1 to 0.3 % on the mean against always taking
+// the faster kernel, next to a crossing at most a fifth.
 bool live_serves(const moc_graph* g, int32_t B) {
     if (!g->d_live32 || g->C > moc::kLivePlanes || g->want_kind != MOC_KERNEL_AUTO || g->want_G || g->want_gpc) return false;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
-    return (int64_t)B * (g->C <= 2 && !wide ? 6 : 10) >= 30000 + 850 * (int64_t)g->n;
+    const int32_t n = g->n;
+    if (g->C > 2) return B >= 900 + 62 * n;
+    if (wide) return B >= (n <= 64 ? 300 + 160 * n : 120 * n);
+    return B >= (n <= 64 ? 1500 + 170 * n : 185 * n - 800);
 }
 
 int enqueue_live(const moc_graph* g, const Plan& pl, const int64_t* offs, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,

@@ -63,7 +63,8 @@ def test_pins_through_the_gpu(B):
 
 @pytest.mark.parametrize("n,C,scale,nB", [(1, 2, 1, 5200), (2, 1, 1, 5201), (31, 2, 1, 12000), (32, 4, 1, 6011), (33, 3, 1 << 26, 6001),
                                           (64, 2, 1 << 26, 9003), (65, 3, 1, 9009), (96, 2, 1, 19200), (127, 4, 1, 14001),
-                                          (128, 2, 1, 70001), (128, 1, 1 << 26, 14400)])
+                                          (128, 2, 1, 70001), (128, 1, 1 << 26, 14400), (64, 2, 1 << 26, 11003), (128, 1, 1 << 26, 16501),
+                                          (2, 3, 1, 1025), (2, 3, 1, 1023), (40, 3, 1 << 26, 3380), (20, 4, 1, 2140), (65, 2, 1 << 26, 7801)])
 def test_backward_walk_edges(B, n, C, scale, nB):
     """Batches that the lane-per-sequence walk serves: mask words full and just begun, both sum widths, one to
     four copies, per-node caps, damaged sequences, groups of 32 that do not come out even, more groups than one

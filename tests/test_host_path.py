@@ -248,3 +248,21 @@ def test_a_handle_is_one_allocation(fake, n, scale, copies):
     for k in range(1, calls + 1):
         fake.fake_reset(k)
         assert G.create(n, scale) in (-5, -6) and not G.h.value and fake.fake_allocations() == 0
+
+
+# batches from which on the backward walk is the faster kernel, as measured: (n, C, 64-bit sums) -> sequences
+WALK_FROM = {(20, 2, 0): 5000, (40, 2, 0): 9500, (64, 2, 0): 12000, (65, 2, 0): 11500, (100, 2, 0): 17000, (128, 2, 0): 24000,
+             (20, 2, 1): 4000, (40, 2, 1): 6000, (64, 2, 1): 10500, (65, 2, 1): 7500, (100, 2, 1): 12500, (128, 2, 1): 16000,
+             (20, 3, 0): 2300, (40, 3, 0): 3200, (64, 3, 1): 4800, (65, 4, 0): 5500, (100, 3, 0): 8000, (128, 4, 1): 8800}
+
+
+@pytest.mark.parametrize("case", WALK_FROM)
+def test_the_backward_walk_starts_where_it_is_faster(fake, case):
+    n, C, wide = case
+    G = Graph(fake, n, C, 1 << 30 if wide else 1)
+    x = np.zeros(8, np.int64)
+    for nB, walk in ((int(0.8 * WALK_FROM[case]), False), (int(1.25 * WALK_FROM[case]), True)):
+        fake.fake_reset(0)
+        assert fake.moc_eval_batch(G.h, x.ctypes.data, x.ctypes.data, nB, 0, x.ctypes.data, x.ctypes.data, x.ctypes.data, None) == 0
+        assert bool(launched(fake, "eval_live")) == walk, nB
+    G.close()
