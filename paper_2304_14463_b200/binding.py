@@ -3,8 +3,9 @@
 Function names mirror the C ABI.  PyTorch supplies device memory and streams: tensors are passed as
 ``data_ptr()`` and the stream as ``torch.cuda.current_stream().cuda_stream``.  The calls that only
 enqueue work on device tensors take their arguments apart in native code (_moc_torch.so, built from
-csrc/moc_torch.cpp): on small batches the interpreter would otherwise take longer than the GPU.  If the
-libraries have not been built, importing this module raises -- there is no CPU path.
+csrc/moc_torch.cpp): on small batches the interpreter would otherwise take longer than the GPU.  Where that
+module was built for another torch, the same calls go through ctypes, with a warning.  If
+libmoc_b200.so has not been built, importing this module raises -- there is no CPU path.
 """
 from __future__ import annotations
 
@@ -31,12 +32,34 @@ if not os.path.exists(LIB_PATH):
                       "(nvcc, sm_100a). There is no CPU fallback.")
 
 import torch  # noqa: E402  (its libraries have to be loaded in front of _moc_torch.so)
-try:
-    from . import _moc_torch as _fast
-except ImportError as _e:
-    raise ImportError(f"_moc_torch.so is missing or does not load ({_e}): build it with "
-                      "`python -m paper_2304_14463_b200.build`") from _e
 
+
+class _Slow:
+    """In place of _moc_torch: leaves every call to ctypes."""
+    @staticmethod
+    def bind(entry_points):
+        pass
+
+    eval_batch = eval_batch_host = mem_profile = check_intervals = cache_build = eval_edits = search_run = search_state = \
+        staticmethod(lambda *args: None)
+
+
+def _load_fast():
+    from . import build
+    why = f"built for another torch than {torch.__version__}, or not built"
+    if build.torch_lib_fits():
+        try:
+            from . import _moc_torch
+            return _moc_torch
+        except ImportError as e:
+            why = str(e)
+    import warnings
+    warnings.warn(f"_moc_torch.so cannot be used ({why}): calls go through ctypes, 10 us slower each; "
+                  "build it with `python -m paper_2304_14463_b200.build`", RuntimeWarning, stacklevel=3)
+    return _Slow
+
+
+_fast = _load_fast()
 lib = ctypes.CDLL(LIB_PATH)
 _P, _i32, _i64 = ctypes.c_void_p, ctypes.c_int32, ctypes.c_int64
 lib.moc_graph_create.restype = ctypes.c_int

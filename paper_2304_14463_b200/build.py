@@ -17,6 +17,7 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
 
 
 TORCH_LIB = os.path.join(HERE, "_moc_torch.so")
+TORCH_KEY = TORCH_LIB + ".key"      # torch and Python that _moc_torch.so was built for
 TORCH_SOURCES = ["moc_torch.cpp", os.path.join("..", "..", "include", "moc.h")]
 
 
@@ -28,8 +29,22 @@ def _stale(lib, files):
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def torch_key() -> str:
+    import torch
+    return f"torch {torch.__version__} cxx11abi {int(torch._C._GLIBCXX_USE_CXX11_ABI)} {sys.implementation.cache_tag}"
+
+
+def torch_lib_fits() -> bool:
+    """Whether _moc_torch.so was built for this torch (its C++ interface is not stable) and Python."""
+    try:
+        with open(TORCH_KEY) as f:
+            return os.path.exists(TORCH_LIB) and f.read() == torch_key()
+    except OSError:
+        return False
+
+
 def build_torch(force: bool = False) -> str:
-    if not force and not _stale(TORCH_LIB, TORCH_SOURCES):
+    if not force and torch_lib_fits() and not _stale(TORCH_LIB, TORCH_SOURCES):
         return TORCH_LIB
     import sysconfig
     import torch
@@ -43,6 +58,8 @@ def build_torch(force: bool = False) -> str:
     cmd += ["-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"]
     subprocess.run(cmd, check=True)
     os.replace(tmp, TORCH_LIB)
+    with open(TORCH_KEY, "w") as f:
+        f.write(torch_key())
     return TORCH_LIB
 
 

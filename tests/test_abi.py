@@ -104,3 +104,48 @@ def test_budget_rounding_matches_printed_budgets():
         p0 = int(line.split(":")[1].split("|")[0])
         budgets = [int(x) for x in line.split("|")[1].split()]
         assert [workloads.budget_from_peak(p0, pct) for pct in (90, 85, 80, 75)] == budgets
+
+
+@pytest.mark.parametrize("damage", ["key of another torch", "no key", "library that does not load", "no library"])
+def test_binding_without_its_native_side(binding, damage, tmp_path):
+    """_moc_torch.so is tied to one torch: with another, the import warns and every call goes through ctypes."""
+    import shutil
+    import subprocess
+    import sys
+    from paper_2304_14463_b200 import build
+    pkg = tmp_path / "paper_2304_14463_b200"
+    shutil.copytree(os.path.join(ROOT, "paper_2304_14463_b200"), pkg, ignore=shutil.ignore_patterns("csrc", "__pycache__"))
+    lib, key = pkg / "_moc_torch.so", pkg / "_moc_torch.so.key"
+    if damage == "key of another torch":
+        key.write_text(build.torch_key().replace("torch ", "torch 9."))
+    elif damage == "no key":
+        key.unlink()
+    elif damage == "no library":
+        lib.unlink()
+    else:
+        lib.unlink()
+        lib.write_bytes(b"not a library")
+    code = ("import warnings\nwith warnings.catch_warnings(record=True) as w:\n warnings.simplefilter('always')\n"
+            " from paper_2304_14463_b200 import binding as b\n"
+            "assert any('_moc_torch' in str(x.message) for x in w) and b._fast is b._Slow\n"
+            "assert b.lib.moc_graph_info(None, None, None, None, None) == -1\n"
+            "try: b.moc_search_set_kinds(None, 7)\n"
+            "except b.MocError as e: print('error', e.code)\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=tmp_path, capture_output=True, text=True)
+    assert r.returncode == 0 and r.stdout.strip() == "error -1", r.stderr
+
+
+def test_native_side_is_rebuilt_for_another_torch(binding, monkeypatch, tmp_path):
+    from paper_2304_14463_b200 import build
+    assert build.torch_lib_fits()
+    key = tmp_path / "key"
+    key.write_text(build.torch_key() + " and more")
+    monkeypatch.setattr(build, "TORCH_KEY", str(key))
+    assert not build.torch_lib_fits()
+    ran = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, check: ran.append(cmd))
+    monkeypatch.setattr(build.os, "replace", lambda a, b: None)
+    build.build_torch()
+    assert len(ran) == 1 and build.torch_lib_fits()
+    build.build_torch()
+    assert len(ran) == 1

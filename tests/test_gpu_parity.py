@@ -595,3 +595,40 @@ def test_node_caps_parity(B, idx):
     assert (st >= 0).any()
     with pytest.raises(B.MocError):
         G.set_caps(np.full(wl.n, wl.C + 1, np.int32))
+
+
+def test_every_call_through_ctypes(B, monkeypatch):
+    """The path of a binding whose native side does not fit the installed torch: same results, call by call."""
+    wl = W.make(2, seed=3, B=300)
+    seqs, lens = W.mutate(wl.seqs, wl.lens, wl.n, wl.C, seed=2, frac=1 / 16)
+    M = 300000
+    first = dev(wl.seqs[:wl.lens[0]])
+    T = len(first)
+    iv = torch.zeros((3, 1, wl.n, wl.C), dtype=torch.int32, device="cuda")       # one solution: the nodes in order, second slots idle
+    iv[0, 0, :, 0] = iv[1, 0, :, 0] = torch.arange(1, wl.n + 1)
+    iv[0, 0, :, 1] = iv[1, 0, :, 1] = torch.arange(wl.n + 1, 2 * wl.n + 1)
+    iv[2, 0, :, 0] = 1
+
+    def all_calls():
+        G = B.Graph(wl.n, wl.edges, wl.w, wl.m, wl.C)
+        out = list(G.eval_batch(dev(seqs), dev(lens), M)) + list(G.mem_profile(first)) + [G.mem_profile(first, want_free=False)[0]]
+        for bits in (16, 32):
+            host = [torch.empty(wl.B, dtype=d) for d in (torch.int64, torch.int64, torch.int32)]
+            ids = np.where(seqs < 0, 65535, seqs).astype(np.uint16 if bits == 16 else np.int32)
+            out += (G.eval_batch_host16 if bits == 16 else G.eval_batch_host)(torch.from_numpy(ids), torch.from_numpy(lens), M, *host)
+        out += G.check_intervals(*iv, M).values()
+        S = B.Search(G, dev(wl.seqs), dev(wl.lens), M, seed=5)
+        S.run(5)
+        out += S.state().values()
+        E = B.EditCache(G, wl.B)
+        out += E.build(dev(wl.seqs), dev(wl.lens), M)
+        k = torch.arange(600, dtype=torch.int32, device="cuda")
+        out += E.eval_edits(k % wl.B, k % 3, k % T, (7 * k) % T, M)
+        torch.cuda.synchronize()
+        return [x.cpu() for x in out]
+
+    fast = all_calls()
+    assert B._fast is not B._Slow
+    monkeypatch.setattr(B, "_fast", B._Slow)
+    slow = all_calls()
+    assert len(fast) == len(slow) and all(a.dtype == b.dtype and torch.equal(a, b) for a, b in zip(fast, slow))
