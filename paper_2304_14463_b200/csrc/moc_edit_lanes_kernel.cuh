@@ -48,10 +48,6 @@ struct LaneParent {
     __device__ __forceinline__ MemT prof(int32_t s) const { return __ldg(prof_ + s); }
     __device__ __forceinline__ MemT pm(int32_t s) const { return __ldg(pm_ + s); }
     __device__ __forceinline__ MemT sm(int32_t s) const { return __ldg(sm_ + s); }
-    // announcements of later reads: into L2, without a register or a wait
-    static constexpr bool kFar = true;
-    __device__ __forceinline__ void touch_occ(int32_t v) const { asm volatile("prefetch.global.L2 [%0];" ::"l"(occ_ + v)); }
-    __device__ __forceinline__ void touch_fre(int32_t s) const { asm volatile("prefetch.global.L2 [%0];" ::"l"(fre_ + s)); }
     // the usage array of lane l's parent, for all lanes of the warp
     __device__ __forceinline__ View prof_view(int l) const {
         const unsigned long long a = __shfl_sync(0xFFFFFFFFu, (unsigned long long)reinterpret_cast<uintptr_t>(prof_), l);

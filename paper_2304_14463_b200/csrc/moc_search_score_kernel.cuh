@@ -73,9 +73,6 @@ struct ScoreParent {
     __device__ __forceinline__ MemT prof(int32_t s) const { return prof_[s]; }
     __device__ __forceinline__ MemT pm(int32_t s) const { return pm_[s]; }
     __device__ __forceinline__ MemT sm(int32_t s) const { return sm_[s]; }
-    static constexpr bool kFar = false;
-    __device__ __forceinline__ void touch_occ(int32_t) const {}
-    __device__ __forceinline__ void touch_fre(int32_t) const {}
     __device__ __forceinline__ View prof_view(int) const { return View{prof_}; }
 };
 
