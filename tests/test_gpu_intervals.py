@@ -171,3 +171,85 @@ def test_interval_full_size_sampled(B):
         k = int(perm[b])
         got = (int(mask[b]), int(peak[b]), int(dur[b]), int(lens[b]))
         assert first.setdefault(k, got) == got, b
+
+
+def check_against_oracle(G, O, s, e, a, M, D, topo=None, tensors=None):
+    t = tensors or [dev(x) for x in (s, e, a)]
+    r = G.check_intervals(*t, M, D=D, topo_index=None if topo is None else dev(topo))
+    torch.cuda.synchronize()
+    r = {k: v.cpu().numpy() for k, v in r.items()}
+    seen = set()
+    for b in range(len(s)):
+        ref = O.check_intervals(s[b], e[b], a[b], M, D=D, topo_index=topo)
+        assert (int(r["mask"][b]), int(r["peak"][b]), int(r["dur"][b])) == (ref["mask"], ref["peak"], ref["dur"]), b
+        seq = O.intervals_to_sequence(s[b], e[b], a[b], D=D)
+        k = -1 if seq is None else len(seq)
+        assert r["lens"][b] == k and (seq is None or (r["seqs"][b, :k] == seq).all()) and (r["seqs"][b, max(k, 0):] == -1).all(), b
+        seen.add(ref["mask"])
+    return seen
+
+
+@pytest.mark.parametrize("idx,nB,shift", [(0, 200, 20), (0, 37, 34), (2, 40, 20), (2, 13, 30), (2, 9, 41)])
+def test_interval_sums_in_64_bits(B, idx, nB, shift):
+    """Two slots per node in the plain domain with sums beyond 32 bits: in two 32-bit parts, and (the last)
+    beyond what the parts cover, where another kernel serves them."""
+    wl = W.make(idx, seed=5, B=nB)
+    m = np.minimum(wl.m, 255) << shift
+    O, G = OracleGraph(wl.n, wl.edges, wl.w, m, wl.C), B.Graph(wl.n, wl.edges, wl.w, m, wl.C)
+    assert G.info()["wide"]
+    s, e, a, D, _ = build_batch(O, wl, np.random.default_rng(idx), nB, False)
+    assert len(check_against_oracle(G, O, s, e, a, O.eval(np.arange(wl.n), BIG)["peak"] * 80 // 100, D)) >= 3
+
+
+@pytest.mark.parametrize("shift", [0, 20])
+@pytest.mark.parametrize("D", [7102, 7103, 14205, 14206, 14207, 32766, 32767, 40001])
+def test_interval_long_plain_domains(B, D, shift):
+    """Few intervals spread over more and more events: from the kernel for two slots per node (whose events have to fit an SM
+    four times: up to 14206, 7102 with 64-bit sums) to the general one, last events and the ones behind them included."""
+    nB = 24
+    wl = W.make(0, seed=6, B=nB)
+    m = wl.m << shift
+    O, G = OracleGraph(wl.n, wl.edges, wl.w, m, wl.C), B.Graph(wl.n, wl.edges, wl.w, m, wl.C)
+    rng = np.random.default_rng(D)
+    s, e, a, D0, _ = build_batch(O, wl, rng, nB, False)
+    for b in range(nB):                                      # events moved apart, in order; what lies outside stays outside
+        place = np.concatenate([[0], np.sort(rng.choice(np.arange(1, D + 1), D0, replace=False)), [D + 1]])
+        place[D0] = D
+        for x in (s, e):
+            inside = (x[b] >= 0) & (x[b] <= D0 + 1)
+            x[b][inside] = place[x[b][inside]]
+    assert len(check_against_oracle(G, O, s, e, a, O.eval(np.arange(wl.n), BIG)["peak"], D)) >= 3
+
+
+@pytest.mark.parametrize("k", [0, 1, 2])
+def test_interval_arrays_off_an_eight_byte_boundary(B, k):
+    """One of the three arrays starts four bytes off: the pairs of slots cannot be read as one word."""
+    wl = W.make(2, seed=7, B=12)
+    O, G = OracleGraph(wl.n, wl.edges, wl.w, wl.m, wl.C), B.Graph(wl.n, wl.edges, wl.w, wl.m, wl.C)
+    s, e, a, D, _ = build_batch(O, wl, np.random.default_rng(k), 12, False)
+    t = []
+    for i, x in enumerate((s, e, a)):
+        flat = torch.zeros(x.size + 1, dtype=torch.int32, device="cuda")
+        t.append((flat[1:] if i == k else flat[:-1]).view(x.shape))
+        t[-1].copy_(dev(x))
+        assert t[-1].data_ptr() % 8 == (4 if i == k else 0)
+    check_against_oracle(G, O, s, e, a, O.eval(np.arange(wl.n), BIG)["peak"] * 80 // 100, D, tensors=t)
+
+
+@pytest.mark.parametrize("n,shift", [(361, 0), (361, 20), (362, 0), (600, 0), (600, 20), (1000, 0), (1200, 0)])
+def test_interval_staged_around_the_rule_for_kept_solutions(B, n, shift):
+    """Staged domains whose solutions stay on chip (16 bits per event up to n = 361, 32 beyond) while two fit an SM, and
+    domains too large for that."""
+    nB = 3
+    edges = W.layered_dag(n, 3 * n, 20, n)
+    w, m = W.weights_uniform(n, 1, 30, n, 1), W.weights_lognormal(n, 4.0, 1.0, n, 2) << shift
+    O, G = OracleGraph(n, edges, w, m, 2), B.Graph(n, edges, w, m, 2)
+
+    class Shape:
+        pass
+
+    wl = Shape()
+    wl.n, wl.C, wl.lens = n, 2, np.zeros(nB, np.int32)
+    s, e, a, D, topo = build_batch(O, wl, np.random.default_rng(n), nB, True)
+    seen = check_against_oracle(G, O, s, e, a, O.eval(np.arange(n), BIG)["peak"], D, topo=topo)
+    assert any(x & ~4 == 0 for x in seen) and len(seen) >= 2

@@ -171,6 +171,33 @@ def test_mem_profile_parity(B, idx):
     assert free is None and (prof.cpu().numpy() == r["profile"]).all()
 
 
+@pytest.mark.parametrize("C", [1, 2, 3, 4])
+@pytest.mark.parametrize("n,shift", [(199, 0), (199, 26), (601, 0), (601, 26), (1600, 26)])
+@pytest.mark.parametrize("tiles", [True, False])
+def test_mem_profile_both_sums_with_and_without_tiles(B, C, n, shift, tiles):
+    """The profile kernel's four variants: 32- and 64-bit sums, graphs with successor tiles and (a node with a successor in
+    every other one) without, one to four copies, 128 to 1024 threads."""
+    if tiles:
+        edges = W.layered_dag(n, 2 * n, 6, n)
+    else:
+        edges = np.array([(0, v) for v in range(1, n)] + [(v, v + 1) for v in range(1, n - 1)], np.int32)
+    w, m = W.weights_uniform(n, 1, 30, n, 1), W.weights_lognormal(n, 5.0, 1.0, n, 2) << shift
+    O, G = OracleGraph(n, edges, w, m, C), B.Graph(n, edges, w, m, C)
+    assert G.info()["wide"] == (shift > 0)
+    seqs, lens = W.schedules(n, edges, C, 0.4, 6, n + C)
+    seqs, lens = W.mutate(seqs, lens, n, C, seed=2, frac=0.4)
+    seen = set()
+    for seq in W.unpack(seqs, lens):
+        r = O.eval(seq, BIG)
+        prof, free, st = G.mem_profile(dev(seq))
+        only, none, _ = G.mem_profile(dev(seq), want_free=False)
+        torch.cuda.synchronize()
+        assert int(st[0]) == r["status"] and none is None
+        assert (prof.cpu().numpy() == r["profile"]).all() and (free.cpu().numpy() == r["free"]).all() and torch.equal(only, prof)
+        seen.add(r["status"])
+    assert 1 in seen
+
+
 # ------------------------------------------------------------------ every kernel family
 LANE_SHAPES = [(0, 0), (32, 32), (16, 32), (16, 16), (8, 32), (8, 24), (8, 16), (8, 8)]
 

@@ -31,6 +31,8 @@ def fake(tmp_path_factory):
     L.moc_graph_destroy.argtypes = [P]
     L.moc_graph_destroy.restype = None
     L.moc_eval_batch.argtypes = [P, P, P, i32, i64, P, P, P, P]
+    L.moc_mem_profile.argtypes = [P, P, i32, P, P, P, P]
+    L.moc_check_intervals.argtypes = [P, P, P, P, i32, i64, P, i64, P, P, P, P, P, P]
     for f in (L.moc_eval_batch_host, L.moc_eval_batch_host16):
         f.argtypes = [P, P, i64, P, i32, i64, P, P, P, P]
     yield L
@@ -38,13 +40,15 @@ def fake(tmp_path_factory):
 
 
 class Graph:
-    def __init__(self, L, n, C=2, scale=1):
-        self.L, self.n, self.h = L, n, P()
+    def __init__(self, L, n, C=2, scale=1, star=False):
+        self.L, self.n, self.h, self.star = L, n, P(), star
         assert self.create(n, scale) == 0
         assert L.moc_graph_set_max_copies(self.h, C) == 0
 
     def create(self, n, scale):
         edges = workloads.layered_dag(n, 2 * n, max(2, n // 10), 1) if n >= 20 else np.zeros((0, 2), np.int32)
+        if self.star:              # too uneven for successor tiles
+            edges = [(0, v) for v in range(1, n)]
         edges = np.ascontiguousarray(edges, np.int32)
         w, m = np.ones(n, np.int64), np.full(n, scale, np.int64)
         return self.L.moc_graph_create(n, len(edges), edges.ctypes.data, w.ctypes.data, m.ctypes.data, ctypes.byref(self.h))
@@ -265,4 +269,35 @@ def test_the_backward_walk_starts_where_it_is_faster(fake, case):
         fake.fake_reset(0)
         assert fake.moc_eval_batch(G.h, x.ctypes.data, x.ctypes.data, nB, 0, x.ctypes.data, x.ctypes.data, x.ctypes.data, None) == 0
         assert bool(launched(fake, "eval_live")) == walk, nB
+    G.close()
+
+
+@pytest.mark.parametrize("n,C,scale,D,staged,off,kernel", [
+    (20, 2, 1, 40, False, 0, "check_plain_kernelIi"), (20, 2, 1, 14206, False, 0, "check_plain_kernelIi"),
+    (20, 2, 1, 14207, False, 0, "check_intervals_kernelILb1ELi2EiLb1Et"), (20, 2, 1, 65536, False, 0, "check_intervals_kernelILb1ELi2EiLb1Ei"),
+    (20, 2, 1, 40, False, 4, "check_intervals_kernelILb1ELi2EiLb1Et"), (20, 3, 1, 40, False, 0, "check_intervals_kernelILb1ELi4EiLb1Et"),
+    (20, 2, 1 << 30, 7102, False, 0, "check_plain_kernelIl"), (20, 2, 1 << 30, 7103, False, 0, "check_intervals_kernelILb1ELi2ElLb1Et"),
+    (20, 2, 1 << 54, 40, False, 0, "check_intervals_kernelILb1ELi2ElLb1Et"),
+    (361, 2, 1, 361 * 181, True, 0, "check_intervals_kernelILb0ELi2EiLb1Et"), (362, 2, 1, 181 * 363, True, 0, "check_intervals_kernelILb0ELi2EiLb1Ei"),
+    (1000, 2, 1, 500 * 1001, True, 0, "check_intervals_kernelILb0ELi2EiLb1Ei"), (1200, 2, 1, 600 * 1201, True, 0, "check_intervals_kernelILb0ELi2EiLb0Ei")])
+def test_which_kernel_checks_intervals(fake, n, C, scale, D, staged, off, kernel):
+    G = Graph(fake, n, C, scale)
+    x = np.zeros(n * C + 8, np.int64)
+    fake.fake_reset(0)
+    rc = fake.moc_check_intervals(G.h, x.ctypes.data + off, x.ctypes.data, x.ctypes.data, 1, D, x.ctypes.data if staged else None, 0,
+                                  x.ctypes.data, x.ctypes.data, x.ctypes.data, x.ctypes.data, x.ctypes.data, None)
+    assert rc == 0 and len(launched(fake, kernel)) == 1, log(fake)
+    G.close()
+
+
+@pytest.mark.parametrize("n", [199, 601, 1600])
+@pytest.mark.parametrize("C", [2, 4, 5])
+@pytest.mark.parametrize("scale", [1, 1 << 30])
+@pytest.mark.parametrize("star", [False, True])
+def test_which_kernel_makes_a_profile(fake, n, C, scale, star):
+    G, x = Graph(fake, n, C, scale, star), np.zeros(8, np.int64)
+    fake.fake_reset(0)
+    assert fake.moc_mem_profile(G.h, x.ctypes.data, 4, x.ctypes.data, None, x.ctypes.data, None) == 0
+    wide, tiles = "l" if scale > 1 else "i", 0 if star else 1
+    assert len(launched(fake, f"eval_quad_kernelI{wide}Li{4 if C == 4 else 3}ELb{tiles}ELb1E" if C <= 4 else "eval_shared_kernelILi1024")) == 1, log(fake)
     G.close()
