@@ -417,7 +417,7 @@ def run_edits(args):
         torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / steps
     last = ring[(steps - 1) % 4]
-    st = out[2].cpu().numpy()
+    pk, du, st = (x.cpu().numpy() for x in out)          # before the second figure's runs write over them
     # ---- second figure: admissible edits only (random edits are mostly refused early: precedence, copy count).
     # The admissible edits of the four batches, repeated to the same batch size, timed the same way.
     adm = []
@@ -471,7 +471,6 @@ def run_edits(args):
         from oracle import OracleGraph
         O = OracleGraph(base.n, base.edges, base.w, base.m, base.C)
         offs = np.concatenate([[0], np.cumsum(base.lens)])
-        pk, du = out[0].cpu().numpy(), out[1].cpu().numpy()
         t0, k, same = time.perf_counter(), 0, True
         while time.perf_counter() - t0 < 8.0 and k < nE:
             c = last[4][k]
