@@ -16,7 +16,7 @@
 // Memory.  A step looks up its node's predecessor mask and record, and m of the outputs that become live, at
 // addresses the data decide.  The tables are replicated so that every lane has banks of its own (128 bytes per
 // row), which makes those reads conflict-free; one block per SM holds them (66 KB at n = 128) and the sequence is
-// read in place, 32 bytes per lane and eight steps, the next sixteen on their way (eight: 42 us at the size below).
+// read in place, 32 bytes per lane and eight steps, the next sixteen on their way (eight: 42.0 us at the size below).
 //
 // Latency.  A lane's steps follow one another, and a batch of 65536 is only 14 warps per SM.  So the part of a
 // step that depends on the step before is kept to the mask operations; m of what becomes live is
@@ -25,8 +25,8 @@
 // different words where possible, and more bits than that are left to a loop that few steps need.  (A loop
 // over the set bits of each word instead: 69 us at the size below, 1200 cycles per step.)
 //
-// n = 100, B = 65536, C = 2: 39.6 us (one launch) against 84 us for the warp-per-sequence kernel behind the offsets kernel.
-// Bound: the integer pipe, about 80 warp instructions per step of 32 sequences, a fifth of them for bits beyond one per word.
+// n = 100, B = 65536, C = 2: 38.9 us (one launch) against 84 us for the warp-per-sequence kernel behind the offsets kernel.
+// Bound: the integer pipe, about 87 warp instructions per step of 32 sequences (issue slots 63 %, ALU pipe 54 %), a fifth of them for bits beyond one per word.
 // The warp-per-sequence kernel pays a warp's fixed costs (clearing, scans, reductions) per sequence, which a
 // sequence of 120 steps does not repay; at n > 128 the masks outgrow the registers.
 #pragma once
