@@ -369,7 +369,12 @@ int moc_search_set_samples(moc_search* s, int32_t samples, int32_t incremental) 
         return MOC_OK;
     }
     // every chain needs a valid evaluation to start from
-    std::vector<int32_t> st((size_t)s->P);
+    std::vector<int32_t> st;
+    try {
+        st.resize((size_t)s->P);
+    } catch (const std::bad_alloc&) {
+        return fail(MOC_ERR_NOMEM, "host allocation failed");
+    }
     MOC_CUDA(cudaMemcpy(st.data(), s->p.status, (size_t)s->P * 4, cudaMemcpyDeviceToHost));
     for (int32_t c = 0; c < s->P; ++c)
         if (st[c] < 0)

@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 #include <set>
 #include <string>
 #include <vector>
@@ -40,6 +41,11 @@ std::map<const void*, std::string>& names() {        // kernels register themsel
 std::vector<Range> g_pinned;
 std::string g_log;
 int g_calls = 0, g_fail_at = 0, g_next_handle = 1;
+int g_news = 0, g_new_fails_at = 0, g_quiet = 0;
+struct Quiet {      // allocations of the stand-in itself neither count nor fail
+    Quiet() { ++g_quiet; }
+    ~Quiet() { --g_quiet; }
+};
 std::set<void*> g_device;
 
 void note(const std::string& s) { g_log += s + "\n"; }
@@ -56,10 +62,31 @@ std::string name_of(const void* fn) {
 std::string at(const void* p) { return std::to_string((unsigned long long)(uintptr_t)p); }
 }  // namespace
 
+// Host allocations of the library: the k-th fails.
+void* operator new(size_t n) {
+    if (!g_quiet && ++g_news == g_new_fails_at) throw std::bad_alloc();
+    void* p = malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void* operator new(size_t n, const std::nothrow_t&) noexcept {
+    if (!g_quiet && ++g_news == g_new_fails_at) return nullptr;
+    return malloc(n ? n : 1);
+}
+void operator delete(void* p) noexcept { free(p); }
+void operator delete(void* p, size_t) noexcept { free(p); }
+void operator delete(void* p, const std::nothrow_t&) noexcept { free(p); }
+
 extern "C" {
 
 // ---- control
+void fake_fail_new(int at) {
+    g_news = 0;
+    g_new_fails_at = at;
+}
+int fake_news() { return g_news; }
 void fake_reset(int fail_at) {
+    Quiet quiet;
     g_ops.clear();
     g_streams.clear();
     g_events.clear();
@@ -75,7 +102,10 @@ int fake_in_flight() {
     return k;
 }
 int fake_allocations() { return (int)g_device.size(); }
-void fake_pin(const void* p, size_t size) { g_pinned.push_back({(uintptr_t)p, size}); }
+void fake_pin(const void* p, size_t size) {
+    Quiet quiet;
+    g_pinned.push_back({(uintptr_t)p, size});
+}
 void fake_unpin_all() { g_pinned.clear(); }
 
 // ---- runtime
@@ -92,6 +122,7 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
     return cudaSuccess;
 }
 cudaError_t cudaMalloc(void** p, size_t n) {
+    Quiet quiet;
     note("malloc " + std::to_string(n));
     if (fails()) return cudaErrorMemoryAllocation;
     *p = aligned_alloc(256, (n + 255) & ~size_t(255));
@@ -99,6 +130,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
     return cudaSuccess;
 }
 cudaError_t cudaFree(void* p) {
+    Quiet quiet;
     if (p) {
         note("free");
         if (!g_device.erase(p)) note("free of a foreign pointer");
@@ -107,17 +139,20 @@ cudaError_t cudaFree(void* p) {
     return cudaSuccess;
 }
 cudaError_t cudaMallocHost(void** p, size_t n) {
+    Quiet quiet;
     note("malloc_host " + std::to_string(n));
     if (fails()) return cudaErrorMemoryAllocation;
     return *p = malloc(n), cudaSuccess;
 }
 cudaError_t cudaFreeHost(void* p) { return free(p), cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+    Quiet quiet;
     note("memcpy " + std::to_string(n));
     if (fails()) return cudaErrorUnknown;
     return memcpy(d, s, n), cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kind, cudaStream_t st) {
+    Quiet quiet;
     note(std::string("copy ") + (kind == cudaMemcpyHostToDevice ? "h2d " : "d2h ") + at(s) + " " + std::to_string(n));
     if (fails()) return cudaErrorUnknown;
     enqueue(st, "copy");
@@ -136,11 +171,13 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
 }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st) {
+    Quiet quiet;
     if (fails() || !e) return cudaErrorUnknown;
     g_events[e].behind = g_streams[st].ops;
     return cudaSuccess;
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned) {
+    Quiet quiet;
     if (fails() || !e) return cudaErrorUnknown;
     std::vector<size_t>& ops = g_streams[st].ops;
     for (size_t i : g_events[e].behind)
@@ -148,22 +185,26 @@ cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned) {
     return cudaSuccess;
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t st) {
+    Quiet quiet;
     note("sync");
     const bool bad = fails();       // reported, but the work is over all the same
     for (size_t i : g_streams[st].ops) g_ops[i].done = true;
     return bad ? cudaErrorUnknown : cudaSuccess;
 }
 cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* a, const void* fn) {
+    Quiet quiet;
     note("lookup " + name_of(fn));
     if (fails()) return cudaErrorUnknown;
     memset(a, 0, sizeof *a);
     return cudaSuccess;
 }
 cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute, int) {
+    Quiet quiet;
     note("lookup " + name_of(fn));
     return fails() ? cudaErrorUnknown : cudaSuccess;
 }
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* nb, const void* fn, int threads, size_t smem) {
+    Quiet quiet;
     note("lookup " + name_of(fn));
     if (fails()) return cudaErrorUnknown;
     const size_t regs = 64, by_smem = 233472 / (smem + 1024), by_regs = 65536 / (regs * threads);
@@ -174,6 +215,7 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* nb, cons
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, threads, smem);
 }
 cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void**, size_t, cudaStream_t st) {
+    Quiet quiet;
     note("launch " + name_of(fn));
     if (fails()) return cudaErrorUnknown;
     return enqueue(st, "launch"), cudaSuccess;

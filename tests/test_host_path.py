@@ -31,6 +31,11 @@ def fake(tmp_path_factory):
     L.moc_graph_destroy.argtypes = [P]
     L.moc_graph_destroy.restype = None
     L.moc_eval_batch.argtypes = [P, P, P, i32, i64, P, P, P, P]
+    L.moc_graph_set_node_caps.argtypes = [P, P]
+    L.moc_search_create.argtypes = [P, P, P, i32, i64, ctypes.c_uint64, ctypes.c_uint32, P, ctypes.POINTER(P)]
+    L.moc_search_set_samples.argtypes = [P, i32, i32]
+    L.moc_search_destroy.argtypes = [P]
+    L.moc_search_destroy.restype = None
     L.moc_mem_profile.argtypes = [P, P, i32, P, P, P, P]
     L.moc_check_intervals.argtypes = [P, P, P, P, i32, i64, P, i64, P, P, P, P, P, P]
     for f in (L.moc_eval_batch_host, L.moc_eval_batch_host16):
@@ -301,3 +306,43 @@ def test_which_kernel_makes_a_profile(fake, n, C, scale, star):
     wide, tiles = "l" if scale > 1 else "i", 0 if star else 1
     assert len(launched(fake, f"eval_quad_kernelI{wide}Li{4 if C == 4 else 3}ELb{tiles}ELb1E" if C <= 4 else "eval_shared_kernelILi1024")) == 1, log(fake)
     G.close()
+
+
+@pytest.mark.parametrize("n,scale,star", [(1, 1, False), (20, 1, False), (128, 1 << 30, False), (442, 1, False), (601, 1, True)])
+def test_host_allocations_that_fail(fake, n, scale, star):
+    """Every allocation on the host fails in turn: MOC_ERR_NOMEM, no exception across the C ABI, nothing left behind."""
+    fake.fake_reset(0)
+    G = Graph(fake, n, 2, scale, star)
+    caps = np.ones(n, np.int32)
+    k = 0
+    while True:
+        k += 1
+        fake.fake_fail_new(k)
+        rc = fake.moc_graph_set_node_caps(G.h, caps.ctypes.data)
+        used = fake.fake_news()
+        fake.fake_fail_new(0)
+        assert rc == (-6 if used >= k else 0)
+        if used < k:
+            break
+    seqs, lens, s = np.zeros(2 * n + 8, np.int32), np.full(3, n, np.int32), P()
+    assert fake.moc_search_create(G.h, seqs.ctypes.data, lens.ctypes.data, 3, 0, 1, 0, None, ctypes.byref(s)) == 0
+    fake.fake_fail_new(1)
+    assert fake.moc_search_set_samples(s, 4, 1) == -6
+    fake.fake_fail_new(0)
+    fake.moc_search_destroy(s)
+    G.close()
+    k = 0
+    while True:
+        k += 1
+        fake.fake_fail_new(k)
+        rc = G.create(n, scale)
+        used = fake.fake_news()
+        fake.fake_fail_new(0)
+        if used < k:
+            break
+        assert rc in (0, -6) and (rc == 0) == bool(G.h.value)         # 0: the sort did without its buffer
+        if rc == 0:
+            G.close()
+        assert fake.fake_allocations() == 0
+    G.close()
+    assert k > (10 if n > 1 else 3)
