@@ -659,3 +659,43 @@ def test_every_call_through_ctypes(B, monkeypatch):
     monkeypatch.setattr(B, "_fast", B._Slow)
     slow = all_calls()
     assert len(fast) == len(slow) and all(a.dtype == b.dtype and torch.equal(a, b) for a, b in zip(fast, slow))
+
+
+CAPTURE = """
+import numpy as np, torch
+from paper_2304_14463_b200 import binding as B, workloads as W
+for idx, sizes in ((0, (64, 60000)), (2, (5000, 64)), (3, (4096, 64))):
+    wl = W.make(idx, seed=1, B=max(sizes))
+    G = B.Graph(wl.n, wl.edges, wl.w, wl.m, wl.C)
+    def batch(k):
+        outs = [torch.zeros(k, dtype=d, device="cuda") for d in (torch.int64, torch.int64, torch.int32)]
+        return (torch.from_numpy(wl.seqs[:int(wl.lens[:k].sum())]).cuda(), torch.from_numpy(wl.lens[:k]).cuda(),
+                dict(zip(("out_peak", "out_dur", "out_feasible"), outs)))
+    s, l, o = batch(sizes[0])
+    if {warm}:
+        G.eval_batch(s, l, 30000, **o)
+    s, l, o = batch(sizes[1])
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        G.eval_batch(s, l, 30000, **o)
+    assert not any(x.any() for x in o.values())
+    g.replay()
+    torch.cuda.synchronize()
+    got = [x.clone() for x in o.values()]
+    G.eval_batch(s, l, 30000, **o)
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(got, o.values())) and got[0].any()
+print("captured")
+"""
+
+
+@pytest.mark.parametrize("warm", [True, False])
+def test_first_call_inside_a_capture(B, warm):
+    """A process whose first evaluation, or the first of a size that another kernel serves, is captured into a CUDA
+    graph: kernels are loaded and looked up while the stream is being captured."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", CAPTURE.replace("{warm}", str(warm))], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "captured" in r.stdout, r.stderr[-2000:]
