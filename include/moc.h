@@ -124,11 +124,13 @@ int moc_eval_batch(const moc_graph* g, const int32_t* seqs, const int32_t* lens,
  * with respect to the host, pageable memory works too): copies seqs (n_steps ints, which must be
  * at least sum(max(lens[b],0))) and lens to device staging owned by the handle, evaluates, copies
  * the three outputs back and synchronises `stream` before returning.  Large batches travel in
- * three parts (11, 4 and 1 sixteenths of the ids; what lies behind the batch in seqs is not needed and not sent, but for a
- * few ids where that is cheaper than to know): a copy stream owned by the handle brings one part while
+ * three parts (11, 4 and 1 sixteenths of the ids): a copy stream owned by the handle brings one part while
  * `stream` evaluates the sequences that are complete with the one before, so that only the evaluation of
  * the small last part is not hidden; results return to pinned arrays straight from the device and to
- * pageable ones through a pinned block of the handle.  One call at a time per handle.
+ * pageable ones through a pinned block of the handle.  A buffer may be larger than the batch in it:
+ * the staging follows the batch, and the ids behind it are not sent (unless 64 lengths, looked at before
+ * the first part starts, make the batch look as long as the buffer).  When the call returns, with an error
+ * too, nothing reads or writes the caller's arrays any more.  One call at a time per handle.
  */
 int moc_eval_batch_host(const moc_graph* g, const int32_t* seqs, int64_t n_steps,
                         const int32_t* lens, int32_t B, int64_t M, int64_t* out_peak,
@@ -161,8 +163,8 @@ int moc_eval_batch_host16(const moc_graph* g, const uint16_t* seqs, int64_t n_st
  *     does not fit in shared memory (more than 65534 steps per sequence, or n*C too large): that
  *     case needs a global workspace, which only moc_eval_batch provides.
  *   - The first call on each device looks up the array's device address (once per device, with
- *     that device current) and prepares the launch plan of the handle.  Make that first call
- *     outside of any stream capture.
+ *     that device current), and a handle's first call, or its first of a batch size that
+ *     another kernel serves, prepares a launch plan.  Make those calls outside of any stream capture.
  *   - All calls on a device, from every handle and stream, share the one array.  Each call
  *     rewrites the B+1 entries it uses before reading them, so stale contents of an earlier call
  *     never matter and nothing needs clearing; but two calls that overlap on the GPU (different
