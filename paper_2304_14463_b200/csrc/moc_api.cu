@@ -108,19 +108,52 @@ const char* plan_lane(const moc_graph* g, size_t smem_cap, Plan* out) {
     return "the state of a group of sequences exceeds shared memory in the requested shape, n >= 4096, or a degree above 255";
 }
 
+// Shared memory of the block-per-sequence kernel: the state of a sequence and, behind it, the block's copy of the tiles.
+struct QuadBytes {
+    size_t word, cnt, delta, rec, w, sell, row;
+    size_t state() const { return word + cnt + delta; }
+    size_t graph() const { return rec + w + sell + row; }
+};
+QuadBytes quad_bytes(const moc_graph* g, bool wide, bool profile) {
+    const size_t n = (size_t)g->n, t_max = (size_t)g->C * n, msz = wide ? 8 : 4;
+    QuadBytes z;
+    z.word = (g->C <= 2 && !profile ? 1 : 2) * align16(4 * (n + 2)) + 16;
+    z.cnt = align16(2 * (n + 2));
+    z.delta = align16(msz * (t_max + 4));
+    z.rec = (wide ? 16 : 8) * 64 * (size_t)g->n_tiles;
+    z.w = 8 * 64 * (size_t)g->n_tiles;
+    z.sell = align16(4 * (size_t)g->sell_len);
+    z.row = align16(4 * (size_t)g->n_tiles);
+    return z;
+}
+
+// Whether the block-per-sequence kernel takes a batch of B with the tiles in the block's shared memory.  It saves the L2's
+// latency three times per sequence and costs every block of an SM its own copy (0.5 us each, one after the other), so it
+// pays while an SM has one sequence, for small graphs up to three; and the copies have to fit beside all of them.  Measured, copied / through
+// L1 (C = 3, best thread count of each): n = 442 6.4 / 8.4 us at B = 148, 8.4 / 10.5 at 444, 12.5 / 12.5 at 888; n = 700 7.5 / 8.4 at 148, 10.5 /
+// 10.5 at 444, 14.6 / 10.5 at 592; n = 1000 8.4 / 9.2 (C = 4), 12.5 / 10.5 at 444 (C = 2); n = 3300 12.5 / 14.6 at 148, 18.7 / 16.5 at 296;
+// n = 5000 14.5 / 12.6 at 148 (C = 2).
+bool quad_chip_fits(const moc_graph* g, int32_t B, bool profile) {
+    const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    if (!g->n_tiles || g->C > 4 || g->sum_w >= (int64_t)1 << moc::kPairCntShift) return false;
+    const int64_t per_sm = ((int64_t)B + g->sm_count - 1) / g->sm_count;
+    if (per_sm > (g->n <= 700 ? 3 : 1) || g->n > 4000) return false;
+    const QuadBytes z = quad_bytes(g, wide, profile);
+    return (size_t)per_sm * (z.state() + z.graph() + 2048) <= g->smem_optin;
+}
+
 // Plan of the block-per-sequence path with packed words (C <= 4).  Returns nullptr on success.
-const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, Plan* out) {
+const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, bool chip, Plan* out) {
     Plan pl = *out;
     const int64_t n = g->n, C = g->C, t_max = C * n;
     if (C > 4) return "C > 4";
     if (!g->d_rec32 && !g->d_order) return "n above 32000 or a degree above 65535";
     if (t_max > 32766) return "sequences of more than 32766 steps";
     if (pl.wide && !g->split_ok) return "sum(m) too large for two-part sums";
-    const size_t msz = pl.wide ? 8 : 4;
-    const size_t word_b = 2 * align16(4 * (size_t)(n + 2)) + 16, cnt_b = align16(2 * (size_t)(n + 2)), delta_b = align16(msz * (size_t)(t_max + 4));
-    const size_t sm = word_b + cnt_b + delta_b;
+    const QuadBytes z = quad_bytes(g, pl.wide, profile);
+    const size_t sm = z.state() + (chip ? z.graph() : 0);
     if (sm > smem_cap) return "the state of a sequence exceeds shared memory";
-    QuadFn fn = quad_fn(pl.wide, (int)C, g->d_rec32 != nullptr, profile);
+    QuadFn fn = quad_fn(pl.wide, (int)C, g->d_rec32 != nullptr, chip, profile);
     if (raise_smem_limit((const void*)fn, g->smem_optin) != cudaSuccess) { cudaGetLastError(); return "cudaFuncSetAttribute failed"; }
     const int forced = !profile && g->want_kind == MOC_KERNEL_BLOCK ? g->want_a : 0;
     bool any = false;
@@ -133,40 +166,44 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, Plan* o
     }
     if (!any) return "kernel does not fit on an SM";
     pl.quad = true;
+    pl.quad_chip = chip;
     pl.quad_fn = fn;
     pl.quad_forced = forced;
     pl.gpc = 1;
     pl.smem = sm;
     pl.sm_count = g->sm_count;
     pl.grid = g->sm_count * std::max(1, pl.quad_nb[1]);
-    pl.quad_word_b = (uint32_t)word_b;
-    pl.quad_cnt_b = (uint32_t)cnt_b;
+    pl.quad_word_b = (uint32_t)z.word;
+    pl.quad_cnt_b = (uint32_t)z.cnt;
+    pl.quad_delta_b = (uint32_t)z.delta;
+    pl.rec_bytes = (uint32_t)z.rec;
+    pl.w_bytes = (uint32_t)z.w;
+    pl.sell_bytes = (uint32_t)z.sell;
+    pl.quad_row_b = (uint32_t)z.row;
     pl.valid = true;
     *out = pl;
     return nullptr;
 }
 
-// Shape of the block-per-sequence kernel for a batch: threads per sequence (64 << k) and blocks per SM.  The time is
-// rounds x (latency or throughput of the sequences on an SM, whichever is longer, and a third of the other); both
-// follow measurements at n = 442, 1000 and 5000 (C = 3, 64 to 1024 threads, B = 1 to 16384; microseconds):
-//     latency of a sequence      0.93 per 64 nodes and 64 threads + 1.2 + 0.35 per 64 threads (barriers)
-//     SM time of a sequence      0.10 per 64 nodes + 0.16 per 64 threads
-// With the blocks per SM that the state and the registers allow, a batch takes ceil(sequences per SM / blocks) rounds;
-// as few blocks as that number of rounds needs keeps them even.
-// The other variants are close enough to use the same two lines: over 566 shapes (n = 60 to 5000, B = 1 to 8192, C = 2, 3, 4
-// with 32- and 64-bit sums) the choice costs 1 to 1.5 % on the mean of each variant against the best of the five thread
-// counts, 3 to 6 % or less in nine of ten, and 24 % at worst (n = 250, C = 4, B = 220: 10.7 against 8.7 us).
-void quad_shape(const Plan& pl, int64_t n, int32_t B, int* threads, int* blocks) {
+// Shape of the block-per-sequence kernel for a batch: threads per sequence (64 << k) and blocks per SM.  With the blocks
+// per SM that the state and the registers allow, a batch takes ceil(sequences per SM / blocks) rounds; as few
+// blocks as that number of rounds needs keeps them even.  Time in microseconds, with u = n / 64 and w = threads / 64, from
+// a fit to 4035 timed shapes (n = 40 to 5000, C = 2, 3, 4, 32- and 64-bit sums, B = 1 to 8192, every thread count):
+//     through L1:   rounds (1.27 + (0.40 + 0.15 C) u / w + 0.046 w) + sequences per SM (0.10 + 0.040 w + 0.010 C u)
+//     copied:       rounds (1.36 + (0.10 + 0.14 C) u / w + 0.018 w) + sequences per SM (0.055 w + 0.015 C u)
+// The choice costs 0.5 % and 0.7 % on the mean against the best of the five thread counts, 1.6 % or less in nine of ten,
+// and 38 % at worst (n = 1500, C = 4, B = 148: 14.5 against 10.6 us through L1).
+void quad_shape(const Plan& pl, int64_t n, int32_t C, int32_t B, int* threads, int* blocks) {
     const int64_t per_sm = ((int64_t)B + pl.sm_count - 1) / pl.sm_count;
-    const double units = (double)n / 64.0;
+    const double u = (double)n / 64.0;
     double best = 0;
     *threads = 0;
     for (int k = 0; k < 5; ++k) {
-        const int nb = pl.quad_nb[k], wide = 1 << k;
+        const int nb = pl.quad_nb[k], w = 1 << k;
         if (nb < 1) continue;
         const int64_t rounds = (per_sm + nb - 1) / nb, even = (per_sm + rounds - 1) / rounds;
-        const double lat = 0.93 * units / wide + 1.2 + 0.35 * wide, thr = (double)even * (0.10 * units + 0.16 * wide);
-        const double cost = (double)rounds * (std::max(lat, thr) + 0.35 * std::min(lat, thr));
+        const double cost = pl.quad_chip ? (double)rounds * (1.36 + (0.10 + 0.14 * C) * u / w + 0.018 * w) + (double)per_sm * (0.055 * w + 0.015 * C * u)
+                                         : (double)rounds * (1.27 + (0.40 + 0.15 * C) * u / w + 0.046 * w) + (double)per_sm * (0.10 + 0.040 * w + 0.010 * C * u);
         if (*threads == 0 || cost < best) {
             best = cost;
             *threads = pl.quad_forced ? pl.quad_forced : 64 << k;
@@ -207,7 +244,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     const size_t smem_cap = g->smem_optin > 1024 ? g->smem_optin - 1024 : 0;  // 1 KB per block is reserved
     const int kind = profile ? MOC_KERNEL_GROUP : g->want_kind;
     const bool shape_given = g->want_G != 0 || g->want_gpc != 0;       // moc_graph_set_launch
-    if (profile && !plan_quad(g, smem_cap, true, &pl)) {
+    if (profile && !plan_quad(g, smem_cap, true, quad_chip_fits(g, 1, true), &pl)) {
         *out = pl;
         return MOC_OK;
     }
@@ -224,7 +261,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         if (kind == MOC_KERNEL_LANE) return fail(MOC_ERR_ARG, "the sequence-per-lane kernel cannot serve this graph: %s", why);
     }
     if (kind == MOC_KERNEL_BLOCK || (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C >= 3)) {
-        const char* why = plan_quad(g, smem_cap, profile, &pl);
+        const char* why = plan_quad(g, smem_cap, profile, false, &pl);
         if (!why) {
             *out = pl;
             return MOC_OK;
@@ -277,7 +314,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     }
     // sequences too long for eight warps of the warp-per-sequence kernel on an SM (n = 2000, B = 2000: 69.6 us with a
     // thread group per sequence, 53.5 with the block-per-sequence kernel)
-    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, profile, &pl)) {
+    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, profile, false, &pl)) {
         *out = pl;
         return MOC_OK;
     }
@@ -738,6 +775,13 @@ moc::QuadParams quad_params(const moc_graph* g, const Plan& pl) {
     q.cap = g->d_cap;
     q.word_bytes = pl.quad_word_b;
     q.cnt_bytes = pl.quad_cnt_b;
+    q.delta_bytes = pl.quad_delta_b;
+    q.wslot = (const uint64_t*)g->d_wslot;
+    q.rec_bytes = pl.rec_bytes;
+    q.w_bytes = pl.w_bytes;
+    q.sell_bytes = pl.sell_bytes;
+    q.row_bytes = pl.quad_row_b;
+    q.small_w = (__int128)g->C * g->sum_w < ((int64_t)1 << 32) ? 1 : 0;
     return q;
 }
 
@@ -834,7 +878,7 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
     }
     if (pl.quad) {
         int nb = 1;
-        quad_shape(pl, g->n, B, &block, &nb);
+        quad_shape(pl, g->n, g->C, B, &block, &nb);
         grid = (int)std::min<int64_t>((int64_t)pl.sm_count * nb, B);
     }
     if (offs && fill_offs) {
@@ -850,6 +894,8 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
     if (pl.quad) {
         moc::QuadParams q = quad_params(g, pl);
         q.B = B;
+        q.per_block = B / grid;
+        q.spare = B % grid;
         q.M = M;
         q.seqs = seqs;
         q.lens = lens;
@@ -946,21 +992,29 @@ const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
         if (!g->plan_live.valid) plan_live(g, &g->plan_live);
         if (g->plan_live.live_fn) return &g->plan_live;
     }
-    if (block_serves(g, B)) {
-        if (!g->plan_block.valid) {
+    const bool block = block_serves(g, B), wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    const size_t cap = g->smem_optin > 1024 ? g->smem_optin - 1024 : 0;
+    auto quad = [&](Plan& kept, bool chip) -> const Plan* {
+        if (!kept.valid) {
             Plan pl;
-            pl.wide = g->sum_m > (int64_t)INT32_MAX / g->C;
-            plan_quad(g, g->smem_optin > 1024 ? g->smem_optin - 1024 : 0, false, &pl);
+            pl.wide = wide;
+            plan_quad(g, cap, false, chip, &pl);
             pl.valid = true;
-            g->plan_block = pl;
+            kept = pl;
         }
-        if (g->plan_block.quad) return &g->plan_block;
-    }
+        return kept.quad ? &kept : nullptr;
+    };
+    // small batches of the block-per-sequence kernel: with the graph in its shared memory
+    const bool any_block = block || g->want_kind == MOC_KERNEL_BLOCK || (g->want_kind == MOC_KERNEL_AUTO && !g->want_G && !g->want_gpc && g->C >= 3);
+    if (any_block && quad_chip_fits(g, B, false))
+        if (const Plan* pl = quad(g->plan_chip, true)) return pl;
+    if (block)
+        if (const Plan* pl = quad(g->plan_block, false)) return pl;
     if (!g->plan_eval.valid) *rc = make_plan(g, false, &g->plan_eval);
     return *rc == MOC_OK ? &g->plan_eval : nullptr;
 }
 
-void forget_plans(moc_graph* g) { g->plan_eval = g->plan_block = g->plan_live = Plan(); }
+void forget_plans(moc_graph* g) { g->plan_eval = g->plan_block = g->plan_chip = g->plan_live = Plan(); }
 
 int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
                 int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {

@@ -31,7 +31,7 @@ KernelFn shared_fn(bool wide, int G, int CP, bool profile);
 KernelFn global_fn(int CP, bool profile);
 PairFn pair_fn(bool wide, int pre);
 LaneFn lane_fn(bool wide, int lg, int kp);
-QuadFn quad_fn(bool wide, int C, bool tiles, bool profile);
+QuadFn quad_fn(bool wide, int C, bool tiles, bool chip, bool profile);
 LiveFn live_fn(bool wide, int words, int C);
 const void* check_plain_fn(bool wide);
 IntervalFn check_general_fn(int cp, bool wide, int kept);      // kept: bytes per event of the solution kept on chip, 0: not kept
@@ -59,7 +59,8 @@ struct Plan {
     // block-per-sequence path with packed words for C <= 4
     bool quad = false;
     QuadFn quad_fn = nullptr;
-    uint32_t quad_word_b = 0, quad_cnt_b = 0;
+    bool quad_chip = false;        // the block keeps a copy of the graph's tiles
+    uint32_t quad_word_b = 0, quad_cnt_b = 0, quad_delta_b = 0, quad_row_b = 0;
     int quad_nb[5] = {0};          // blocks per SM with 64 << k threads
     int quad_forced = 0;           // threads per sequence the caller asked for
     // small graphs, large batches: a lane per sequence, walked backwards (null: another kernel)
@@ -161,6 +162,7 @@ struct moc_graph {
     // grow-only scratch; mutable because evaluation takes a const handle
     mutable moc_host::Plan plan_eval, plan_profile;
     mutable moc_host::Plan plan_block;    // block-per-sequence kernel beside the warp-per-sequence one in plan_eval
+    mutable moc_host::Plan plan_chip;     // ... and the same with the graph in shared memory, for small batches
     mutable moc_host::Plan plan_live;     // backward walk beside either
     mutable int64_t* d_offs = nullptr;
     mutable size_t offs_cap = 0;

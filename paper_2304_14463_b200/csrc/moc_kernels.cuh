@@ -89,6 +89,38 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// Sum of values whose sum is below 2^59 over the warp, by two warp reductions (five rounds of 64-bit shuffles take three
+// times as long).
+__device__ __forceinline__ uint64_t warp_sum_u59(uint64_t v) {
+    const uint32_t lo = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)v & 0x7FFFFFFu), hi = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(v >> 27));
+    return ((uint64_t)hi << 27) + lo;
+}
+// This thread's part (of `nthr` threads) of the sum of max(lens[i], 0) over i < b.
+__device__ __forceinline__ uint64_t lengths_before(const int32_t* lens, int b, int tid, int nthr) {
+    uint64_t sum = 0;
+    auto add = [&](int32_t v) { asm("mad.wide.u32 %0, %1, 1, %0;" : "+l"(sum) : "r"((uint32_t)max(v, 0))); };
+    int i = tid;
+    if ((reinterpret_cast<uintptr_t>(lens) & 15) == 0) {
+        const int4* l4 = reinterpret_cast<const int4*>(lens);
+        const int q = b >> 2;
+        int k = tid;
+        for (; k + 3 * nthr < q; k += 4 * nthr) {       // four loads in flight
+            const int4 x0 = __ldg(l4 + k), x1 = __ldg(l4 + k + nthr), x2 = __ldg(l4 + k + 2 * nthr), x3 = __ldg(l4 + k + 3 * nthr);
+            add(x0.x); add(x0.y); add(x0.z); add(x0.w);
+            add(x1.x); add(x1.y); add(x1.z); add(x1.w);
+            add(x2.x); add(x2.y); add(x2.z); add(x2.w);
+            add(x3.x); add(x3.y); add(x3.z); add(x3.w);
+        }
+        for (; k < q; k += nthr) {
+            const int4 x = __ldg(l4 + k);
+            add(x.x); add(x.y); add(x.z); add(x.w);
+        }
+        i += b & ~3;
+    }
+    for (; i < b; i += nthr) add(__ldg(lens + i));
+    return sum;
+}
+
 __device__ __forceinline__ void atomic_add_mem(int32_t* p, int32_t v) { atomicAdd(p, v); }
 __device__ __forceinline__ void atomic_add_mem(int64_t* p, int64_t v) {
     atomicAdd(reinterpret_cast<unsigned long long*>(p), static_cast<unsigned long long>(v));

@@ -32,12 +32,16 @@
 //   4.  reductions        peak (Section 2), status against the budget.
 //
 // Stage 2 walks the successor tiles of the warp-per-sequence kernel (two node slots per lane, uniform trip counts, packed
-// word offsets; read through L1, a block has no room for a copy) where the graph has them, else a record per node
-// with bounds tests.  Rows are found from the lengths (each block sums those in front of its range), or through `offs`.
-// The kernel is bound by instruction issue and by the barriers between its stages; the threads per sequence
-// follow the batch (quad_shape).  n = 1000, C = 3, B = 4096: 60.5 -> 53.3 us (issue slots 61 % busy, shared-memory data
-// pipe 47 %); n = 5000, C = 3, B = 1024: 93 -> 81 us; n = 442, C = 3, B = 64: 12.4 -> 8.3 us (before: rows through the
-// offsets kernel, every word sorted, a fixed number of threads).
+// word offsets) where the graph has them, else a record per node with bounds tests.  Where a batch leaves room for it
+// (kChip) the block copies records, durations and tiles into its shared memory behind the search for the rows: a
+// batch of a few sequences per SM is a chain of latencies, and every read of the graph from L2 is one of them.  Rows are found from the lengths (each
+// block sums those in front of its range), or through `offs`.
+// The kernel is bound by instruction issue and by the barriers between its stages (four per sequence: behind 1a, 1b, 2
+// and the prefix sum; the words are cleared for the next sequence behind stage 2); the threads per sequence
+// follow the batch (quad_shape).  Cold latencies that were taken out of a small batch: a 64-bit division for the range of a
+// block, sums of the lengths and of the chunks by shuffles and by loops over the warps (now warp reductions), the
+// graph through L2, three barriers.  n = 442, B = 148: C = 2 8.7 -> 6.2 us, C = 3 8.7 -> 6.2, C = 4 10.2 -> 8.2; n = 1000, C = 2, one sequence
+// 10.2 -> 6.1; n = 2192, C = 2 (words of 32 bits), B = 1184 32.5 -> 24.9; n = 5000, C = 3, B = 1024 75.9 -> 71.4; profile of n = 1000 8.2 -> 6.2.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -51,11 +55,14 @@ struct QuadParams {
     int32_t C;                 // 3 or 4 accumulators are compiled; C itself bounds the copy count
     int32_t max_T;             // C * n
     int32_t B;
+    int32_t per_block, spare;  // rows found by the kernel: block c takes per_block sequences, one more when c < spare
     int64_t M;
-    int32_t n_tiles, split;    // as in PairParams
+    int32_t n_tiles, split, small_w;    // as in PairParams
     const void* rec;
     const uint32_t* sell;
     const int32_t* tile_row;   // first row of every tile in `sell`
+    const uint64_t* wslot;     // durations by slot, as in PairParams
+    uint32_t rec_bytes, w_bytes, sell_bytes, row_bytes;   // kChip: sizes of the copies of rec, wslot, sell and tile_row
     const uint4* order;        // without tiles: n records of 32 bytes in order of falling out-degree (below)
     const uint16_t* succ;      // ... and the successors beyond the eighth of the nodes that have more
     const void* m;             // n output sizes, int32 or int64
@@ -71,8 +78,9 @@ struct QuadParams {
     int32_t single_len;        // profile: length of the one sequence at seqs[0..)
     int64_t* out_profile;      // ... usage per step, free step per step (may be null)
     int32_t* out_free;
-    uint32_t word_bytes;       // 8 (n + 2) rounded to 32, and 16 for the word of empty node slots
+    uint32_t word_bytes;       // 8 (n + 2) rounded to 32 (kAcc = 2: 4 (n + 2) rounded to 16), and 16 for the word of empty node slots
     uint32_t cnt_bytes;        // 2 (n + 2), rounded to 16
+    uint32_t delta_bytes;      // the deltas, rounded to 16 (kChip: the graph follows them)
 };
 
 // Node record of `order`: word 0 = node | out-degree << 16 (a sink: 1, its successor the id n + 1), word 1 = index
@@ -105,26 +113,41 @@ __device__ __forceinline__ void quad_store(uint32_t addr, Amount<int64_t> a) {
     asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(addr), "r"(a.lo), "r"(a.hi) : "memory");
 }
 
+// A node's word: four positions, or two where no node may have more (kAcc = 2).
+template <int kAcc> struct QuadWord { uint2 v; };
+template <> struct QuadWord<2> { uint32_t v; };
+template <int kAcc>
+__device__ __forceinline__ QuadWord<kAcc> quad_lds(uint32_t addr) {
+    QuadWord<kAcc> r;
+    if constexpr (kAcc == 2) r.v = lds_u32(addr);
+    else r.v = lds_v2(addr);
+    return r;
+}
+
 // The copies a_1 <= ... of one node and its running reductions over successor words.
 template <int kAcc>
 struct QuadNode {
     uint32_t base[kAcc], na[kAcc], G[kAcc];
     // own word after stage 1b
-    __device__ __forceinline__ void open(uint2 own) {
+    __device__ __forceinline__ void open(QuadWord<kAcc> own) {
         uint32_t last;
-        if constexpr (kAcc == 3) {          // the fourth quarter is a repetition
-            const uint32_t x0 = own.x & 0xFFFFu, x1 = own.x >> 16, x2 = own.y & 0xFFFFu;
+        if constexpr (kAcc == 2) {
+            const uint32_t x0 = own.v & 0xFFFFu, x1 = own.v >> 16;
+            base[0] = min(x0, x1);
+            base[1] = last = max(x0, x1);
+        } else if constexpr (kAcc == 3) {          // the fourth quarter is a repetition
+            const uint32_t x0 = own.v.x & 0xFFFFu, x1 = own.v.x >> 16, x2 = own.v.y & 0xFFFFu;
             const uint32_t lo = min(x0, x1), hi = max(x0, x1), mid = min(hi, x2);
             last = max(hi, x2);
             base[0] = min(lo, mid);
             base[1] = max(lo, mid);
             base[2] = last;
         } else {
-            sort4_u16(own.x, own.y);
-            base[0] = own.x & 0xFFFFu;
-            base[1] = own.x >> 16;
-            base[2] = own.y & 0xFFFFu;
-            base[3] = last = own.y >> 16;
+            sort4_u16(own.v.x, own.v.y);
+            base[0] = own.v.x & 0xFFFFu;
+            base[1] = own.v.x >> 16;
+            base[2] = own.v.y & 0xFFFFu;
+            base[3] = last = own.v.y >> 16;
         }
 #pragma unroll
         for (int j = 0; j < kAcc; ++j) na[j] = 0x00010000u - base[j] * 0x10001u;     // (-a, -a) mod 2^16
@@ -132,11 +155,15 @@ struct QuadNode {
 #pragma unroll
         for (int j = 1; j < kAcc; ++j) G[j] = ((base[j - 1] - base[j]) & 0xFFFFu) * 0x10001u;   // copy j ends at itself at least
     }
-    __device__ __forceinline__ void visit(uint2 r) {
+    __device__ __forceinline__ void visit(QuadWord<kAcc> r) {
 #pragma unroll
         for (int j = 0; j < kAcc; ++j) {
-            G[j] = __viaddmax_u16x2(r.x, na[j], G[j]);
-            G[j] = __viaddmax_u16x2(r.y, na[j], G[j]);
+            if constexpr (kAcc == 2) {
+                G[j] = __viaddmax_u16x2(r.v, na[j], G[j]);
+            } else {
+                G[j] = __viaddmax_u16x2(r.v.x, na[j], G[j]);
+                G[j] = __viaddmax_u16x2(r.v.y, na[j], G[j]);
+            }
         }
     }
     // -m behind the end of every copy (and the ends themselves to `ends`, for a profile); returns a word whose bit 15
@@ -157,27 +184,65 @@ struct QuadNode {
     }
 };
 
-// kAcc: number of copies the node pass keeps apart (3 or 4).
+// Stage 1b for one node: c copies arrived in its word at `wv`; fills the empty places and writes +m at every copy.
+template <typename MemT, int kAcc, int kShift>
+__device__ __forceinline__ void quad_settle(uint32_t wv, uint32_t c, uint32_t dm1, Amount<MemT> mv) {
+    if constexpr (kAcc == 2) {
+        const uint32_t q = lds_u32(wv), x = c == 1 ? q * 0x10001u : q;
+        if (c == 1) sts_u32(wv, x);
+        quad_store(dm1 + ((x & 0xFFFFu) << kShift), mv);
+        if (c > 1) quad_store(dm1 + ((x >> 16) << kShift), mv);
+    } else {
+        const uint2 q = lds_v2(wv);
+        const uint32_t lo = c == 1 ? q.x * 0x10001u : q.x;
+        const uint32_t hi = c < 3 ? lo : (c == 3 ? __byte_perm(q.y, q.x, 0x5410) : q.y);
+        if (c < 4) sts_u64(wv, (uint64_t)lo | ((uint64_t)hi << 32));
+        quad_store(dm1 + ((lo & 0xFFFFu) << kShift), mv);
+        if (c > 1) quad_store(dm1 + ((lo >> 16) << kShift), mv);
+        if (c > 2) quad_store(dm1 + ((hi & 0xFFFFu) << kShift), mv);
+        if (kAcc > 3 && c > 3) quad_store(dm1 + ((hi >> 16) << kShift), mv);
+    }
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t addr) {
+    uint32_t c;
+    asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(c) : "r"(addr) : "memory");
+    return c;
+}
+
+// kAcc: number of copies the node pass keeps apart (2, 3 or 4; C <= kAcc).
 // kProfile: one sequence, whose usage per step and free steps are written out (moc_mem_profile).
-template <typename MemT, int kAcc, bool kTiles, bool kProfile>
+// kChip: the block keeps a copy of the graph's tiles in shared memory.
+template <typename MemT, int kAcc, bool kTiles, bool kProfile, bool kChip>
 __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
+    static_assert(kTiles || !kChip, "only tiles are copied");
     extern __shared__ __align__(16) char smem[];
-    __shared__ int64_t s_dur[32];
+    __shared__ int64_t s_dur[32], s_top[32];
     __shared__ uint32_t s_lo[32], s_hi[32];
-    __shared__ int64_t s_top[32];
-    __shared__ uint32_t s_flags;
     constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
+    constexpr int kWord = kAcc == 2 ? 2 : 3;                // log2 of the bytes of a node's word
     constexpr uint32_t kFull = 0xFFFFFFFFu;
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, n_warps = nthr >> 5;
     const int warp = __shfl_sync(kFull, tid >> 5, 0);
     int n = p.n;
     MOC_KEEP(n);
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
-    uint32_t wa = sbase, ca = sbase + p.word_bytes, da = ca + p.cnt_bytes;   // words | counters | delta[0..]
+    uint32_t wa = sbase, ca = sbase + p.word_bytes, da = ca + p.cnt_bytes;   // words | counters | delta[0..] | graph
     MOC_KEEP(wa);
     MOC_KEEP(ca);
     MOC_KEEP(da);
     const uint32_t dm1 = da - (uint32_t)sizeof(MemT);
+    const uint32_t recs = da + p.delta_bytes, wsl = recs + p.rec_bytes, sells = wsl + p.w_bytes, rows = sells + p.sell_bytes;   // kChip
+    if constexpr (kChip) {
+        // asynchronous copies: complete behind the search for the rows and, for one sequence, the arrival of its row
+        auto copy = [&](uint32_t to, const void* from, uint32_t bytes) {
+            for (uint32_t i = 16u * (uint32_t)tid; i < bytes; i += 16u * (uint32_t)nthr)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i), "l"(reinterpret_cast<const char*>(from) + i) : "memory");
+        };
+        copy(recs, p.rec, p.rec_bytes);
+        copy(wsl, p.wslot, p.w_bytes);
+        copy(sells, p.sell, p.sell_bytes);
+        copy(rows, p.tile_row, p.row_bytes);
+    }
     auto amount = [&](int v) -> Amount<MemT> {       // m of node v in the form of the deltas
         Amount<MemT> a;
         if constexpr (sizeof(MemT) == 4) {
@@ -189,30 +254,34 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
         }
         return a;
     };
+    // words and counters are zero when a sequence begins (stage 1b writes every delta that the prefix sum reads)
+    auto clear = [&]() {
+        const int4 z = make_int4(0, 0, 0, 0);
+        int4* s4 = reinterpret_cast<int4*>(smem);
+        const int nz = (int)((p.word_bytes + p.cnt_bytes) >> 4);
+        for (int i = tid; i < nz; i += nthr) s4[i] = z;
+    };
 
-    // ---- rows: block c takes [c * B / grid, (c + 1) * B / grid), or every grid-th one with the offsets given
+    // ---- rows: block c takes a contiguous range of the sequences, or every grid-th one with the offsets given
     const bool self = !kProfile && p.offs == nullptr;
-    int b = self ? (int)((int64_t)blockIdx.x * p.B / gridDim.x) : (int)blockIdx.x, b_end = p.B, b_step = gridDim.x;
+    int b = (int)blockIdx.x, b_end = p.B, b_step = gridDim.x;
+    if (self) {
+        b = (int)blockIdx.x * p.per_block + min((int)blockIdx.x, p.spare);
+        b_end = b + p.per_block + ((int)blockIdx.x < p.spare ? 1 : 0);
+        b_step = 1;
+    }
     int64_t off = 0;
     int32_t T_next = kProfile ? p.single_len : (b < p.B ? __ldg(p.lens + b) : 0);      // one sequence ahead
     if (self) {
-        b_end = (int)(((int64_t)blockIdx.x + 1) * p.B / gridDim.x);
-        b_step = 1;
-        int64_t sum = 0;
-        int i = tid;
-        if ((reinterpret_cast<uintptr_t>(p.lens) & 15) == 0) {
-            const int4* l4 = reinterpret_cast<const int4*>(p.lens);
-            for (int k = tid; k < b >> 2; k += nthr) {
-                const int4 x = __ldg(l4 + k);
-                sum += (int64_t)max(x.x, 0) + max(x.y, 0) + max(x.z, 0) + max(x.w, 0);
-            }
-            i += b & ~3;
-        }
-        for (; i < b; i += nthr) sum += max(__ldg(p.lens + i), 0);
-        sum = warp_sum64(sum);
-        if (lane == 0) s_dur[warp] = sum;
+        const uint64_t sum = lengths_before(p.lens, b, tid, nthr);
+        clear();
+        const uint64_t part = warp_sum_u59(sum);
+        if (lane == 0) s_dur[warp] = (int64_t)part;
         __syncthreads();
-        for (int k = 0; k < n_warps; ++k) off += s_dur[k];
+        off = (int64_t)warp_sum_u59(lane < n_warps ? (uint64_t)s_dur[lane] : 0);
+    } else {
+        clear();
+        __syncthreads();
     }
     for (; b < b_end; b += b_step) {
         const int32_t T = T_next;
@@ -221,25 +290,15 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
         if (T >= n && T <= p.max_T) {      // uniform over the block
-            // ---- clear words and counters (stage 1b writes every delta the prefix sum reads)
-            {
-                const int4 z = make_int4(0, 0, 0, 0);
-                int4* s4 = reinterpret_cast<int4*>(smem);
-                const int nz = (int)((p.word_bytes + p.cnt_bytes) >> 4);
-                for (int i = tid; i < nz; i += nthr) s4[i] = z;
-                if (tid == 0) s_flags = 0;
-            }
-            __syncthreads();
-            Amount<MemT> m_next = amount(min(tid, n - 1));          // for stage 1b, one round ahead
             // ---- stage 1a
-            uint32_t flags = 0;    // bit 0: malformed, bit 1: precedence violated
+            uint32_t flags = 0;
             {
                 const int32_t* row = p.seqs + off;
                 auto put = [&](uint32_t id, int t) {
                     if (id < (uint32_t)n) {
                         const uint32_t sh = (id & 1u) << 4;
                         const uint32_t k = (atom_add_shared_u32(ca + ((id >> 1) << 2), 1u << sh) >> sh) & 0xFFFFu;
-                        if (k < 4) sts_u16(wa + (id << 3) + (k << 1), (uint32_t)t + 1u);
+                        if (k < (kAcc == 2 ? 2u : 4u)) sts_u16(wa + (id << kWord) + (k << 1), (uint32_t)t + 1u);
                     } else {
                         flags = 1;
                     }
@@ -253,72 +312,111 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                     put(i2, t + 2 * nthr);
                     put(i3, t + 3 * nthr);
                 }
-                for (; t < T; t += nthr) put((uint32_t)__ldg(row + t), t);
+                if (t < T) {                                   // up to three more
+                    const bool h1 = t + nthr < T, h2 = t + 2 * nthr < T;
+                    const uint32_t i0 = (uint32_t)__ldg(row + t), i1 = h1 ? (uint32_t)__ldg(row + t + nthr) : 0u,
+                                   i2 = h2 ? (uint32_t)__ldg(row + t + 2 * nthr) : 0u;
+                    put(i0, t);
+                    if (h1) put(i1, t + nthr);
+                    if (h2) put(i2, t + 2 * nthr);
+                }
                 if (tid == 0) {
-                    sts_u64(wa + ((uint32_t)(n + 1) << 3), (uint64_t)(uint32_t)T * 0x0001000100010001ull);
-                    sts_u64(wa + p.word_bytes - 16u, 0x0001000100010001ull);      // owned by empty node slots
+                    // the made-up successor of sinks, and the word that empty node slots own
+                    if constexpr (kAcc == 2) {
+                        sts_u32(wa + ((uint32_t)(n + 1) << 2), (uint32_t)T * 0x10001u);
+                        sts_u32(wa + p.word_bytes - 16u, 0x00010001u);
+                    } else {
+                        sts_u64(wa + ((uint32_t)(n + 1) << 3), (uint64_t)(uint32_t)T * 0x0001000100010001ull);
+                        sts_u64(wa + p.word_bytes - 16u, 0x0001000100010001ull);
+                    }
                 }
             }
+            if constexpr (kChip) asm volatile("cp.async.wait_all;" ::: "memory");
             __syncthreads();
             // records and first successor row of a tile are requested while the tile before it (or stage 1b) is worked on
             uint4 r_next[2];
             const uint32_t* ps_next = nullptr;
-            uint32_t e_first = 0;
+            uint32_t ss_next = 0, e_first = 0;
             auto request = [&](int d) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
+                    const int slot = (2 * d + h) * 32 + lane;
                     if constexpr (sizeof(MemT) == 4) {
-                        const uint2 r = __ldg(reinterpret_cast<const uint2*>(p.rec) + (2 * d + h) * 32 + lane);
+                        const uint2 r = kChip ? lds_v2(recs + 8u * (uint32_t)slot) : __ldg(reinterpret_cast<const uint2*>(p.rec) + slot);
                         r_next[h].x = r.x;
                         r_next[h].z = r.y;
                     } else {
-                        r_next[h] = __ldg(reinterpret_cast<const uint4*>(p.rec) + (2 * d + h) * 32 + lane);
+                        r_next[h] = kChip ? lds_v4(recs + 16u * (uint32_t)slot) : __ldg(reinterpret_cast<const uint4*>(p.rec) + slot);
                     }
                 }
-                ps_next = p.sell + 32 * __ldg(p.tile_row + d) + lane;
-                e_first = __ldg(ps_next);
+                if constexpr (kChip) {
+                    ss_next = sells + 128u * lds_u32(rows + 4u * (uint32_t)d) + 4u * (uint32_t)lane;
+                    e_first = lds_u32(ss_next);
+                } else {
+                    ps_next = p.sell + 32 * __ldg(p.tile_row + d) + lane;
+                    e_first = __ldg(ps_next);
+                }
             };
-            if (kTiles && warp < p.n_tiles) request(warp);
+            if (kTiles && !kChip && warp < p.n_tiles) request(warp);
             // ---- stage 1b
             int64_t dur = 0;
-            for (int v = tid; v < n; v += nthr) {
-                uint32_t c, limit = (uint32_t)p.C;
-                asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(c) : "r"(ca + 2u * (uint32_t)v) : "memory");
-                if (p.cap != nullptr) limit = min(limit, (uint32_t)__ldg(p.cap + v));
-                const uint2 q = lds_v2(wa + ((uint32_t)v << 3));
-                const Amount<MemT> mv = m_next;
-                m_next = amount(min(v + nthr, n - 1));
-                if (c - 1u >= limit) {       // absent or overfull: its word holds no usable positions
-                    flags |= 1;
-                    continue;
+            if constexpr (kChip) {
+                const int n_halves = 2 * p.n_tiles;
+                for (int hh = warp; hh < n_halves; hh += n_warps) {
+                    const uint32_t slot = 32u * (uint32_t)hh + (uint32_t)lane;
+                    uint32_t x;
+                    Amount<MemT> mv;
+                    if constexpr (sizeof(MemT) == 4) {
+                        const uint2 r = lds_v2(recs + 8u * slot);
+                        x = r.x & 0xFFFFu;
+                        mv.v = (MemT)r.y;
+                    } else {
+                        const uint4 r = lds_v4(recs + 16u * slot);
+                        x = r.x & 0xFFFFu;
+                        mv.lo = r.z;
+                        mv.hi = r.w;
+                    }
+                    const uint32_t wv = wa + (x << (kWord - 2));
+                    if (wv == wa + p.word_bytes - 16u) continue;              // an empty slot
+                    const uint32_t c = lds_u16(ca + (x >> 1));
+                    uint32_t limit = (uint32_t)p.C;
+                    if (p.cap != nullptr) limit = min(limit, (uint32_t)__ldg(p.cap + (x >> 2)));
+                    if (c - 1u >= limit) {       // absent or overfull: its word holds no usable positions
+                        flags |= 1;
+                        continue;
+                    }
+                    if (c > 1) dur += (int64_t)(c - 1) * (int64_t)(lds_u64(wsl + 8u * slot) & kPairDurMask);
+                    quad_settle<MemT, kAcc, kShift>(wv, c, dm1, mv);
                 }
-                if (c > 1) dur += (int64_t)(c - 1) * __ldg(p.w + v);
-                const uint32_t lo = c == 1 ? q.x * 0x10001u : q.x;
-                const uint32_t hi = c < 3 ? lo : (c == 3 ? __byte_perm(q.y, q.x, 0x5410) : q.y);
-                if (c < 4) sts_u64(wa + ((uint32_t)v << 3), (uint64_t)lo | ((uint64_t)hi << 32));
-                quad_store(dm1 + ((lo & 0xFFFFu) << kShift), mv);
-                if (c > 1) quad_store(dm1 + ((lo >> 16) << kShift), mv);
-                if (c > 2) quad_store(dm1 + ((hi & 0xFFFFu) << kShift), mv);
-                if (kAcc > 3 && c > 3) quad_store(dm1 + ((hi >> 16) << kShift), mv);
+            } else {
+                Amount<MemT> m_next = amount(min(tid, n - 1));          // one round ahead
+                for (int v = tid; v < n; v += nthr) {
+                    uint32_t limit = (uint32_t)p.C;
+                    const uint32_t c = lds_u16(ca + 2u * (uint32_t)v);
+                    if (p.cap != nullptr) limit = min(limit, (uint32_t)__ldg(p.cap + v));
+                    const Amount<MemT> mv = m_next;
+                    m_next = amount(min(v + nthr, n - 1));
+                    if (c - 1u >= limit) {
+                        flags |= 1;
+                        continue;
+                    }
+                    if (c > 1) dur += (int64_t)(c - 1) * __ldg(p.w + v);
+                    quad_settle<MemT, kAcc, kShift>(wa + ((uint32_t)v << kWord), c, dm1, mv);
+                }
             }
-            flags = __reduce_or_sync(kFull, flags);
-            dur = warp_sum64(dur);
-            if (lane == 0) {
-                if (flags) atomicOr(&s_flags, flags);
-                s_dur[warp] = dur;
-            }
-            __syncthreads();
-            const bool malformed = (s_flags & 1u) != 0;
+            const bool malformed = __syncthreads_or((int)flags) != 0;
+            bool dep = false;
             if (!malformed) {
                 // ---- stage 2 and the scatter of stage 3
                 uint32_t depw = 0;
                 if constexpr (kTiles) {
+                    if (kChip && warp < p.n_tiles) request(warp);
                     for (int d = warp; d < p.n_tiles; d += n_warps) {
                         QuadNode<kAcc> u[2];
                         Amount<MemT> m[2];
                         const uint32_t x0 = r_next[0].x, x1 = r_next[1].x;
                         const uint32_t* ps = ps_next;
-                        uint32_t e_next = e_first;
+                        uint32_t ss = ss_next, e_next = e_first;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             if constexpr (sizeof(MemT) == 4) {
@@ -327,20 +425,23 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                                 m[h].lo = r_next[h].z;
                                 m[h].hi = r_next[h].w;
                             }
-                            u[h].open(lds_v2(wa + ((r_next[h].x & 0xFFFFu) << 1)));
+                            u[h].open(quad_lds<kAcc>(wa + ((r_next[h].x & 0xFFFFu) << (kWord - 2))));
                         }
                         if (d + n_warps < p.n_tiles) request(d + n_warps);
-                        const int rows = __shfl_sync(kFull, (int)(x0 >> 16), 0);
-                        for (int k = 0; k < rows; ++k) {
+                        const int n_rows = __shfl_sync(kFull, (int)(x0 >> 16), 0);
+                        for (int k = 0; k < n_rows; ++k) {
                             const uint32_t e = e_next;
                             ps += 32;
-                            if (k + 1 < rows) e_next = __ldg(ps);
-                            const uint2 r0 = lds_v2(wa + ((e & 0xFFFFu) << 1)), r1 = lds_v2(wa + ((e >> 16) << 1));
+                            ss += 128u;
+                            if (k + 1 < n_rows) e_next = kChip ? lds_u32(ss) : __ldg(ps);
+                            const QuadWord<kAcc> r0 = quad_lds<kAcc>(wa + ((e & 0xFFFFu) << (kWord - 2))),
+                                                 r1 = quad_lds<kAcc>(wa + ((e >> 16) << (kWord - 2)));
                             u[0].visit(r0);
                             u[1].visit(r1);
                         }
                         // an empty node slot owns the last word of the area: no step is its own
-                        const bool real0 = !kProfile || (x0 & 0xFFFFu) << 1 != p.word_bytes - 16u, real1 = !kProfile || (x1 & 0xFFFFu) << 1 != p.word_bytes - 16u;
+                        const uint32_t none = (p.word_bytes - 16u) >> (kWord - 2);
+                        const bool real0 = !kProfile || (x0 & 0xFFFFu) != none, real1 = !kProfile || (x1 & 0xFFFFu) != none;
                         depw |= u[0].template close<MemT, kShift, kProfile>(da, m[0], p.out_free, real0 && p.out_free != nullptr);
                         depw |= u[1].template close<MemT, kShift, kProfile>(da, m[1], p.out_free, real1 && p.out_free != nullptr);
                     }
@@ -358,32 +459,31 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                         }
                         const int rounds = __reduce_max_sync(kFull, (int)deg);
                         QuadNode<kAcc> u;
-                        u.open(lds_v2(wa + (node << 3)));
+                        u.open(quad_lds<kAcc>(wa + (node << kWord)));
                         const uint32_t in8[4] = {inl.x, inl.y, inl.z, inl.w};
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
                             if (k < rounds) {
-                                if ((uint32_t)k < deg) u.visit(lds_v2(wa + (((k & 1) ? in8[k >> 1] >> 16 : in8[k >> 1] & 0xFFFFu) << 3)));
+                                if ((uint32_t)k < deg) u.visit(quad_lds<kAcc>(wa + (((k & 1) ? in8[k >> 1] >> 16 : in8[k >> 1] & 0xFFFFu) << kWord)));
                             }
                         }
                         for (int k = 8; k < rounds; ++k)
-                            if ((uint32_t)k < deg) u.visit(lds_v2(wa + ((uint32_t)__ldg(p.succ + e8 + (k - 8)) << 3)));
+                            if ((uint32_t)k < deg) u.visit(quad_lds<kAcc>(wa + ((uint32_t)__ldg(p.succ + e8 + (k - 8)) << kWord)));
                         if (i < n) depw |= u.template close<MemT, kShift, kProfile>(da, amount((int)node), p.out_free, p.out_free != nullptr);
                     }
                 }
-                if (__any_sync(kFull, (depw & 0x8000u) != 0) && lane == 0) atomicOr(&s_flags, 2u);
+                dep = __syncthreads_or((int)(depw & 0x8000u)) != 0;
+                // per-warp sums of the durations, read behind the next barrier
+                const int64_t dw = p.small_w ? (int64_t)__reduce_add_sync(kFull, (uint32_t)dur) : warp_sum64(dur);
+                if (lane == 0) s_dur[warp] = dw;
             }
-            __syncthreads();
-            const uint32_t fl = s_flags;
-            if (!(fl & 1u)) {
-                out_du = p.base_dur;
-                for (int k = 0; k < n_warps; ++k) out_du += s_dur[k];
-                out_st = -1;
-            }
-            if (fl == 0) {
-                // ---- stages 3 and 4: prefix sum, each thread a chunk of consecutive steps (odd length: no bank conflicts)
-                const int chunk = ((T + nthr - 1) / nthr) | 1;
-                const int tb = min(tid * chunk, T), te = min(tb + chunk, T);
+            if (b + b_step < b_end) clear();       // for the next sequence: nothing reads the words any more
+            const int chunk = ((T + nthr - 1) / nthr) | 1;
+            const int tb = min(tid * chunk, T), te = min(tb + chunk, T);
+            uint32_t lo_in = 0, hi_in = 0;          // deltas of the warp's threads in front of this one
+            if (!malformed && !dep) {
+                // ---- stages 3 and 4: prefix sum, each thread a chunk of consecutive steps (odd length: no bank conflicts);
+                // a warp's largest usage counts from the usage in front of the warp
                 uint32_t ad = da + ((uint32_t)tb << kShift), lo = 0, hi = 0;
                 MemT top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
                 for (int t = tb; t < te; ++t, ad += (uint32_t)sizeof(MemT)) {
@@ -399,62 +499,66 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                     }
                     top = at > top ? at : top;
                 }
-                // chunk sums -> usage in front of every chunk; a thread without steps passes its prefix on
-                uint32_t lo_in = warp_inclusive_sum(lo, lane), hi_in = 0;
+                lo_in = warp_inclusive_sum(lo, lane);
                 if constexpr (sizeof(MemT) == 8) hi_in = warp_inclusive_sum(hi, lane);
                 if (lane == 31) {
                     s_lo[warp] = lo_in;
                     s_hi[warp] = hi_in;
                 }
-                __syncthreads();
                 lo_in -= lo;
                 hi_in -= hi;
-                for (int k = 0; k < warp; ++k) {
-                    lo_in += s_lo[k];
-                    if constexpr (sizeof(MemT) == 8) hi_in += s_hi[k];
-                }
                 MemT before;
                 if constexpr (sizeof(MemT) == 4) before = (MemT)lo_in;
                 else before = split_value(lo_in, hi_in, p.split);
-                MemT peak = tb < te ? before + top : MemT(0);
-                if constexpr (kProfile) {
-                    ad = da + ((uint32_t)tb << kShift);
-                    lo = lo_in;
-                    hi = hi_in;
-                    for (int t = tb; t < te; ++t, ad += (uint32_t)sizeof(MemT)) {
-                        if constexpr (sizeof(MemT) == 4) {
-                            lo += lds_u32(ad);
-                            p.out_profile[t] = (int64_t)(MemT)lo;
-                        } else {
-                            const uint2 q = lds_v2(ad);
-                            lo += q.x;
-                            hi += q.y;
-                            p.out_profile[t] = split_value(lo, hi, p.split);
+                // a thread without steps counts nothing (the first step of the warp is one of the others', or the warp's usage in front)
+                MemT w_top = warp_max_t(tb < te ? (MemT)(before + top) : (sizeof(MemT) == 8 ? (MemT)(INT64_MIN / 4) : (MemT)INT32_MIN));
+                if (lane == 0) s_top[warp] = (int64_t)w_top;
+            }
+            __syncthreads();
+            if (!malformed) {
+                if (warp == 0) out_du = p.base_dur + warp_sum64(lane < n_warps ? s_dur[lane] : 0);
+                out_st = -1;
+                if (!dep) {
+                    if (kProfile || warp == 0) {
+                        // usage in front of every warp
+                        uint32_t lo_w = lane < n_warps ? s_lo[lane] : 0u, hi_w = lane < n_warps ? s_hi[lane] : 0u;
+                        const uint32_t lo_i = warp_inclusive_sum(lo_w, lane) - lo_w, hi_i = sizeof(MemT) == 8 ? warp_inclusive_sum(hi_w, lane) - hi_w : 0u;
+                        MemT in_front;
+                        if constexpr (sizeof(MemT) == 4) in_front = (MemT)lo_i;
+                        else in_front = split_value(lo_i, hi_i, p.split);
+                        // a warp without steps holds the smallest value and stays below the others (which are usages, 0 or more)
+                        const MemT pk = warp_max_t(lane < n_warps && s_top[lane] > (sizeof(MemT) == 8 ? INT64_MIN / 4 : (int64_t)INT32_MIN)
+                                                       ? (MemT)(in_front + (MemT)s_top[lane]) : MemT(0));
+                        out_pk = (int64_t)pk;
+                        out_st = out_pk <= p.M ? 1 : 0;
+                        if constexpr (kProfile) {
+                            uint32_t lo = __shfl_sync(kFull, lo_i, warp) + lo_in, hi = __shfl_sync(kFull, hi_i, warp) + hi_in,
+                                     ad = da + ((uint32_t)tb << kShift);
+                            for (int t = tb; t < te; ++t, ad += (uint32_t)sizeof(MemT)) {
+                                if constexpr (sizeof(MemT) == 4) {
+                                    lo += lds_u32(ad);
+                                    p.out_profile[t] = (int64_t)(MemT)lo;
+                                } else {
+                                    const uint2 q = lds_v2(ad);
+                                    lo += q.x;
+                                    hi += q.y;
+                                    p.out_profile[t] = split_value(lo, hi, p.split);
+                                }
+                            }
                         }
                     }
-                }
-                peak = warp_max_t(peak);
-                if (lane == 0) s_top[warp] = (int64_t)peak;
-                __syncthreads();
-                if (tid == 0) {
-                    out_pk = s_top[0];
-                    for (int k = 1; k < n_warps; ++k) out_pk = s_top[k] > out_pk ? s_top[k] : out_pk;
-                    out_st = out_pk <= p.M ? 1 : 0;
                 }
             }
         }
         if constexpr (kProfile) {
-            if (tid == 0) s_flags = (uint32_t)out_st;      // only thread 0 knows 0 or 1; nothing reads the flags any more
-            __syncthreads();
-            const int32_t st = (int32_t)s_flags;
-            if (tid == 0) p.out_status[0] = st;
-            if (st < 0) {
+            if (tid == 0) p.out_status[0] = out_st;
+            if (out_st < 0) {
                 for (int t = tid; t < T; t += nthr) {
                     p.out_profile[t] = -1;
                     if (p.out_free) p.out_free[t] = -1;
                 }
             }
-            return;
+            break;
         }
         if (tid == 0) {
             p.out_peak[b] = out_pk;
@@ -462,8 +566,8 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
             p.out_status[b] = out_st;
         }
         off += max(T, 0);
-        __syncthreads();    // the state is reused by the next sequence
     }
+    if constexpr (kChip) asm volatile("cp.async.wait_all;" ::: "memory");      // nothing under way where no sequence was evaluated
 }
 
 }  // namespace moc

@@ -106,6 +106,25 @@ def test_small_batches_and_two_part_sums(B, n, C, bits, nB):
         assert_batch_equal(G, O, seqs, lens, M, f"n {n}, thread groups")
 
 
+@pytest.mark.parametrize("n,C,bits,nB", [(20, 3, 0, 1), (63, 3, 37, 148), (64, 4, 0, 149), (65, 3, 0, 444), (65, 4, 37, 445), (440, 2, 0, 149),
+                                         (441, 3, 20, 296), (700, 4, 0, 297), (701, 3, 0, 148), (701, 3, 0, 149), (2111, 4, 20, 9), (4000, 2, 0, 20), (4001, 2, 0, 20)])
+def test_block_kernel_with_and_without_its_own_copy_of_the_graph(B, n, C, bits, nB):
+    """Batches on both sides of the line between the block kernel's two variants, ends of tiles of 64 nodes, packed rows
+    and rows at given offsets (the entry point that does not allocate)."""
+    edges = W.layered_dag(n, 3 * n, max(4, n // 40), n)
+    w, m = W.weights_uniform(n, 0, 30, n, 1), np.minimum(W.weights_lognormal(n, 3.0, 1.0, n, 2), 255) << bits
+    seqs, lens = W.schedules(n, edges, C, 0.3, nB, n)
+    seqs, lens = W.mutate(seqs, lens, n, C, seed=5, frac=1 / 8)
+    O, G = OracleGraph(n, edges, w, m, C), B.Graph(n, edges, w, m, C)
+    M = O.eval(np.arange(n), 1 << 62)["peak"] * 90 // 100
+    want = assert_batch_equal(G, O, seqs, lens, M, f"n {n}")
+    out = tuple(torch.full((nB,), 77, dtype=d, device="cuda") for d in (torch.int64, torch.int64, torch.int32))
+    B.moc_eval_batch_noalloc(G.h, dev(seqs), dev(lens), M, *out)
+    torch.cuda.synchronize()
+    for a, b in zip(out, want):
+        assert (a.cpu().numpy() == b).all()
+
+
 # ------------------------------------------------------------------ the five configurations
 SMALL_B = [1024, 4096, 2048, 512, 64]
 

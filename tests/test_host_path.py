@@ -308,6 +308,17 @@ def test_which_kernel_makes_a_profile(fake, n, C, scale, star):
     G.close()
 
 
+@pytest.mark.parametrize("n,C,nB,kernel", [(65, 3, 444, "ILi3ELb1ELb0ELb1E"), (65, 3, 445, "ILi3ELb1ELb0ELb0E"), (700, 4, 444, "ILi4ELb1ELb0ELb1E"),
+                                           (701, 4, 148, "ILi4ELb1ELb0ELb1E"), (701, 4, 149, "ILi4ELb1ELb0ELb0E"), (442, 2, 148, "ILi2ELb1ELb0ELb1E"),
+                                           (4000, 2, 148, "ILi2ELb1ELb0ELb1E"), (4001, 2, 148, "ILi2ELb1ELb0ELb0E")])
+def test_the_block_kernel_copies_the_graph_for_small_batches(fake, n, C, nB, kernel):
+    G, x = Graph(fake, n, C), np.zeros(8, np.int64)
+    fake.fake_reset(0)
+    assert fake.moc_eval_batch(G.h, x.ctypes.data, x.ctypes.data, nB, 0, x.ctypes.data, x.ctypes.data, x.ctypes.data, None) == 0
+    assert len(launched(fake, "eval_quad_kernel" + kernel.replace("I", "Ii", 1))) == 1, log(fake)
+    G.close()
+
+
 @pytest.mark.parametrize("n,scale,star", [(1, 1, False), (20, 1, False), (128, 1 << 30, False), (442, 1, False), (601, 1, True)])
 def test_host_allocations_that_fail(fake, n, scale, star):
     """Every allocation on the host fails in turn: MOC_ERR_NOMEM, no exception across the C ABI, nothing left behind."""
