@@ -228,6 +228,46 @@ bool warp_serves(const moc_graph* g) {
     return g->C <= 2 && g->d_rec32 != nullptr && (!wide || g->split_ok) && (__int128)g->C * g->sum_w < ((__int128)1 << 48);
 }
 
+// Shared memory of the warp-per-sequence kernel: the graph once per block, the state of every sequence in flight.
+void pair_bytes(const moc_graph* g, Plan* pl) {
+    const size_t n = (size_t)g->n, msz = pl->wide ? 8 : 4, per_vec = 16 / msz;
+    const size_t nvec_d = (g->C * n + 2 + per_vec - 1) / per_vec, v_max = ((nvec_d + 31) / 32) | 1;
+    pl->rec_bytes = (uint32_t)((pl->wide ? 16 : 8) * 64 * (size_t)g->n_tiles);
+    pl->w_bytes = (uint32_t)(8 * 64 * (size_t)g->n_tiles);
+    pl->sell_bytes = (uint32_t)align16(4 * (size_t)g->sell_len);
+    pl->word_bytes = (uint32_t)align16(4 * (n + 2));
+    pl->delta_bytes = (uint32_t)(moc::kPairDeltaFront + 32 * v_max * 16);
+    pl->pair_graph_b = (size_t)pl->rec_bytes + pl->w_bytes + pl->sell_bytes;
+    pl->pair_warp_b = (size_t)pl->word_bytes + moc::kPairWordTail + pl->delta_bytes;
+}
+
+// Warps that share a sequence in the warp-per-sequence kernel, for batches that leave most of an SM's warps without
+// a sequence of their own (1: none do), and the shape of the launch: one block per SM, up to 16 warps.  Sharing divides the
+// latency of a sequence and costs barriers; with more than eight sequences on an SM the warps have enough to do (n = 1000, 12 per SM:
+// 15.7 us without, 14.6 with two; n = 250, 64-bit sums 9.0 and 10.4).  Measured with 1 / 2 / 4 / 8 warps on a sequence (us; 32-bit sums): n = 153, B = 296
+// 7.2 (before) / 6.1 / 6.0; n = 353, B = 592 8.3 / 6.4 / 6.4; n = 600, B = 148 10.4 / 8.3 / 6.3 / 6.0; n = 1000, B = 592 12.5 / 10.4 / 8.4; B = 1184 14.5 / 12.4;
+// with 8 / 16: n = 1000, B = 148 6.2 / 6.2, n = 1400 6.9 / 6.6, n = 5000 12.0 / 10.4.
+struct TeamShape {
+    int team = 1, groups = 0, grid = 0;
+};
+TeamShape team_shape(const moc_graph* g, int32_t B) {
+    TeamShape s;
+    if (!warp_serves(g) || g->want_gpc || g->want_G || (g->want_kind != MOC_KERNEL_AUTO && g->want_kind != MOC_KERNEL_WARP)) return s;
+    Plan pl;
+    pl.wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    pair_bytes(g, &pl);
+    const int64_t per_sm = ((int64_t)B + g->sm_count - 1) / g->sm_count;
+    for (int team = 16; team > 1; team >>= 1) {
+        if (per_sm * team > 16 || team > g->n_tiles || g->n < (team == 16 ? 1400 : team == 8 ? 600 : 0)) continue;
+        if (pl.pair_graph_b + per_sm * pl.pair_warp_b + 2048 > g->smem_optin) return s;
+        s.team = team;
+        s.groups = (int)per_sm;
+        s.grid = std::min(B, g->sm_count);
+        return s;
+    }
+    return s;
+}
+
 // Chooses kernel variant, group size and grid for the handle's current n and C.  The dynamic
 // shared-memory limit of a kernel is a property of the kernel, not of the handle: it is always
 // raised to the device maximum, so that handles with different needs can share one kernel.
@@ -272,13 +312,8 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         return fail(MOC_ERR_ARG, "the warp-per-sequence kernel cannot serve this graph (C > 2, degrees too uneven, C * sum(w) >= 2^48 or sum(m) too large)");
     if (!profile && g->want_G == 0 && kind != MOC_KERNEL_GROUP && warp_ok) {
         // warp-per-sequence fast path
-        const size_t msz = pl.wide ? 8 : 4, per_vec = 16 / msz;
-        const size_t nvec_d = (t_max + 2 + per_vec - 1) / per_vec;
-        const size_t v_max = ((nvec_d + 31) / 32) | 1;
-        const size_t rec_b = (pl.wide ? 16 : 8) * 64 * (size_t)g->n_tiles, jds_b = align16(4 * (size_t)g->sell_len),
-                     word_b = align16(4 * (n + 2)), delta_b = moc::kPairDeltaFront + 32 * v_max * 16;
-        const size_t w_b = 8 * 64 * (size_t)g->n_tiles;
-        const size_t graph_b = rec_b + w_b + jds_b, warp_b = word_b + moc::kPairWordTail + delta_b;
+        pair_bytes(g, &pl);
+        const size_t graph_b = pl.pair_graph_b, warp_b = pl.pair_warp_b;
         // vectors of the next row fetched ahead per lane: enough for a typical row of about 1.3 n steps
         const int pre = n < 256 ? 0 : (int)std::min<int64_t>(5, (n * 13 / 10 + 96) / 128);
         PairFn fn = pair_fn(pl.wide, pre);
@@ -294,10 +329,8 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
             pl.pair_nb[wpb] = nb;
             if (nb * wpb > best_warps) { best_warps = nb * wpb; best_wpb = wpb; best_nb = nb; }
         }
-        pl.pair_graph_b = graph_b;
-        pl.pair_warp_b = warp_b;
         pl.sm_count = g->sm_count;
-        if (best_warps >= 8) {
+        if (best_warps >= 10) {
             pl.pair = true;
             pl.pair_fn = fn;
             pl.G = 32;
@@ -305,15 +338,14 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
             pl.block = 32 * best_wpb;
             pl.smem = graph_b + best_wpb * warp_b;
             pl.grid = g->sm_count * best_nb;
-            pl.rec_bytes = (uint32_t)rec_b; pl.w_bytes = (uint32_t)w_b;
-            pl.sell_bytes = (uint32_t)jds_b; pl.word_bytes = (uint32_t)word_b; pl.delta_bytes = (uint32_t)delta_b;
             pl.valid = true;
             *out = pl;
             return MOC_OK;
         }
     }
-    // sequences too long for eight warps of the warp-per-sequence kernel on an SM (n = 2000, B = 2000: 69.6 us with a
-    // thread group per sequence, 53.5 with the block-per-sequence kernel)
+    // Sequences too long for ten warps of the warp-per-sequence kernel on an SM: warp / block with 16 warps 18.6 / 24.7 us (n = 1000, 32-bit
+    // sums, B = 2368), with 14 37.0 / 39.1 (700, 64 bits, 4736), with 11 45.1 / 51.2 (1432, 32 bits, 3919), with 9 43.8 / 42.4 (1000, 64 bits,
+    // 3552), with 6 61.8 / 30.9 (1400, 64 bits, 1776)
     if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, profile, false, &pl)) {
         *out = pl;
         return MOC_OK;
@@ -662,9 +694,11 @@ void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::ve
             // a list that is used up continues with the node's own word
             std::vector<uint32_t> sell((size_t)std::max<int64_t>(sell_len, 1), word_b | (word_b << 16));
             auto own_word = [&](int32_t v) { return v >= 0 ? 4u * (uint32_t)v : word_b; };
+            std::vector<int32_t> tile_row((size_t)n_tiles, 0);
+            for (int32_t d = 1; d < n_tiles; ++d) tile_row[d] = tile_row[d - 1] + rows[d - 1];
             for (size_t r = 0; r < slot.size(); ++r) {
                 const int32_t v = slot[r];
-                const uint32_t x = own_word(v) | ((uint32_t)rows[r / 64] << 16);
+                const uint32_t x = own_word(v) | ((uint32_t)((r & 32) ? tile_row[r / 64] : rows[r / 64]) << 16);
                 const uint64_t mv = v >= 0 ? (uint64_t)m[v] : 0;
                 rec32[2 * r + 0] = x;
                 rec32[2 * r + 1] = v >= 0 ? (uint32_t)m32[v] : 0u;
@@ -712,8 +746,6 @@ void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::ve
                 }
                 pos += 32 * (uint32_t)rows[d];
             }
-            std::vector<int32_t> tile_row((size_t)n_tiles, 0);
-            for (int32_t d = 1; d < n_tiles; ++d) tile_row[d] = tile_row[d - 1] + rows[d - 1];
             // the same tiles for the interval checker: its padding repeats a successor, a sink reads its own word
             std::vector<uint32_t> sell_iv(sell);
             for (size_t r = 0; r < slot.size(); ++r) {
@@ -843,7 +875,12 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
     int grid = (int)std::min<int64_t>(pl.grid, ((int64_t)B + pl.gpc - 1) / pl.gpc);   // lane path: gpc = sequences per group
     int block = pl.block;
     size_t smem = pl.smem;
-    if (pl.pair) {
+    const TeamShape team = pl.pair_team ? team_shape(g, B) : TeamShape();
+    if (pl.pair_team) {
+        grid = team.grid;
+        block = 32 * team.team * team.groups;
+        smem = pl.pair_graph_b + (size_t)team.groups * pl.pair_warp_b;
+    } else if (pl.pair) {
         // Shape of this launch.  A warp works through its sequences one after the other, so a launch
         // takes ceil(sequences per block / warps per block) rounds, and a round costs about as much as
         // the SM has warps (the kernel is bound by on-chip throughput) but never less than a round of a
@@ -945,6 +982,9 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         q.word_bytes = pl.word_bytes; q.delta_bytes = pl.delta_bytes;
         q.split = g->split;
         q.small_w = g->sum_w < ((int64_t)1 << 32) ? 1 : 0;
+        q.per_block = B / grid;
+        q.spare = B % grid;
+        q.team = team.team;
         MOC_CUDA(cudaLaunchKernelEx(&cfg, pl.pair_fn, q));
     } else {
         moc::EvalParams p = base_params(g, pl);
@@ -971,15 +1011,11 @@ bool rows_without_scratch(const Plan& pl, int32_t B) {
     return (pl.pair || pl.lane || pl.quad) && (int64_t)pl.grid * B * 2 <= (int64_t)16 << 20;
 }
 
-// Where the warp-per-sequence kernel serves the graph, the block-per-sequence kernel still
-// takes the batches in which a warp's latency decides (a sequence has several warps there) and the long sequences,
-// whose state leaves too few warps on an SM (make_plan).  Measured at C = 2, warp / block: n = 442 10.4 / 8.8 us at B = 148,
-// 10.3 / 10.3 at 296, 10.4 / 12.4 at 600; n = 1000 16.5 / 10.3 at 296, 16.5 / 14.5 at 600, 16.5 / 16.5 at 1000, 18.6 / 26.8
-// at 2000; n = 1500 36 / 37 at 2000.
+// Where the warp-per-sequence kernel serves the graph, the block-per-sequence kernel still takes middle-sized graphs while
+// every SM has one sequence: as fast as eight or four warps on a sequence there (n = 442: 5.7 / 5.8 us at B = 1, 5.9 / 5.8 at 37,
+// 6.3 / 6.3 at 148), slower beyond (6.9 / 6.3 at 296; n = 1000, B = 148 8.0 / 6.4).
 bool block_serves(const moc_graph* g, int32_t B) {
-    if (g->want_kind != MOC_KERNEL_AUTO || g->want_G || !warp_serves(g)) return false;
-    const int64_t n = g->n, sm = g->sm_count;
-    return (n >= 700 && B <= 6 * sm) || (n >= 400 && B <= 2 * sm);
+    return g->want_kind == MOC_KERNEL_AUTO && !g->want_G && warp_serves(g) && g->n >= 400 && g->n < 600 && B <= g->sm_count;
 }
 
 // The plan for a batch of B, made when a batch first needs it: looking a kernel up loads it, and a kernel that is never
@@ -1010,11 +1046,28 @@ const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
         if (const Plan* pl = quad(g->plan_chip, true)) return pl;
     if (block)
         if (const Plan* pl = quad(g->plan_block, false)) return pl;
+    if (team_shape(g, B).team > 1) {
+        Plan& kept = g->plan_team;
+        if (!kept.valid) {
+            Plan pl;
+            pl.wide = wide;
+            pair_bytes(g, &pl);
+            pl.pair_fn = pair_fn(wide, -1);
+            pl.pair = pl.pair_team = raise_smem_limit((const void*)pl.pair_fn, g->smem_optin) == cudaSuccess;
+            if (!pl.pair) cudaGetLastError();
+            pl.sm_count = g->sm_count;
+            pl.grid = 2 * g->sm_count;
+            pl.gpc = 1;
+            pl.valid = true;
+            kept = pl;
+        }
+        if (kept.pair) return &kept;
+    }
     if (!g->plan_eval.valid) *rc = make_plan(g, false, &g->plan_eval);
     return *rc == MOC_OK ? &g->plan_eval : nullptr;
 }
 
-void forget_plans(moc_graph* g) { g->plan_eval = g->plan_block = g->plan_chip = g->plan_live = Plan(); }
+void forget_plans(moc_graph* g) { g->plan_eval = g->plan_team = g->plan_block = g->plan_chip = g->plan_live = Plan(); }
 
 int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
                 int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {

@@ -5,13 +5,14 @@ namespace moc_host {
 namespace {
 template <typename MemT>
 PairFn pair_fn_t(int pre) {
+    if (pre < 0) return (PairFn)moc::eval_pair_kernel<MemT, 0, true>;
     switch (pre) {
-        case 0: return (PairFn)moc::eval_pair_kernel<MemT, 0>;
-        case 1: return (PairFn)moc::eval_pair_kernel<MemT, 1>;
-        case 2: return (PairFn)moc::eval_pair_kernel<MemT, 2>;
-        case 3: return (PairFn)moc::eval_pair_kernel<MemT, 3>;
-        case 4: return (PairFn)moc::eval_pair_kernel<MemT, 4>;
-        default: return (PairFn)moc::eval_pair_kernel<MemT, 5>;
+        case 0: return (PairFn)moc::eval_pair_kernel<MemT, 0, false>;
+        case 1: return (PairFn)moc::eval_pair_kernel<MemT, 1, false>;
+        case 2: return (PairFn)moc::eval_pair_kernel<MemT, 2, false>;
+        case 3: return (PairFn)moc::eval_pair_kernel<MemT, 3, false>;
+        case 4: return (PairFn)moc::eval_pair_kernel<MemT, 4, false>;
+        default: return (PairFn)moc::eval_pair_kernel<MemT, 5, false>;
     }
 }
 }  // namespace

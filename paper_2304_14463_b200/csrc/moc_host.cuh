@@ -29,7 +29,7 @@ using IntervalFn = void (*)(const moc::IntervalParams);
 // evaluator in one module, 1.0 ms so).  nullptr: no such variant.
 KernelFn shared_fn(bool wide, int G, int CP, bool profile);
 KernelFn global_fn(int CP, bool profile);
-PairFn pair_fn(bool wide, int pre);
+PairFn pair_fn(bool wide, int pre);      // pre < 0: several warps per sequence
 LaneFn lane_fn(bool wide, int lg, int kp);
 QuadFn quad_fn(bool wide, int C, bool tiles, bool chip, bool profile);
 LiveFn live_fn(bool wide, int words, int C);
@@ -50,8 +50,9 @@ struct Plan {
     uint32_t cnt_bytes = 0, occ_bytes = 0, delta_bytes = 0, group_bytes = 0;
     // fast path for C <= 2: a warp per sequence, graph staged in shared memory
     bool pair = false;
+    bool pair_team = false;        // several warps per sequence (team_shape)
     PairFn pair_fn = nullptr;
-    uint32_t rec_bytes = 0, w_bytes = 0, sell_bytes = 0, word_bytes = 0;
+    uint32_t rec_bytes = 0, w_bytes = 0, sell_bytes = 0, word_bytes = 0;   // delta_bytes: above
     // blocks per SM the fast path reaches with 1..16 warps per block (0: does not fit), and its sizes
     int pair_nb[17] = {0};
     size_t pair_graph_b = 0, pair_warp_b = 0;
@@ -163,6 +164,7 @@ struct moc_graph {
     mutable moc_host::Plan plan_eval, plan_profile;
     mutable moc_host::Plan plan_block;    // block-per-sequence kernel beside the warp-per-sequence one in plan_eval
     mutable moc_host::Plan plan_chip;     // ... and the same with the graph in shared memory, for small batches
+    mutable moc_host::Plan plan_team;     // warp-per-sequence kernel with several warps on each
     mutable moc_host::Plan plan_live;     // backward walk beside either
     mutable int64_t* d_offs = nullptr;
     mutable size_t offs_cap = 0;

@@ -57,17 +57,20 @@ struct PairParams {
     const int32_t* lens;
     const int64_t* offs;       // exclusive prefix sum of the lengths, or nullptr: the kernel finds the rows itself
     int32_t B;
+    int32_t per_block, spare;  // rows found by the kernel: block c takes per_block sequences, one more when c < spare
+    int32_t team;              // kTeam: warps per sequence (a divisor of the block's warps)
     int64_t M;
     int64_t* out_peak;
     int64_t* out_dur;
     int32_t* out_status;
     // shared-memory layout, bytes (multiples of 16)
     uint32_t rec_bytes, w_bytes, sell_bytes;     // graph, once per block
-    uint32_t word_bytes, delta_bytes;            // per warp; 16 bytes after the words hold the constant (1, 1)
+    uint32_t word_bytes, delta_bytes;            // per sequence in flight; 16 bytes after the words hold the constant (1, 1)
     int32_t split;                               // 64-bit sums: position k of the high part of an amount (below)
 };
 
-// Node record: {byte offset of the node's word | rows of the tile << 16, m}; m takes 32 bits, or, for 64-bit
+// Node record: {byte offset of the node's word | x << 16, m}, where x is, in a tile's first half, the rows of the tile and, in its
+// second, its first row in `sell` (which has fewer than 2^15); m takes 32 bits, or, for 64-bit
 // sums, two words after a pad word: m mod 2^32 and m >> k.
 //
 // 64-bit sums without 64-bit atomics (which shared memory emulates with compare-and-swap loops: twice the time
@@ -180,40 +183,58 @@ __device__ __forceinline__ void sts_u16_if_nonzero(uint32_t old, uint32_t addr, 
 #define MOC_KEEP(x) asm volatile("" : "+r"(x))
 
 
-// Bound: the shared-memory data pipe (76 % of one wavefront per clock, 528 wavefronts per sequence) and instruction issue
-// (66 %, 1750 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 43.0 -> 41.0 us (duration
-// and copy count by two warp reductions instead of ten 64-bit shuffles, row offsets added up once per sequence,
-// deltas cleared by the scan that reads them).  n = 353 with 64-bit sums, B = 1501: 18.4 -> 12.3 us (sums in two parts,
-// batch spread over all SMs).
+// Barrier of the warps that share a sequence.
+template <bool kTeam>
+__device__ __forceinline__ void team_sync(int id, int threads) {
+    if constexpr (kTeam) asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+    else __syncwarp();
+}
+
+// Bound, large batches: the shared-memory data pipe (three quarters of one wavefront per clock, about 520 wavefronts per
+// sequence) and instruction issue (1700 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 41.0 -> 39.7 us (four
+// exchanges in flight before their results are looked at, ragged ends of a row through the same code, no second search for
+// the end of the row).  Bound, small batches: a chain of latencies; the division for a block's range, the sums of the
+// lengths by shuffles and loops, and the copy of the graph behind one another were half of it (n = 20, B = 1024: 6.15 -> 5.9 us,
+// where the host's calls are what is left; n = 442, B = 592 10.2 -> 7.3; n = 1000, B = 592 12.3 -> 8.4, the latter two with kTeam).
 //
 // kPre: how many 16-byte vectors of the next row each lane fetches ahead (rows of about 128*kPre
 // steps; 0 for short rows, where the extra registers cost more than the wait).  Blocks have up to 16
 // warps and two of them share an SM (62 registers per thread, no spills).
-template <typename MemT, int kPre>
+//
+// kTeam: p.team warps share a sequence, for batches that leave most of an SM's warps without one: the latency of a
+// sequence is then what counts, and the row, the tiles and the scan are dealt to the warps.
+template <typename MemT, int kPre, bool kTeam>
 __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
+    static_assert(!kTeam || kPre == 0, "a team has one sequence at a time and fetches nothing ahead");
     extern __shared__ __align__(16) char smem[];
     __shared__ int64_t s_part[16];
+    __shared__ uint64_t s_acc[16];               // kTeam: what the warps of a sequence tell one another
+    __shared__ uint32_t s_flag[16], s_lo[16], s_hi[16];
+    __shared__ int64_t s_top[16];
     constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u;
+    constexpr uint32_t kFull = 0xFFFFFFFFu;
     // ---- graph -> shared memory, once per block: records | durations | successor tiles.  Asynchronous copies: they
     // complete behind the search for the rows (a launch of few sequences is a chain of such latencies).
     const uint32_t graph_bytes = p.rec_bytes + p.w_bytes + p.sell_bytes;
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
     {
-        const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
-        const uint32_t n_rec = p.rec_bytes >> 4, n_w = p.w_bytes >> 4, n_all = graph_bytes >> 4;
-        for (uint32_t i = threadIdx.x; i < n_all; i += blockDim.x) {
-            const void* src = i < n_rec ? (const void*)(reinterpret_cast<const int4*>(p.rec) + i)
-                                        : i < n_rec + n_w ? (const void*)(reinterpret_cast<const int4*>(p.wslot) + (i - n_rec))
-                                                          : (const void*)(reinterpret_cast<const int4*>(p.sell) + (i - n_rec - n_w));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s0 + 16u * i), "l"(src) : "memory");
-        }
+        auto copy = [&](uint32_t to, const void* from, uint32_t bytes) {
+            for (uint32_t i = 16u * threadIdx.x; i < bytes; i += 16u * blockDim.x)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i), "l"(reinterpret_cast<const char*>(from) + i) : "memory");
+        };
+        copy(sbase, p.rec, p.rec_bytes);
+        copy(sbase + p.rec_bytes, p.wslot, p.w_bytes);
+        copy(sbase + p.rec_bytes + p.w_bytes, p.sell, p.sell_bytes);
     }
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     // broadcast from lane 0 so that the compiler knows the warp index is uniform across the warp
-    const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
-    char* ws = smem + graph_bytes + (size_t)warp * (p.word_bytes + kPairWordTail + p.delta_bytes);
+    const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    // sequences in flight per block, this warp's, and its place among the warps of that one
+    const int tw = kTeam ? p.team : 1, group = kTeam ? warp / tw : warp, wt = kTeam ? warp - group * tw : 0, groups = kTeam ? wpb / tw : wpb;
+    const int tl = 32 * wt + lane, tn = 32 * tw;
+    char* ws = smem + graph_bytes + (size_t)group * (p.word_bytes + kPairWordTail + p.delta_bytes);
     uint32_t* word = reinterpret_cast<uint32_t*>(ws);
     char* delta_base = ws + p.word_bytes + kPairWordTail;          // includes the front pad
-    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
     uint32_t wa = (uint32_t)__cvta_generic_to_shared(word);
     uint32_t da = (uint32_t)__cvta_generic_to_shared(delta_base) + kPairDeltaFront;  // &delta[0]
     uint32_t da1 = da - (uint32_t)sizeof(MemT);                                     // &delta[-1]
@@ -228,70 +249,71 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
     MOC_KEEP(w0);
     MOC_KEEP(sell0);
     MOC_KEEP(n_tiles);
-    if (lane == 0) *reinterpret_cast<uint32_t*>(ws + p.word_bytes) = 0x00010001u;   // owned by empty node slots
 
     const int n = p.n;
-    const int n_warps = gridDim.x * wpb;
-    auto clear_deltas = [&]() {             // all of them, with the front pad: after a sequence that was not scanned
-        int4* d4 = reinterpret_cast<int4*>(delta_base);
-        for (int i = lane; i < (int)(p.delta_bytes >> 4); i += 32) d4[i] = make_int4(0, 0, 0, 0);
-        __syncwarp();
-    };
-    clear_deltas();
-    constexpr int kPerVec = 16 / (int)sizeof(MemT);  // delta entries per 16-byte vector
-    constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
-
     // Two ways to find the rows.  With p.offs (written by the offsets kernel) warps stride over the
-    // whole batch.  Without it (p.offs == nullptr) block c takes the contiguous range
-    // [c*B/grid, (c+1)*B/grid): it adds up the lengths in front of its range once, and every warp then
-    // walks the range with the lengths themselves -- no scratch, no second kernel.
+    // whole batch.  Without it (p.offs == nullptr) block c takes a contiguous range: it adds up the lengths in
+    // front of its range once, and every warp then walks the range with the lengths themselves -- no scratch,
+    // no second kernel.
     const bool self = p.offs == nullptr;
     int b, b_end, b_step;
     int64_t off = 0;
     int32_t T = 0;
-    // self mode: lanes 0..wpb-1 hold the lengths of sequences b .. b+wpb-1 (next: of the following wpb)
-    int32_t len_raw = 0;
+    // self mode: lanes 0..groups-1 hold the lengths of sequences b .. b+groups-1 (next: of the following ones)
+    int32_t len_raw = 0, len_c0 = 0;
+    uint64_t sum = 0;
     auto group_sum = [&](int32_t raw, int lanes) -> int64_t {   // sum of max(raw, 0) over lanes < `lanes`
         const uint32_t v = (lane < lanes && raw > 0) ? (uint32_t)raw : 0u;
-        const uint32_t lo = __reduce_add_sync(0xFFFFFFFFu, v & 0xFFFFu), hi = __reduce_add_sync(0xFFFFFFFFu, v >> 16);
+        const uint32_t lo = __reduce_add_sync(kFull, v & 0xFFFFu), hi = __reduce_add_sync(kFull, v >> 16);
         return (int64_t)lo + ((int64_t)hi << 16);
     };
     if (!self) {
-        b = blockIdx.x + gridDim.x * warp;      // a batch smaller than the grid's warps spreads over all blocks
+        b = blockIdx.x + gridDim.x * group;      // a batch smaller than the grid's warps spreads over all blocks
         b_end = p.B;
-        b_step = n_warps;
+        b_step = gridDim.x * groups;
         if (b < b_end) { off = __ldg(&p.offs[b]); T = __ldg(&p.lens[b]); }
     } else {
-        const int c0 = (int)((int64_t)blockIdx.x * p.B / gridDim.x);
-        b_end = (int)(((int64_t)blockIdx.x + 1) * p.B / gridDim.x);
-        b_step = wpb;
-        int64_t sum = 0;
-        b = c0 + warp;
-        // lengths of the first wpb sequences of the range (this warp starts at the warp-th of them), and of those from b on
-        const int32_t len_c0 = (c0 + lane < p.B) ? __ldg(p.lens + c0 + lane) : 0;
+        const int c0 = (int)blockIdx.x * p.per_block + min((int)blockIdx.x, p.spare);
+        b_end = c0 + p.per_block + ((int)blockIdx.x < p.spare ? 1 : 0);
+        b_step = groups;
+        b = c0 + group;
+        // lengths of the first sequences of the range (this warp starts at the group-th of them), and of those from b on
+        len_c0 = (c0 + lane < p.B) ? __ldg(p.lens + c0 + lane) : 0;
         len_raw = (b + lane < p.B) ? __ldg(p.lens + b + lane) : 0;
-        if ((reinterpret_cast<uintptr_t>(p.lens) & 15) == 0) {
-            const int4* l4 = reinterpret_cast<const int4*>(p.lens);
-            for (int i = threadIdx.x; i < (c0 >> 2); i += 8 * blockDim.x) {       // eight loads in flight
-                int4 q[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) q[k] = i + k * (int)blockDim.x < (c0 >> 2) ? __ldg(l4 + i + k * blockDim.x) : make_int4(0, 0, 0, 0);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) sum += (int64_t)max(q[k].x, 0) + max(q[k].y, 0) + max(q[k].z, 0) + max(q[k].w, 0);
-            }
-            for (int i = (c0 & ~3) + threadIdx.x; i < c0; i += blockDim.x) sum += max(__ldg(p.lens + i), 0);
-        } else {
-            for (int i = threadIdx.x; i < c0; i += blockDim.x) sum += max(__ldg(p.lens + i), 0);
-        }
-        sum = warp_sum64(sum);
-        if (lane == 0) s_part[warp] = sum;
-        __syncthreads();
-        for (int k = 0; k < wpb; ++k) off += s_part[k];
-        off += group_sum(len_c0, warp);
-        T = __shfl_sync(0xFFFFFFFFu, len_raw, 0);
+        sum = lengths_before(p.lens, c0, threadIdx.x, blockDim.x);
+    }
+    // words and deltas are zero when a sequence begins: the words are cleared behind stage 2, the deltas by the scan
+    auto clear = [&](uint32_t at, uint32_t bytes) {
+        for (uint32_t i = 16u * (uint32_t)tl; i < bytes; i += 16u * (uint32_t)tn)
+            asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(at + i), "r"(0) : "memory");
+    };
+    auto clear_deltas = [&]() { clear(da - kPairDeltaFront, p.delta_bytes); };   // all of them, with the front pad
+    clear(wa, p.word_bytes);
+    clear_deltas();
+    if (tl == 0) sts_u32(wa + p.word_bytes, 0x00010001u);   // owned by empty node slots
+    if (self) {
+        sum = warp_sum_u59(sum);
+        if (lane == 0) s_part[warp] = (int64_t)sum;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();                        // the graph is there
+    __syncthreads();                        // the graph is there, the state is zero, the sums of the warps stand
+    if (self) {
+        off = (int64_t)warp_sum_u59(lane < wpb ? (uint64_t)s_part[lane] : 0) + group_sum(len_c0, group);
+        T = __shfl_sync(kFull, len_raw, 0);
+    }
+    constexpr int kPerVec = 16 / (int)sizeof(MemT);  // delta entries per 16-byte vector
+    constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
+
+    // Vector i of a row: its steps 4 i - a .. + 3, where steps outside the row count as the spare id n.
+    auto fetch = [&](const int32_t* row, int32_t len, int t0) -> int4 {
+        if (t0 >= 0 && t0 + 4 <= len) return __ldg(reinterpret_cast<const int4*>(row + t0));
+        int4 v = make_int4(n, n, n, n);
+        if (t0 >= 0) v.x = __ldg(row + t0);
+        if (t0 + 1 >= 0 && t0 + 1 < len) v.y = __ldg(row + t0 + 1);
+        if (t0 + 2 >= 0 && t0 + 2 < len) v.z = __ldg(row + t0 + 2);
+        if (t0 + 3 >= 0 && t0 + 3 < len) v.w = __ldg(row + t0 + 3);
+        return v;
+    };
     // The first kPre 16-byte vectors per lane of the NEXT row are loaded into registers while the
     // current sequence is still being worked on, so that stage 1 does not wait for HBM.
     int4 pre[kPre > 0 ? kPre : 1];
@@ -305,7 +327,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
             if (b_next < b_end) { off_next = __ldg(&p.offs[b_next]); T_next = __ldg(&p.lens[b_next]); }
         } else {
             if (b_next < b_end) len_next = (b_next + lane < p.B) ? __ldg(p.lens + b_next + lane) : 0;
-            off_next = off + group_sum(len_raw, wpb);   // skip the wpb sequences b .. b+wpb-1
+            off_next = off + group_sum(len_raw, groups);   // skip the sequences b .. b+groups-1
         }
 
         const bool use_pre = have_pre;   // pre[] holds this row only if the previous iteration fetched it
@@ -313,71 +335,45 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
         if (T >= n && T <= p.max_T) {
-            // ---- clear the words (the deltas are zero: the scan clears behind itself)
             const int nvec_d = (T + 2 + kPerVec - 1) / kPerVec;        // vectors covering delta[0..T+1]
-            const int V = ((nvec_d + 31) >> 5) | 1;                      // vectors per lane, odd
-            {
-                const int4 z = make_int4(0, 0, 0, 0);
-                int4* w4 = reinterpret_cast<int4*>(word);
-                for (int i = lane; i < (int)(p.word_bytes >> 4); i += 32) w4[i] = z;
-            }
-            __syncwarp();
-            if (lane == 0) word[n + 1] = (uint32_t)T * 0x10001u;   // the made-up successor of sinks
+            const int V = kTeam ? ((nvec_d + tn - 1) / tn) | 1 : ((nvec_d + 31) >> 5) | 1;      // vectors per lane, odd
 
             // ---- stage 1: occurrence words
+            if (tl == 0) sts_u32(wa + 4u * (uint32_t)(n + 1), (uint32_t)T * 0x10001u);   // the made-up successor of sinks
             {
                 const int32_t* row = p.seqs + off;
                 const int a = (int)((reinterpret_cast<uintptr_t>(row) & 15) >> 2);
                 const int nvec = (T + a + 3) >> 2;
-                auto put = [&](int node, uint32_t t1) {
-                    // ids outside [0, n) go to the spare word n; the copy count exposes them
-                    const uint32_t addr = wa + 4u * min((uint32_t)node, (uint32_t)n);
-                    const uint32_t old = exch_shared(addr, t1 * 0x10001u);
-                    sts_u16_if_nonzero(old, addr + 2, old);
+                // ids outside [0, n) and steps outside the row go to the spare word n; the copy count exposes the former
+                auto put4 = [&](int4 v, int t0) {
+                    const uint32_t t1 = (uint32_t)(t0 + 1) * 0x10001u;
+                    const uint32_t a0 = wa + 4u * min((uint32_t)v.x, (uint32_t)n), a1 = wa + 4u * min((uint32_t)v.y, (uint32_t)n),
+                                   a2 = wa + 4u * min((uint32_t)v.z, (uint32_t)n), a3 = wa + 4u * min((uint32_t)v.w, (uint32_t)n);
+                    const uint32_t o0 = exch_shared(a0, t1), o1 = exch_shared(a1, t1 + 0x10001u), o2 = exch_shared(a2, t1 + 0x20002u),
+                                   o3 = exch_shared(a3, t1 + 0x30003u);
+                    sts_u16_if_nonzero(o0, a0 + 2, o0);
+                    sts_u16_if_nonzero(o1, a1 + 2, o1);
+                    sts_u16_if_nonzero(o2, a2 + 2, o2);
+                    sts_u16_if_nonzero(o3, a3 + 2, o3);
                 };
-                // vectors that lie completely inside the row (the first kPre per lane may already be here)
+                // (the first kPre vectors per lane may already be here)
 #pragma unroll
                 for (int j = 0; j < kPre; ++j) {
                     const int i = lane + 32 * j;
-                    const int t0 = 4 * i - a;
-                    if (i < nvec && t0 >= 0 && t0 + 4 <= T) {
+                    if (i < nvec) {
                         int4 v = pre[j];
-                        if (!use_pre) v = __ldg(reinterpret_cast<const int4*>(row + t0));
-                        put(v.x, (uint32_t)t0 + 1);
-                        put(v.y, (uint32_t)t0 + 2);
-                        put(v.z, (uint32_t)t0 + 3);
-                        put(v.w, (uint32_t)t0 + 4);
+                        if (!use_pre) v = fetch(row, T, 4 * i - a);
+                        put4(v, 4 * i - a);
                     }
                 }
-                for (int i = lane + 32 * kPre; i < nvec; i += 32) {
-                    const int t0 = 4 * i - a;
-                    if (t0 >= 0 && t0 + 4 <= T) {
-                        const int4 v = __ldg(reinterpret_cast<const int4*>(row + t0));
-                        put(v.x, (uint32_t)t0 + 1);
-                        put(v.y, (uint32_t)t0 + 2);
-                        put(v.z, (uint32_t)t0 + 3);
-                        put(v.w, (uint32_t)t0 + 4);
-                    }
-                }
-                // the ragged first and last vectors, element by element
-                if (lane < 2) {
-                    const int i = lane == 0 ? 0 : nvec - 1;
-                    const int t0 = 4 * i - a;
-                    if ((lane == 0 || nvec > 1) && !(t0 >= 0 && t0 + 4 <= T)) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int t = t0 + k;
-                            if (t >= 0 && t < T) put(__ldg(row + t), (uint32_t)t + 1);
-                        }
-                    }
-                }
+                for (int i = tl + 32 * kPre; i < nvec; i += tn) put4(fetch(row, T, 4 * i - a), 4 * i - a);
             }
-            __syncwarp();
+            team_sync<kTeam>(group + 1, tn);
 
             // request the next row now: the loads complete behind stages 2-4
             if (kPre > 0 && b_next < b_end) {
                 const int64_t off_n = off_next;
-                const int32_t T_n = self ? __shfl_sync(0xFFFFFFFFu, len_next, 0) : T_next;
+                const int32_t T_n = self ? __shfl_sync(kFull, len_next, 0) : T_next;
                 if (T_n >= n && T_n <= p.max_T) {
                     const int32_t* nrow = p.seqs + off_n;
                     const int an = (int)((reinterpret_cast<uintptr_t>(nrow) & 15) >> 2);
@@ -385,17 +381,16 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
 #pragma unroll
                     for (int j = 0; j < kPre; ++j) {
                         const int i = lane + 32 * j;
-                        const int t0 = 4 * i - an;
-                        if (i < nvn && t0 >= 0 && t0 + 4 <= T_n) pre[j] = __ldg(reinterpret_cast<const int4*>(nrow + t0));
+                        if (i < nvn) pre[j] = fetch(nrow, T_n, 4 * i - an);
                     }
                     have_pre = true;
                 }
             }
 
-            if (kPre == 0 && b_next < b_end) {
+            if (kPre == 0 && !kTeam && b_next < b_end) {
                 // short rows are read in place; ask for the next one to be brought into L2 meanwhile
                 const int64_t off_n = off_next;
-                const int32_t T_n = self ? __shfl_sync(0xFFFFFFFFu, len_next, 0) : T_next;
+                const int32_t T_n = self ? __shfl_sync(kFull, len_next, 0) : T_next;
                 if (T_n >= n && T_n <= p.max_T) {
                     const char* nrow = reinterpret_cast<const char*>(p.seqs + off_n);
                     const int bytes = 4 * T_n;
@@ -408,8 +403,8 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
             uint32_t vmin = 0xFFFFFFFFu, depw = 0, capw = 0;
             uint64_t acc = 0;
             {
-                uint32_t prec = rec0, pw = w0, ps = sell0;
-                for (int d = 0; d < n_tiles; ++d, prec += 64u * kRecB, pw += 512u) {
+                uint32_t prec = rec0 + 64u * kRecB * (uint32_t)wt, pw = w0 + 512u * (uint32_t)wt, ps = sell0;
+                for (int d = wt; d < n_tiles; d += tw, prec += 64u * kRecB * (uint32_t)tw, pw += 512u * (uint32_t)tw) {
                     uint32_t ab[2], naa[2], nbb[2], Ga[2], Gb[2];
                     Amount<MemT> m[2];
                     int rows = 0;
@@ -427,6 +422,7 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                             m[h].hi = r.w;
                         }
                         if (h == 0) rows = (int)(x >> 16);
+                        if (kTeam && h == 1) ps = sell0 + ((x >> 16) << 7);
                         const uint32_t own = lds_u32(wa + (x & 0xFFFFu));
                         vmin = min(vmin, own);
                         const uint32_t sw = swap_halves(own);
@@ -468,15 +464,29 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                     }
                 }
             }
-            vmin = __reduce_min_sync(0xFFFFFFFFu, vmin);
+            vmin = __reduce_min_sync(kFull, vmin);
             // the low words add up without a carry when all durations together fit 32 bits
-            const uint64_t acc_all = p.small_w ? (uint64_t)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)(acc >> 32)) << 32 | __reduce_add_sync(0xFFFFFFFFu, (uint32_t)acc)
-                                               : (uint64_t)warp_sum64((int64_t)acc);
-            const bool cap_ok = !__any_sync(0xFFFFFFFFu, (int32_t)capw < 0);
+            uint64_t acc_all = p.small_w ? (uint64_t)__reduce_add_sync(kFull, (uint32_t)(acc >> 32)) << 32 | __reduce_add_sync(kFull, (uint32_t)acc)
+                                         : (uint64_t)warp_sum64((int64_t)acc);
+            bool cap_ok = !__any_sync(kFull, (int32_t)capw < 0), dep = __any_sync(kFull, (depw & 0x80008000u) != 0);
+            if constexpr (kTeam) {
+                if (lane == 0) {
+                    s_acc[warp] = acc_all;
+                    s_flag[warp] = (vmin == 0 ? 1u : 0u) | (cap_ok ? 0u : 2u) | (dep ? 4u : 0u);
+                }
+                team_sync<kTeam>(group + 1, tn);
+                const bool in = lane < tw;
+                const uint32_t f = __reduce_or_sync(kFull, in ? s_flag[group * tw + lane] : 0u);
+                acc_all = (uint64_t)warp_sum64(in ? (int64_t)s_acc[group * tw + lane] : 0);
+                vmin = f & 1u ? 0u : 1u;
+                cap_ok = !(f & 2u);
+                dep = (f & 4u) != 0;
+            } else {
+                __syncwarp();
+            }
+            clear(wa, p.word_bytes);
             const bool well_formed = cap_ok && vmin != 0 && (int)((acc_all >> kPairCntShift) & 0x7FFFu) == T - n;
-            const bool dep = __any_sync(0xFFFFFFFFu, (depw & 0x80008000u) != 0);
             const int64_t dur_extra = (int64_t)(acc_all & kPairDurMask);
-            __syncwarp();
             if (!well_formed || dep) clear_deltas();
 
             if (!well_formed) {
@@ -488,57 +498,76 @@ __global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
                 // ---- stage 3 + 4: prefix sum and running maximum; lane owns V consecutive vectors
                 // One pass: the lane's running prefix and the largest prefix it sees; the largest
                 // usage inside the lane's chunk is then (sum of the chunks before it) + that maximum.
-                int4* d4 = reinterpret_cast<int4*>(delta_base + kPairDeltaFront) + lane * V;
-                const int4 z = make_int4(0, 0, 0, 0);
+                const int v0 = tl * V, v1 = kTeam ? min(v0 + V, nvec_d) : v0 + V;     // (a team's arrays end with the last vector)
+                uint32_t d4 = da + 16u * (uint32_t)v0;
                 MemT peak;
+                uint32_t lo = 0, hi = 0;
+                auto take = [&](uint32_t at) -> int4 {
+                    const uint4 q = lds_v4(at);
+                    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(at), "r"(0) : "memory");
+                    return make_int4((int)q.x, (int)q.y, (int)q.z, (int)q.w);
+                };
                 if constexpr (sizeof(MemT) == 4) {
-                    MemT run = 0, top;
-                    {
-                        const int4 q = d4[0];
-                        d4[0] = z;
-                        run = q.x; top = run;
-                        run += q.y; top = max(top, run);
-                        run += q.z; top = max(top, run);
-                        run += q.w; top = max(top, run);
-                    }
-                    for (int j = 1; j < V; ++j) {
-                        const int4 q = d4[j];
-                        d4[j] = z;
+                    MemT run = 0, top = INT32_MIN;
+                    for (int j = v0; j < v1; ++j, d4 += 16u) {
+                        const int4 q = take(d4);
                         run += q.x; top = max(top, run);
                         run += q.y; top = max(top, run);
                         run += q.z; top = max(top, run);
                         run += q.w; top = max(top, run);
                     }
-                    peak = warp_inclusive_sum(run, lane) - run + top;
+                    lo = warp_inclusive_sum((uint32_t)run, lane);
+                    peak = (MemT)(lo - (uint32_t)run) + top;
+                    if (kTeam && v0 >= v1) peak = INT32_MIN;
                 } else {
-                    uint32_t lo = 0, hi = 0;
                     int64_t top = INT64_MIN;
-                    for (int j = 0; j < V; ++j) {
-                        const int4 q = d4[j];
-                        d4[j] = z;
-                        lo += (uint32_t)q.x; hi += (uint32_t)q.y;
-                        const int64_t u = split_value(lo, hi, p.split);
-                        lo += (uint32_t)q.z; hi += (uint32_t)q.w;
-                        const int64_t w = split_value(lo, hi, p.split);
+                    uint32_t l = 0, h = 0;
+                    for (int j = v0; j < v1; ++j, d4 += 16u) {
+                        const int4 q = take(d4);
+                        l += (uint32_t)q.x; h += (uint32_t)q.y;
+                        const int64_t u = split_value(l, h, p.split);
+                        l += (uint32_t)q.z; h += (uint32_t)q.w;
+                        const int64_t w = split_value(l, h, p.split);
                         top = u > top ? u : top;
                         top = w > top ? w : top;
                     }
-                    peak = split_value(warp_inclusive_sum(lo, lane) - lo, warp_inclusive_sum(hi, lane) - hi, p.split) + top;
+                    lo = warp_inclusive_sum(l, lane);
+                    hi = warp_inclusive_sum(h, lane);
+                    peak = split_value(lo - l, hi - h, p.split) + top;
+                    if (kTeam && v0 >= v1) peak = INT64_MIN;
                 }
                 out_pk = (int64_t)warp_max_t(peak);
+                if constexpr (kTeam) {
+                    // the warp's largest usage counts from the usage in front of it
+                    if (lane == 31) { s_lo[warp] = lo; s_hi[warp] = hi; s_top[warp] = out_pk; }
+                }
                 out_du = p.base_dur + dur_extra;
-                out_st = out_pk <= p.M ? 1 : 0;
+                out_st = 1;
             }
-            __syncwarp();
+            team_sync<kTeam>(group + 1, tn);
+            if constexpr (kTeam) {
+                if (out_st == 1 && wt == 0) {
+                    const bool in = lane < tw;
+                    const uint32_t l = in ? s_lo[group * tw + lane] : 0u, h = in ? s_hi[group * tw + lane] : 0u;
+                    const int64_t top = in ? s_top[group * tw + lane] : 0;
+                    MemT front;
+                    if constexpr (sizeof(MemT) == 4) front = (MemT)(warp_inclusive_sum(l, lane) - l);
+                    else front = split_value(warp_inclusive_sum(l, lane) - l, warp_inclusive_sum(h, lane) - h, p.split);
+                    // usages are 0 or more: a warp without vectors counts as 0
+                    const bool has = in && top != (sizeof(MemT) == 4 ? (int64_t)INT32_MIN : INT64_MIN);
+                    out_pk = (int64_t)warp_max_t(has ? (MemT)(front + (MemT)top) : (MemT)0);
+                }
+            }
+            if (out_st == 1) out_st = out_pk <= p.M ? 1 : 0;
         }
-        if (lane == 0) {
+        if (tl == 0) {
             p.out_peak[b] = out_pk;
             p.out_dur[b] = out_du;
             p.out_status[b] = out_st;
         }
         if (self) {
             len_raw = len_next;
-            T_next = __shfl_sync(0xFFFFFFFFu, len_next, 0);
+            T_next = __shfl_sync(kFull, len_next, 0);
         }
         b = b_next;
         off = off_next;

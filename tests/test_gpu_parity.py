@@ -125,6 +125,29 @@ def test_block_kernel_with_and_without_its_own_copy_of_the_graph(B, n, C, bits, 
         assert (a.cpu().numpy() == b).all()
 
 
+@pytest.mark.parametrize("n,bits,nB", [(65, 0, 1), (65, 20, 1184), (65, 0, 1185), (128, 37, 592), (255, 0, 593), (256, 37, 444), (447, 0, 149), (600, 0, 296),
+                                       (600, 20, 297), (1399, 0, 148), (1400, 37, 148), (1400, 0, 149), (5000, 0, 3), (3, 0, 5)])
+def test_warps_that_share_a_sequence(B, n, bits, nB):
+    """Two to sixteen warps on a sequence, on both sides of the lines between them, with one and with two copies allowed and
+    with per-node caps; damaged sequences between good ones; packed rows and rows at given offsets."""
+    edges = W.layered_dag(n, 3 * n, max(4, n // 40), n) if n > 20 else np.array([[0, 1]], np.int32)
+    w, m = W.weights_uniform(n, 0, 30, n, 1), np.minimum(W.weights_lognormal(n, 3.0, 1.0, n, 2), 255) << bits
+    seqs, lens = W.schedules(n, edges, 2, 0.3, nB, n)
+    seqs, lens = W.mutate(seqs, lens, n, 2, seed=5, frac=1 / 4)
+    for C, caps in ((2, None), (1, None), (2, np.where(np.arange(n) % 7 == 0, 1, 2).astype(np.int32))):
+        O, G = OracleGraph(n, edges, w, m, C), B.Graph(n, edges, w, m, C)
+        if caps is not None:
+            O.set_caps(caps)
+            G.set_caps(caps)
+        M = O.eval(np.arange(n), 1 << 62)["peak"] * 90 // 100
+        want = assert_batch_equal(G, O, seqs, lens, M, f"n {n} C {C}")
+        out = tuple(torch.full((nB,), 77, dtype=d, device="cuda") for d in (torch.int64, torch.int64, torch.int32))
+        B.moc_eval_batch_noalloc(G.h, dev(seqs), dev(lens), M, *out)
+        torch.cuda.synchronize()
+        for a, b in zip(out, want):
+            assert (a.cpu().numpy() == b).all()
+
+
 # ------------------------------------------------------------------ the five configurations
 SMALL_B = [1024, 4096, 2048, 512, 64]
 

@@ -310,12 +310,12 @@ def test_which_kernel_makes_a_profile(fake, n, C, scale, star):
 
 @pytest.mark.parametrize("n,C,nB,kernel", [(65, 3, 444, "ILi3ELb1ELb0ELb1E"), (65, 3, 445, "ILi3ELb1ELb0ELb0E"), (700, 4, 444, "ILi4ELb1ELb0ELb1E"),
                                            (701, 4, 148, "ILi4ELb1ELb0ELb1E"), (701, 4, 149, "ILi4ELb1ELb0ELb0E"), (442, 2, 148, "ILi2ELb1ELb0ELb1E"),
-                                           (4000, 2, 148, "ILi2ELb1ELb0ELb1E"), (4001, 2, 148, "ILi2ELb1ELb0ELb0E")])
+                                           (442, 2, 149, None), (399, 2, 1, None), (600, 2, 1, None), (4000, 3, 148, "ILi3ELb1ELb0ELb1E"), (4001, 3, 148, "ILi3ELb1ELb0ELb0E")])
 def test_the_block_kernel_copies_the_graph_for_small_batches(fake, n, C, nB, kernel):
     G, x = Graph(fake, n, C), np.zeros(8, np.int64)
     fake.fake_reset(0)
     assert fake.moc_eval_batch(G.h, x.ctypes.data, x.ctypes.data, nB, 0, x.ctypes.data, x.ctypes.data, x.ctypes.data, None) == 0
-    assert len(launched(fake, "eval_quad_kernel" + kernel.replace("I", "Ii", 1))) == 1, log(fake)
+    assert len(launched(fake, "eval_quad_kernel" + kernel.replace("I", "Ii", 1) if kernel else "eval_pair_kernelIiLi0ELb1E")) == 1, log(fake)
     G.close()
 
 
