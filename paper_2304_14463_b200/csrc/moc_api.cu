@@ -127,23 +127,56 @@ QuadBytes quad_bytes(const moc_graph* g, bool wide, bool profile) {
     return z;
 }
 
-// Whether the block-per-sequence kernel takes a batch of B with the tiles in the block's shared memory.  It saves the L2's
-// latency three times per sequence and costs every block of an SM its own copy (0.5 us each, one after the other), so it
-// pays while an SM has one sequence, for small graphs up to three; and the copies have to fit beside all of them.  Measured, copied / through
-// L1 (C = 3, best thread count of each): n = 442 6.4 / 8.4 us at B = 148, 8.4 / 10.5 at 444, 12.5 / 12.5 at 888; n = 700 7.5 / 8.4 at 148, 10.5 /
-// 10.5 at 444, 14.6 / 10.5 at 592; n = 1000 8.4 / 9.2 (C = 4), 12.5 / 10.5 at 444 (C = 2); n = 3300 12.5 / 14.6 at 148, 18.7 / 16.5 at 296;
-// n = 5000 14.5 / 12.6 at 148 (C = 2).
-bool quad_chip_fits(const moc_graph* g, int32_t B, bool profile) {
+// How the block-per-sequence kernel's code takes a batch: `team` warps on a sequence, `groups` sequences in flight per
+// block, one block per SM, with the graph in shared memory.  team = 0: a block per sequence, the graph through L1.
+struct QuadShape {
+    int team = 0, groups = 0, grid = 0;
+};
+// Time in microseconds of a batch with u = n / 64 and s sequences per SM, in `rounds` rounds of what an SM holds at a time (fits to 354 batches
+// with every team size: n = 24 to 5000, C = 3, 4, B = 1 to 18944, 32- and 64-bit sums; mean error 5 %):
+//     a warp per sequence         4.3 + rounds (1.5 + (0.19 + 0.31 C) u) + s (0.07 + 0.009 C u)
+//     t warps per sequence        5.0 + rounds (1.0 + (0.15 + 0.28 C) u / t) + s (0.09 + 0.054 t + 0.012 C u)
+//     a block of 64 w threads     5.3 + rounds (1.3 + (0.40 + 0.15 C) u / w + 0.046 w) + s (0.10 + 0.040 w + 0.010 C u)
+// The smallest of them costs 1.2 % on the mean against always taking the fastest, 4 % or less in nine of ten.  Before / now (C = 3): n = 153,
+// B = 18944 68 -> 39 us, n = 24 45 -> 21, n = 442, B = 4736 33 -> 27, n = 1000, B = 1776 26.9 -> 24.8.
+double quad_block_cost(int64_t n, int32_t C, int64_t per_sm, int blocks, int w) {
+    const double u = (double)n / 64.0, rounds = (double)((per_sm + blocks - 1) / blocks);
+    return 5.3 + rounds * (1.27 + (0.40 + 0.15 * C) * u / w + 0.046 * w) + (double)per_sm * (0.10 + 0.040 * w + 0.010 * C * u);
+}
+QuadShape quad_shape(const moc_graph* g, int32_t B, bool profile) {
+    QuadShape best;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
-    if (!g->n_tiles || g->C > 4 || g->sum_w >= (int64_t)1 << moc::kPairCntShift) return false;
-    const int64_t per_sm = ((int64_t)B + g->sm_count - 1) / g->sm_count;
-    if (per_sm > (g->n <= 700 ? 3 : 1) || g->n > 4000) return false;
+    if (!g->n_tiles || g->C > 4 || g->sum_w >= (int64_t)1 << moc::kPairCntShift || (wide && !g->split_ok)) return best;
+    if (g->want_kind == MOC_KERNEL_BLOCK && g->want_a && !profile) return best;
     const QuadBytes z = quad_bytes(g, wide, profile);
-    return (size_t)per_sm * (z.state() + z.graph() + 2048) <= g->smem_optin;
+    if (z.graph() + z.state() + 2048 > g->smem_optin) return best;
+    const int64_t per_sm = ((int64_t)B + g->sm_count - 1) / g->sm_count, fit = (int64_t)((g->smem_optin - 2048 - z.graph()) / z.state());
+    const double u = (double)g->n / 64.0;
+    const int32_t C = g->C;
+    double least = 0;
+    auto offer = [&](double cost, int team, int64_t groups) {
+        if (least != 0 && cost >= least) return;
+        least = cost;
+        best.team = team;
+        best.groups = (int)groups;
+    };
+    for (int w = 1; w <= 16; w <<= 1) {         // registers: 64 a thread
+        const int64_t blocks = std::min<int64_t>((int64_t)((g->smem_optin + 1024) / (z.state() + 2048)), 16 / w);
+        if (blocks > 0) offer(quad_block_cost(g->n, C, per_sm, (int)blocks, w), 0, 0);
+    }
+    for (int team = 1; team <= 32; team <<= 1) {
+        if (team == 1 && C < 3) continue;
+        const int64_t most = std::min<int64_t>(fit, std::min(32 / team, team > 1 ? 16 : 32)), rounds = (per_sm + most - 1) / most;
+        offer(team == 1 ? 4.3 + (double)rounds * (1.5 + (0.19 + 0.31 * C) * u) + (double)per_sm * (0.07 + 0.009 * C * u)
+                        : 5.0 + (double)rounds * (1.0 + (0.15 + 0.28 * C) * u / team) + (double)per_sm * (0.09 + 0.054 * team + 0.012 * C * u),
+              team, (per_sm + rounds - 1) / rounds);
+    }
+    best.grid = std::min(g->sm_count, B);
+    return best;
 }
 
 // Plan of the block-per-sequence path with packed words (C <= 4).  Returns nullptr on success.
-const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, bool chip, Plan* out) {
+const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, int mode, Plan* out) {
     Plan pl = *out;
     const int64_t n = g->n, C = g->C, t_max = C * n;
     if (C > 4) return "C > 4";
@@ -151,13 +184,13 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, bool ch
     if (t_max > 32766) return "sequences of more than 32766 steps";
     if (pl.wide && !g->split_ok) return "sum(m) too large for two-part sums";
     const QuadBytes z = quad_bytes(g, pl.wide, profile);
-    const size_t sm = z.state() + (chip ? z.graph() : 0);
+    const size_t sm = z.state() + (mode ? z.graph() : 0);
     if (sm > smem_cap) return "the state of a sequence exceeds shared memory";
-    QuadFn fn = quad_fn(pl.wide, (int)C, g->d_rec32 != nullptr, chip, profile);
+    QuadFn fn = mode == moc::kQuadWarps ? quad_warp_fn(pl.wide, (int)C) : quad_fn(pl.wide, (int)C, g->d_rec32 != nullptr, mode == moc::kQuadTeams, profile);
     if (raise_smem_limit((const void*)fn, g->smem_optin) != cudaSuccess) { cudaGetLastError(); return "cudaFuncSetAttribute failed"; }
     const int forced = !profile && g->want_kind == MOC_KERNEL_BLOCK ? g->want_a : 0;
-    bool any = false;
-    for (int k = 0; k < 5; ++k) {
+    bool any = mode != moc::kQuadBlock;
+    for (int k = 0; k < 5 && mode == moc::kQuadBlock; ++k) {
         const int thr = forced ? forced : 64 << k;
         int nb = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, thr, sm) != cudaSuccess) { cudaGetLastError(); nb = 0; }
@@ -166,7 +199,7 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, bool ch
     }
     if (!any) return "kernel does not fit on an SM";
     pl.quad = true;
-    pl.quad_chip = chip;
+    pl.quad_mode = mode;
     pl.quad_fn = fn;
     pl.quad_forced = forced;
     pl.gpc = 1;
@@ -185,29 +218,24 @@ const char* plan_quad(const moc_graph* g, size_t smem_cap, bool profile, bool ch
     return nullptr;
 }
 
-// Shape of the block-per-sequence kernel for a batch: threads per sequence (64 << k) and blocks per SM.  With the blocks
+// Threads per sequence (64 << k) and blocks per SM of the block-per-sequence kernel proper.  With the blocks
 // per SM that the state and the registers allow, a batch takes ceil(sequences per SM / blocks) rounds; as few
-// blocks as that number of rounds needs keeps them even.  Time in microseconds, with u = n / 64 and w = threads / 64, from
-// a fit to 4035 timed shapes (n = 40 to 5000, C = 2, 3, 4, 32- and 64-bit sums, B = 1 to 8192, every thread count):
-//     through L1:   rounds (1.27 + (0.40 + 0.15 C) u / w + 0.046 w) + sequences per SM (0.10 + 0.040 w + 0.010 C u)
-//     copied:       rounds (1.36 + (0.10 + 0.14 C) u / w + 0.018 w) + sequences per SM (0.055 w + 0.015 C u)
-// The choice costs 0.5 % and 0.7 % on the mean against the best of the five thread counts, 1.6 % or less in nine of ten,
-// and 38 % at worst (n = 1500, C = 4, B = 148: 14.5 against 10.6 us through L1).
-void quad_shape(const Plan& pl, int64_t n, int32_t C, int32_t B, int* threads, int* blocks) {
+// blocks as that number of rounds needs keeps them even.  The line for the time (quad_block_cost) is a fit to 2175 timed shapes (n = 40 to 5000,
+// C = 2, 3, 4, 32- and 64-bit sums, B = 1 to 8192, every thread count); the choice costs 0.5 % on the mean against the best of the five
+// thread counts, 0.3 % or less in nine of ten, and 38 % at worst (n = 1500, C = 4, B = 148: 14.5 against 10.6 us).
+void quad_threads(const Plan& pl, int64_t n, int32_t C, int32_t B, int* threads, int* blocks) {
     const int64_t per_sm = ((int64_t)B + pl.sm_count - 1) / pl.sm_count;
-    const double u = (double)n / 64.0;
     double best = 0;
     *threads = 0;
     for (int k = 0; k < 5; ++k) {
-        const int nb = pl.quad_nb[k], w = 1 << k;
+        const int nb = pl.quad_nb[k];
         if (nb < 1) continue;
-        const int64_t rounds = (per_sm + nb - 1) / nb, even = (per_sm + rounds - 1) / rounds;
-        const double cost = pl.quad_chip ? (double)rounds * (1.36 + (0.10 + 0.14 * C) * u / w + 0.018 * w) + (double)per_sm * (0.055 * w + 0.015 * C * u)
-                                         : (double)rounds * (1.27 + (0.40 + 0.15 * C) * u / w + 0.046 * w) + (double)per_sm * (0.10 + 0.040 * w + 0.010 * C * u);
+        const int64_t rounds = (per_sm + nb - 1) / nb;
+        const double cost = quad_block_cost(n, C, per_sm, nb, 1 << k);
         if (*threads == 0 || cost < best) {
             best = cost;
             *threads = pl.quad_forced ? pl.quad_forced : 64 << k;
-            *blocks = (int)even;
+            *blocks = (int)((per_sm + rounds - 1) / rounds);
         }
     }
 }
@@ -284,7 +312,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     const size_t smem_cap = g->smem_optin > 1024 ? g->smem_optin - 1024 : 0;  // 1 KB per block is reserved
     const int kind = profile ? MOC_KERNEL_GROUP : g->want_kind;
     const bool shape_given = g->want_G != 0 || g->want_gpc != 0;       // moc_graph_set_launch
-    if (profile && !plan_quad(g, smem_cap, true, quad_chip_fits(g, 1, true), &pl)) {
+    if (profile && !plan_quad(g, smem_cap, true, quad_shape(g, 1, true).team ? moc::kQuadTeams : moc::kQuadBlock, &pl)) {
         *out = pl;
         return MOC_OK;
     }
@@ -301,7 +329,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         if (kind == MOC_KERNEL_LANE) return fail(MOC_ERR_ARG, "the sequence-per-lane kernel cannot serve this graph: %s", why);
     }
     if (kind == MOC_KERNEL_BLOCK || (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C >= 3)) {
-        const char* why = plan_quad(g, smem_cap, profile, false, &pl);
+        const char* why = plan_quad(g, smem_cap, profile, moc::kQuadBlock, &pl);
         if (!why) {
             *out = pl;
             return MOC_OK;
@@ -346,7 +374,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
     // Sequences too long for ten warps of the warp-per-sequence kernel on an SM: warp / block with 16 warps 18.6 / 24.7 us (n = 1000, 32-bit
     // sums, B = 2368), with 14 37.0 / 39.1 (700, 64 bits, 4736), with 11 45.1 / 51.2 (1432, 32 bits, 3919), with 9 43.8 / 42.4 (1000, 64 bits,
     // 3552), with 6 61.8 / 30.9 (1400, 64 bits, 1776)
-    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, profile, false, &pl)) {
+    if (kind == MOC_KERNEL_AUTO && !shape_given && !profile && C <= 2 && !plan_quad(g, smem_cap, profile, moc::kQuadBlock, &pl)) {
         *out = pl;
         return MOC_OK;
     }
@@ -829,7 +857,7 @@ bool live_serves(const moc_graph* g, int32_t B) {
     if (!g->d_live32 || g->C > moc::kLivePlanes || g->want_kind != MOC_KERNEL_AUTO || g->want_G || g->want_gpc) return false;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
     const int32_t n = g->n;
-    if (g->C > 2) return B >= 900 + 62 * n;
+    if (g->C > 2) return B >= 900 + 76 * n;
     if (wide) return B >= (n <= 64 ? 300 + 160 * n : 120 * n);
     return B >= (n <= 64 ? 1500 + 170 * n : 185 * n - 800);
 }
@@ -913,9 +941,16 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         block = 32 * best_w;
         smem = pl.pair_graph_b + (size_t)best_w * pl.pair_warp_b;
     }
-    if (pl.quad) {
+    QuadShape teams;
+    if (pl.quad && pl.quad_mode != moc::kQuadBlock) {
+        teams = quad_shape(g, B, false);
+        grid = teams.grid;
+        block = 32 * teams.team * teams.groups;
+        const QuadBytes z = quad_bytes(g, pl.wide, false);
+        smem = z.graph() + (size_t)teams.groups * z.state();
+    } else if (pl.quad) {
         int nb = 1;
-        quad_shape(pl, g->n, g->C, B, &block, &nb);
+        quad_threads(pl, g->n, g->C, B, &block, &nb);
         grid = (int)std::min<int64_t>((int64_t)pl.sm_count * nb, B);
     }
     if (offs && fill_offs) {
@@ -933,6 +968,7 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         q.B = B;
         q.per_block = B / grid;
         q.spare = B % grid;
+        q.team = teams.team;
         q.M = M;
         q.seqs = seqs;
         q.lens = lens;
@@ -1030,22 +1066,22 @@ const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
     }
     const bool block = block_serves(g, B), wide = g->sum_m > (int64_t)INT32_MAX / g->C;
     const size_t cap = g->smem_optin > 1024 ? g->smem_optin - 1024 : 0;
-    auto quad = [&](Plan& kept, bool chip) -> const Plan* {
+    auto quad = [&](Plan& kept, int mode) -> const Plan* {
         if (!kept.valid) {
             Plan pl;
             pl.wide = wide;
-            plan_quad(g, cap, false, chip, &pl);
+            plan_quad(g, cap, false, mode, &pl);
             pl.valid = true;
             kept = pl;
         }
         return kept.quad ? &kept : nullptr;
     };
-    // small batches of the block-per-sequence kernel: with the graph in its shared memory
     const bool any_block = block || g->want_kind == MOC_KERNEL_BLOCK || (g->want_kind == MOC_KERNEL_AUTO && !g->want_G && !g->want_gpc && g->C >= 3);
-    if (any_block && quad_chip_fits(g, B, false))
-        if (const Plan* pl = quad(g->plan_chip, true)) return pl;
+    if (any_block)
+        if (const int team = quad_shape(g, B, false).team)
+            if (const Plan* pl = team > 1 || g->C < 3 ? quad(g->plan_chip, moc::kQuadTeams) : quad(g->plan_warps, moc::kQuadWarps)) return pl;
     if (block)
-        if (const Plan* pl = quad(g->plan_block, false)) return pl;
+        if (const Plan* pl = quad(g->plan_block, moc::kQuadBlock)) return pl;
     if (team_shape(g, B).team > 1) {
         Plan& kept = g->plan_team;
         if (!kept.valid) {
@@ -1067,7 +1103,7 @@ const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
     return *rc == MOC_OK ? &g->plan_eval : nullptr;
 }
 
-void forget_plans(moc_graph* g) { g->plan_eval = g->plan_team = g->plan_block = g->plan_chip = g->plan_live = Plan(); }
+void forget_plans(moc_graph* g) { g->plan_eval = g->plan_team = g->plan_block = g->plan_chip = g->plan_warps = g->plan_live = Plan(); }
 
 int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
                 int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {
@@ -1704,6 +1740,7 @@ int moc_mem_profile(const moc_graph* g, const int32_t* seq, int32_t len, int64_t
         // threads from measurements at n = 20, 100, 442, 1000, 2000 and 5000 (us per call with 128 / 512 / 1024 threads:
         // 6.1 / 6.2 / 10.6, 6.1 / 6.9 / 8.6, 8.2 / 7.4 / 8.2, 12.3 / 8.3 / 8.2, 17.0 / 10.3 / 10.3, 32.8 / 18.0 / 16.4)
         const int thr = g->n < 200 ? 128 : (g->n < 1500 ? 512 : 1024);
+        q.team = thr / 32;
         pl.quad_fn<<<1, thr, pl.smem, st>>>(q);
         ++g_launches;
         MOC_CUDA(cudaGetLastError());

@@ -31,7 +31,8 @@ KernelFn shared_fn(bool wide, int G, int CP, bool profile);
 KernelFn global_fn(int CP, bool profile);
 PairFn pair_fn(bool wide, int pre);      // pre < 0: several warps per sequence
 LaneFn lane_fn(bool wide, int lg, int kp);
-QuadFn quad_fn(bool wide, int C, bool tiles, bool chip, bool profile);
+QuadFn quad_fn(bool wide, int C, bool tiles, bool chip, bool profile);      // chip: the graph in shared memory, teams of warps
+QuadFn quad_warp_fn(bool wide, int C);      // a warp per sequence
 LiveFn live_fn(bool wide, int words, int C);
 const void* check_plain_fn(bool wide);
 IntervalFn check_general_fn(int cp, bool wide, int kept);      // kept: bytes per event of the solution kept on chip, 0: not kept
@@ -60,7 +61,7 @@ struct Plan {
     // block-per-sequence path with packed words for C <= 4
     bool quad = false;
     QuadFn quad_fn = nullptr;
-    bool quad_chip = false;        // the block keeps a copy of the graph's tiles
+    int quad_mode = 0;             // moc::kQuadBlock, kQuadTeams, kQuadWarps
     uint32_t quad_word_b = 0, quad_cnt_b = 0, quad_delta_b = 0, quad_row_b = 0;
     int quad_nb[5] = {0};          // blocks per SM with 64 << k threads
     int quad_forced = 0;           // threads per sequence the caller asked for
@@ -163,7 +164,7 @@ struct moc_graph {
     // grow-only scratch; mutable because evaluation takes a const handle
     mutable moc_host::Plan plan_eval, plan_profile;
     mutable moc_host::Plan plan_block;    // block-per-sequence kernel beside the warp-per-sequence one in plan_eval
-    mutable moc_host::Plan plan_chip;     // ... and the same with the graph in shared memory, for small batches
+    mutable moc_host::Plan plan_chip, plan_warps;     // ... and the same with the graph in shared memory, teams of warps and single warps
     mutable moc_host::Plan plan_team;     // warp-per-sequence kernel with several warps on each
     mutable moc_host::Plan plan_live;     // backward walk beside either
     mutable int64_t* d_offs = nullptr;

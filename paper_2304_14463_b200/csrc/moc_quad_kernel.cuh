@@ -32,16 +32,18 @@
 //   4.  reductions        peak (Section 2), status against the budget.
 //
 // Stage 2 walks the successor tiles of the warp-per-sequence kernel (two node slots per lane, uniform trip counts, packed
-// word offsets) where the graph has them, else a record per node with bounds tests.  Where a batch leaves room for it
-// (kChip) the block copies records, durations and tiles into its shared memory behind the search for the rows: a
-// batch of a few sequences per SM is a chain of latencies, and every read of the graph from L2 is one of them.  Rows are found from the lengths (each
+// word offsets) where the graph has them, else a record per node with bounds tests.  Rows are found from the lengths (each
 // block sums those in front of its range), or through `offs`.
-// The kernel is bound by instruction issue and by the barriers between its stages (four per sequence: behind 1a, 1b, 2
-// and the prefix sum; the words are cleared for the next sequence behind stage 2); the threads per sequence
-// follow the batch (quad_shape).  Cold latencies that were taken out of a small batch: a 64-bit division for the range of a
+//
+// Who shares a sequence (quad_shape, from the size of the batch): a warp (kQuadWarps: large batches of graphs up to some 600 nodes), a
+// team of warps (kQuadTeams), both with the graph copied into the block's shared memory once and several sequences in flight
+// beside it, or the block (kQuadBlock: sequences whose state leaves no room for the graph, and large graphs).  Bound: instruction issue and
+// the barriers between the stages (four per sequence: behind 1a, 1b, 2 and the prefix sum; the words are cleared for the next
+// sequence behind stage 2); a small batch is a chain of latencies, of which a 64-bit division for the range of a
 // block, sums of the lengths and of the chunks by shuffles and by loops over the warps (now warp reductions), the
-// graph through L2, three barriers.  n = 442, B = 148: C = 2 8.7 -> 6.2 us, C = 3 8.7 -> 6.2, C = 4 10.2 -> 8.2; n = 1000, C = 2, one sequence
-// 10.2 -> 6.1; n = 2192, C = 2 (words of 32 bits), B = 1184 32.5 -> 24.9; n = 5000, C = 3, B = 1024 75.9 -> 71.4; profile of n = 1000 8.2 -> 6.2.
+// graph through L2 and three barriers were taken out.  n = 442, B = 148, C = 3 8.7 -> 6.2 us; n = 153, C = 3, B = 18944 68 -> 39 (a warp
+// per sequence; a block of 64 threads spent most of its instructions on barriers and sums); n = 24 45 -> 21; n = 442, C = 3, B = 4736 33 -> 27 (teams of two);
+// n = 2192, C = 2 (words of 32 bits), B = 1184 32.5 -> 24.9; n = 1000, C = 3, B = 4096 53.3 -> 52.4; n = 5000, B = 1024 81 -> 73; profile of n = 1000 8.2 -> 6.2.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -58,11 +60,12 @@ struct QuadParams {
     int32_t per_block, spare;  // rows found by the kernel: block c takes per_block sequences, one more when c < spare
     int64_t M;
     int32_t n_tiles, split, small_w;    // as in PairParams
+    int32_t team;              // kQuadTeams: warps per sequence (a divisor of the block's warps; at most 16 teams)
     const void* rec;
     const uint32_t* sell;
     const int32_t* tile_row;   // first row of every tile in `sell`
     const uint64_t* wslot;     // durations by slot, as in PairParams
-    uint32_t rec_bytes, w_bytes, sell_bytes, row_bytes;   // kChip: sizes of the copies of rec, wslot, sell and tile_row
+    uint32_t rec_bytes, w_bytes, sell_bytes, row_bytes;   // the block's copies of rec, wslot, sell and tile_row
     const uint4* order;        // without tiles: n records of 32 bytes in order of falling out-degree (below)
     const uint16_t* succ;      // ... and the successors beyond the eighth of the nodes that have more
     const void* m;             // n output sizes, int32 or int64
@@ -211,9 +214,14 @@ __device__ __forceinline__ uint32_t lds_u16(uint32_t addr) {
 
 // kAcc: number of copies the node pass keeps apart (2, 3 or 4; C <= kAcc).
 // kProfile: one sequence, whose usage per step and free steps are written out (moc_mem_profile).
-// kChip: the block keeps a copy of the graph's tiles in shared memory.
-template <typename MemT, int kAcc, bool kTiles, bool kProfile, bool kChip>
-__global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
+// kMode: kQuadBlock  one sequence per block, the graph through L1
+//        kQuadTeams  the block keeps a copy of the graph's tiles in shared memory; p.team warps share a sequence
+//        kQuadWarps  the same with a warp per sequence
+constexpr int kQuadBlock = 0, kQuadTeams = 1, kQuadWarps = 2;
+
+template <typename MemT, int kAcc, bool kTiles, bool kProfile, int kMode>
+__device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
+    constexpr bool kChip = kMode != kQuadBlock;
     static_assert(kTiles || !kChip, "only tiles are copied");
     extern __shared__ __align__(16) char smem[];
     __shared__ int64_t s_dur[32], s_top[32];
@@ -221,21 +229,47 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
     constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
     constexpr int kWord = kAcc == 2 ? 2 : 3;                // log2 of the bytes of a node's word
     constexpr uint32_t kFull = 0xFFFFFFFFu;
-    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, n_warps = nthr >> 5;
-    const int warp = __shfl_sync(kFull, tid >> 5, 0);
+    const int lane = threadIdx.x & 31, block_warps = blockDim.x >> 5;
+    const int block_warp = __shfl_sync(kFull, (int)threadIdx.x >> 5, 0);
+    // sequences in flight per block, this warp's, and its place among the warps of that one
+    const int n_warps = kMode == kQuadBlock ? block_warps : (kMode == kQuadTeams ? p.team : 1);
+    const int group = kMode == kQuadBlock ? 0 : (kMode == kQuadTeams ? block_warp / n_warps : block_warp);
+    const int groups = kMode == kQuadBlock ? 1 : (kMode == kQuadTeams ? block_warps / n_warps : block_warps);
+    const int warp = kMode == kQuadWarps ? 0 : block_warp - group * n_warps, first_warp = group * n_warps;
+    const int tid = 32 * warp + lane, nthr = 32 * n_warps;
+    auto sync = [&]() {
+        if constexpr (kMode == kQuadBlock) __syncthreads();
+        else if constexpr (kMode == kQuadTeams) asm volatile("bar.sync %0, %1;" ::"r"(group), "r"(nthr) : "memory");
+        else __syncwarp();
+    };
+    auto sync_or = [&](uint32_t x) -> bool {          // the same, and whether any thread of the sequence had x != 0
+        if constexpr (kMode == kQuadBlock) return __syncthreads_or((int)x) != 0;
+        else if constexpr (kMode == kQuadTeams) {
+            uint32_t any;
+            asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.u32 a, %1, 0;\n\tbar.red.or.pred b, %2, %3, a;\n\tselp.u32 %0, 1, 0, b;\n\t}"
+                         : "=r"(any) : "r"(x), "r"(group), "r"(nthr) : "memory");
+            return any != 0;
+        } else {
+            const bool any = __any_sync(kFull, x != 0);
+            __syncwarp();
+            return any;
+        }
+    };
     int n = p.n;
     MOC_KEEP(n);
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
-    uint32_t wa = sbase, ca = sbase + p.word_bytes, da = ca + p.cnt_bytes;   // words | counters | delta[0..] | graph
+    // graph (kChip) | per sequence in flight: words | counters | delta[0..]
+    const uint32_t recs = sbase, wsl = recs + p.rec_bytes, sells = wsl + p.w_bytes, rows = sells + p.sell_bytes;
+    uint32_t wa = sbase + (kChip ? p.rec_bytes + p.w_bytes + p.sell_bytes + p.row_bytes : 0u) + (uint32_t)group * (p.word_bytes + p.cnt_bytes + p.delta_bytes);
+    uint32_t ca = wa + p.word_bytes, da = ca + p.cnt_bytes;
     MOC_KEEP(wa);
     MOC_KEEP(ca);
     MOC_KEEP(da);
     const uint32_t dm1 = da - (uint32_t)sizeof(MemT);
-    const uint32_t recs = da + p.delta_bytes, wsl = recs + p.rec_bytes, sells = wsl + p.w_bytes, rows = sells + p.sell_bytes;   // kChip
     if constexpr (kChip) {
         // asynchronous copies: complete behind the search for the rows and, for one sequence, the arrival of its row
         auto copy = [&](uint32_t to, const void* from, uint32_t bytes) {
-            for (uint32_t i = 16u * (uint32_t)tid; i < bytes; i += 16u * (uint32_t)nthr)
+            for (uint32_t i = 16u * threadIdx.x; i < bytes; i += 16u * blockDim.x)
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i), "l"(reinterpret_cast<const char*>(from) + i) : "memory");
         };
         copy(recs, p.rec, p.rec_bytes);
@@ -256,37 +290,63 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
     };
     // words and counters are zero when a sequence begins (stage 1b writes every delta that the prefix sum reads)
     auto clear = [&]() {
-        const int4 z = make_int4(0, 0, 0, 0);
-        int4* s4 = reinterpret_cast<int4*>(smem);
-        const int nz = (int)((p.word_bytes + p.cnt_bytes) >> 4);
-        for (int i = tid; i < nz; i += nthr) s4[i] = z;
+        const uint32_t nz = p.word_bytes + p.cnt_bytes;
+        for (uint32_t i = 16u * (uint32_t)tid; i < nz; i += 16u * (uint32_t)nthr)
+            asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(wa + i), "r"(0) : "memory");
     };
 
-    // ---- rows: block c takes a contiguous range of the sequences, or every grid-th one with the offsets given
+    // ---- rows: a block takes a contiguous range of the sequences, its teams in turn, or every grid-th one with the offsets given
     const bool self = !kProfile && p.offs == nullptr;
-    int b = (int)blockIdx.x, b_end = p.B, b_step = gridDim.x;
-    if (self) {
-        b = (int)blockIdx.x * p.per_block + min((int)blockIdx.x, p.spare);
-        b_end = b + p.per_block + ((int)blockIdx.x < p.spare ? 1 : 0);
-        b_step = 1;
-    }
+    int b = (int)blockIdx.x + (int)gridDim.x * group, b_end = p.B, b_step = (int)gridDim.x * groups;
     int64_t off = 0;
-    int32_t T_next = kProfile ? p.single_len : (b < p.B ? __ldg(p.lens + b) : 0);      // one sequence ahead
+    // the lengths of b, b + 1 .. by lane (rows found by the kernel: what lies between this sequence and the team's next)
+    int32_t T_next = 0, len_raw = 0, len_c0 = 0;
+    auto lanes_sum = [&](int32_t raw, int lanes) -> int64_t {   // sum of max(raw, 0) over lanes < `lanes`
+        const uint32_t v = (lane < lanes && raw > 0) ? (uint32_t)raw : 0u;
+        const uint32_t lo = __reduce_add_sync(kFull, v & 0xFFFFu), hi = __reduce_add_sync(kFull, v >> 16);
+        return (int64_t)lo + ((int64_t)hi << 16);
+    };
     if (self) {
-        const uint64_t sum = lengths_before(p.lens, b, tid, nthr);
+        const int c0 = (int)blockIdx.x * p.per_block + min((int)blockIdx.x, p.spare);
+        b = c0 + group;
+        b_end = c0 + p.per_block + ((int)blockIdx.x < p.spare ? 1 : 0);
+        b_step = groups;
+        if constexpr (kMode != kQuadBlock) {
+            len_c0 = c0 + lane < p.B ? __ldg(p.lens + c0 + lane) : 0;
+            len_raw = b + lane < p.B ? __ldg(p.lens + b + lane) : 0;
+        } else {
+            T_next = b < p.B ? __ldg(p.lens + b) : 0;
+        }
+        const uint64_t sum = lengths_before(p.lens, c0, threadIdx.x, blockDim.x);
         clear();
         const uint64_t part = warp_sum_u59(sum);
-        if (lane == 0) s_dur[warp] = (int64_t)part;
+        if (lane == 0) s_dur[block_warp] = (int64_t)part;
         __syncthreads();
-        off = (int64_t)warp_sum_u59(lane < n_warps ? (uint64_t)s_dur[lane] : 0);
+        off = (int64_t)warp_sum_u59(lane < block_warps ? (uint64_t)s_dur[lane] : 0);
+        if constexpr (kMode != kQuadBlock) {
+            off += lanes_sum(len_c0, group);
+            T_next = __shfl_sync(kFull, len_raw, 0);
+        }
     } else {
+        T_next = kProfile ? p.single_len : (b < p.B ? __ldg(p.lens + b) : 0);      // one sequence ahead
         clear();
+        if (!kChip || kProfile) sync();
+    }
+    if constexpr (kChip && !kProfile) {          // (a profile waits for the graph behind the arrival of its row)
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
     }
-    for (; b < b_end; b += b_step) {
+    while (b < b_end) {
         const int32_t T = T_next;
-        if (!kProfile && b + b_step < b_end) T_next = __ldg(p.lens + b + b_step);
-        if (!self && !kProfile) off = __ldg(p.offs + b);
+        const int b_next = b + b_step;
+        int64_t off_next = 0;
+        if (kMode != kQuadBlock && self) {
+            off_next = off + lanes_sum(len_raw, groups);
+            if (b_next < b_end) len_raw = b_next + lane < p.B ? __ldg(p.lens + b_next + lane) : 0;
+        } else if (!kProfile) {
+            if (!self) off = __ldg(p.offs + b);
+            if (b_next < b_end) T_next = __ldg(p.lens + b_next);
+        }
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
         if (T >= n && T <= p.max_T) {      // uniform over the block
@@ -331,8 +391,8 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                     }
                 }
             }
-            if constexpr (kChip) asm volatile("cp.async.wait_all;" ::: "memory");
-            __syncthreads();
+            if constexpr (kChip && kProfile) asm volatile("cp.async.wait_all;" ::: "memory");
+            sync();
             // records and first successor row of a tile are requested while the tile before it (or stage 1b) is worked on
             uint4 r_next[2];
             const uint32_t* ps_next = nullptr;
@@ -404,8 +464,9 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                     quad_settle<MemT, kAcc, kShift>(wa + ((uint32_t)v << kWord), c, dm1, mv);
                 }
             }
-            const bool malformed = __syncthreads_or((int)flags) != 0;
+            const bool malformed = sync_or(flags);
             bool dep = false;
+            int64_t dw = 0;
             if (!malformed) {
                 // ---- stage 2 and the scatter of stage 3
                 uint32_t depw = 0;
@@ -472,15 +533,16 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                         if (i < n) depw |= u.template close<MemT, kShift, kProfile>(da, amount((int)node), p.out_free, p.out_free != nullptr);
                     }
                 }
-                dep = __syncthreads_or((int)(depw & 0x8000u)) != 0;
+                dep = sync_or(depw & 0x8000u);
                 // per-warp sums of the durations, read behind the next barrier
-                const int64_t dw = p.small_w ? (int64_t)__reduce_add_sync(kFull, (uint32_t)dur) : warp_sum64(dur);
-                if (lane == 0) s_dur[warp] = dw;
+                dw = p.small_w ? (int64_t)__reduce_add_sync(kFull, (uint32_t)dur) : warp_sum64(dur);
+                if (lane == 0) s_dur[first_warp + warp] = dw;
             }
-            if (b + b_step < b_end) clear();       // for the next sequence: nothing reads the words any more
+            if (b_next < b_end) clear();       // for the next sequence: nothing reads the words any more
             const int chunk = ((T + nthr - 1) / nthr) | 1;
             const int tb = min(tid * chunk, T), te = min(tb + chunk, T);
             uint32_t lo_in = 0, hi_in = 0;          // deltas of the warp's threads in front of this one
+            MemT w_top = 0;
             if (!malformed && !dep) {
                 // ---- stages 3 and 4: prefix sum, each thread a chunk of consecutive steps (odd length: no bank conflicts);
                 // a warp's largest usage counts from the usage in front of the warp
@@ -502,8 +564,8 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 lo_in = warp_inclusive_sum(lo, lane);
                 if constexpr (sizeof(MemT) == 8) hi_in = warp_inclusive_sum(hi, lane);
                 if (lane == 31) {
-                    s_lo[warp] = lo_in;
-                    s_hi[warp] = hi_in;
+                    s_lo[first_warp + warp] = lo_in;
+                    s_hi[first_warp + warp] = hi_in;
                 }
                 lo_in -= lo;
                 hi_in -= hi;
@@ -511,24 +573,33 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
                 if constexpr (sizeof(MemT) == 4) before = (MemT)lo_in;
                 else before = split_value(lo_in, hi_in, p.split);
                 // a thread without steps counts nothing (the first step of the warp is one of the others', or the warp's usage in front)
-                MemT w_top = warp_max_t(tb < te ? (MemT)(before + top) : (sizeof(MemT) == 8 ? (MemT)(INT64_MIN / 4) : (MemT)INT32_MIN));
-                if (lane == 0) s_top[warp] = (int64_t)w_top;
+                w_top = warp_max_t(tb < te ? (MemT)(before + top) : (sizeof(MemT) == 8 ? (MemT)(INT64_MIN / 4) : (MemT)INT32_MIN));
+                if (lane == 0) s_top[first_warp + warp] = (int64_t)w_top;
             }
-            __syncthreads();
-            if (!malformed) {
-                if (warp == 0) out_du = p.base_dur + warp_sum64(lane < n_warps ? s_dur[lane] : 0);
+            sync();
+            if (kMode == kQuadWarps) {
+                if (!malformed) {
+                    out_du = p.base_dur + dw;
+                    out_st = -1;
+                    if (!dep) {
+                        out_pk = (int64_t)w_top;
+                        out_st = out_pk <= p.M ? 1 : 0;
+                    }
+                }
+            } else if (!malformed) {
+                if (warp == 0) out_du = p.base_dur + warp_sum64(lane < n_warps ? s_dur[first_warp + lane] : 0);
                 out_st = -1;
                 if (!dep) {
                     if (kProfile || warp == 0) {
                         // usage in front of every warp
-                        uint32_t lo_w = lane < n_warps ? s_lo[lane] : 0u, hi_w = lane < n_warps ? s_hi[lane] : 0u;
+                        uint32_t lo_w = lane < n_warps ? s_lo[first_warp + lane] : 0u, hi_w = lane < n_warps ? s_hi[first_warp + lane] : 0u;
                         const uint32_t lo_i = warp_inclusive_sum(lo_w, lane) - lo_w, hi_i = sizeof(MemT) == 8 ? warp_inclusive_sum(hi_w, lane) - hi_w : 0u;
                         MemT in_front;
                         if constexpr (sizeof(MemT) == 4) in_front = (MemT)lo_i;
                         else in_front = split_value(lo_i, hi_i, p.split);
                         // a warp without steps holds the smallest value and stays below the others (which are usages, 0 or more)
-                        const MemT pk = warp_max_t(lane < n_warps && s_top[lane] > (sizeof(MemT) == 8 ? INT64_MIN / 4 : (int64_t)INT32_MIN)
-                                                       ? (MemT)(in_front + (MemT)s_top[lane]) : MemT(0));
+                        const MemT pk = warp_max_t(lane < n_warps && s_top[first_warp + lane] > (sizeof(MemT) == 8 ? INT64_MIN / 4 : (int64_t)INT32_MIN)
+                                                       ? (MemT)(in_front + (MemT)s_top[first_warp + lane]) : MemT(0));
                         out_pk = (int64_t)pk;
                         out_st = out_pk <= p.M ? 1 : 0;
                         if constexpr (kProfile) {
@@ -565,9 +636,25 @@ __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
             p.out_dur[b] = out_du;
             p.out_status[b] = out_st;
         }
-        off += max(T, 0);
+        if constexpr (kMode == kQuadBlock) {
+            off += max(T, 0);
+        } else if (self) {
+            off = off_next;
+            T_next = __shfl_sync(kFull, len_raw, 0);
+        }
+        b = b_next;
     }
-    if constexpr (kChip) asm volatile("cp.async.wait_all;" ::: "memory");      // nothing under way where no sequence was evaluated
+    if constexpr (kChip && kProfile) asm volatile("cp.async.wait_all;" ::: "memory");      // nothing under way where no sequence was evaluated
+}
+
+template <typename MemT, int kAcc, bool kTiles, bool kProfile, int kMode>
+__global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
+    quad_evaluate<MemT, kAcc, kTiles, kProfile, kMode>(p);
+}
+// a warp per sequence: a module of its own
+template <typename MemT, int kAcc>
+__global__ void __launch_bounds__(1024) eval_quad_warp_kernel(const QuadParams p) {
+    quad_evaluate<MemT, kAcc, true, false, kQuadWarps>(p);
 }
 
 }  // namespace moc

@@ -106,11 +106,12 @@ def test_small_batches_and_two_part_sums(B, n, C, bits, nB):
         assert_batch_equal(G, O, seqs, lens, M, f"n {n}, thread groups")
 
 
-@pytest.mark.parametrize("n,C,bits,nB", [(20, 3, 0, 1), (63, 3, 37, 148), (64, 4, 0, 149), (65, 3, 0, 444), (65, 4, 37, 445), (440, 2, 0, 149),
-                                         (441, 3, 20, 296), (700, 4, 0, 297), (701, 3, 0, 148), (701, 3, 0, 149), (2111, 4, 20, 9), (4000, 2, 0, 20), (4001, 2, 0, 20)])
-def test_block_kernel_with_and_without_its_own_copy_of_the_graph(B, n, C, bits, nB):
-    """Batches on both sides of the line between the block kernel's two variants, ends of tiles of 64 nodes, packed rows
-    and rows at given offsets (the entry point that does not allocate)."""
+@pytest.mark.parametrize("n,C,bits,nB", [(20, 3, 0, 1), (63, 3, 37, 148), (64, 4, 0, 149), (65, 3, 0, 444), (65, 4, 37, 445), (440, 2, 0, 148),
+                                         (441, 3, 20, 296), (700, 4, 0, 297), (701, 3, 0, 149), (2111, 4, 20, 9), (4001, 3, 0, 20),
+                                         (129, 3, 37, 4000), (130, 4, 0, 5000), (192, 3, 0, 2371), (442, 3, 0, 5000), (443, 4, 20, 1200)])
+def test_block_kernel_variants(B, n, C, bits, nB):
+    """A block, a team of warps and a warp per sequence, in one round and in several, at ends of tiles of 64 nodes; packed
+    rows and rows at given offsets (the entry point that does not allocate)."""
     edges = W.layered_dag(n, 3 * n, max(4, n // 40), n)
     w, m = W.weights_uniform(n, 0, 30, n, 1), np.minimum(W.weights_lognormal(n, 3.0, 1.0, n, 2), 255) << bits
     seqs, lens = W.schedules(n, edges, C, 0.3, nB, n)

@@ -308,14 +308,16 @@ def test_which_kernel_makes_a_profile(fake, n, C, scale, star):
     G.close()
 
 
-@pytest.mark.parametrize("n,C,nB,kernel", [(65, 3, 444, "ILi3ELb1ELb0ELb1E"), (65, 3, 445, "ILi3ELb1ELb0ELb0E"), (700, 4, 444, "ILi4ELb1ELb0ELb1E"),
-                                           (701, 4, 148, "ILi4ELb1ELb0ELb1E"), (701, 4, 149, "ILi4ELb1ELb0ELb0E"), (442, 2, 148, "ILi2ELb1ELb0ELb1E"),
-                                           (442, 2, 149, None), (399, 2, 1, None), (600, 2, 1, None), (4000, 3, 148, "ILi3ELb1ELb0ELb1E"), (4001, 3, 148, "ILi3ELb1ELb0ELb0E")])
-def test_the_block_kernel_copies_the_graph_for_small_batches(fake, n, C, nB, kernel):
+# rows of the block kernel's code: a warp per sequence, teams of warps, a block and the graph through L1; and the warp kernel's teams
+@pytest.mark.parametrize("n,C,nB,kernel", [(65, 3, 3000, "eval_quad_warp_kernelIiLi3E"), (130, 4, 18944, "eval_quad_warp_kernelIiLi4E"), (442, 3, 1, "eval_quad_kernelIiLi3ELb1ELb0ELi1E"),
+                                           (1000, 4, 148, "eval_quad_kernelIiLi4ELb1ELb0ELi1E"), (5000, 4, 300, "eval_quad_kernelIiLi4ELb1ELb0ELi0E"),
+                                           (442, 2, 148, "eval_quad_kernelIiLi2ELb1ELb0ELi1E"), (442, 2, 149, "eval_pair_kernelIiLi0ELb1E"),
+                                           (399, 2, 1, "eval_pair_kernelIiLi0ELb1E"), (600, 2, 1, "eval_pair_kernelIiLi0ELb1E"), (600, 2, 1300, "eval_pair_kernelIiLi5ELb0E")])
+def test_which_variant_takes_a_batch(fake, n, C, nB, kernel):
     G, x = Graph(fake, n, C), np.zeros(8, np.int64)
     fake.fake_reset(0)
     assert fake.moc_eval_batch(G.h, x.ctypes.data, x.ctypes.data, nB, 0, x.ctypes.data, x.ctypes.data, x.ctypes.data, None) == 0
-    assert len(launched(fake, "eval_quad_kernel" + kernel.replace("I", "Ii", 1) if kernel else "eval_pair_kernelIiLi0ELb1E")) == 1, log(fake)
+    assert len(launched(fake, kernel)) == 1, log(fake)
     G.close()
 
 
