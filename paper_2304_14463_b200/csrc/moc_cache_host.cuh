@@ -19,6 +19,7 @@ struct moc_cache {
     mutable int lanes_state = 0;
     mutable moc::LanesParams lanes{};
     mutable const void* lanes_fn = nullptr;
+    mutable int lanes_wpb = 0;
     mutable size_t lanes_smem = 0;
     mutable int lanes_grid_cap = 0;
 };

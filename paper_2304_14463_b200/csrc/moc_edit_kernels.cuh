@@ -31,6 +31,7 @@ struct EditCacheDev {
     int32_t n, C, P, stride, occ_stride;
     int32_t stride16;           // row stride of the 16-bit arrays row and fre
     int32_t max_T;              // C * n
+    int32_t n_edges;
     const int32_t* succ_start;  // successor and predecessor lists (CSR)
     const int32_t* succ;
     const int32_t* pred_start;

@@ -8,7 +8,7 @@
 
 namespace moc {
 
-constexpr int kLanesThreads = 256;
+constexpr int kLanesThreads = 512;   // at most: 64 registers, 32 warps on an SM in blocks of 4 to 16
 
 struct LanesParams {
     EditParams e;
@@ -17,6 +17,7 @@ struct LanesParams {
     uint32_t warp_bytes;                                  // correction list and difference array of one warp
     uint32_t lh_b, diff_b;                                // after the list values, which come first
     int32_t list_cap;
+    int32_t per_warp;                                     // edits that a warp takes at a time (1 .. 32)
 };
 
 // Bytes of one warp: list values, list ranges (list_cap each), difference array (stride + 4).
@@ -56,7 +57,7 @@ struct LaneParent {
 };
 
 template <typename MemT, bool kGraphOnChip>
-__global__ void __launch_bounds__(kLanesThreads, 4) edit_eval_lanes_kernel(const LanesParams p) {
+__global__ void __launch_bounds__(kLanesThreads, 2) edit_eval_lanes_kernel(const LanesParams p) {
     extern __shared__ __align__(16) char smem[];
     const EditParams& e = p.e;
     const EditCacheDev& c = e.c;
@@ -73,10 +74,12 @@ __global__ void __launch_bounds__(kLanesThreads, 4) edit_eval_lanes_kernel(const
     for (int32_t i = lane; i < c.stride + 4; i += 32) diff[i] = 0;
     __syncwarp();
 
-    const int64_t n_groups = ((int64_t)e.B + 31) / 32;
-    for (int64_t g = (int64_t)blockIdx.x * wpb + warp; g < n_groups; g += (int64_t)gridDim.x * wpb) {
-        const int64_t i = g * 32 + lane;
-        const bool have = i < e.B;
+    const uint32_t per_warp = p.per_warp, n_groups = ((uint32_t)e.B + per_warp - 1u) / per_warp;
+    // one round or less: groups follow one another over the blocks, so that a batch of few spreads over all of them
+    const uint32_t first = n_groups <= gridDim.x * wpb ? blockIdx.x + gridDim.x * warp : blockIdx.x * wpb + warp;
+    for (uint32_t g = first; g < n_groups; g += gridDim.x * wpb) {
+        const int64_t i = (int64_t)g * per_warp + lane;
+        const bool have = lane < (int)per_warp && i < e.B;
         int32_t ci = 0, o = 0, qq = 0, jj = 0;
         if (have) {
             ci = __ldg(&e.parent[i]);

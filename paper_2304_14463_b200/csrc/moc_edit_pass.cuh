@@ -59,24 +59,33 @@ struct ScoreGraph {
     __device__ __forceinline__ MemT m(int32_t v) const { return kChip ? s_m[v] : (MemT)__ldg(&c->m[v]); }
 };
 
-// Fills the block's copy of the graph (all threads of the block; ends with a barrier).
+// Fills the block's copy of the graph (all threads of the block; ends with a barrier).  Reads whole 16-byte vectors, which the
+// handle's arrays are padded to, one of every array in flight per thread: a batch of few edits waits for this (n = 442,
+// 256 threads: seven round trips to L2 element by element, two so).
 template <typename MemT>
 __device__ __forceinline__ void score_stage_graph(const EditCacheDev& c, char* smem, uint32_t pred_b, uint32_t m_b, uint32_t succ_b,
                                                   uint32_t predl_b) {
-    uint32_t* ss = reinterpret_cast<uint32_t*>(smem);
-    uint32_t* ps = reinterpret_cast<uint32_t*>(smem + pred_b);
-    MemT* sm = reinterpret_cast<MemT*>(smem + m_b);
-    uint16_t* sl = reinterpret_cast<uint16_t*>(smem + succ_b);
-    uint16_t* pl = reinterpret_cast<uint16_t*>(smem + predl_b);
-    const int32_t E = __ldg(&c.succ_start[c.n]);
-    for (int32_t i = threadIdx.x; i <= c.n; i += blockDim.x) {
-        ss[i] = (uint32_t)__ldg(&c.succ_start[i]);
-        ps[i] = (uint32_t)__ldg(&c.pred_start[i]);
-        if (i < c.n) sm[i] = (MemT)__ldg(&c.m[i]);
-    }
-    for (int32_t i = threadIdx.x; i < E; i += blockDim.x) {
-        sl[i] = (uint16_t)__ldg(&c.succ[i]);
-        pl[i] = (uint16_t)__ldg(&c.pred[i]);
+    const int32_t n_start = (c.n + 4) >> 2, n_list = (c.n_edges + 3) >> 2, n_m = (c.n + 1) >> 1;       // vectors
+    auto packed = [](int4 v) { return make_uint2((uint32_t)(v.x & 0xFFFF) | (uint32_t)v.y << 16, (uint32_t)(v.z & 0xFFFF) | (uint32_t)v.w << 16); };
+    for (int32_t i = threadIdx.x; i < max(max(n_start, n_list), n_m); i += blockDim.x) {
+        int4 a, b, l, q;
+        longlong2 m;
+        const bool hs = i < n_start, hl = i < n_list, hm = i < n_m;
+        if (hs) { a = __ldg(reinterpret_cast<const int4*>(c.succ_start) + i); b = __ldg(reinterpret_cast<const int4*>(c.pred_start) + i); }
+        if (hl) { l = __ldg(reinterpret_cast<const int4*>(c.succ) + i); q = __ldg(reinterpret_cast<const int4*>(c.pred) + i); }
+        if (hm) m = __ldg(reinterpret_cast<const longlong2*>(c.m) + i);
+        if (hs) {
+            reinterpret_cast<int4*>(smem)[i] = a;
+            reinterpret_cast<int4*>(smem + pred_b)[i] = b;
+        }
+        if (hl) {
+            reinterpret_cast<uint2*>(smem + succ_b)[i] = packed(l);
+            reinterpret_cast<uint2*>(smem + predl_b)[i] = packed(q);
+        }
+        if (hm) {
+            if constexpr (sizeof(MemT) == 4) reinterpret_cast<int2*>(smem + m_b)[i] = make_int2((int)m.x, (int)m.y);
+            else reinterpret_cast<longlong2*>(smem + m_b)[i] = m;
+        }
     }
     __syncthreads();
 }

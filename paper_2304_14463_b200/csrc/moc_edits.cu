@@ -121,6 +121,7 @@ int moc_cache_create(const moc_graph* g, int32_t max_parents, moc_cache** out) {
     c.occ_stride = occ_stride;
     c.stride16 = stride16;
     c.max_T = (int32_t)max_T;
+    c.n_edges = (int32_t)g->n_edges;
     c.succ_start = g->d_succ_start;
     c.succ = g->d_succ;
     c.pred_start = g->d_pred_start;
@@ -196,20 +197,26 @@ int moc_eval_edits(const moc_cache* h, const int32_t* parent, const int32_t* op,
         lp.list_cap = std::max(128, (4 + 2 * g->max_indeg + 31) & ~31);
         lp.warp_bytes = (uint32_t)moc::lanes_warp_bytes(h->c.stride, msz, lp.list_cap, &lp.lh_b, &lp.diff_b);
         const size_t cap = g->smem_optin > 2048 ? g->smem_optin - 2048 : 0;
-        const int wpb = moc::kLanesThreads / 32;
         const size_t graph_b = moc::score_graph_bytes(g->n, g->n_edges, msz, &lp.gs_pred_b, &lp.gs_m_b, &lp.gs_succ_b, &lp.gs_predl_b);
         for (int chip = 1; chip >= 0 && h->lanes_state < 0; --chip) {
             if (chip && (g->n > 65535 || graph_b > cap / 8)) continue;
-            const size_t smem = (chip ? graph_b : 0) + (size_t)lp.warp_bytes * wpb;
-            if (smem > cap) continue;
             const void* fn = chip ? (h->wide ? (const void*)moc::edit_eval_lanes_kernel<int64_t, true> : (const void*)moc::edit_eval_lanes_kernel<int32_t, true>)
                                   : (h->wide ? (const void*)moc::edit_eval_lanes_kernel<int64_t, false> : (const void*)moc::edit_eval_lanes_kernel<int32_t, false>);
             MOC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(g->smem_optin - 1024)));
-            int nb = 0;
-            MOC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, moc::kLanesThreads, smem));
+            // the block size that puts most warps on an SM, eight warps among equals
+            int wpb = 0, nb = 0;
+            for (int w : {8, 16, 12, 6, 4}) {
+                const size_t sm = (chip ? graph_b : 0) + (size_t)lp.warp_bytes * w;
+                int k = 0;
+                if (sm > cap) continue;
+                MOC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, fn, 32 * w, sm));
+                if (k * w > nb * wpb) { wpb = w; nb = k; }
+            }
             if (nb < 1) continue;
+            const size_t smem = (chip ? graph_b : 0) + (size_t)lp.warp_bytes * wpb;
             lp.graph_bytes = chip ? (uint32_t)graph_b : 0u;
             h->lanes_fn = fn;
+            h->lanes_wpb = wpb;
             h->lanes_smem = smem;
             h->lanes_grid_cap = g->sm_count * nb;
             h->lanes_state = 1;
@@ -219,11 +226,18 @@ int moc_eval_edits(const moc_cache* h, const int32_t* parent, const int32_t* op,
         moc::LanesParams lp = h->lanes;
         lp.e = p;
         lp.e.c.cap = g->d_cap;
-        const int wpb = moc::kLanesThreads / 32;
-        const int64_t n_groups = ((int64_t)B + 31) / 32;
-        const int grid = (int)std::min<int64_t>(h->lanes_grid_cap, (n_groups + wpb - 1) / wpb);
+        const int wpb = h->lanes_wpb;
+        // Edits per warp: as few as keep the number of rounds of the warps that the device holds, at most 32.  A warp finishes its
+        // admissible edits one after the other, so that a batch that leaves warps idle should not fill any (us with 32 / with this
+        // rule: 112 edits at n = 442 18.8 / 10.8, 1712 at n = 221 27.2 / 12.7, 16000 at n = 442 31.1 / 18.9), and two rounds of 28
+        // beat one of 32 and a shorter one where the windows are long (262144 edits: n = 442 82.1 / 74.3, n = 200 70.1 / 64.2; n = 25 65.5 / 66.6,
+        // n = 36 with 64-bit sums 71.7 / 73.0).
+        const int64_t warps = (int64_t)h->lanes_grid_cap * wpb, rounds = ((int64_t)B + 32 * warps - 1) / (32 * warps);
+        lp.per_warp = rounds > 1 && g->n < 100 ? 32 : (int32_t)std::max<int64_t>(1, (B + rounds * warps - 1) / (rounds * warps));
+        const int64_t n_groups = ((int64_t)B + lp.per_warp - 1) / lp.per_warp;
+        const int grid = (int)std::min<int64_t>(h->lanes_grid_cap, n_groups);
         void* args[] = {&lp};
-        MOC_CUDA(cudaLaunchKernel(h->lanes_fn, dim3(grid), dim3(moc::kLanesThreads), args, h->lanes_smem, (cudaStream_t)stream));
+        MOC_CUDA(cudaLaunchKernel(h->lanes_fn, dim3(grid), dim3(32 * wpb), args, h->lanes_smem, (cudaStream_t)stream));
         launch_counter() = 1;
         return MOC_OK;
     }

@@ -223,3 +223,23 @@ def test_stale_cache_is_refused(B):
     want = reference(O, seqs, lens, parent, op, q, j, M, O.eval_batch(seqs, lens, M)[2])
     assert (got == want).all()
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("n,shift,nE", [(21, 0, 1), (22, 33, 37), (23, 0, 1184), (99, 33, 4735), (100, 0, 4736), (101, 33, 4737), (100, 33, 160000), (1642, 33, 300)])
+def test_edits_per_warp(B, n, shift, nE):
+    """Batches from one edit per warp to several rounds, ends of the block's copy of the graph (odd numbers of nodes and edges), and
+    state that leaves room for few warps: against the oracle, and every edit the same in batches of other sizes."""
+    edges = W.layered_dag(n, 3 * n + n % 4, max(4, n // 40), n)
+    wl = type("WL", (), dict(n=n, edges=edges, C=2, w=W.weights_uniform(n, 0, 30, n, 1), m=W.weights_lognormal(n, 3.0, 1.0, n, 2) << shift))
+    seqs, lens = W.schedules(n, edges, 2, 0.3, 9, n)
+    rng = np.random.default_rng(n)
+    M = OracleGraph(n, edges, wl.w, wl.m, 2).eval(np.arange(n), BIG)["peak"] * 90 // 100
+    rec = random_edits(rng, lens, nE)
+    some = np.sort(rng.choice(nE, min(nE, 5000), replace=False))
+    run_case(B, wl, seqs, lens, M, *(x[some] for x in rec), what=f"n {n}")
+    cache = B.EditCache(B.Graph(n, edges, wl.w, wl.m, 2), len(lens))
+    cache.build(dev(seqs), dev(lens), M)
+    whole = cache.eval_edits(*(dev(x) for x in rec), M)
+    part = cache.eval_edits(*(dev(x[some]) for x in rec), M)
+    for a, b in zip(whole, part):
+        assert torch.equal(a[torch.from_numpy(some).cuda()], b)
