@@ -56,7 +56,8 @@ struct PrepParams {
     EditCacheDev c;
     const int32_t* seqs;        // packed parents
     const int32_t* lens;
-    const int64_t* offs;        // exclusive prefix sum of the lengths
+    const int64_t* offs;        // row offsets, or nullptr (then without todo): packed rows, found from the lengths
+    int32_t per_block, spare;   // rows found by the kernel: block c takes per_block parents, one more when c < spare
     int64_t M;
     int64_t* out_peak;          // may be null
     int64_t* out_dur;
@@ -68,6 +69,7 @@ struct PrepParams {
     // n_tiles = 0: not available, the node pass walks the plain successor lists
     int32_t n_tiles;
     int32_t split;              // records with 64-bit sums: bits of the low part of m
+    int32_t split_ok;           // ... and the two parts may be added up separately (moc_pair_kernel.cuh)
     const void* rec;
     const uint64_t* wslot;
     const uint32_t* sell;
@@ -131,22 +133,23 @@ __host__ __device__ inline size_t edit_warp_bytes(int32_t n, int32_t stride, siz
 // Full evaluation of every parent (same quantities as the evaluation kernels: Section 2, Eqs. 1-8)
 // that also writes the cache.  One warp per parent.
 template <typename MemT, bool kChip>
-__global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepParams p) {
+__global__ void __launch_bounds__(kPrepThreads, 1) edit_prepare_kernel(const PrepParams p) {
     extern __shared__ __align__(16) char smem[];
     const EditCacheDev& c = p.c;
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
     if (kChip) {
         // what the L1 keeps of the tiles between parents is little beside the warps' arrays: the block holds its own copy
-        const uint32_t rec_v = (sizeof(MemT) == 4 ? 8u : 16u) * 64u * (uint32_t)p.n_tiles / 16u, w_v = 8u * 64u * (uint32_t)p.n_tiles / 16u;
-        const uint32_t sell_v = ((uint32_t)p.sell_len * 4u + 15u) / 16u;
-        const uint4* g_rec = reinterpret_cast<const uint4*>(p.rec);
-        const uint4* g_w = reinterpret_cast<const uint4*>(p.wslot);
-        const uint4* g_sell = reinterpret_cast<const uint4*>(p.sell);
-        for (uint32_t i = threadIdx.x; i < rec_v; i += blockDim.x) reinterpret_cast<uint4*>(smem)[i] = __ldg(g_rec + i);
-        for (uint32_t i = threadIdx.x; i < w_v; i += blockDim.x) reinterpret_cast<uint4*>(smem + p.chip_w_b)[i] = __ldg(g_w + i);
-        for (uint32_t i = threadIdx.x; i < sell_v; i += blockDim.x) reinterpret_cast<uint4*>(smem + p.chip_sell_b)[i] = __ldg(g_sell + i);
-        __syncthreads();
+        // (asynchronous copies, complete behind the search for the rows)
+        const uint32_t rec_b = (sizeof(MemT) == 4 ? 8u : 16u) * 64u * (uint32_t)p.n_tiles, w_b = 8u * 64u * (uint32_t)p.n_tiles;
+        const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
+        auto copy = [&](uint32_t to, const void* from, uint32_t bytes) {
+            for (uint32_t i = 16u * threadIdx.x; i < bytes; i += 16u * blockDim.x)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i), "l"(reinterpret_cast<const char*>(from) + i) : "memory");
+        };
+        copy(s0, p.rec, rec_b);
+        copy(s0 + p.chip_w_b, p.wslot, w_b);
+        copy(s0 + p.chip_sell_b, p.sell, (uint32_t)p.sell_len * 4u);
     }
     char* ws = smem + (kChip ? p.chip_bytes : 0u) + (size_t)warp * p.warp_bytes;
     uint32_t* word = reinterpret_cast<uint32_t*>(ws);
@@ -156,25 +159,59 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
     MemT* arrB = reinterpret_cast<MemT*>(ws + (size_t)wstride * 4 + arr_bytes);
     constexpr uint32_t kFull = 0xFFFFFFFFu;
 
-    const int32_t count = p.todo != nullptr ? min(*p.todo_count, c.P) : c.P;
+    // 64-bit sums: every delta as two 32-bit words that are added to separately, where the graph's sums permit (a 64-bit addition in
+    // shared memory is a compare-and-swap loop: n = 442, build of 16384 parents and 32768 edits 205 us with it, 171 so)
+    const bool parts = sizeof(MemT) == 8 && p.n_tiles > 0 && p.split_ok;
+    // Parents: with offsets the blocks' warps stride over all of them (or over the listed ones); without, block c takes a contiguous
+    // range and sums the lengths in front of it (`lens` by lane: the lengths of it, it + 1 ..).
+    __shared__ int64_t s_part[kPrepThreads / 32];
+    const bool self = p.offs == nullptr;
+    int32_t count = p.todo != nullptr ? min(*p.todo_count, c.P) : c.P;
+    int32_t it_step = gridDim.x * wpb, it = blockIdx.x + gridDim.x * warp;
+    int64_t off_self = 0;
+    int32_t lens = 0;
+    auto lanes_sum = [&](int32_t raw, int lanes) -> int64_t {   // sum of max(raw, 0) over lanes < `lanes`
+        const uint32_t v = (lane < lanes && raw > 0) ? (uint32_t)raw : 0u;
+        const uint32_t lo = __reduce_add_sync(kFull, v & 0xFFFFu), hi = __reduce_add_sync(kFull, v >> 16);
+        return (int64_t)lo + ((int64_t)hi << 16);
+    };
+    if (self) {
+        const int32_t c0 = (int32_t)blockIdx.x * p.per_block + min((int32_t)blockIdx.x, p.spare);
+        it = c0 + warp;
+        it_step = wpb;
+        const int32_t lens_c0 = c0 + lane < count ? __ldg(p.lens + c0 + lane) : 0;
+        lens = it + lane < count ? __ldg(p.lens + it + lane) : 0;
+        const uint64_t part = warp_sum_u59(lengths_before(p.lens, c0, threadIdx.x, blockDim.x));
+        if (lane == 0) s_part[warp] = (int64_t)part;
+        __syncthreads();
+        off_self = (int64_t)warp_sum_u59(lane < wpb ? (uint64_t)s_part[lane] : 0) + lanes_sum(lens_c0, warp);
+        count = c0 + p.per_block + ((int32_t)blockIdx.x < p.spare ? 1 : 0);
+    }
+    if (kChip) {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+    }
     // the parent after this one is looked up while this one is evaluated (index, then length and row offset)
-    const int32_t it_step = gridDim.x * wpb;
-    int32_t it = blockIdx.x * wpb + warp;
     int32_t b_nx = it < count ? (p.todo != nullptr ? p.todo[it] : it) : 0;
-    int32_t T_nx = it < count ? p.lens[b_nx] : 0;
-    int64_t off_nx = it < count ? p.offs[b_nx] : 0;
+    int32_t T_nx = self ? __shfl_sync(kFull, lens, 0) : (it < count ? p.lens[b_nx] : 0);
+    int64_t off_nx = self ? off_self : (it < count ? p.offs[b_nx] : 0);
     for (; it < count; it += it_step) {
         const int32_t b = b_nx, T = T_nx;
         const int64_t off = off_nx;
         const bool more = it + it_step < count;
         b_nx = more ? (p.todo != nullptr ? p.todo[it + it_step] : it + it_step) : 0;
         bool got_nx = false;
+        if (self) {
+            off_nx = off + lanes_sum(lens, wpb);             // skip the parents it .. it + wpb - 1
+            lens = b_nx + lane < c.P ? __ldg(p.lens + b_nx + lane) : 0;
+        }
         int64_t out_pk = -1, out_du = -1;
         int32_t out_st = -2;
         uint16_t* row = c.row + (int64_t)b * c.stride16;
         if (T >= n && T <= c.max_T) {
             for (int32_t i = lane; i < wstride / 4; i += 32) reinterpret_cast<uint4*>(word)[i] = make_uint4(0, 0, 0, 0);
-            for (int32_t i = lane; i < (int32_t)arr_bytes / 16; i += 32) reinterpret_cast<uint4*>(arrA)[i] = make_uint4(0, 0, 0, 0);
+            // (deltas 0 .. T and what pads the last vector; an absent node's go to entry 0)
+            for (int32_t i = lane; i < min((int32_t)arr_bytes, (T + 2) * (int32_t)sizeof(MemT) + 15) / 16; i += 32) reinterpret_cast<uint4*>(arrA)[i] = make_uint4(0, 0, 0, 0);
             __syncwarp();
             // ---- occurrence words (1-based steps, 16 bits each) and the copy of the row
             const int32_t* src = p.seqs + off;
@@ -194,7 +231,7 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                     if (t0 + 32 * k < T) put(v[k], t0 + 32 * k);
             }
             __syncwarp();
-            if (more) { T_nx = p.lens[b_nx]; off_nx = p.offs[b_nx]; got_nx = true; }
+            if (more && !self) { T_nx = p.lens[b_nx]; off_nx = p.offs[b_nx]; got_nx = true; }
             // ---- per node: both copies a <= b, free steps from the successors' copies, profile deltas
             uint32_t vsum = 0;
             bool absent = false, dep = false, over = false;
@@ -214,6 +251,18 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                 auto ld64 = [&](const uint64_t* q) -> uint64_t { return kChip ? lds_u64((uint32_t)__cvta_generic_to_shared(q)) : __ldg(q); };
                 uint32_t vmin = 0xFFFFFFFFu, depw = 0, capw = 0;
                 uint64_t acc = 0;
+                const uint32_t aa = (uint32_t)__cvta_generic_to_shared(arrA);
+                auto range_add = [&](uint32_t from, uint32_t behind, MemT v) {      // += v on steps from .. behind - 1
+                    if (parts) {
+                        red_add_shared(aa + 8u * from, (int32_t)v);
+                        red_add_shared(aa + 8u * from + 4u, (int32_t)((uint64_t)v >> 32));
+                        red_add_shared(aa + 8u * behind, -(int32_t)v);
+                        red_add_shared(aa + 8u * behind + 4u, -(int32_t)((uint64_t)v >> 32));
+                    } else {
+                        edit_add(&arrA[from], v);
+                        edit_add(&arrA[behind], (MemT)(-v));
+                    }
+                };
                 const uint32_t empty_off = 4u * (((uint32_t)n + 2u + 3u) & ~3u);   // where the records of empty slots point
                 if (lane == 0) {
                     word[n + 1] = (uint32_t)T * 0x10001u;               // the made-up successor of sinks
@@ -222,7 +271,8 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                 __syncwarp();
                 for (int d = 0; d < p.n_tiles; ++d, prec += 64 * kRecB, pw += 64) {
                     uint32_t ab[2], naa[2], nbb[2], Ga[2], Gb[2], xoff[2];
-                    MemT mm[2];
+                    MemT mm[2];                                          // or, with `parts`, its two parts
+
                     int rows = 0;
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -237,7 +287,8 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                                                   : __ldg(reinterpret_cast<const uint4*>(prec + 32 * kRecB * h));
                             x = r.x;
                             // m from its two parts (moc_pair_kernel.cuh)
-                            mm[h] = (MemT)((uint64_t)r.w << p.split | (r.z & (uint32_t)(((uint64_t)1 << p.split) - 1)));
+                            mm[h] = parts ? (MemT)((uint64_t)r.w << 32 | r.z)
+                                          : (MemT)((uint64_t)r.w << p.split | (r.z & (uint32_t)(((uint64_t)1 << p.split) - 1)));
                         }
                         if (h == 0) rows = (int)(x >> 16);
                         xoff[h] = x & 0xFFFFu;
@@ -271,12 +322,10 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                         const bool real = xoff[h] != empty_off;          // empty slots own the constant word: no step is theirs
                         if (real && b16 != 0) {
                             fre16[b16 - 1] = (uint16_t)(fb - 1);         // free steps gather on chip, written out in order below
-                            edit_add(&arrA[b16 - 1], mm[h]);
-                            edit_add(&arrA[fb], (MemT)(-mm[h]));
+                            range_add(b16 - 1, fb, mm[h]);
                             if (a16 != b16) {
                                 fre16[a16 - 1] = (uint16_t)(fa - 1);
-                                edit_add(&arrA[a16 - 1], mm[h]);
-                                edit_add(&arrA[fa], (MemT)(-mm[h]));
+                                range_add(a16 - 1, fa, mm[h]);
                                 const uint64_t wx = ld64(pw + 32 * h);
                                 capw |= (uint32_t)(wx >> 32);
                                 acc += wx;
@@ -350,11 +399,18 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                 auto stv = [](MemT* a, const MemT (&v)[VW]) { *reinterpret_cast<uint4*>(a) = *reinterpret_cast<const uint4*>(v); };
                 // pass 1: sum and largest running sum of the run, both relative to its start
                 MemT sum = 0, top = 0;
+                uint32_t p_lo = 0, p_hi = 0;                                // `parts`: the words since the start of the run
+                auto step = [&](MemT at, MemT d) -> MemT {                  // the running sum `at` (from the run's start) after delta d
+                    if (!parts) return at + d;
+                    p_lo += (uint32_t)d;
+                    p_hi += (uint32_t)((uint64_t)d >> 32);
+                    return (MemT)split_value(p_lo, p_hi, p.split);
+                };
                 for (int32_t t = t0; t < t1; t += VW) {
                     alignas(16) MemT v[VW];
                     ldv(arrA + t, v);
 #pragma unroll
-                    for (int i = 0; i < VW; ++i) { sum += v[i]; top = sum > top ? sum : top; }
+                    for (int i = 0; i < VW; ++i) { sum = step(sum, v[i]); top = sum > top ? sum : top; }
                 }
                 MemT run = edit_warp_incl_sum(sum, lane) - sum;             // usage in front of the run
                 top += run;                                                 // largest usage inside the run (0 for an empty one)
@@ -363,12 +419,16 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
                 carry = __shfl_up_sync(kFull, carry, 1);
                 if (lane == 0) carry = 0;
                 // pass 2: usage and prefix maxima
+                const MemT front = run;
+                p_lo = p_hi = 0;
+                sum = 0;
                 for (int32_t t = t0; t < t1; t += VW) {
                     alignas(16) MemT v[VW], w[VW];
                     ldv(arrA + t, v);
 #pragma unroll
                     for (int i = 0; i < VW; ++i) {
-                        run += v[i];
+                        sum = step(sum, v[i]);
+                        run = front + sum;
                         v[i] = run;
                         carry = run > carry ? run : carry;
                         w[i] = carry;
@@ -409,7 +469,8 @@ __global__ void __launch_bounds__(kPrepThreads) edit_prepare_kernel(const PrepPa
             }
             __syncwarp();
         }
-        if (more && !got_nx) { T_nx = p.lens[b_nx]; off_nx = p.offs[b_nx]; }
+        if (self) T_nx = __shfl_sync(kFull, lens, 0);
+        else if (more && !got_nx) { T_nx = p.lens[b_nx]; off_nx = p.offs[b_nx]; }
         if (lane == 0) {
             c.len[b] = T;
             c.status[b] = out_st;

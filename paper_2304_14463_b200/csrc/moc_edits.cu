@@ -39,6 +39,7 @@ int cache_prepare(moc_cache* h, const int32_t* seqs, const int32_t* lens, const 
     p.n_tiles = tiles ? g->n_tiles : 0;
     p.rec = h->wide ? g->d_rec64 : g->d_rec32;
     p.split = g->split;
+    p.split_ok = g->split_ok ? 1 : 0;
     p.wslot = g->d_wslot;
     p.sell = g->d_sell;
     p.base_dur = g->sum_w;
@@ -60,7 +61,11 @@ int cache_prepare(moc_cache* h, const int32_t* seqs, const int32_t* lens, const 
     const void* fn = chip ? (h->wide ? (const void*)moc::edit_prepare_kernel<int64_t, true> : (const void*)moc::edit_prepare_kernel<int32_t, true>)
                           : (h->wide ? (const void*)moc::edit_prepare_kernel<int64_t, false> : (const void*)moc::edit_prepare_kernel<int32_t, false>);
     MOC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(optin - 1024)));
-    const int grid = (int)std::min<int64_t>(grid_cap, ((int64_t)P + wpb - 1) / wpb);
+    // a build of few parents spreads over the SMs
+    const int grid = (int)std::min<int64_t>(grid_cap, std::max<int64_t>(((int64_t)P + wpb - 1) / wpb, std::min(P, g->sm_count)));
+    wpb = (int)std::min<int64_t>(wpb, ((int64_t)P + grid - 1) / grid);
+    p.per_block = P / grid;
+    p.spare = P % grid;
     void* args[] = {&p};
     MOC_CUDA(cudaLaunchKernel(fn, dim3(grid), dim3(32 * wpb), args, (chip ? chip_b : 0) + h->warp_bytes * wpb, st));
     MOC_CUDA(cudaGetLastError());
@@ -155,10 +160,12 @@ int moc_cache_build(moc_cache* h, const int32_t* seqs, const int32_t* lens, int3
     DeviceGuard dg(h->device);
     if (!dg.ok) return fail(MOC_ERR_CUDA, "cannot select device %d", h->device);
     cudaStream_t st = (cudaStream_t)stream;
-    moc::offsets_kernel<<<(P + moc::kOffsTile - 1) / moc::kOffsTile, moc::kOffsThreads, 0, st>>>(lens, P, h->d_offs);
-    int rc = cache_prepare(h, seqs, lens, h->d_offs, P, nullptr, nullptr, M, out_peak, out_dur, out_status, st);
+    // every block adds up the lengths in front of its parents while that is little next to a launch (4 us)
+    const bool self = (int64_t)h->g->sm_count * P * 2 <= (int64_t)16 << 20;
+    if (!self) moc::offsets_kernel<<<(P + moc::kOffsTile - 1) / moc::kOffsTile, moc::kOffsThreads, 0, st>>>(lens, P, h->d_offs);
+    int rc = cache_prepare(h, seqs, lens, self ? nullptr : h->d_offs, P, nullptr, nullptr, M, out_peak, out_dur, out_status, st);
     if (rc != MOC_OK) return rc;
-    launch_counter() = 2;
+    launch_counter() = self ? 1 : 2;
     return MOC_OK;
 }
 

@@ -243,3 +243,15 @@ def test_edits_per_warp(B, n, shift, nE):
     part = cache.eval_edits(*(dev(x[some]) for x in rec), M)
     for a, b in zip(whole, part):
         assert torch.equal(a[torch.from_numpy(some).cuda()], b)
+
+
+@pytest.mark.parametrize("n,shift,P", [(100, 0, 1), (100, 33, 147), (101, 0, 149), (100, 44, 149), (442, 33, 300), (101, 0, 3553), (64, 33, 8000)])
+def test_build_of_few_and_many_parents(B, n, shift, P):
+    """Parents by block and warp, in one round and in several, with sums in one, two and 64-bit parts; some edits of damaged and good ones."""
+    edges = W.layered_dag(n, 3 * n, max(4, n // 40), n)
+    m = np.minimum(W.weights_lognormal(n, 3.0, 1.0, n, 2), 255) << shift
+    wl = type("WL", (), dict(n=n, edges=edges, C=2, w=W.weights_uniform(n, 0, 30, n, 1), m=m))
+    seqs, lens = W.schedules(n, edges, 2, 0.3, P, n)
+    seqs, lens = W.mutate(seqs, lens, n, 2, seed=5, frac=1 / 8)
+    M = OracleGraph(n, edges, wl.w, wl.m, 2).eval(np.arange(n), BIG)["peak"] * 90 // 100
+    run_case(B, wl, seqs, lens, M, *random_edits(np.random.default_rng(P), np.clip(lens, 0, None), 1500), what=f"n {n} P {P}")
