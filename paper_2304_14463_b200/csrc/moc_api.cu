@@ -641,6 +641,21 @@ void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::ve
         for (int64_t k = 0; k < ne; ++k) pred[fill[keys[k] & 0xFFFFFFFFu]++] = (int32_t)(keys[k] >> 32);
         for (int32_t v = 0; v < n; ++v)
             if (succ_start[v + 1] == succ_start[v]) g->sink_m += m[v];
+        if (ne <= 65535 && g->sum_w < ((int64_t)1 << 31) && g->n <= 16000) {
+            const size_t list = ((size_t)ne + 3) & ~size_t(3);
+            std::vector<uint32_t> near((2 * ((size_t)n + 1) + list + 3) & ~size_t(3), 0u);
+            uint16_t* lists = reinterpret_cast<uint16_t*>(near.data() + 2 * ((size_t)n + 1));
+            for (int32_t v = 0; v <= n; ++v) {
+                near[2 * (size_t)v] = (uint32_t)succ_start[v] | (uint32_t)pred_start[v] << 16;
+                near[2 * (size_t)v + 1] = v < n ? (uint32_t)w[v] : 0u;
+            }
+            for (int64_t k = 0; k < ne; ++k) {
+                lists[k] = (uint16_t)succ[k];
+                lists[list + k] = (uint16_t)pred[k];
+            }
+            g->near_bytes = near.size() * 4;
+            tables->add(&g->d_near, std::move(near));
+        }
         tables->add(&g->d_pred_start, std::move(pred_start));
         tables->add(&g->d_pred, std::move(pred));
     }

@@ -123,26 +123,32 @@ void plan_walk(moc_search* s) {
     w.word_bytes = (4u * ((uint32_t)g->n + 2u) + 15u) & ~15u;
     w.delta_bytes = (uint32_t)(moc::kPairDeltaFront + 32 * v_max * 16);
     const size_t warp_b = moc::walk_warp_bytes(w.word_bytes, w.delta_bytes), graph_b = (size_t)w.rec_bytes + w.sell_bytes;
-    const void* fn = walk_fn(wide);
     const size_t cap = g->smem_optin;
     if (graph_b + 4 * warp_b > cap) return;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
     // Chains that fit the device at once get one round with as few warps per SM as that takes; larger
-    // populations the shape with the smallest rounds * warps (an SM's rate hardly depends on its warps beyond 16).
+    // populations the shape with the smallest rounds * (warps + 10): a round is a chain's latency and the SM's work.
     const int sm = g->sm_count, most = (int)std::min<size_t>(moc::kWalkThreads / 32, (cap - graph_b) / warp_b);
     int best = 0;
     int64_t best_cost = 0;
     for (int k = most; k >= 1; --k) {
         const int64_t rounds = ((int64_t)s->P + (int64_t)sm * k - 1) / ((int64_t)sm * k);
-        const int64_t cost = rounds * std::max(k, std::min(most, 16));
-        if (best == 0 || cost < best_cost || (cost == best_cost && rounds == 1)) { best = k; best_cost = cost; }
+        const int64_t cost = rounds * (k + 10);
+        if (best == 0 || cost < best_cost) { best = k; best_cost = cost; }
+    }
+    // the neighbours' lists where they fit beside that many warps
+    w.n_edges = (int32_t)g->n_edges;
+    const size_t list_b = g->near_bytes;
+    const bool lists = g->d_near != nullptr && graph_b + list_b + (size_t)best * warp_b <= cap;
+    w.lists = g->d_near;
+    w.list_bytes = (uint32_t)list_b;
+    const void* fn = walk_fn(wide, lists);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
+        cudaGetLastError();
+        return;
     }
     s->walk_wpb = best;
     s->walk_grid = (int)std::min<int64_t>(sm, ((int64_t)s->P + best - 1) / best);
-    s->walk_smem = graph_b + (size_t)best * warp_b;
+    s->walk_smem = graph_b + (lists ? list_b : 0) + (size_t)best * warp_b;
     s->walk_fn = fn;
 }
 

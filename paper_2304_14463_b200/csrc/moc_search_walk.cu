@@ -3,5 +3,8 @@
 #include "moc_search_walk_kernel.cuh"
 
 namespace moc_host {
-const void* walk_fn(bool wide) { return wide ? (const void*)moc::search_walk_kernel<int64_t> : (const void*)moc::search_walk_kernel<int32_t>; }
+const void* walk_fn(bool wide, bool lists) {
+    if (lists) return wide ? (const void*)moc::search_walk_kernel<int64_t, true> : (const void*)moc::search_walk_kernel<int32_t, true>;
+    return wide ? (const void*)moc::search_walk_kernel<int64_t, false> : (const void*)moc::search_walk_kernel<int32_t, false>;
+}
 }  // namespace moc_host

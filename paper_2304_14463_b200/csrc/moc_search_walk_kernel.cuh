@@ -20,11 +20,11 @@
 // Chains without a valid sequence (status < 0) have no test to rely on: their proposals are evaluated from
 // the written-out order, one generation at a time, until one is valid.
 //
-// Bound: instruction issue (53 % of the slots, 2100 instructions per generation of 32 proposals) and the latency of
-// its dependent shared-memory reads; 28 warps beat 24 and 20 with more registers each, and 30 with fewer.
+// Bound: instruction issue (72 % of the slots with 32 proposals a generation, 2000 instructions each) and, for small populations,
+// the latency of its dependent shared-memory reads; 28 warps beat 24 and 20 with more registers each, and 30 with fewer.
 // n = 442, state copied out: 4096 chains x 20 generations 436 -> 41.9 us against two kernels per generation that
-// write every proposal out; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us against a cached
-// evaluation per chain that is rebuilt after every acceptance.
+// write every proposal out, 38.9 with the neighbours' lists on chip; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us
+// against a cached evaluation per chain that is rebuilt after every acceptance, 1010 -> 951 with the lists.
 #pragma once
 #include "moc_edit_kernels.cuh"
 #include "moc_search_kernels.cuh"
@@ -50,6 +50,9 @@ struct WalkParams {
     const int64_t* w;
     const int32_t* cap;        // per-node caps or nullptr
     uint32_t rec_bytes, sell_bytes;      // graph, once per block
+    int32_t n_edges;
+    const uint32_t* lists;     // kLists: the neighbours' lists (walk_lists), behind the graph in shared memory
+    uint32_t list_bytes;
     uint32_t word_bytes;       // occurrence words (n + 2, padded) without the constant word behind them
     uint32_t delta_bytes;      // front pad + deltas for C * n steps
 };
@@ -191,22 +194,39 @@ static __device__ __noinline__ void walk_apply(int32_t* row, int32_t T, int32_t 
     __syncwarp();
 }
 
-template <typename MemT>
+// kLists: the test of a proposal reads the neighbours' lists from the block's shared memory (durations below 2^31, at most 65535 edges);
+// through L1, of which the chains' state leaves little, a third of the kernel's stalls were waits for them.
+template <typename MemT, bool kLists>
 __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const WalkParams p) {
     extern __shared__ __align__(16) char smem[];
     const SearchParams& s = p.s;
     constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
-    {
-        int4* s4 = reinterpret_cast<int4*>(smem);
-        const uint32_t n_rec = p.rec_bytes >> 4, n_all = (p.rec_bytes + p.sell_bytes) >> 4;
-        for (uint32_t i = threadIdx.x; i < n_all; i += blockDim.x)
-            s4[i] = i < n_rec ? __ldg(reinterpret_cast<const int4*>(p.rec) + i) : __ldg(reinterpret_cast<const int4*>(p.sell) + (i - n_rec));
-    }
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
+    const uint32_t l_node = sbase + p.rec_bytes + p.sell_bytes, l_succ = l_node + 8u * (uint32_t)(p.n + 1), l_pred = l_succ + 2u * (uint32_t)((p.n_edges + 3) & ~3);
+    {
+        // asynchronous copies: a block of a small population has few threads for them
+        auto copy = [&](uint32_t to, const void* from, uint32_t bytes) {
+            for (uint32_t i = 16u * threadIdx.x; i < bytes; i += 16u * blockDim.x)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i), "l"(reinterpret_cast<const char*>(from) + i) : "memory");
+        };
+        copy(sbase, p.rec, p.rec_bytes);
+        copy(sbase + p.rec_bytes, p.sell, p.sell_bytes);
+        if constexpr (kLists) copy(l_node, p.lists, p.list_bytes);
+    }
     const uint32_t word_set = p.word_bytes + kPairWordTail;
-    const uint32_t mine = sbase + p.rec_bytes + p.sell_bytes + (uint32_t)warp * (2u * word_set + kWalkNoteBytes + p.delta_bytes);
+    auto duration = [&](int32_t v) -> int64_t { return kLists ? (int64_t)lds_u32_nv(l_node + 8u * (uint32_t)v + 4u) : __ldg(p.w + v); };
+    auto neighbour = [&](uint32_t list, const int32_t* far, int32_t k) -> uint32_t {
+        if constexpr (kLists) {
+            uint32_t x;
+            asm("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(x) : "r"(list + 2u * (uint32_t)k));
+            return x;
+        } else {
+            return (uint32_t)__ldg(far + k);
+        }
+    };
+    const uint32_t mine = sbase + p.rec_bytes + p.sell_bytes + (kLists ? p.list_bytes : 0u) + (uint32_t)warp * (2u * word_set + kWalkNoteBytes + p.delta_bytes);
     const uint32_t note = mine + 2u * word_set;
     const uint32_t da = note + kWalkNoteBytes + kPairDeltaFront;     // &delta[0]
     const uint32_t rec0 = sbase + kRecB * (uint32_t)lane, sell0 = sbase + p.rec_bytes + 4u * (uint32_t)lane;
@@ -214,6 +234,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
     if (lane < 2) sts_u32(mine + word_set * (uint32_t)lane + p.word_bytes, 0x00010001u);   // owned by empty node slots
     for (uint32_t o = 16u * (uint32_t)lane; o < p.delta_bytes; o += 512u)
         asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(da - kPairDeltaFront + o), "r"(0) : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
     for (int32_t c = blockIdx.x * wpb + warp; c < s.P; c += gridDim.x * wpb) {
@@ -241,7 +262,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                     const int32_t k = t - (t > ji ? 1 : 0);
                     v = row[k + (k >= qd ? 1 : 0)];
                 }
-                if ((uint32_t)v < (uint32_t)n) sum += __ldg(p.w + v);
+                if ((uint32_t)v < (uint32_t)n) sum += duration(v);
                 const uint32_t addr = w0 + 4u * min((uint32_t)v, (uint32_t)n);
                 const uint32_t old = exch_shared(addr, ((uint32_t)t + 1u) * 0x10001u);
                 sts_u16_if_nonzero(old, addr + 2, old);
@@ -278,7 +299,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             const int32_t xa = (int32_t)min(wx & 0xFFFFu, wx >> 16) - 1, xb = (int32_t)max(wx & 0xFFFFu, wx >> 16) - 1;
             const int32_t cnt = xa == xb ? 1 : 2, cnt2 = cnt - (op >= 1 ? 1 : 0) + (op != 1 ? 1 : 0);
             if (!(cnt2 == 1 || (cnt2 == 2 && p.C >= 2 && (p.cap == nullptr || __ldg(p.cap + x) >= 2)))) return false;
-            const int64_t more = __ldg(p.w + x) * (cnt2 - cnt);
+            const int64_t more = duration(x) * (cnt2 - cnt);
             du_c = (int64_t)lds_u64(note + kWalkDu) + more;
             const bool longer = more > 0;
             if (longer && !over) return false;      // within the budget only the duration decides
@@ -303,19 +324,34 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             const int32_t tmax = tp + 16 / (int32_t)sizeof(MemT) - 1;
             if (must_drop && !(xa + 1 < tmax && ji >= tp)) return false;
             bool viol = false, later = false;
-            const int32_t p0 = __ldg(p.pred_start + x), p1 = __ldg(p.pred_start + x + 1);
-            const int32_t s0 = __ldg(p.succ_start + x), s1 = __ldg(p.succ_start + x + 1);
-#pragma unroll 1
-            for (int32_t k = p0; k < p1; ++k) {
-                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.pred + k));
-                viol |= (int32_t)min(wv & 0xFFFFu, wv >> 16) > ta0;
+            int32_t p0, p1, s0, s1;
+            if constexpr (kLists) {
+                const uint32_t from = lds_u32_nv(l_node + 8u * (uint32_t)x), to = lds_u32_nv(l_node + 8u * (uint32_t)x + 8u);
+                s0 = (int32_t)(from & 0xFFFFu);
+                s1 = (int32_t)(to & 0xFFFFu);
+                p0 = (int32_t)(from >> 16);
+                p1 = (int32_t)(to >> 16);
+            } else {
+                p0 = __ldg(p.pred_start + x); p1 = __ldg(p.pred_start + x + 1);
+                s0 = __ldg(p.succ_start + x); s1 = __ldg(p.succ_start + x + 1);
             }
+            // two reads of each kind in flight
 #pragma unroll 1
-            for (int32_t k = s0; k < s1; ++k) {
-                const uint32_t wv = lds_u32(wa + 4u * (uint32_t)__ldg(p.succ + k));
-                const int32_t r0 = (int32_t)min(wv & 0xFFFFu, wv >> 16), r1 = (int32_t)max(wv & 0xFFFFu, wv >> 16);
-                viol |= r0 < tb0 || (must_drop && ((r0 >= tmax && r0 <= ji) || (r1 >= tmax && r1 <= ji)));
-                later |= r1 > ji;
+            for (int32_t k = 0; k < max(p1 - p0, s1 - s0); k += 2) {
+                uint32_t pw[2], sw[2];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    pw[i] = p0 + k + i < p1 ? lds_u32(wa + 4u * neighbour(l_pred, p.pred, p0 + k + i)) : 0u;
+                    sw[i] = s0 + k + i < s1 ? lds_u32(wa + 4u * neighbour(l_succ, p.succ, s0 + k + i)) : 0xFFFFFFFFu;
+                }
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    viol |= (int32_t)min(pw[i] & 0xFFFFu, pw[i] >> 16) > ta0;
+                    const int32_t r0 = (int32_t)min(sw[i] & 0xFFFFu, sw[i] >> 16), r1 = (int32_t)max(sw[i] & 0xFFFFu, sw[i] >> 16);
+                    const bool is = s0 + k + i < s1;
+                    viol |= is && (r0 < tb0 || (must_drop && ((r0 >= tmax && r0 <= ji) || (r1 >= tmax && r1 <= ji))));
+                    later |= is && r1 > ji;
+                }
             }
             return !viol && (!must_drop || later || s0 == s1);
         };

@@ -414,3 +414,23 @@ def test_population_split_over_two_ranks_on_the_gpu():
         p.join(120)
         assert p.exitcode == 0
     assert out == (True, True, True, True)
+
+
+@pytest.mark.parametrize("n,P,w_shift,samples", [(61, 64, 0, 3), (62, 40, 26, 3), (331, 149, 0, 1), (331, 30, 25, 1), (1003, 5, 0, 2), (600, 4200, 0, 1)])
+def test_search_walk_with_and_without_lists(B, n, P, w_shift, samples):
+    """The neighbours' lists in shared memory and, for durations beyond 31 bits or where they do not fit beside the chains, in
+    global memory; odd numbers of nodes and edges; long rows copied out."""
+    edges = W.layered_dag(n, 3 * n + 1, max(4, n // 40), n)
+    w, m = W.weights_uniform(n, 1, 30, n, 1) << w_shift, W.weights_lognormal(n, 3.0, 1.0, n, 2)
+    assert w_shift == 0 or int(w.sum()) >= 1 << 31
+    seqs, lens = W.schedules(n, edges, 2, 0.3, P, n)
+    M = OracleGraph(n, edges, w, m, 2).eval(np.arange(n), 1 << 60)["peak"] * 80 // 100
+    wl = type("WL", (), dict(n=n, edges=edges, C=2, w=w, m=m))
+    if samples == 1:
+        G, O, S, OS = make_pair(B, wl, seqs, lens, M, seed=n)
+        for g in (1, 33):
+            S.run(g)
+            OS.run(g)
+            assert_state_equal(S, OS, f"n {n}, {g} generations")
+    else:
+        _run_scored(B, n, edges, w, m, 2, seqs, lens, M, samples, 1, (2, 9), what=f"n {n}")
