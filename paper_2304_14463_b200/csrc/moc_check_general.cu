@@ -4,21 +4,22 @@
 
 namespace moc_host {
 namespace {
-template <int CP, typename MemT>
+template <int CP, typename MemT, bool kTeams>
 IntervalFn kept_fn(int kept) {
     switch (kept) {
-        case 0: return moc::check_intervals_kernel<true, CP, MemT, false, int32_t>;
-        case 2: return moc::check_intervals_kernel<true, CP, MemT, true, uint16_t>;
-        default: return moc::check_intervals_kernel<true, CP, MemT, true, int32_t>;
+        case 0: return moc::check_intervals_kernel<true, CP, MemT, false, int32_t, kTeams>;
+        case 2: return moc::check_intervals_kernel<true, CP, MemT, true, uint16_t, kTeams>;
+        default: return moc::check_intervals_kernel<true, CP, MemT, true, int32_t, kTeams>;
     }
 }
-template <int CP>
+template <int CP, bool kTeams>
 IntervalFn wide_fn(bool wide, int kept) {
-    return wide ? kept_fn<CP, int64_t>(kept) : kept_fn<CP, int32_t>(kept);
+    return wide ? kept_fn<CP, int64_t, kTeams>(kept) : kept_fn<CP, int32_t, kTeams>(kept);
 }
 }  // namespace
 
-IntervalFn check_general_fn(int cp, bool wide, int kept) {
-    return cp == 2 ? wide_fn<2>(wide, kept) : (cp == 4 ? wide_fn<4>(wide, kept) : wide_fn<8>(wide, kept));
+IntervalFn check_general_fn(int cp, bool wide, int kept, bool team) {
+    if (cp == 2) return team ? wide_fn<2, true>(wide, kept) : wide_fn<2, false>(wide, kept);
+    return cp == 4 ? wide_fn<4, true>(wide, kept) : wide_fn<8, true>(wide, kept);      // one variant for both
 }
 }  // namespace moc_host

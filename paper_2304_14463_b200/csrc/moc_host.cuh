@@ -35,8 +35,8 @@ QuadFn quad_fn(bool wide, int C, bool tiles, bool chip, bool profile);      // c
 QuadFn quad_warp_fn(bool wide, int C);      // a warp per sequence
 LiveFn live_fn(bool wide, int words, int C);
 const void* check_plain_fn(bool wide);
-IntervalFn check_general_fn(int cp, bool wide, int kept);      // kept: bytes per event of the solution kept on chip, 0: not kept
-IntervalFn check_staged_fn(int cp, bool wide, int kept);
+IntervalFn check_general_fn(int cp, bool wide, int kept, bool team);      // kept: bytes per event of the solution kept on chip, 0: not kept
+IntervalFn check_staged_fn(int cp, bool wide, int kept, bool team);      // team: a block per solution
 const void* score_fn(bool wide, bool graph_on_chip);
 const void* walk_fn(bool wide, bool lists);      // lists: the neighbours' lists in shared memory
 

@@ -3,8 +3,9 @@
 // event domain of "Complexity Reduction by Enforcing an Initial Topological Ordering") is checked
 // constraint by constraint, with the duration (Eq. 1) and the peak of the usage of Eq. 4.
 //
-// One warp per solution at a time, warp-synchronous (no block barriers); a block is a few warps that
-// share nothing but the launch.  The event domain can be far larger than the number of intervals
+// One warp per solution at a time, warp-synchronous, a block being a few warps that share nothing but the launch;
+// or, where an SM would have few warps at work (bitmaps of a large domain, small batches), a block of up to 16 warps per
+// solution.  The event domain can be far larger than the number of intervals
 // (n(n+1)/2 staged events for n*C intervals), so usage is not accumulated per event.  It can only
 // rise at the start of an active interval, hence the peak is the largest usage over those start
 // events.  A bitmap over the domain marks them, a prefix count over its words turns an event t into
@@ -14,7 +15,8 @@
 //
 // Bound: latency at the few warps whose bitmaps fit an SM (staged domain, n = 442: 97903 events, 12 KB a warp).  The rank
 // bases therefore take 16 bits per four bitmap words, and the staged rule a 32-bit float root: staged, 16384 solutions,
-// n = 442: 1355 -> 529 us (6 -> 9 warps per SM), n = 900, 2000 solutions: 900 -> 559 us, n = 100: 66.7 -> 58.8 us.
+// n = 442: 1355 -> 529 us (6 -> 9 warps per SM), n = 900, 2000 solutions: 900 -> 559 us, n = 100: 66.7 -> 58.8 us.  Blocks per solution:
+// n = 442, 6000 solutions 222 -> 101 us, 148 39 -> 11; n = 932, 1500 solutions 433 -> 68.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -22,6 +24,7 @@
 namespace moc {
 
 constexpr int kIvMaxWarps = 8;   // warps (solutions in flight) per block, fewer when shared memory is short
+constexpr int kIvMaxTeam = 16;   // warps per solution, where few solutions are in flight
 constexpr int32_t kIvEq2 = 1, kIvEq3 = 2, kIvEq4 = 4, kIvEq5 = 8, kIvEq6 = 16, kIvEq7 = 32, kIvEq8 = 64, kIvStage = 128;
 constexpr int kIvMaxC = 8;       // slots per node held in registers
 
@@ -45,6 +48,7 @@ struct IntervalParams {
     int32_t* out_lens;           // B, or nullptr
     uint32_t words;              // bitmap words: (D + 32) / 32, rounded up to a multiple of 4  (bit t of the bitmap = event t, bit 0 unused)
     uint32_t warp_bytes;         // shared memory of one warp
+    int32_t team;                // a block per solution (else a warp)
     int32_t byte_marks;          // plain model, and two bytes per event fit the space of the difference array
 };
 
@@ -79,14 +83,28 @@ __device__ __forceinline__ void iv_add(int64_t* p, int64_t v) {
 // of the usage sums (int32 when C * sum(m) < 2^31); kStage: the solution is kept in shared memory
 // after the first pass (otherwise the second pass reads it again through L1/L2), as PosT (uint16 when
 // D < 65536).
-template <bool kPlain, int CP, typename MemT, bool kStage, typename PosT>
-__global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const IntervalParams p) {
+// kTeams: p.team may ask for a block per solution (without, a warp has each: eight registers less, which small graphs need to
+// fill an SM: n = 60, 16384 solutions 37.0 us, 39.5 with).
+template <bool kPlain, int CP, typename MemT, bool kStage, typename PosT, bool kTeams>
+__global__ void __launch_bounds__(32 * (kTeams ? kIvMaxTeam : kIvMaxWarps)) check_intervals_kernel(const IntervalParams p) {
     extern __shared__ __align__(16) char smem[];
+    // what the warps of a solution tell one another (p.team)
+    __shared__ int64_t s_dur[kIvMaxTeam], s_sum[kIvMaxTeam], s_top[kIvMaxTeam];
+    __shared__ int32_t s_act[kIvMaxTeam], s_distinct[kIvMaxTeam], s_bits[kIvMaxTeam], s_marks[kIvMaxTeam], s_mask[kIvMaxTeam];
     const int lane = threadIdx.x & 31;
     const int warp = __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0);
     const int wpb = blockDim.x >> 5;
+    // a solution has this warp or, with p.team, the block
+    const bool team = kTeams && p.team != 0;
+    const int tid = team ? (int)threadIdx.x : lane, tn = team ? (int)blockDim.x : 32;
+    auto sync = [&]() {
+        if (team) __syncthreads();
+        else __syncwarp();
+    };
+    // sum of the warps' values, which have been written to `part` in front of the last barrier
+    auto warps_sum = [&](const int32_t* part) -> int32_t { return (int32_t)__reduce_add_sync(0xFFFFFFFFu, lane < wpb ? (uint32_t)part[lane] : 0u); };
     const int32_t n = p.n, C = p.C, K = n * C;
-    char* ws = smem + (size_t)warp * p.warp_bytes;
+    char* ws = smem + (team ? (size_t)0 : (size_t)warp * p.warp_bytes);
     uint32_t* bm_act = reinterpret_cast<uint32_t*>(ws);
     uint32_t* bm_all = bm_act + p.words;                               // plain model only
     uint16_t* rbase = reinterpret_cast<uint16_t*>(bm_act + p.words * (kPlain ? 2u : 1u));
@@ -100,15 +118,15 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
     constexpr uint32_t kFull = 0xFFFFFFFFu;
     const int nz = (int)(interval_clear_bytes(p.words, K, kPlain, sizeof(MemT)) >> 4);
 
-    for (int32_t b = blockIdx.x * wpb + warp; b < p.B; b += gridDim.x * wpb) {
+    for (int32_t b = team ? blockIdx.x : blockIdx.x * wpb + warp; b < p.B; b += team ? gridDim.x : gridDim.x * wpb) {
         const int32_t* __restrict__ gs = p.s + (int64_t)b * K;
         const int32_t* __restrict__ ge = p.e + (int64_t)b * K;
         const int32_t* __restrict__ ga = p.a + (int64_t)b * K;
         {
             int4* z4 = reinterpret_cast<int4*>(ws);
-            for (int i = lane; i < nz; i += 32) z4[i] = make_int4(0, 0, 0, 0);
+            for (int i = tid; i < nz; i += tn) z4[i] = make_int4(0, 0, 0, 0);
         }
-        __syncwarp();
+        sync();
         // C = 2 and the three rows of this solution start on 8 bytes: slots are read in pairs
         const bool pairs = C == 2 && ((reinterpret_cast<uintptr_t>(gs) | reinterpret_cast<uintptr_t>(ge) | reinterpret_cast<uintptr_t>(ga)) & 7) == 0;
 
@@ -117,7 +135,7 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
         // Eq. 8 holds everywhere.
         int32_t mask = 0, n_act = 0, n_distinct = 0;
         int64_t dur = 0;
-        for (int32_t v = lane; v < n; v += 32) {
+        for (int32_t v = tid; v < n; v += tn) {
             int32_t sv[CP], ev[CP], av[CP];
             if (CP == 2 && pairs) {                         // two slots per node: one 8-byte load per array
                 const int2 s2 = __ldg(reinterpret_cast<const int2*>(gs) + v), e2 = __ldg(reinterpret_cast<const int2*>(ge) + v),
@@ -183,8 +201,13 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
                 }
             }
         }
-        if (__any_sync(kFull, mask & kIvEq8)) {     // nothing else is evaluated
-            if (lane == 0) {
+        int32_t total_act = (int32_t)__reduce_add_sync(kFull, (uint32_t)n_act), distinct = kPlain ? (int32_t)__reduce_add_sync(kFull, (uint32_t)n_distinct) : 0;
+        if (team && lane == 0) {
+            s_act[warp] = total_act;
+            s_distinct[warp] = distinct;
+        }
+        if (team ? __syncthreads_or(mask & kIvEq8) != 0 : __any_sync(kFull, mask & kIvEq8) != 0) {     // nothing else is evaluated
+            if (tid == 0) {
                 p.out_mask[b] = kIvEq8;
                 p.out_peak[b] = -1;
                 p.out_dur[b] = -1;
@@ -194,12 +217,16 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
             continue;
         }
         __syncwarp();
+        if (team) {
+            total_act = warps_sum(s_act);
+            distinct = warps_sum(s_distinct);
+        }
         if (kPlain && p.byte_marks) {
             // bytes -> bitmaps: the warp reads the byte pairs of 32 consecutive events, the two ballots are their
             // bitmap words, kept by lane (word mod 32) and stored 32 words at a time; then the bytes, which
             // borrowed the difference array, are cleared again
             const uint16_t* by2 = reinterpret_cast<const uint16_t*>(by_act);
-            for (uint32_t w0 = 0; w0 < p.words; w0 += 32) {
+            for (uint32_t w0 = team ? 32u * (uint32_t)warp : 0u; w0 < p.words; w0 += (uint32_t)tn) {
                 uint32_t keep_a = 0, keep_l = 0;
                 const uint32_t w1 = min(p.words, w0 + 32u);
                 for (uint32_t wd = w0; wd < w1; ++wd) {
@@ -216,17 +243,17 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
                     bm_all[w0 + lane] = keep_l;
                 }
             }
-            __syncwarp();
+            sync();
             int4* z4 = reinterpret_cast<int4*>(by_act);
-            for (uint32_t i = lane; i < (2u * by_stride + 15u) / 16u; i += 32) z4[i] = make_int4(0, 0, 0, 0);
-            __syncwarp();
+            for (uint32_t i = tid; i < (2u * by_stride + 15u) / 16u; i += tn) z4[i] = make_int4(0, 0, 0, 0);
+            sync();
         }
 
         // ---- rank base of every four bitmap words: exclusive prefix sum of the popcounts
         int32_t R;
         {
-            const uint32_t groups = p.words / 4, per = ((groups + 31) / 32) | 1u;      // odd: the lanes' vectors fall into different banks
-            const uint32_t g0 = min(groups, (uint32_t)lane * per), g1 = min(groups, g0 + per);
+            const uint32_t groups = p.words / 4, per = ((groups + (uint32_t)tn - 1u) / (uint32_t)tn) | 1u;      // odd: the lanes' vectors fall into different banks
+            const uint32_t g0 = min(groups, (uint32_t)tid * per), g1 = min(groups, g0 + per);
             const uint4* v4 = reinterpret_cast<const uint4*>(bm_act);
             uint32_t cnt = 0;
             for (uint32_t i = g0; i < g1; ++i) {
@@ -239,24 +266,27 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
                 if (lane >= d) incl += o;
             }
             uint32_t run = incl - cnt;
+            R = (int32_t)__shfl_sync(kFull, incl, 31);       // number of distinct active starts
+            if (team) {
+                if (lane == 0) s_marks[warp] = R;
+                __syncthreads();
+                run += __reduce_add_sync(kFull, lane < warp ? (uint32_t)s_marks[lane] : 0u);
+                R = warps_sum(s_marks);
+            }
             for (uint32_t i = g0; i < g1; ++i) {
                 rbase[i] = (uint16_t)run;
                 const uint4 v = v4[i];
                 run += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
             }
-            R = (int32_t)__shfl_sync(kFull, incl, 31);       // number of distinct active starts
         }
-        int32_t total_act = n_act;
-        for (int d = 16; d > 0; d >>= 1) total_act += __shfl_xor_sync(kFull, total_act, d);
+        int32_t bits = 0;
         if (kPlain) {
-            int32_t bits = 0;
-            for (uint32_t i = lane; i < p.words; i += 32) bits += __popc(bm_all[i]);
+            for (uint32_t i = tid; i < p.words; i += tn) bits += __popc(bm_all[i]);
             bits = __reduce_add_sync(kFull, bits);
-            if (bits != __reduce_add_sync(kFull, n_distinct)) mask |= kIvEq6;
         }
         const bool has_seq = R == total_act;
         int32_t* row = (p.out_seqs != nullptr && has_seq) ? p.out_seqs + (int64_t)b * K : nullptr;
-        __syncwarp();
+        sync();
         auto rank = [&](int32_t t) -> int32_t {   // marked events <= t
             const uint4 v = reinterpret_cast<const uint4*>(bm_act)[t >> 7];
             const int32_t w = t >> 5 & 3;
@@ -281,7 +311,7 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
 
         // ---- pass 2, per node u: Eq. 4 (its active intervals with s <= e cover the marked events
         // rank(s)..rank(e)), the sequence, and Eq. 5 for its successors
-        for (int32_t u = lane; u < n; u += 32) {
+        for (int32_t u = tid; u < n; u += tn) {
             int32_t us[CP], ue[CP];
             const MemT mv = (MemT)__ldg(&p.m[u]);
             if (kPairStage && C == 2) {
@@ -339,13 +369,13 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
                 }
             }
         }
-        __syncwarp();
+        sync();
 
-        // ---- prefix sum over the ranks 1..R and its maximum: lane owns a run of consecutive ranks
-        int64_t peak;
+        // ---- prefix sum over the ranks 1..R and its maximum: a thread owns a run of consecutive ranks
+        int64_t peak, carry;
         {
-            const int32_t per = (R + 31) / 32;
-            const int32_t r0 = min(R, lane * per) + 1, r1 = min(R, lane * per + per) + 1;   // ranks [r0, r1)
+            const int32_t per = (R + tn - 1) / tn;
+            const int32_t r0 = min(R, tid * per) + 1, r1 = min(R, tid * per + per) + 1;   // ranks [r0, r1)
             int64_t sum = 0, top = INT64_MIN;
             for (int32_t r = r0; r < r1; ++r) {
                 sum += (int64_t)delta[r];
@@ -356,18 +386,47 @@ __global__ void __launch_bounds__(32 * kIvMaxWarps) check_intervals_kernel(const
                 const int64_t o = __shfl_up_sync(kFull, incl, d);
                 if (lane >= d) incl += o;
             }
-            peak = r1 > r0 ? incl - sum + top : 0;
+            // largest usage in the warp's runs, from the usage in front of the warp on
+            peak = r1 > r0 ? incl - sum + top : (team ? INT64_MIN : 0);
             for (int d = 16; d > 0; d >>= 1) {
                 const int64_t o = __shfl_xor_sync(kFull, peak, d);
                 peak = o > peak ? o : peak;
             }
+            carry = __shfl_sync(kFull, incl, 31);
         }
-        if (peak > p.M) mask |= kIvEq4;
-
         // ---- duration, flags, outputs
         for (int d = 16; d > 0; d >>= 1) dur += __shfl_xor_sync(kFull, dur, d);
         mask = __reduce_or_sync(kFull, mask);
-        if (lane == 0) {
+        if (team) {
+            if (lane == 0) {
+                s_sum[warp] = carry;
+                s_top[warp] = peak;
+                s_dur[warp] = dur;
+                s_mask[warp] = mask;
+                s_bits[warp] = bits;
+            }
+            __syncthreads();
+            if (warp != 0) continue;
+            const bool in = lane < wpb;
+            const int64_t part = in ? s_sum[lane] : 0, most = in ? s_top[lane] : INT64_MIN;
+            int64_t incl = part;
+            for (int d = 1; d < 32; d <<= 1) {
+                const int64_t o = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += o;
+            }
+            peak = most == INT64_MIN ? 0 : incl - part + most;         // usages are 0 or more
+            dur = in ? s_dur[lane] : 0;
+            for (int d = 16; d > 0; d >>= 1) {
+                const int64_t o = __shfl_xor_sync(kFull, peak, d);
+                peak = o > peak ? o : peak;
+                dur += __shfl_xor_sync(kFull, dur, d);
+            }
+            mask = __reduce_or_sync(kFull, in ? s_mask[lane] : 0);
+            bits = warps_sum(s_bits);
+        }
+        if (kPlain && bits != distinct) mask |= kIvEq6;
+        if (peak > p.M) mask |= kIvEq4;
+        if (tid == 0) {
             p.out_mask[b] = mask;
             p.out_peak[b] = peak;
             p.out_dur[b] = dur;

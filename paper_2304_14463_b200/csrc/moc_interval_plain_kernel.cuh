@@ -14,9 +14,11 @@
 // An inactive slot's start is replaced by that of the other slot (it then asks for nothing new); a solution in which
 // some node has no active slot at all takes a plain loop over the edges instead.
 //
-// Bound: instruction issue (58 % of the slots, 3330 instructions per solution against 6310) and the shared-memory
-// data pipe (52 %).  n = 442, D = 884, 16384 solutions with their sequences: 179.8 -> 90.5 us, where the 207 MB of
-// DRAM traffic alone take 32.  Fetching the next solution into L2 ahead of time cost 5 us and 60 MB of traffic.
+// Bound: instruction issue (58 % of the slots), the shared-memory data pipe (52 %) and the latency of the solution's loads.
+// n = 442, D = 884, 16384 solutions with their sequences: 179.8 -> 90.5 us, where the 207 MB of DRAM traffic alone
+// take 32; 91.9 -> 88.5 with both slots of a node in one packed word (36 operations for 55 in a half of a tile) and the walk over the
+// events ended at the last active start.  Taken back: the next solution fetched into L2 (+5 us and 60 MB of traffic), two nodes'
+// loads ahead instead of four at a time (+3.5), one mark for active and inactive starts (+2.7, with a third fewer stores).
 #pragma once
 #include "moc_interval_kernels.cuh"
 #include "moc_pair_kernel.cuh"
@@ -43,6 +45,13 @@ __host__ __device__ inline size_t interval_plain_event_bytes(int32_t D, size_t m
     return 32 * 16 * ((((vec > marks ? vec : marks) + 31) / 32) | 1);
 }
 
+// 0xFFFF in each half whose bit 15 is set, else 0 (prmt's sign mode, which __byte_perm masks out)
+__device__ __forceinline__ uint32_t iv_half_signs(uint32_t x) {
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %1, 0xBB99;" : "=r"(r) : "r"(x));
+    return r;
+}
+
 template <typename MemT>
 __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const IntervalPlainParams pp) {
     extern __shared__ __align__(16) char smem[];
@@ -51,14 +60,17 @@ __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const I
     constexpr int kShift = sizeof(MemT) == 4 ? 2 : 3;
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
     {
-        int4* s4 = reinterpret_cast<int4*>(smem);
-        const uint32_t n_rec = pp.rec_bytes >> 4, n_all = (pp.rec_bytes + pp.sell_bytes) >> 4;
-        for (uint32_t i = threadIdx.x; i < n_all; i += blockDim.x)
-            s4[i] = i < n_rec ? __ldg(reinterpret_cast<const int4*>(pp.rec) + i) : __ldg(reinterpret_cast<const int4*>(pp.sell) + (i - n_rec));
+        // asynchronous copies: the graph is first read in pass 2
+        auto copy = [&](uint32_t to, const void* from, uint32_t bytes) {
+            for (uint32_t i = 16u * threadIdx.x; i < bytes; i += 16u * blockDim.x)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + i), "l"(reinterpret_cast<const char*>(from) + i) : "memory");
+        };
+        copy(sbase, pp.rec, pp.rec_bytes);
+        copy(sbase + pp.rec_bytes, pp.sell, pp.sell_bytes);
     }
     const int32_t n = p.n, K = 2 * n, D = p.D;
-    const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
     const uint32_t word_set = pp.word_bytes + kPairWordTail;
     const uint32_t sa = sbase + pp.rec_bytes + pp.sell_bytes + (uint32_t)warp * (2u * word_set + pp.event_bytes);   // start words
     const uint32_t ea = sa + word_set;                               // end words: e | active << 15 per slot
@@ -69,6 +81,7 @@ __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const I
         sts_u32(sa + pp.word_bytes, 0u);          // empty node slots: inactive
         sts_u32(ea + pp.word_bytes, 0u);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     auto clear_events = [&]() {
         for (uint32_t o = 16u * (uint32_t)lane; o < pp.event_bytes; o += 512u)
@@ -163,6 +176,7 @@ __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const I
                 const uint32_t owner = owner_of(t), here = __ballot_sync(kFull, owner != 0);
                 if (pass == 1 && owner != 0) row[at + __popc(here & ((1u << lane) - 1u))] = (int32_t)owner - 1;
                 at += __popc(here);
+                if (at == total) break;          // there are no more active starts than that
             }
             R = at;
         }
@@ -194,19 +208,24 @@ __global__ void __launch_bounds__(kIvPlainThreads, 1) check_plain_kernel(const I
                 if (h == 0) rows_x = x;
                 const uint32_t off = x & 0xFFFFu, sp = lds_u32(sa + off), ep = lds_u32(ea + off);
                 const bool sink = (h == 0 ? e_first & 0xFFFFu : e_first >> 16) == off;       // no successor: everything is served
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const uint32_t s = i == 0 ? sp & 0xFFFFu : sp >> 16, e = (i == 0 ? ep : ep >> 16) & 0x7FFFu;
-                    const bool act = (ep & (i == 0 ? 0x8000u : 0x80000000u)) != 0;
-                    if (act && s <= e) {
-                        red_add_amount(da + (s << kShift), m);
-                        red_sub_amount(da + ((e + 1u) << kShift), m);
-                    }
-                    const bool serves = act && e > s;
-                    const uint32_t lo = serves ? s + 1u : 0xFFFFu, ln = serves ? e - s - 1u : 0u;
-                    nlo[i][h] = sink ? 0u : ((0u - lo) & 0xFFFFu) * 0x10001u;
-                    len[i][h] = sink ? 0xFFFFFFFFu : ln * 0x10001u;
+                // both slots at once, 16 bits each: 2^15 + e - s (bit 15: e >= s), and with 1 taken off (bit 15: e > s); bit 15 of
+                // ep tells that the slot is active
+                const uint32_t d = (ep | 0x80008000u) - sp, gap = d - 0x00010001u, held = d & ep;
+                const uint32_t serves = iv_half_signs(gap & ep);       // 0xFFFF where the slot is active and e > s
+                if (held & 0x8000u) {
+                    red_add_amount(da + ((sp & 0xFFFFu) << kShift), m);
+                    red_sub_amount(da + (((ep & 0x7FFFu) + 1u) << kShift), m);
                 }
+                if (held & 0x80000000u) {
+                    red_add_amount(da + ((sp >> 16) << kShift), m);
+                    red_sub_amount(da + (((ep >> 16 & 0x7FFFu) + 1u) << kShift), m);
+                }
+                // lo = s + 1 and len = e - lo where the slot serves, else 2^16 - 1 and 0
+                const uint32_t ln = sink ? 0xFFFFFFFFu : gap & 0x7FFF7FFFu & serves, nl = sink ? 0u : (serves & ~sp) | (~serves & 0x00010001u);
+                nlo[0][h] = __byte_perm(nl, 0u, 0x1010u);
+                nlo[1][h] = __byte_perm(nl, 0u, 0x3232u);
+                len[0][h] = __byte_perm(ln, 0u, 0x1010u);
+                len[1][h] = __byte_perm(ln, 0u, 0x3232u);
             }
             const int rows = __shfl_sync(kFull, (int)(rows_x >> 16), 0);
             uint32_t e = e_first;

@@ -102,15 +102,23 @@ int check_intervals(const moc_graph* g, const int32_t* s, const int32_t* e, cons
         const int fit = blk <= cap + 1024 ? (int)((g->smem_optin) / blk) * k : 0;
         if (fit > best) { best = fit; wpb = k; }
     }
+    // Several warps on a solution where an SM would have few at work (bitmaps of a large domain, or a small batch), as many as leave it some
+    // 48 and each 16 nodes.  Staged, 1 / 2 / 4 / 8 / 16 warps (us): n = 111, B = 500 14.8 / 12.3 / 10.6 / 11.0 / 14.7; n = 300, B = 6000 80 / 62 / 68 / 85 / 107;
+    // n = 442, B = 1500 77 / 47 / 33 / 33 / 38, B = 148 40 / 24 / 17 / 13 / 11; n = 932, B = 1500 433 / 231 / 136 / 89 / 68.
+    const int64_t per_sm = ((int64_t)B + g->sm_count - 1) / g->sm_count, at_work = std::max<int64_t>(1, std::min<int64_t>(best, per_sm));
+    int team = 1;
+    while (team < moc::kIvMaxTeam && 2 * team * at_work <= 48 && 32 * team <= n) team *= 2;
+    p.team = team > 1 ? 1 : 0;
+    if (team > 1) wpb = team;
     if (fill && out_seqs) MOC_CUDA(cudaMemsetAsync(out_seqs, 0xFF, (size_t)B * (size_t)K * 4, (cudaStream_t)stream));
-    const size_t smem = warp_b * wpb;
+    const size_t smem = team > 1 ? warp_b : warp_b * wpb;
     const int cp = g->C <= 2 ? 2 : (g->C <= 4 ? 4 : 8), kept = !stage ? 0 : (D < 65536 ? 2 : 4);      // bytes per kept event
-    const IntervalFn fn = plain ? check_general_fn(cp, wide, kept) : check_staged_fn(cp, wide, kept);
+    const IntervalFn fn = plain ? check_general_fn(cp, wide, kept, team > 1) : check_staged_fn(cp, wide, kept, team > 1);
     MOC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
     int nb = 0;
     MOC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, 32 * wpb, smem));
     if (nb < 1) return fail(MOC_ERR_CUDA, "moc_check_intervals: kernel does not fit on an SM");
-    const int grid = (int)std::min<int64_t>((int64_t)g->sm_count * nb, ((int64_t)B + wpb - 1) / wpb);
+    const int grid = (int)std::min<int64_t>((int64_t)g->sm_count * nb, team > 1 ? (int64_t)B : ((int64_t)B + wpb - 1) / wpb);
     fn<<<grid, 32 * wpb, smem, (cudaStream_t)stream>>>(p);
     MOC_CUDA(cudaGetLastError());
     launch_counter() = 1;
