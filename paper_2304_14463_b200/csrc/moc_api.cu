@@ -1577,6 +1577,14 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         rc = copy_part(k);
         if (rc != MOC_OK) return rc;
     }
+    int launches = 0;
+    if (m_lens) {                  // under way while the rest is prepared
+        const int blocks = (int)std::min<int64_t>((std::max<int64_t>(need / 4, B) + 255) / 256, (int64_t)g->sm_count * 2);
+        if (wide_ids) moc::fetch_kernel<int32_t><<<blocks, 256, 0, st>>>((const int32_t*)m_ids, need, g->d_stage_seqs, m_lens, B, d_lens);
+        else moc::fetch_kernel<uint16_t><<<blocks, 256, 0, st>>>((const uint16_t*)m_ids, need, g->d_stage_seqs, m_lens, B, d_lens);
+        MOC_CUDA(cudaGetLastError());
+        ++launches;
+    }
     // sequences that are complete with each part
     int32_t cb[kHostParts + 1] = {0};
     int64_t co[kHostParts + 1] = {0};
@@ -1608,14 +1616,6 @@ int eval_host(const moc_graph* g, const void* ids, bool wide_ids, int64_t n_step
         g->h_stage_cap = 0;
         MOC_CUDA(cudaMallocHost((void**)&g->h_stage, res_bytes * 2));
         g->h_stage_cap = res_bytes * 2;
-    }
-    int launches = 0;
-    if (m_lens) {
-        const int blocks = (int)std::min<int64_t>((std::max<int64_t>(need / 4, B) + 255) / 256, (int64_t)g->sm_count * 2);
-        if (wide_ids) moc::fetch_kernel<int32_t><<<blocks, 256, 0, st>>>((const int32_t*)m_ids, need, g->d_stage_seqs, m_lens, B, d_lens);
-        else moc::fetch_kernel<uint16_t><<<blocks, 256, 0, st>>>((const uint16_t*)m_ids, need, g->d_stage_seqs, m_lens, B, d_lens);
-        MOC_CUDA(cudaGetLastError());
-        ++launches;
     }
     for (int k = 0; k < n_parts; ++k) {
         if (parts) MOC_CUDA(cudaStreamWaitEvent(st, g->chunk_ev[k], 0));

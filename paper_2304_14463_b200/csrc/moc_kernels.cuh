@@ -448,12 +448,16 @@ template <typename Id>
 static __global__ void __launch_bounds__(256) fetch_kernel(const Id* __restrict__ ids, int64_t count, int32_t* __restrict__ dst,
                                                     const int32_t* __restrict__ lens, int32_t B, int32_t* __restrict__ dst_lens) {
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = tid; i < B; i += stride) dst_lens[i] = __ldg(lens + i);
     constexpr int kPer = 16 / (int)sizeof(Id);
     const bool aligned = (reinterpret_cast<uintptr_t>(ids) & 15) == 0;
     const int64_t nv = aligned ? count / kPer : 0;
+    // a thread's first length and first vector cross the link together: one after the other they are two of its latencies
+    const int32_t len0 = tid < B ? __ldg(lens + tid) : 0;
+    const uint4 v0 = tid < nv ? __ldg(reinterpret_cast<const uint4*>(ids) + tid) : make_uint4(0, 0, 0, 0);
+    if (tid < B) dst_lens[tid] = len0;
+    for (int64_t i = tid + stride; i < B; i += stride) dst_lens[i] = __ldg(lens + i);
     for (int64_t i = tid; i < nv; i += stride) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(ids) + i);
+        const uint4 v = i == tid ? v0 : __ldg(reinterpret_cast<const uint4*>(ids) + i);
         if constexpr (sizeof(Id) == 4) {
             reinterpret_cast<uint4*>(dst)[i] = v;
         } else {
