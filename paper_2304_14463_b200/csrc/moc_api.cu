@@ -1752,9 +1752,9 @@ int moc_mem_profile(const moc_graph* g, const int32_t* seq, int32_t len, int64_t
         q.out_status = out_status;
         q.out_profile = out_profile;
         q.out_free = out_free;
-        // threads from measurements at n = 20, 100, 442, 1000, 2000 and 5000 (us per call with 128 / 512 / 1024 threads:
-        // 6.1 / 6.2 / 10.6, 6.1 / 6.9 / 8.6, 8.2 / 7.4 / 8.2, 12.3 / 8.3 / 8.2, 17.0 / 10.3 / 10.3, 32.8 / 18.0 / 16.4)
-        const int thr = g->n < 200 ? 128 : (g->n < 1500 ? 512 : 1024);
+        // threads (us per call with 128 / 256 / 512 / 1024; calls of 5.6 are the host's time): n = 60 5.6 / 5.6 / 5.6 / 5.6, 442 6.7 / 5.7 / 5.7 / 6.2, 1000 10.3 / 8.2 /
+        // 6.2 / 7.2, 2600 17.5 / 12.3 / 10.9 / 12.3, 4800 27.7 / 18.5 / 16.4 / 15.9
+        const int thr = g->n < 200 ? 256 : (g->n < 3000 ? 512 : 1024);
         q.team = thr / 32;
         pl.quad_fn<<<1, thr, pl.smem, st>>>(q);
         ++g_launches;

@@ -272,7 +272,27 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             __syncwarp();
             return sum;
         };
-        if (valid) words_of(wa, T, kEditNone, kEditNone, 0);
+        if (valid) {
+            // the words of the chain's sequence, eight elements of the row in flight per lane
+            for (uint32_t o = 16u * (uint32_t)lane; o < p.word_bytes; o += 512u)
+                asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(wa + o), "r"(0) : "memory");
+            __syncwarp();
+            for (int32_t t0 = lane; t0 < T; t0 += 256) {
+                int32_t v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = t0 + 32 * k < T ? row[t0 + 32 * k] : n;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    if (t0 + 32 * k >= T) break;
+                    const uint32_t addr = wa + 4u * min((uint32_t)v[k], (uint32_t)n);
+                    const uint32_t old = exch_shared(addr, (uint32_t)(t0 + 32 * k + 1) * 0x10001u);
+                    sts_u16_if_nonzero(old, addr + 2, old);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) sts_u32(wa + 4u * (uint32_t)(n + 1), (uint32_t)T * 0x10001u);
+            __syncwarp();
+        }
         // out with step qd_s, in at index ji_s: the words of the edited sequence at w1, from the parent's at w0
         auto shift_words = [&](uint32_t w0, uint32_t w1, int32_t Tc_s, int32_t qd_s, int32_t ji_s, int32_t x_s, uint32_t wx_s) {
             const uint32_t kq = qd_s == kEditNone ? 0x7FFFu : (uint32_t)qd_s + 1u, kj = ji_s == kEditNone ? 0x7FFFu : (uint32_t)ji_s;
