@@ -348,12 +348,13 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
         int best_wpb = 0, best_warps = 0, best_nb = 0;
         cudaError_t e = raise_smem_limit((const void*)fn, g->smem_optin);
         if (e != cudaSuccess) return fail(MOC_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-        for (int wpb = 16; wpb >= 4; --wpb) {    // every kernel variant is compiled for up to 512 threads, two blocks per SM
+        for (int wpb = moc::pair_max_warps(pre, false); wpb >= 4; --wpb) {    // every variant is compiled for two blocks of so many on an SM
             if (g->want_gpc && wpb != std::min(g->want_gpc, 16)) continue;
             const size_t sm = graph_b + wpb * warp_b;
             if (sm > smem_cap) continue;
             int nb = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, wpb * 32, sm) != cudaSuccess) { cudaGetLastError(); continue; }
+            nb = std::min(nb, 2);          // more and smaller blocks only stage the graph more often
             pl.pair_nb[wpb] = nb;
             if (nb * wpb > best_warps) { best_warps = nb * wpb; best_wpb = wpb; best_nb = nb; }
         }
@@ -930,7 +931,7 @@ int enqueue_eval(const moc_graph* g, const Plan& pl, int64_t* offs, bool fill_of
         // half-empty SM.  Pick the warps per block and blocks per SM with the least rounds x warps.
         int64_t best_cost = INT64_MAX;
         int best_w = pl.gpc, best_nb = std::max(1, pl.grid / std::max(1, pl.sm_count));
-        for (int wpb = 4; wpb <= 16; ++wpb) {
+        for (int wpb = 4; wpb <= 19; ++wpb) {
             const int nb = pl.pair_nb[wpb];
             if (nb < 1) continue;
             const int64_t blocks = (int64_t)pl.sm_count * nb;

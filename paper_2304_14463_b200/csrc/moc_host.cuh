@@ -54,8 +54,8 @@ struct Plan {
     bool pair_team = false;        // several warps per sequence (team_shape)
     PairFn pair_fn = nullptr;
     uint32_t rec_bytes = 0, w_bytes = 0, sell_bytes = 0, word_bytes = 0;   // delta_bytes: above
-    // blocks per SM the fast path reaches with 1..16 warps per block (0: does not fit), and its sizes
-    int pair_nb[17] = {0};
+    // blocks per SM the fast path reaches with 1..19 warps per block (0: does not fit), and its sizes
+    int pair_nb[20] = {0};
     size_t pair_graph_b = 0, pair_warp_b = 0;
     int sm_count = 0;
     // block-per-sequence path with packed words for C <= 4

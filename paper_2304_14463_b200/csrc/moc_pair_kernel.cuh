@@ -190,6 +190,9 @@ __device__ __forceinline__ void team_sync(int id, int threads) {
     else __syncwarp();
 }
 
+// Warps per block, at most.
+__host__ __device__ constexpr int pair_max_warps(int pre, bool team) { return pre == 0 && !team ? 19 : 16; }
+
 // Bound, large batches: the shared-memory data pipe (three quarters of one wavefront per clock, about 520 wavefronts per
 // sequence) and instruction issue (1700 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 41.0 -> 39.7 us (four
 // exchanges in flight before their results are looked at, ragged ends of a row through the same code, no second search for
@@ -199,15 +202,16 @@ __device__ __forceinline__ void team_sync(int id, int threads) {
 //
 // kPre: how many 16-byte vectors of the next row each lane fetches ahead (rows of about 128*kPre
 // steps; 0 for short rows, where the extra registers cost more than the wait).  Blocks have up to 16
-// warps and two of them share an SM (62 registers per thread, no spills).
+// warps and two of them share an SM (62 registers per thread, no spills); without fetched rows 48 registers do, and 19
+// warps (n = 250, B = 25000 44.5 -> 42.2 us; n = 442 without fetching, 38 warps on an SM 41.2, 28 with it 40.7).
 //
 // kTeam: p.team warps share a sequence, for batches that leave most of an SM's warps without one: the latency of a
 // sequence is then what counts, and the row, the tiles and the scan are dealt to the warps.
 template <typename MemT, int kPre, bool kTeam>
-__global__ void __launch_bounds__(512, 2) eval_pair_kernel(const PairParams p) {
+__global__ void __launch_bounds__(32 * pair_max_warps(kPre, kTeam), 2) eval_pair_kernel(const PairParams p) {
     static_assert(!kTeam || kPre == 0, "a team has one sequence at a time and fetches nothing ahead");
     extern __shared__ __align__(16) char smem[];
-    __shared__ int64_t s_part[16];
+    __shared__ int64_t s_part[19];
     __shared__ uint64_t s_acc[16];               // kTeam: what the warps of a sequence tell one another
     __shared__ uint32_t s_flag[16], s_lo[16], s_hi[16];
     __shared__ int64_t s_top[16];
