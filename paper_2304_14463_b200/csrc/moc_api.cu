@@ -354,7 +354,7 @@ int make_plan(const moc_graph* g, bool profile, Plan* out) {
             if (sm > smem_cap) continue;
             int nb = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, (const void*)fn, wpb * 32, sm) != cudaSuccess) { cudaGetLastError(); continue; }
-            nb = std::min(nb, 2);          // more and smaller blocks only stage the graph more often
+            if (pre == 0) nb = std::min(nb, 2);          // more and smaller blocks only stage the graph more often
             pl.pair_nb[wpb] = nb;
             if (nb * wpb > best_warps) { best_warps = nb * wpb; best_wpb = wpb; best_nb = nb; }
         }
