@@ -430,13 +430,14 @@ int moc_graph_set_launch(moc_graph* g, int32_t threads_per_sequence, int32_t seq
  *   MOC_KERNEL_AUTO   a = b = 0.
  *   MOC_KERNEL_GROUP  a group of a threads (0, 32 .. 1024) per sequence, b sequences per block
  *                     (0 = choose); any C <= MOC_MAX_COPIES.  Same as moc_graph_set_launch(a, b).
- *   MOC_KERNEL_WARP   one warp per sequence, b warps per block (0 or 4..16), a = 0; C <= 2.
+ *   MOC_KERNEL_WARP   one warp per sequence, b warps per block (4..16, or 0 = choose, which lets several warps
+ *                     share a sequence in small batches), a = 0; C <= 2.
  *   MOC_KERNEL_LANE   one sequence per lane: a block keeps a group of a sequences (0, 8, 16, 32)
  *                     on chip and its b warps (0, 8, 16, 24 or 32; a multiple of a) share the work on them;
  *                     C <= 2 and a graph whose state for a group fits in shared memory.
- *   MOC_KERNEL_BLOCK  one block of a threads (0, or a multiple of 32 in 64..1024) per sequence with
- *                     the copies of a node packed into one 64-bit word, b = 0; C <= 4 and sequences
- *                     of at most 32766 steps whose state fits in shared memory.
+ *   MOC_KERNEL_BLOCK  one block of a threads (a multiple of 32 in 64..1024; 0 = choose between a block, a
+ *                     team of warps and a warp) per sequence with the copies of a node packed into one
+ *                     word, b = 0; C <= 4 and sequences of at most 32766 steps whose state fits in shared memory.
  * MOC_ERR_ARG for an unknown kind or shape; a kind that cannot serve the graph with its current C
  * is reported by the next moc_eval_batch (MOC_ERR_ARG), which evaluates nothing.
  */

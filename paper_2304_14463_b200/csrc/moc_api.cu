@@ -901,6 +901,8 @@ int enqueue_live(const moc_graph* g, const Plan& pl, const int64_t* offs, const 
     const int64_t groups = ((int64_t)B + 31) / 32, per_sm = (groups + g->sm_count - 1) / g->sm_count, rounds = (per_sm + 15) / 16;
     const int wpb = (int)std::max<int64_t>((per_sm + rounds - 1) / rounds, 1);
     const int grid = (int)std::min<int64_t>(g->sm_count, (groups + wpb - 1) / wpb);
+    q.per_block = (int32_t)(groups / grid);
+    q.spare = (int32_t)(groups % grid);
     if (g->ev_before) MOC_CUDA(cudaEventRecord(g->ev_before, st));
     pl.live_fn<<<grid, 32 * wpb, moc::live_smem_bytes(g->n, live_words(g->n)), st>>>(q);
     ++g_launches;

@@ -95,7 +95,8 @@ __device__ __forceinline__ uint64_t warp_sum_u59(uint64_t v) {
     const uint32_t lo = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)v & 0x7FFFFFFu), hi = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(v >> 27));
     return ((uint64_t)hi << 27) + lo;
 }
-// This thread's part (of `nthr` threads) of the sum of max(lens[i], 0) over i < b.
+// This thread's part (of `nthr` threads) of the sum of max(lens[i], 0) over i < b, with kFlight 16-byte loads in flight.
+template <int kFlight = 4>
 __device__ __forceinline__ uint64_t lengths_before(const int32_t* lens, int b, int tid, int nthr) {
     uint64_t sum = 0;
     auto add = [&](int32_t v) { asm("mad.wide.u32 %0, %1, 1, %0;" : "+l"(sum) : "r"((uint32_t)max(v, 0))); };
@@ -104,12 +105,12 @@ __device__ __forceinline__ uint64_t lengths_before(const int32_t* lens, int b, i
         const int4* l4 = reinterpret_cast<const int4*>(lens);
         const int q = b >> 2;
         int k = tid;
-        for (; k + 3 * nthr < q; k += 4 * nthr) {       // four loads in flight
-            const int4 x0 = __ldg(l4 + k), x1 = __ldg(l4 + k + nthr), x2 = __ldg(l4 + k + 2 * nthr), x3 = __ldg(l4 + k + 3 * nthr);
-            add(x0.x); add(x0.y); add(x0.z); add(x0.w);
-            add(x1.x); add(x1.y); add(x1.z); add(x1.w);
-            add(x2.x); add(x2.y); add(x2.z); add(x2.w);
-            add(x3.x); add(x3.y); add(x3.z); add(x3.w);
+        for (; k + (kFlight - 1) * nthr < q; k += kFlight * nthr) {
+            int4 x[kFlight];
+#pragma unroll
+            for (int j = 0; j < kFlight; ++j) x[j] = __ldg(l4 + k + j * nthr);
+#pragma unroll
+            for (int j = 0; j < kFlight; ++j) { add(x[j].x); add(x[j].y); add(x[j].z); add(x[j].w); }
         }
         for (; k < q; k += nthr) {
             const int4 x = __ldg(l4 + k);

@@ -26,6 +26,8 @@
 // over the set bits of each word instead: 69 us at the size below, 1200 cycles per step.)
 //
 // n = 100, B = 65536, C = 2: 38.9 us (one launch) against 84 us for the warp-per-sequence kernel behind the offsets kernel.
+// The range of a block from the host and sums by warp reductions instead of 64-bit divisions, shuffles and loops over the warps:
+// 36.7 -> 36.1 us, n = 34, B = 65536 15.8 -> 14.9, n = 46, B = 32100 16.1 -> 14.6.  Eight steps at a time instead of four: 38.5.
 // Bound: the integer pipe, about 87 warp instructions per step of 32 sequences (issue slots 63 %, ALU pipe 54 %), a fifth of them for bits beyond one per word.
 // The warp-per-sequence kernel pays a warp's fixed costs (clearing, scans, reductions) per sequence, which a
 // sequence of 120 steps does not repay; at n > 128 the masks outgrow the registers.
@@ -46,6 +48,7 @@ constexpr int kLivePlanes = 4;     // C <= 4
 struct LiveParams {
     int32_t n, C;
     int32_t B;
+    int32_t per_block, spare;      // block c takes per_block groups of 32 sequences, one more when c < spare
     int64_t M;
     const uint4* image;            // the tables as they lie in shared memory (live_image)
     uint32_t sinks[kLiveMaxN / 32];
@@ -133,33 +136,14 @@ __global__ void __launch_bounds__(kLiveThreads, 1) eval_live_kernel(const LivePa
     uint32_t ma = sbase + (uint32_t)(n + 1) * 384u + 128u + (kWide ? 8u * (lane & 15) : 4u * lane);    // row of bit 0 of word 0
     uint32_t own = (uint32_t)(n + 1) * 128u;                                                          // from a mask row to the node's own
 
-    // ---- rows: block c takes the groups [c * G / grid, (c + 1) * G / grid) of 32 consecutive sequences
-    const int64_t G = ((int64_t)p.B + 31) / 32;
-    const int g_begin = (int)(blockIdx.x * G / gridDim.x), g_end = (int)((blockIdx.x + 1) * G / gridDim.x);
+    // ---- rows: block c takes a contiguous range of the groups of 32 consecutive sequences
+    const int g_begin = (int)blockIdx.x * p.per_block + min((int)blockIdx.x, p.spare), g_end = g_begin + p.per_block + ((int)blockIdx.x < p.spare ? 1 : 0);
     int64_t base = 0;              // offset of the first row of the groups at hand
     if (p.offs == nullptr) {
-        const int c0 = 32 * g_begin;
-        int64_t sum = 0;
-        if ((reinterpret_cast<uintptr_t>(p.lens) & 15) == 0) {
-            const int4* l4 = reinterpret_cast<const int4*>(p.lens);
-            const int q = c0 >> 2;
-            auto add = [&](int4 x) { sum += (int64_t)max(x.x, 0) + max(x.y, 0) + max(x.z, 0) + max(x.w, 0); };
-            int i = tid;
-            for (; i + 7 * (int)blockDim.x < q; i += 8 * blockDim.x) {
-                int4 x[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) x[k] = __ldg(l4 + i + k * blockDim.x);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) add(x[k]);
-            }
-            for (; i < q; i += blockDim.x) add(__ldg(l4 + i));
-        } else {
-            for (int i = tid; i < c0; i += blockDim.x) sum += max(__ldg(p.lens + i), 0);
-        }
-        sum = warp_sum64(sum);
-        if (lane == 0) s_part[warp] = sum;
+        const uint64_t sum = warp_sum_u59(lengths_before<8>(p.lens, 32 * g_begin, tid, blockDim.x));
+        if (lane == 0) s_part[warp] = (int64_t)sum;
         __syncthreads();
-        for (int k = 0; k < wpb; ++k) base += s_part[k];
+        base = (int64_t)warp_sum_u59(lane < wpb ? (uint64_t)s_part[lane] : 0);
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     for (int g0 = g_begin; g0 < g_end; g0 += wpb) {
@@ -172,11 +156,9 @@ __global__ void __launch_bounds__(kLiveThreads, 1) eval_live_kernel(const LivePa
             __syncthreads();       // the last readers of s_part are done (and the tables stand)
             if (lane == 31) s_part[warp] = incl;
             __syncthreads();
-            off = base + incl - l;
-            for (int k = 0; k < wpb; ++k) {
-                if (k < warp) off += s_part[k];
-                base += s_part[k];
-            }
+            const uint64_t part = lane < wpb ? (uint64_t)s_part[lane] : 0;
+            off = base + incl - l + (int64_t)warp_sum_u59(lane < warp ? part : 0);
+            base += (int64_t)warp_sum_u59(part);
         } else {
             off = mine ? __ldg(p.offs + b) : 0;
             if (g0 == g_begin) __syncthreads();
