@@ -43,7 +43,7 @@
 // block, sums of the lengths and of the chunks by shuffles and by loops over the warps (now warp reductions), the
 // graph through L2 and three barriers were taken out.  n = 442, B = 148, C = 3 8.7 -> 6.2 us; n = 153, C = 3, B = 18944 68 -> 39 (a warp
 // per sequence; a block of 64 threads spent most of its instructions on barriers and sums); n = 24 45 -> 21; n = 442, C = 3, B = 4736 33 -> 27 (teams of two);
-// n = 2192, C = 2 (words of 32 bits), B = 1184 32.5 -> 24.9; n = 1000, C = 3, B = 4096 53.3 -> 52.4; n = 5000, B = 1024 81 -> 73; profile of n = 1000 8.2 -> 6.2.
+// n = 2192, C = 2 (words of 32 bits), B = 1184 32.5 -> 24.9; n = 1000, C = 3, B = 4096 53.3 -> 45.3 (teams of four); n = 5000, B = 1024 80 -> 71.7 (one of 32); profile of n = 1000 8.2 -> 6.2.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
