@@ -43,7 +43,8 @@
 // block, sums of the lengths and of the chunks by shuffles and by loops over the warps (now warp reductions), the
 // graph through L2 and three barriers were taken out.  n = 442, B = 148, C = 3 8.7 -> 6.2 us; n = 153, C = 3, B = 18944 68 -> 39 (a warp
 // per sequence; a block of 64 threads spent most of its instructions on barriers and sums); n = 24 45 -> 21; n = 442, C = 3, B = 4736 33 -> 27 (teams of two);
-// n = 2192, C = 2 (words of 32 bits), B = 1184 32.5 -> 24.9; n = 1000, C = 3, B = 4096 53.3 -> 45.3 (teams of four); n = 5000, B = 1024 80 -> 71.7 (one of 32); profile of n = 1000 8.2 -> 6.2.
+// n = 2192, C = 2 (words of 32 bits), B = 1184 32.5 -> 24.9; n = 1000, C = 3, B = 4096 53.3 -> 45.3 (teams of four); n = 5000, B = 1024 80 -> 71.7 (one of 32); profile of n = 1000 8.2 -> 6.2, of n = 442 6.15 -> 5.6
+// (no peak, no duration, first elements of the row requested before the state is clear).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -301,6 +302,7 @@ __device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
     int64_t off = 0;
     // the lengths of b, b + 1 .. by lane (rows found by the kernel: what lies between this sequence and the team's next)
     int32_t T_next = 0, len_raw = 0, len_c0 = 0;
+    uint32_t early[2] = {0u, 0u};        // kProfile: a thread's first elements of the row, requested before the state is clear
     auto lanes_sum = [&](int32_t raw, int lanes) -> int64_t {   // sum of max(raw, 0) over lanes < `lanes`
         const uint32_t v = (lane < lanes && raw > 0) ? (uint32_t)raw : 0u;
         const uint32_t lo = __reduce_add_sync(kFull, v & 0xFFFFu), hi = __reduce_add_sync(kFull, v >> 16);
@@ -329,6 +331,10 @@ __device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
         }
     } else {
         T_next = kProfile ? p.single_len : (b < p.B ? __ldg(p.lens + b) : 0);      // one sequence ahead
+        if constexpr (kProfile) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) early[k] = tid + k * nthr < T_next ? (uint32_t)__ldg(p.seqs + tid + k * nthr) : 0u;
+        }
         clear();
         if (!kChip || kProfile) sync();
     }
@@ -364,6 +370,11 @@ __device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
                     }
                 };
                 int t = tid;
+                if constexpr (kProfile) {
+                    if (t < T) put(early[0], t);
+                    if (t + nthr < T) put(early[1], t + nthr);
+                    t += 2 * nthr;
+                }
                 for (; t + 3 * nthr < T; t += 4 * nthr) {      // four loads in flight per thread
                     const uint32_t i0 = (uint32_t)__ldg(row + t), i1 = (uint32_t)__ldg(row + t + nthr),
                                    i2 = (uint32_t)__ldg(row + t + 2 * nthr), i3 = (uint32_t)__ldg(row + t + 3 * nthr);
@@ -535,8 +546,10 @@ __device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
                 }
                 dep = sync_or(depw & 0x8000u);
                 // per-warp sums of the durations, read behind the next barrier
-                dw = p.small_w ? (int64_t)__reduce_add_sync(kFull, (uint32_t)dur) : warp_sum64(dur);
-                if (lane == 0) s_dur[first_warp + warp] = dw;
+                if constexpr (!kProfile) {
+                    dw = p.small_w ? (int64_t)__reduce_add_sync(kFull, (uint32_t)dur) : warp_sum64(dur);
+                    if (lane == 0) s_dur[first_warp + warp] = dw;
+                }
             }
             if (b_next < b_end) clear();       // for the next sequence: nothing reads the words any more
             const int chunk = ((T + nthr - 1) / nthr) | 1;
@@ -569,12 +582,14 @@ __device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
                 }
                 lo_in -= lo;
                 hi_in -= hi;
-                MemT before;
-                if constexpr (sizeof(MemT) == 4) before = (MemT)lo_in;
-                else before = split_value(lo_in, hi_in, p.split);
-                // a thread without steps counts nothing (the first step of the warp is one of the others', or the warp's usage in front)
-                w_top = warp_max_t(tb < te ? (MemT)(before + top) : (sizeof(MemT) == 8 ? (MemT)(INT64_MIN / 4) : (MemT)INT32_MIN));
-                if (lane == 0) s_top[first_warp + warp] = (int64_t)w_top;
+                if constexpr (!kProfile) {          // (a profile is asked for neither peak nor duration)
+                    MemT before;
+                    if constexpr (sizeof(MemT) == 4) before = (MemT)lo_in;
+                    else before = split_value(lo_in, hi_in, p.split);
+                    // a thread without steps counts nothing (the first step of the warp is one of the others', or the warp's usage in front)
+                    w_top = warp_max_t(tb < te ? (MemT)(before + top) : (sizeof(MemT) == 8 ? (MemT)(INT64_MIN / 4) : (MemT)INT32_MIN));
+                    if (lane == 0) s_top[first_warp + warp] = (int64_t)w_top;
+                }
             }
             sync();
             if (kMode == kQuadWarps) {
@@ -587,21 +602,25 @@ __device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
                     }
                 }
             } else if (!malformed) {
-                if (warp == 0) out_du = p.base_dur + warp_sum64(lane < n_warps ? s_dur[first_warp + lane] : 0);
+                if (!kProfile && warp == 0) out_du = p.base_dur + warp_sum64(lane < n_warps ? s_dur[first_warp + lane] : 0);
                 out_st = -1;
                 if (!dep) {
                     if (kProfile || warp == 0) {
                         // usage in front of every warp
                         uint32_t lo_w = lane < n_warps ? s_lo[first_warp + lane] : 0u, hi_w = lane < n_warps ? s_hi[first_warp + lane] : 0u;
                         const uint32_t lo_i = warp_inclusive_sum(lo_w, lane) - lo_w, hi_i = sizeof(MemT) == 8 ? warp_inclusive_sum(hi_w, lane) - hi_w : 0u;
-                        MemT in_front;
-                        if constexpr (sizeof(MemT) == 4) in_front = (MemT)lo_i;
-                        else in_front = split_value(lo_i, hi_i, p.split);
-                        // a warp without steps holds the smallest value and stays below the others (which are usages, 0 or more)
-                        const MemT pk = warp_max_t(lane < n_warps && s_top[first_warp + lane] > (sizeof(MemT) == 8 ? INT64_MIN / 4 : (int64_t)INT32_MIN)
-                                                       ? (MemT)(in_front + (MemT)s_top[first_warp + lane]) : MemT(0));
-                        out_pk = (int64_t)pk;
-                        out_st = out_pk <= p.M ? 1 : 0;
+                        if constexpr (kProfile) {
+                            out_st = 1;
+                        } else {
+                            MemT in_front;
+                            if constexpr (sizeof(MemT) == 4) in_front = (MemT)lo_i;
+                            else in_front = split_value(lo_i, hi_i, p.split);
+                            // a warp without steps holds the smallest value and stays below the others (which are usages, 0 or more)
+                            const MemT pk = warp_max_t(lane < n_warps && s_top[first_warp + lane] > (sizeof(MemT) == 8 ? INT64_MIN / 4 : (int64_t)INT32_MIN)
+                                                           ? (MemT)(in_front + (MemT)s_top[first_warp + lane]) : MemT(0));
+                            out_pk = (int64_t)pk;
+                            out_st = out_pk <= p.M ? 1 : 0;
+                        }
                         if constexpr (kProfile) {
                             uint32_t lo = __shfl_sync(kFull, lo_i, warp) + lo_in, hi = __shfl_sync(kFull, hi_i, warp) + hi_in,
                                      ad = da + ((uint32_t)tb << kShift);
