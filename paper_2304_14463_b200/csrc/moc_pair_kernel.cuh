@@ -194,7 +194,7 @@ __device__ __forceinline__ void team_sync(int id, int threads) {
 __host__ __device__ constexpr int pair_max_warps(int pre, bool team) { return pre == 0 && !team ? 19 : 16; }
 
 // Bound, large batches: the shared-memory data pipe (three quarters of one wavefront per clock, 528 wavefronts per
-// sequence) and instruction issue (68 %, 1795 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 41.0 -> 40.5 us (four
+// sequence) and instruction issue (68 %, 1795 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 41.0 -> 39.7 to 40.95 us over five boxes (four
 // exchanges in flight before their results are looked at, ragged ends of a row through the same code, no second search for
 // the end of the row).  Bound, small batches: a chain of latencies; the division for a block's range, the sums of the
 // lengths by shuffles and loops, and the copy of the graph behind one another were half of it (n = 20, B = 1024: 6.15 -> 5.9 us,

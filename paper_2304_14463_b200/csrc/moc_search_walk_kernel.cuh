@@ -23,7 +23,7 @@
 // Bound: instruction issue (72 % of the slots with 32 proposals a generation, 2000 instructions each) and, for small populations,
 // the latency of its dependent shared-memory reads; 28 warps beat 24 and 20 with more registers each, and 30 with fewer.
 // n = 442, state copied out: 4096 chains x 20 generations 436 -> 41.9 us against two kernels per generation that
-// write every proposal out, 38.9 with the neighbours' lists on chip; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us
+// write every proposal out, 38.9 with the neighbours' lists on chip, 37.1 with the words of a sequence from eight loads in flight; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us
 // against a cached evaluation per chain that is rebuilt after every acceptance, 1010 -> 951 with the lists.
 #pragma once
 #include "moc_edit_kernels.cuh"
