@@ -151,6 +151,8 @@ __global__ void __launch_bounds__(kPrepThreads, 1) edit_prepare_kernel(const Pre
         copy(s0 + p.chip_w_b, p.wslot, w_b);
         copy(s0 + p.chip_sell_b, p.sell, (uint32_t)p.sell_len * 4u);
     }
+    // this lane's column of the successor entries: shared address, or bytes from p.sell
+    uint32_t sell0 = 4u * (uint32_t)lane + (kChip ? (uint32_t)__cvta_generic_to_shared(smem) + p.chip_sell_b : 0u);
     char* ws = smem + (kChip ? p.chip_bytes : 0u) + (size_t)warp * p.warp_bytes;
     uint32_t* word = reinterpret_cast<uint32_t*>(ws);
     const size_t arr_bytes = (((size_t)c.stride + 8) * sizeof(MemT) + 15) & ~size_t(15);
@@ -190,6 +192,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) edit_prepare_kernel(const Pre
     if (kChip) {
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
+        MOC_STAGED(sell0);
     }
     // the parent after this one is looked up while this one is evaluated (index, then length and row offset)
     int32_t b_nx = it < count ? (p.todo != nullptr ? p.todo[it] : it) : 0;
@@ -246,8 +249,8 @@ __global__ void __launch_bounds__(kPrepThreads, 1) edit_prepare_kernel(const Pre
                 uint16_t* fre16 = reinterpret_cast<uint16_t*>(arrB);
                 const char* prec = (kChip ? smem : reinterpret_cast<const char*>(p.rec)) + kRecB * lane;
                 const uint64_t* pw = (kChip ? reinterpret_cast<const uint64_t*>(smem + p.chip_w_b) : p.wslot) + lane;
-                const uint32_t* ps = (kChip ? reinterpret_cast<const uint32_t*>(smem + p.chip_sell_b) : p.sell) + lane;
-                auto ld32 = [&](const uint32_t* q) -> uint32_t { return kChip ? lds_u32_nv((uint32_t)__cvta_generic_to_shared(q)) : __ldg(q); };
+                uint32_t ps = sell0;
+                auto ld32 = [&](uint32_t at) -> uint32_t { return kChip ? lds_u32_nv(at) : __ldg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(p.sell) + at)); };
                 auto ld64 = [&](const uint64_t* q) -> uint64_t { return kChip ? lds_u64((uint32_t)__cvta_generic_to_shared(q)) : __ldg(q); };
                 uint32_t vmin = 0xFFFFFFFFu, depw = 0, capw = 0;
                 uint64_t acc = 0;
@@ -304,9 +307,9 @@ __global__ void __launch_bounds__(kPrepThreads, 1) edit_prepare_kernel(const Pre
                     }
 
                     uint32_t e_next = rows > 0 ? ld32(ps) : 0u;            // one row ahead
-                    for (int k = 0; k < rows; ++k, ps += 32) {
+                    for (int k = 0; k < rows; ++k, ps += 128u) {
                         const uint32_t e = e_next;
-                        if (k + 1 < rows) e_next = ld32(ps + 32);
+                        if (k + 1 < rows) e_next = ld32(ps + 128u);
                         const uint32_t r0 = lds_u32(wa + (e & 0xFFFFu)), r1 = lds_u32(wa + (e >> 16));
                         Ga[0] = __viaddmax_u16x2(r0, naa[0], Ga[0]);
                         Ga[1] = __viaddmax_u16x2(r1, naa[1], Ga[1]);

@@ -142,7 +142,6 @@ __global__ void __launch_bounds__(1024, 1) eval_lane_kernel(const LaneParams p) 
     uint32_t wlane = a_word + 4u * j;                                         // word of sequence j in the first node row
     uint32_t dlane = a_delta + kMemRow + (uint32_t)sizeof(MemT) * j;          // delta of sequence j at step 0
     uint32_t dlane1 = dlane - kMemRow;                                        // ... at step -1
-    MOC_KEEP(a_succ);
     MOC_KEEP(a_word);
     MOC_KEEP(wlane);
     MOC_KEEP(dlane);
@@ -196,6 +195,7 @@ __global__ void __launch_bounds__(1024, 1) eval_lane_kernel(const LaneParams p) 
         }
     }
     __syncthreads();
+    MOC_STAGED(a_succ);
     if (threadIdx.x < g) sts_u32(a_word - kSpecial + kWordRow + 4u * threadIdx.x, 0x00010001u);   // read by empty node slots
     if (self)
         for (int k = 0; k < W; ++k) base += s_red[k];

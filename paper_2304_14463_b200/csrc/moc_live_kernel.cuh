@@ -88,7 +88,7 @@ inline std::vector<uint32_t> live_image(int32_t n, int words, bool wide, const s
     return t;
 }
 
-// Table reads: free to move between the steps (the tables do not change).
+// Table reads: free to move between the steps (the tables do not change), as lds_u32_nv.
 __device__ __forceinline__ uint2 live_lds_v2(uint32_t addr) {
     uint2 v;
     asm("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
@@ -163,7 +163,10 @@ __global__ void __launch_bounds__(kLiveThreads, 1) eval_live_kernel(const LivePa
             off = mine ? __ldg(p.offs + b) : 0;
             if (g0 == g_begin) __syncthreads();
         }
-        asm volatile("" : "+r"(pa), "+r"(ra), "+r"(ma), "+r"(own) : : "memory");     // the tables are read behind the barrier
+        MOC_STAGED(pa);                        // the tables are read behind the barrier
+        MOC_STAGED(ra);
+        MOC_STAGED(ma);
+        MOC_STAGED(own);
         const int32_t T = (len >= n && (int64_t)len <= (int64_t)p.C * n) ? len : 0;
         // ---- the walk.  Vectors of four steps between 16-byte boundaries; steps outside the row count as the empty node n.
         const int32_t* row = p.seqs + off;

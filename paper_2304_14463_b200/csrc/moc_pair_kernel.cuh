@@ -142,6 +142,8 @@ __device__ __forceinline__ void red_sub_amount(uint32_t addr, Amount<int64_t> a)
     red_add_shared(addr, (int32_t)(0u - a.lo));
     red_add_shared(addr + 4u, (int32_t)(0u - a.hi));
 }
+// Free to move, for tables that do not change once they stand: its address comes from a base that went through
+// MOC_STAGED, without which nothing would keep the read behind the barrier that the table arrives with.
 __device__ __forceinline__ uint32_t lds_u32_nv(uint32_t addr) {
     uint32_t v;
     asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
@@ -181,6 +183,8 @@ __device__ __forceinline__ void sts_u16_if_nonzero(uint32_t old, uint32_t addr, 
 // being recomputed from the kernel parameters wherever it is used (the hot loops are short of
 // instruction slots, not of registers).
 #define MOC_KEEP(x) asm volatile("" : "+r"(x))
+// The same for the address of a table in shared memory, at the point from which the table may be read (behind the barrier).
+#define MOC_STAGED(x) asm volatile("" : "+r"(x) : : "memory")
 
 
 // Barrier of the warps that share a sequence.
@@ -251,7 +255,6 @@ __global__ void __launch_bounds__(32 * pair_max_warps(kPre, kTeam), 2) eval_pair
     MOC_KEEP(da1);
     MOC_KEEP(rec0);
     MOC_KEEP(w0);
-    MOC_KEEP(sell0);
     MOC_KEEP(n_tiles);
 
     const int n = p.n;
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(32 * pair_max_warps(kPre, kTeam), 2) eval_pair
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();                        // the graph is there, the state is zero, the sums of the warps stand
+    MOC_STAGED(sell0);
     if (self) {
         off = (int64_t)warp_sum_u59(lane < wpb ? (uint64_t)s_part[lane] : 0) + group_sum(len_c0, group);
         T = __shfl_sync(kFull, len_raw, 0);
