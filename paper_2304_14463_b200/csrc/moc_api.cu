@@ -274,7 +274,8 @@ void pair_bytes(const moc_graph* g, Plan* pl) {
 // latency of a sequence and costs barriers; with more than eight sequences on an SM the warps have enough to do (n = 1000, 12 per SM:
 // 15.7 us without, 14.6 with two; n = 250, 64-bit sums 9.0 and 10.4).  Measured with 1 / 2 / 4 / 8 warps on a sequence (us; 32-bit sums): n = 153, B = 296
 // 7.2 (before) / 6.1 / 6.0; n = 353, B = 592 8.3 / 6.4 / 6.4; n = 600, B = 148 10.4 / 8.3 / 6.3 / 6.0; n = 1000, B = 592 12.5 / 10.4 / 8.4; B = 1184 14.5 / 12.4;
-// with 8 / 16: n = 1000, B = 148 6.2 / 6.2, n = 1400 6.9 / 6.6, n = 5000 12.0 / 10.4.
+// with 8 / 16: n = 1000, B = 148 6.2 / 6.2, n = 1400 6.9 / 6.6, n = 5000 12.0 / 10.4.  The block-per-sequence kernel's teams are nowhere faster at
+// one sequence per SM (block / team, 56 batches, n = 400 to 598): n = 442, B = 1 5.9 / 5.9, B = 148 6.2 / 6.2; 64-bit sums n = 560, B = 148 8.2 / 7.2.
 struct TeamShape {
     int team = 1, groups = 0, grid = 0;
 };
@@ -1065,13 +1066,6 @@ bool rows_without_scratch(const Plan& pl, int32_t B) {
     return (pl.pair || pl.lane || pl.quad) && (int64_t)pl.grid * B * 2 <= (int64_t)16 << 20;
 }
 
-// Where the warp-per-sequence kernel serves the graph, the block-per-sequence kernel still takes middle-sized graphs while
-// every SM has one sequence: as fast as eight or four warps on a sequence there (n = 442: 5.7 / 5.8 us at B = 1, 5.9 / 5.8 at 37,
-// 6.3 / 6.3 at 148), slower beyond (6.9 / 6.3 at 296; n = 1000, B = 148 8.0 / 6.4).
-bool block_serves(const moc_graph* g, int32_t B) {
-    return g->want_kind == MOC_KERNEL_AUTO && !g->want_G && warp_serves(g) && g->n >= 400 && g->n < 600 && B <= g->sm_count;
-}
-
 // The plan for a batch of B, made when a batch first needs it: looking a kernel up loads it, and a kernel that is never
 // launched should cost a program nothing (first evaluation of a handle, kernels loaded: 28 us with every kernel that may
 // serve it looked up, 25 with one; the next evaluation takes 18).  `walk`: the backward walk may serve it (which is
@@ -1082,7 +1076,7 @@ const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
         if (!g->plan_live.valid) plan_live(g, &g->plan_live);
         if (g->plan_live.live_fn) return &g->plan_live;
     }
-    const bool block = block_serves(g, B), wide = g->sum_m > (int64_t)INT32_MAX / g->C;
+    const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
     const size_t cap = g->smem_optin > 1024 ? g->smem_optin - 1024 : 0;
     auto quad = [&](Plan& kept, int mode) -> const Plan* {
         if (!kept.valid) {
@@ -1094,12 +1088,10 @@ const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
         }
         return kept.quad ? &kept : nullptr;
     };
-    const bool any_block = block || g->want_kind == MOC_KERNEL_BLOCK || (g->want_kind == MOC_KERNEL_AUTO && !g->want_G && !g->want_gpc && g->C >= 3);
+    const bool any_block = g->want_kind == MOC_KERNEL_BLOCK || (g->want_kind == MOC_KERNEL_AUTO && !g->want_G && !g->want_gpc && g->C >= 3);
     if (any_block)
         if (const int team = quad_shape(g, B, false).team)
             if (const Plan* pl = team > 1 || g->C < 3 ? quad(g->plan_chip, moc::kQuadTeams) : quad(g->plan_warps, moc::kQuadWarps)) return pl;
-    if (block)
-        if (const Plan* pl = quad(g->plan_block, moc::kQuadBlock)) return pl;
     if (team_shape(g, B).team > 1) {
         Plan& kept = g->plan_team;
         if (!kept.valid) {
@@ -1121,7 +1113,7 @@ const Plan* plan_for(const moc_graph* g, int32_t B, bool walk, int* rc) {
     return *rc == MOC_OK ? &g->plan_eval : nullptr;
 }
 
-void forget_plans(moc_graph* g) { g->plan_eval = g->plan_team = g->plan_block = g->plan_chip = g->plan_warps = g->plan_live = Plan(); }
+void forget_plans(moc_graph* g) { g->plan_eval = g->plan_team = g->plan_chip = g->plan_warps = g->plan_live = Plan(); }
 
 int launch_eval(const moc_graph* g, const int32_t* seqs, const int32_t* lens, int32_t B, int64_t M,
                 int64_t* out_peak, int64_t* out_dur, int32_t* out_feasible, cudaStream_t st) {

@@ -165,8 +165,7 @@ struct moc_graph {
     int32_t* d_tile_row = nullptr;        // first row of every successor tile
     // grow-only scratch; mutable because evaluation takes a const handle
     mutable moc_host::Plan plan_eval, plan_profile;
-    mutable moc_host::Plan plan_block;    // block-per-sequence kernel beside the warp-per-sequence one in plan_eval
-    mutable moc_host::Plan plan_chip, plan_warps;     // ... and the same with the graph in shared memory, teams of warps and single warps
+    mutable moc_host::Plan plan_chip, plan_warps;     // block-per-sequence kernel with the graph in shared memory, teams of warps and single warps
     mutable moc_host::Plan plan_team;     // warp-per-sequence kernel with several warps on each
     mutable moc_host::Plan plan_live;     // backward walk beside either
     mutable int64_t* d_offs = nullptr;

@@ -211,7 +211,7 @@ def test_lengths_that_lie(fake):
 
 @pytest.mark.parametrize("n,C,scale,nB,kernel", [(20, 2, 1, 64, "eval_pair"), (20, 2, 1, 60000, "eval_live"), (100, 2, 1 << 30, 64, "eval_pair"),
                                                  (100, 3, 1, 64, "eval_quad"), (100, 4, 1, 60000, "eval_live"), (100, 5, 1, 64, "eval_shared"),
-                                                 (442, 2, 1, 64, "eval_quad"), (442, 2, 1, 5000, "eval_pair"), (442, 3, 1, 5000, "eval_quad")])
+                                                 (442, 2, 1, 64, "eval_pair"), (442, 2, 1, 5000, "eval_pair"), (442, 3, 1, 5000, "eval_quad")])
 def test_only_kernels_that_run_are_looked_up(fake, n, C, scale, nB, kernel):
     """A first evaluation on a handle prepares the kernel it launches and no other; a later one of another size adds its own."""
     G = Graph(fake, n, C, scale)
@@ -311,7 +311,7 @@ def test_which_kernel_makes_a_profile(fake, n, C, scale, star):
 # rows of the block kernel's code: a warp per sequence, teams of warps, a block and the graph through L1; and the warp kernel's teams
 @pytest.mark.parametrize("n,C,nB,kernel", [(65, 3, 3000, "eval_quad_warp_kernelIiLi3E"), (130, 4, 18944, "eval_quad_warp_kernelIiLi4E"), (442, 3, 1, "eval_quad_kernelIiLi3ELb1ELb0ELi1E"),
                                            (1000, 4, 148, "eval_quad_kernelIiLi4ELb1ELb0ELi1E"), (5000, 4, 300, "eval_quad_kernelIiLi4ELb1ELb0ELi0E"),
-                                           (442, 2, 148, "eval_quad_kernelIiLi2ELb1ELb0ELi1E"), (442, 2, 149, "eval_pair_kernelIiLi0ELb1E"),
+                                           (442, 2, 148, "eval_pair_kernelIiLi0ELb1E"), (442, 2, 149, "eval_pair_kernelIiLi0ELb1E"),
                                            (399, 2, 1, "eval_pair_kernelIiLi0ELb1E"), (600, 2, 1, "eval_pair_kernelIiLi0ELb1E"), (600, 2, 1300, "eval_pair_kernelIiLi5ELb0E")])
 def test_which_variant_takes_a_batch(fake, n, C, nB, kernel):
     G, x = Graph(fake, n, C), np.zeros(8, np.int64)
