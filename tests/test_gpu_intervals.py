@@ -253,3 +253,44 @@ def test_interval_staged_around_the_rule_for_kept_solutions(B, n, shift):
     s, e, a, D, topo = build_batch(O, wl, np.random.default_rng(n), nB, True)
     seen = check_against_oracle(G, O, s, e, a, O.eval(np.arange(n), BIG)["peak"], D, topo=topo)
     assert any(x & ~4 == 0 for x in seen) and len(seen) >= 2
+
+
+@pytest.mark.parametrize("n,C,D,staged,shift,nB", [(300, 2, 0, True, 0, 9000), (420, 2, 0, True, 20, 5000), (1140, 2, 0, True, 0, 800),
+                                                   (200, 3, 40001, False, 0, 9000), (700, 3, 2100, False, 20, 8500)])
+def test_interval_blocks_that_take_several_solutions(B, n, C, D, staged, shift, nB):
+    """A block per solution and more solutions than blocks can be resident at once, so that a block takes several in turn, valid ones,
+    damaged ones and ones outside the domain (which end early) in any order: every kept form (16 and 32 bits, none), marks by bytes
+    and by bits, 32- and 64-bit sums."""
+    distinct = 16 if n < 1000 else 8                         # (the oracle walks the events of the domain: 3 s per solution at n = 1140)
+    rng = np.random.default_rng(n)
+    edges = W.layered_dag(n, 3 * n, 20, n)
+    w, m = W.weights_uniform(n, 1, 30, n, 1), W.weights_lognormal(n, 4.0, 1.0, n, 2) << shift
+    O, G = OracleGraph(n, edges, w, m, C), B.Graph(n, edges, w, m, C)
+    assert G.info()["wide"] == (shift > 0)
+
+    class Shape:
+        pass
+
+    wl = Shape()
+    wl.n, wl.C = n, C
+    wl.seqs, wl.lens = W.schedules(n, edges, C, 0.2, distinct, n)
+    s, e, a, D0, topo = build_batch(O, wl, rng, distinct, staged)
+    if not staged and D > D0:                                # events moved apart, in order; what lies outside stays outside
+        place = np.concatenate([[0], np.sort(rng.choice(np.arange(1, D + 1), D0, replace=False)), [D + 1]])
+        for x in (s, e):
+            inside = (x >= 0) & (x <= D0 + 1)
+            x[inside] = place[x[inside]]
+    D = max(D, D0)
+    s[5, n // 2, 0], e[6, n - 1, 1], a[7, 0, 0] = 0, D + 1, 2
+    sms, per_solution = torch.cuda.get_device_properties(0).multi_processor_count, (D // 8) * (1 if staged else 2) + 4 * n * C
+    assert nB > sms * min(32, 232448 // per_solution)        # more than the blocks (of two warps at least) that fit
+    M = O.eval(np.arange(n), BIG)["peak"] * 80 // 100
+    masks = check_against_oracle(G, O, s, e, a, M, D, topo=topo)
+    assert 64 in masks and any(x & ~4 == 0 for x in masks) and len(masks) >= 3
+    t = [dev(x) for x in (s, e, a)]
+    topo = None if topo is None else dev(topo)
+    few = G.check_intervals(*t, M, D=D, topo_index=topo)
+    which = torch.from_numpy(rng.integers(0, distinct, nB)).cuda()
+    many = G.check_intervals(*(x[which] for x in t), M, D=D, topo_index=topo)
+    for k in ("mask", "peak", "dur", "lens", "seqs"):
+        assert torch.equal(many[k], few[k][which]), k
