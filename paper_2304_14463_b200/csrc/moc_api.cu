@@ -133,11 +133,15 @@ struct QuadShape {
     int team = 0, groups = 0, grid = 0;
 };
 // Time in microseconds of a batch with u = n / 64 and s sequences per SM, in `rounds` rounds of what an SM holds at a time (fits to 354 batches
-// with every team size: n = 24 to 5000, C = 3, 4, B = 1 to 18944, 32- and 64-bit sums; mean error 5 %):
+// with every team size: n = 24 to 5000, C = 3, 4, B = 1 to 18944; mean error 5 % with 32-bit sums):
 //     a warp per sequence         4.3 + rounds (1.5 + (0.19 + 0.31 C) u) + s (0.07 + 0.009 C u)
 //     t warps per sequence        5.0 + rounds (1.0 + (0.15 + 0.28 C) u / t) + s (0.09 + 0.054 t + 0.012 C u)
 //     a block of 64 w threads     5.3 + rounds (1.3 + (0.40 + 0.15 C) u / w + 0.046 w) + s (0.10 + 0.040 w + 0.010 C u)
-// The smallest of them costs 1.2 % on the mean against always taking the fastest, 4 % or less in nine of ten.  Before / now (C = 3): n = 153,
+// The smallest of them costs on the mean, against always taking the fastest, 0.3 % at C = 3 and 1.7 % at C = 4 (108 batches), with 64-bit sums
+// 0.5 and 1.4 % (330 batches), 2 and 7 % or less in nine of ten, 22 % at worst.  64-bit sums take 4 to 20 % longer than the lines, much the
+// same on all three, so that a factor on one line only costs and lines of their own gain 0.3 %.  Against the version with a block per sequence for
+// every batch they are faster by 1.20 (C = 3) and 1.16 (C = 4) on the mean of 112 batches; n = 1500, C = 4, B = 1776 (53 -> 58 us) and n = 700, C = 4,
+// B = 592 (13.3 -> 14.3) lose.  Before / now (C = 3): n = 153,
 // B = 18944 68 -> 39 us, n = 24 45 -> 21, n = 442, B = 4736 33 -> 27, n = 1000, B = 1776 26.9 -> 24.8.
 double quad_block_cost(int64_t n, int32_t C, int64_t per_sm, int blocks, int w) {
     const double u = (double)n / 64.0, rounds = (double)((per_sm + blocks - 1) / blocks);
@@ -643,6 +647,7 @@ void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::ve
         for (int64_t k = 0; k < ne; ++k) pred[fill[keys[k] & 0xFFFFFFFFu]++] = (int32_t)(keys[k] >> 32);
         for (int32_t v = 0; v < n; ++v)
             if (succ_start[v + 1] == succ_start[v]) g->sink_m += m[v];
+        // (for the search; 1 to 2 % of creating a handle: n = 442 490 us, n = 5000 1790 -> 1815)
         if (ne <= 65535 && g->sum_w < ((int64_t)1 << 31) && g->n <= 16000) {
             const size_t list = ((size_t)ne + 3) & ~size_t(3);
             std::vector<uint32_t> near((2 * ((size_t)n + 1) + list + 3) & ~size_t(3), 0u);

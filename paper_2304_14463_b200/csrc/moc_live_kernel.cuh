@@ -25,10 +25,10 @@
 // different words where possible, and more bits than that are left to a loop that few steps need.  (A loop
 // over the set bits of each word instead: 69 us at the size below, 1200 cycles per step.)
 //
-// n = 100, B = 65536, C = 2: 38.9 us (one launch) against 84 us for the warp-per-sequence kernel behind the offsets kernel.
+// n = 100, B = 65536, C = 2: 36.2 to 37.0 us (one launch) against 84 us for the warp-per-sequence kernel behind the offsets kernel.
 // The range of a block from the host and sums by warp reductions instead of 64-bit divisions, shuffles and loops over the warps:
-// 36.7 -> 36.1 us, n = 34, B = 65536 15.8 -> 14.9, n = 46, B = 32100 16.1 -> 14.6.  Eight steps at a time instead of four: 38.5.
-// Bound: the integer pipe, about 87 warp instructions per step of 32 sequences (issue slots 63 %, ALU pipe 54 %), a fifth of them for bits beyond one per word.
+// kernel time 39.3 -> 37.2 us (ncu, caches kept), n = 34, B = 65536 15.8 -> 14.9, n = 46, B = 32100 16.1 -> 14.6.  Eight steps at a time instead of four: + 1.5.
+// Bound: the integer pipe, about 87 warp instructions per step of 32 sequences (issue slots 65 %, ALU pipe 55 %), a fifth of them for bits beyond one per word.
 // The warp-per-sequence kernel pays a warp's fixed costs (clearing, scans, reductions) per sequence, which a
 // sequence of 120 steps does not repay; at n > 128 the masks outgrow the registers.
 #pragma once

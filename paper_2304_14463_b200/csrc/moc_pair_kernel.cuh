@@ -198,11 +198,12 @@ __device__ __forceinline__ void team_sync(int id, int threads) {
 __host__ __device__ constexpr int pair_max_warps(int pre, bool team) { return pre == 0 && !team ? 19 : 16; }
 
 // Bound, large batches: the shared-memory data pipe (three quarters of one wavefront per clock, 528 wavefronts per
-// sequence) and instruction issue (68 %, 1795 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 41.0 -> 39.7 to 40.95 us over five boxes (four
-// exchanges in flight before their results are looked at, ragged ends of a row through the same code, no second search for
-// the end of the row).  Bound, small batches: a chain of latencies; the division for a block's range, the sums of the
-// lengths by shuffles and loops, and the copy of the graph behind one another were half of it (n = 20, B = 1024: 6.15 -> 5.9 us,
-// where the host's calls are what is left; n = 442, B = 592 10.2 -> 7.3; n = 1000, B = 592 12.3 -> 8.4, the latter two with kTeam).
+// sequence) and instruction issue (68 %, 1795 instructions per sequence); DRAM traffic equals the rows.  n = 442, B = 16384: 41.9 -> 41.6 us
+// of kernel time (ncu, caches kept), 40.95 -> 40.4 to 40.95 us a launch back to back, by four exchanges in flight before their results
+// are looked at, ragged ends of a row through the same code, no second search for the end of the row.  Bound, small
+// batches: a chain of latencies; the division for a block's range, the sums of the lengths by shuffles and loops, and the copy
+// of the graph behind one another were part of it (kernel time at n = 20, B = 1024 5.4 -> 4.7 us, where a call takes 5.8 to 6.1;
+// a call at n = 442, B = 592 10.2 -> 7.3, n = 1000, B = 592 12.3 -> 8.4, these two with kTeam).
 //
 // kPre: how many 16-byte vectors of the next row each lane fetches ahead (rows of about 128*kPre
 // steps; 0 for short rows, where the extra registers cost more than the wait).  Blocks have up to 16

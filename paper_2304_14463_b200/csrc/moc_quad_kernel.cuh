@@ -666,6 +666,9 @@ __device__ __forceinline__ void quad_evaluate(const QuadParams& p) {
     if constexpr (kChip && kProfile) asm volatile("cp.async.wait_all;" ::: "memory");      // nothing under way where no sequence was evaluated
 }
 
+// Blocks of up to 1024 threads leave 64 registers a thread.  Four copies kept apart need more: with 64-bit sums 52 bytes a
+// thread are spilled for a block per sequence, 88 for teams and 116 for a warp per sequence (32-bit sums: 24 for teams; three
+// copies, 64 bits: 12 to 24).
 template <typename MemT, int kAcc, bool kTiles, bool kProfile, int kMode>
 __global__ void __launch_bounds__(1024) eval_quad_kernel(const QuadParams p) {
     quad_evaluate<MemT, kAcc, kTiles, kProfile, kMode>(p);
