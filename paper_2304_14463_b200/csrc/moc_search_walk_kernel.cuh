@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
     const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
     const int warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
-    uint32_t l_node = sbase + p.rec_bytes + p.sell_bytes, l_succ = l_node + 8u * (uint32_t)(p.n + 1), l_pred = l_succ + 2u * (uint32_t)((p.n_edges + 3) & ~3);
+    uint32_t l_node = sbase + p.rec_bytes + p.sell_bytes;
     {
         // asynchronous copies: a block of a small population has few threads for them
         auto copy = [&](uint32_t to, const void* from, uint32_t bytes) {
@@ -236,11 +236,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
         asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(da - kPairDeltaFront + o), "r"(0) : "memory");
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    if constexpr (kLists) {
-        MOC_STAGED(l_node);
-        MOC_STAGED(l_succ);
-        MOC_STAGED(l_pred);
-    }
+    if constexpr (kLists) MOC_STAGED(l_node);
+    const uint32_t l_succ = l_node + 8u * (uint32_t)(p.n + 1), l_pred = l_succ + 2u * (uint32_t)((p.n_edges + 3) & ~3);
 
     for (int32_t c = blockIdx.x * wpb + warp; c < s.P; c += gridDim.x * wpb) {
         int32_t* row = s.rows + ((int64_t)s.cur[c] * s.P + c) * s.stride;

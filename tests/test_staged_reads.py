@@ -11,7 +11,7 @@ from paper_2304_14463_b200 import build
 
 # kernel -> bases of the tables that it reads freely
 FREE = {"eval_pair_kernel": {"sell0"}, "eval_live_kernel": {"pa", "ra", "ma", "own"}, "eval_lane_kernel": {"a_succ"},
-        "edit_prepare_kernel": {"sell0"}, "search_walk_kernel": {"l_node", "l_succ", "l_pred"}}
+        "edit_prepare_kernel": {"sell0"}, "search_walk_kernel": {"l_node"}}
 
 
 def functions():
