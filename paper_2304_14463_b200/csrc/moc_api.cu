@@ -650,7 +650,7 @@ void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::ve
         // (for the search; 1 to 2 % of creating a handle: n = 442 490 us, n = 5000 1790 -> 1815)
         if (ne <= 65535 && g->sum_w < ((int64_t)1 << 31) && g->n <= 16000) {
             const size_t list = ((size_t)ne + 3) & ~size_t(3);
-            std::vector<uint32_t> near((2 * ((size_t)n + 1) + list + 3) & ~size_t(3), 0u);
+            std::vector<uint32_t> near((2 * ((size_t)n + 1) + list + (size_t)n + 3) & ~size_t(3), 0u);
             uint16_t* lists = reinterpret_cast<uint16_t*>(near.data() + 2 * ((size_t)n + 1));
             for (int32_t v = 0; v <= n; ++v) {
                 near[2 * (size_t)v] = (uint32_t)succ_start[v] | (uint32_t)pred_start[v] << 16;
@@ -660,6 +660,7 @@ void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::ve
                 lists[k] = (uint16_t)succ[k];
                 lists[list + k] = (uint16_t)pred[k];
             }
+            for (int32_t v = 0; v < n; ++v) near[2 * ((size_t)n + 1) + list + (size_t)v] = (uint32_t)m32[v];
             g->near_bytes = near.size() * 4;
             tables->add(&g->d_near, std::move(near));
         }

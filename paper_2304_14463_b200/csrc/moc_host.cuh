@@ -38,7 +38,7 @@ const void* check_plain_fn(bool wide);
 IntervalFn check_general_fn(int cp, bool wide, int kept, bool team);      // kept: bytes per event of the solution kept on chip, 0: not kept
 IntervalFn check_staged_fn(int cp, bool wide, int kept, bool team);      // team: a block per solution
 const void* score_fn(bool wide, bool graph_on_chip);
-const void* walk_fn(bool wide, bool lists);      // lists: the neighbours' lists in shared memory
+const void* walk_fn(bool wide, bool lists, bool floor);      // lists: the neighbours' lists in shared memory; floor: its test bounds the new peak
 
 constexpr int kHostParts = 3;          // parts in which the host entry points send a large batch
 
@@ -133,7 +133,7 @@ struct moc_graph {
     int32_t* d_pred_start = nullptr;     // predecessor lists (CSR), for the incremental evaluation
     int32_t* d_pred = nullptr;
     uint32_t* d_near = nullptr;           // both lists with 16 bits an entry, for the search: per node {first successor | first predecessor << 16,
-    size_t near_bytes = 0;                // duration}, the successors, the predecessors (null: more than 65535 edges, or durations of 2^31)
+    size_t near_bytes = 0;                // duration}, the successors, the predecessors, m32 (null: more than 65535 edges, or durations of 2^31)
     int64_t sink_m = 0;                   // sum of m over the nodes without successors
     int32_t max_indeg = 0;                // largest number of predecessors of a node
     int64_t* d_w = nullptr;

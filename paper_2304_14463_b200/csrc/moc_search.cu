@@ -39,6 +39,7 @@ struct moc_search {
     uint64_t graph_generation = 0;     // the graph's C and caps when the chains were evaluated
     moc::WalkParams wp{};
     const void* walk_fn = nullptr;     // null: not planned yet, or the graph does not fit (walk_planned)
+    const void* walk_fn_floor = nullptr;     // the same with the bound on the new peak
     bool walk_planned = false;
     bool walk_scores = false;          // incremental, and the walk kernel does it (no cache)
     int walk_wpb = 0, walk_grid = 0;
@@ -118,6 +119,7 @@ void plan_walk(moc_search* s) {
     w.pred_start = g->d_pred_start;
     w.pred = g->d_pred;
     w.w = g->d_w;
+    w.m = g->d_m64;
     w.rec_bytes = (wide ? 16u : 8u) * 64u * (uint32_t)g->n_tiles;
     w.sell_bytes = (4u * (uint32_t)g->sell_len + 15u) & ~15u;
     w.word_bytes = (4u * ((uint32_t)g->n + 2u) + 15u) & ~15u;
@@ -141,15 +143,17 @@ void plan_walk(moc_search* s) {
     const bool lists = g->d_near != nullptr && graph_b + list_b + (size_t)best * warp_b <= cap;
     w.lists = g->d_near;
     w.list_bytes = (uint32_t)list_b;
-    const void* fn = walk_fn(wide, lists);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
+    const void* const fn[2] = {walk_fn(wide, lists, false), walk_fn(wide, lists, true)};
+    for (const void* f : fn)
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
     s->walk_wpb = best;
     s->walk_grid = (int)std::min<int64_t>(sm, ((int64_t)s->P + best - 1) / best);
     s->walk_smem = graph_b + (lists ? list_b : 0) + (size_t)best * warp_b;
-    s->walk_fn = fn;
+    s->walk_fn = fn[0];
+    s->walk_fn_floor = fn[1];
 }
 
 // Proposals per chain of one launch: enough that the launch does not show, few enough for a caller who waits.
@@ -275,12 +279,17 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
         while (w.lanes_per_gen < std::min(s->samples, 32)) w.lanes_per_gen *= 2;
         w.cap = g->d_cap;
         const int32_t most = std::max(1, kWalkProposals / s->samples);
+        // With a bound on the new peak where enough evaluations fall away for what it costs: many proposals of a generation (one in three of
+        // them is evaluated then) or expensive evaluations.  With / without, 10 generations: n = 30, E = 32, 20000 chains 243 / 287 us, n = 78, E = 8, 255
+        // chains 20.6 / 23.4, n = 260, E = 8, 8000 chains 63 / 93; n = 442, E = 1, 4096 chains x 20 32.8 / 38.2.  No gain: n = 200, E = 8, a layered
+        // graph 212 / 201, n = 300, E = 1 the same; n = 30, E = 1 158 / 149.
+        const void* fn = s->samples >= 8 || g->n_tiles > 4 ? s->walk_fn_floor : s->walk_fn;
         for (int32_t k = 0; k < n_generations; k += most) {
             w.s = p;
             w.s.generation = s->generation + (uint32_t)k;
             w.n_gen = std::min(most, n_generations - k);
             void* args[] = {&w};
-            MOC_CUDA(cudaLaunchKernel(s->walk_fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, s->walk_smem, st));
+            MOC_CUDA(cudaLaunchKernel(fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, s->walk_smem, st));
             ++launches;
         }
         s->generation += (uint32_t)n_generations;

@@ -12,6 +12,9 @@
 // the occurrence pass of the evaluation kernel (data-dependent exchanges) falls away.  A proposal that
 // cannot be accepted whatever its peak (longer duration while the chain is within the budget) is not
 // evaluated: the key of the chain decides already.
+// With kFloor the test also works out the usage that the edited sequence has at the step where the chain reaches its peak.  The new
+// peak is no lower, which refuses proposals and orders the others: the first of them that reaches its bound ends the generation.  Of 3.3 admissible proposals
+// of 32 0.95 are evaluated (n = 442, over the budget; counted on the CPU), and nearly every one of those is accepted.
 //
 // The sequence itself stays in global memory (L2): the tests read one element per proposal, and an
 // accepted edit shifts the elements between its two places by one.  It is kept there because 3.5 KB per warp
@@ -24,7 +27,9 @@
 // the latency of its dependent shared-memory reads; 28 warps beat 24 and 20 with more registers each, and 30 with fewer.
 // n = 442, state copied out: 4096 chains x 20 generations 436 -> 41.9 us against two kernels per generation that
 // write every proposal out, 38.9 with the neighbours' lists on chip, 37.1 with the words of a sequence from eight loads in flight; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us
-// against a cached evaluation per chain that is rebuilt after every acceptance, 1010 -> 951 with the lists.
+// against a cached evaluation per chain that is rebuilt after every acceptance, 1010 -> 951 with the lists, 870 -> 500 (another GPU 1004 -> 508) with the bound.
+// Tried: the chain's deltas kept and corrected for the few intervals that an edit changes instead of stages 2 and 3 over all nodes (two more calls and
+// serial chains per evaluation: 503 -> 578 us there, small graphs 20 to 40 % slower; n = 900 gained 20 %).
 #pragma once
 #include "moc_edit_kernels.cuh"
 #include "moc_search_kernels.cuh"
@@ -38,7 +43,7 @@ struct WalkParams {
     int32_t n_gen;             // generations of this launch
     int32_t samples;           // E: proposals per chain and generation
     int32_t lanes_per_gen;     // E rounded up to a power of two, at most 32
-    int32_t* peak_at;          // P: where the peak of each chain's sequence lies (walk_eval's `at`), 0: not known
+    int32_t* peak_at;          // P: walk_eval's `at` of each chain's sequence, 0: not known
     int32_t n, C, n_tiles;
     int32_t split;             // 64-bit sums: as in PairParams
     const void* rec;           // node records and successor tiles of the warp-per-sequence layout
@@ -48,6 +53,7 @@ struct WalkParams {
     const int32_t* pred_start;
     const int32_t* pred;
     const int64_t* w;
+    const int64_t* m;
     const int32_t* cap;        // per-node caps or nullptr
     uint32_t rec_bytes, sell_bytes;      // graph, once per block
     int32_t n_edges;
@@ -76,9 +82,9 @@ __device__ __forceinline__ uint32_t walk_above(uint32_t p, uint32_t k) {
 }
 
 // Stages 2 to 4 of the evaluation (moc_pair_kernel.cuh) on the occurrence words at `wa`: the peak, whether a
-// consumer lacks a producer copy, and `at`: the peak is reached at one of the steps at .. at + 16 / sizeof(MemT) - 1
-// (1-based; one vector of deltas).  The deltas are zero on entry and on return.
-template <typename MemT>
+// consumer lacks a producer copy, and `at`: a step at which the peak is reached (1-based) or, without kExact, minus the first step of a
+// vector of deltas that has one.  The deltas are zero on entry and on return.
+template <typename MemT, bool kExact>
 __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec0, uint32_t sell0, int n_tiles, int32_t T, int lane,
                                        int32_t split, bool& dep, int32_t& at) {
     constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
@@ -137,7 +143,7 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
     }
     dep = __any_sync(kFull, (depw & 0x80008000u) != 0);
     __syncwarp();
-    // prefix sum and running maximum; lane owns V consecutive vectors, which it clears behind itself
+    // prefix sum and running maximum; lane owns V consecutive vectors
     const int nvec = (T + 2 + kPerVec - 1) / kPerVec, V = ((nvec + 31) >> 5) | 1;
     uint32_t ad = da + 16u * (uint32_t)(lane * V);
     MemT top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
@@ -146,7 +152,7 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
     uint32_t lo = 0, hi = 0;           // 64-bit sums: the two parts of the running sum (moc_pair_kernel.cuh)
     for (int j = 0; j < V; ++j, ad += 16u) {
         const uint4 q = lds_v4(ad);
-        asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(ad), "r"(0) : "memory");
+        if constexpr (!kExact) asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(ad), "r"(0) : "memory");
         MemT most;
         if constexpr (sizeof(MemT) == 4) {
             run += (MemT)q.x; most = run;
@@ -166,7 +172,22 @@ __device__ __forceinline__ MemT walk_eval(uint32_t wa, uint32_t da, uint32_t rec
     else top += split_value(warp_inclusive_sum(lo, lane) - lo, warp_inclusive_sum(hi, lane) - hi, split);
     const MemT peak = warp_max_t(top);
     const int src = __ffs(__ballot_sync(kFull, top == peak)) - 1;
-    at = kPerVec * (src * V + __shfl_sync(kFull, vec, src)) + 1;
+    vec = src * V + __shfl_sync(kFull, vec, src);
+    at = kPerVec * vec + 1;
+    if constexpr (kExact) {
+        const uint4 q = lds_v4(da + 16u * (uint32_t)vec);       // the first of its steps with the largest sum of deltas
+        if constexpr (sizeof(MemT) == 4) {
+            const MemT s1 = (MemT)q.y, s2 = s1 + (MemT)q.z, s3 = s2 + (MemT)q.w, most = max(max(s1, s2), max(s3, (MemT)0));
+            at += most == 0 ? 0 : most == s1 ? 1 : most == s2 ? 2 : 3;
+        } else {
+            at += split_value(q.z, q.w, split) > 0 ? 1 : 0;
+        }
+        __syncwarp();
+        ad = da + 16u * (uint32_t)(lane * V);
+        for (int j = 0; j < V; ++j, ad += 16u) asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(ad), "r"(0) : "memory");
+    } else {
+        at = -at;
+    }
     __syncwarp();
     return peak;
 }
@@ -196,7 +217,7 @@ static __device__ __noinline__ void walk_apply(int32_t* row, int32_t T, int32_t 
 
 // kLists: the test of a proposal reads the neighbours' lists from the block's shared memory (durations below 2^31, at most 65535 edges);
 // through L1, of which the chains' state leaves little, a third of the kernel's stalls were waits for them.
-template <typename MemT, bool kLists>
+template <typename MemT, bool kLists, bool kFloor>
 __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const WalkParams p) {
     extern __shared__ __align__(16) char smem[];
     const SearchParams& s = p.s;
@@ -237,11 +258,25 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if constexpr (kLists) MOC_STAGED(l_node);
-    const uint32_t l_succ = l_node + 8u * (uint32_t)(p.n + 1), l_pred = l_succ + 2u * (uint32_t)((p.n_edges + 3) & ~3);
+    const uint32_t l_succ = l_node + 8u * (uint32_t)(p.n + 1), l_pred = l_succ + 2u * (uint32_t)((p.n_edges + 3) & ~3), l_size = l_pred + 2u * (uint32_t)((p.n_edges + 3) & ~3);
+    auto size_of = [&](int32_t v) -> MemT {
+        if constexpr (kLists && sizeof(MemT) == 4) return (MemT)lds_u32_nv(l_size + 4u * (uint32_t)v);
+        else return (MemT)__ldg(p.m + v);
+    };
+    auto successors = [&](int32_t v, int32_t& from, int32_t& to) {
+        if constexpr (kLists) {
+            from = (int32_t)(lds_u32_nv(l_node + 8u * (uint32_t)v) & 0xFFFFu);
+            to = (int32_t)(lds_u32_nv(l_node + 8u * (uint32_t)v + 8u) & 0xFFFFu);
+        } else {
+            from = __ldg(p.succ_start + v);
+            to = __ldg(p.succ_start + v + 1);
+        }
+    };
 
     for (int32_t c = blockIdx.x * wpb + warp; c < s.P; c += gridDim.x * wpb) {
         int32_t* row = s.rows + ((int64_t)s.cur[c] * s.P + c) * s.stride;
-        int32_t T = s.lens[c], tp = p.peak_at[c];
+        int32_t T = s.lens[c], tp = p.peak_at[c];       // without kFloor a step of either kind, else 0 for one that is not exact
+        tp = kFloor ? max(tp, 0) : abs(tp);
         bool valid = s.status[c] >= 0;
         bool over = valid && s.peak[c] > s.M;       // over the budget
         if (lane == 0) {
@@ -315,16 +350,26 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
         };
 
         // The edit (qd, ji) of node x against the chain's valid sequence: can it be accepted, as far as the copies of x
-        // and of its neighbours tell; the node's word after the edit and the new duration.
-        auto test = [&](int32_t op, int32_t qd, int32_t ji, int32_t x, uint32_t& wx_new, int64_t& du_c) -> bool {
+        // and of its neighbours tell; the node's word after the edit, the new duration, and, with kFloor, what the new peak cannot be below: at
+        // most the usage after the edit at the step where the chain reaches its peak (0: that step is not known, or is the one taken out).
+        // An edit of x changes what is resident there for x and its predecessors only.  A node is resident at step tp when its last copy
+        // up to tp is the step itself, or has a consumer at tp or behind it and in front of the node's next copy.
+        auto test = [&](int32_t op, int32_t qd, int32_t ji, int32_t x, uint32_t& wx_new, int64_t& du_c, MemT& floor_c) -> bool {
             const uint32_t wx = lds_u32(wa + 4u * (uint32_t)x);
             const int32_t xa = (int32_t)min(wx & 0xFFFFu, wx >> 16) - 1, xb = (int32_t)max(wx & 0xFFFFu, wx >> 16) - 1;
             const int32_t cnt = xa == xb ? 1 : 2, cnt2 = cnt - (op >= 1 ? 1 : 0) + (op != 1 ? 1 : 0);
             if (!(cnt2 == 1 || (cnt2 == 2 && p.C >= 2 && (p.cap == nullptr || __ldg(p.cap + x) >= 2)))) return false;
             const int64_t more = duration(x) * (cnt2 - cnt);
             du_c = (int64_t)lds_u64(note + kWalkDu) + more;
+            floor_c = 0;
             const bool longer = more > 0;
             if (longer && !over) return false;      // within the budget only the duration decides
+            const bool known = tp > 0 && (!kFloor || tp != qd + 1);
+            const int32_t tmax = kFloor ? tp : tp + 16 / (int32_t)sizeof(MemT) - 1;
+            // Over the budget a longer sequence has to lower the peak.  A second copy of x lowers the usage at the
+            // peak's step only when x is resident there for a later consumer, which the second copy can serve.
+            // (Everything else an inserted copy does to the profile adds to it.)
+            if (longer && known && !(xa + 1 < tmax && ji >= tp)) return false;
             auto map = [&](int32_t t) -> int32_t { const int32_t t1 = t - (t > qd ? 1 : 0); return t1 + (t1 >= ji ? 1 : 0); };
             // first child copy c0 (and c1), with the parent steps of other nodes' copies that lie in front of c0
             // (r < tb0) and behind it (r > ta0), 1-based, as in moc_edit_pass.cuh
@@ -334,48 +379,98 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                 else if (cs < c0) { c1 = c0; c0 = cs; ta0 = ta; tb0 = tb; }
                 else { c1 = cs; }
             };
+            const int32_t thr = ji == kEditNone ? -1 : ji + (ji >= qd ? 1 : 0);     // steps in front of the inserted copy
             if (xa != qd) push(map(xa), xa + 1, xa + 1);
             if (cnt == 2 && xb != qd) push(map(xb), xb + 1, xb + 1);
-            if (ji != kEditNone) { const int32_t thr = ji + (ji >= qd ? 1 : 0); push(ji, thr, thr + 1); }
+            if (ji != kEditNone) push(ji, thr, thr + 1);
             wx_new = (uint32_t)(c0 + 1) | (uint32_t)((c1 == kEditNone ? c0 : c1) + 1) << 16;
-            // Over the budget a longer sequence has to lower the peak.  A second copy of x lowers the usage at the
-            // peak's step only when the first copy, which is resident there for a later consumer, can end in front of it:
-            // the peak lies behind the first copy and in front of the second, and so does no consumer from the
-            // peak on.  (Everything else an inserted copy does to the profile adds to it.)
-            const bool must_drop = longer && tp > 0;
-            const int32_t tmax = tp + 16 / (int32_t)sizeof(MemT) - 1;
-            if (must_drop && !(xa + 1 < tmax && ji >= tp)) return false;
-            bool viol = false, later = false;
+            bool viol = false;
             int32_t p0, p1, s0, s1;
+            successors(x, s0, s1);
             if constexpr (kLists) {
-                const uint32_t from = lds_u32_nv(l_node + 8u * (uint32_t)x), to = lds_u32_nv(l_node + 8u * (uint32_t)x + 8u);
-                s0 = (int32_t)(from & 0xFFFFu);
-                s1 = (int32_t)(to & 0xFFFFu);
-                p0 = (int32_t)(from >> 16);
-                p1 = (int32_t)(to >> 16);
+                p0 = (int32_t)(lds_u32_nv(l_node + 8u * (uint32_t)x) >> 16);
+                p1 = (int32_t)(lds_u32_nv(l_node + 8u * (uint32_t)x + 8u) >> 16);
             } else {
-                p0 = __ldg(p.pred_start + x); p1 = __ldg(p.pred_start + x + 1);
-                s0 = __ldg(p.succ_start + x); s1 = __ldg(p.succ_start + x + 1);
+                p0 = __ldg(p.pred_start + x);
+                p1 = __ldg(p.pred_start + x + 1);
             }
+            // without kFloor: a longer sequence needs a consumer of x that the second copy serves, and none from the peak to that copy
+            const bool must_drop = !kFloor && longer && known;
+            bool served = false;
+            const uint32_t from_tp = ((0x00010000u - (uint32_t)tp) & 0xFFFFu) * 0x10001u;     // -tp in both halves
+            uint32_t next = 0xFFFFFFFFu;            // first consumer of x at tp or behind it, counted from there
             // two reads of each kind in flight
 #pragma unroll 1
             for (int32_t k = 0; k < max(p1 - p0, s1 - s0); k += 2) {
                 uint32_t pw[2], sw[2];
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    pw[i] = p0 + k + i < p1 ? lds_u32(wa + 4u * neighbour(l_pred, p.pred, p0 + k + i)) : 0u;
-                    sw[i] = s0 + k + i < s1 ? lds_u32(wa + 4u * neighbour(l_succ, p.succ, s0 + k + i)) : 0xFFFFFFFFu;
+                    pw[i] = p0 + k + i < p1 ? lds_u32(wa + 4u * (int32_t)neighbour(l_pred, p.pred, p0 + k + i)) : 0u;
+                    sw[i] = s0 + k + i < s1 ? lds_u32(wa + 4u * (int32_t)neighbour(l_succ, p.succ, s0 + k + i)) : 0xFFFFFFFFu;
                 }
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    viol |= (int32_t)min(pw[i] & 0xFFFFu, pw[i] >> 16) > ta0;
-                    const int32_t r0 = (int32_t)min(sw[i] & 0xFFFFu, sw[i] >> 16), r1 = (int32_t)max(sw[i] & 0xFFFFu, sw[i] >> 16);
-                    const bool is = s0 + k + i < s1;
-                    viol |= is && (r0 < tb0 || (must_drop && ((r0 >= tmax && r0 <= ji) || (r1 >= tmax && r1 <= ji))));
-                    later |= is && r1 > ji;
+                    const int32_t ua = (int32_t)min(pw[i] & 0xFFFFu, pw[i] >> 16), r0 = (int32_t)min(sw[i] & 0xFFFFu, sw[i] >> 16);
+                    viol |= ua > ta0 || r0 < tb0;
+                    if constexpr (kFloor) {
+                        next = __viaddmin_u16x2(sw[i], from_tp, next);
+                    } else if (s0 + k + i < s1) {
+                        const int32_t r1 = (int32_t)max(sw[i] & 0xFFFFu, sw[i] >> 16);
+                        viol |= must_drop && ((r0 >= tmax && r0 <= ji) || (r1 >= tmax && r1 <= ji));
+                        served |= r1 > ji;
+                    }
                 }
             }
-            return !viol && (!must_drop || later || s0 == s1);
+            if (viol) return false;
+            if (!kFloor) return !must_drop || served || s0 == s1;
+            if (!known) return true;
+            // copies of x at tp or in front of it, before and after; the last step in front of the next one
+            bool had = xa < tp, has = thr >= 0 && thr < tp;
+            int32_t lim_old = had && xb >= tp ? xb : 0x7FFF, lim_new = thr >= tp ? thr : 0x7FFF;
+            if (xa != qd) {
+                has |= xa < tp;
+                if (xa >= tp) lim_new = min(lim_new, xa);
+            }
+            if (xb != qd) {
+                has |= xb < tp;
+                if (xb >= tp) lim_new = min(lim_new, xb);
+            }
+            const int64_t pk = (int64_t)lds_u64(note + kWalkPk);
+            MemT change = 0;
+            if (xa + 1 != tp && xb + 1 != tp) {
+                const int32_t first = s0 == s1 ? 0x7FFF : (int32_t)min(next & 0xFFFFu, next >> 16) + tp;    // a sink is kept to the end
+                const bool now = has && first <= lim_new, then = had && first <= lim_old;
+                if (now != then) change = now ? size_of(x) : -size_of(x);
+            }
+            // A predecessor that loses a consumer: qd lies behind tp in the range of its copy, ji does not, and no other consumer does.
+            // What one gains is left out (0.95 instead of 0.92 evaluations a generation, for less than half of the lists to go through).
+            if (qd >= tp && qd != kEditNone) {
+                const int32_t j_won = thr >= tp ? thr : 0x8000;
+                uint32_t rest = 0xFFFFFFFFu;            // the copies of x that stay
+                if (xa != qd) rest = (uint32_t)(xa + 1) * 0x10001u;
+                if (xb != qd) rest = xa != qd ? (rest & 0xFFFFu) | (uint32_t)(xb + 1) << 16 : (uint32_t)(xb + 1) * 0x10001u;
+#pragma unroll 1
+                for (int32_t k = p0; k < p1; ++k) {
+                    const int32_t u = (int32_t)neighbour(l_pred, p.pred, k);
+                    const uint32_t pw = lds_u32(wa + 4u * (uint32_t)u);
+                    const int32_t ua = (int32_t)min(pw & 0xFFFFu, pw >> 16), ub = (int32_t)max(pw & 0xFFFFu, pw >> 16), end = ub > tp ? ub : 0x7FFF;
+                    if (qd + 1 >= end || end > j_won || ua >= tp || ub == tp) continue;
+                    int32_t t0, t1;
+                    successors(u, t0, t1);
+                    uint32_t near = 0xFFFFFFFFu;        // another consumer
+#pragma unroll 1
+                    for (int32_t i = t0; i < t1; i += 2) {
+                        const int32_t v0 = (int32_t)neighbour(l_succ, p.succ, i), v1 = (int32_t)neighbour(l_succ, p.succ, min(i + 1, t1 - 1));
+                        const uint32_t w0 = lds_u32(wa + 4u * (uint32_t)v0), w1 = lds_u32(wa + 4u * (uint32_t)v1);
+                        near = __viaddmin_u16x2(v0 == x ? rest : w0, from_tp, near);
+                        near = __viaddmin_u16x2(v1 == x ? rest : w1, from_tp, near);
+                    }
+                    if ((int32_t)min(near & 0xFFFFu, near >> 16) + tp >= end) change -= size_of(u);
+                }
+            }
+            floor_c = (MemT)pk + change;
+            const int64_t a_c = (int64_t)floor_c > s.M ? (int64_t)floor_c : s.M, a_p = over ? pk : s.M;
+            return a_c < a_p || (a_c == a_p && more <= 0);
         };
         // smallest of the lanes' values >= 0
         auto min64 = [&](int64_t v, bool in) -> int64_t {
@@ -386,8 +481,11 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
 
         // A batch is `span` generations of E proposals with a lane each, or, for E > 32, 32 proposals of one
         // generation; the best proposal of the generation is then carried from batch to batch.
+        const int64_t m_cap = sizeof(MemT) == 4 ? (int64_t)INT32_MAX : INT64_MAX;
+        const MemT m_low = (MemT)min(max(s.M, (int64_t)0), m_cap);
         const int32_t E = p.samples, per = p.lanes_per_gen, span = 32 / per, my_gen = lane / per, my_e = lane % per;
         bool b_has = false, b_here = false;         // a proposal is chosen; its words are at wb
+        int32_t b_e = 0;                            // its number (with E <= 32 its lane: generations are settled one at a time)
         auto fresh = [&]() {                        // a chain without a valid sequence takes any valid proposal
             b_has = false;
             if (lane == 0) {
@@ -406,7 +504,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             wa = wb;
             wb = sw;
             T = Tc_s;
-            tp = (int32_t)lds_u32(note + kWalkBestAt);
+            tp = abs((int32_t)lds_u32(note + kWalkBestAt));
             valid = true;
             over = (int64_t)lds_u64(note + kWalkBestPk) > s.M;
             if (lane == 0) {
@@ -437,12 +535,14 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                     bool adm = (pending >> lane & 1u) != 0 && Tc >= n && Tc <= s.max_T;
                     uint32_t wx_new = 0;
                     int64_t du_c = 0;
-                    if (adm && valid) adm = test(op, qd, ji, x, wx_new, du_c);
+                    MemT floor_c = 0;
+                    if (adm && valid) adm = test(op, qd, ji, x, wx_new, du_c, floor_c);
+                    const MemT a_low = kFloor && floor_c > m_low ? floor_c : m_low;       // the least the key's first part can be
                     const uint32_t places = (uint32_t)q | (uint32_t)j << 15 | (uint32_t)op << 30;     // T < 2^15
                     uint32_t todo = __ballot_sync(kFull, adm);
                     pending = 0;
                     while (todo) {
-                        // ---- the earliest generation that has proposals left: in order of duration, then number
+                        // ---- the earliest generation that has proposals left: in order of the least their key can be, then number
                         const int gen = (__ffs(todo) - 1) / per;
                         const uint32_t group = (per == 32 ? kFull : (1u << per) - 1u) << (gen * per);
                         uint32_t cand = todo & group;
@@ -450,7 +550,13 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                         while (cand) {
                             int sl = __ffs(cand) - 1;
                             if (cand & (cand - 1u)) {
-                                const bool in = (cand >> lane & 1u) != 0;
+                                bool in = (cand >> lane & 1u) != 0;
+                                if constexpr (kFloor) {
+                                    MemT a_min;             // by all lanes, whether or not theirs is left
+                                    if constexpr (sizeof(MemT) == 4) a_min = __reduce_min_sync(kFull, in ? a_low : (MemT)INT32_MAX);
+                                    else a_min = min64(a_low, in);
+                                    in = in && a_low == a_min;
+                                }
                                 const int64_t d_min = min64(du_c, in);
                                 sl = __ffs(__ballot_sync(kFull, in && du_c == d_min)) - 1;
                             }
@@ -460,8 +566,16 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                             const int32_t qd_s = op_s >= 1 ? (int32_t)(at_s & 0x7FFFu) : kEditNone, ji_s = op_s != 1 ? (int32_t)(at_s >> 15 & 0x7FFFu) : kEditNone;
                             const int32_t Tc_s = T + (op_s == 0 ? 1 : 0) - (op_s == 1 ? 1 : 0);
                             int64_t du_s = __shfl_sync(kFull, du_c, sl);
-                            // a proposal within the budget is known: those that are no shorter cannot be better
-                            if (b_has && (int64_t)lds_u64(note + kWalkBestA) == s.M && du_s >= (int64_t)lds_u64(note + kWalkBestD)) break;
+                            // nothing behind the chosen proposal in this order can be better
+                            if constexpr (kFloor) {
+                                if (b_has) {
+                                    const MemT l_s = __shfl_sync(kFull, a_low, sl);
+                                    const int64_t a_s = (int64_t)l_s > s.M ? (int64_t)l_s : s.M, b_a = (int64_t)lds_u64(note + kWalkBestA), b_d = (int64_t)lds_u64(note + kWalkBestD);
+                                    if (a_s > b_a || (a_s == b_a && (du_s > b_d || (du_s == b_d && e0 + sl > b_e)))) break;
+                                }
+                            } else {
+                                if (b_has && (int64_t)lds_u64(note + kWalkBestA) == s.M && du_s >= (int64_t)lds_u64(note + kWalkBestD)) break;
+                            }
                             b_here = false;
                             if (valid) {
                                 shift_words(wa, wb, Tc_s, qd_s, ji_s, x_s, wx_s);
@@ -481,10 +595,11 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                             }
                             bool dep;
                             int32_t at;
-                            const int64_t pk_s = (int64_t)walk_eval<MemT>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, p.split, dep, at);
+                            const int64_t pk_s = (int64_t)walk_eval<MemT, kFloor>(wb, da, rec0, sell0, n_tiles, Tc_s, lane, p.split, dep, at);
                             const int64_t a_s = pk_s > s.M ? pk_s : s.M, b_a = (int64_t)lds_u64(note + kWalkBestA), b_d = (int64_t)lds_u64(note + kWalkBestD);
-                            if (dep || a_s > b_a || (a_s == b_a && (b_has ? du_s >= b_d : du_s > b_d))) continue;
+                            if (dep || a_s > b_a || (a_s == b_a && (du_s > b_d || (du_s == b_d && b_has && (!kFloor || e0 + sl > b_e))))) continue;
                             b_has = b_here = true;
+                            b_e = e0 + sl;
                             __syncwarp();
                             if (lane == 0) {
                                 sts_u64(note + kWalkBestA, (uint64_t)a_s);
@@ -519,7 +634,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             s.dur[c] = (int64_t)lds_u64(note + kWalkDu);
             s.status[c] = pk <= s.M ? 1 : 0;
             s.n_acc[c] += (int32_t)n_acc;
-            p.peak_at[c] = tp;
+            p.peak_at[c] = kFloor ? tp : -tp;
         }
         __syncwarp();
     }

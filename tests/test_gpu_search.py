@@ -434,3 +434,32 @@ def test_search_walk_with_and_without_lists(B, n, P, w_shift, samples):
             assert_state_equal(S, OS, f"n {n}, {g} generations")
     else:
         _run_scored(B, n, edges, w, m, 2, seqs, lens, M, samples, 1, (2, 9), what=f"n {n}")
+
+
+@pytest.mark.parametrize("graph,scale,pct", [("dense", 1, 70), ("layered", 1, 5), ("layered", 1, 80), ("layered", 1 << 36, 80), ("training", 1, 80),
+                                             ("training", 1 << 36, 10**6), ("training", 1, 10**9), ("resnet", 0, 80), ("resnet", 1, 95)])
+def test_search_bound_on_the_new_peak(B, graph, scale, pct):
+    """Proposals refused and ordered by a bound on their peak (from 8 proposals a generation or 257 nodes on) leave the outcome as it is: chains over and
+    within the budget, budgets beyond 32 bits, outputs of size 0, more predecessors than the test keeps apart, changes of the number of proposals,
+    after which the place of the peak may be known less exactly."""
+    if graph == "dense":
+        n, edges, w, m = _layered_dense(33, 3, 5)
+        rng = np.random.default_rng(4)
+        seqs, lens = W.pack([np.concatenate([rng.permutation(33) + 33 * a for a in range(3)]).astype(np.int32) for _ in range(40)])
+    else:
+        n = {"layered": 75, "training": 290, "resnet": 96}[graph]
+        edges = {"layered": lambda: W.layered_dag(n, 3 * n, 8, 7), "training": lambda: W.training_dag(n // 2, n // 2 + 40, 2, 8, 7),
+                 "resnet": lambda: W.resnet_dag(n // 2)}[graph]()
+        w, m = W.weights_uniform(n, 0, 9, 7, 1), W.weights_lognormal(n, 4.0, 1.5, 7, 2) * scale
+        seqs, lens = W.schedules(n, edges, 2, 0.25, 70, 7)
+    G, O = B.Graph(n, edges, w, m, 2), OracleGraph(n, edges, w, m, 2)
+    M = O.eval(np.arange(n), 1 << 60)["peak"] * pct // 100
+    S = B.Search(G, dev(seqs), dev(lens), M, 29)
+    OS = OracleSearch(O, seqs, lens, M, 29, stride=S.info()["stride"])
+    for samples, g in ((32, 3), (1, 33), (8, 13), (3, 12), (40, 6), (9, 11)):
+        S.set_samples(samples, incremental=True)
+        OS.samples = samples
+        S.run(g)
+        OS.run(g)
+        assert_state_equal(S, OS, f"{graph} {pct} %, {samples} proposals, after {OS.generation}")
+    assert OS.accepted > 0
