@@ -42,6 +42,7 @@ struct LaneParent {
     struct View {
         const MemT* p;
         __device__ __forceinline__ MemT operator()(int32_t s) const { return __ldg(p + s); }
+        __device__ __forceinline__ longlong2 vec(int32_t k) const { return __ldg(reinterpret_cast<const longlong2*>(p) + k); }
     };
     __device__ __forceinline__ uint32_t occ(int32_t v) const { return __ldg(occ_ + v); }
     __device__ __forceinline__ int32_t fre(int32_t s) const { return (int32_t)__ldg(fre_ + s); }

@@ -17,7 +17,7 @@
 // built on this when one edit's worst case (4 + 2 * largest in-degree) fits.
 //
 // Parent (per lane): occ(v) the node's copy-position word, fre(s), row(s), prof(s), pm(s), sm(s) of the
-// lane's parent, and prof_view(l), a callable that reads the usage array of lane l's parent.
+// lane's parent, and prof_view(l), which reads the usage array of lane l's parent by step and, as vec(k), by pairs of 64-bit sums.
 // Graph: succ_start(v), pred_start(v), succ(k), pred(k), m(v).
 #pragma once
 #include "moc_edit_kernels.cuh"
@@ -105,6 +105,7 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
     out_st = -2;
     out_win = 0;
     constexpr uint32_t kFull = 0xFFFFFFFFu;
+    constexpr bool kPairs = sizeof(MemT) == 8;      // 64-bit sums: the window by pairs of the parent's steps
     bool go = live && qq < T;
     if (go && pst < 0) { out_st = kStatusParentInvalid; go = false; }
     // ---- per proposal: the edit in parent and child steps
@@ -171,7 +172,7 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
         if (act_mask == 0) break;                   // cannot happen: one proposal's worst case fits
         const int32_t lbase = incl - nd;
         int32_t lcnt = 0, lo_w = kEditNone, hi_w = -1;
-        MemT cross = 0, edge = 0;
+        MemT cross = 0, edge = 0, at_ji = 0;       // at_ji (kPairs): corrections of the inserted step
         if (act) {
             const bool x_sink = ss0 == ss1;
             auto emit = [&](int32_t l, int32_t h, MemT val) {       // += val on child steps l..h
@@ -179,6 +180,7 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
                 rl[lbase + lcnt] = (uint32_t)l | (uint32_t)(h + 1) << 16;
                 rv[lbase + lcnt] = val;
                 ++lcnt;
+                if (kPairs && l <= ji && ji <= h) at_ji += val;
                 lo_w = min(lo_w, l);
                 hi_w = max(hi_w, h);
             };
@@ -277,8 +279,9 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
                     if (x_sink && qd == xb) cross -= Gr.m(x);
                 }
             }
-            // the parent's maxima outside the window
+            // the parent's maxima outside the window, and with kPairs the inserted step
             if (lo_w > 0) edge = P.pm(inv(lo_w - 1));
+            if (kPairs && ji != kEditNone) edge = cross + at_ji > edge ? cross + at_ji : edge;
             if (hi_w < Tc - 1) { const MemT v = P.sm(inv(hi_w + 1)); edge = v > edge ? v : edge; }
         }
         __syncwarp();
@@ -288,34 +291,70 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
             const int32_t lo = __shfl_sync(kFull, lo_w, sl), hi = __shfl_sync(kFull, hi_w, sl);
             const int32_t ji_s = __shfl_sync(kFull, ji, sl), qd_s = __shfl_sync(kFull, qd, sl);
             const int32_t lb = __shfl_sync(kFull, lbase, sl), lc = __shfl_sync(kFull, lcnt, sl);
-            const MemT cr_s = __shfl_sync(kFull, cross, sl);
             const auto view = P.prof_view(sl);
-            // corrections as a difference array over the child steps (zero outside this block of code)
-            for (int32_t k = lane; k < lc; k += 32) {
-                const uint32_t lh = rl[lb + k];
-                const MemT v = rv[lb + k];
-                edit_add(&diff[lh & 0xFFFFu], v);
-                edit_add(&diff[lh >> 16], (MemT)(-v));
+            MemT top;
+            if constexpr (kPairs) {
+                // The corrections and the window in the parent's steps, whose usage is read by 16-byte vectors: a child step stands for
+                // the parent's step that it was, an end on the inserted step for the step behind it; the inserted step itself is in
+                // `edge`, the deleted one is left out.  Step by step each of a warp's reads was spread over the whole window
+                // (n = 900, 8 edits of 3000 parents: 60.8 -> 42.2 us, n = 300, 4 of 4000 22.4 -> 20.6; sums of 32 bits, whose steps lie closer, gained nothing).
+                const int32_t T_s = __shfl_sync(kFull, T, sl);
+                auto inv_s = [&](int32_t t) -> int32_t { const int32_t t1 = t - (t > ji_s ? 1 : 0); return t1 + (t1 >= qd_s ? 1 : 0); };
+                const int32_t end_s = inv_s(hi + 1), v0 = inv_s(lo) >> 1;
+                const int32_t nv = hi < lo ? 0 : ((min(end_s, T_s) + 1) >> 1) - v0, per = (nv + 31) >> 5;
+                const int32_t w0 = v0 + min(nv, lane * per), w1 = v0 + min(nv, (lane + 1) * per);
+                for (int32_t k = lane; k < lc; k += 32) {
+                    const uint32_t lh = rl[lb + k];
+                    const MemT v = rv[lb + k];
+                    edit_add(&diff[inv_s((int32_t)(lh & 0xFFFFu))], v);
+                    edit_add(&diff[inv_s((int32_t)(lh >> 16))], (MemT)(-v));
+                }
+                __syncwarp();
+                MemT run = 0;
+                top = (MemT)INT64_MIN;
+                for (int32_t w = w0; w < w1; ++w) {
+                    const longlong2 use = view.vec(w);
+                    longlong2* const dv = reinterpret_cast<longlong2*>(diff) + w;
+                    const longlong2 d = *dv;
+                    *dv = make_longlong2(0, 0);
+                    run += d.x;
+                    top = 2 * w != qd_s && run + use.x > top ? run + use.x : top;
+                    run += d.y;
+                    top = 2 * w + 1 != qd_s && 2 * w + 1 < T_s && run + use.y > top ? run + use.y : top;
+                }
+                const MemT carry = edit_warp_incl_sum(run, lane) - run;
+                top = top != (MemT)INT64_MIN ? top + carry : (MemT)0;          // usage is never negative: 0 is neutral
+                if (lane == 0 && nv > 0) diff[end_s] = 0;
+            } else {
+                const MemT cr_s = __shfl_sync(kFull, cross, sl);
+                // corrections as a difference array over the child steps (zero outside this block of code)
+                for (int32_t k = lane; k < lc; k += 32) {
+                    const uint32_t lh = rl[lb + k];
+                    const MemT v = rv[lb + k];
+                    edit_add(&diff[lh & 0xFFFFu], v);
+                    edit_add(&diff[lh >> 16], (MemT)(-v));
+                }
+                __syncwarp();
+                // lane owns a run of consecutive window steps (odd length: the runs start in different banks)
+                const int32_t L = hi - lo + 1;
+                const int32_t per = ((L + 31) / 32) | 1;
+                const int32_t t0 = lo + min(L, lane * per), t1 = lo + min(L, (lane + 1) * per);
+                // one pass: running correction and usage relative to the start of the run, then the carry
+                // from the runs in front (max over the run of carry + x = carry + max x)
+                MemT run = 0;
+                top = (MemT)INT32_MIN;
+                const bool any = t0 < t1;
+                for (int32_t t = t0; t < t1; ++t) {
+                    run += diff[t];
+                    diff[t] = 0;
+                    const int32_t tt = t - (t > ji_s ? 1 : 0);
+                    const MemT u = run + (t == ji_s ? cr_s : view(tt + (tt >= qd_s ? 1 : 0)));
+                    top = u > top ? u : top;
+                }
+                const MemT carry = edit_warp_incl_sum(run, lane) - run;
+                top = any ? top + carry : (MemT)0;          // usage is never negative: 0 is neutral
+                if (lane == 0) diff[hi + 1] = 0;
             }
-            __syncwarp();
-            // lane owns a run of consecutive window steps (odd length: the runs start in different banks)
-            const int32_t L = hi - lo + 1;
-            const int32_t per = ((L + 31) / 32) | 1;
-            const int32_t t0 = lo + min(L, lane * per), t1 = lo + min(L, (lane + 1) * per);
-            // one pass: running correction and usage relative to the start of the run, then the carry
-            // from the runs in front (max over the run of carry + x = carry + max x)
-            MemT run = 0, top = sizeof(MemT) == 8 ? (MemT)INT64_MIN : (MemT)INT32_MIN;
-            const bool any = t0 < t1;
-            for (int32_t t = t0; t < t1; ++t) {
-                run += diff[t];
-                diff[t] = 0;
-                const int32_t tt = t - (t > ji_s ? 1 : 0);
-                const MemT u = run + (t == ji_s ? cr_s : view(tt + (tt >= qd_s ? 1 : 0)));
-                top = u > top ? u : top;
-            }
-            const MemT carry = edit_warp_incl_sum(run, lane) - run;
-            top = any ? top + carry : (MemT)0;          // usage is never negative: 0 is neutral
-            if (lane == 0) diff[hi + 1] = 0;
             top = score_warp_max(top);
             if (lane == sl) best = top > best ? top : best;
             __syncwarp();

@@ -255,3 +255,26 @@ def test_build_of_few_and_many_parents(B, n, shift, P):
     seqs, lens = W.mutate(seqs, lens, n, 2, seed=5, frac=1 / 8)
     M = OracleGraph(n, edges, wl.w, wl.m, 2).eval(np.arange(n), BIG)["peak"] * 90 // 100
     run_case(B, wl, seqs, lens, M, *random_edits(np.random.default_rng(P), np.clip(lens, 0, None), 1500), what=f"n {n} P {P}")
+
+
+@pytest.mark.parametrize("n,edges", [(3, []), (5, [(0, 1), (0, 2), (1, 3), (2, 3), (3, 4)]), (6, [(0, 2), (1, 2), (2, 3), (2, 4)]), (33, None), (34, None)])
+def test_edits_by_pairs_of_steps(B, n, edges):
+    """64-bit sums, whose windows are read by pairs of the parent's steps: every edit of sequences of even and odd length, and with one pair a
+    lane and two: insertions in front of the first step and behind the last, the deleted step first or second of a pair."""
+    rng = np.random.default_rng(n)
+    edges = W.layered_dag(n, 2 * n, 5, n) if edges is None else np.array(edges, np.int32).reshape(-1, 2)
+    wl = type("WL", (), dict(n=n, edges=edges, C=2, w=rng.integers(0, 9, n).astype(np.int64), m=rng.integers(1, 20, n).astype(np.int64) << 33))
+    rows = []
+    for extra in (0, 1, 2, n // 2):
+        r = list(range(n))
+        for v in rng.permutation(n)[:extra]:
+            r.insert(int(rng.integers(r.index(v) + 1, len(r) + 1)), int(v))
+        rows.append(r)
+    seqs, lens = W.pack([np.array(r, np.int32) for r in rows])
+    every = [(c, o, q, j) for c, r in enumerate(rows) for o in range(3) for q in range(len(r)) for j in range(len(r) + (o == 0) if o != 1 else 1)]
+    if len(every) > 4000:       # the ends of the sequences and a sample of the rest
+        near = [e for e in every if min(e[2], e[3]) < 2 or max(e[2], e[3]) >= len(rows[e[0]]) - 2]
+        every = [near[k] for k in rng.permutation(len(near))[:2500]] + [every[k] for k in rng.permutation(len(every))[:2500]]
+    parent, op, q, j = (np.array(x, np.int32) for x in zip(*every))
+    want = run_case(B, wl, seqs, lens, int(wl.m.sum()) // 2, parent, op, q, j, what=f"n {n}")
+    assert (want[:, 2] >= 0).any()
