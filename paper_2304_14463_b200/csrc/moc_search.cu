@@ -108,6 +108,10 @@ void plan_walk(moc_search* s) {
     if (wide && !g->split_ok) return;
     const size_t per_vec = wide ? 2 : 4, nvec = ((size_t)g->C * g->n + 2 + per_vec - 1) / per_vec, v_max = ((nvec + 31) / 32) | 1;
     moc::WalkParams& w = s->wp;
+    for (uint32_t r = 0; r < 10; ++r) {
+        w.round_key[2 * r] = s->p.seed_lo + r * moc::kPhiloxWeyl0;
+        w.round_key[2 * r + 1] = s->p.seed_hi + r * moc::kPhiloxWeyl1;
+    }
     w.n = g->n;
     w.C = g->C;
     w.n_tiles = g->n_tiles;

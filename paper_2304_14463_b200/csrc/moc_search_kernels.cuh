@@ -24,18 +24,21 @@ namespace moc {
 
 // Ten rounds of the 4x32 variant: the products of two counter words with the two multipliers are
 // crossed with the other words and the round key, which advances by the two Weyl constants.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
+// `key(r)`: the key of round r.
+constexpr uint32_t kPhiloxWeyl0 = 0x9E3779B9u, kPhiloxWeyl1 = 0xBB67AE85u;
+template <typename Key>
+__device__ __forceinline__ uint4 philox4x32_10_by(uint4 c, Key&& key) {
     constexpr uint32_t kMul0 = 0xD2511F53u, kMul1 = 0xCD9E8D57u;
-    constexpr uint32_t kWeyl0 = 0x9E3779B9u, kWeyl1 = 0xBB67AE85u;
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t hi0 = __umulhi(kMul0, c.x), lo0 = kMul0 * c.x;
-        const uint32_t hi1 = __umulhi(kMul1, c.z), lo1 = kMul1 * c.z;
-        c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
-        k.x += kWeyl0;
-        k.y += kWeyl1;
+        const uint64_t p0 = (uint64_t)kMul0 * c.x, p1 = (uint64_t)kMul1 * c.z;
+        const uint2 k = key(r);
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k.x, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k.y, (uint32_t)p0);
     }
     return c;
+}
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
+    return philox4x32_10_by(c, [&](int r) { return make_uint2(k.x + (uint32_t)r * kPhiloxWeyl0, k.y + (uint32_t)r * kPhiloxWeyl1); });
 }
 
 struct SearchParams {
@@ -75,14 +78,9 @@ constexpr int kSearchThreads = 256;  // 8 chains per block, one warp each
 
 // The (r0 mod k)-th enabled kind of edit, k = number of enabled kinds (order: insert, delete, move).
 __device__ __forceinline__ uint32_t search_pick_kind(uint32_t kinds, uint32_t r0) {
-    uint32_t pick = r0 % (uint32_t)__popc(kinds), op = 0;
-    for (uint32_t o = 0; o < 3; ++o) {
-        if (kinds >> o & 1u) {
-            if (pick == 0) { op = o; break; }
-            --pick;
-        }
-    }
-    return op;
+    const int count = __popc(kinds);        // the (r0 mod count)-th enabled kind
+    if (count == 3) return r0 % 3u;
+    return count == 2 && (r0 & 1u) ? 31u - (uint32_t)__clz((int)kinds) : (uint32_t)__ffs((int)kinds) - 1u;
 }
 
 // Writes the edited copy of src[0..T) to dst with the lanes of one warp: element qd taken out (none:

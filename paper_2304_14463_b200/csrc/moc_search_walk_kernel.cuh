@@ -44,6 +44,7 @@ struct WalkParams {
     int32_t samples;           // E: proposals per chain and generation
     int32_t lanes_per_gen;     // E rounded up to a power of two, at most 32
     int32_t* peak_at;          // P: walk_eval's `at` of each chain's sequence, 0: not known
+    uint32_t round_key[20];    // of the draws: operands from the constant bank instead of twenty additions
     int32_t n, C, n_tiles;
     int32_t split;             // 64-bit sums: as in PairParams
     const void* rec;           // node records and successor tiles of the warp-per-sequence layout
@@ -522,10 +523,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                 {
                     // the lane's draw, kept for the tests after an acceptance; in shared memory, whose 384 bytes a warp leave 28 warps at
                     // n = 442 (drawn again each time: n = 30, 32768 chains x 20 158 -> 150 us, n = 442, 4096 x 20 32.8 -> 31.0)
-                    uint2 key = make_uint2(s.seed_lo, s.seed_hi);
-                    MOC_KEEP(key.x);        // the twenty round keys are not worth holding (and spilling) over the loop
-                    MOC_KEEP(key.y);
-                    const uint4 r = philox4x32_10(make_uint4(s.generation + (uint32_t)(g0 + my_gen), s.chain0 + (uint32_t)c, (uint32_t)(e0 + my_e), 0u), key);
+                    const uint4 r = philox4x32_10_by(make_uint4(s.generation + (uint32_t)(g0 + my_gen), s.chain0 + (uint32_t)c, (uint32_t)(e0 + my_e), 0u),
+                                                     [&](int k) { return make_uint2(p.round_key[2 * k], p.round_key[2 * k + 1]); });
                     sts_u32(note + kWalkDraw + 8u * (uint32_t)lane, r.y);
                     sts_u32(note + kWalkDraw + 8u * (uint32_t)lane + 4u, r.z);
                     sts_u32(note + kWalkKind + 4u * (uint32_t)lane, search_pick_kind(s.kinds, r.x));
