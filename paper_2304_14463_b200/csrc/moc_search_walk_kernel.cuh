@@ -14,7 +14,7 @@
 // evaluated: the key of the chain decides already.
 // With kFloor the test also works out the usage that the edited sequence has at the step where the chain reaches its peak.  The new
 // peak is no lower, which refuses proposals and orders the others: the first of them that reaches its bound ends the generation.  Of 3.3 admissible proposals
-// of 32 0.95 are evaluated (n = 442, over the budget; counted on the CPU), and nearly every one of those is accepted.
+// of 32 0.97 are evaluated (n = 442, over the budget; counted on the CPU), and nearly every one of those is accepted.
 //
 // The sequence itself stays in global memory (L2): the tests read one element per proposal, and an
 // accepted edit shifts the elements between its two places by one.  It is kept there because 3.5 KB per warp
@@ -23,11 +23,12 @@
 // Chains without a valid sequence (status < 0) have no test to rely on: their proposals are evaluated from
 // the written-out order, one generation at a time, until one is valid.
 //
-// Bound: instruction issue (72 % of the slots with 32 proposals a generation, 2000 instructions each) and, for small populations,
+// Bound: instruction issue (76 % of the slots with 32 proposals a generation, 2600 instructions each while the chains are over the budget) and, for small populations,
 // the latency of its dependent shared-memory reads; 28 warps beat 24 and 20 with more registers each, and 30 with fewer.
 // n = 442, state copied out: 4096 chains x 20 generations 436 -> 41.9 us against two kernels per generation that
 // write every proposal out, 38.9 with the neighbours' lists on chip, 37.1 with the words of a sequence from eight loads in flight; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us
-// against a cached evaluation per chain that is rebuilt after every acceptance, 1010 -> 951 with the lists, 870 -> 500 (another GPU 1004 -> 508) with the bound.
+// against a cached evaluation per chain that is rebuilt after every acceptance, 1010 -> 951 with the lists, 870 -> 500 (another GPU 1004 -> 508) with the bound,
+// 508 -> 472 with the draws kept between tests and their keys in the constant bank.
 // Tried: the chain's deltas kept and corrected for the few intervals that an edit changes instead of stages 2 and 3 over all nodes (two more calls and
 // serial chains per evaluation: 503 -> 578 us there, small graphs 20 to 40 % slower; n = 900 gained 20 %).
 #pragma once
@@ -445,7 +446,7 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                 if (now != then) change = now ? size_of(x) : -size_of(x);
             }
             // A predecessor that loses a consumer: qd lies behind tp in the range of its copy, ji does not, and no other consumer does.
-            // What one gains is left out (0.95 instead of 0.92 evaluations a generation, for less than half of the lists to go through).
+            // What one gains is left out (0.97 instead of 0.95 evaluations a generation, for less than half of the lists to go through).
             if (qd >= tp && qd != kEditNone) {
                 const int32_t j_won = thr >= tp ? thr : 0x8000;
                 uint32_t rest = 0xFFFFFFFFu;            // the copies of x that stay
