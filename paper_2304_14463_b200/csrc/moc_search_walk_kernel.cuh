@@ -72,7 +72,7 @@ constexpr uint32_t kWalkQd = 0, kWalkJi = 4, kWalkX = 8, kWalkWx = 12;          
 constexpr uint32_t kWalkBestA = 16, kWalkBestD = 24, kWalkBestPk = 32;           // its key and peak (without one: the chain's key)
 constexpr uint32_t kWalkBestAt = 40, kWalkAcc = 44, kWalkPk = 48, kWalkDu = 56;  // its `at`; the chain: accepted, peak, duration
 constexpr uint32_t kWalkDraw = 64, kWalkKind = 64 + 256;                          // the lanes' draws: {r1, r2}, kind of the edit
-constexpr uint32_t kWalkNoteBytes = 64 + 384;
+constexpr uint32_t kWalkDrawBytes = 384, kWalkNoteBytes = 64 + kWalkDrawBytes;
 
 // Bytes of one warp: two sets of words, each followed by the constant word, the scalars, and the deltas.
 __host__ __device__ inline size_t walk_warp_bytes(uint32_t word_bytes, uint32_t delta_bytes) {
