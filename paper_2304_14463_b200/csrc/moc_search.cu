@@ -130,7 +130,7 @@ void plan_walk(moc_search* s) {
     w.delta_bytes = (uint32_t)(moc::kPairDeltaFront + 32 * v_max * 16);
     const size_t warp_b = moc::walk_warp_bytes(w.word_bytes, w.delta_bytes), graph_b = (size_t)w.rec_bytes + w.sell_bytes;
     const size_t cap = g->smem_optin;
-    if (graph_b + 4 * (warp_b - moc::kWalkDrawBytes) > cap) return;      // (four warps but for the draws: three then)
+    if (graph_b + 4 * warp_b > cap) return;
     // Chains that fit the device at once get one round with as few warps per SM as that takes; larger
     // populations the shape with the smallest rounds * (warps + 10): a round is a chain's latency and the SM's work.
     const int sm = g->sm_count, most = (int)std::min<size_t>(moc::kWalkThreads / 32, (cap - graph_b) / warp_b);

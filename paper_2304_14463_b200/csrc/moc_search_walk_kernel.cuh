@@ -71,8 +71,7 @@ struct WalkParams {
 constexpr uint32_t kWalkQd = 0, kWalkJi = 4, kWalkX = 8, kWalkWx = 12;           // the chosen proposal
 constexpr uint32_t kWalkBestA = 16, kWalkBestD = 24, kWalkBestPk = 32;           // its key and peak (without one: the chain's key)
 constexpr uint32_t kWalkBestAt = 40, kWalkAcc = 44, kWalkPk = 48, kWalkDu = 56;  // its `at`; the chain: accepted, peak, duration
-constexpr uint32_t kWalkDraw = 64, kWalkKind = 64 + 256;                          // the lanes' draws: {r1, r2}, kind of the edit
-constexpr uint32_t kWalkDrawBytes = 384, kWalkNoteBytes = 64 + kWalkDrawBytes;
+constexpr uint32_t kWalkNoteBytes = 64;
 
 // Bytes of one warp: two sets of words, each followed by the constant word, the scalars, and the deltas.
 __host__ __device__ inline size_t walk_warp_bytes(uint32_t word_bytes, uint32_t delta_bytes) {
@@ -521,21 +520,23 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             fresh();
             for (int32_t e0 = 0; e0 < E; e0 += 32) {
                 const uint32_t drawn = __ballot_sync(kFull, g0 + my_gen < p.n_gen && e0 + my_e < E);
+                // The lane's draw {r1, r2, kind of the edit}, kept for the tests after an acceptance (drawn again each time: n = 30, 32768 chains x 20
+                // 158 -> 150 us, n = 442, 4096 x 20 32.8 -> 31.0).  In the lane's own memory (volatile: not in registers over the evaluations): 384 bytes
+                // of shared memory a warp take as long at n = 442, but cost others a warp, that is a round of chains, or the lists (32 proposals x 10: n = 790,
+                // 64-bit sums, 1600 chains 250 -> 176 us, n = 620, 8000 395 -> 360; one proposal 79 -> 57 and 110 -> 102).
+                volatile uint32_t draw[3];
                 {
-                    // the lane's draw, kept for the tests after an acceptance; in shared memory, whose 384 bytes a warp leave 28 warps at
-                    // n = 442 (drawn again each time: n = 30, 32768 chains x 20 158 -> 150 us, n = 442, 4096 x 20 32.8 -> 31.0)
                     const uint4 r = philox4x32_10_by(make_uint4(s.generation + (uint32_t)(g0 + my_gen), s.chain0 + (uint32_t)c, (uint32_t)(e0 + my_e), 0u),
                                                      [&](int k) { return make_uint2(p.round_key[2 * k], p.round_key[2 * k + 1]); });
-                    sts_u32(note + kWalkDraw + 8u * (uint32_t)lane, r.y);
-                    sts_u32(note + kWalkDraw + 8u * (uint32_t)lane + 4u, r.z);
-                    sts_u32(note + kWalkKind + 4u * (uint32_t)lane, search_pick_kind(s.kinds, r.x));
+                    draw[0] = r.y;
+                    draw[1] = r.z;
+                    draw[2] = search_pick_kind(s.kinds, r.x);
                 }
                 uint32_t pending = drawn;
                 while (pending && T > 0) {
                     // ---- the pending proposals against the present sequence, a lane each
-                    const uint2 r = lds_v2(note + kWalkDraw + 8u * (uint32_t)lane);
-                    const int32_t op = (int32_t)lds_u32(note + kWalkKind + 4u * (uint32_t)lane);
-                    const int32_t q = (int32_t)(r.x % (uint32_t)T), j = (int32_t)(r.y % ((uint32_t)T + (op == 0 ? 1u : 0u)));
+                    const int32_t op = (int32_t)draw[2];
+                    const int32_t q = (int32_t)(draw[0] % (uint32_t)T), j = (int32_t)(draw[1] % ((uint32_t)T + (op == 0 ? 1u : 0u)));
                     const int32_t qd = op >= 1 ? q : kEditNone, ji = op != 1 ? j : kEditNone;
                     const int32_t Tc = T + (op == 0 ? 1 : 0) - (op == 1 ? 1 : 0);
                     const int32_t x = row[q];

@@ -39,7 +39,7 @@ std::map<const void*, std::string>& names() {        // kernels register themsel
     return m;
 }
 std::vector<Range> g_pinned;
-std::string g_log;
+std::string g_log, g_shapes;
 int g_calls = 0, g_fail_at = 0, g_next_handle = 1;
 int g_news = 0, g_new_fails_at = 0, g_quiet = 0;
 struct Quiet {      // allocations of the stand-in itself neither count nor fail
@@ -91,11 +91,14 @@ void fake_reset(int fail_at) {
     g_streams.clear();
     g_events.clear();
     g_log.clear();
+    g_shapes.clear();
     g_calls = 0;
     g_fail_at = fail_at;
 }
 int fake_calls() { return g_calls; }
 const char* fake_log() { return g_log.c_str(); }
+// "<kernel> <blocks> <threads> <dynamic shared memory>" of every launch by cudaLaunchKernel
+const char* fake_shapes() { return g_shapes.c_str(); }
 int fake_in_flight() {
     int k = 0;
     for (const Op& o : g_ops) k += !o.done;
@@ -214,9 +217,10 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* nb, const void* f
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* nb, const void* fn, int threads, size_t smem, unsigned) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, threads, smem);
 }
-cudaError_t cudaLaunchKernel(const void* fn, dim3, dim3, void**, size_t, cudaStream_t st) {
+cudaError_t cudaLaunchKernel(const void* fn, dim3 grid, dim3 block, void**, size_t smem, cudaStream_t st) {
     Quiet quiet;
     note("launch " + name_of(fn));
+    g_shapes += name_of(fn) + " " + std::to_string(grid.x) + " " + std::to_string(block.x) + " " + std::to_string(smem) + "\n";
     if (fails()) return cudaErrorUnknown;
     return enqueue(st, "launch"), cudaSuccess;
 }

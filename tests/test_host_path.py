@@ -23,7 +23,7 @@ def fake(tmp_path_factory):
                     "-Xcompiler", "-fPIC", "-Xlinker", "-Bsymbolic,--no-undefined", "-t", "8", "-o", lib,
                     *[os.path.join(build.CSRC, f) for f in build.SOURCES], os.path.join(HERE, "fake_cudart.cpp")], check=True)
     L = ctypes.CDLL(lib)
-    L.fake_log.restype = L.fake_modules.restype = ctypes.c_char_p
+    L.fake_log.restype = L.fake_modules.restype = L.fake_shapes.restype = ctypes.c_char_p
     L.fake_pin.argtypes = [P, ctypes.c_size_t]
     L.moc_last_error.restype = ctypes.c_char_p
     L.moc_graph_create.argtypes = [i32, i64, P, P, P, ctypes.POINTER(P)]
@@ -34,6 +34,7 @@ def fake(tmp_path_factory):
     L.moc_graph_set_node_caps.argtypes = [P, P]
     L.moc_search_create.argtypes = [P, P, P, i32, i64, ctypes.c_uint64, ctypes.c_uint32, P, ctypes.POINTER(P)]
     L.moc_search_set_samples.argtypes = [P, i32, i32]
+    L.moc_search_run.argtypes = [P, i32, P]
     L.moc_search_destroy.argtypes = [P]
     L.moc_search_destroy.restype = None
     L.moc_mem_profile.argtypes = [P, P, i32, P, P, P, P]
@@ -359,3 +360,36 @@ def test_host_allocations_that_fail(fake, n, scale, star):
         assert fake.fake_allocations() == 0
     G.close()
     assert k > (10 if n > 1 else 3)
+
+
+class Search:
+    def __init__(self, L, G, chains, samples=1):
+        self.L, self.h, self.chains = L, P(), chains
+        lens = np.full(chains, G.n, np.int32)
+        assert L.moc_search_create(G.h, lens.ctypes.data, lens.ctypes.data, chains, 0, 1, 0, None, ctypes.byref(self.h)) == 0
+        if samples > 1:
+            assert L.moc_search_set_samples(self.h, samples, 1) == 0
+
+    def launches(self):
+        """(kernel, warps of a block, rounds of chains) of the launches of one generation."""
+        self.L.fake_reset(0)
+        assert self.L.moc_search_run(self.h, 1, None) == 0
+        rows = [x.split() for x in self.L.fake_shapes().decode().splitlines()]
+        return [(k, int(t) // 32, -(-self.chains // (int(b) * int(t) // 32))) for k, b, t, _ in rows]
+
+    def close(self):
+        self.L.moc_search_destroy(self.h)
+
+
+# what fits an SM beside the graph when a warp holds two sets of words, 64 bytes of scalars and the deltas
+@pytest.mark.parametrize("n,scale,chains,warps,rounds", [(442, 1, 4096, 28, 1), (500, 1, 3700, 25, 1), (600, 1, 3000, 21, 1), (940, 1, 4000, 14, 2), (990, 1, 3700, 13, 2),
+                                                         (390, 1 << 30, 16000, 22, 5), (450, 1 << 30, 8000, 19, 3), (780, 1 << 30, 1600, 11, 1), (930, 1 << 30, 3700, 9, 3),
+                                                         (2990, 1, 592, 4, 1)])
+@pytest.mark.parametrize("samples", [1, 32])
+def test_rounds_of_a_search(fake, n, scale, chains, warps, rounds, samples):
+    G = Graph(fake, n, 2, scale)
+    S = Search(fake, G, chains, samples)
+    (kernel, *shape), = S.launches()
+    assert "search_walk_kernel" in kernel and shape == [warps, rounds]
+    S.close()
+    G.close()
