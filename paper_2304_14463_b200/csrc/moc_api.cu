@@ -661,7 +661,8 @@ void build_tables(moc_graph* g, const std::vector<uint64_t>& keys, const std::ve
                 lists[list + k] = (uint16_t)pred[k];
             }
             for (int32_t v = 0; v < n; ++v) near[2 * ((size_t)n + 1) + list + (size_t)v] = (uint32_t)m32[v];
-            g->near_bytes = near.size() * 4;
+            g->near_bytes = (4 * (2 * ((size_t)n + 1) + list) + 15) & ~size_t(15);
+            g->near_size_bytes = near.size() * 4;
             tables->add(&g->d_near, std::move(near));
         }
         tables->add(&g->d_pred_start, std::move(pred_start));

@@ -133,7 +133,8 @@ struct moc_graph {
     int32_t* d_pred_start = nullptr;     // predecessor lists (CSR), for the incremental evaluation
     int32_t* d_pred = nullptr;
     uint32_t* d_near = nullptr;           // both lists with 16 bits an entry, for the search: per node {first successor | first predecessor << 16,
-    size_t near_bytes = 0;                // duration}, the successors, the predecessors, m32 (null: more than 65535 edges, or durations of 2^31)
+                                          // duration}, the successors, the predecessors, m32 (null: more than 65535 edges, or durations of 2^31)
+    size_t near_bytes = 0, near_size_bytes = 0;      // without m32, with it
     int64_t sink_m = 0;                   // sum of m over the nodes without successors
     int32_t max_indeg = 0;                // largest number of predecessors of a node
     int64_t* d_w = nullptr;

@@ -42,8 +42,9 @@ struct moc_search {
     const void* walk_fn_floor = nullptr;     // the same with the bound on the new peak
     bool walk_planned = false;
     bool walk_scores = false;          // incremental, and the walk kernel does it (no cache)
+    bool walk_sizes = false;           // with the bound on the new peak, the output sizes lie on chip
     int walk_wpb = 0, walk_grid = 0;
-    size_t walk_smem = 0;
+    size_t walk_smem = 0, walk_smem_floor = 0;
 };
 
 namespace {
@@ -141,12 +142,14 @@ void plan_walk(moc_search* s) {
         const int64_t cost = rounds * (k + 10);
         if (best == 0 || cost < best_cost) { best = k; best_cost = cost; }
     }
-    // the neighbours' lists where they fit beside that many warps
+    // the neighbours' lists where they fit beside that many warps (10 generations, with / without: 64-bit sums, n = 510, 16000 chains x 32 809 / 878 us, n = 600,
+    // 8000 x 1 135 / 145, n = 430 x 32 the same; 32-bit sums, n = 620, 8000 x 1 102 / 110); behind them, where they fit too, the output sizes for the one
+    // variant that reads them from there (32-bit sums, bound on the new peak).  Copied and counted for all, their 4 n bytes displaced lists.
     w.n_edges = (int32_t)g->n_edges;
-    const size_t list_b = g->near_bytes;
-    const bool lists = g->d_near != nullptr && graph_b + list_b + (size_t)best * warp_b <= cap;
+    const size_t used = graph_b + (size_t)best * warp_b;
+    const bool lists = g->d_near != nullptr && used + g->near_bytes <= cap;
+    s->walk_sizes = lists && !wide && used + g->near_size_bytes <= cap;
     w.lists = g->d_near;
-    w.list_bytes = (uint32_t)list_b;
     const void* const fn[2] = {walk_fn(wide, lists, false), walk_fn(wide, lists, true)};
     for (const void* f : fn)
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
@@ -155,7 +158,8 @@ void plan_walk(moc_search* s) {
         }
     s->walk_wpb = best;
     s->walk_grid = (int)std::min<int64_t>(sm, ((int64_t)s->P + best - 1) / best);
-    s->walk_smem = graph_b + (lists ? list_b : 0) + (size_t)best * warp_b;
+    s->walk_smem = used + (lists ? g->near_bytes : 0);
+    s->walk_smem_floor = s->walk_sizes ? used + g->near_size_bytes : s->walk_smem;
     s->walk_fn = fn[0];
     s->walk_fn_floor = fn[1];
 }
@@ -287,13 +291,15 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
         // them is evaluated then) or expensive evaluations.  With / without, 10 generations: n = 30, E = 32, 20000 chains 243 / 287 us, n = 78, E = 8, 255
         // chains 20.6 / 23.4, n = 260, E = 8, 8000 chains 63 / 93; n = 442, E = 1, 4096 chains x 20 32.8 / 38.2.  No gain: n = 200, E = 8, a layered
         // graph 212 / 201, n = 300, E = 1 the same; n = 30, E = 1 158 / 149.
-        const void* fn = s->samples >= 8 || g->n_tiles > 4 ? s->walk_fn_floor : s->walk_fn;
+        const bool floor = s->samples >= 8 || g->n_tiles > 4;
+        w.sizes = floor && s->walk_sizes;
+        w.list_bytes = (uint32_t)(w.sizes ? g->near_size_bytes : g->near_bytes);
         for (int32_t k = 0; k < n_generations; k += most) {
             w.s = p;
             w.s.generation = s->generation + (uint32_t)k;
             w.n_gen = std::min(most, n_generations - k);
             void* args[] = {&w};
-            MOC_CUDA(cudaLaunchKernel(fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, s->walk_smem, st));
+            MOC_CUDA(cudaLaunchKernel(floor ? s->walk_fn_floor : s->walk_fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, floor ? s->walk_smem_floor : s->walk_smem, st));
             ++launches;
         }
         s->generation += (uint32_t)n_generations;

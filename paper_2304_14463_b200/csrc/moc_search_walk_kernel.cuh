@@ -60,7 +60,8 @@ struct WalkParams {
     uint32_t rec_bytes, sell_bytes;      // graph, once per block
     int32_t n_edges;
     const uint32_t* lists;     // kLists: the neighbours' lists (walk_lists), behind the graph in shared memory
-    uint32_t list_bytes;
+    uint32_t list_bytes;                 // of the lists, with m behind them where `sizes`
+    int32_t sizes;
     uint32_t word_bytes;       // occurrence words (n + 2, padded) without the constant word behind them
     uint32_t delta_bytes;      // front pad + deltas for C * n steps
 };
@@ -262,8 +263,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
     if constexpr (kLists) MOC_STAGED(l_node);
     const uint32_t l_succ = l_node + 8u * (uint32_t)(p.n + 1), l_pred = l_succ + 2u * (uint32_t)((p.n_edges + 3) & ~3), l_size = l_pred + 2u * (uint32_t)((p.n_edges + 3) & ~3);
     auto size_of = [&](int32_t v) -> MemT {
-        if constexpr (kLists && sizeof(MemT) == 4) return (MemT)lds_u32_nv(l_size + 4u * (uint32_t)v);
-        else return (MemT)__ldg(p.m + v);
+        if (kLists && sizeof(MemT) == 4 && p.sizes) return (MemT)lds_u32_nv(l_size + 4u * (uint32_t)v);
+        return (MemT)__ldg(p.m + v);
     };
     auto successors = [&](int32_t v, int32_t& from, int32_t& to) {
         if constexpr (kLists) {

@@ -370,12 +370,12 @@ class Search:
         if samples > 1:
             assert L.moc_search_set_samples(self.h, samples, 1) == 0
 
-    def launches(self):
-        """(kernel, warps of a block, rounds of chains) of the launches of one generation."""
+    def launches(self, generations=1):
+        """(kernel, warps of a block, rounds of chains, bytes of shared memory) of the launches of a run."""
         self.L.fake_reset(0)
-        assert self.L.moc_search_run(self.h, 1, None) == 0
+        assert self.L.moc_search_run(self.h, generations, None) == 0
         rows = [x.split() for x in self.L.fake_shapes().decode().splitlines()]
-        return [(k, int(t) // 32, -(-self.chains // (int(b) * int(t) // 32))) for k, b, t, _ in rows]
+        return [(k, int(t) // 32, -(-self.chains // (int(b) * int(t) // 32)), int(smem)) for k, b, t, smem in rows]
 
     def close(self):
         self.L.moc_search_destroy(self.h)
@@ -389,7 +389,34 @@ class Search:
 def test_rounds_of_a_search(fake, n, scale, chains, warps, rounds, samples):
     G = Graph(fake, n, 2, scale)
     S = Search(fake, G, chains, samples)
-    (kernel, *shape), = S.launches()
+    (kernel, *shape, _), = S.launches()
     assert "search_walk_kernel" in kernel and shape == [warps, rounds]
     S.close()
     G.close()
+
+
+# the neighbours' lists fit beside the chains, but not the lists and n output sizes (and at the last three not even the lists)
+@pytest.mark.parametrize("n,scale,chains,lists", [(490, 1, 3700, 1), (660, 1, 8000, 1), (770, 1, 16000, 1), (850, 1, 4000, 1), (2950, 1, 400, 1), (380, 1 << 30, 16000, 1), (440, 1 << 30, 8000, 1),
+                                                  (540, 1 << 30, 16000, 1), (620, 1 << 30, 3700, 1), (870, 1 << 30, 3700, 1), (980, 1 << 30, 8000, 1),
+                                                  (500, 1, 3700, 0), (390, 1 << 30, 16000, 0), (780, 1 << 30, 1600, 0)])
+@pytest.mark.parametrize("samples", [1, 32])
+def test_lists_of_a_search_on_chip(fake, n, scale, chains, lists, samples):
+    G = Graph(fake, n, 2, scale)
+    S = Search(fake, G, chains, samples)
+    (kernel, *_), = S.launches()
+    assert f"search_walk_kernelI{'l' if scale > 1 else 'i'}Lb{lists}E" in kernel
+    S.close()
+    G.close()
+
+
+def test_sizes_go_on_chip_for_the_variant_that_reads_them(fake):
+    """32-bit sums with the bound on the new peak, where they fit behind the lists."""
+    for n, scale, chains, more in ((200, 1, 4000, 4 * 200), (490, 1, 3700, 0), (200, 1 << 30, 4000, 0)):
+        G = Graph(fake, n, 2, scale)
+        smem = {}
+        for samples in (1, 32):
+            S = Search(fake, G, chains, samples)
+            (kernel, _, _, smem[samples]), = S.launches()
+            S.close()
+        assert more - 16 < smem[32] - smem[1] <= (more + 16 if more else 0), (n, scale, smem)
+        G.close()
