@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmoc_b200.so")
 SOURCES = ["moc_api.cu", "moc_search.cu", "moc_intervals.cu", "moc_edits.cu", "moc_eval_general.cu", "moc_eval_pair.cu", "moc_eval_lane.cu",
-           "moc_eval_quad.cu", "moc_eval_quad_warp.cu", "moc_eval_live.cu", "moc_check_plain.cu", "moc_check_general.cu", "moc_check_staged.cu", "moc_search_score.cu", "moc_search_walk.cu"]
+           "moc_eval_quad.cu", "moc_eval_quad_warp.cu", "moc_eval_live.cu", "moc_check_plain.cu", "moc_check_general.cu", "moc_check_staged.cu", "moc_search_score.cu", "moc_search_walk.cu", "moc_search_walk_floor.cu"]
 HEADERS = ["moc_kernels.cuh", "moc_pair_kernel.cuh", "moc_lane_kernel.cuh", "moc_quad_kernel.cuh", "moc_live_kernel.cuh", "moc_host.cuh", "moc_search_kernels.cuh", "moc_search_score_kernel.cuh", "moc_search_walk_kernel.cuh", "moc_edit_pass.cuh", "moc_edit_lanes_kernel.cuh", "moc_interval_kernels.cuh", "moc_interval_plain_kernel.cuh", "moc_edit_kernels.cuh", "moc_cache_host.cuh", os.path.join("..", "..", "include", "moc.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-shared", "--use_fast_math"]

@@ -38,7 +38,8 @@ const void* check_plain_fn(bool wide);
 IntervalFn check_general_fn(int cp, bool wide, int kept, bool team);      // kept: bytes per event of the solution kept on chip, 0: not kept
 IntervalFn check_staged_fn(int cp, bool wide, int kept, bool team);      // team: a block per solution
 const void* score_fn(bool wide, bool graph_on_chip);
-const void* walk_fn(bool wide, bool lists, bool floor);      // lists: the neighbours' lists in shared memory; floor: its test bounds the new peak
+const void* walk_fn(bool wide, bool lists);      // lists: the neighbours' lists in shared memory
+const void* walk_floor_fn(bool wide, bool lists);      // its test bounds the new peak
 
 constexpr int kHostParts = 3;          // parts in which the host entry points send a large batch
 

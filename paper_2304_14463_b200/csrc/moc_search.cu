@@ -38,9 +38,9 @@ struct moc_search {
     // all generations of a call in one kernel (moc_search_walk_kernel.cuh)
     uint64_t graph_generation = 0;     // the graph's C and caps when the chains were evaluated
     moc::WalkParams wp{};
-    const void* walk_fn = nullptr;     // null: not planned yet, or the graph does not fit (walk_planned)
-    const void* walk_fn_floor = nullptr;     // the same with the bound on the new peak
-    bool walk_planned = false;
+    bool walk_planned = false, walk_fits = false;
+    bool walk_wide = false, walk_lists = false;
+    const void* walk_fn[2] = {};       // without and with the bound on the new peak; null: not prepared (walk_variant)
     bool walk_scores = false;          // incremental, and the walk kernel does it (no cache)
     bool walk_sizes = false;           // with the bound on the new peak, the output sizes lie on chip
     int walk_wpb = 0, walk_grid = 0;
@@ -98,11 +98,11 @@ bool plan_fused(moc_search* s) {
     return true;
 }
 
-// Launch shape of the kernel that takes a warp per chain through all generations; leaves walk_fn null when the
+// Launch shape of the kernel that takes a warp per chain through all generations; leaves walk_fits false when the
 // graph has no warp-per-sequence layout (C > 2, very uneven degrees) or fewer than four warps fit an SM.
 void plan_walk(moc_search* s) {
     s->walk_planned = true;
-    s->walk_fn = nullptr;
+    s->walk_fits = false;
     const moc_graph* g = s->g;
     if (g->C > 2 || g->d_rec32 == nullptr) return;
     const bool wide = g->sum_m > (int64_t)INT32_MAX / g->C;
@@ -150,18 +150,33 @@ void plan_walk(moc_search* s) {
     const bool lists = g->d_near != nullptr && used + g->near_bytes <= cap;
     s->walk_sizes = lists && !wide && used + g->near_size_bytes <= cap;
     w.lists = g->d_near;
-    const void* const fn[2] = {walk_fn(wide, lists, false), walk_fn(wide, lists, true)};
-    for (const void* f : fn)
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap) != cudaSuccess) {
-            cudaGetLastError();
-            return;
-        }
+    s->walk_wide = wide;
+    s->walk_lists = lists;
     s->walk_wpb = best;
     s->walk_grid = (int)std::min<int64_t>(sm, ((int64_t)s->P + best - 1) / best);
     s->walk_smem = used + (lists ? g->near_bytes : 0);
     s->walk_smem_floor = s->walk_sizes ? used + g->near_size_bytes : s->walk_smem;
-    s->walk_fn = fn[0];
-    s->walk_fn_floor = fn[1];
+    s->walk_fits = true;
+}
+
+// Whether the next generations are tested with a bound on the new peak: where enough evaluations fall away for what it costs, with many proposals of a
+// generation (one in three of them is evaluated then) or expensive evaluations.  With / without, 10 generations: n = 30, E = 32, 20000 chains 243 / 287 us, n = 78, E = 8, 255
+// chains 20.6 / 23.4, n = 260, E = 8, 8000 chains 63 / 93; n = 442, E = 1, 4096 chains x 20 32.8 / 38.2.  No gain: n = 200, E = 8, a layered
+// graph 212 / 201, n = 300, E = 1 the same; n = 30, E = 1 158 / 149.
+bool walk_floor(const moc_search* s) { return s->samples >= 8 || s->g->n_tiles > 4; }
+
+// The variant to launch, prepared when it is first asked for: preparing loads it.  Null: it cannot be.
+const void* walk_variant(moc_search* s, bool floor) {
+    if (!s->walk_fits) return nullptr;
+    if (!s->walk_fn[floor]) {
+        const void* f = floor ? walk_floor_fn(s->walk_wide, s->walk_lists) : walk_fn(s->walk_wide, s->walk_lists);
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->g->smem_optin) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        s->walk_fn[floor] = f;
+    }
+    return s->walk_fn[floor];
 }
 
 // Proposals per chain of one launch: enough that the launch does not show, few enough for a caller who waits.
@@ -279,19 +294,17 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
         return fail(MOC_ERR_ARG, "moc_search_run: the graph's C or node caps changed after the search's chains were evaluated");
     if (!s->walk_planned) plan_walk(s);
     if (s->incremental ? s->walk_scores
-                       : s->walk_fn && g->generation == s->graph_generation && g->want_G == 0 &&
-                             (g->want_kind == MOC_KERNEL_AUTO || g->want_kind == MOC_KERNEL_WARP)) {
+                       : s->walk_fits && g->generation == s->graph_generation && g->want_G == 0 &&
+                             (g->want_kind == MOC_KERNEL_AUTO || g->want_kind == MOC_KERNEL_WARP) && walk_variant(s, walk_floor(s))) {
         moc::WalkParams& w = s->wp;
         w.samples = s->samples;
         w.lanes_per_gen = 1;
         while (w.lanes_per_gen < std::min(s->samples, 32)) w.lanes_per_gen *= 2;
         w.cap = g->d_cap;
         const int32_t most = std::max(1, kWalkProposals / s->samples);
-        // With a bound on the new peak where enough evaluations fall away for what it costs: many proposals of a generation (one in three of
-        // them is evaluated then) or expensive evaluations.  With / without, 10 generations: n = 30, E = 32, 20000 chains 243 / 287 us, n = 78, E = 8, 255
-        // chains 20.6 / 23.4, n = 260, E = 8, 8000 chains 63 / 93; n = 442, E = 1, 4096 chains x 20 32.8 / 38.2.  No gain: n = 200, E = 8, a layered
-        // graph 212 / 201, n = 300, E = 1 the same; n = 30, E = 1 158 / 149.
-        const bool floor = s->samples >= 8 || g->n_tiles > 4;
+        const bool floor = walk_floor(s);
+        const void* const fn = walk_variant(s, floor);
+        if (!fn) return fail(MOC_ERR_CUDA, "moc_search_run: the search kernel cannot be prepared");
         w.sizes = floor && s->walk_sizes;
         w.list_bytes = (uint32_t)(w.sizes ? g->near_size_bytes : g->near_bytes);
         for (int32_t k = 0; k < n_generations; k += most) {
@@ -299,7 +312,7 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
             w.s.generation = s->generation + (uint32_t)k;
             w.n_gen = std::min(most, n_generations - k);
             void* args[] = {&w};
-            MOC_CUDA(cudaLaunchKernel(floor ? s->walk_fn_floor : s->walk_fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, floor ? s->walk_smem_floor : s->walk_smem, st));
+            MOC_CUDA(cudaLaunchKernel(fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, floor ? s->walk_smem_floor : s->walk_smem, st));
             ++launches;
         }
         s->generation += (uint32_t)n_generations;
@@ -407,11 +420,16 @@ int moc_search_set_samples(moc_search* s, int32_t samples, int32_t incremental) 
                         "evaluation starts from valid sequences only", c, st[c]);
     // by default the kernel that takes a warp per chain through all generations (no cache), where the graph fits it
     if (!s->walk_planned) plan_walk(s);
-    s->walk_scores = incremental == MOC_SEARCH_SCORE_AUTO && s->walk_fn && s->g->generation == s->graph_generation;
-    if (s->walk_scores) {
+    s->walk_scores = false;
+    if (incremental == MOC_SEARCH_SCORE_AUTO && s->walk_fits && s->g->generation == s->graph_generation) {
+        const int32_t before = s->samples;
         s->samples = samples;
-        s->incremental = true;
-        return MOC_OK;
+        if (walk_variant(s, walk_floor(s))) {
+            s->walk_scores = true;
+            s->incremental = true;
+            return MOC_OK;
+        }
+        s->samples = before;
     }
     if (!s->cache) {
         moc_cache* h = nullptr;

@@ -390,7 +390,7 @@ def test_rounds_of_a_search(fake, n, scale, chains, warps, rounds, samples):
     G = Graph(fake, n, 2, scale)
     S = Search(fake, G, chains, samples)
     (kernel, *shape, _), = S.launches()
-    assert "search_walk_kernel" in kernel and shape == [warps, rounds]
+    assert "search_walk_" in kernel and shape == [warps, rounds]
     S.close()
     G.close()
 
@@ -404,7 +404,7 @@ def test_lists_of_a_search_on_chip(fake, n, scale, chains, lists, samples):
     G = Graph(fake, n, 2, scale)
     S = Search(fake, G, chains, samples)
     (kernel, *_), = S.launches()
-    assert f"search_walk_kernelI{'l' if scale > 1 else 'i'}Lb{lists}E" in kernel
+    assert f"kernelI{'l' if scale > 1 else 'i'}Lb{lists}E" in kernel
     S.close()
     G.close()
 
@@ -420,3 +420,25 @@ def test_sizes_go_on_chip_for_the_variant_that_reads_them(fake):
             S.close()
         assert more - 16 < smem[32] - smem[1] <= (more + 16 if more else 0), (n, scale, smem)
         G.close()
+
+
+@pytest.mark.parametrize("n,samples", [(100, 1), (100, 7), (100, 8), (300, 8)])
+def test_a_search_prepares_the_variant_that_it_launches(fake, n, samples):
+    """With and without the bound on the new peak lie in two modules, of which a search loads the one that it launches; another number
+    of proposals prepares its own when it is set."""
+    modules = fake.fake_modules().decode().splitlines()
+    for f in ("search_walk_kernel", "search_walk_floor_kernel"):
+        assert sum(f in m for m in modules) == 1
+    assert not any("search_walk_kernel" in m and "search_walk_floor_kernel" in m for m in modules)
+    G = Graph(fake, n)
+    for k in (samples, 32, 1):
+        fake.fake_reset(0)
+        S = Search(fake, G, 300, k)
+        before = {x.split()[1] for x in log(fake) if x.startswith("lookup ") and "search_walk" in x}
+        (kernel, *_), = S.launches()
+        assert before == ({kernel} if k > 1 else set())
+        assert {x.split()[1] for x in log(fake) if x.startswith("lookup ")} == ({kernel} if k == 1 else set())
+        S.launches()
+        assert not [x for x in log(fake) if x.startswith("lookup ")]
+        S.close()
+    G.close()
