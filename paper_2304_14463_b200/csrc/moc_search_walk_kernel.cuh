@@ -221,7 +221,7 @@ static __device__ __noinline__ void walk_apply(int32_t* row, int32_t T, int32_t 
 // kLists: the test of a proposal reads the neighbours' lists from the block's shared memory (durations below 2^31, at most 65535 edges);
 // through L1, of which the chains' state leaves little, a third of the kernel's stalls were waits for them.
 template <typename MemT, bool kLists, bool kFloor>
-__device__ __forceinline__ void search_walk(const WalkParams& p) {
+__global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const WalkParams p) {
     extern __shared__ __align__(16) char smem[];
     const SearchParams& s = p.s;
     constexpr uint32_t kRecB = sizeof(MemT) == 4 ? 8u : 16u, kFull = 0xFFFFFFFFu;
@@ -648,10 +648,5 @@ __device__ __forceinline__ void search_walk(const WalkParams& p) {
         __syncwarp();
     }
 }
-
-template <typename MemT, bool kLists>
-__global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const __grid_constant__ WalkParams p) { search_walk<MemT, kLists, false>(p); }
-template <typename MemT, bool kLists>
-__global__ void __launch_bounds__(kWalkThreads, 1) search_walk_floor_kernel(const __grid_constant__ WalkParams p) { search_walk<MemT, kLists, true>(p); }
 
 }  // namespace moc
