@@ -129,6 +129,7 @@ cudaError_t cudaMalloc(void** p, size_t n) {
     note("malloc " + std::to_string(n));
     if (fails()) return cudaErrorMemoryAllocation;
     *p = aligned_alloc(256, (n + 255) & ~size_t(255));
+    memset(*p, 0, n);      // no kernel writes it: a status is that of a valid sequence
     g_device.insert(*p);
     return cudaSuccess;
 }
