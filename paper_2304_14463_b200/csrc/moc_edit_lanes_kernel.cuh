@@ -40,6 +40,7 @@ struct LaneParent {
     const MemT* pm_;
     const MemT* sm_;
     struct View {
+        static constexpr bool kShared = false;
         const MemT* p;
         __device__ __forceinline__ MemT operator()(int32_t s) const { return __ldg(p + s); }
         __device__ __forceinline__ longlong2 vec(int32_t k) const { return __ldg(reinterpret_cast<const longlong2*>(p) + k); }

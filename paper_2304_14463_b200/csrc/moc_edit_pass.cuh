@@ -17,7 +17,7 @@
 // built on this when one edit's worst case (4 + 2 * largest in-degree) fits.
 //
 // Parent (per lane): occ(v) the node's copy-position word, fre(s), row(s), prof(s), pm(s), sm(s) of the
-// lane's parent, and prof_view(l), which reads the usage array of lane l's parent by step and, as vec(k), by pairs of 64-bit sums.
+// lane's parent, and prof_view(l), which reads the usage array of lane l's parent by step and, as vec(k), by pairs of 64-bit sums (kShared: from shared memory).
 // Graph: succ_start(v), pred_start(v), succ(k), pred(k), m(v).
 #pragma once
 #include "moc_edit_kernels.cuh"
@@ -89,6 +89,12 @@ __device__ __forceinline__ void score_stage_graph(const EditCacheDev& c, char* s
     }
     __syncthreads();
 }
+
+// Vectors that each of 32 lanes takes of a window of nv 16-byte vectors.  An odd number where the usage lies in shared memory: eight lanes'
+// reads then fall on different banks, and so do those of the difference array.  The chain-scoring kernel, 64-bit sums, 3000 chains x 5 generations
+// of 32 proposals, step by step / by vectors, nv / 32 rounded up / odd: n = 442 479 / 497 / 456 us, n = 900 1171 / 1178 / 1125.  Where only the differences
+// lie there, more lanes at work are worth more: eval_edits, 8 edits of 3000 parents, n = 900, 57.3 us, with odd numbers 63.5, n = 350 34.8 and 36.9.
+__host__ __device__ constexpr int32_t edit_run(int32_t nv, bool shared) { return shared ? ((nv + 31) >> 5) | 1 : (nv + 31) >> 5; }
 
 // live: the lane holds an edit record whose fields are in range; pst, T, pdur: status, length and duration of its
 // parent; o, qq, jj: kind (0 insert, 1 delete, 2 move), step of the parent, insertion index.  rl, rv (list_cap
@@ -301,7 +307,7 @@ __device__ __forceinline__ void edit_pass(const Parent& P, const Graph& Gr, cons
                 const int32_t T_s = __shfl_sync(kFull, T, sl);
                 auto inv_s = [&](int32_t t) -> int32_t { const int32_t t1 = t - (t > ji_s ? 1 : 0); return t1 + (t1 >= qd_s ? 1 : 0); };
                 const int32_t end_s = inv_s(hi + 1), v0 = inv_s(lo) >> 1;
-                const int32_t nv = hi < lo ? 0 : ((min(end_s, T_s) + 1) >> 1) - v0, per = (nv + 31) >> 5;
+                const int32_t nv = hi < lo ? 0 : ((min(end_s, T_s) + 1) >> 1) - v0, per = edit_run(nv, decltype(view)::kShared);
                 const int32_t w0 = v0 + min(nv, lane * per), w1 = v0 + min(nv, (lane + 1) * per);
                 for (int32_t k = lane; k < lc; k += 32) {
                     const uint32_t lh = rl[lb + k];

@@ -64,6 +64,7 @@ struct ScoreParent {
     const MemT* pm_;
     const MemT* sm_;
     struct View {
+        static constexpr bool kShared = true;
         const MemT* p;
         __device__ __forceinline__ MemT operator()(int32_t s) const { return p[s]; }
         __device__ __forceinline__ longlong2 vec(int32_t k) const { return reinterpret_cast<const longlong2*>(p)[k]; }
