@@ -159,11 +159,16 @@ void plan_walk(moc_search* s) {
     s->walk_fits = true;
 }
 
-// Whether the next generations are tested with a bound on the new peak: where enough evaluations fall away for what it costs, with many proposals of a
-// generation (one in three of them is evaluated then) or expensive evaluations.  With / without, 10 generations: n = 30, E = 32, 20000 chains 243 / 287 us, n = 78, E = 8, 255
-// chains 20.6 / 23.4, n = 260, E = 8, 8000 chains 63 / 93; n = 442, E = 1, 4096 chains x 20 32.8 / 38.2.  No gain: n = 200, E = 8, a layered
-// graph 212 / 201, n = 300, E = 1 the same; n = 30, E = 1 158 / 149.
-bool walk_floor(const moc_search* s) { return s->samples >= 8 || s->g->n_tiles > 4; }
+// Whether the generations from `generation` on are tested with a bound on the new peak: where enough evaluations fall away for what it costs, with many
+// proposals of a generation or expensive evaluations.  Time of 10 generations with / without it, of that of the kernel before there was one (geometric mean over layered, training and
+// convolutional graphs, 203 to 24576 chains, both sums, call after 0 to 440 generations): 8 proposals, n = 30 0.90 / 0.96, n = 60 0.95 / 0.96, n = 92 0.85 / 0.96,
+// n = 200 0.80 / 0.97, n = 442 0.81 / 0.97; n > 256: 5 proposals 0.88 / 0.97, 3 0.94 / 0.97, 2 0.99 / 0.97.  With one proposal, n > 256: 1.04 / 0.97 in the first
+// 500 generations, 1.00 / 0.96 behind 1000 and 2000, 0.92 / 0.97 behind 10000, when few proposals gain anything and the bound refuses the others (n = 442, 4096 chains
+// x 20, behind 100000: 31.0 us, 37.8 before).  n <= 256: 2 proposals 1.00 / 0.95, 5 at n = 60 0.98 / 0.96.
+constexpr uint32_t kWalkSettled = 4096;
+bool walk_floor(const moc_search* s, uint32_t generation) {
+    return s->samples >= 8 || (s->g->n_tiles > 4 && (s->samples > 1 || generation >= kWalkSettled));
+}
 
 // The variant to launch, prepared when it is first asked for: preparing loads it.  Null: it cannot be.
 const void* walk_variant(moc_search* s, bool floor) {
@@ -295,24 +300,26 @@ int moc_search_run(moc_search* s, int32_t n_generations, void* stream) {
     if (!s->walk_planned) plan_walk(s);
     if (s->incremental ? s->walk_scores
                        : s->walk_fits && g->generation == s->graph_generation && g->want_G == 0 &&
-                             (g->want_kind == MOC_KERNEL_AUTO || g->want_kind == MOC_KERNEL_WARP) && walk_variant(s, walk_floor(s))) {
+                             (g->want_kind == MOC_KERNEL_AUTO || g->want_kind == MOC_KERNEL_WARP) && walk_variant(s, walk_floor(s, s->generation))) {
         moc::WalkParams& w = s->wp;
         w.samples = s->samples;
         w.lanes_per_gen = 1;
         while (w.lanes_per_gen < std::min(s->samples, 32)) w.lanes_per_gen *= 2;
         w.cap = g->d_cap;
         const int32_t most = std::max(1, kWalkProposals / s->samples);
-        const bool floor = walk_floor(s);
-        const void* const fn = walk_variant(s, floor);
-        if (!fn) return fail(MOC_ERR_CUDA, "moc_search_run: the search kernel cannot be prepared");
-        w.sizes = floor && s->walk_sizes;
-        w.list_bytes = (uint32_t)(w.sizes ? g->near_size_bytes : g->near_bytes);
+        // the variants of the first and of the last launch, before either
+        const int32_t last = n_generations > 0 ? (n_generations - 1) / most * most : 0;
+        if (!walk_variant(s, walk_floor(s, s->generation)) || !walk_variant(s, walk_floor(s, s->generation + (uint32_t)last)))
+            return fail(MOC_ERR_CUDA, "moc_search_run: the search kernel cannot be prepared");
         for (int32_t k = 0; k < n_generations; k += most) {
             w.s = p;
             w.s.generation = s->generation + (uint32_t)k;
             w.n_gen = std::min(most, n_generations - k);
+            const bool floor = walk_floor(s, w.s.generation);
+            w.sizes = floor && s->walk_sizes;
+            w.list_bytes = (uint32_t)(w.sizes ? g->near_size_bytes : g->near_bytes);
             void* args[] = {&w};
-            MOC_CUDA(cudaLaunchKernel(fn, dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, floor ? s->walk_smem_floor : s->walk_smem, st));
+            MOC_CUDA(cudaLaunchKernel(s->walk_fn[floor], dim3(s->walk_grid), dim3(32 * s->walk_wpb), args, floor ? s->walk_smem_floor : s->walk_smem, st));
             ++launches;
         }
         s->generation += (uint32_t)n_generations;
@@ -424,7 +431,7 @@ int moc_search_set_samples(moc_search* s, int32_t samples, int32_t incremental) 
     if (incremental == MOC_SEARCH_SCORE_AUTO && s->walk_fits && s->g->generation == s->graph_generation) {
         const int32_t before = s->samples;
         s->samples = samples;
-        if (walk_variant(s, walk_floor(s))) {
+        if (walk_variant(s, walk_floor(s, s->generation))) {
             s->walk_scores = true;
             s->incremental = true;
             return MOC_OK;

@@ -278,8 +278,8 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
 
     for (int32_t c = blockIdx.x * wpb + warp; c < s.P; c += gridDim.x * wpb) {
         int32_t* row = s.rows + ((int64_t)s.cur[c] * s.P + c) * s.stride;
-        int32_t T = s.lens[c], tp = p.peak_at[c];       // without kFloor a step of either kind, else 0 for one that is not exact
-        tp = kFloor ? max(tp, 0) : abs(tp);
+        int32_t T = s.lens[c], tp = p.peak_at[c];
+        if constexpr (!kFloor) tp = abs(tp);            // a step of either kind
         bool valid = s.status[c] >= 0;
         bool over = valid && s.peak[c] > s.M;       // over the budget
         if (lane == 0) {
@@ -332,6 +332,12 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
             __syncwarp();
             if (lane == 0) sts_u32(wa + 4u * (uint32_t)(n + 1), (uint32_t)T * 0x10001u);
             __syncwarp();
+        }
+        if constexpr (kFloor) {
+            // A place from the other variant is not exact.  One evaluation finds it; without it a chain that hardly accepts any more would stay without a bound.
+            bool dep;
+            if (valid && tp < 0) walk_eval<MemT, true>(wa, da, rec0, sell0, n_tiles, T, lane, p.split, dep, tp);
+            tp = max(tp, 0);
         }
         // out with step qd_s, in at index ji_s: the words of the edited sequence at w1, from the parent's at w0
         auto shift_words = [&](uint32_t w0, uint32_t w1, int32_t Tc_s, int32_t qd_s, int32_t ji_s, int32_t x_s, uint32_t wx_s) {

@@ -463,3 +463,22 @@ def test_search_bound_on_the_new_peak(B, graph, scale, pct):
         OS.run(g)
         assert_state_equal(S, OS, f"{graph} {pct} %, {samples} proposals, after {OS.generation}")
     assert OS.accepted > 0
+
+
+@pytest.mark.parametrize("n,scale", [(290, 1), (290, 1 << 36), (601, 1)])
+def test_search_goes_on_with_the_bound(B, n, scale):
+    """One proposal a generation: without the bound at first, with it from generation 4096 on, inside a call and between two; the place of
+    the peak, known by a vector of steps until then, is found once more."""
+    edges = W.layered_dag(n, 3 * n, 12, 7)
+    w, m = W.weights_uniform(n, 0, 9, 7, 1), W.weights_lognormal(n, 4.0, 1.5, 7, 2) * scale
+    seqs, lens = W.schedules(n, edges, 2, 0.25, 9, 7)
+    M = OracleGraph(n, edges, w, m, 2).eval(np.arange(n), 1 << 60)["peak"] * 80 // 100
+    G, O, S, OS = make_pair(B, type("WL", (), dict(n=n, edges=edges, C=2, w=w, m=m)), seqs, lens, M, seed=n)
+    for g in (1, 4094, 1, 1, 300):
+        S.run(g)
+        OS.run(g)
+        assert_state_equal(S, OS, f"after {OS.generation}")
+    S2 = B.Search(G, dev(seqs), dev(lens), M, n)
+    S2.run(OS.generation)
+    assert_state_equal(S2, OS, "in one call")
+    assert OS.accepted > 0
