@@ -162,12 +162,13 @@ void plan_walk(moc_search* s) {
 // Whether the generations from `generation` on are tested with a bound on the new peak: where enough evaluations fall away for what it costs, with many
 // proposals of a generation or expensive evaluations.  Time of 10 generations with / without it, of that of the kernel before there was one (geometric mean over layered, training and
 // convolutional graphs, 203 to 24576 chains, both sums, call after 0 to 440 generations): 8 proposals, n = 30 0.90 / 0.96, n = 60 0.95 / 0.96, n = 92 0.85 / 0.96,
-// n = 200 0.80 / 0.97, n = 442 0.81 / 0.97; n > 256: 5 proposals 0.88 / 0.97, 3 0.94 / 0.97, 2 0.99 / 0.97.  With one proposal, n > 256: 1.04 / 0.97 in the first
+// n = 200 0.80 / 0.97, n = 442 0.81 / 0.97; n > 256: 5 proposals 0.88 / 0.97, 3 0.94 / 0.97.  With one proposal, n > 256: 1.04 / 0.97 in the first
 // 500 generations, 1.00 / 0.96 behind 1000 and 2000, 0.92 / 0.97 behind 10000, when few proposals gain anything and the bound refuses the others (n = 442, 4096 chains
 // x 20, behind 100000: 31.0 us, 37.8 before).  n <= 256: 2 proposals 1.00 / 0.95, 5 at n = 60 0.98 / 0.96.
-constexpr uint32_t kWalkSettled = 4096;
+// Two proposals: 1.00 / 0.96 in the first 500 generations (64-bit sums, a layered graph, n = 442, 24576 chains 1.05), 0.93 / 0.97 behind 1000, 0.83 / 0.97 behind 10000 at n = 442.
 bool walk_floor(const moc_search* s, uint32_t generation) {
-    return s->samples >= 8 || (s->g->n_tiles > 4 && (s->samples > 1 || generation >= kWalkSettled));
+    const uint32_t settled = s->samples == 1 ? 4096u : s->samples == 2 ? 1024u : 0u;
+    return s->samples >= 8 || (s->g->n_tiles > 4 && generation >= settled);
 }
 
 // The variant to launch, prepared when it is first asked for: preparing loads it.  Null: it cannot be.

@@ -445,10 +445,10 @@ def test_a_search_prepares_the_variant_that_it_launches(fake, n, samples):
 
 
 @pytest.mark.parametrize("n,samples,calls", [(100, 1, [(10, "0"), (9000, "000")]), (256, 1, [(4096, "0"), (10, "0")]), (300, 1, [(9000, "011"), (10, "1")]),
-                                             (300, 1, [(4095, "0"), (1, "0"), (1, "1")]), (300, 2, [(10, "1")]), (100, 7, [(10, "0")]), (100, 8, [(10, "1")])])
+                                             (300, 1, [(4095, "0"), (1, "0"), (1, "1")]), (300, 2, [(5000, "011")]), (300, 2, [(1023, "0"), (1, "0"), (1, "1")]), (300, 3, [(10, "1")]), (100, 7, [(10, "0")]), (100, 8, [(10, "1")])])
 def test_when_a_search_is_tested_with_a_bound(fake, n, samples, calls):
-    """A digit per launch (4096 proposals a chain).  One proposal a generation, more than 256 nodes: from generation 4096 on; until then the bound
-    costs more than it saves."""
+    """A digit per launch (4096 proposals a chain).  More than 256 nodes: with one proposal a generation from generation 4096 on, with two from 1024 on;
+    until then the bound costs more than it saves."""
     G = Graph(fake, n)
     S = Search(fake, G, 300, samples)
     for generations, want in calls:
