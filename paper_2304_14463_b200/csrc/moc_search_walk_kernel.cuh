@@ -530,20 +530,28 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
                 // The lane's draw {r1, r2, kind of the edit}, kept for the tests after an acceptance (drawn again each time: n = 30, 32768 chains x 20
                 // 158 -> 150 us, n = 442, 4096 x 20 32.8 -> 31.0).  In the lane's own memory (volatile: not in registers over the evaluations): 384 bytes
                 // of shared memory a warp take as long at n = 442, but cost others a warp, that is a round of chains, or the lists (32 proposals x 10: n = 790,
-                // 64-bit sums, 1600 chains 250 -> 176 us, n = 620, 8000 395 -> 360; one proposal 79 -> 57 and 110 -> 102).
-                volatile uint32_t draw[3];
-                {
+                // 64-bit sums, 1600 chains 250 -> 176 us, n = 620, 8000 395 -> 360; one proposal 79 -> 57 and 110 -> 102).  With 64-bit sums, the lists read
+                // through L1 and most proposals refused at once, the draws' lines cost more there than they save: one proposal x 10, 12288 chains, n = 900
+                // 379 us drawn again, 393 kept, n = 600 221 and 227; with the bound on the new peak (8 proposals, n = 900) 1330 and 1285.
+                constexpr bool kKeep = kLists || kFloor || sizeof(MemT) == 4;
+                auto draw = [&]() -> uint3 {
                     const uint4 r = philox4x32_10_by(make_uint4(s.generation + (uint32_t)(g0 + my_gen), s.chain0 + (uint32_t)c, (uint32_t)(e0 + my_e), 0u),
                                                      [&](int k) { return make_uint2(p.round_key[2 * k], p.round_key[2 * k + 1]); });
-                    draw[0] = r.y;
-                    draw[1] = r.z;
-                    draw[2] = search_pick_kind(s.kinds, r.x);
+                    return make_uint3(r.y, r.z, search_pick_kind(s.kinds, r.x));
+                };
+                volatile uint32_t kept[3];
+                if constexpr (kKeep) {
+                    const uint3 r = draw();
+                    kept[0] = r.x;
+                    kept[1] = r.y;
+                    kept[2] = r.z;
                 }
                 uint32_t pending = drawn;
                 while (pending && T > 0) {
                     // ---- the pending proposals against the present sequence, a lane each
-                    const int32_t op = (int32_t)draw[2];
-                    const int32_t q = (int32_t)(draw[0] % (uint32_t)T), j = (int32_t)(draw[1] % ((uint32_t)T + (op == 0 ? 1u : 0u)));
+                    const uint3 r = kKeep ? make_uint3(kept[0], kept[1], kept[2]) : draw();
+                    const int32_t op = (int32_t)r.z;
+                    const int32_t q = (int32_t)(r.x % (uint32_t)T), j = (int32_t)(r.y % ((uint32_t)T + (op == 0 ? 1u : 0u)));
                     const int32_t qd = op >= 1 ? q : kEditNone, ji = op != 1 ? j : kEditNone;
                     const int32_t Tc = T + (op == 0 ? 1 : 0) - (op == 1 ? 1 : 0);
                     const int32_t x = row[q];

@@ -482,3 +482,21 @@ def test_search_goes_on_with_the_bound(B, n, scale):
     S2.run(OS.generation)
     assert_state_equal(S2, OS, "in one call")
     assert OS.accepted > 0
+
+
+@pytest.mark.parametrize("n,P,samples", [(61, 64, 1), (61, 64, 3), (200, 40, 7), (61, 64, 9), (256, 30, 33), (331, 30, 1), (331, 40, 2), (331, 40, 8)])
+def test_search_walk_wide_sums_without_lists(B, n, P, samples):
+    """64-bit sums with the neighbours' lists and the output sizes in global memory (durations beyond 31 bits), without and with the bound on the new peak."""
+    edges = W.layered_dag(n, 3 * n + 1, max(4, n // 40), n)
+    w, m = W.weights_uniform(n, 1, 30, n, 1) << 26, W.weights_lognormal(n, 4.0, 1.5, n, 2) << 30
+    assert int(w.sum()) >= 1 << 31 and int(m.sum()) >= 1 << 31
+    seqs, lens = W.schedules(n, edges, 2, 0.3, P, n)
+    M = OracleGraph(n, edges, w, m, 2).eval(np.arange(n), 1 << 60)["peak"] * 80 // 100
+    if samples == 1:
+        G, O, S, OS = make_pair(B, type("WL", (), dict(n=n, edges=edges, C=2, w=w, m=m)), seqs, lens, M, seed=n)
+        for g in (1, 33, 66):
+            S.run(g)
+            OS.run(g)
+            assert_state_equal(S, OS, f"n {n}, after {OS.generation}")
+    else:
+        _run_scored(B, n, edges, w, m, 2, seqs, lens, M, samples, 1, (2, 9, 40), what=f"n {n}")
