@@ -336,7 +336,10 @@ __global__ void __launch_bounds__(kWalkThreads, 1) search_walk_kernel(const Walk
         if constexpr (kFloor) {
             // A place from the other variant is not exact.  One evaluation finds it; without it a chain that hardly accepts any more would stay without a bound.
             bool dep;
-            if (valid && tp < 0) walk_eval<MemT, true>(wa, da, rec0, sell0, n_tiles, T, lane, p.split, dep, tp);
+            if (valid && tp < 0) {
+                walk_eval<MemT, true>(wa, da, rec0, sell0, n_tiles, T, lane, p.split, dep, tp);
+                if (lane == 0) p.peak_at[c] = tp;       // once, whether or not the chain accepts in this launch
+            }
             tp = max(tp, 0);
         }
         // out with step qd_s, in at index ji_s: the words of the edited sequence at w1, from the parent's at w0
