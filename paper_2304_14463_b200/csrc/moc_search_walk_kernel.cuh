@@ -23,7 +23,7 @@
 // Chains without a valid sequence (status < 0) have no test to rely on: their proposals are evaluated from
 // the written-out order, one generation at a time, until one is valid.
 //
-// Bound: instruction issue (76 % of the slots with 32 proposals a generation, 2600 instructions each while the chains are over the budget) and, for small populations,
+// Bound: instruction issue (76 % of the slots with 32 proposals a generation; a generation of new chains takes 3300 instructions, behind ten of them 2600) and, for small populations,
 // the latency of its dependent shared-memory reads; 28 warps beat 24 and 20 with more registers each, and 30 with fewer.
 // n = 442, state copied out: 4096 chains x 20 generations 436 -> 41.9 us against two kernels per generation that
 // write every proposal out, 38.9 with the neighbours' lists on chip, 37.1 with the words of a sequence from eight loads in flight; 32768 chains x 32 proposals x 10 generations 2409 -> 1052 us
